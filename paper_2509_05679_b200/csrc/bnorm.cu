@@ -1,0 +1,264 @@
+// Batch-norm with fp32 storage (statistics per worker), two launches per layer and direction at most:
+//   forward : the producing convolution has left per-tile (mean, sum of squared deviations) (fconv.cu); ONE kernel merges them
+//             and normalises.  Backward: one kernel of partial sums, one that finishes the sums and applies them.
+// The generic kernels (kernels.cu) take three launches each, read 4 bytes per thread and load instruction and use half of
+// their lanes at 16 channels; the paper's ResNet-20 has 21 batch-norms per step, all of them resident in L2 (12.6 MB at the most),
+// so that launches and bytes in flight count, not DRAM.  A thread keeps 4 consecutive channels (16-byte accesses) for every row
+// it visits; a CTA owns a contiguous row range of one worker.  Used when C / 4 is a power of two <= 256.
+// Every sum has a fixed order.
+#include "kernels.h"
+
+#include <cuda_bf16.h>
+
+namespace fdg {
+
+namespace {
+
+constexpr int BT = 256;
+constexpr int BNF_MAX_CHUNKS = 64;
+
+struct BnfArgs {
+    const float* x; const float* out; const float* dout; const float* res;
+    const float* gamma; const float* beta; size_t p_group;      // floats between the workers' gamma / beta (0: shared)
+    float* stats;                                               // [worker][C][4]: mean, invstd, and what those fp32 values are off by
+    const float* tile_part; int tiles;                          // forward: the convolution's records (see fconv_stat_tiles)
+    float* part;                                                // backward: [chunk][worker][C][2]
+    float* y; float* dres; int accum_dx, accum_dres;
+    float* dgamma; float* dbeta; size_t g_group; int accum_params;
+    long rpw; int C, relu, mask_from_x;
+};
+
+// (mean, invstd) of worker w from its tiles' (mean, sum of squared deviations, count):
+//   mean = sum n_t m_t / N,  N var = sum (q_t + n_t (m_t - mean)^2), in double, for the channels c0 .. c0 + nc - 1 (nc <= 256, a power
+// of two or a multiple of 256 handled by the caller's loop).  tmp: BT doubles.
+__device__ __forceinline__ void merge_tiles(const float* __restrict__ part, int tiles, int w, int nw, int C, int c0, int nc, long rows, float4* dst, double* tmp) {
+    const int tid = threadIdx.x, lanes = BT / nc, c = tid % nc, pt = tid / nc;
+    const float2* p = (const float2*)part + (size_t)w * tiles * C + c0 + c;
+    const float* cnt = part + (size_t)nw * tiles * C * 2 + (size_t)w * tiles;
+    double s = 0.0;
+    for (int t = pt; t < tiles; t += lanes) s += (double)cnt[t] * (double)p[(size_t)t * C].x;
+    tmp[tid] = s;
+    __syncthreads();
+    double mean = 0.0;
+    for (int q = 0; q < lanes; ++q) mean += tmp[q * nc + c];
+    mean /= (double)rows;
+    __syncthreads();
+    s = 0.0;
+    for (int t = pt; t < tiles; t += lanes) { const float2 v = p[(size_t)t * C]; const double d = (double)v.x - mean; s += (double)v.y + (double)cnt[t] * d * d; }
+    tmp[tid] = s;
+    __syncthreads();
+    if (pt == 0) {
+        double m2 = 0.0;
+        for (int q = 0; q < lanes; ++q) m2 += tmp[q * nc + c];
+        const double istd = 1.0 / sqrt(m2 / (double)rows + 1e-5);
+        const float mh = (float)mean, ih = (float)istd;
+        dst[c] = make_float4(mh, ih, (float)(mean - (double)mh), (float)(istd - (double)ih));
+    }
+    __syncthreads();
+}
+
+// stats only (bf16 storage: the streamed apply kernel of kernels.cu follows).  grid = (channel blocks of min(C, 64), workers)
+__global__ void __launch_bounds__(BT) bn_merge_tiles_k(const float* __restrict__ part, float* __restrict__ stats, int tiles, int C, int nc, long rows) {
+    __shared__ double tmp[BT];
+    __shared__ float4 res[BT];
+    const int c0 = blockIdx.x * nc, w = blockIdx.y;
+    merge_tiles(part, tiles, w, gridDim.y, C, c0, nc, rows, res, tmp);
+    if ((int)threadIdx.x < nc) *(float2*)(stats + ((size_t)w * C + c0 + threadIdx.x) * 2) = make_float2(res[threadIdx.x].x, res[threadIdx.x].y);
+}
+
+// gamma * (x - mean) * invstd + beta with the roundings that matter near zero carried along: a ReLU decides on the sign of this
+// value, and the plain fp32 expression (four roundings, two of them of constants that a whole channel shares) is off by more
+// than the stored x and the stored result are.  scale + scale_lo = gamma * invstd, mean + mean_lo, invstd + invstd_lo from the double-
+// precision merge.  One expression for both directions, so that the backward pass finds the same sign.
+struct BnCoef { float mean, scale, scale_lo, beta, mean_lo; };
+__device__ __forceinline__ BnCoef bn_coef(float4 st, float gamma, float beta) {
+    BnCoef k;
+    k.mean = st.x; k.mean_lo = st.z; k.beta = beta;
+    k.scale = __fmul_rn(gamma, st.y);
+    k.scale_lo = __fmaf_rn(gamma, st.w, __fmaf_rn(gamma, st.y, -k.scale));
+    return k;
+}
+__device__ __forceinline__ float bn_value(float x, const BnCoef& k) {
+    const float d = __fsub_rn(x, k.mean), t = __fadd_rn(d, k.mean);          // two-sum: x - mean = d + e exactly (as far as fp32 holds e)
+    const float e = __fadd_rn(__fsub_rn(x, t), __fsub_rn(__fsub_rn(t, d), k.mean));
+    return __fadd_rn(__fmaf_rn(d, k.scale, k.beta), __fmaf_rn(d, k.scale_lo, __fmul_rn(__fsub_rn(e, k.mean_lo), k.scale)));
+}
+
+__device__ __forceinline__ float2 warp_sum(float2 v) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) { v.x += __shfl_xor_sync(0xffffffffu, v.x, d); v.y += __shfl_xor_sync(0xffffffffu, v.y, d); }
+    return v;
+}
+
+// MODE 0: y = bn(x) (+ res) (relu).  MODE 1: partial sums of (dy, dy * xhat), dy = dout * [out > 0] if relu.
+// MODE 2: dx (+)= gamma * invstd * (dy - mean(dy) - xhat * mean(dy xhat)), dres (+)= dy, dgamma, dbeta.
+template <int MODE>
+__global__ void __launch_bounds__(BT) bnf_kernel(const BnfArgs a) {
+    __shared__ double tmp[BT];
+    __shared__ float4 st4[1024];                 // MODE 0: statistics; MODE 2: (sum dy, sum dy xhat); MODE 1: reduction
+    float2* const st = (float2*)st4;
+    const int C = a.C, cgs = C / 4, rows_it = BT / cgs, tid = threadIdx.x, cg = tid % cgs, rl = tid / cgs;
+    const int w = blockIdx.y, nw = gridDim.y, chunks = gridDim.x;
+    long per = (a.rpw + chunks - 1) / chunks;
+    per = (per + rows_it - 1) / rows_it * rows_it;
+    const long r0 = (long)blockIdx.x * per, r1 = min(a.rpw, r0 + per);
+    if (MODE == 0) {
+        const int nc = C < BT ? C : BT;
+        for (int c0 = 0; c0 < C; c0 += nc) merge_tiles(a.tile_part, a.tiles, w, nw, C, c0, nc, a.rpw, st4 + c0, tmp);
+        if (blockIdx.x == 0) for (int c = tid; c < C; c += BT) *(float4*)(a.stats + ((size_t)w * C + c) * 4) = st4[c];
+    }
+    if (MODE == 2) {
+        const float2* const part = (const float2*)a.part;
+        float2* const t2 = (float2*)tmp;
+        const int nc = C < BT ? C : BT, lanes = BT / nc, c = tid % nc, pt = tid / nc;
+        for (int c0 = 0; c0 < C; c0 += nc) {
+            float2 s = make_float2(0.f, 0.f);
+            for (int k = pt; k < chunks; k += lanes) { const float2 v = part[((size_t)k * nw + w) * C + c0 + c]; s.x += v.x; s.y += v.y; }
+            t2[tid] = s;
+            __syncthreads();
+            if (pt == 0) {
+                float2 t = make_float2(0.f, 0.f);
+                for (int q = 0; q < lanes; ++q) { t.x += t2[q * nc + c].x; t.y += t2[q * nc + c].y; }
+                st[c0 + c] = t;
+            }
+            __syncthreads();
+        }
+        if (a.g_group) {                         // every worker has parameters of its own
+            if (blockIdx.x == 0) for (int e = tid; e < C; e += BT) { a.dbeta[w * a.g_group + e] = st[e].x; a.dgamma[w * a.g_group + e] = st[e].y; }
+        } else {                                 // sums over all workers: one warp per channel, spread over the launch's CTAs
+            const int warp = tid >> 5, lane = tid & 31, rows = nw * chunks, me = w * chunks + blockIdx.x;
+            for (int e = me + warp * rows; e < C; e += (BT / 32) * rows) {
+                float2 s = make_float2(0.f, 0.f);
+                for (int r = lane; r < rows; r += 32) { const float2 v = part[((size_t)(r % chunks) * nw + r / chunks) * C + e]; s.x += v.x; s.y += v.y; }
+                s = warp_sum(s);
+                if (lane == 0) { a.dbeta[e] = a.accum_params ? a.dbeta[e] + s.x : s.x; a.dgamma[e] = a.accum_params ? a.dgamma[e] + s.y : s.y; }
+            }
+        }
+    }
+    float mean[4], istd[4], ga[4], c1[4], c2[4], s1[4], s2[4];
+    BnCoef k[4];
+    const float inv_n = 1.f / (float)a.rpw;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int c = cg * 4 + j;
+        const float4 ms = MODE == 0 ? st4[c] : *(const float4*)(a.stats + ((size_t)w * C + c) * 4);
+        mean[j] = ms.x; istd[j] = ms.y;
+        ga[j] = a.gamma[w * a.p_group + c];
+        k[j] = bn_coef(ms, ga[j], a.beta[w * a.p_group + c]);
+        if (MODE == 2) { c1[j] = st[c].x * inv_n; c2[j] = st[c].y * inv_n; }
+        s1[j] = s2[j] = 0.f;
+    }
+    const size_t base = ((size_t)w * a.rpw) * C + (size_t)cg * 4;
+    const bool need_out = MODE != 0 && a.relu && !a.mask_from_x;
+    constexpr int U = 4;                         // rows in flight per thread
+    for (long r = r0 + rl; r < r1; r += (long)rows_it * U) {
+        float4 xv[U], dv[U], ov[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long rr = r + (long)u * rows_it;
+            if (rr >= r1) continue;
+            const size_t o = base + (size_t)rr * C;
+            xv[u] = *(const float4*)(a.x + o);
+            if (MODE == 0) { if (a.res) ov[u] = *(const float4*)(a.res + o); }
+            else { dv[u] = *(const float4*)(a.dout + o); if (need_out) ov[u] = *(const float4*)(a.out + o); }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long rr = r + (long)u * rows_it;
+            if (rr >= r1) continue;
+            const size_t o = base + (size_t)rr * C;
+            const float x[4] = {xv[u].x, xv[u].y, xv[u].z, xv[u].w};
+            if (MODE == 0) {
+                float v[4];
+                const float re[4] = {ov[u].x, ov[u].y, ov[u].z, ov[u].w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    v[j] = bn_value(x[j], k[j]);
+                    if (a.res) v[j] += re[j];
+                    if (a.relu) v[j] = fmaxf(v[j], 0.f);
+                }
+                *(float4*)(a.y + o) = make_float4(v[0], v[1], v[2], v[3]);
+            } else {
+                float d[4] = {dv[u].x, dv[u].y, dv[u].z, dv[u].w};
+                const float ou[4] = {ov[u].x, ov[u].y, ov[u].z, ov[u].w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (a.relu && !((need_out ? ou[j] : bn_value(x[j], k[j])) > 0.f)) d[j] = 0.f;
+                    if (MODE == 1) { s1[j] += d[j]; s2[j] += d[j] * (x[j] - mean[j]) * istd[j]; }
+                }
+                if (MODE == 2) {
+                    float v[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) { const float xh = (x[j] - mean[j]) * istd[j]; v[j] = ga[j] * istd[j] * (d[j] - c1[j] - xh * c2[j]); }
+                    if (a.y) {
+                        if (a.accum_dx) { const float4 old = *(const float4*)(a.y + o); v[0] += old.x; v[1] += old.y; v[2] += old.z; v[3] += old.w; }
+                        *(float4*)(a.y + o) = make_float4(v[0], v[1], v[2], v[3]);
+                    }
+                    if (a.dres) {
+                        if (a.accum_dres) { const float4 old = *(const float4*)(a.dres + o); d[0] += old.x; d[1] += old.y; d[2] += old.z; d[3] += old.w; }
+                        *(float4*)(a.dres + o) = make_float4(d[0], d[1], d[2], d[3]);
+                    }
+                }
+            }
+        }
+    }
+    if (MODE == 1) {
+        static_assert(sizeof(float) * BT * 8 <= sizeof(st4), "reduction space");
+        float* const r8 = (float*)st;            // [8][256]: value i of thread t at i * 256 + t (no bank conflicts)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { r8[j * BT + tid] = s1[j]; r8[(4 + j) * BT + tid] = s2[j]; }
+        __syncthreads();
+        for (int t = tid; t < 2 * C; t += BT) {
+            const int c = t >> 1, v = (t & 1) * 4 + (c & 3), q = c >> 2;
+            float acc = 0.f;
+            for (int i = 0; i < rows_it; ++i) acc += r8[v * BT + i * cgs + q];
+            a.part[(((size_t)blockIdx.x * nw + w) * C + c) * 2 + (t & 1)] = acc;
+        }
+    }
+}
+
+// Three CTAs per SM over all workers, at least four rows per thread.
+int bnf_chunks(int nw, long rpw, int C) {
+    const long rows_it = BT / (C / 4), want = (3 * 148 + nw - 1) / nw, maxc = (rpw + rows_it * 4 - 1) / (rows_it * 4);
+    long c = want < maxc ? want : maxc;
+    if (c > BNF_MAX_CHUNKS) c = BNF_MAX_CHUNKS;
+    return (int)(c < 1 ? 1 : c);
+}
+
+}  // namespace
+
+bool bnf_supported(int dt, int C) { return dt == 0 && C % 4 == 0 && C / 4 <= BT && ((C / 4) & (C / 4 - 1)) == 0; }
+
+void bn_merge_tiles(const float* tile_part, float* stats, int tiles, int nw, long rpw, int C, cudaStream_t s) {
+    int nc = 1;                                  // channels per block: a power of two that divides C
+    while (nc < 64 && C % (2 * nc) == 0) nc *= 2;
+    Scope sc(KC_BN_FWD_STATS, 0.0, 8.0 * tiles * nw * C, s);
+    bn_merge_tiles_k<<<dim3(C / nc, nw), BT, 0, s>>>(tile_part, stats, tiles, C, nc, rpw);
+}
+
+void bnf_forward(const float* x, const float* gamma, const float* beta, size_t p_group, const float* res, float* y, float* stats, const float* tile_part,
+                 int tiles, int nw, long rpw, int C, bool relu, cudaStream_t s) {
+    BnfArgs a{};
+    a.x = x; a.gamma = gamma; a.beta = beta; a.p_group = p_group; a.res = res; a.y = y; a.stats = stats; a.tile_part = tile_part; a.tiles = tiles;
+    a.rpw = rpw; a.C = C; a.relu = relu;
+    Scope sc(KC_BN_FWD_APPLY, 0.0, 4.0 * nw * rpw * C * (res ? 3 : 2), s);
+    bnf_kernel<0><<<dim3(bnf_chunks(nw, rpw, C), nw), BT, 0, s>>>(a);
+}
+
+void bnf_backward(const float* x, const float* out, const float* dout, const float* gamma, const float* beta, size_t p_group, const float* stats, float* dx,
+                  bool accum_dx, float* dres, bool accum_dres, float* dgamma, float* dbeta, size_t g_group, float* scratch, int nw, long rpw, int C, bool relu,
+                  bool mask_from_x, bool accum_params, cudaStream_t s) {
+    BnfArgs a{};
+    a.x = x; a.out = out; a.dout = dout; a.gamma = gamma; a.beta = beta; a.p_group = p_group; a.stats = (float*)stats; a.y = dx; a.accum_dx = accum_dx;
+    a.dres = dres; a.accum_dres = accum_dres; a.dgamma = dgamma; a.dbeta = dbeta; a.g_group = g_group; a.accum_params = accum_params; a.part = scratch;
+    a.rpw = rpw; a.C = C; a.relu = relu; a.mask_from_x = mask_from_x;
+    const dim3 grid(bnf_chunks(nw, rpw, C), nw);
+    const double total = (double)nw * rpw * C;
+    const int reads = 2 + (relu && !mask_from_x ? 1 : 0);
+    { Scope sc(KC_BN_BWD_REDUCE, 0.0, 4.0 * total * reads, s);
+      bnf_kernel<1><<<grid, BT, 0, s>>>(a); }
+    Scope sc(KC_BN_BWD_APPLY, 0.0, 4.0 * total * (reads + 1 + (accum_dx ? 1 : 0) + (dres ? (accum_dres ? 2 : 1) : 0)), s);
+    bnf_kernel<2><<<grid, BT, 0, s>>>(a);
+}
+
+}  // namespace fdg

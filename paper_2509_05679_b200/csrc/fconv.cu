@@ -1,0 +1,652 @@
+// FMA convolutions (CUDA cores, fp32 arithmetic, fp32 or bf16 storage) for the layers the tensor-core kernels do not take:
+// the whole fp32 path (TF32 would break its 1e-5 tolerance) and, with bf16 storage, channel counts that are no multiple of
+// 64 (the paper's ResNet-20 has 16 and 32).  3x3 and 1x1, stride 1 and 2, any channel counts, any image size.
+//
+//   fc_kernel : forward and input gradient.  A CTA computes 128 pixels x 16 output channels: the input region of its
+//               pixels (halo included) is fetched ONCE per 16-channel chunk and every filter tap reads it from shared memory.
+//   fw_kernel : weight gradient.  A CTA keeps a 16 c_out x (taps x 16 c_in) tile of dW in registers over all the pixels of
+//               its split; partial sums per CTA, added in a fixed order by fw_reduce_kernel.
+//
+// Arithmetic: packed fp32 (fma.rn.f32x2: 65.6 TFLOP/s on a B200 where scalar fma gives 46.7).  The pairs lie along the
+// contraction (channels 2i and 2i + 1) in fc_kernel and along c_in in fw_kernel, so that operands come out of NHWC data as
+// 16-byte vectors without shuffling.  Chains of at most 16 products are added to a compensated (Kahan) running sum, as in
+// igemm_simt: the rounding error of a long contraction stays at a few ulps.
+//
+// What bounds them: the FMA pipe (fc_kernel issues 32 packed FMAs for eight 16-byte shared loads, fw_kernel 16 for four).
+// The implicit-GEMM kernel they replace fetched every operand element by itself with two integer divisions and reached
+// 2.5-9 TFLOP/s on the ResNet-20 layers.
+#include "kernels.h"
+
+#include <cuda_bf16.h>
+
+namespace fdg {
+
+typedef __nv_bfloat16 bf16;
+
+namespace {
+
+constexpr int FC_THREADS = 128;          // 4 warps: 32 pixels x 16 output channels each, 4 pixels x 4 channels per thread
+constexpr int FC_PIX = 128;
+constexpr int FC_CO = 16;
+constexpr int FC_KC = 16;                // channels per chunk
+constexpr int PITCH = 20;                // floats per pixel (or weight row) in shared memory: 16 + 4, so that the eight 16-byte reads
+                                         // of neighbouring pixels fall into different banks
+constexpr int FW_THREADS = 288;          // 9 taps x 2 groups of 8 c_in x 4 groups of 4 c_out x 4 pixel slices
+constexpr int FW_CO = 16, FW_CI = 16;
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
+    const int n = valid ? 16 : 0;        // 0: the 16 bytes are zero-filled
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+__device__ __forceinline__ float to_f(float v) { return v; }
+__device__ __forceinline__ float to_f(bf16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ void put(float* p, float v) { *p = v; }
+__device__ __forceinline__ void put(bf16* p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ float4 ld4(const float* p) { return *(const float4*)p; }
+__device__ __forceinline__ float4 ld4(const bf16* p) {
+    const uint2 v = *(const uint2*)p;
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+}
+__device__ __forceinline__ void st4(float* p, float4 v) { *(float4*)p = v; }
+__device__ __forceinline__ void st4(bf16* p, float4 v) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+    *(uint2*)p = make_uint2(*(const uint32_t*)&a, *(const uint32_t*)&b);
+}
+
+// The input region of a tile, channels c0 .. c0 + 15, into dst[pixel][PITCH]: nimg images x RH rows x RW pixels whose first
+// pixel is (h0, w0) and whose neighbours are `step` pixels apart in the tensor; zeros outside the image, past image n_end
+// and past channel C.  A warp takes whole rows, so that the loop has no division.
+// VEC: C is a multiple of 4 (16-byte fp32 / 8-byte bf16 pieces); fp32 pieces travel by cp.async.
+template <typename T, bool VEC>
+__device__ __forceinline__ void load_region(const T* __restrict__ x, float* dst, int n0, int n_end, int nimg, int h0, int w0, int RH, int RW, int step,
+                                            int H, int W, int C, int c0, int nq, int warp, int nwarps, int lane) {
+    int ni = 0, rh = warp;
+    while (rh >= RH) { rh -= RH; ++ni; }
+    while (ni < nimg) {
+        const int n = n0 + ni, h = h0 + rh * step;
+        const bool row_ok = n < n_end && h >= 0 && h < H;
+        const T* src = x + (((size_t)(row_ok ? n : n0) * H + (row_ok ? h : 0)) * W) * C + c0;
+        float* d = dst + (size_t)((ni * RH + rh) * RW) * PITCH;
+        for (int j = lane; j < RW * 4; j += 32) {
+            const int rw = j >> 2, q = j & 3;
+            if (q >= nq) continue;
+            const int w = w0 + rw * step, c = 4 * q;
+            const bool ok = row_ok && w >= 0 && w < W;
+            if (VEC) {
+                const bool in = ok && c0 + c < C;
+                const T* s = src + (in ? (size_t)w * C + c : 0);
+                if (sizeof(T) == 4) cp_async16(smem_addr(d + rw * PITCH + c), s, in);
+                else *(float4*)(d + rw * PITCH + c) = in ? ld4(s) : make_float4(0.f, 0.f, 0.f, 0.f);
+            } else {
+                float v[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = ok && c0 + c + e < C ? to_f(src[(size_t)w * C + c + e]) : 0.f;
+                *(float4*)(d + rw * PITCH + c) = make_float4(v[0], v[1], v[2], v[3]);
+            }
+        }
+        rh += nwarps;
+        while (rh >= RH) { rh -= RH; ++ni; }
+    }
+}
+
+template <typename T> __device__ __forceinline__ float stored(float v);
+template <> __device__ __forceinline__ float stored<float>(float v) { return v; }
+template <> __device__ __forceinline__ float stored<bf16>(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
+
+struct Yes { static constexpr bool value = true; };
+struct No { static constexpr bool value = false; };
+
+struct FcParams {
+    int H, W, C;                         // input tensor (the error gradient in the backward direction)
+    int Ho, Wo, Co;                      // output tensor
+    int Hd, Wd, os, xs;                  // destination grid of a class, its stride in the output, stride of the input per destination pixel
+    int ngroup;                          // images per group (a group has its own weights)
+    int ncls, cls_tap0[5], cls_oph[4], cls_opw[4];       // output parity classes (one, unless this is a stride-2 input gradient)
+    int cls_h0[4], cls_w0[4], cls_rh[4], cls_rw[4];      // per class: offset and size of the input region of a tile
+    int toff[9], wtap[9];                // per tap: offset inside the region (floats), index of its weights
+    int Wt, Ht, Nt, lw, lh, tiles_w, tiles_h;            // tile = Wt x Ht x Nt = 128 destination pixels (powers of two)
+    int taps;                            // taps of the weight tensor
+    int back;                            // 0: B[n][k] = W[n][tap][k]; 1: B[n][k] = W[k][tap][n]
+    size_t w_group, b_group;             // elements between the groups' weights / biases
+    int epi;
+    int x_floats, w_floats, buffers;     // shared memory of one buffer
+};
+
+// 16 output channels x up to 16 input channels of every tap of the class into dst[tap][row][PITCH]; channel n sits in row
+// (n % 4) * 4 + n / 4, so that the four channel groups of a warp read neighbouring rows.
+template <typename T, bool VEC>
+__device__ __forceinline__ void load_weights(const T* __restrict__ w, float* dst, const FcParams& p, int t0, int t1, int co0, int c0, int nq, int tid) {
+    for (int i = tid; i < (t1 - t0) * 64; i += FC_THREADS) {
+        const int t = i >> 6, e = i & 63;
+        const int tap = p.wtap[t0 + t];
+        if (!p.back) {
+            const int n = e >> 2, q = e & 3;
+            if (q >= nq) continue;
+            const int co = co0 + n, c = c0 + 4 * q;
+            const T* s = w + ((size_t)(co < p.Co ? co : 0) * p.taps + tap) * p.C;
+            float4 v;
+            if (VEC) v = co < p.Co && c < p.C ? ld4(s + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            else {
+                float f[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) f[j] = co < p.Co && c + j < p.C ? to_f(s[c + j]) : 0.f;
+                v = make_float4(f[0], f[1], f[2], f[3]);
+            }
+            *(float4*)(dst + (t * 16 + (n & 3) * 4 + (n >> 2)) * PITCH + 4 * q) = v;
+        } else {
+            // k runs over the layer's output channels, n over its input channels (contiguous in memory)
+            const int k = e >> 2, g = e & 3;
+            if (k >= 4 * nq) continue;
+            const bool kin = c0 + k < p.C;
+            const T* s = w + ((size_t)(kin ? c0 + k : 0) * p.taps + tap) * p.Co;
+            float f[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) { const int n = co0 + 4 * g + j; f[j] = kin && n < p.Co ? to_f(s[n]) : 0.f; }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) dst[(t * 16 + j * 4 + g) * PITCH + k] = f[j];          // channel 4 g + j: row j * 4 + g
+        }
+    }
+}
+
+// grid = (pixel tiles, blocks of 16 output channels, groups x classes).  NQ: 4-channel quads per chunk (1: at most 4 channels).
+template <typename T, int NQ, bool VEC>
+__global__ void __launch_bounds__(FC_THREADS, 4) fc_kernel(const T* __restrict__ x, const T* __restrict__ w, const float* __restrict__ bias, T* __restrict__ y,
+                                                           float* __restrict__ stat, const __grid_constant__ FcParams p) {
+    extern __shared__ __align__(16) float fsm[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int cls = blockIdx.z % p.ncls, grp = blockIdx.z / p.ncls;
+    int tile = blockIdx.x;
+    const int tw = tile % p.tiles_w; tile /= p.tiles_w;
+    const int th = tile % p.tiles_h, tn = tile / p.tiles_h;
+    const int n_end = (grp + 1) * p.ngroup, n0 = grp * p.ngroup + tn * p.Nt;
+    const int hd0 = th * p.Ht, wd0 = tw * p.Wt, co0 = blockIdx.y * FC_CO;
+    const int t0 = p.cls_tap0[cls], t1 = p.cls_tap0[cls + 1];
+    const int RH = p.cls_rh[cls], RW = p.cls_rw[cls], h0 = hd0 * p.xs + p.cls_h0[cls], w0 = wd0 * p.xs + p.cls_w0[cls];
+    w += (size_t)grp * p.w_group;
+
+    // this thread: pixels warp * 32 + g + 8 i (i = 0..3), channels co0 + 4 cg + j
+    const int g = lane & 7, cg = lane >> 3;
+    uint32_t xb[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int px = warp * 32 + g + 8 * i;
+        const int pw = px & (p.Wt - 1), ph = (px >> p.lw) & (p.Ht - 1), pn = px >> (p.lw + p.lh);
+        xb[i] = (uint32_t)(((pn * RH + ph * p.xs) * RW + pw * p.xs) * PITCH);
+    }
+    float2 acc[4][2], comp[4][2], part[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) { acc[i][j] = make_float2(0.f, 0.f); comp[i][j] = make_float2(0.f, 0.f); }
+
+    const int chunks = t1 > t0 ? (p.C + FC_KC - 1) / FC_KC : 0;
+    auto fetch = [&](int c, int buf) {
+        float* xs_ = fsm + (size_t)buf * (p.x_floats + p.w_floats);
+        load_region<T, VEC>(x, xs_, n0, n_end, p.Nt, h0, w0, RH, RW, 1, p.H, p.W, p.C, c * FC_KC, NQ, warp, FC_THREADS / 32, lane);
+        load_weights<T, VEC>(w, xs_ + p.x_floats, p, t0, t1, co0, c * FC_KC, NQ, tid);
+        cp_commit();
+    };
+    if (chunks) fetch(0, 0);
+    for (int c = 0; c < chunks; ++c) {
+        const int buf = p.buffers > 1 ? c & 1 : 0;
+        if (p.buffers > 1 && c + 1 < chunks) { fetch(c + 1, buf ^ 1); cp_wait<1>(); } else cp_wait<0>();
+        __syncthreads();
+        const float* xs_ = fsm + (size_t)buf * (p.x_floats + p.w_floats);
+        const float* ws_ = xs_ + p.x_floats + cg * PITCH;
+        auto tap = [&](int t, auto first) {
+            const float* xt = xs_ + p.toff[t0 + t];
+            const float* wt = ws_ + t * (16 * PITCH);
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                float4 wv[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) wv[j] = *(const float4*)(wt + j * (4 * PITCH) + 4 * q);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 xv = *(const float4*)(xt + xb[i] + 4 * q);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float2 lo = make_float2(xv.x, xv.y), hi = make_float2(xv.z, xv.w);
+                        if (decltype(first)::value && q == 0) part[i][j] = __fmul2_rn(lo, make_float2(wv[j].x, wv[j].y));
+                        else part[i][j] = __ffma2_rn(lo, make_float2(wv[j].x, wv[j].y), part[i][j]);
+                        part[i][j] = __ffma2_rn(hi, make_float2(wv[j].z, wv[j].w), part[i][j]);
+                    }
+                }
+            }
+        };
+        auto flush = [&]() {             // Kahan: acc += even + odd part, two channels per instruction
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const float2 s = make_float2(part[i][2 * j].x + part[i][2 * j].y, part[i][2 * j + 1].x + part[i][2 * j + 1].y);
+                    const float2 yv = __fadd2_rn(s, make_float2(-comp[i][j].x, -comp[i][j].y));
+                    const float2 t = __fadd2_rn(acc[i][j], yv);
+                    const float2 d = __fadd2_rn(t, make_float2(-acc[i][j].x, -acc[i][j].y));
+                    comp[i][j] = __fadd2_rn(d, make_float2(-yv.x, -yv.y));
+                    acc[i][j] = t;
+                }
+        };
+        int t = 0;
+#pragma unroll 1
+        for (; t + 1 < t1 - t0; t += 2) { tap(t, Yes()); tap(t + 1, No()); flush(); }      // two taps x 16 channels: pair chains of 16 products
+        if (t < t1 - t0) { tap(t, Yes()); flush(); }
+        __syncthreads();
+        if (p.buffers == 1 && c + 1 < chunks) fetch(c + 1, 0);
+    }
+
+    float val[4][4];
+    bool valid[4];
+    const int co = co0 + 4 * cg;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int px = warp * 32 + g + 8 * i;
+        const int wd = wd0 + (px & (p.Wt - 1)), hd = hd0 + ((px >> p.lw) & (p.Ht - 1)), n = n0 + (px >> (p.lw + p.lh));
+        valid[i] = n < n_end && hd < p.Hd && wd < p.Wd;
+        float (&v)[4] = val[i];
+        v[0] = acc[i][0].x; v[1] = acc[i][0].y; v[2] = acc[i][1].x; v[3] = acc[i][1].y;
+        if (!valid[i] || co >= p.Co) continue;
+        const size_t o = (((size_t)n * p.Ho + (hd * p.os + p.cls_oph[cls])) * p.Wo + (wd * p.os + p.cls_opw[cls])) * p.Co + co;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (bias && co + j < p.Co) v[j] += bias[(size_t)grp * p.b_group + co + j];
+            if (p.epi & EPI_RELU) v[j] = fmaxf(v[j], 0.f);
+        }
+        if ((p.Co & 3) == 0) {
+            if (p.epi & EPI_ACCUM) { const float4 old = ld4(y + o); v[0] += old.x; v[1] += old.y; v[2] += old.z; v[3] += old.w; }
+            st4(y + o, make_float4(v[0], v[1], v[2], v[3]));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (co + j < p.Co) { if (p.epi & EPI_ACCUM) v[j] += to_f(y[o + j]); put(y + o + j, v[j]); }
+        }
+    }
+    if (!stat) return;
+    // batch-norm statistics of the tile, from the values as stored: per channel the mean over its pixels and the sum of squared
+    // deviations from that mean (no cancellation, whatever the mean)
+    const int cnt = min(p.Wt, p.Wd - wd0) * min(p.Ht, p.Hd - hd0) * min(p.Nt, n_end - n0);
+    float s[4], m[4];
+    float* const red = fsm + warp * 16 + 4 * cg;
+    auto over_pixels = [&](float* out) {             // sums over the tile's pixels: 4 per thread, 8 lanes, 4 warps, in a fixed order
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+#pragma unroll
+            for (int d = 1; d < 8; d <<= 1) out[j] += __shfl_xor_sync(0xffffffffu, out[j], d);
+            if (g == 0) red[j] = out[j];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) out[j] = (fsm[4 * cg + j] + fsm[16 + 4 * cg + j]) + (fsm[32 + 4 * cg + j] + fsm[48 + 4 * cg + j]);
+        __syncthreads();
+    };
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        s[j] = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { val[i][j] = stored<T>(val[i][j]); if (valid[i]) s[j] += val[i][j]; }
+    }
+    over_pixels(s);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        m[j] = s[j] / (float)cnt; s[j] = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) if (valid[i]) { const float d = val[i][j] - m[j]; s[j] = fmaf(d, d, s[j]); }
+    }
+    over_pixels(s);
+    if (warp == 0 && g == 0) {
+        const int tiles = gridDim.x, groups = gridDim.z;
+        const size_t rec = (size_t)grp * tiles + blockIdx.x;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) if (co + j < p.Co) *(float2*)(stat + (rec * p.Co + co + j) * 2) = make_float2(m[j], s[j]);
+        if (blockIdx.y == 0 && cg == 0) stat[(size_t)groups * tiles * p.Co * 2 + rec] = (float)cnt;
+    }
+}
+
+struct FwParams {
+    int H, W, C, Ho, Wo, Co;
+    int step;                            // pixels of x between neighbours of the region (the stride for 1x1 layers, else 1)
+    int pad, hstep;                      // region origin = tile origin * hstep - pad
+    int RH, RW, ntaps, toff[9];          // region of a tile; per tap: offset inside it (floats)
+    int Wt, Ht, Nt, lw, lh, tiles_w, tiles_h, tiles;     // tile = Wt x Ht x Nt output pixels (powers of two)
+    int ngroup, splits, max_splits, ci_blocks;
+    int nslices, pps;                    // pixel slices of a tile, pixels per slice
+    int x_floats;
+};
+
+// grid = (splits, c_out blocks x c_in blocks, groups).  Thread = 4 c_out x 8 c_in of one tap, for one slice of every tile's
+// pixels.  dy is kept twice in shared memory ((d, d) pairs: the multiplier of a packed FMA), x as in fc_kernel.
+// part: [group][block][split][16 c_out][taps][8 * G c_in]
+template <typename T, int XS, int G, int RUN, bool VEC>
+__global__ void __launch_bounds__(FW_THREADS, 2) fw_kernel(const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ part_out,
+                                                           const __grid_constant__ FwParams p) {
+    extern __shared__ __align__(16) float fsm[];
+    float* const xs_ = fsm;
+    float* const ds_ = fsm + p.x_floats;                     // [pixel][16][2]
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int grp = blockIdx.z, cob = blockIdx.y / p.ci_blocks, cib = blockIdx.y % p.ci_blocks;
+    const int co0 = cob * FW_CO, ci0 = cib * FW_CI;
+    const int per_slice = p.ntaps * G * 4;
+    const int slice = tid / per_slice, rest = tid - slice * per_slice;
+    const int cog = rest & 3, ng = rest >> 2, tap = ng / G, half = ng - tap * G;
+    const bool active = slice < p.nslices;
+    const int npix = p.Wt * p.Ht * p.Nt;
+    float2 acc[4][4], comp[4][4];                            // [c_out][c_in pair]
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { acc[i][j] = make_float2(0.f, 0.f); comp[i][j] = make_float2(0.f, 0.f); }
+    const float* const xt = xs_ + (active ? p.toff[tap] : 0) + half * 8;
+    const float* const dt = ds_ + cog * 8;
+    const int per = (p.tiles + p.splits - 1) / p.splits;
+    const int tile_end = min(p.tiles, ((int)blockIdx.x + 1) * per);
+    for (int tile = blockIdx.x * per; tile < tile_end; ++tile) {
+        int tl = tile;
+        const int tw = tl % p.tiles_w; tl /= p.tiles_w;
+        const int th = tl % p.tiles_h, tn = tl / p.tiles_h;
+        const int n_end = (grp + 1) * p.ngroup, n0 = grp * p.ngroup + tn * p.Nt;
+        const int ho0 = th * p.Ht, wo0 = tw * p.Wt;
+        __syncthreads();                                     // the previous tile is consumed
+        load_region<T, VEC>(x, xs_, n0, n_end, p.Nt, ho0 * p.hstep - p.pad, wo0 * p.hstep - p.pad, p.RH, p.RW, p.step, p.H, p.W, p.C, ci0,
+                            G == 2 ? 4 : 2, warp, FW_THREADS / 32, lane);
+        cp_commit();
+        for (int i = tid; i < npix * 4; i += FW_THREADS) {
+            const int px = i >> 2, q = i & 3;
+            const int w = wo0 + (px & (p.Wt - 1)), h = ho0 + ((px >> p.lw) & (p.Ht - 1)), n = n0 + (px >> (p.lw + p.lh));
+            const bool ok = n < n_end && h < p.Ho && w < p.Wo;
+            const int c = co0 + 4 * q;
+            const T* s = dy + (((size_t)(ok ? n : 0) * p.Ho + (ok ? h : 0)) * p.Wo + (ok ? w : 0)) * p.Co;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if ((p.Co & 3) == 0) { if (ok && c < p.Co) v = ld4(s + c); }
+            else if (ok) {
+                v.x = c < p.Co ? to_f(s[c]) : 0.f; v.y = c + 1 < p.Co ? to_f(s[c + 1]) : 0.f;
+                v.z = c + 2 < p.Co ? to_f(s[c + 2]) : 0.f; v.w = c + 3 < p.Co ? to_f(s[c + 3]) : 0.f;
+            }
+            float* d = ds_ + px * 32 + q * 8;
+            *(float4*)d = make_float4(v.x, v.x, v.y, v.y);
+            *(float4*)(d + 4) = make_float4(v.z, v.z, v.w, v.w);
+        }
+        cp_wait<0>();
+        __syncthreads();
+        if (!active) continue;
+        for (int r = 0; r < p.pps; r += 16) {                // 16 pixels = one compensated step
+            float2 part[4][4];
+#pragma unroll
+            for (int rr = 0; rr < 16; rr += RUN) {
+                const int px = slice * p.pps + r + rr;
+                if (rr > 0 && r + rr >= p.pps) break;
+                const int pw = px & (p.Wt - 1), ph = (px >> p.lw) & (p.Ht - 1), pn = px >> (p.lw + p.lh);
+                const float* xp = xt + ((pn * p.RH + ph * XS) * p.RW + pw * XS) * PITCH;
+                const float* dp = dt + px * 32;
+#pragma unroll
+                for (int k = 0; k < RUN; ++k) {
+                    const float4 xa = *(const float4*)(xp + k * XS * PITCH), xc = *(const float4*)(xp + k * XS * PITCH + 4);
+                    const float4 d0 = *(const float4*)(dp + k * 32), d1 = *(const float4*)(dp + k * 32 + 4);
+                    const float2 xv[4] = {make_float2(xa.x, xa.y), make_float2(xa.z, xa.w), make_float2(xc.x, xc.y), make_float2(xc.z, xc.w)};
+                    const float2 dv[4] = {make_float2(d0.x, d0.y), make_float2(d0.z, d0.w), make_float2(d1.x, d1.y), make_float2(d1.z, d1.w)};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) part[i][j] = rr == 0 && k == 0 ? __fmul2_rn(dv[i], xv[j]) : __ffma2_rn(dv[i], xv[j], part[i][j]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 yv = __fadd2_rn(part[i][j], make_float2(-comp[i][j].x, -comp[i][j].y));
+                    const float2 t = __fadd2_rn(acc[i][j], yv);
+                    const float2 d = __fadd2_rn(t, make_float2(-acc[i][j].x, -acc[i][j].y));
+                    comp[i][j] = __fadd2_rn(d, make_float2(-yv.x, -yv.y));
+                    acc[i][j] = t;
+                }
+        }
+    }
+    // the slices' sums in slice order, then the CTA's partial matrix
+    __syncthreads();
+    const int nout = FW_CO * p.ntaps * 8 * G;
+    float* const red = fsm;                                  // [slice][16][taps][8 G]
+    if (active) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                *(float2*)(red + (size_t)slice * nout + ((cog * 4 + i) * p.ntaps + tap) * (8 * G) + half * 8 + 2 * j) = acc[i][j];
+    }
+    __syncthreads();
+    float* out = part_out + (((size_t)grp * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * nout;
+    for (int i = tid; i < nout; i += FW_THREADS) {
+        float s = 0.f;
+        for (int k = 0; k < p.nslices; ++k) s += red[(size_t)k * nout + i];
+        out[i] = s;
+    }
+}
+
+// dW[c_out][tap][c_in] = sum over the splits; 8 lanes per element take every 8th split, then a fixed tree.
+__global__ void __launch_bounds__(256) fw_reduce_kernel(const float* __restrict__ part, float* __restrict__ dw, int splits, int nout, int ntaps, int cw, int ci_blocks,
+                                                        int C, int Co, size_t w_group, bool accum) {
+    __shared__ float sh[8][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + tx, blk = blockIdx.y, grp = blockIdx.z;
+    const float* src = part + ((size_t)grp * gridDim.y + blk) * splits * nout + e;
+    float s = 0.f;
+    if (e < nout) {
+        int k = ty;
+        for (; k + 24 < splits; k += 32) {                   // four loads in flight
+            const float a = src[(size_t)k * nout], b = src[(size_t)(k + 8) * nout], c = src[(size_t)(k + 16) * nout], d = src[(size_t)(k + 24) * nout];
+            s += (a + b) + (c + d);
+        }
+        for (; k < splits; k += 8) s += src[(size_t)k * nout];
+    }
+    sh[ty][tx] = s;
+    __syncthreads();
+    if (ty != 0 || e >= nout) return;
+    s = ((sh[0][tx] + sh[1][tx]) + (sh[2][tx] + sh[3][tx])) + ((sh[4][tx] + sh[5][tx]) + (sh[6][tx] + sh[7][tx]));
+    const int co = (blk / ci_blocks) * FW_CO + e / (ntaps * cw), tap = e / cw % ntaps, ci = (blk % ci_blocks) * FW_CI + e % cw;
+    if (co >= Co || ci >= C) return;
+    float* d = dw + (size_t)grp * w_group + ((size_t)co * ntaps + tap) * C + ci;
+    *d = accum ? *d + s : s;
+}
+
+int ilog2(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
+
+// The largest power of two <= cap that wastes least when it tiles `n`.
+int best_tile(int n, int cap) {
+    int best = 1; long best_cover = n;
+    for (int t = 2; t <= cap; t *= 2) {
+        const long cover = (long)((n + t - 1) / t) * t;
+        if (t / 2 >= n) break;
+        if (cover <= best_cover + best_cover / 8) { best = t; if (cover < best_cover) best_cover = cover; }   // a wider tile may waste an eighth
+    }
+    return best;
+}
+
+struct Tile { int Wt, Ht, Nt; };
+Tile pick_tile(int H, int W, int pixels) {
+    Tile t;
+    t.Wt = best_tile(W, pixels < 32 ? pixels : 32);
+    t.Ht = best_tile(H, pixels / t.Wt);
+    t.Nt = pixels / (t.Wt * t.Ht);
+    return t;
+}
+
+constexpr size_t FC_SMEM_MAX = 200 * 1024;
+
+// Geometry of a forward (back == 0) or input-gradient launch over `groups` groups of g.N / groups images; false: not covered.
+bool plan_fc(const ConvGeom& g, int groups, bool back, FcParams& p) {
+    if (g.H * g.W == 1 || (g.R != 3 && g.R != 1) || (g.stride != 1 && g.stride != 2) || g.N % groups) return false;
+    p = FcParams{};
+    p.taps = g.R * g.R; p.back = back; p.ngroup = g.N / groups;
+    p.w_group = 0; p.b_group = 0;
+    int dh[9], dw[9];
+    if (!back) {
+        p.H = g.H; p.W = g.W; p.C = g.C; p.Ho = g.Ho; p.Wo = g.Wo; p.Co = g.Co; p.Hd = g.Ho; p.Wd = g.Wo; p.os = 1; p.xs = g.stride;
+        p.ncls = 1; p.cls_tap0[0] = 0; p.cls_tap0[1] = p.taps;
+        for (int t = 0; t < p.taps; ++t) { dh[t] = t / g.R - g.pad; dw[t] = t % g.R - g.pad; p.wtap[t] = t; }
+    } else {
+        // dx[h][w] = sum over taps of dy[(h + pad - r) / stride][(w + pad - s) / stride] . W[:][r][s][:]; a stride-2 layer by output parity
+        p.H = g.Ho; p.W = g.Wo; p.C = g.Co; p.Ho = g.H; p.Wo = g.W; p.Co = g.C; p.os = g.stride; p.xs = 1;
+        p.Hd = (g.H + g.stride - 1) / g.stride; p.Wd = (g.W + g.stride - 1) / g.stride;
+        if (g.stride == 2 && ((g.H | g.W) & 1)) return false;
+        int n = 0;
+        for (int ph = 0; ph < g.stride; ++ph) for (int pw = 0; pw < g.stride; ++pw) {
+            p.cls_oph[p.ncls] = ph; p.cls_opw[p.ncls] = pw; p.cls_tap0[p.ncls] = n;
+            for (int r = 0; r < g.R; ++r) for (int s = 0; s < g.R; ++s) {
+                const int a = ph + g.pad - r, b = pw + g.pad - s;
+                if (a % g.stride || b % g.stride) continue;
+                dh[n] = a / g.stride; dw[n] = b / g.stride; p.wtap[n] = r * g.R + s; ++n;
+            }
+            p.cls_tap0[++p.ncls] = n;
+        }
+    }
+    const Tile t = pick_tile(p.Hd, p.Wd, FC_PIX);
+    p.Wt = t.Wt; p.Ht = t.Ht; p.Nt = t.Nt; p.lw = ilog2(t.Wt); p.lh = ilog2(t.Ht);
+    p.tiles_w = (p.Wd + t.Wt - 1) / t.Wt; p.tiles_h = (p.Hd + t.Ht - 1) / t.Ht;
+    int maxt = 0;
+    for (int c = 0; c < p.ncls; ++c) {
+        const int a = p.cls_tap0[c], b = p.cls_tap0[c + 1];
+        int h0 = 0, h1 = 0, w0 = 0, w1 = 0;
+        for (int i = a; i < b; ++i) {
+            if (i == a || dh[i] < h0) h0 = dh[i];
+            if (i == a || dh[i] > h1) h1 = dh[i];
+            if (i == a || dw[i] < w0) w0 = dw[i];
+            if (i == a || dw[i] > w1) w1 = dw[i];
+        }
+        p.cls_h0[c] = h0; p.cls_w0[c] = w0;
+        p.cls_rh[c] = (t.Ht - 1) * p.xs + (h1 - h0) + 1; p.cls_rw[c] = (t.Wt - 1) * p.xs + (w1 - w0) + 1;
+        for (int i = a; i < b; ++i) p.toff[i] = ((dh[i] - h0) * p.cls_rw[c] + (dw[i] - w0)) * PITCH;
+        const int f = t.Nt * p.cls_rh[c] * p.cls_rw[c] * PITCH;
+        if (f > p.x_floats) p.x_floats = f;
+        if (b - a > maxt) maxt = b - a;
+    }
+    p.w_floats = maxt * 16 * PITCH;
+    const size_t one = (size_t)(p.x_floats + p.w_floats) * sizeof(float);
+    // two buffers as long as four CTAs (the register limit) or at least two fit on an SM
+    p.buffers = p.C > FC_KC && 2 * one <= 110 * 1024 ? 2 : 1;
+    return one <= FC_SMEM_MAX;
+}
+
+template <typename T, int NQ, bool VEC>
+void launch_fc(const void* x, const void* w, const float* bias, void* y, float* stat, const FcParams& p, int groups, cudaStream_t s) {
+    const size_t smem = (size_t)p.buffers * (p.x_floats + p.w_floats) * sizeof(float);
+    static bool attr = false;
+    if (!attr) { cudaFuncSetAttribute(fc_kernel<T, NQ, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FC_SMEM_MAX); attr = true; }
+    const int tiles = p.tiles_w * p.tiles_h * ((p.ngroup + p.Nt - 1) / p.Nt);
+    fc_kernel<T, NQ, VEC><<<dim3(tiles, (p.Co + FC_CO - 1) / FC_CO, groups * p.ncls), FC_THREADS, smem, s>>>((const T*)x, (const T*)w, bias, (T*)y, stat, p);
+}
+template <typename T>
+void dispatch_fc(const void* x, const void* w, const float* bias, void* y, float* stat, const FcParams& p, int groups, cudaStream_t s) {
+    // 16-byte (fp32) / 8-byte (bf16) pieces of a pixel's channels need a channel count that is a multiple of 4; the weight
+    // rows of the backward direction are read element by element
+    const bool vec = p.C % 4 == 0;
+    if (p.C <= 4) { if (vec) launch_fc<T, 1, true>(x, w, bias, y, stat, p, groups, s); else launch_fc<T, 1, false>(x, w, bias, y, stat, p, groups, s); }
+    else { if (vec) launch_fc<T, 4, true>(x, w, bias, y, stat, p, groups, s); else launch_fc<T, 4, false>(x, w, bias, y, stat, p, groups, s); }
+}
+
+// Weight gradient: 256 pixels per tile (128 for 3x3 stride 2, whose input region is four times its output).
+bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_t& smem) {
+    if (g.H * g.W == 1 || (g.R != 3 && g.R != 1) || (g.stride != 1 && g.stride != 2) || g.N % groups) return false;
+    p = FwParams{};
+    const Tile t = pick_tile(g.Ho, g.Wo, g.R == 3 && g.stride == 2 ? 128 : 256);
+    if (t.Wt < 4) return false;
+    run = t.Wt >= 8 ? 8 : 4;
+    p.H = g.H; p.W = g.W; p.C = g.C; p.Ho = g.Ho; p.Wo = g.Wo; p.Co = g.Co;
+    p.Wt = t.Wt; p.Ht = t.Ht; p.Nt = t.Nt; p.lw = ilog2(t.Wt); p.lh = ilog2(t.Ht);
+    p.tiles_w = (g.Wo + t.Wt - 1) / t.Wt; p.tiles_h = (g.Ho + t.Ht - 1) / t.Ht;
+    p.ngroup = g.N / groups;
+    p.tiles = p.tiles_w * p.tiles_h * ((p.ngroup + t.Nt - 1) / t.Nt);
+    p.pad = g.pad; p.hstep = g.stride; p.ntaps = g.R * g.R;
+    p.step = g.R == 1 ? g.stride : 1;
+    const int xs = g.R == 1 ? 1 : g.stride;
+    p.RH = (t.Ht - 1) * xs + g.R; p.RW = (t.Wt - 1) * xs + g.R;
+    for (int i = 0; i < p.ntaps; ++i) p.toff[i] = ((i / g.R) * p.RW + i % g.R) * PITCH;
+    G = g.C <= 8 ? 1 : 2;
+    const int npix = t.Wt * t.Ht * t.Nt, per_slice = p.ntaps * G * 4;
+    p.nslices = 1;
+    while (p.nslices * 2 * per_slice <= FW_THREADS && npix / (p.nslices * 2) >= run) p.nslices *= 2;
+    p.pps = npix / p.nslices;
+    p.ci_blocks = (g.C + FW_CI - 1) / FW_CI;
+    const int blocks = p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO) * groups;
+    // two CTAs per SM once around the device, each with at least one tile
+    int want = 2 * 148 / blocks;
+    if (want > p.tiles) want = p.tiles;
+    if (want < 1) want = 1;
+    p.max_splits = want;
+    const int per = (p.tiles + want - 1) / want;
+    p.splits = (p.tiles + per - 1) / per;
+    p.x_floats = t.Nt * p.RH * p.RW * PITCH;
+    smem = ((size_t)p.x_floats + (size_t)npix * 32) * sizeof(float);
+    const size_t red = (size_t)p.nslices * FW_CO * p.ntaps * 8 * G * sizeof(float);
+    if (red > smem) smem = red;
+    return smem <= FC_SMEM_MAX;
+}
+template <typename T, int XS, int G, int RUN, bool VEC>
+void launch_fw(const void* x, const void* dy, float* ws, const FwParams& p, int groups, size_t smem, cudaStream_t s) {
+    static bool attr = false;
+    if (!attr) { cudaFuncSetAttribute(fw_kernel<T, XS, G, RUN, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FC_SMEM_MAX); attr = true; }
+    fw_kernel<T, XS, G, RUN, VEC><<<dim3(p.splits, p.ci_blocks * ((p.Co + FW_CO - 1) / FW_CO), groups), FW_THREADS, smem, s>>>((const T*)x, (const T*)dy, ws, p);
+}
+template <typename T, int XS, int G, int RUN>
+void dispatch_fw_vec(const void* x, const void* dy, float* ws, const FwParams& p, int groups, size_t smem, cudaStream_t s) {
+    if (p.C % 4 == 0) launch_fw<T, XS, G, RUN, true>(x, dy, ws, p, groups, smem, s); else launch_fw<T, XS, G, RUN, false>(x, dy, ws, p, groups, smem, s);
+}
+template <typename T>
+void dispatch_fw(const void* x, const void* dy, float* ws, const FwParams& p, int xs, int G, int run, int groups, size_t smem, cudaStream_t s) {
+    if (xs == 1) {
+        if (G == 1) { if (run == 8) dispatch_fw_vec<T, 1, 1, 8>(x, dy, ws, p, groups, smem, s); else dispatch_fw_vec<T, 1, 1, 4>(x, dy, ws, p, groups, smem, s); }
+        else { if (run == 8) dispatch_fw_vec<T, 1, 2, 8>(x, dy, ws, p, groups, smem, s); else dispatch_fw_vec<T, 1, 2, 4>(x, dy, ws, p, groups, smem, s); }
+    } else {
+        if (G == 1) { if (run == 8) dispatch_fw_vec<T, 2, 1, 8>(x, dy, ws, p, groups, smem, s); else dispatch_fw_vec<T, 2, 1, 4>(x, dy, ws, p, groups, smem, s); }
+        else { if (run == 8) dispatch_fw_vec<T, 2, 2, 8>(x, dy, ws, p, groups, smem, s); else dispatch_fw_vec<T, 2, 2, 4>(x, dy, ws, p, groups, smem, s); }
+    }
+}
+
+}  // namespace
+
+bool fconv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
+                   float* stat, cudaStream_t s) {
+    FcParams p;
+    if ((epi & EPI_OUT_F32) || !plan_fc(g, groups, false, p)) return false;
+    p.epi = epi; p.w_group = w_group; p.b_group = b_group;
+    const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
+    Scope sc(KC_FMA_FWD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + g.Co * K + rows * g.Co), s);
+    if (dt) dispatch_fc<bf16>(x, w, bias, y, stat, p, groups, s); else dispatch_fc<float>(x, w, bias, y, stat, p, groups, s);
+    return true;
+}
+bool fconv_dgrad(int dt, const void* dy, const void* w, void* dx, const ConvGeom& g, int epi, int groups, size_t w_group, cudaStream_t s) {
+    FcParams p;
+    if (!plan_fc(g, groups, true, p)) return false;
+    p.epi = epi; p.w_group = w_group;
+    const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
+    Scope sc(KC_FMA_DGRAD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + g.Co * K + rows * g.Co), s);
+    if (dt) dispatch_fc<bf16>(dy, w, nullptr, dx, nullptr, p, groups, s); else dispatch_fc<float>(dy, w, nullptr, dx, nullptr, p, groups, s);
+    return true;
+}
+int fconv_stat_tiles(const ConvGeom& g, int groups) {
+    FcParams p;
+    return plan_fc(g, groups, false, p) ? p.tiles_w * p.tiles_h * ((p.ngroup + p.Nt - 1) / p.Nt) : 0;
+}
+size_t fconv_wgrad_workspace_elems(const ConvGeom& g, int groups) {
+    FwParams p; int G, run; size_t smem;
+    if (!plan_fw(g, groups, p, G, run, smem)) return 0;
+    // a window of the batch (fewer tiles) may use more splits than the whole batch, but never more than max_splits of the whole
+    return (size_t)groups * p.max_splits * p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO) * FW_CO * p.ntaps * 8 * G;
+}
+bool fconv_wgrad(int dt, const void* x, const void* dy, float* dw, float* ws, const ConvGeom& g, int groups, size_t w_group, bool accum, cudaStream_t s) {
+    FwParams p; int G, run; size_t smem;
+    if (!plan_fw(g, groups, p, G, run, smem)) return false;
+    const int xs = g.R == 1 ? 1 : g.stride, blocks = p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO), nout = FW_CO * p.ntaps * 8 * G;
+    const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
+    {
+        Scope sc(KC_FMA_WGRAD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + rows * g.Co) + 4.0 * K * g.Co, s);
+        if (dt) dispatch_fw<bf16>(x, dy, ws, p, xs, G, run, groups, smem, s); else dispatch_fw<float>(x, dy, ws, p, xs, G, run, groups, smem, s);
+    }
+    Scope sc(KC_SPLITK, 0.0, 4.0 * groups * (p.splits + 1) * blocks * nout, s);
+    fw_reduce_kernel<<<dim3((nout + 31) / 32, blocks, groups), 256, 0, s>>>(ws, dw, p.splits, nout, p.ntaps, 8 * G, p.ci_blocks, g.C, g.Co, w_group, accum);
+    return true;
+}
+
+}  // namespace fdg

@@ -68,6 +68,9 @@ struct Op {
     bool dgrad_needs_zero;                                   // some parity classes receive no gradient (1x1 stride 2)
     int stat_chunks;                                         // > 0: the forward epilogue also leaves batch-norm partial sums
                                                              //      (this many per worker) for the batch-norm that follows
+    int fstat_tiles;                                         // > 0: the same from the FMA kernel (fconv.cu): records of this many tiles per worker
+    int stat_buf;                                            // which of the module's two buffers holds them (both ops)
+    bool bn_from_conv;                                       // OP_BN: the convolution in front leaves such records (fp32: bnf_forward)
     tc::WgParams kw;
     std::vector<char*> a_ptrs, dy_ptrs;                      // the buffers the A / dY maps below were built for
     std::vector<char*> y_ptrs, dx_ptrs;                      // where the forward output / the input gradient can be written
@@ -95,11 +98,11 @@ struct Module {
     size_t stash_slot_bytes, wslot_bytes, grad_pool_bytes, in_slot_bytes;
     size_t ws_elems, scratch_elems, red_elems;
     char *in_ring, *stash, *gradpool, *d2, *wring, *wtring;
-    float *master, *grad, *ws, *scratch, *red, *cstat;
+    float *master, *grad, *ws, *scratch, *red, *cstat[2];
     bool fused_update;             // one kernel per step updates all parameters and emits the next weight version (both layouts)
     tc::UpdTable upd;
-    size_t cstat_elems;
-    int fused_stats_tensor, fused_stats_chunks;   // set by a conv that produced statistics partials for this tensor
+    size_t cstat_elems[2];
+    int fused_stats_tensor[2], fused_stats_chunks[2];   // per buffer: set by a conv that produced statistics partials for this tensor
     int64_t *tag_in, *tag_stash, *tag_d2, *tag_w, *trace;
     cudaStream_t stream;           // backward pass, loss, update (and everything in serial mode)
     cudaStream_t fstream;          // forward pass: independent of the backward pass of the same iteration (other batch)
@@ -326,7 +329,7 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
     m.ws_elems = 0; m.scratch_elems = 64; m.red_elems = 4; m.fwd_ws_elems = 0;
     for (Op& o : m.ops) {
         if (o.type == OP_BN) {
-            o.stats_off = soff; soff += align_up((size_t)ctx->n_workers * o.g.C * 2 * sizeof(float), 256);
+            o.stats_off = soff; soff += align_up((size_t)ctx->n_workers * o.g.C * (ctx->dt == 0 ? 4 : 2) * sizeof(float), 256);
             m.scratch_elems = std::max(m.scratch_elems, (size_t)128 * ctx->n_workers * o.g.C * 2);
             m.red_elems = std::max(m.red_elems, (size_t)ctx->n_workers * o.g.C * 2);
         }
@@ -340,19 +343,31 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             if (relu_bias_backward_supported(ctx->dt, o.g.Co)) m.scratch_elems = std::max(m.scratch_elems, relu_bias_backward_scratch_elems(o.g.Co));
         }
     }
-    // a tensor-core conv whose output goes straight into a batch-norm computes that batch-norm's statistics
-    // in its epilogue, if its 128-row tiles never straddle two workers
-    m.cstat_elems = 0;
+    // a conv whose output goes into a batch-norm takes that batch-norm's statistics along in its epilogue (tensor-core kernels: if
+    // their 128-row tiles never straddle two workers).  Between a block's last conv and its batch-norm come the shortcut's conv
+    // and batch-norm, so there are two buffers: 1 for a batch-norm that does not follow its conv directly.
+    m.cstat_elems[0] = m.cstat_elems[1] = 0;
     for (size_t i = 0; i + 1 < m.ops.size(); ++i) {
         Op& o = m.ops[i];
-        const Op& nx = m.ops[i + 1];
-        o.stat_chunks = 0;
-        if (o.type != OP_CONV || !(o.tc || o.stem_tc) || nx.type != OP_BN || nx.in != o.out || !bn_accepts_conv_partials(ctx->dt, o.g.Co)) continue;
-        int wt, ht, nt;
-        tc::pixel_tile(o.g.Ho, o.g.Wo, 128, &wt, &ht, &nt);
-        if (ctx->B % nt != 0) continue;
-        o.stat_chunks = (ctx->B / nt) * (o.g.Ho / ht) * (o.g.Wo / wt) * 4;
-        m.cstat_elems = std::max(m.cstat_elems, (size_t)ctx->n_workers * o.stat_chunks * o.g.Co * 2);
+        if (o.type != OP_CONV) continue;
+        size_t j = i + 1;
+        while (j < m.ops.size() && !(m.ops[j].type == OP_BN && m.ops[j].in == o.out)) ++j;
+        if (j == m.ops.size()) continue;
+        Op& bn = m.ops[j];
+        o.stat_buf = bn.stat_buf = j == i + 1 ? 0 : 1;
+        size_t& elems = m.cstat_elems[o.stat_buf];
+        if (o.tc || o.stem_tc) {
+            if (!bn_accepts_conv_partials(ctx->dt, o.g.Co)) continue;
+            int wt, ht, nt;
+            tc::pixel_tile(o.g.Ho, o.g.Wo, 128, &wt, &ht, &nt);
+            if (ctx->B % nt != 0) continue;
+            o.stat_chunks = (ctx->B / nt) * (o.g.Ho / ht) * (o.g.Wo / wt) * 4;
+            elems = std::max(elems, (size_t)ctx->n_workers * o.stat_chunks * o.g.Co * 2);
+        } else if (!o.stem && (bnf_supported(ctx->dt, o.g.Co) || bn_accepts_conv_partials(ctx->dt, o.g.Co))) {
+            o.fstat_tiles = fconv_stat_tiles(o.g, ctx->n_workers);
+            bn.bn_from_conv = o.fstat_tiles > 0;
+            elems = std::max(elems, (size_t)ctx->n_workers * o.fstat_tiles * (2 * o.g.Co + 1));
+        }
     }
     m.stash_slot_bytes = align_up(soff, 256);
     m.grad_pool_bytes = align_up(goff, 256);
@@ -414,7 +429,7 @@ bool tc_forward(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* y_base, 
     tc::KmParams p = o.kf;
     p.bias = o.bias ? wsmall(c, m, version, o.b_off) : nullptr;
     p.out = y_base; p.epi = o.relu ? EPI_RELU : 0; p.err = c->tc_err; p.sms = c->grid_sms;
-    p.stat_part = o.stat_chunks ? m.cstat : nullptr;
+    p.stat_part = o.stat_chunks ? m.cstat[o.stat_buf] : nullptr;
     p.n_base = wn.n0; p.N = wn.n0 + wn.n; p.tiles_n = (wn.n + p.Nt - 1) / p.Nt;
     const ConvGeom& g = o.g;
     double rows = (double)wn.n * g.Ho * g.Wo;
@@ -423,7 +438,7 @@ bool tc_forward(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* y_base, 
     const tc::KmMaps maps{&o.fa[ia], o.far.empty() ? nullptr : &o.far[ia], &o.fb[version % m.D], o.fbh.empty() ? nullptr : &o.fbh[version % m.D],
                           io >= 0 ? &o.fo[io] : nullptr};
     const bool ok = tc::run_km(maps, p, o.n_tile_f, s) == cudaSuccess;
-    if (ok && o.stat_chunks) { m.fused_stats_tensor = o.out; m.fused_stats_chunks = o.stat_chunks; }
+    if (ok && o.stat_chunks) { m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.stat_chunks; }
     return ok;
 }
 bool tc_dgrad(fdg_ctx* c, Module& m, const Op& o, char* dy_base, char* dx_base, int64_t version, bool accum, const Win& wn, cudaStream_t s) {
@@ -480,8 +495,8 @@ bool tc_stem_forward(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* y_b
     const double pix = (double)g.N * g.H * g.W;
     Scope sc(KC_FMA_FWD, 2.0 * pix * g.Co * 9 * g.C, 2.0 * pix * (g.C + g.Co), s);
     const bool ok = tc::run_stem_fw(o.sxr[ix], o.fo[io], g.H, g.W, g.N, g.Co, wbig(c, m, version, o.w_off), o.bias ? wsmall(c, m, version, o.b_off) : nullptr,
-                                    o.relu, o.stat_chunks ? m.cstat : nullptr, c->tc_err, c->grid_sms, s) == cudaSuccess;
-    if (ok && o.stat_chunks) { m.fused_stats_tensor = o.out; m.fused_stats_chunks = o.stat_chunks; }
+                                    o.relu, o.stat_chunks ? m.cstat[o.stat_buf] : nullptr, c->tc_err, c->grid_sms, s) == cudaSuccess;
+    if (ok && o.stat_chunks) { m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.stat_chunks; }
     return ok;
 }
 
@@ -508,7 +523,7 @@ void forward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int grou
     const int rep = c->R > 1 ? group : 0;               // worker `group` runs on its own weights w_{s,k}
     cudaStream_t s = m.fstream;
     const int dt = c->dt;
-    m.fused_stats_tensor = -1;
+    m.fused_stats_tensor[0] = m.fused_stats_tensor[1] = -1;
     auto T = [&](int id) { return P.tensor(id) + row_off(c, m.t[id], wn); };
     for (const Op& o : m.ops) {
         const TensorDesc& ti = m.t[o.in];
@@ -534,6 +549,12 @@ void forward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int grou
                     profile_detail(nullptr);
                     break;
                 }
+                if (o.fstat_tiles && fconv_forward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.bias ? wsmall(c, m, version, o.b_off, rep) : nullptr, T(o.out), g, epi,
+                                                   wn.nw, 0, 0, m.cstat[o.stat_buf], s)) {
+                    m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.fstat_tiles;
+                    profile_detail(nullptr);
+                    break;
+                }
                 conv_forward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.bias ? wsmall(c, m, version, o.b_off, rep) : nullptr, T(o.out), g, epi,
                              m.fwd_ws, m.fwd_ws_elems, s);
                 profile_detail(nullptr);
@@ -542,13 +563,30 @@ void forward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int grou
                 char tag[40];
                 std::snprintf(tag, sizeof tag, "%dx%dx%d%s%s", ti.h, ti.w, ti.c, o.has_res ? " +res" : "", o.relu ? " relu" : "");
                 profile_detail(tag);
-                const bool fused = m.fused_stats_tensor == o.in;
-                const float* part = fused ? m.cstat + (size_t)wn.w0 * m.fused_stats_chunks * ti.c * 2 : nullptr;
+                const bool fused = m.fused_stats_tensor[o.stat_buf] == o.in;
+                float* const cstat = m.cstat[o.stat_buf];
+                const int fused_chunks = m.fused_stats_chunks[o.stat_buf];
+                if (fused && o.bn_from_conv) {
+                    float* const st = P.stats(o) + (size_t)wn.w0 * ti.c * (dt == 0 ? 4 : 2);     // bnf_*: four floats per channel
+                    const long rpw = (long)c->B * ti.h * ti.w;
+                    if (dt == 0)
+                        bnf_forward((const float*)T(o.in), wsmall(c, m, version, o.gamma_off, rep), wsmall(c, m, version, o.beta_off, rep), 0,
+                                    o.has_res ? (const float*)T(o.in2) : nullptr, (float*)T(o.out), st, cstat, fused_chunks, wn.nw, rpw, ti.c, o.relu, s);
+                    else {
+                        bn_merge_tiles(cstat, st, fused_chunks, wn.nw, rpw, ti.c, s);
+                        bn_forward(dt, T(o.in), wsmall(c, m, version, o.gamma_off, rep), wsmall(c, m, version, o.beta_off, rep), o.has_res ? T(o.in2) : nullptr, T(o.out),
+                                   st, m.scratch_f, wn.nw, rpw, ti.c, o.relu, nullptr, -1, c->grid_sms, c->tc_err, s);
+                    }
+                    profile_detail(nullptr);
+                    m.fused_stats_tensor[o.stat_buf] = -1;
+                    break;
+                }
+                const float* part = fused ? cstat + (size_t)wn.w0 * fused_chunks * ti.c * 2 : nullptr;
                 bn_forward(dt, T(o.in), wsmall(c, m, version, o.gamma_off, rep), wsmall(c, m, version, o.beta_off, rep),
                            o.has_res ? T(o.in2) : nullptr, T(o.out), P.stats(o) + (size_t)wn.w0 * ti.c * 2, m.scratch_f, wn.nw,
-                           (long)c->B * ti.h * ti.w, ti.c, o.relu, part, fused ? m.fused_stats_chunks : 0, c->grid_sms, c->tc_err, s);
+                           (long)c->B * ti.h * ti.w, ti.c, o.relu, part, fused ? fused_chunks : 0, c->grid_sms, c->tc_err, s);
                 profile_detail(nullptr);
-                m.fused_stats_tensor = -1;
+                m.fused_stats_tensor[o.stat_buf] = -1;
                 break; }
             case OP_RELU: relu_forward(dt, T(o.in), T(o.out), n_out, s); break;
             case OP_POOL: maxpool_forward(dt, T(o.in), T(o.out), wn.n, ti.h, ti.w, ti.c, s); break;
@@ -621,6 +659,14 @@ void backward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t
                 std::snprintf(tag, sizeof tag, "%dx%dx%d%s%s", ti.h, ti.w, ti.c, o.has_res ? " +res" : "", o.relu ? " relu" : "");
                 profile_detail(tag);
                 char* gres = o.has_res ? G(o.in2) : nullptr;
+                if (o.bn_from_conv && dt == 0) {
+                    bnf_backward((const float*)T(o.in), (const float*)T(o.out), (const float*)gout, wsmall(c, m, version, o.gamma_off, rep),
+                                 wsmall(c, m, version, o.beta_off, rep), 0, P.stats(o) + (size_t)wn.w0 * ti.c * 4, (float*)gin, o.acc_in, (float*)gres, o.acc_in2,
+                                 mgrad + m.n_big + o.gamma_off, mgrad + m.n_big + o.beta_off, 0, m.scratch, wn.nw, (long)c->B * ti.h * ti.w, ti.c, o.relu,
+                                 o.relu && !o.has_res, acc_p, s);
+                    profile_detail(nullptr);
+                    break;
+                }
                 bn_backward(dt, T(o.in), T(o.out), gout, wsmall(c, m, version, o.gamma_off, rep), wsmall(c, m, version, o.beta_off, rep),
                             P.stats(o) + (size_t)wn.w0 * ti.c * 2, gin, o.acc_in, gres, o.acc_in2, mgrad + m.n_big + o.gamma_off,
                             mgrad + m.n_big + o.beta_off, m.red, m.scratch, wn.nw, (long)c->B * ti.h * ti.w, ti.c, o.relu, o.has_res, acc_p, c->grid_sms, c->tc_err, s);
@@ -1057,7 +1103,7 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
         m.scratch_f = (float*)get(m.scratch_elems * sizeof(float));
         m.fwd_ws = m.fwd_ws_elems ? (float*)get(m.fwd_ws_elems * sizeof(float)) : nullptr;
         m.head_scratch = m.head_elems ? (float*)get(m.head_elems * sizeof(float)) : nullptr;
-        m.cstat = m.cstat_elems ? (float*)get(m.cstat_elems * sizeof(float)) : nullptr;
+        for (int i = 0; i < 2; ++i) m.cstat[i] = m.cstat_elems[i] ? (float*)get(m.cstat_elems[i] * sizeof(float)) : nullptr;
         if (oom) break;
         m.tag_in = ctx->tags + tpos; tpos += 2 * (size_t)m.in_depth;
         m.tag_stash = ctx->tags + tpos; tpos += 2 * (size_t)m.D;

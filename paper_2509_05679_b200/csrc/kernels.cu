@@ -270,6 +270,8 @@ int wgrad_splits(const ConvGeom& g) {
     return s;
 }
 size_t wgrad_workspace_elems(const ConvGeom& g) {
+    const size_t direct = fconv_wgrad_workspace_elems(g, 1);
+    if (direct) return direct;
     int s = wgrad_splits(g);
     return s > 1 ? (size_t)s * g.Co * g.R * g.R * g.C : 0;
 }
@@ -321,6 +323,7 @@ static void conv_forward_t(const void* x, const void* w, const float* bias, void
     igemm_simt<T, M_FWD><<<grid, 256, 0, s>>>((const T*)x, (const T*)w, y, bias, nullptr, g, Mg, Ng, Kg, Kg, epi);
 }
 void conv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, float* ws, size_t ws_elems, cudaStream_t s) {
+    if (fconv_forward(dt, x, w, bias, y, g, epi, 1, 0, 0, nullptr, s)) return;
     if (dt) conv_forward_t<bf16>(x, w, bias, y, g, epi, ws, ws_elems, s); else conv_forward_t<float>(x, w, bias, y, g, epi, ws, ws_elems, s);
 }
 
@@ -332,6 +335,7 @@ static void conv_dgrad_t(const void* dy, const void* w, void* dx, const ConvGeom
     igemm_simt<T, M_DGRAD><<<grid, 256, 0, s>>>((const T*)dy, (const T*)w, dx, nullptr, nullptr, g, Mg, Ng, Kg, Kg, epi);
 }
 void conv_dgrad(int dt, const void* dy, const void* w, void* dx, const ConvGeom& g, int epi, cudaStream_t s) {
+    if (fconv_dgrad(dt, dy, w, dx, g, epi, 1, 0, s)) return;
     if (dt) conv_dgrad_t<bf16>(dy, w, dx, g, epi, s); else conv_dgrad_t<float>(dy, w, dx, g, epi, s);
 }
 
@@ -354,6 +358,7 @@ static void conv_wgrad_t(const void* x, const void* dy, float* dw, float* ws, co
     }
 }
 void conv_wgrad(int dt, const void* x, const void* dy, float* dw, float* ws, const ConvGeom& g, bool accum, cudaStream_t s) {
+    if (fconv_wgrad(dt, x, dy, dw, ws, g, 1, 0, accum, s)) return;
     if (dt) conv_wgrad_t<bf16>(x, dy, dw, ws, g, accum, s); else conv_wgrad_t<float>(x, dy, dw, ws, g, accum, s);
 }
 
@@ -1190,7 +1195,7 @@ void bn_forward(int dt, const void* x, const float* gamma, const float* beta, co
         if (conv_part) {
             Scope sc(KC_BN_FWD_STATS, 0.0, 8.0 * conv_chunks * nw * C, s);
             bnv_stats_final_tiles<<<dim3(C / 4, nw), 256, 0, s>>>(conv_part, stats, conv_chunks, nw, C, rpw);
-        } else {
+        } else if (conv_chunks >= 0) {
             { Scope sc(KC_BN_FWD_STATS, 0.0, 2.0 * total, s);
               BnsArgs r = a; r.part = scratch;
               bns_launch<0>(r, chunks, nw, s); }
@@ -1200,7 +1205,7 @@ void bn_forward(int dt, const void* x, const float* gamma, const float* beta, co
         Scope sc(KC_BN_FWD_APPLY, 0.0, 2.0 * total * (res ? 3 : 2), s);
         a.y = (bf16*)y; a.res = (const bf16*)res;
         if (res) { a.in[1] = (const bf16*)res; a.n_in = 2; }
-        a.reverse = conv_part ? 0 : 1;       // after a statistics pass of its own: x was just read front to back
+        a.reverse = conv_part || conv_chunks < 0 ? 0 : 1;       // after a statistics pass of its own: x was just read front to back
         bns_launch<2>(a, chunks, nw, s);
         return;
     }

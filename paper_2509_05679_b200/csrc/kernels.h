@@ -29,6 +29,17 @@ void conv_dgrad(int dt, const void* dy, const void* w, void* dx, const ConvGeom&
 // worker x batch axis, which is the worker average of Eq. dl_update (b) for P = 11^T/N.
 // accum: dw += (a second group of workers adds to the first group's result)
 void conv_wgrad(int dt, const void* x, const void* dy, float* dw, float* workspace, const ConvGeom& g, bool accum, cudaStream_t st);
+// The same three for convolutions (H * W > 1; 3x3 and 1x1, stride 1 and 2) in the packed-FMA kernels of fconv.cu; the
+// generic functions above take them where they apply.  `groups`: consecutive equal groups of images, each with its own weights
+// (w_group elements apart; biases b_group apart; weight gradients w_group apart).  false: shape not covered, nothing launched.
+bool   fconv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
+                     float* stat_or_null, cudaStream_t st);
+// Batch-norm statistics taken along by fconv_forward (groups = workers): per worker and pixel tile the channels' (mean, sum of
+// squared deviations), then the tiles' pixel counts: [groups][tiles][Co][2], [groups][tiles] floats.  0: shape not covered.
+int    fconv_stat_tiles(const ConvGeom& g, int groups);
+bool   fconv_dgrad(int dt, const void* dy, const void* w, void* dx, const ConvGeom& g, int epi, int groups, size_t w_group, cudaStream_t st);
+size_t fconv_wgrad_workspace_elems(const ConvGeom& g, int groups);
+bool   fconv_wgrad(int dt, const void* x, const void* dy, float* dw, float* workspace, const ConvGeom& g, int groups, size_t w_group, bool accum, cudaStream_t st);
 // db[c] = sum over rows of dy[row][c]; scratch: fp32 [64 * C]
 void bias_grad(int dt, const void* dy, float* db, float* scratch, long rows, int C, bool accum, cudaStream_t st);
 
@@ -68,6 +79,19 @@ void bn_forward(int dt, const void* x, const float* gamma, const float* beta, co
                 void* y, float* stats, float* scratch, int n_workers, long rows_per_worker, int C, bool relu,
                 const float* conv_part, int conv_chunks, int sms, int* err, cudaStream_t st);
 bool bn_accepts_conv_partials(int dt, int C);
+// conv_part == nullptr and conv_chunks < 0: `stats` already holds (mean, invstd) of every worker (bn_merge_tiles).
+
+// fp32 storage (bnorm.cu), C / 4 a power of two: forward from the records fconv_forward left (tile_part, see fconv_stat_tiles), backward in
+// two launches.  p_group / g_group: floats between the workers' parameters / parameter gradients (0: shared by all workers, gradients
+// summed over them).  mask_from_x: the forward output was bnf_forward's without a residual, so its sign can be recomputed from x.
+// scratch: as in bn_backward.  bn_merge_tiles: (mean, invstd) per worker and channel from such records, any storage type.
+bool bnf_supported(int dt, int C);
+void bn_merge_tiles(const float* tile_part, float* stats, int tiles, int nw, long rpw, int C, cudaStream_t st);
+void bnf_forward(const float* x, const float* gamma, const float* beta, size_t p_group, const float* res, float* y, float* stats, const float* tile_part,
+                 int tiles, int nw, long rpw, int C, bool relu, cudaStream_t st);
+void bnf_backward(const float* x, const float* out, const float* dout, const float* gamma, const float* beta, size_t p_group, const float* stats, float* dx,
+                  bool accum_dx, float* dres, bool accum_dres, float* dgamma, float* dbeta, size_t g_group, float* scratch, int nw, long rpw, int C, bool relu,
+                  bool mask_from_x, bool accum_params, cudaStream_t st);
 // dy_eff = dout * (out > 0 if relu).  dx (+)= BN backward of dy_eff; dres (+)= dy_eff;
 // dgamma, dbeta (fp32) = sums over all workers.  red: fp32 [n_workers][C][2] scratch for (sum dy, sum dy xhat).
 void bn_backward(int dt, const void* x, const void* out, const void* dout, const float* gamma, const float* beta,

@@ -1,0 +1,42 @@
+"""The packed-FMA convolutions (fconv.cu) and the fp32 batch-norm (bnorm.cu) at sizes where their tilings can go wrong: images that
+are no power of two, smaller than a tile or one pixel wider, channel counts that are no multiple of 16 or of 4, strides 1 and 2, 3x3 and
+1x1, batches that leave a pixel tile ragged.  ReLU-free networks (no kinks), one step against the oracle: loss, every gradient and
+the updated parameters.  Tolerances: the fp32 path's 1e-5 (tests/harness.py: max_rel_err) on parameters and, in the 2-norm, on
+gradients; the bf16 storage model's 2e-3 of tests/test_gpu_bf16.py for contractions of at most 144 terms and its 2e-2 beyond."""
+import pytest
+
+from paper_2509_05679_b200 import synth as sy
+from harness import run_parity
+
+pytestmark = pytest.mark.gpu
+
+# (H, W), first layer's width, kind, second layer's width, stride
+SHAPES = [((5, 7), 3, sy.CONV3X3, 5, 1), ((12, 20), 20, sy.CONV3X3, 24, 1), ((33, 9), 16, sy.CONV3X3, 8, 1), ((4, 4), 24, sy.CONV3X3, 40, 1),
+          ((2, 2), 8, sy.CONV3X3, 16, 1), ((6, 10), 18, sy.CONV3X3, 16, 2), ((32, 32), 16, sy.CONV3X3, 32, 2), ((16, 16), 32, sy.CONV1X1, 64, 2),
+          ((7, 11), 6, sy.CONV1X1, 12, 1), ((8, 8), 64, sy.CONV3X3, 64, 1), ((16, 1), 4, sy.CONV3X3, 16, 1)]
+
+
+def _net(shape, dtype, workers, batch, bn):
+    (h, w), c, kind, co, stride = shape
+    norm = lambda n: [(sy.BATCHNORM, n, n, 1, 0)] if bn else []
+    bias = 0 if bn else sy.FLAG_BIAS
+    layers = [(sy.CONV3X3, 3, c, 1, bias)] + norm(c) + [(kind, c, co, stride, bias)] + norm(co) + [(sy.GLOBAL_AVGPOOL, co, co, 1, 0), (sy.LINEAR, co, 10, 1, 1)]
+    return sy.Net("fconv", layers, [], h, w, 3, 10, workers, batch, 0.05, dtype)
+
+
+@pytest.mark.parametrize("bn", [False, True])
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: f"{s[0][0]}x{s[0][1]}-{s[1]}-{s[3]}-k{3 if s[2] == sy.CONV3X3 else 1}-s{s[4]}")
+def test_fp32(orc, shape, bn):
+    # per-channel sums of normalised values cancel: with batch-norm in front of the average pool only the parameters have a scale of their own
+    run_parity(orc, _net(shape, "fp32", 3, 5, bn), 2, param_tol=1e-5, loss_tol=1e-5, grad_tol=None if bn else 1e-5)
+
+
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: f"{s[0][0]}x{s[0][1]}-{s[1]}-{s[3]}-k{3 if s[2] == sy.CONV3X3 else 1}-s{s[4]}")
+def test_bf16_storage(orc, shape):
+    terms = shape[1] * (9 if shape[2] == sy.CONV3X3 else 1)
+    run_parity(orc, _net(shape, "bf16", 2, 4, False), 1, grad_tol=2e-3 if terms <= 144 else 2e-2, loss_tol=1e-4)
+
+
+@pytest.mark.parametrize("workers,batch", [(1, 1), (2, 130), (5, 3)])
+def test_batch_sizes(orc, workers, batch):
+    run_parity(orc, _net(((8, 8), 16, sy.CONV3X3, 32, 2), "fp32", workers, batch, True), 2, param_tol=1e-5, loss_tol=1e-5)
