@@ -22,11 +22,14 @@
 #include "kernels.h"
 #include "tc_gemm.h"
 
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
+#include <thread>
 #include <vector>
 
 using namespace fdg;
@@ -125,7 +128,7 @@ struct fdg_ctx {
     int R;                         // weight replicas per module: 1 (exact averaging, P = 11^T/N), or n_workers (general mixing matrix)
     std::vector<double> P;         // R x R mixing matrix (row-major) when R > 1
     float* P_dev;
-    int in_h, in_w, in_c;
+    int in_h, in_w, in_c, device;
     float lr;
     int64_t t;
     bool have_params;
@@ -161,6 +164,76 @@ fdg_status fail(fdg_ctx* c, fdg_status s, const char* fmt, ...) {
 #define CK(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) return fail(ctx, FDG_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e_)); } while (0)
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
+// Pinned staging memory and copy streams for reading parameters back, shared by the contexts of the process: allocated with the first
+// context, given back with the last.  One reader at a time (the lock); LANES x LANE_BYTES = 8 MB whatever the networks are.
+struct HostReader {
+    static constexpr int LANES = 8;
+    static constexpr size_t LANE_BYTES = 1 << 20;
+    std::mutex mu;
+    int users = 0, device = -1;
+    char* pinned = nullptr;
+    cudaStream_t stream[LANES] = {};
+    void acquire() {
+        std::lock_guard<std::mutex> lk(mu);
+        if (users++ > 0) return;
+        cudaGetDevice(&device);
+        bool ok = cudaMallocHost((void**)&pinned, LANES * LANE_BYTES) == cudaSuccess;
+        for (int i = 0; ok && i < LANES; ++i) ok = cudaStreamCreateWithFlags(&stream[i], cudaStreamNonBlocking) == cudaSuccess;
+        if (!ok) { cudaGetLastError(); drop(); }            // plain copies then (see read_floats)
+    }
+    void release() {
+        std::lock_guard<std::mutex> lk(mu);
+        if (--users == 0) drop();
+    }
+    void drop() {
+        for (cudaStream_t& s : stream) { if (s) cudaStreamDestroy(s); s = nullptr; }
+        if (pinned) cudaFreeHost(pinned);
+        pinned = nullptr;
+    }
+};
+HostReader g_reader;
+
+// Device floats [src, src + n) -> pieces of a host array.  piece(off, count, from) copies count floats that start at element off.
+// What this costs is the host side: a plain copy into pageable memory runs through the driver's single staging thread, and the
+// caller's fresh array takes a page fault per 4 KB (11 M parameters: 14-16 ms).  Several threads each take the next chunk, copy it to a
+// pinned lane of their own on a stream of their own (DMA at the link's rate) and move it out while the other lanes' copies run.
+template <typename F>
+cudaError_t read_floats(const float* src, size_t n, int device, F piece) {
+    constexpr size_t chunk = HostReader::LANE_BYTES / sizeof(float);
+    std::lock_guard<std::mutex> lk(g_reader.mu);
+    const size_t jobs = (n + chunk - 1) / chunk;
+    if (!g_reader.pinned || g_reader.device != device) {
+        std::vector<float> h(chunk);
+        for (size_t j = 0; j < jobs; ++j) {
+            const size_t off = j * chunk, cnt = n - off < chunk ? n - off : chunk;
+            cudaError_t e = cudaMemcpy(h.data(), src + off, cnt * sizeof(float), cudaMemcpyDeviceToHost);
+            if (e != cudaSuccess) return e;
+            piece(off, cnt, h.data());
+        }
+        return cudaSuccess;
+    }
+    std::atomic<size_t> next{0};
+    std::atomic<int> err{(int)cudaSuccess};
+    auto work = [&](int lane) {
+        float* const buf = (float*)(g_reader.pinned + lane * HostReader::LANE_BYTES);
+        if (lane > 0) cudaSetDevice(device);
+        for (size_t j; (j = next.fetch_add(1)) < jobs && err.load() == (int)cudaSuccess;) {
+            const size_t off = j * chunk, cnt = n - off < chunk ? n - off : chunk;
+            cudaError_t e = cudaMemcpyAsync(buf, src + off, cnt * sizeof(float), cudaMemcpyDeviceToHost, g_reader.stream[lane]);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(g_reader.stream[lane]);
+            if (e != cudaSuccess) { err.store((int)e); break; }
+            piece(off, cnt, buf);
+        }
+    };
+    // a thread is worth starting from two chunks of its own
+    const int extra = (int)std::min<size_t>(HostReader::LANES - 1, jobs / 2 > 0 ? jobs / 2 - 1 : 0);
+    std::vector<std::thread> threads;
+    try { for (int i = 1; i <= extra; ++i) threads.emplace_back(work, i); } catch (...) {}      // fewer threads then
+    work(0);
+    for (std::thread& t : threads) t.join();
+    return (cudaError_t)err.load();
+}
 
 void* default_alloc(size_t bytes, void*) { void* p = nullptr; return cudaMalloc(&p, bytes) == cudaSuccess ? p : nullptr; }
 void default_free(void* p, void*) { cudaFree(p); }
@@ -971,6 +1044,7 @@ const char* fdg_last_error(const fdg_ctx* ctx) { return ctx ? ctx->err.c_str() :
 void fdg_destroy(fdg_ctx* ctx) {
     if (!ctx) return;
     cudaDeviceSynchronize();
+    g_reader.release();
     for (Module& m : ctx->mod) {
         if (m.done) cudaEventDestroy(m.done);
         if (m.fdone) cudaEventDestroy(m.fdone);
@@ -1035,7 +1109,9 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
     ctx->device_bytes = 0;
     ctx->ingested = nullptr;
     ctx->loss_ready = nullptr;
+    ctx->device = dev;
     ctx->mod.resize(K);
+    g_reader.acquire();                    // released by fdg_destroy, which every error path below goes through
     auto bail = [&](fdg_status s, const std::string& msg) { g_create_error = msg; fdg_destroy(ctx); return s; };
 
     int h = opt->in_h, w = opt->in_w, c = opt->in_c;
@@ -1316,24 +1392,29 @@ static fdg_status gather(fdg_ctx* ctx, bool grads, int worker, float* host_out, 
     { fdg_status es = check_device_error(ctx); if (es != FDG_OK) return es; }
     for (Module& m : ctx->mod) {
         const size_t n = npar(m);
-        std::vector<float> h(n, 0.f);
-        if (!grads || m.had_bwd) {
-            if (grads && worker < 0 && ctx->R > 1) {
-                // (1/N) sum_s g_{s,k}, accumulated in double
-                std::vector<float> one(n);
-                std::vector<double> acc(n, 0.0);
-                for (int r = 0; r < ctx->R; ++r) {
-                    CK(cudaMemcpy(one.data(), m.grad + (size_t)r * n, n * sizeof(float), cudaMemcpyDeviceToHost));
-                    for (size_t i = 0; i < n; ++i) acc[i] += one[i];
-                }
-                for (size_t i = 0; i < n; ++i) h[i] = (float)(acc[i] / ctx->R);
-            } else {
-                const int r = (ctx->R > 1 && worker > 0) ? worker : 0;       // one copy: every worker has the same
-                CK(cudaMemcpy(h.data(), (grads ? m.grad : m.master) + (size_t)r * n, n * sizeof(float), cudaMemcpyDeviceToHost));
+        // internal elements [off, off + cnt) -> their places in the canonical vector (m.segs is in internal order within each segment class)
+        auto scatter = [&](size_t off, size_t cnt, const float* from) {
+            for (const Segment& s : m.segs) {
+                const size_t at = (s.big ? 0 : m.n_big) + s.internal, lo = std::max(at, off), hi = std::min(at + s.count, off + cnt);
+                if (lo < hi) std::memcpy(host_out + s.canon + (lo - at), from + (lo - off), (hi - lo) * sizeof(float));
             }
+        };
+        if (grads && !m.had_bwd) {
+            for (const Segment& s : m.segs) std::memset(host_out + s.canon, 0, s.count * sizeof(float));
+        } else if (grads && worker < 0 && ctx->R > 1) {
+            // (1/N) sum_s g_{s,k}, accumulated in double
+            std::vector<float> one(n);
+            std::vector<double> acc(n, 0.0);
+            for (int r = 0; r < ctx->R; ++r) {
+                CK(cudaMemcpy(one.data(), m.grad + (size_t)r * n, n * sizeof(float), cudaMemcpyDeviceToHost));
+                for (size_t i = 0; i < n; ++i) acc[i] += one[i];
+            }
+            for (size_t i = 0; i < n; ++i) one[i] = (float)(acc[i] / ctx->R);
+            scatter(0, n, one.data());
+        } else {
+            const int r = (ctx->R > 1 && worker > 0) ? worker : 0;       // one copy: every worker has the same
+            CK(read_floats((grads ? m.grad : m.master) + (size_t)r * n, n, ctx->device, scatter));
         }
-        for (const Segment& s : m.segs)
-            std::memcpy(host_out + s.canon, h.data() + (s.big ? 0 : m.n_big) + s.internal, s.count * sizeof(float));
     }
     if (count) *count = ctx->n_params;
     return FDG_OK;
