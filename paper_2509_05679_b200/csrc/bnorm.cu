@@ -7,6 +7,7 @@
 // it visits; a CTA owns a contiguous row range of one worker.  Used when C / 4 is a power of two <= 256.
 // Every sum has a fixed order.
 #include "kernels.h"
+#include "launch.h"
 
 #include <cuda_bf16.h>
 
@@ -233,7 +234,7 @@ void bn_merge_tiles(const float* tile_part, float* stats, int tiles, int nw, lon
     int nc = 1;                                  // channels per block: a power of two that divides C
     while (nc < 64 && C % (2 * nc) == 0) nc *= 2;
     Scope sc(KC_BN_FWD_STATS, 0.0, 8.0 * tiles * nw * C, s);
-    bn_merge_tiles_k<<<dim3(C / nc, nw), BT, 0, s>>>(tile_part, stats, tiles, C, nc, rpw);
+    klaunch(bn_merge_tiles_k, dim3(C / nc, nw), BT, 0, s, tile_part, stats, tiles, C, nc, rpw);
 }
 
 void bnf_forward(const float* x, const float* gamma, const float* beta, size_t p_group, const float* res, float* y, float* stats, const float* tile_part,
@@ -242,7 +243,7 @@ void bnf_forward(const float* x, const float* gamma, const float* beta, size_t p
     a.x = x; a.gamma = gamma; a.beta = beta; a.p_group = p_group; a.res = res; a.y = y; a.stats = stats; a.tile_part = tile_part; a.tiles = tiles;
     a.rpw = rpw; a.C = C; a.relu = relu;
     Scope sc(KC_BN_FWD_APPLY, 0.0, 4.0 * nw * rpw * C * (res ? 3 : 2), s);
-    bnf_kernel<0><<<dim3(bnf_chunks(nw, rpw, C), nw), BT, 0, s>>>(a);
+    klaunch(bnf_kernel<0>, dim3(bnf_chunks(nw, rpw, C), nw), BT, 0, s, a);
 }
 
 void bnf_backward(const float* x, const float* out, const float* dout, const float* gamma, const float* beta, size_t p_group, const float* stats, float* dx,
@@ -256,9 +257,9 @@ void bnf_backward(const float* x, const float* out, const float* dout, const flo
     const double total = (double)nw * rpw * C;
     const int reads = 2 + (relu && !mask_from_x ? 1 : 0);
     { Scope sc(KC_BN_BWD_REDUCE, 0.0, 4.0 * total * reads, s);
-      bnf_kernel<1><<<grid, BT, 0, s>>>(a); }
+      klaunch(bnf_kernel<1>, grid, BT, 0, s, a); }
     Scope sc(KC_BN_BWD_APPLY, 0.0, 4.0 * total * (reads + 1 + (accum_dx ? 1 : 0) + (dres ? (accum_dres ? 2 : 1) : 0)), s);
-    bnf_kernel<2><<<grid, BT, 0, s>>>(a);
+    klaunch(bnf_kernel<2>, grid, BT, 0, s, a);
 }
 
 }  // namespace fdg

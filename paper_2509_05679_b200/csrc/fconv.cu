@@ -9,13 +9,13 @@
 //
 // Arithmetic: packed fp32 (fma.rn.f32x2: 65.6 TFLOP/s on a B200 where scalar fma gives 46.7).  The pairs lie along the
 // contraction (channels 2i and 2i + 1) in fc_kernel and along c_in in fw_kernel, so that operands come out of NHWC data as
-// 16-byte vectors without shuffling.  Chains of at most 16 products are added to a compensated (Kahan) running sum, as in
-// igemm_simt: the rounding error of a long contraction stays at a few ulps.
+// 16-byte vectors without shuffling.  Chains of at most 16 products are added to a compensated (Kahan) running sum, so the rounding error of a long contraction stays at a few ulps.
 //
 // What bounds them: the FMA pipe (fc_kernel issues 32 packed FMAs for eight 16-byte shared loads, fw_kernel 16 for four).
 // The implicit-GEMM kernel they replace fetched every operand element by itself with two integer divisions and reached
 // 2.5-9 TFLOP/s on the ResNet-20 layers.
 #include "kernels.h"
+#include "launch.h"
 
 #include <cuda_bf16.h>
 
@@ -61,8 +61,8 @@ __device__ __forceinline__ void st4(bf16* p, float4 v) {
 // pixel is (h0, w0) and whose neighbours are `step` pixels apart in the tensor; zeros outside the image, past image n_end
 // and past channel C.  A warp takes whole rows, so that the loop has no division.
 // VEC: C is a multiple of 4 (16-byte fp32 / 8-byte bf16 pieces); fp32 pieces travel by cp.async.
-template <typename T, bool VEC>
-__device__ __forceinline__ void load_region(const T* __restrict__ x, float* dst, int n0, int n_end, int nimg, int h0, int w0, int RH, int RW, int step,
+template <typename T>
+__device__ __forceinline__ void load_region(const bool VEC, const T* __restrict__ x, float* dst, int n0, int n_end, int nimg, int h0, int w0, int RH, int RW, int step,
                                             int H, int W, int C, int c0, int nq, int warp, int nwarps, int lane) {
     int ni = 0, rh = warp;
     while (rh >= RH) { rh -= RH; ++ni; }
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(FC_THREADS, 4) fc_kernel(const T* __restrict__
     const int chunks = t1 > t0 ? (p.C + FC_KC - 1) / FC_KC : 0;
     auto fetch = [&](int c, int buf) {
         float* xs_ = fsm + (size_t)buf * (p.x_floats + p.w_floats);
-        load_region<T, VEC>(x, xs_, n0, n_end, p.Nt, h0, w0, RH, RW, 1, p.H, p.W, p.C, c * FC_KC, NQ, warp, FC_THREADS / 32, lane);
+        load_region<T>(VEC, x, xs_, n0, n_end, p.Nt, h0, w0, RH, RW, 1, p.H, p.W, p.C, c * FC_KC, NQ, warp, FC_THREADS / 32, lane);
         load_weights<T, VEC>(w, xs_ + p.x_floats, p, t0, t1, co0, c * FC_KC, NQ, tid);
         cp_commit();
     };
@@ -256,7 +256,10 @@ __global__ void __launch_bounds__(FC_THREADS, 4) fc_kernel(const T* __restrict__
             if (bias && co + j < p.Co) v[j] += bias[(size_t)grp * p.b_group + co + j];
             if (p.epi & EPI_RELU) v[j] = fmaxf(v[j], 0.f);
         }
-        if ((p.Co & 3) == 0) {
+        if (p.epi & EPI_OUT_F32) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) if (co + j < p.Co) ((float*)y)[o + j] = v[j];
+        } else if ((p.Co & 3) == 0) {
             if (p.epi & EPI_ACCUM) { const float4 old = ld4(y + o); v[0] += old.x; v[1] += old.y; v[2] += old.z; v[3] += old.w; }
             st4(y + o, make_float4(v[0], v[1], v[2], v[3]));
         } else {
@@ -320,7 +323,7 @@ struct FwParams {
 // grid = (splits, c_out blocks x c_in blocks, groups).  Thread = 4 c_out x 8 c_in of one tap, for one slice of every tile's
 // pixels.  dy is kept twice in shared memory ((d, d) pairs: the multiplier of a packed FMA), x as in fc_kernel.
 // part: [group][block][split][16 c_out][taps][8 * G c_in]
-template <typename T, int XS, int G, int RUN, bool VEC>
+template <typename T, int XS, int G, int RUN>
 __global__ void __launch_bounds__(FW_THREADS, 2) fw_kernel(const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ part_out,
                                                            const __grid_constant__ FwParams p) {
     extern __shared__ __align__(16) float fsm[];
@@ -350,7 +353,7 @@ __global__ void __launch_bounds__(FW_THREADS, 2) fw_kernel(const T* __restrict__
         const int n_end = (grp + 1) * p.ngroup, n0 = grp * p.ngroup + tn * p.Nt;
         const int ho0 = th * p.Ht, wo0 = tw * p.Wt;
         __syncthreads();                                     // the previous tile is consumed
-        load_region<T, VEC>(x, xs_, n0, n_end, p.Nt, ho0 * p.hstep - p.pad, wo0 * p.hstep - p.pad, p.RH, p.RW, p.step, p.H, p.W, p.C, ci0,
+        load_region<T>((p.C & 3) == 0, x, xs_, n0, n_end, p.Nt, ho0 * p.hstep - p.pad, wo0 * p.hstep - p.pad, p.RH, p.RW, p.step, p.H, p.W, p.C, ci0,
                             G == 2 ? 4 : 2, warp, FW_THREADS / 32, lane);
         cp_commit();
         for (int i = tid; i < npix * 4; i += FW_THREADS) {
@@ -477,7 +480,7 @@ constexpr size_t FC_SMEM_MAX = 200 * 1024;
 
 // Geometry of a forward (back == 0) or input-gradient launch over `groups` groups of g.N / groups images; false: not covered.
 bool plan_fc(const ConvGeom& g, int groups, bool back, FcParams& p) {
-    if (g.H * g.W == 1 || (g.R != 3 && g.R != 1) || (g.stride != 1 && g.stride != 2) || g.N % groups) return false;
+    if ((g.H * g.W == 1 && g.R == 1) || (g.R != 3 && g.R != 1) || (g.stride != 1 && g.stride != 2) || g.N % groups) return false;
     p = FcParams{};
     p.taps = g.R * g.R; p.back = back; p.ngroup = g.N / groups;
     p.w_group = 0; p.b_group = 0;
@@ -535,7 +538,7 @@ void launch_fc(const void* x, const void* w, const float* bias, void* y, float* 
     static bool attr = false;
     if (!attr) { cudaFuncSetAttribute(fc_kernel<T, NQ, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FC_SMEM_MAX); attr = true; }
     const int tiles = p.tiles_w * p.tiles_h * ((p.ngroup + p.Nt - 1) / p.Nt);
-    fc_kernel<T, NQ, VEC><<<dim3(tiles, (p.Co + FC_CO - 1) / FC_CO, groups * p.ncls), FC_THREADS, smem, s>>>((const T*)x, (const T*)w, bias, (T*)y, stat, p);
+    klaunch(fc_kernel<T, NQ, VEC>, dim3(tiles, (p.Co + FC_CO - 1) / FC_CO, groups * p.ncls), FC_THREADS, smem, s, (const T*)x, (const T*)w, bias, (T*)y, stat, p);
 }
 template <typename T>
 void dispatch_fc(const void* x, const void* w, const float* bias, void* y, float* stat, const FcParams& p, int groups, cudaStream_t s) {
@@ -548,11 +551,11 @@ void dispatch_fc(const void* x, const void* w, const float* bias, void* y, float
 
 // Weight gradient: 256 pixels per tile (128 for 3x3 stride 2, whose input region is four times its output).
 bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_t& smem) {
-    if (g.H * g.W == 1 || (g.R != 3 && g.R != 1) || (g.stride != 1 && g.stride != 2) || g.N % groups) return false;
+    if ((g.H * g.W == 1 && g.R == 1) || (g.R != 3 && g.R != 1) || (g.stride != 1 && g.stride != 2) || g.N % groups) return false;
+  for (int pixels = g.R == 3 && g.stride == 2 ? 128 : 256; pixels >= 32; pixels /= 2) {        // smaller tiles where the halo of tiny images outgrows shared memory
     p = FwParams{};
-    const Tile t = pick_tile(g.Ho, g.Wo, g.R == 3 && g.stride == 2 ? 128 : 256);
-    if (t.Wt < 4) return false;
-    run = t.Wt >= 8 ? 8 : 4;
+    const Tile t = pick_tile(g.Ho, g.Wo, pixels);
+    run = t.Wt >= 8 ? 8 : (t.Wt >= 4 ? 4 : 1);
     p.H = g.H; p.W = g.W; p.C = g.C; p.Ho = g.Ho; p.Wo = g.Wo; p.Co = g.Co;
     p.Wt = t.Wt; p.Ht = t.Ht; p.Nt = t.Nt; p.lw = ilog2(t.Wt); p.lh = ilog2(t.Ht);
     p.tiles_w = (g.Wo + t.Wt - 1) / t.Wt; p.tiles_h = (g.Ho + t.Ht - 1) / t.Ht;
@@ -581,35 +584,38 @@ bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_
     smem = ((size_t)p.x_floats + (size_t)npix * 32) * sizeof(float);
     const size_t red = (size_t)p.nslices * FW_CO * p.ntaps * 8 * G * sizeof(float);
     if (red > smem) smem = red;
-    return smem <= FC_SMEM_MAX;
-}
-template <typename T, int XS, int G, int RUN, bool VEC>
-void launch_fw(const void* x, const void* dy, float* ws, const FwParams& p, int groups, size_t smem, cudaStream_t s) {
-    static bool attr = false;
-    if (!attr) { cudaFuncSetAttribute(fw_kernel<T, XS, G, RUN, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FC_SMEM_MAX); attr = true; }
-    fw_kernel<T, XS, G, RUN, VEC><<<dim3(p.splits, p.ci_blocks * ((p.Co + FW_CO - 1) / FW_CO), groups), FW_THREADS, smem, s>>>((const T*)x, (const T*)dy, ws, p);
+    if (smem <= FC_SMEM_MAX) return true;
+  }
+    return false;
 }
 template <typename T, int XS, int G, int RUN>
-void dispatch_fw_vec(const void* x, const void* dy, float* ws, const FwParams& p, int groups, size_t smem, cudaStream_t s) {
-    if (p.C % 4 == 0) launch_fw<T, XS, G, RUN, true>(x, dy, ws, p, groups, smem, s); else launch_fw<T, XS, G, RUN, false>(x, dy, ws, p, groups, smem, s);
+void launch_fw(const void* x, const void* dy, float* ws, const FwParams& p, int groups, size_t smem, cudaStream_t s) {
+    static bool attr = false;
+    if (!attr) { cudaFuncSetAttribute(fw_kernel<T, XS, G, RUN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FC_SMEM_MAX); attr = true; }
+    klaunch(fw_kernel<T, XS, G, RUN>, dim3(p.splits, p.ci_blocks * ((p.Co + FW_CO - 1) / FW_CO), groups), FW_THREADS, smem, s, (const T*)x, (const T*)dy, ws, p);
+}
+template <typename T, int XS, int G>
+void dispatch_fw_run(const void* x, const void* dy, float* ws, const FwParams& p, int run, int groups, size_t smem, cudaStream_t s) {
+    if (run == 8) launch_fw<T, XS, G, 8>(x, dy, ws, p, groups, smem, s);
+    else if (run == 4) launch_fw<T, XS, G, 4>(x, dy, ws, p, groups, smem, s);
+    else launch_fw<T, XS, G, 1>(x, dy, ws, p, groups, smem, s);
 }
 template <typename T>
 void dispatch_fw(const void* x, const void* dy, float* ws, const FwParams& p, int xs, int G, int run, int groups, size_t smem, cudaStream_t s) {
-    if (xs == 1) {
-        if (G == 1) { if (run == 8) dispatch_fw_vec<T, 1, 1, 8>(x, dy, ws, p, groups, smem, s); else dispatch_fw_vec<T, 1, 1, 4>(x, dy, ws, p, groups, smem, s); }
-        else { if (run == 8) dispatch_fw_vec<T, 1, 2, 8>(x, dy, ws, p, groups, smem, s); else dispatch_fw_vec<T, 1, 2, 4>(x, dy, ws, p, groups, smem, s); }
-    } else {
-        if (G == 1) { if (run == 8) dispatch_fw_vec<T, 2, 1, 8>(x, dy, ws, p, groups, smem, s); else dispatch_fw_vec<T, 2, 1, 4>(x, dy, ws, p, groups, smem, s); }
-        else { if (run == 8) dispatch_fw_vec<T, 2, 2, 8>(x, dy, ws, p, groups, smem, s); else dispatch_fw_vec<T, 2, 2, 4>(x, dy, ws, p, groups, smem, s); }
-    }
+    if (xs == 1) { if (G == 1) dispatch_fw_run<T, 1, 1>(x, dy, ws, p, run, groups, smem, s); else dispatch_fw_run<T, 1, 2>(x, dy, ws, p, run, groups, smem, s); }
+    else { if (G == 1) dispatch_fw_run<T, 2, 1>(x, dy, ws, p, run, groups, smem, s); else dispatch_fw_run<T, 2, 2>(x, dy, ws, p, run, groups, smem, s); }
 }
 
 }  // namespace
 
+bool fconv_supported(const ConvGeom& g) {
+    FcParams p; FwParams q; int G, run; size_t smem;
+    return plan_fc(g, 1, false, p) && plan_fc(g, 1, true, p) && plan_fw(g, 1, q, G, run, smem);
+}
 bool fconv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
                    float* stat, cudaStream_t s) {
     FcParams p;
-    if ((epi & EPI_OUT_F32) || !plan_fc(g, groups, false, p)) return false;
+    if (!plan_fc(g, groups, false, p)) return false;
     p.epi = epi; p.w_group = w_group; p.b_group = b_group;
     const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
     Scope sc(KC_FMA_FWD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + g.Co * K + rows * g.Co), s);
@@ -645,7 +651,7 @@ bool fconv_wgrad(int dt, const void* x, const void* dy, float* dw, float* ws, co
         if (dt) dispatch_fw<bf16>(x, dy, ws, p, xs, G, run, groups, smem, s); else dispatch_fw<float>(x, dy, ws, p, xs, G, run, groups, smem, s);
     }
     Scope sc(KC_SPLITK, 0.0, 4.0 * groups * (p.splits + 1) * blocks * nout, s);
-    fw_reduce_kernel<<<dim3((nout + 31) / 32, blocks, groups), 256, 0, s>>>(ws, dw, p.splits, nout, p.ntaps, 8 * G, p.ci_blocks, g.C, g.Co, w_group, accum);
+    klaunch(fw_reduce_kernel, dim3((nout + 31) / 32, blocks, groups), 256, 0, s, ws, dw, p.splits, nout, p.ntaps, 8 * G, p.ci_blocks, g.C, g.Co, w_group, accum);
     return true;
 }
 

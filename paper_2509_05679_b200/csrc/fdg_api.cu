@@ -20,6 +20,7 @@
 // k-1 (reader of the hand-off slot it overwrites); its update for its own forward pass.
 #include "../../include/fdg.h"
 #include "kernels.h"
+#include "launch.h"
 #include "tc_gemm.h"
 
 #include <atomic>
@@ -111,10 +112,14 @@ struct Module {
     cudaStream_t fstream;          // forward pass: independent of the backward pass of the same iteration (other batch)
     cudaStream_t wstream;          // weight gradients: off the chain input gradient -> batch-norm backward -> input gradient
     cudaEvent_t wev, wdone;        // dy ready for the weight-gradient stream / its work of this iteration finished
-    cudaEvent_t done, fdone, ev0, ev1;
+    cudaEvent_t done[2], fdone;    // this module's iteration t has finished: done[t & 1]; its forward pass: fdone (not when the iteration ran as one graph)
+    cudaEvent_t fork;              // opens the side streams inside a capture
+    StepGraph graph[3];            // the steady-state iteration of this module (module 1: [1] with inputs from host memory, no ingest kernel), or, `split`,
+                                   // its forward pass; [2]: its backward pass and update
+    bool split;
+    bool fdone_valid, ran_direct;  // the last iteration recorded fdone / a full iteration was enqueued kernel by kernel before
+    long long* stamps;             // device: start and end of the last iteration, ns
     float* scratch_f;              // reduction scratch of the forward stream
-    float* fwd_ws;                 // forward stream: partial sums of a forward pass that is split over its contraction
-    size_t fwd_ws_elems;
     float* head_scratch;           // classifier head: weight-gradient partials, then loss partials
     size_t head_elems, head_part_elems;
     bool had_bwd;
@@ -144,12 +149,14 @@ struct fdg_ctx {
     int32_t* labels;
     float* logits;
     char* dlogits;
-    float* loss_ring;
+    LossRecord* loss_ring;         // pinned host memory, 64 records
     int64_t* tags;
     int* tc_err;                   // device word: set by a tensor-core kernel whose bounded wait gave up
     bool any_tc;
+    bool graphs;                   // steady-state iterations run as graphs (off once recording one has failed)
     cudaEvent_t ingested;
-    cudaEvent_t loss_ready;        // recorded behind the kernel that writes the step's loss
+    cudaStream_t cap;              // captures are recorded on it
+    cudaStream_t copy;             // host-to-device copies of the inputs
     std::string err;
 };
 
@@ -268,6 +275,7 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             g.H = ti.h; g.W = ti.w; g.C = cin; g.R = kind == FDG_CONV3X3 ? 3 : 1; g.stride = stride; g.pad = kind == FDG_CONV3X3 ? 1 : 0;
         }
         g.Co = cout; g.Ho = (g.H + 2 * g.pad - g.R) / g.stride + 1; g.Wo = (g.W + 2 * g.pad - g.R) / g.stride + 1;
+        if (!conv_supported(g)) return "convolution shape not covered";
         o.g = g;
         o.w_off = seg((size_t)g.R * g.R * g.C * g.Co, true);
         if (bias) o.b_off = seg(cout, false);
@@ -399,7 +407,7 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
         if (d.loc == LOC_STASH) { d.off = soff; soff += align_up(d.elems() * ctx->M * ctx->esz, 256); }
         if (d.own_grad) { d.goff = goff; goff += align_up(d.elems() * ctx->M * ctx->esz, 256); }
     }
-    m.ws_elems = 0; m.scratch_elems = 64; m.red_elems = 4; m.fwd_ws_elems = 0;
+    m.ws_elems = 0; m.scratch_elems = 64; m.red_elems = 4;
     for (Op& o : m.ops) {
         if (o.type == OP_BN) {
             o.stats_off = soff; soff += align_up((size_t)ctx->n_workers * o.g.C * (ctx->dt == 0 ? 4 : 2) * sizeof(float), 256);
@@ -411,7 +419,6 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             if (o.stem) m.ws_elems = std::max(m.ws_elems, stem_wgrad_workspace_elems(o.g));
             if (o.stem_tc) m.ws_elems = std::max(m.ws_elems, tc::stem_wg_workspace_elems(o.g.Co, (long)o.g.N * o.g.H, ctx->grid_sms));
             m.ws_elems = std::max(m.ws_elems, wgrad_workspace_elems(o.g));
-            m.fwd_ws_elems = std::max(m.fwd_ws_elems, forward_workspace_elems(o.g));
             m.scratch_elems = std::max(m.scratch_elems, (size_t)64 * o.g.Co);
             if (relu_bias_backward_supported(ctx->dt, o.g.Co)) m.scratch_elems = std::max(m.scratch_elems, relu_bias_backward_scratch_elems(o.g.Co));
         }
@@ -521,7 +528,7 @@ bool tc_dgrad(fdg_ctx* c, Module& m, const Op& o, char* dy_base, char* dx_base, 
     double rows = (double)wn.n * g.H * g.W;
     if (o.dgrad_needs_zero && !accum) {
         Scope sc(KC_TC_AUX, 0.0, 2.0 * rows * g.C, s);
-        cudaMemsetAsync(dx_base + (size_t)wn.n0 * g.H * g.W * g.C * 2, 0, (size_t)rows * g.C * 2, s);
+        zero_fill(dx_base + (size_t)wn.n0 * g.H * g.W * g.C * 2, (size_t)rows * g.C * 2, s);
     }
     tc::KmParams p = o.kd;
     p.bias = nullptr; p.out = dx_base; p.epi = accum ? EPI_ACCUM : 0; p.err = c->tc_err; p.stat_part = nullptr; p.sms = c->grid_sms;
@@ -611,7 +618,7 @@ void forward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int grou
                     // logits, loss and dphi/dlogits / M of batch `batch` in one launch (version == the iteration t)
                     head_forward_loss(dt, T(o.in), wbig(c, m, version, o.w_off), o.bias ? wsmall(c, m, version, o.b_off) : nullptr,
                                       c->labels + (size_t)(batch % c->label_depth) * c->M, c->logits, c->dlogits, m.head_scratch + m.head_part_elems,
-                                      (unsigned*)(c->tc_err + 16), c->loss_ring + (version % 64), c->M, g.C, g.Co, 1.f / (float)c->M, s);
+                                      (unsigned*)(c->tc_err + 16), c->loss_ring + (version % 64), c->tc_err, version + 1, c->M, g.C, g.Co, 1.f / (float)c->M, s);
                     profile_detail(nullptr);
                     break;
                 }
@@ -628,8 +635,7 @@ void forward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int grou
                     profile_detail(nullptr);
                     break;
                 }
-                conv_forward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.bias ? wsmall(c, m, version, o.b_off, rep) : nullptr, T(o.out), g, epi,
-                             m.fwd_ws, m.fwd_ws_elems, s);
+                conv_forward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.bias ? wsmall(c, m, version, o.b_off, rep) : nullptr, T(o.out), g, epi, s);
                 profile_detail(nullptr);
                 break; }
             case OP_BN: {
@@ -709,6 +715,13 @@ void backward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t
                     profile_detail(nullptr);
                     break;
                 }
+                if (!o.tc && linear_supported(g)) {
+                    profile_detail(o.shape);
+                    linear_backward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.relu ? T(o.out) : nullptr, gout, gin, o.acc_in, mgrad + o.w_off,
+                                    o.bias ? mgrad + m.n_big + o.b_off : nullptr, g, acc_p, s);
+                    profile_detail(nullptr);
+                    break;
+                }
                 // dZ = dA * (A > 0) in place and the bias gradient, in one pass over dA where the width allows
                 const long orows = (long)g.N * g.Ho * g.Wo;
                 const bool fused_rb = (o.relu || o.bias) && relu_bias_backward_supported(dt, g.Co);
@@ -717,14 +730,14 @@ void backward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t
                 profile_detail(o.shape);
                 // the weight gradient needs dy as it stands now and is needed only by the update: it goes to its own stream
                 cudaStream_t ws = m.wstream;
-                if (ws != s) { cudaEventRecord(m.wev, s); cudaStreamWaitEvent(ws, m.wev, 0); }
+                if (ws != s) { step_record(m.wev, s); step_wait(ws, m.wev); }
                 if (o.stem && tc_stem_wgrad(c, m, o, P.tensor(o.in), grad_ptr(c, kk, o.out, t), mgrad + o.w_off, wn, ws)) {}
                 else if (o.stem) stem_wgrad(T(o.in), gout, mgrad + o.w_off, m.ws, g, acc_p, ws);
                 else if (!(o.tc && tc_wgrad(c, m, o, P.tensor(o.in), grad_ptr(c, kk, o.out, t), mgrad + o.w_off, wn, ws)))
-                    conv_wgrad(dt, T(o.in), gout, mgrad + o.w_off, m.ws, g, acc_p, ws);
+                    fconv_wgrad(dt, T(o.in), gout, mgrad + o.w_off, m.ws, g, 1, 0, acc_p, ws);
                 if (o.bias && !fused_rb) bias_grad(dt, gout, mgrad + m.n_big + o.b_off, m.scratch, orows, g.Co, acc_p, s);
                 if (gin && !(o.tc && tc_dgrad(c, m, o, grad_ptr(c, kk, o.out, t), grad_ptr(c, kk, o.in, t), version, o.acc_in, wn, s)))
-                    conv_dgrad(dt, gout, wbig(c, m, version, o.w_off, rep), gin, g, o.acc_in ? EPI_ACCUM : 0, s);
+                    fconv_dgrad(dt, gout, wbig(c, m, version, o.w_off, rep), gin, g, o.acc_in ? EPI_ACCUM : 0, 1, 0, s);
                 profile_detail(nullptr);
                 break; }
             case OP_BN: {
@@ -919,7 +932,8 @@ fdg_status reset_state(fdg_ctx* ctx) {
     CK(cudaMemcpy(ctx->tags, h.data(), n_tags * sizeof(int64_t), cudaMemcpyHostToDevice));
     CK(cudaDeviceSynchronize());
     ctx->t = 0;
-    for (Module& m : ctx->mod) m.had_bwd = false;
+    std::memset((void*)ctx->loss_ring, 0, 64 * sizeof(LossRecord));      // a record carries its iteration's number: none is left from an earlier run
+    for (Module& m : ctx->mod) m.had_bwd = m.fdone_valid = false;
     return FDG_OK;
 }
 
@@ -932,6 +946,132 @@ fdg_status check_device_error(fdg_ctx* ctx) {
     return FDG_OK;
 }
 
+// Where the batch of iteration t comes from when it already is in device memory (module 1 copies it into its FIFO slot).
+struct Ingest { const void* x; const int32_t* y; };
+
+// One iteration of module kk on its streams.  FORWARD: ingest (module 1), forward on tau_f.  BACKWARD: tags, loss, backward on tau_b, update.
+enum { FORWARD = 1, BACKWARD = 2, WHOLE = 3 };
+fdg_status module_step(fdg_ctx* ctx, int kk, int64_t t, const Ingest* in, int part) {
+    Module& m = ctx->mod[kk];
+    const int K = ctx->K;
+    const int64_t tau_f = t - kk;                         // t - k + 1
+    const int64_t tau_b = t - 2 * (int64_t)K + kk + 2;    // t - 2K + k + 1
+    const int64_t v_b = tau_b + kk;                       // t - 2K + 2k: the version the forward of tau_b used
+    const bool lastm = kk == K - 1;
+    if (in && (part & FORWARD)) {
+        ingest(in->x, m.in_ring + (size_t)(t % m.in_depth) * m.in_slot_bytes, (size_t)ctx->M * m.in_elems * ctx->esz, in->y,
+               ctx->labels + (size_t)(t % ctx->label_depth) * ctx->M, ctx->M, m.fstream);
+        // inside a graph: an event the host can wait for
+        if (StepGraph* g = StepGraph::current()) { if (g->mode() == StepGraph::CAPTURE) CK(cudaEventRecordWithFlags(ctx->ingested, m.fstream, cudaEventRecordExternal)); }
+        else CK(cudaEventRecord(ctx->ingested, m.fstream));
+    }
+    if (part & BACKWARD) {
+    TagOps tg{};
+    if (tau_f >= 0) {
+        tg.rd_act = m.tag_in + 2 * (tau_f % m.in_depth);
+        tg.rd_wfwd = m.tag_w + 2 * (t % m.D);
+        tg.wr_stash = m.tag_stash + 2 * (tau_f % m.D);
+        if (!lastm) { Module& n = ctx->mod[kk + 1]; tg.wr_out = n.tag_in + 2 * (tau_f % n.in_depth); }
+    }
+    if (kk == 0) tg.wr_in = m.tag_in + 2 * (t % m.in_depth);   // the ingest filled this slot with batch t
+    if (tau_b >= 0) {
+        tg.rd_stash = m.tag_stash + 2 * (tau_b % m.D);
+        tg.rd_wbwd = m.tag_w + 2 * (v_b % m.D);
+        if (!lastm) tg.rd_grad = ctx->mod[kk + 1].tag_d2 + 2 * ((t - 1) & 1);
+        if (kk > 0) tg.wr_grad = m.tag_d2 + 2 * (t & 1);
+    }
+    tg.wr_wnext = m.tag_w + 2 * ((t + 1) % m.D);
+    tg.fwd_batch = tau_f >= 0 ? tau_f : -1; tg.bwd_batch = tau_b >= 0 ? tau_b : -1; tg.version_now = t;
+    tg.trace = m.trace; tg.time_start = m.stamps;
+    tags_step(tg, m.stream);
+    }
+
+    if (part & FORWARD) {
+    if (tau_f >= 0) for (int g = 0; g < m.groups; ++g) forward_module(ctx, kk, tau_f, t, g);
+    if (part == WHOLE) CK(step_record(m.fdone, m.fstream));
+    }
+    if (!(part & BACKWARD)) return FDG_OK;
+    if (lastm && m.fstream != m.stream) CK(step_wait(m.stream, m.fdone));   // the last module back-propagates the batch it just forwarded
+    if (lastm) {
+        LossRecord* const rec = ctx->loss_ring + (t % 64);
+        // one replica: dphi/dlogits / M, the mean over all samples.  One replica per worker: / B, worker s's own
+        // gradient scale 1/per_worker_batch of Eq. dl_update (the mixing matrix does the averaging)
+        const bool fused_head = m.ops.back().head && m.groups == 1;     // the forward pass above has computed loss and dlogits
+        if (tau_f < 0) publish_loss_value(rec, NAN, ctx->tc_err, t + 1, m.stream);
+        else if (!fused_head) softmax_ce(ctx->dt, ctx->logits, ctx->labels + (size_t)(tau_f % ctx->label_depth) * ctx->M, ctx->dlogits, rec, ctx->tc_err, t + 1,
+                                         ctx->M, ctx->classes, ctx->R > 1 ? 1.f / (float)ctx->B : 1.f / (float)ctx->M, m.stream);
+    }
+    if (tau_b >= 0) for (int g = 0; g < m.groups; ++g) backward_module(ctx, kk, tau_b, v_b, t, g);
+    // Eq. dl_update with P = 11^T/N: w(t+1) = w(t) - lr * averaged gradient; also emits version t+1
+    // (after the forward pass has read version t: with a one-slot ring the update overwrites it)
+    if (part == WHOLE && !lastm && m.fstream != m.stream) CK(step_wait(m.stream, m.fdone));
+    if (tau_b >= 0 && m.wstream != m.stream) { CK(step_record(m.wdone, m.wstream)); CK(step_wait(m.stream, m.wdone)); }
+    long long* const end = m.stamps + 1;
+    if (ctx->R > 1) {
+        // Eq. dl_update (a), (b) with a general P: u_r = w_r - lr g_r, w_s(t+1) = sum_r P_sr u_r, all replicas in one pass
+        mix_update(ctx->dt, m.master, tau_b >= 0 ? m.grad : nullptr, wslot(ctx, m, t + 1, 0), m.n_big, m.n_small, m.wslot_bytes, ctx->R, ctx->P_dev,
+                   ctx->lr, end, m.stream);
+    } else if (m.fused_update) {
+        Scope sc(KC_SGD, 0.0, (double)npar(m) * (tau_b >= 0 ? 12.0 : 4.0) + 2.0 * m.n_big + 4.0 * m.n_small + 2.0 * m.n_big, m.stream);
+        CK(tc::run_update_module(m.upd, m.master, m.grad, wslot(ctx, m, t + 1), wtslot(m, t + 1, 0), wsmall(ctx, m, t + 1, 0), ctx->lr, tau_b >= 0, end, m.stream));
+    } else {
+        sgd_update(ctx->dt, m.master, tau_b >= 0 ? m.grad : nullptr, wslot(ctx, m, t + 1), m.n_big, ctx->lr, end, m.stream);
+        if (m.n_small)
+            sgd_update(0, m.master + m.n_big, tau_b >= 0 ? m.grad + m.n_big : nullptr,
+                       wsmall(ctx, m, t + 1, 0), m.n_small, ctx->lr, end, m.stream);
+        emit_transposed_weights(ctx, m, t + 1);
+    }
+    m.had_bwd = tau_b >= 0;
+    return FDG_OK;
+}
+
+// The module's iteration as a graph: recorded the first time (on the context's capture stream), refreshed afterwards.
+// false: not possible, nothing was enqueued.
+bool module_step_graph(fdg_ctx* ctx, int kk, int64_t t, const Ingest* in, int part) {
+    Module& m = ctx->mod[kk];
+    StepGraph& graph = part == BACKWARD ? m.graph[2] : m.graph[kk == 0 && !in ? 1 : 0];
+    if (!graph.ready()) {
+        const cudaStream_t s = m.stream, f = m.fstream, w = m.wstream;
+        if (!graph.begin_capture(ctx->cap)) return false;
+        bool ok = true;
+        // the part's main stream becomes the capture's origin, its side streams fork from it
+        const bool side_f = part == WHOLE && f != s, side_w = part != FORWARD && w != s;
+        m.stream = ctx->cap;
+        if (!side_f) m.fstream = ctx->cap;
+        if (!side_w) m.wstream = ctx->cap;
+        if (side_f || side_w) ok = cudaEventRecord(m.fork, ctx->cap) == cudaSuccess;
+        if (ok && side_f) ok = cudaStreamWaitEvent(f, m.fork, 0) == cudaSuccess;
+        if (ok && side_w) ok = cudaStreamWaitEvent(w, m.fork, 0) == cudaSuccess;
+        ok = module_step(ctx, kk, t, in, part) == FDG_OK && ok;
+        m.stream = s; m.fstream = f; m.wstream = w;
+        if (!graph.end_capture(ctx->cap) || !ok) { graph.clear(); ctx->graphs = false; return false; }
+    } else {
+        graph.begin_update();
+        const bool ok = module_step(ctx, kk, t, in, part) == FDG_OK;
+        if (!graph.end_update() || !ok) return false;
+    }
+    return graph.launch(part == FORWARD ? m.fstream : m.stream) == cudaSuccess;
+}
+
+// Waits until the step numbered `seq` has published its loss.
+fdg_status wait_loss(fdg_ctx* ctx, const LossRecord* rec, int64_t seq, float* loss) {
+    const volatile LossRecord* const r = rec;
+    for (long spin = 0; r->seq != seq; ++spin) {
+        if ((spin & 4095) == 4095) {                    // a failed launch or kernel would leave the record as it is
+            const cudaError_t e = cudaStreamQuery(ctx->mod[ctx->K - 1].stream);
+            if (e == cudaSuccess && r->seq != seq) return fail(ctx, FDG_ERR_CUDA, "the step ended without a loss");
+            if (e != cudaSuccess && e != cudaErrorNotReady) return fail(ctx, FDG_ERR_CUDA, "step: %s", cudaGetErrorString(e));
+        }
+#if defined(__x86_64__)
+        __builtin_ia32_pause();
+#endif
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    if (r->err) return fail(ctx, FDG_ERR_TIMEOUT, "a kernel gave up waiting on an mbarrier (code %d)", r->err);
+    *loss = r->loss;
+    return FDG_OK;
+}
+
 fdg_status run_step(fdg_ctx* ctx, const void* inputs, const int32_t* labels, bool host_src, float* host_loss) {
     if (!ctx) return FDG_ERR_INVALID_ARG;
     if (!inputs || !labels) return fail(ctx, FDG_ERR_INVALID_ARG, "inputs and labels must not be NULL");
@@ -939,96 +1079,70 @@ fdg_status run_step(fdg_ctx* ctx, const void* inputs, const int32_t* labels, boo
     if (ctx->broken) return fail(ctx, FDG_ERR_STATE, "an earlier step failed after part of its work was enqueued; call fdg_set_params to start over");
     const int K = ctx->K;
     const int64_t t = ctx->t;
-    // 1. dependencies on the neighbours' previous iteration (all waits first, so that no wait sees an
-    //    event recorded for THIS iteration)
+    const int now = (int)(t & 1), prev = now ^ 1;
+    // which modules run as graphs: those whose iteration has both passes, once it has been enqueued kernel by kernel before
+    // (so that nothing is set up for the first time inside a capture)
+    const bool graphs = ctx->graphs && !profile_active();
+    auto as_graph = [&](const Module& m, int kk) { return graphs && m.ran_direct && t - kk >= 0 && t - 2 * (int64_t)K + kk + 2 >= 0; };
+    // 1. dependencies on the neighbours' previous iteration.  The forward stream: the module's own previous iteration (weights t; slots the
+    //    forward pass overwrites) and its input.  The main stream: the reader of the hand-off slot it overwrites, the error gradient it consumes.
+    auto wait_forward = [&](int kk) -> fdg_status {
+        Module& m = ctx->mod[kk];
+        CK(cudaStreamWaitEvent(m.fstream, m.done[prev], 0));
+        if (kk > 0) { Module& p = ctx->mod[kk - 1]; CK(cudaStreamWaitEvent(m.fstream, p.fdone_valid ? p.fdone : p.done[prev], 0)); }
+        return FDG_OK;
+    };
     if (!ctx->serial && t > 0)
         for (int kk = 0; kk < K; ++kk) {
             Module& m = ctx->mod[kk];
-            CK(cudaStreamWaitEvent(m.fstream, m.done, 0));                                   // weights t; slots its forward overwrites
-            if (kk > 0) CK(cudaStreamWaitEvent(m.fstream, ctx->mod[kk - 1].fdone, 0));       // its input
-            if (kk > 0) CK(cudaStreamWaitEvent(m.stream, ctx->mod[kk - 1].done, 0));         // reader of the hand-off slot it overwrites
-            if (kk + 1 < K) CK(cudaStreamWaitEvent(m.stream, ctx->mod[kk + 1].done, 0));     // the error gradient it consumes
+            if (!as_graph(m, kk) || m.split) { const fdg_status st = wait_forward(kk); if (st != FDG_OK) return st; }
+            if (kk > 0) CK(cudaStreamWaitEvent(m.stream, ctx->mod[kk - 1].done[prev], 0));
+            if (kk + 1 < K) CK(cudaStreamWaitEvent(m.stream, ctx->mod[kk + 1].done[prev], 0));
         }
-    // 2. module 1 "samples" the batch of iteration t: copy into its FIFO slot; labels into the label FIFO
-    {
+    // 2. module 1 "samples" the batch of iteration t into its FIFO slot, the labels go into the label FIFO: from device memory by a
+    //    kernel of its own iteration, from host memory by copies on their own stream.  Those may run beside iteration t-1: the slots
+    //    they fill were last read in iteration t-3 (inputs; t-2 with K = 1) or before iteration t-2 of module 1 ended (labels).
+    Ingest in{inputs, labels};
+    if (host_src) {
         Module& m0 = ctx->mod[0];
-        cudaMemcpyKind kind = host_src ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
-        CK(cudaMemcpyAsync(m0.in_ring + (size_t)(t % m0.in_depth) * m0.in_slot_bytes, inputs,
-                           (size_t)ctx->M * m0.in_elems * ctx->esz, kind, m0.fstream));
-        CK(cudaMemcpyAsync(ctx->labels + (size_t)(t % ctx->label_depth) * ctx->M, labels, (size_t)ctx->M * sizeof(int32_t), kind, m0.fstream));
-        CK(cudaEventRecord(ctx->ingested, m0.fstream));
+        if (t > 1) CK(cudaStreamWaitEvent(ctx->copy, m0.done[now], 0));                      // iteration t-2 (this iteration's record comes later)
+        CK(cudaMemcpyAsync(m0.in_ring + (size_t)(t % m0.in_depth) * m0.in_slot_bytes, inputs, (size_t)ctx->M * m0.in_elems * ctx->esz, cudaMemcpyHostToDevice, ctx->copy));
+        CK(cudaMemcpyAsync(ctx->labels + (size_t)(t % ctx->label_depth) * ctx->M, labels, (size_t)ctx->M * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->copy));
+        CK(cudaEventRecord(ctx->ingested, ctx->copy));
+        CK(cudaStreamWaitEvent(as_graph(m0, 0) && !m0.split ? m0.stream : m0.fstream, ctx->ingested, 0));
+        // the last module reads the labels: K - 1 iterations from now, ordered by the hand-offs; with one module in this iteration's forward pass
     }
     // 3. every module: forward on tau_f, backward on tau_b, update
     for (int kk = 0; kk < K; ++kk) {
         Module& m = ctx->mod[kk];
-        const int64_t tau_f = t - kk;                         // t - k + 1
-        const int64_t tau_b = t - 2 * (int64_t)K + kk + 2;    // t - 2K + k + 1
-        const int64_t v_b = tau_b + kk;                       // t - 2K + 2k: the version the forward of tau_b used
-        const bool lastm = kk == K - 1;
-        CK(cudaEventRecord(m.ev0, m.stream));
-        TagOps tg{};
-        if (tau_f >= 0) {
-            tg.rd_act = m.tag_in + 2 * (tau_f % m.in_depth);
-            tg.rd_wfwd = m.tag_w + 2 * (t % m.D);
-            tg.wr_stash = m.tag_stash + 2 * (tau_f % m.D);
-            if (!lastm) { Module& n = ctx->mod[kk + 1]; tg.wr_out = n.tag_in + 2 * (tau_f % n.in_depth); }
+        const Ingest* const src = kk == 0 && !host_src ? &in : nullptr;
+        bool ran = false, half = false;
+        if (as_graph(m, kk)) {
+            if (!m.split) ran = module_step_graph(ctx, kk, t, src, WHOLE);
+            else if ((half = module_step_graph(ctx, kk, t, src, FORWARD))) {
+                CK(cudaEventRecord(m.fdone, m.fstream));
+                ran = module_step_graph(ctx, kk, t, src, BACKWARD);
+            }
         }
-        if (kk == 0) tg.wr_in = m.tag_in + 2 * (t % m.in_depth);   // the ingest above filled this slot with batch t
-        if (tau_b >= 0) {
-            tg.rd_stash = m.tag_stash + 2 * (tau_b % m.D);
-            tg.rd_wbwd = m.tag_w + 2 * (v_b % m.D);
-            if (!lastm) tg.rd_grad = ctx->mod[kk + 1].tag_d2 + 2 * ((t - 1) & 1);
-            if (kk > 0) tg.wr_grad = m.tag_d2 + 2 * (t & 1);
+        if (!ran) {
+            if (as_graph(m, kk) && !m.split) {
+                // the waits of a kernel-by-kernel iteration, which were not made above
+                if (!ctx->serial && t > 0) { const fdg_status st = wait_forward(kk); if (st != FDG_OK) return st; }
+                if (host_src && kk == 0) CK(cudaStreamWaitEvent(m.fstream, ctx->ingested, 0));
+            }
+            const fdg_status st = module_step(ctx, kk, t, src, half ? BACKWARD : WHOLE);
+            if (st != FDG_OK) return st;
+            if (t - kk >= 0 && m.had_bwd) m.ran_direct = true;
         }
-        tg.wr_wnext = m.tag_w + 2 * ((t + 1) % m.D);
-        tg.fwd_batch = tau_f >= 0 ? tau_f : -1; tg.bwd_batch = tau_b >= 0 ? tau_b : -1; tg.version_now = t;
-        tg.trace = m.trace;
-        tags_step(tg, m.stream);
-
-        if (tau_f >= 0) for (int g = 0; g < m.groups; ++g) forward_module(ctx, kk, tau_f, t, g);
-        CK(cudaEventRecord(m.fdone, m.fstream));
-        if (lastm && m.fstream != m.stream) CK(cudaStreamWaitEvent(m.stream, m.fdone, 0));   // the last module back-propagates the batch it just forwarded
-        if (lastm) {
-            float* loss_slot = ctx->loss_ring + (t % 64);
-            // one replica: dphi/dlogits / M, the mean over all samples.  One replica per worker: / B, worker s's own
-            // gradient scale 1/per_worker_batch of Eq. dl_update (the mixing matrix does the averaging)
-            const bool fused_head = m.ops.back().head && m.groups == 1;     // the forward pass above has computed loss and dlogits
-            if (tau_f >= 0 && fused_head) CK(cudaEventRecord(ctx->loss_ready, m.fstream));
-            else if (tau_f >= 0) softmax_ce(ctx->dt, ctx->logits, ctx->labels + (size_t)(tau_f % ctx->label_depth) * ctx->M, ctx->dlogits,
-                                       loss_slot, ctx->M, ctx->classes, ctx->R > 1 ? 1.f / (float)ctx->B : 1.f / (float)ctx->M, m.stream);
-            else fill_f32(loss_slot, NAN, 1, m.stream);
-            if (!(tau_f >= 0 && fused_head)) CK(cudaEventRecord(ctx->loss_ready, m.stream));
-        }
-        if (tau_b >= 0) for (int g = 0; g < m.groups; ++g) backward_module(ctx, kk, tau_b, v_b, t, g);
-        // Eq. dl_update with P = 11^T/N: w(t+1) = w(t) - lr * averaged gradient; also emits version t+1
-        // (after the forward pass has read version t: with a one-slot ring the update overwrites it)
-        if (!lastm && m.fstream != m.stream) CK(cudaStreamWaitEvent(m.stream, m.fdone, 0));
-        if (tau_b >= 0 && m.wstream != m.stream) { CK(cudaEventRecord(m.wdone, m.wstream)); CK(cudaStreamWaitEvent(m.stream, m.wdone, 0)); }
-        if (ctx->R > 1) {
-            // Eq. dl_update (a), (b) with a general P: u_r = w_r - lr g_r, w_s(t+1) = sum_r P_sr u_r, all replicas in one pass
-            mix_update(ctx->dt, m.master, tau_b >= 0 ? m.grad : nullptr, wslot(ctx, m, t + 1, 0), m.n_big, m.n_small, m.wslot_bytes, ctx->R, ctx->P_dev,
-                       ctx->lr, m.stream);
-        } else if (m.fused_update) {
-            Scope sc(KC_SGD, 0.0, (double)npar(m) * (tau_b >= 0 ? 12.0 : 4.0) + 2.0 * m.n_big + 4.0 * m.n_small + 2.0 * m.n_big, m.stream);
-            CK(tc::run_update_module(m.upd, m.master, m.grad, wslot(ctx, m, t + 1), wtslot(m, t + 1, 0), wsmall(ctx, m, t + 1, 0), ctx->lr, tau_b >= 0, m.stream));
-        } else {
-            sgd_update(ctx->dt, m.master, tau_b >= 0 ? m.grad : nullptr, wslot(ctx, m, t + 1), m.n_big, ctx->lr, m.stream);
-            if (m.n_small)
-                sgd_update(0, m.master + m.n_big, tau_b >= 0 ? m.grad + m.n_big : nullptr,
-                           wsmall(ctx, m, t + 1, 0), m.n_small, ctx->lr, m.stream);
-            emit_transposed_weights(ctx, m, t + 1);
-        }
-        m.had_bwd = tau_b >= 0;
-        CK(cudaEventRecord(m.ev1, m.stream));
-        CK(cudaEventRecord(m.done, m.stream));
+        if (half) CK(cudaStreamWaitEvent(m.stream, m.fdone, 0));        // `done` covers the forward pass too
+        m.fdone_valid = !ran || half;
+        CK(cudaEventRecord(m.done[now], m.stream));
     }
     CK(cudaGetLastError());
     ctx->t = t + 1;
     if (host_loss) {
-        CK(cudaEventSynchronize(ctx->loss_ready));          // the loss only: the last module's backward pass and update go on
-        float l = 0.f;
-        CK(cudaMemcpy(&l, ctx->loss_ring + (t % 64), sizeof(float), cudaMemcpyDeviceToHost));
-        fdg_status es = check_device_error(ctx);
+        float l = 0.f;                                  // the loss only: the last module's backward pass and update go on
+        fdg_status es = wait_loss(ctx, ctx->loss_ring + (t % 64), t + 1, &l);
         if (es != FDG_OK) return es;
         *host_loss = l;
     }
@@ -1046,15 +1160,15 @@ void fdg_destroy(fdg_ctx* ctx) {
     cudaDeviceSynchronize();
     g_reader.release();
     for (Module& m : ctx->mod) {
-        if (m.done) cudaEventDestroy(m.done);
+        for (cudaEvent_t e : m.done) if (e) cudaEventDestroy(e);
+        if (m.fork) cudaEventDestroy(m.fork);
+        for (StepGraph& g : m.graph) g.clear();
         if (m.fdone) cudaEventDestroy(m.fdone);
         if (m.wev) cudaEventDestroy(m.wev);
         if (m.wdone) cudaEventDestroy(m.wdone);
-        if (m.ev0) cudaEventDestroy(m.ev0);
-        if (m.ev1) cudaEventDestroy(m.ev1);
     }
     if (ctx->ingested) cudaEventDestroy(ctx->ingested);
-    if (ctx->loss_ready) cudaEventDestroy(ctx->loss_ready);
+    if (ctx->loss_ring) cudaFreeHost(ctx->loss_ring);
     for (cudaStream_t s : ctx->owned) cudaStreamDestroy(s);
     for (void* p : ctx->blocks) ctx->alloc.free(p, ctx->alloc.user);
     delete ctx;
@@ -1108,7 +1222,7 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
     ctx->own_streams = opt->streams == nullptr;
     ctx->device_bytes = 0;
     ctx->ingested = nullptr;
-    ctx->loss_ready = nullptr;
+    ctx->loss_ring = nullptr; ctx->cap = ctx->copy = nullptr; ctx->graphs = true;
     ctx->device = dev;
     ctx->mod.resize(K);
     g_reader.acquire();                    // released by fdg_destroy, which every error path below goes through
@@ -1139,6 +1253,15 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
         m.in_slot_bytes = align_up((size_t)ctx->M * m.in_elems * ctx->esz, 256);
         m.wslot_bytes = align_up(m.n_big * ctx->esz + m.n_small * sizeof(float), 256);
     }
+    // Two graphs per module (forward / backward + update) let a module's next forward pass start before its neighbours' backward passes are
+    // done, as the kernel-by-kernel order does; one graph costs a launch less.  Measured: ResNet-20, K = 2 (2.5 ms per step) 4 % faster
+    // with two, a four-module MLP of 25 us per step 12 % slower; equal for the ResNet-18- and VGG-shaped networks.  The line: half a
+    // millisecond of estimated work per step (20 TFLOP/s on the CUDA cores, 500 on the tensor cores).
+    double work_us = 0.0;
+    for (const Module& m : ctx->mod)
+        for (const Op& o : m.ops)
+            if (o.type == OP_CONV) work_us += 6.0 * o.g.N * o.g.Ho * o.g.Wo * (double)o.g.Co * o.g.R * o.g.R * o.g.C / (o.tc ? 500e6 : 20e6);
+    for (int kk = 0; kk < K; ++kk) ctx->mod[kk].split = kk + 1 < K && !ctx->serial && work_us > 500.0;
     if (h * w * c != opt->num_classes) return bail(FDG_ERR_INVALID_ARG, "the last layer's width differs from num_classes");
     ctx->n_params = canon;
     ctx->label_depth = 2 * K;
@@ -1159,12 +1282,13 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
     ctx->labels = (int32_t*)get((size_t)ctx->label_depth * ctx->M * sizeof(int32_t));
     ctx->logits = (float*)get((size_t)ctx->M * ctx->classes * sizeof(float));
     ctx->dlogits = get((size_t)ctx->M * ctx->classes * ctx->esz);
-    ctx->loss_ring = (float*)get(64 * sizeof(float));
+    long long* const stamps = (long long*)get((size_t)2 * K * sizeof(long long));
     ctx->tc_err = (int*)get(256);
     if (ctx->R > 1) ctx->P_dev = (float*)get((size_t)ctx->R * ctx->R * sizeof(float));
     size_t tpos = 0;
     for (int kk = 0; kk < K && !oom; ++kk) {
         Module& m = ctx->mod[kk];
+        m.stamps = stamps + 2 * kk;
         m.in_ring = get((size_t)m.in_depth * m.in_slot_bytes);
         m.stash = get((size_t)m.D * m.stash_slot_bytes);
         m.gradpool = get(m.grad_pool_bytes);
@@ -1177,7 +1301,6 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
         m.scratch = (float*)get(m.scratch_elems * sizeof(float));
         m.red = (float*)get(m.red_elems * sizeof(float));
         m.scratch_f = (float*)get(m.scratch_elems * sizeof(float));
-        m.fwd_ws = m.fwd_ws_elems ? (float*)get(m.fwd_ws_elems * sizeof(float)) : nullptr;
         m.head_scratch = m.head_elems ? (float*)get(m.head_elems * sizeof(float)) : nullptr;
         for (int i = 0; i < 2; ++i) m.cstat[i] = m.cstat_elems[i] ? (float*)get(m.cstat_elems[i] * sizeof(float)) : nullptr;
         if (oom) break;
@@ -1203,16 +1326,20 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
         if (e == cudaSuccess && !ctx->serial) { e = cudaStreamCreateWithFlags(&m.wstream, cudaStreamNonBlocking); if (e == cudaSuccess) ctx->owned.push_back(m.wstream); }
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.wev, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.wdone, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.done, cudaEventDisableTiming);
+        for (cudaEvent_t& d : m.done) if (e == cudaSuccess) e = cudaEventCreateWithFlags(&d, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.fork, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.fdone, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreate(&m.ev0);
-        if (e == cudaSuccess) e = cudaEventCreate(&m.ev1);
         if (e == cudaSuccess) e = cudaMemset(m.grad, 0, (size_t)ctx->R * (m.n_big + m.n_small) * sizeof(float));
         if (e == cudaSuccess) e = cudaMemset(m.master, 0, (size_t)ctx->R * (m.n_big + m.n_small) * sizeof(float));
         if (e != cudaSuccess) return bail(FDG_ERR_CUDA, cudaGetErrorString(e));
     }
     if (cudaEventCreateWithFlags(&ctx->ingested, cudaEventDisableTiming) != cudaSuccess) return bail(FDG_ERR_CUDA, "cudaEventCreate failed");
-    if (cudaEventCreateWithFlags(&ctx->loss_ready, cudaEventDisableTiming) != cudaSuccess) return bail(FDG_ERR_CUDA, "cudaEventCreate failed");
+    for (cudaStream_t* q : {&ctx->cap, &ctx->copy}) {
+        if (cudaStreamCreateWithFlags(q, cudaStreamNonBlocking) != cudaSuccess) return bail(FDG_ERR_CUDA, "cudaStreamCreate failed");
+        ctx->owned.push_back(*q);
+    }
+    if (cudaHostAlloc((void**)&ctx->loss_ring, 64 * sizeof(LossRecord), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) return bail(FDG_ERR_CUDA, "cudaHostAlloc failed");
+    if (cudaMemset(stamps, 0, (size_t)2 * K * sizeof(long long)) != cudaSuccess) return bail(FDG_ERR_CUDA, "cudaMemset failed");
     if (cudaMemset(ctx->tc_err, 0, 256) != cudaSuccess) return bail(FDG_ERR_CUDA, "cudaMemset failed");
     if (ctx->R > 1) {
         std::vector<float> pf(ctx->P.begin(), ctx->P.end());
@@ -1262,7 +1389,7 @@ fdg_status fdg_wait_ingest(fdg_ctx* ctx) {
 fdg_status fdg_join(fdg_ctx* ctx, void* stream) {
     if (!ctx) return FDG_ERR_INVALID_ARG;
     if (ctx->t > 0)
-        for (Module& m : ctx->mod) CK(cudaStreamWaitEvent((cudaStream_t)stream, m.done, 0));
+        for (Module& m : ctx->mod) CK(cudaStreamWaitEvent((cudaStream_t)stream, m.done[(ctx->t - 1) & 1], 0));
     return FDG_OK;
 }
 
@@ -1333,8 +1460,8 @@ static fdg_status load_replicas(fdg_ctx* ctx, const float* host_params, int work
             CK(cudaMemcpyAsync(master, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice, m.stream));
             CK(cudaStreamSynchronize(m.stream));
             // version 0 into weight slot 0
-            sgd_update(ctx->dt, master, nullptr, wslot(ctx, m, 0, r), m.n_big, 0.f, m.stream);
-            if (m.n_small) sgd_update(0, master + m.n_big, nullptr, wsmall(ctx, m, 0, 0, r), m.n_small, 0.f, m.stream);
+            sgd_update(ctx->dt, master, nullptr, wslot(ctx, m, 0, r), m.n_big, 0.f, nullptr, m.stream);
+            if (m.n_small) sgd_update(0, master + m.n_big, nullptr, wsmall(ctx, m, 0, 0, r), m.n_small, 0.f, nullptr, m.stream);
         }
         if (ctx->R == 1) emit_transposed_weights(ctx, m, 0);
         CK(cudaMemsetAsync(m.grad, 0, (size_t)ctx->R * npar(m) * sizeof(float), m.stream));
@@ -1523,7 +1650,11 @@ fdg_status fdg_module_times(fdg_ctx* ctx, float* ms, int32_t K) {
     if (!ctx || !ms || K != ctx->K) return FDG_ERR_INVALID_ARG;
     if (ctx->t == 0) return fail(ctx, FDG_ERR_STATE, "no step has run yet");
     CK(cudaDeviceSynchronize());
-    for (int kk = 0; kk < K; ++kk) CK(cudaEventElapsedTime(&ms[kk], ctx->mod[kk].ev0, ctx->mod[kk].ev1));
+    for (int kk = 0; kk < K; ++kk) {
+        long long st[2];
+        CK(cudaMemcpy(st, ctx->mod[kk].stamps, sizeof st, cudaMemcpyDeviceToHost));
+        ms[kk] = (float)((double)(st[1] - st[0]) * 1e-6);
+    }
     return FDG_OK;
 }
 

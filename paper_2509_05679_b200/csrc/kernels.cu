@@ -3,6 +3,7 @@
 // and, on the bf16 path, serve the shapes the tensor-core kernels do not take (3-channel stem,
 // strided convs, 10-class head) plus all memory-bound elementwise / reduction work.
 #include "kernels.h"
+#include "launch.h"
 
 #include <cuda_bf16.h>
 #include <atomic>
@@ -96,6 +97,7 @@ int profile_read_detail(KernelStat* out, char (*names)[48], int capacity) {
 
 typedef __nv_bfloat16 bf16;
 
+__device__ __forceinline__ long long device_time_ns() { long long t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t; }
 __device__ __forceinline__ float ld(const float* p) { return *p; }
 __device__ __forceinline__ float ld(const bf16* p) { return __bfloat162float(*p); }
 __device__ __forceinline__ void st(float* p, float v) { *p = v; }
@@ -103,263 +105,12 @@ __device__ __forceinline__ void st(bf16* p, float v) { *p = __float2bfloat16_rn(
 
 static inline unsigned cdiv(size_t a, size_t b) { return (unsigned)((a + b - 1) / b); }
 
-// ------------------------------------------------------------------------------------------
-// Implicit GEMM  C[m][n] = sum_k A(m,k) * B(k,n)  with the operands gathered on the fly.
-//   FWD  : m = output pixel, n = c_out, k = (r,s,c_in)
-//   DGRAD: m = input pixel,  n = c_in,  k = (r,s,c_out)
-//   WGRAD: m = c_out,        n = (r,s,c_in), k = output pixel   (split over blockIdx.z)
-// 64x64 tile, 16-deep k slices, 256 threads, 4x4 outputs per thread.
-// ------------------------------------------------------------------------------------------
-enum { M_FWD = 0, M_DGRAD = 1, M_WGRAD = 2 };
-constexpr int BM = 64, BN = 64, BK = 16;
-
-template <typename T, int MODE>
-__global__ void __launch_bounds__(256) igemm_simt(const T* __restrict__ P0, const T* __restrict__ P1,
-                                                  void* __restrict__ out, const float* __restrict__ bias,
-                                                  float* __restrict__ partial, ConvGeom g, int Mg, int Ng, int Kg,
-                                                  int k_per_split, int epi) {
-    __shared__ float As[BK][BM + 4];
-    __shared__ float Bs[BK][BN + 4];
-    const int tid = threadIdx.x;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    const int kbeg = blockIdx.z * k_per_split;
-    const int kend = min(Kg, kbeg + k_per_split);
-
-    // which element of the A / B tile this thread fetches: one row (column) and 4 consecutive k
-    int a_row, a_kq, b_col, b_kq;
-    if (MODE == M_WGRAD) { a_row = tid & 63; a_kq = tid >> 6; b_col = tid & 63; b_kq = tid >> 6; }
-    else if (MODE == M_DGRAD) { a_row = tid >> 2; a_kq = tid & 3; b_col = tid & 63; b_kq = tid >> 6; }
-    else { a_row = tid >> 2; a_kq = tid & 3; b_col = tid >> 2; b_kq = tid & 3; }
-
-    const int HoWo = g.Ho * g.Wo, HW = g.H * g.W, RC = g.R * g.C, RCo = g.R * g.Co;
-    const int am = m0 + a_row, bn = n0 + b_col;
-    // per-thread decode of the fixed index
-    int a_n = 0, a_y = 0, a_x = 0;       // FWD: (n, oy*st-pad, ox*st-pad); DGRAD: (n, iy+pad, ix+pad)
-    if (MODE == M_FWD && am < Mg) { a_n = am / HoWo; int p = am - a_n * HoWo; int oy = p / g.Wo; a_y = oy * g.stride - g.pad; a_x = (p - oy * g.Wo) * g.stride - g.pad; }
-    if (MODE == M_DGRAD && am < Mg) { a_n = am / HW; int p = am - a_n * HW; int iy = p / g.W; a_y = iy + g.pad; a_x = (p - iy * g.W) + g.pad; }
-    int b_r = 0, b_s = 0, b_c = 0;       // WGRAD: n -> (r, s, ci)
-    if (MODE == M_WGRAD && bn < Ng) { b_r = bn / RC; int q = bn - b_r * RC; b_s = q / g.C; b_c = q - b_s * g.C; }
-
-    // acc + comp: compensated (Kahan) running sum of the per-slice partial sums, so that the rounding
-    // error of a long contraction (3072 terms in the first MLP layer) stays at a few ulps
-    float acc[4][4], comp[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) { acc[i][j] = 0.f; comp[i][j] = 0.f; }
-    const int tx = tid & 15, ty = tid >> 4;
-
-    for (int k0 = kbeg; k0 < kend; k0 += BK) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            // ---- A element
-            int k = k0 + a_kq * 4 + j;
-            float v = 0.f;
-            if (am < Mg && k < kend) {
-                if (MODE == M_FWD) {
-                    int rs = k / g.C, ci = k - rs * g.C; int r = rs / g.R, s = rs - r * g.R;
-                    int iy = a_y + r, ix = a_x + s;
-                    if (iy >= 0 && iy < g.H && ix >= 0 && ix < g.W) v = ld(P0 + (((size_t)a_n * g.H + iy) * g.W + ix) * g.C + ci);
-                } else if (MODE == M_DGRAD) {
-                    int rs = k / g.Co, co = k - rs * g.Co; int r = rs / g.R, s = rs - r * g.R;
-                    int ty_ = a_y - r, tx_ = a_x - s;
-                    if (ty_ >= 0 && tx_ >= 0) {
-                        int oy = ty_ / g.stride, ox = tx_ / g.stride;
-                        if (oy * g.stride == ty_ && ox * g.stride == tx_ && oy < g.Ho && ox < g.Wo)
-                            v = ld(P0 + (((size_t)a_n * g.Ho + oy) * g.Wo + ox) * g.Co + co);
-                    }
-                } else {
-                    v = ld(P0 + (size_t)k * g.Co + am);
-                }
-            }
-            As[a_kq * 4 + j][a_row] = v;
-            // ---- B element
-            k = k0 + b_kq * 4 + j;
-            v = 0.f;
-            if (bn < Ng && k < kend) {
-                if (MODE == M_FWD) {
-                    v = ld(P1 + (size_t)bn * Kg + k);
-                } else if (MODE == M_DGRAD) {
-                    int rs = k / g.Co, co = k - rs * g.Co;
-                    v = ld(P1 + ((size_t)co * g.R * g.R + rs) * g.C + bn);
-                } else {
-                    int n = k / HoWo; int p = k - n * HoWo; int oy = p / g.Wo, ox = p - oy * g.Wo;
-                    int iy = oy * g.stride - g.pad + b_r, ix = ox * g.stride - g.pad + b_s;
-                    if (iy >= 0 && iy < g.H && ix >= 0 && ix < g.W) v = ld(P1 + (((size_t)n * g.H + iy) * g.W + ix) * g.C + b_c);
-                }
-            }
-            Bs[b_kq * 4 + j][b_col] = v;
-        }
-        __syncthreads();
-        float part[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) part[i][j] = 0.f;
-#pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) part[i][j] = fmaf(a[i], b[j], part[i][j]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                float y = part[i][j] - comp[i][j];
-                float t = acc[i][j] + y;
-                comp[i][j] = (t - acc[i][j]) - y;
-                acc[i][j] = t;
-            }
-        __syncthreads();
-    }
-    (void)RCo;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int m = m0 + ty * 4 + i;
-        if (m >= Mg) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            int n = n0 + tx * 4 + j;
-            if (n >= Ng) continue;
-            size_t o = (size_t)m * Ng + n;
-            float v = acc[i][j];
-            if (partial) { partial[(size_t)blockIdx.z * Mg * Ng + o] = v; continue; }
-            if (bias) v += bias[n];
-            if (epi & EPI_RELU) v = fmaxf(v, 0.f);
-            if (epi & EPI_OUT_F32) {
-                float* c = (float*)out;
-                c[o] = (epi & EPI_ACCUM) ? c[o] + v : v;
-            } else {
-                T* c = (T*)out;
-                if (epi & EPI_ACCUM) v += ld(c + o);
-                st(c + o, v);
-            }
-        }
-    }
-}
-
-// out[i] = sum_z partial[z][i], z ascending (fixed order => run-to-run identical results)
-__global__ void splitk_reduce(const float* __restrict__ partial, float* __restrict__ out, size_t n, int splits, bool accum) {
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float s = 0.f;
-    for (int z = 0; z < splits; ++z) s += partial[(size_t)z * n + i];
-    out[i] = accum ? out[i] + s : s;
-}
-
-void splitk_reduce_launch(const float* partial, float* out, size_t n, int splits, bool accum, cudaStream_t s) {
-    Scope sc(KC_SPLITK, 0.0, 4.0 * n * (splits + 1), s);
-    splitk_reduce<<<cdiv(n, 256), 256, 0, s>>>(partial, out, n, splits, accum);
-}
-
-int wgrad_splits(const ConvGeom& g) {
-    long Kg = (long)g.N * g.Ho * g.Wo;
-    int tiles = (int)(cdiv(g.Co, BM) * cdiv((size_t)g.R * g.R * g.C, BN));
-    int want = (148 * 4 + tiles - 1) / tiles;               // about four waves of CTAs
-    int maxs = (int)((Kg + 255) / 256);                     // at least 256 contraction rows per split
-    int s = want < maxs ? want : maxs;
-    if (s < 1) s = 1;
-    if (s > 256) s = 256;
-    return s;
-}
-size_t wgrad_workspace_elems(const ConvGeom& g) {
-    const size_t direct = fconv_wgrad_workspace_elems(g, 1);
-    if (direct) return direct;
-    int s = wgrad_splits(g);
-    return s > 1 ? (size_t)s * g.Co * g.R * g.R * g.C : 0;
-}
-
-// out[m][n] = epilogue(sum_z partial[z][m][n] + bias[n]), z ascending
-template <typename T>
-__global__ void splitk_forward_epilogue(const float* __restrict__ partial, void* __restrict__ out, const float* __restrict__ bias, size_t n, int Ng, int splits, int epi) {
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float v = 0.f;
-    for (int z = 0; z < splits; ++z) v += partial[(size_t)z * n + i];
-    if (bias) v += bias[i % Ng];
-    if (epi & EPI_RELU) v = fmaxf(v, 0.f);
-    if (epi & EPI_OUT_F32) ((float*)out)[i] = v; else st((T*)out + i, v);
-}
-// A forward pass with few output tiles and a long contraction (a linear layer on a small batch: 8 CTAs walking 3072 terms)
-// is split over the contraction so that it fills the GPU; the partial sums go through `ws`.
-int forward_splits(const ConvGeom& g) {
-    const long Mg = (long)g.N * g.Ho * g.Wo, Ng = g.Co, Kg = (long)g.R * g.R * g.C;
-    const long tiles = (long)cdiv(Ng, BN) * cdiv(Mg, BM);
-    if (tiles >= 74 || Kg < 512 || Mg * Ng > (1 << 18)) return 1;
-    long s = (148 * 2) / tiles, maxs = Kg / 128;
-    if (s > maxs) s = maxs;
-    if (s > 32) s = 32;
-    return (int)(s < 1 ? 1 : s);
-}
-size_t forward_workspace_elems(const ConvGeom& g) {
-    const int s = forward_splits(g);
-    return s > 1 ? (size_t)s * g.N * g.Ho * g.Wo * g.Co : 0;
-}
-template <typename T>
-static void conv_forward_t(const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, float* ws, size_t ws_elems, cudaStream_t s) {
-    int Mg = g.N * g.Ho * g.Wo, Ng = g.Co, Kg = g.R * g.R * g.C;
-    const double flops = 2.0 * Mg * Ng * Kg, bytes = sizeof(T) * ((double)g.N * g.H * g.W * g.C + (double)Ng * Kg + (double)Mg * Ng);
-    int splits = ws ? forward_splits(g) : 1;
-    while (splits > 1 && (size_t)splits * Mg * Ng > ws_elems) --splits;          // a window of the batch: stay inside the workspace sized for the whole batch
-    if (splits > 1) {
-        const int kps = ((Kg + splits - 1) / splits + BK - 1) / BK * BK;
-        splits = (Kg + kps - 1) / kps;
-        dim3 grid(cdiv(Ng, BN), cdiv(Mg, BM), splits);
-        { Scope sc(KC_FMA_FWD, flops, bytes, s);
-          igemm_simt<T, M_FWD><<<grid, 256, 0, s>>>((const T*)x, (const T*)w, nullptr, nullptr, ws, g, Mg, Ng, Kg, kps, 0); }
-        Scope sc(KC_SPLITK, 0.0, 4.0 * (splits + 1) * Mg * Ng, s);
-        splitk_forward_epilogue<T><<<cdiv((size_t)Mg * Ng, 256), 256, 0, s>>>(ws, y, bias, (size_t)Mg * Ng, Ng, splits, epi);
-        return;
-    }
-    dim3 grid(cdiv(Ng, BN), cdiv(Mg, BM), 1);
-    Scope sc(KC_FMA_FWD, flops, bytes, s);
-    igemm_simt<T, M_FWD><<<grid, 256, 0, s>>>((const T*)x, (const T*)w, y, bias, nullptr, g, Mg, Ng, Kg, Kg, epi);
-}
-void conv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, float* ws, size_t ws_elems, cudaStream_t s) {
-    if (fconv_forward(dt, x, w, bias, y, g, epi, 1, 0, 0, nullptr, s)) return;
-    if (dt) conv_forward_t<bf16>(x, w, bias, y, g, epi, ws, ws_elems, s); else conv_forward_t<float>(x, w, bias, y, g, epi, ws, ws_elems, s);
-}
-
-template <typename T>
-static void conv_dgrad_t(const void* dy, const void* w, void* dx, const ConvGeom& g, int epi, cudaStream_t s) {
-    int Mg = g.N * g.H * g.W, Ng = g.C, Kg = g.R * g.R * g.Co;
-    dim3 grid(cdiv(Ng, BN), cdiv(Mg, BM), 1);
-    Scope sc(KC_FMA_DGRAD, 2.0 * Mg * Ng * Kg, sizeof(T) * ((double)g.N * g.Ho * g.Wo * g.Co + (double)Ng * Kg + (double)Mg * Ng), s);
-    igemm_simt<T, M_DGRAD><<<grid, 256, 0, s>>>((const T*)dy, (const T*)w, dx, nullptr, nullptr, g, Mg, Ng, Kg, Kg, epi);
-}
-void conv_dgrad(int dt, const void* dy, const void* w, void* dx, const ConvGeom& g, int epi, cudaStream_t s) {
-    if (fconv_dgrad(dt, dy, w, dx, g, epi, 1, 0, s)) return;
-    if (dt) conv_dgrad_t<bf16>(dy, w, dx, g, epi, s); else conv_dgrad_t<float>(dy, w, dx, g, epi, s);
-}
-
-template <typename T>
-static void conv_wgrad_t(const void* x, const void* dy, float* dw, float* ws, const ConvGeom& g, bool accum, cudaStream_t s) {
-    int Mg = g.Co, Ng = g.R * g.R * g.C, Kg = g.N * g.Ho * g.Wo;
-    int splits = wgrad_splits(g);
-    int kps = ((Kg + splits - 1) / splits + BK - 1) / BK * BK;
-    splits = (Kg + kps - 1) / kps;
-    dim3 grid(cdiv(Ng, BN), cdiv(Mg, BM), splits);
-    double flops = 2.0 * Mg * Ng * Kg, bytes = sizeof(T) * ((double)g.N * g.H * g.W * g.C + (double)Kg * Mg) + 4.0 * Mg * Ng;
-    if (splits == 1) {
-        Scope sc(KC_FMA_WGRAD, flops, bytes, s);
-        igemm_simt<T, M_WGRAD><<<grid, 256, 0, s>>>((const T*)dy, (const T*)x, dw, nullptr, nullptr, g, Mg, Ng, Kg, kps,
-                                                   EPI_OUT_F32 | (accum ? EPI_ACCUM : 0));
-    } else {
-        { Scope sc(KC_FMA_WGRAD, flops, bytes, s);
-          igemm_simt<T, M_WGRAD><<<grid, 256, 0, s>>>((const T*)dy, (const T*)x, dw, nullptr, ws, g, Mg, Ng, Kg, kps, EPI_OUT_F32); }
-        splitk_reduce_launch(ws, dw, (size_t)Mg * Ng, splits, accum, s);
-    }
-}
-void conv_wgrad(int dt, const void* x, const void* dy, float* dw, float* ws, const ConvGeom& g, bool accum, cudaStream_t s) {
-    if (fconv_wgrad(dt, x, dy, dw, ws, g, 1, 0, accum, s)) return;
-    if (dt) conv_wgrad_t<bf16>(x, dy, dw, ws, g, accum, s); else conv_wgrad_t<float>(x, dy, dw, ws, g, accum, s);
+// Convolutions and linear layers on the CUDA cores: fconv.cu and linear.cu.
+size_t wgrad_workspace_elems(const ConvGeom& g) { return linear_supported(g) ? 0 : fconv_wgrad_workspace_elems(g, 1); }
+bool conv_supported(const ConvGeom& g) { return linear_supported(g) || fconv_supported(g); }
+void conv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, cudaStream_t s) {
+    if (linear_supported(g)) linear_forward(dt, x, w, bias, y, g, epi, s);
+    else fconv_forward(dt, x, w, bias, y, g, epi, 1, 0, 0, nullptr, s);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -394,10 +145,10 @@ void bias_grad(int dt, const void* dy, float* db, float* scratch, long rows, int
     int chunks = (int)(rows < RED_CHUNKS ? rows : RED_CHUNKS);
     dim3 grid(cdiv(C, 32), chunks), blk(32, 8);
     { Scope sc(KC_BIAS_GRAD, 0.0, (dt ? 2.0 : 4.0) * rows * C, s);
-      if (dt) colsum_partial<bf16><<<grid, blk, 0, s>>>((const bf16*)dy, scratch, rows, C);
-      else colsum_partial<float><<<grid, blk, 0, s>>>((const float*)dy, scratch, rows, C); }
+      if (dt) klaunch(colsum_partial<bf16>, grid, blk, 0, s, (const bf16*)dy, scratch, rows, C);
+      else klaunch(colsum_partial<float>, grid, blk, 0, s, (const float*)dy, scratch, rows, C); }
     Scope sc(KC_BIAS_GRAD, 0.0, 4.0 * chunks * C, s);
-    colsum_final<<<cdiv(C, 128), 128, 0, s>>>(scratch, db, chunks, C, accum);
+    klaunch(colsum_final, cdiv(C, 128), 128, 0, s, scratch, db, chunks, C, accum);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -463,8 +214,8 @@ static void ew_launch(int dt, const void* a, const void* b, void* o, size_t n, b
     // a window of a tensor whose rows are no multiple of 16 bytes can start anywhere: such calls go element by element
     const bool aligned = (((uintptr_t)a | (uintptr_t)b | (uintptr_t)o) & 15) == 0;
     const size_t work = aligned ? n / (dt ? 8 : 4) : n;
-    if (dt) ew_k<bf16, OP><<<ew_grid(work), 256, 0, s>>>((const bf16*)a, (const bf16*)b, (bf16*)o, n, accum, aligned);
-    else ew_k<float, OP><<<ew_grid(work), 256, 0, s>>>((const float*)a, (const float*)b, (float*)o, n, accum, aligned);
+    if (dt) klaunch(ew_k<bf16, OP>, ew_grid(work), 256, 0, s, (const bf16*)a, (const bf16*)b, (bf16*)o, n, accum, aligned);
+    else klaunch(ew_k<float, OP>, ew_grid(work), 256, 0, s, (const float*)a, (const float*)b, (float*)o, n, accum, aligned);
 }
 
 void relu_forward(int dt, const void* x, void* y, size_t n, cudaStream_t s) {
@@ -552,11 +303,11 @@ void relu_bias_backward(int dt, const void* y_or_null, void* dy, float* db_or_nu
     chunks = (rows + per - 1) / per;
     const double esz = dt ? 2.0 : 4.0;
     { Scope sc(db_or_null ? KC_BIAS_GRAD : KC_RELU_BWD, 0.0, esz * rows * C * (y_or_null ? 3 : 1), s);
-      if (dt) relu_bias_bwd_k<bf16><<<(unsigned)chunks, 256, 0, s>>>((const bf16*)y_or_null, (bf16*)dy, db_or_null ? scratch : nullptr, rows, C, per);
-      else relu_bias_bwd_k<float><<<(unsigned)chunks, 256, 0, s>>>((const float*)y_or_null, (float*)dy, db_or_null ? scratch : nullptr, rows, C, per); }
+      if (dt) klaunch(relu_bias_bwd_k<bf16>, (unsigned)chunks, 256, 0, s, (const bf16*)y_or_null, (bf16*)dy, db_or_null ? scratch : nullptr, rows, C, per);
+      else klaunch(relu_bias_bwd_k<float>, (unsigned)chunks, 256, 0, s, (const float*)y_or_null, (float*)dy, db_or_null ? scratch : nullptr, rows, C, per); }
     if (db_or_null) {
         Scope sc(KC_BIAS_GRAD, 0.0, 4.0 * chunks * C, s);
-        colsum_final_warp<<<cdiv((size_t)C * 32, 256), 256, 0, s>>>(scratch, db_or_null, (int)chunks, C, accum);
+        klaunch(colsum_final_warp, cdiv((size_t)C * 32, 256), 256, 0, s, scratch, db_or_null, (int)chunks, C, accum);
     }
 }
 
@@ -640,24 +391,24 @@ void maxpool_forward(int dt, const void* x, void* y, int N, int H, int W, int C,
     Scope sc(KC_POOL_FWD, 0.0, 1.25 * esz_ * (double)N * H * W * C, s);
     size_t n = (size_t)N * (H / 2) * (W / 2) * C;
     if (C % (dt ? 8 : 4) == 0) {
-        if (dt) maxpool_fwd_vk<bf16><<<ew_grid(n / 8), 256, 0, s>>>((const bf16*)x, (bf16*)y, N, H, W, C);
-        else maxpool_fwd_vk<float><<<ew_grid(n / 4), 256, 0, s>>>((const float*)x, (float*)y, N, H, W, C);
+        if (dt) klaunch(maxpool_fwd_vk<bf16>, ew_grid(n / 8), 256, 0, s, (const bf16*)x, (bf16*)y, N, H, W, C);
+        else klaunch(maxpool_fwd_vk<float>, ew_grid(n / 4), 256, 0, s, (const float*)x, (float*)y, N, H, W, C);
         return;
     }
-    if (dt) maxpool_fwd_k<bf16><<<cdiv(n, 256), 256, 0, s>>>((const bf16*)x, (bf16*)y, N, H, W, C);
-    else maxpool_fwd_k<float><<<cdiv(n, 256), 256, 0, s>>>((const float*)x, (float*)y, N, H, W, C);
+    if (dt) klaunch(maxpool_fwd_k<bf16>, cdiv(n, 256), 256, 0, s, (const bf16*)x, (bf16*)y, N, H, W, C);
+    else klaunch(maxpool_fwd_k<float>, cdiv(n, 256), 256, 0, s, (const float*)x, (float*)y, N, H, W, C);
 }
 void maxpool_backward(int dt, const void* x, const void* dy, void* dx, int N, int H, int W, int C, bool accum, cudaStream_t s) {
     const double esz_ = dt ? 2.0 : 4.0;
     Scope sc(KC_POOL_BWD, 0.0, 2.25 * esz_ * (double)N * H * W * C, s);
     size_t n = (size_t)N * (H / 2) * (W / 2) * C;
     if (C % (dt ? 8 : 4) == 0) {
-        if (dt) maxpool_bwd_vk<bf16><<<ew_grid(n / 8), 256, 0, s>>>((const bf16*)x, (const bf16*)dy, (bf16*)dx, N, H, W, C, accum);
-        else maxpool_bwd_vk<float><<<ew_grid(n / 4), 256, 0, s>>>((const float*)x, (const float*)dy, (float*)dx, N, H, W, C, accum);
+        if (dt) klaunch(maxpool_bwd_vk<bf16>, ew_grid(n / 8), 256, 0, s, (const bf16*)x, (const bf16*)dy, (bf16*)dx, N, H, W, C, accum);
+        else klaunch(maxpool_bwd_vk<float>, ew_grid(n / 4), 256, 0, s, (const float*)x, (const float*)dy, (float*)dx, N, H, W, C, accum);
         return;
     }
-    if (dt) maxpool_bwd_k<bf16><<<cdiv(n, 256), 256, 0, s>>>((const bf16*)x, (const bf16*)dy, (bf16*)dx, N, H, W, C, accum);
-    else maxpool_bwd_k<float><<<cdiv(n, 256), 256, 0, s>>>((const float*)x, (const float*)dy, (float*)dx, N, H, W, C, accum);
+    if (dt) klaunch(maxpool_bwd_k<bf16>, cdiv(n, 256), 256, 0, s, (const bf16*)x, (const bf16*)dy, (bf16*)dx, N, H, W, C, accum);
+    else klaunch(maxpool_bwd_k<float>, cdiv(n, 256), 256, 0, s, (const float*)x, (const float*)dy, (float*)dx, N, H, W, C, accum);
 }
 
 template <typename T>
@@ -696,8 +447,8 @@ void gap_forward(int dt, const void* x, void* y, int N, int HW, int C, cudaStrea
     const double esz_ = dt ? 2.0 : 4.0; (void)esz_;
     Scope sc(KC_GAP_FWD, 0.0, esz_ * (double)N * (HW + 1) * C, s);
     size_t n = (size_t)N * C;
-    if (dt) gap_fwd_k<bf16><<<cdiv(n, 128), 128, 0, s>>>((const bf16*)x, (bf16*)y, N, HW, C);
-    else gap_fwd_k<float><<<cdiv(n, 128), 128, 0, s>>>((const float*)x, (float*)y, N, HW, C);
+    if (dt) klaunch(gap_fwd_k<bf16>, cdiv(n, 128), 128, 0, s, (const bf16*)x, (bf16*)y, N, HW, C);
+    else klaunch(gap_fwd_k<float>, cdiv(n, 128), 128, 0, s, (const float*)x, (float*)y, N, HW, C);
     
 }
 void gap_backward(int dt, const void* dy, void* dx, int N, int HW, int C, bool accum, cudaStream_t s) {
@@ -707,12 +458,12 @@ void gap_backward(int dt, const void* dy, void* dx, int N, int HW, int C, bool a
     const int V = dt ? 8 : 4;
     if (C % V == 0 && ((uintptr_t)dy | (uintptr_t)dx) % 16 == 0) {
         const size_t nvec = n / V;
-        if (dt) gap_bwd_vk<bf16><<<ew_grid(nvec), 256, 0, s>>>((const bf16*)dy, (bf16*)dx, nvec, HW, C / V, accum);
-        else gap_bwd_vk<float><<<ew_grid(nvec), 256, 0, s>>>((const float*)dy, (float*)dx, nvec, HW, C / V, accum);
+        if (dt) klaunch(gap_bwd_vk<bf16>, ew_grid(nvec), 256, 0, s, (const bf16*)dy, (bf16*)dx, nvec, HW, C / V, accum);
+        else klaunch(gap_bwd_vk<float>, ew_grid(nvec), 256, 0, s, (const float*)dy, (float*)dx, nvec, HW, C / V, accum);
         return;
     }
-    if (dt) gap_bwd_k<bf16><<<cdiv(n, 256), 256, 0, s>>>((const bf16*)dy, (bf16*)dx, N, HW, C, accum);
-    else gap_bwd_k<float><<<cdiv(n, 256), 256, 0, s>>>((const float*)dy, (float*)dx, N, HW, C, accum);
+    if (dt) klaunch(gap_bwd_k<bf16>, cdiv(n, 256), 256, 0, s, (const bf16*)dy, (bf16*)dx, N, HW, C, accum);
+    else klaunch(gap_bwd_k<float>, cdiv(n, 256), 256, 0, s, (const float*)dy, (float*)dx, N, HW, C, accum);
     
 }
 
@@ -1180,7 +931,7 @@ static void bns_launch(const BnsArgs& a, int chunks, int nw, cudaStream_t s) {
     static bool attr = false;
     constexpr int smem = BNS_SMEM + (MODE == 3 ? BNS_RED_BYTES : 0);
     if (!attr) { cudaFuncSetAttribute(bns_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); attr = true; }
-    bns_kernel<MODE><<<dim3(chunks, nw), BNV_THREADS, smem, s>>>(a);
+    klaunch(bns_kernel<MODE>, dim3(chunks, nw), BNV_THREADS, smem, s, a);
 }
 
 bool bn_accepts_conv_partials(int dt, int C) { return bnv_ok(dt, C); }
@@ -1194,13 +945,13 @@ void bn_forward(int dt, const void* x, const float* gamma, const float* beta, co
         a.in[0] = (const bf16*)x; a.n_in = 1; a.gamma = gamma; a.beta = beta; a.stats = stats; a.rpw = rpw; a.C = C; a.relu = relu; a.err = err;
         if (conv_part) {
             Scope sc(KC_BN_FWD_STATS, 0.0, 8.0 * conv_chunks * nw * C, s);
-            bnv_stats_final_tiles<<<dim3(C / 4, nw), 256, 0, s>>>(conv_part, stats, conv_chunks, nw, C, rpw);
+            klaunch(bnv_stats_final_tiles, dim3(C / 4, nw), 256, 0, s, conv_part, stats, conv_chunks, nw, C, rpw);
         } else if (conv_chunks >= 0) {
             { Scope sc(KC_BN_FWD_STATS, 0.0, 2.0 * total, s);
               BnsArgs r = a; r.part = scratch;
               bns_launch<0>(r, chunks, nw, s); }
             { Scope sc(KC_BN_FWD_STATS, 0.0, 8.0 * chunks * nw * C, s);
-              bnv_stats_final<<<cdiv((size_t)nw * C * 32, 256), 256, 0, s>>>(scratch, stats, chunks, nw * C, rpw); }
+              klaunch(bnv_stats_final, cdiv((size_t)nw * C * 32, 256), 256, 0, s, scratch, stats, chunks, nw * C, rpw); }
         }
         Scope sc(KC_BN_FWD_APPLY, 0.0, 2.0 * total * (res ? 3 : 2), s);
         a.y = (bf16*)y; a.res = (const bf16*)res;
@@ -1214,14 +965,14 @@ void bn_forward(int dt, const void* x, const float* gamma, const float* beta, co
     const double esz_ = dt ? 2.0 : 4.0;
     size_t total = (size_t)nw * rpw * C;
     { Scope sc(KC_BN_FWD_STATS, 0.0, esz_ * total, s);
-      if (dt) bn_reduce_partial<bf16, false><<<grid, blk, 0, s>>>((const bf16*)x, nullptr, nullptr, nullptr, scratch, rpw, C, false);
-      else bn_reduce_partial<float, false><<<grid, blk, 0, s>>>((const float*)x, nullptr, nullptr, nullptr, scratch, rpw, C, false); }
+      if (dt) klaunch(bn_reduce_partial<bf16, false>, grid, blk, 0, s, (const bf16*)x, nullptr, nullptr, nullptr, scratch, rpw, C, false);
+      else klaunch(bn_reduce_partial<float, false>, grid, blk, 0, s, (const float*)x, nullptr, nullptr, nullptr, scratch, rpw, C, false); }
     { Scope sc(KC_BN_FWD_STATS, 0.0, 8.0 * chunks * nw * C, s);
-      if (dt) bn_stats_final<bf16><<<cdiv((size_t)nw * C, 128), 128, 0, s>>>(scratch, (const bf16*)x, stats, chunks, nw * C, C, rpw);
-      else bn_stats_final<float><<<cdiv((size_t)nw * C, 128), 128, 0, s>>>(scratch, (const float*)x, stats, chunks, nw * C, C, rpw); }
+      if (dt) klaunch(bn_stats_final<bf16>, cdiv((size_t)nw * C, 128), 128, 0, s, scratch, (const bf16*)x, stats, chunks, nw * C, C, rpw);
+      else klaunch(bn_stats_final<float>, cdiv((size_t)nw * C, 128), 128, 0, s, scratch, (const float*)x, stats, chunks, nw * C, C, rpw); }
     Scope sc(KC_BN_FWD_APPLY, 0.0, esz_ * total * (res ? 3 : 2), s);
-    if (dt) bn_apply_k<bf16><<<cdiv(total, 256), 256, 0, s>>>((const bf16*)x, gamma, beta, (const bf16*)res, (bf16*)y, stats, rpw, C, total, relu);
-    else bn_apply_k<float><<<cdiv(total, 256), 256, 0, s>>>((const float*)x, gamma, beta, (const float*)res, (float*)y, stats, rpw, C, total, relu);
+    if (dt) klaunch(bn_apply_k<bf16>, cdiv(total, 256), 256, 0, s, (const bf16*)x, gamma, beta, (const bf16*)res, (bf16*)y, stats, rpw, C, total, relu);
+    else klaunch(bn_apply_k<float>, cdiv(total, 256), 256, 0, s, (const float*)x, gamma, beta, (const float*)res, (float*)y, stats, rpw, C, total, relu);
 }
 
 void bn_backward(int dt, const void* x, const void* out, const void* dout, const float* gamma, const float* beta,
@@ -1251,23 +1002,37 @@ void bn_backward(int dt, const void* x, const void* out, const void* dout, const
     const double esz_ = dt ? 2.0 : 4.0;
     size_t total = (size_t)nw * rpw * C;
     { Scope sc(KC_BN_BWD_REDUCE, 0.0, esz_ * total * (relu ? 3 : 2), s);
-      if (dt) bn_reduce_partial<bf16, true><<<grid, blk, 0, s>>>((const bf16*)x, (const bf16*)out, (const bf16*)dout, stats, scratch, rpw, C, relu);
-      else bn_reduce_partial<float, true><<<grid, blk, 0, s>>>((const float*)x, (const float*)out, (const float*)dout, stats, scratch, rpw, C, relu); }
+      if (dt) klaunch(bn_reduce_partial<bf16, true>, grid, blk, 0, s, (const bf16*)x, (const bf16*)out, (const bf16*)dout, stats, scratch, rpw, C, relu);
+      else klaunch(bn_reduce_partial<float, true>, grid, blk, 0, s, (const float*)x, (const float*)out, (const float*)dout, stats, scratch, rpw, C, relu); }
     { Scope sc(KC_BN_BWD_REDUCE, 0.0, 8.0 * chunks * nw * C, s);
-      bn_bwd_final<<<cdiv(C, 128), 128, 0, s>>>(scratch, red, dgamma, dbeta, chunks, nw, C, accum_params); }
+      klaunch(bn_bwd_final, cdiv(C, 128), 128, 0, s, scratch, red, dgamma, dbeta, chunks, nw, C, accum_params); }
     Scope sc(KC_BN_BWD_APPLY, 0.0, esz_ * total * ((relu ? 3 : 2) + 1 + (dres ? (accum_dres ? 2 : 1) : 0) + (accum_dx ? 1 : 0)), s);
-    if (dt) bn_bwd_apply_k<bf16><<<cdiv(total, 256), 256, 0, s>>>((const bf16*)x, (const bf16*)out, (const bf16*)dout, gamma, stats, red,
+    if (dt) klaunch(bn_bwd_apply_k<bf16>, cdiv(total, 256), 256, 0, s, (const bf16*)x, (const bf16*)out, (const bf16*)dout, gamma, stats, red,
                                                                   (bf16*)dx, accum_dx, (bf16*)dres, accum_dres, rpw, C, total, relu);
-    else bn_bwd_apply_k<float><<<cdiv(total, 256), 256, 0, s>>>((const float*)x, (const float*)out, (const float*)dout, gamma, stats, red,
+    else klaunch(bn_bwd_apply_k<float>, cdiv(total, 256), 256, 0, s, (const float*)x, (const float*)out, (const float*)dout, gamma, stats, red,
                                                                 (float*)dx, accum_dx, (float*)dres, accum_dres, rpw, C, total, relu);
 }
 
 // ------------------------------------------------------------------------------------------
 // softmax cross-entropy: one block; thread i handles rows i, i+256, ...; fixed-order tree sum
 // ------------------------------------------------------------------------------------------
+// The loss goes straight to the host (a record in pinned memory): loss and error word first, then the number the host waits for.
+__device__ __forceinline__ void publish_loss(LossRecord* rec, float loss, const int* err, long long seq) {
+    volatile LossRecord* const r = rec;
+    r->loss = loss;
+    r->err = err ? *(const volatile int*)err : 0;
+    __threadfence_system();
+    r->seq = seq;
+}
+__global__ void publish_k(LossRecord* rec, float loss, const int* err, long long seq) { publish_loss(rec, loss, err, seq); }
+void publish_loss_value(LossRecord* rec, float loss, const int* err, long long seq, cudaStream_t s) {
+    Scope sc(KC_FILL, 0.0, sizeof(LossRecord), s);
+    klaunch(publish_k, 1, 1, 0, s, rec, loss, err, seq);
+}
+
 template <typename T>
 __global__ void softmax_ce_k(const float* __restrict__ z, const int32_t* __restrict__ labels, T* __restrict__ dz,
-                             float* __restrict__ loss_out, int M, int C, float scale) {
+                             LossRecord* rec, const int* err, long long seq, int M, int C, float scale) {
     __shared__ float sh[256];
     float local = 0.f;
     const float inv_m = 1.f / (float)M;
@@ -1287,12 +1052,13 @@ __global__ void softmax_ce_k(const float* __restrict__ z, const int32_t* __restr
     sh[threadIdx.x] = local;
     __syncthreads();
     for (int s = 128; s > 0; s >>= 1) { if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s]; __syncthreads(); }
-    if (threadIdx.x == 0) *loss_out = sh[0] * inv_m;
+    if (threadIdx.x == 0) publish_loss(rec, sh[0] * inv_m, err, seq);
 }
-void softmax_ce(int dt, const float* logits, const int32_t* labels, void* dlogits, float* loss_out, int M, int classes, float scale, cudaStream_t s) {
+void softmax_ce(int dt, const float* logits, const int32_t* labels, void* dlogits, LossRecord* rec, const int* err, long long seq, int M, int classes, float scale,
+                cudaStream_t s) {
     Scope sc(KC_SOFTMAX_CE, 0.0, (double)M * classes * (dt ? 6.0 : 8.0) + 4.0 * M, s);
-    if (dt) softmax_ce_k<bf16><<<1, 256, 0, s>>>(logits, labels, (bf16*)dlogits, loss_out, M, classes, scale);
-    else softmax_ce_k<float><<<1, 256, 0, s>>>(logits, labels, (float*)dlogits, loss_out, M, classes, scale);
+    if (dt) klaunch(softmax_ce_k<bf16>, 1, 256, 0, s, logits, labels, (bf16*)dlogits, rec, err, seq, M, classes, scale);
+    else klaunch(softmax_ce_k<float>, 1, 256, 0, s, logits, labels, (float*)dlogits, rec, err, seq, M, classes, scale);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1311,7 +1077,7 @@ constexpr int HEAD_ROWS_PER_CTA = 32;       // samples per CTA of head_bwd_k
 template <typename T>
 __global__ void __launch_bounds__(256) head_fwd_loss_k(const T* __restrict__ x, const T* __restrict__ W, const float* __restrict__ bias,
                                                        const int32_t* __restrict__ labels, float* __restrict__ logits, T* __restrict__ dz,
-                                                       float* __restrict__ loss_part, unsigned* __restrict__ counter, float* __restrict__ loss_out,
+                                                       float* __restrict__ loss_part, unsigned* __restrict__ counter, LossRecord* rec, const int* err, long long seq,
                                                        int M, int K, int C, float scale) {
     constexpr int V = Vec<T>::V;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1375,8 +1141,8 @@ __global__ void __launch_bounds__(256) head_fwd_loss_k(const T* __restrict__ x, 
         __threadfence();
         float s = 0.f;
         for (unsigned i = 0; i < gridDim.x; ++i) s += ((volatile float*)loss_part)[i];
-        *loss_out = s / (float)M;
         *counter = 0u;
+        publish_loss(rec, s / (float)M, err, seq);
     }
 }
 // grid = ceil(M / HEAD_ROWS_PER_CTA).  part: [CTA][C][K + 1]
@@ -1452,20 +1218,20 @@ size_t head_scratch_elems(int M, int K, int C) {
     return ctas * C * (K + 1) + (M + 7) / 8;
 }
 void head_forward_loss(int dt, const void* x, const void* W, const float* bias, const int32_t* labels, float* logits, void* dlogits, float* scratch,
-                       unsigned* counter, float* loss_out, int M, int K, int C, float scale, cudaStream_t s) {
+                       unsigned* counter, LossRecord* rec, const int* err, long long seq, int M, int K, int C, float scale, cudaStream_t s) {
     Scope sc(KC_SOFTMAX_CE, 2.0 * M * K * C, (dt ? 2.0 : 4.0) * ((double)M * K + (double)C * K + (double)M * C) + 4.0 * M * C, s);
     const unsigned grid = (M + 7) / 8;
-    if (dt) head_fwd_loss_k<bf16><<<grid, 256, 0, s>>>((const bf16*)x, (const bf16*)W, bias, labels, logits, (bf16*)dlogits, scratch, counter, loss_out, M, K, C, scale);
-    else head_fwd_loss_k<float><<<grid, 256, 0, s>>>((const float*)x, (const float*)W, bias, labels, logits, (float*)dlogits, scratch, counter, loss_out, M, K, C, scale);
+    if (dt) klaunch(head_fwd_loss_k<bf16>, grid, 256, 0, s, (const bf16*)x, (const bf16*)W, bias, labels, logits, (bf16*)dlogits, scratch, counter, rec, err, seq, M, K, C, scale);
+    else klaunch(head_fwd_loss_k<float>, grid, 256, 0, s, (const float*)x, (const float*)W, bias, labels, logits, (float*)dlogits, scratch, counter, rec, err, seq, M, K, C, scale);
 }
 void head_backward(int dt, const void* x, const void* W, const void* dlogits, void* dx_or_null, bool accum_dx, float* dW, float* db_or_null, float* scratch,
                    int M, int K, int C, cudaStream_t s) {
     const unsigned ctas = (M + HEAD_ROWS_PER_CTA - 1) / HEAD_ROWS_PER_CTA;
     { Scope sc(KC_FMA_WGRAD, (dx_or_null ? 4.0 : 2.0) * M * K * C, (dt ? 2.0 : 4.0) * ((double)M * K * (dx_or_null ? 2 : 1) + (double)C * K + (double)M * C), s);
-      if (dt) head_bwd_k<bf16><<<ctas, 256, 0, s>>>((const bf16*)x, (const bf16*)W, (const bf16*)dlogits, (bf16*)dx_or_null, scratch, M, K, C, accum_dx);
-      else head_bwd_k<float><<<ctas, 256, 0, s>>>((const float*)x, (const float*)W, (const float*)dlogits, (float*)dx_or_null, scratch, M, K, C, accum_dx); }
+      if (dt) klaunch(head_bwd_k<bf16>, ctas, 256, 0, s, (const bf16*)x, (const bf16*)W, (const bf16*)dlogits, (bf16*)dx_or_null, scratch, M, K, C, accum_dx);
+      else klaunch(head_bwd_k<float>, ctas, 256, 0, s, (const float*)x, (const float*)W, (const float*)dlogits, (float*)dx_or_null, scratch, M, K, C, accum_dx); }
     Scope sc(KC_SPLITK, 0.0, 4.0 * (ctas + 1) * C * (K + 1), s);
-    head_reduce_k<<<cdiv((size_t)C * (K + 1), 256), 256, 0, s>>>(scratch, dW, db_or_null, (int)ctas, K, C);
+    klaunch(head_reduce_k, cdiv((size_t)C * (K + 1), 256), 256, 0, s, scratch, dW, db_or_null, (int)ctas, K, C);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1473,7 +1239,7 @@ void head_backward(int dt, const void* x, const void* W, const void* dlogits, vo
 // 128-bit loads and stores; grid sized to a multiple of the SM count by the grid-stride loop.
 // ------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void sgd_k(float4* __restrict__ master, const float4* __restrict__ grad, T* __restrict__ copy, size_t n4, float lr) {
+__global__ void sgd_k(float4* __restrict__ master, const float4* __restrict__ grad, T* __restrict__ copy, size_t n4, float lr, long long* stamp) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
         float4 w = master[i];
         if (grad) {
@@ -1489,16 +1255,17 @@ __global__ void sgd_k(float4* __restrict__ master, const float4* __restrict__ gr
             ((uint2*)copy)[i] = pk;
         }
     }
+    if (stamp && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *stamp = device_time_ns();
 }
-void sgd_update(int dt, float* master, const float* grad, void* copy_next, size_t n, float lr, cudaStream_t s) {
+void sgd_update(int dt, float* master, const float* grad, void* copy_next, size_t n, float lr, long long* stamp, cudaStream_t s) {
     size_t n4 = n / 4;
     if (n4 == 0) return;
     unsigned blocks = cdiv(n4, 256);
     if (blocks > 148 * 8) blocks = 148 * 8;
     // per parameter: read master (4) [+ read grad (4) + write master (4)] + write the copy (2 or 4)
     Scope sc(KC_SGD, 0.0, (double)n * ((grad ? 12.0 : 4.0) + (dt ? 2.0 : 4.0)), s);
-    if (dt) sgd_k<bf16><<<blocks, 256, 0, s>>>((float4*)master, (const float4*)grad, (bf16*)copy_next, n4, lr);
-    else sgd_k<float><<<blocks, 256, 0, s>>>((float4*)master, (const float4*)grad, (float*)copy_next, n4, lr);
+    if (dt) klaunch(sgd_k<bf16>, blocks, 256, 0, s, (float4*)master, (const float4*)grad, (bf16*)copy_next, n4, lr, stamp);
+    else klaunch(sgd_k<float>, blocks, 256, 0, s, (float4*)master, (const float4*)grad, (float*)copy_next, n4, lr, stamp);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1511,7 +1278,7 @@ void sgd_update(int dt, float* master, const float* grad, void* copy_next, size_
 constexpr int MIX_MAX_R = 32;
 template <typename T>
 __global__ void __launch_bounds__(256) mix_k(float* master, const float* __restrict__ grad, char* copy0, size_t n_big, size_t n_small, size_t slot_bytes,
-                                              int R, const float* __restrict__ P, float lr) {
+                                              int R, const float* __restrict__ P, float lr, long long* stamp) {
     __shared__ float Ps[MIX_MAX_R * MIX_MAX_R];
     for (int i = threadIdx.x; i < R * R; i += blockDim.x) Ps[i] = P[i];
     __syncthreads();
@@ -1547,17 +1314,18 @@ __global__ void __launch_bounds__(256) mix_k(float* master, const float* __restr
             }
         }
     }
+    if (stamp && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *stamp = device_time_ns();
 }
 int mix_max_replicas() { return MIX_MAX_R; }
 void mix_update(int dt, float* master, const float* grad, void* copy0, size_t n_big, size_t n_small, size_t slot_bytes, int R, const float* P, float lr,
-                cudaStream_t s) {
+                long long* stamp, cudaStream_t s) {
     const size_t n4 = (n_big + n_small) / 4;
     if (n4 == 0) return;
     unsigned blocks = cdiv(n4, 256);
     if (blocks > 148 * 4) blocks = 148 * 4;
     Scope sc(KC_SGD, 0.0, (double)R * (n_big + n_small) * ((grad ? 12.0 : 8.0) + (dt ? 2.0 : 4.0)), s);
-    if (dt) mix_k<bf16><<<blocks, 256, 0, s>>>(master, grad, (char*)copy0, n_big, n_small, slot_bytes, R, P, lr);
-    else mix_k<float><<<blocks, 256, 0, s>>>(master, grad, (char*)copy0, n_big, n_small, slot_bytes, R, P, lr);
+    if (dt) klaunch(mix_k<bf16>, blocks, 256, 0, s, master, grad, (char*)copy0, n_big, n_small, slot_bytes, R, P, lr, stamp);
+    else klaunch(mix_k<float>, blocks, 256, 0, s, master, grad, (char*)copy0, n_big, n_small, slot_bytes, R, P, lr, stamp);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1565,6 +1333,7 @@ void mix_update(int dt, float* master, const float* grad, void* copy0, size_t n_
 // ------------------------------------------------------------------------------------------
 __global__ void tags_k(TagOps o) {
     if (threadIdx.x != 0) return;
+    if (o.time_start) *o.time_start = device_time_ns();
     // tags of what this step produces first: the last module reads the stash slot it fills itself
     if (o.wr_in) { o.wr_in[0] = o.version_now; o.wr_in[1] = -1; }      // module 1: the batch sampled now
     if (o.wr_out) { o.wr_out[0] = o.fwd_batch; o.wr_out[1] = -1; }
@@ -1582,9 +1351,35 @@ __global__ void tags_k(TagOps o) {
     // the next weight version replaces a slot only at the end of the step, after the reads above
     if (o.wr_wnext) { o.wr_wnext[0] = -1; o.wr_wnext[1] = o.version_now + 1; }
 }
-void tags_step(const TagOps& ops, cudaStream_t s) { Scope sc(KC_TAGS, 0.0, 128.0, s); tags_k<<<1, 32, 0, s>>>(ops); }
+void tags_step(const TagOps& ops, cudaStream_t s) { Scope sc(KC_TAGS, 0.0, 128.0, s); klaunch(tags_k, 1, 32, 0, s, ops); }
 
-__global__ void fill_k(float* p, float v, size_t n) { size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; if (i < n) p[i] = v; }
-void fill_f32(float* p, float v, size_t n, cudaStream_t s) { if (!n) return; Scope sc(KC_FILL, 0.0, 4.0 * n, s); fill_k<<<cdiv(n, 256), 256, 0, s>>>(p, v, n); }
+// Zeros, 16 bytes per thread and access (n16 vectors).
+__global__ void __launch_bounds__(256) zero_k(uint4* p, size_t n16) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x) p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+void zero_fill(void* p, size_t bytes, cudaStream_t s) { klaunch(zero_k, ew_grid(bytes / 16), 256, 0, s, (uint4*)p, bytes / 16); }
+
+// The step's batch and labels into their FIFO slots, one launch.  vec: all four addresses are 16-byte aligned.
+__global__ void __launch_bounds__(256) ingest_k(const char* __restrict__ x, char* __restrict__ xd, size_t x_bytes, const int32_t* __restrict__ y, int32_t* __restrict__ yd, int m, bool vec) {
+    const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+    const size_t n16 = vec ? x_bytes / 16 : 0;
+    size_t i = t0;
+    for (; i + 3 * stride < n16; i += 4 * stride) {              // four loads in flight
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = ((const uint4*)x)[i + u * stride];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) ((uint4*)xd)[i + u * stride] = v[u];
+    }
+    for (; i < n16; i += stride) ((uint4*)xd)[i] = ((const uint4*)x)[i];
+    for (size_t b = n16 * 16 + 2 * t0; b < x_bytes; b += 2 * stride) *(uint16_t*)(xd + b) = *(const uint16_t*)(x + b);     // both storage types are whole 2-byte words
+    for (size_t l = t0; l < (size_t)m; l += stride) yd[l] = y[l];
+}
+void ingest(const void* x, void* xd, size_t x_bytes, const int32_t* y, int32_t* yd, int m, cudaStream_t s) {
+    const bool vec = (((uintptr_t)x | (uintptr_t)xd) & 15) == 0;
+    klaunch(ingest_k, ew_grid(vec ? x_bytes / 64 : x_bytes / 2), 256, 0, s, (const char*)x, (char*)xd, x_bytes, y, yd, m, vec);
+}
+
+bool profile_active() { return prof::g_on; }
 
 }  // namespace fdg

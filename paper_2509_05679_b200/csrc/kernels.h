@@ -12,26 +12,22 @@ struct ConvGeom {            // x: [N,H,W,C]  ->  y: [N,Ho,Wo,Co], R x R window
 
 enum { EPI_RELU = 1, EPI_ACCUM = 2, EPI_OUT_F32 = 4 };
 
-// Number of k-splits the weight-gradient kernel will use for this geometry (>= 1) and the
-// fp32 workspace elements it needs (splits * Co * R*R*C when splits > 1, else 0).
-int    wgrad_splits(const ConvGeom& g);
-size_t wgrad_workspace_elems(const ConvGeom& g);
+// y = conv(x, W) (+ bias) (relu)            (Eq. forward_step for linear / conv layers, CUDA cores)
 
-// y = conv(x, W) (+ bias) (relu)            (Eq. forward_step for linear / conv layers)
-// workspace: forward_workspace_elems(g) floats (0: none needed), or nullptr: a forward pass with few output tiles and a
-// long contraction is split over the contraction through it
-size_t forward_workspace_elems(const ConvGeom& g);
-void conv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g,
-                  int epi, float* workspace, size_t workspace_elems, cudaStream_t st);
-// dx (+)= conv_transpose(dy, W)             (Eq. backward_step, gradient w.r.t. the layer input)
-void conv_dgrad(int dt, const void* dy, const void* w, void* dx, const ConvGeom& g, int epi, cudaStream_t st);
-// dW = sum over all N*Ho*Wo rows of dy^T (x) patches(x), fp32 out; the reduction runs over the
-// worker x batch axis, which is the worker average of Eq. dl_update (b) for P = 11^T/N.
-// accum: dw += (a second group of workers adds to the first group's result)
-void conv_wgrad(int dt, const void* x, const void* dy, float* dw, float* workspace, const ConvGeom& g, bool accum, cudaStream_t st);
-// The same three for convolutions (H * W > 1; 3x3 and 1x1, stride 1 and 2) in the packed-FMA kernels of fconv.cu; the
-// generic functions above take them where they apply.  `groups`: consecutive equal groups of images, each with its own weights
+bool   conv_supported(const ConvGeom& g);
+size_t wgrad_workspace_elems(const ConvGeom& g);      // fp32 elements fconv_wgrad needs
+void   conv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, cudaStream_t st);
+// Linear layers (linear.cu).  linear_backward: dx (+)= dy' W (dx_or_null == nullptr: not needed), dW (+)= dy'^T x, db (+)= column sums of
+// dy' in one launch; dy' = dy * [y > 0] if y_or_null is given (the layer ends in a ReLU), else dy.  The sums run over the worker x
+// batch axis, which is the worker average of Eq. dl_update (b) for P = 11^T/N.  accum_p: dW and db are added to (a second group of workers).
+bool   linear_supported(const ConvGeom& g);
+void   linear_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, cudaStream_t st);
+void   linear_backward(int dt, const void* x, const void* w, const void* y_or_null, const void* dy, void* dx_or_null, bool accum_dx, float* dw, float* db_or_null,
+                       const ConvGeom& g, bool accum_p, cudaStream_t st);
+// Convolutions (3x3 and 1x1, stride 1 and 2) in the packed-FMA kernels of fconv.cu: forward, dx (+)= conv_transpose(dy, W), dW (+)= the sum
+// over all N*Ho*Wo rows of dy^T (x) patches(x) (fp32).  `groups`: consecutive equal groups of images, each with its own weights
 // (w_group elements apart; biases b_group apart; weight gradients w_group apart).  false: shape not covered, nothing launched.
+bool   fconv_supported(const ConvGeom& g);
 bool   fconv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
                      float* stat_or_null, cudaStream_t st);
 // Batch-norm statistics taken along by fconv_forward (groups = workers): per worker and pixel tile the channels' (mean, sum of
@@ -99,9 +95,13 @@ void bn_backward(int dt, const void* x, const void* out, const void* dout, const
                  float* red, float* scratch, int n_workers, long rows_per_worker, int C, bool relu, bool has_res, bool accum_params,
                  int sms, int* err, cudaStream_t st);
 
+// Where a step's loss reaches the host: pinned memory the kernel that computes it writes to (seq last).
+struct LossRecord { float loss; int err; long long seq; };
+void publish_loss_value(LossRecord* rec, float loss, const int* err, long long seq, cudaStream_t st);
+
 // Softmax cross-entropy over fp32 logits [M, classes]: dlogits (storage dtype) = (softmax - onehot) * scale,
-// *loss_out = mean loss.  Deterministic single-block reduction.
-void softmax_ce(int dt, const float* logits, const int32_t* labels, void* dlogits, float* loss_out, int M, int classes,
+// rec: the mean loss, the error word `err` and the number `seq`.  Deterministic single-block reduction.
+void softmax_ce(int dt, const float* logits, const int32_t* labels, void* dlogits, LossRecord* rec, const int* err, long long seq, int M, int classes,
                 float scale, cudaStream_t st);
 
 // Classifier head (the last linear layer, c_in = K -> C classes, C <= 16) fused with the loss.  head_forward_loss: logits
@@ -111,32 +111,35 @@ void softmax_ce(int dt, const float* logits, const int32_t* labels, void* dlogit
 bool   head_supported(int dt, int K, int C);
 size_t head_scratch_elems(int M, int K, int C);
 void   head_forward_loss(int dt, const void* x, const void* W, const float* bias, const int32_t* labels, float* logits, void* dlogits, float* scratch,
-                         unsigned* counter, float* loss_out, int M, int K, int C, float scale, cudaStream_t st);
+                         unsigned* counter, LossRecord* rec, const int* err, long long seq, int M, int K, int C, float scale, cudaStream_t st);
 void   head_backward(int dt, const void* x, const void* W, const void* dlogits, void* dx_or_null, bool accum_dx, float* dW, float* db_or_null, float* scratch,
                      int M, int K, int C, cudaStream_t st);
 
 // master -= lr * grad (skipped when grad == nullptr: w(t+1) = w(t)); copy_next = storage-dtype copy of
 // the new master (the next weight version).  n must be a multiple of 4; pointers 16-byte aligned.
-void sgd_update(int dt, float* master, const float* grad, void* copy_next, size_t n, float lr, cudaStream_t st);
+// stamp: device word that receives the device's time in ns at the end, or nullptr.
+void sgd_update(int dt, float* master, const float* grad, void* copy_next, size_t n, float lr, long long* stamp, cudaStream_t st);
 
 // General mixing matrix: R replicas [R][n_big + n_small] of master and grad; u_r = w_r - lr g_r (grad == nullptr: u_r = w_r),
 // w_s = sum_r P[s][r] u_r in place, and the storage-dtype copies of the next version (replica r at copy0 + r * slot_bytes:
 // n_big values of the storage dtype, then n_small floats).  R <= mix_max_replicas().
 int  mix_max_replicas();
 void mix_update(int dt, float* master, const float* grad, void* copy0, size_t n_big, size_t n_small, size_t slot_bytes, int R, const float* P, float lr,
-                cudaStream_t st);
+                long long* stamp, cudaStream_t st);
 
 // Schedule tags (see fdg_trace).  tags are int64 pairs {batch id, weight version}.
 struct TagOps {
     const int64_t* rd_act;  const int64_t* rd_stash; const int64_t* rd_grad; const int64_t* rd_wbwd; const int64_t* rd_wfwd;
     int64_t* wr_in; int64_t* wr_out; int64_t* wr_stash; int64_t* wr_grad; int64_t* wr_wnext;
     int64_t fwd_batch, bwd_batch, version_now;   // what this step produces (-1: nothing)
+    long long* time_start;                       // device time in ns, or nullptr
     int64_t* trace;                              // [4]: fwd batch, bwd batch, bwd weight version, fwd weight version
 };
 void tags_step(const TagOps& ops, cudaStream_t st);
 
-void fill_f32(float* p, float v, size_t n, cudaStream_t st);
-void splitk_reduce_launch(const float* partial, float* out, size_t n, int splits, bool accum, cudaStream_t st);
+void zero_fill(void* p, size_t bytes, cudaStream_t st);          // p and bytes multiples of 16
+// x_bytes of a batch and its m labels into their FIFO slots
+void ingest(const void* x, void* x_slot, size_t x_bytes, const int32_t* y, int32_t* y_slot, int m, cudaStream_t st);
 uint64_t launches();     // kernels launched so far through this interface
 
 // Kernel classes for launch counting and optional device timing.
@@ -155,6 +158,7 @@ struct Scope {
 };
 void profile_detail(const char* detail);                    // tag (e.g. a layer shape) for the Scopes this thread opens next; nullptr clears
 int  profile_read_detail(KernelStat* out, char (*names)[48], int capacity);   // call after profile_read
+bool profile_active();
 void profile_enable(bool on);                               // on: clears the statistics
 int  profile_read(KernelStat* out, const char** names);     // synchronises the device; returns KC_COUNT
 

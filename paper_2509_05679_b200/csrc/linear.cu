@@ -1,0 +1,322 @@
+// Linear layers on the CUDA cores (fp32 arithmetic, fp32 or bf16 storage): the whole fp32 path and, with bf16 storage, widths that are
+// no multiple of 64.  Any sizes.
+//   forward  : one launch, y = x W^T (+ b) (relu).
+//   backward : one launch: dx (+)= dy W and dW (+)= dy^T x, db (+)= column sums of dy; the ReLU mask dy * [y > 0] is applied while dy is
+//              read, so that there is no pass of its own for it, for the bias gradient or for either gradient matrix.
+//
+// What bounds these layers is latency, not arithmetic: 64 samples through 3072 -> 512 are 0.2 GFLOP, and the kernels they replace took
+// two launches each with serial chains of up to 3072 / 16 slices or a few CTAs (62 us for the input gradient of 512 -> 256 on 64
+// samples).  So: 32 x 64 tiles of 128 threads, and a forward or input-gradient tile is split over the contraction among the CTAs of a
+// cluster, which add their partial tiles through distributed shared memory in rank order: no workspace, no second launch.  A
+// weight-gradient tile contracts over the samples, has no split, and the CTAs of a cluster take tiles of their own.
+// Arithmetic as in fconv.cu: packed FMAs with the pairs along the contraction, chains of at most 16 products into a compensated sum.
+#include "kernels.h"
+#include "launch.h"
+
+#include <cuda_bf16.h>
+
+namespace fdg {
+
+typedef __nv_bfloat16 bf16;
+
+namespace {
+
+constexpr int LT = 128, LM = 32, LN = 64, LK = 32;
+constexpr int LP = 36;                   // floats per row of a 32-wide chunk: rows fall into different banks for 16-byte reads
+
+__device__ __forceinline__ float to_f(float v) { return v; }
+__device__ __forceinline__ float to_f(bf16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ void put(float* p, float v) { *p = v; }
+__device__ __forceinline__ void put(bf16* p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ float4 ld4(const float* p) { return *(const float4*)p; }
+__device__ __forceinline__ float4 ld4(const bf16* p) {
+    const uint2 v = *(const uint2*)p;
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+}
+
+// Four consecutive elements of row r (columns c .. c + 3) of a row-major matrix, zero outside rows x cols.
+template <typename T>
+__device__ __forceinline__ float4 fetch4(const T* __restrict__ p, int r, int c, int rows, int cols, bool vec) {
+    if (r >= rows || c >= cols) return make_float4(0.f, 0.f, 0.f, 0.f);
+    const T* s = p + (size_t)r * cols + c;
+    if (vec) return ld4(s);              // cols is a multiple of 4 and the matrix starts on a 4-element boundary
+    return make_float4(to_f(s[0]), c + 1 < cols ? to_f(s[1]) : 0.f, c + 2 < cols ? to_f(s[2]) : 0.f, c + 3 < cols ? to_f(s[3]) : 0.f);
+}
+__device__ __forceinline__ float4 masked(float4 d, float4 y) { return make_float4(y.x > 0.f ? d.x : 0.f, y.y > 0.f ? d.y : 0.f, y.z > 0.f ? d.z : 0.f, y.w > 0.f ? d.w : 0.f); }
+
+struct LinArgs {
+    const void* x; const void* w; const void* dy; const void* y;     // [M][K], [N][K], [M][N], [M][N] (y: mask of the backward pass, or nullptr)
+    const float* bias;
+    void* out;                           // forward: y [M][N]; backward: dx [M][K] or nullptr
+    float* dw; float* db;
+    int M, N, K, epi, accum_p;
+    int vec_k, vec_n;                    // rows of length K / N can be read 4 elements at a time
+    int split;                           // CTAs per cluster
+    int dx_clusters, dx_tiles_n, dw_tiles_n, dw_tiles;
+};
+
+enum { L_FWD, L_DX, L_DW };
+
+// One 32 x 64 tile over the contraction range [k0, k1).  Operands in shared memory as [row][contraction], double buffered; the next
+// chunk travels in registers while this one is used.
+template <typename T, int MODE>
+__device__ __forceinline__ void tile_product(const LinArgs& a, int row0, int col0, int k0, int k1, float* sm, float (&out)[4][4], float* bias_sum) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane & 7, cg = lane >> 3;
+    float2 acc[4][2], comp[4][2], part[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) acc[i][j] = comp[i][j] = make_float2(0.f, 0.f);
+    float4 ra[2], rb[4];
+    const T* const X = (const T*)a.x; const T* const W = (const T*)a.w; const T* const DY = (const T*)a.dy; const T* const Y = (const T*)a.y;
+    // column n of the tile sits in row (n / 16) * 16 + (n % 4) * 4 + (n % 16) / 4 of the B tile: a warp's four channel groups read neighbours
+    auto brow = [](int n) { return (n & ~15) + (n & 3) * 4 + ((n & 15) >> 2); };
+    auto fetch = [&](int kc) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = tid + u * LT;
+            if (MODE == L_FWD) ra[u] = fetch4(X, row0 + (i >> 3), kc + 4 * (i & 7), a.M, a.K, a.vec_k);
+            else if (MODE == L_DX) {
+                ra[u] = fetch4(DY, row0 + (i >> 3), kc + 4 * (i & 7), a.M, a.N, a.vec_n);
+                if (Y) ra[u] = masked(ra[u], fetch4(Y, row0 + (i >> 3), kc + 4 * (i & 7), a.M, a.N, a.vec_n));
+            } else {                     // sample i >> 3, four output features
+                ra[u] = fetch4(DY, kc + (i >> 3), row0 + 4 * (i & 7), a.M, a.N, a.vec_n);
+                if (Y) ra[u] = masked(ra[u], fetch4(Y, kc + (i >> 3), row0 + 4 * (i & 7), a.M, a.N, a.vec_n));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = tid + u * LT;
+            if (MODE == L_FWD) rb[u] = fetch4(W, col0 + (i >> 3), kc + 4 * (i & 7), a.N, a.K, a.vec_k);
+            else if (MODE == L_DX) rb[u] = fetch4(W, kc + (i >> 4), col0 + 4 * (i & 15), a.N, a.K, a.vec_k);
+            else rb[u] = fetch4(X, kc + (i >> 4), col0 + 4 * (i & 15), a.M, a.K, a.vec_k);
+        }
+    };
+    // what lies past k1 belongs to another CTA of the cluster (ranges are multiples of LK except the last, which ends with the matrix)
+    auto stash = [&](float* A, float* B) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = tid + u * LT;
+            if (MODE != L_DW) *(float4*)(A + (i >> 3) * LP + 4 * (i & 7)) = ra[u];
+            else {
+                const float v[4] = {ra[u].x, ra[u].y, ra[u].z, ra[u].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) A[(4 * (i & 7) + e) * LP + (i >> 3)] = v[e];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = tid + u * LT;
+            if (MODE == L_FWD) *(float4*)(B + brow(i >> 3) * LP + 4 * (i & 7)) = rb[u];
+            else {
+                const float v[4] = {rb[u].x, rb[u].y, rb[u].z, rb[u].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) B[brow(4 * (i & 15) + e) * LP + (i >> 4)] = v[e];
+            }
+        }
+    };
+    constexpr int BUF = (LM + LN) * LP;
+    const int chunks = k1 > k0 ? (k1 - k0 + LK - 1) / LK : 0;
+    if (chunks) fetch(k0);
+    float bsum = 0.f;
+    for (int c = 0; c < chunks; ++c) {
+        float* const A = sm + (c & 1) * BUF;
+        float* const B = A + LM * LP;
+        stash(A, B);
+        __syncthreads();                 // the other buffer's readers of chunk c - 1 have all passed here before chunk c + 1 overwrites it
+        if (c + 1 < chunks) fetch(k0 + (c + 1) * LK);
+        const float* const pa = A + g * LP;
+        const float* const pb = B + (warp * 16 + cg) * LP;
+#pragma unroll
+        for (int q = 0; q < LK / 4; ++q) {
+            float4 wv[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) wv[j] = *(const float4*)(pb + j * (4 * LP) + 4 * q);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 xv = *(const float4*)(pa + i * (8 * LP) + 4 * q);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 lo = make_float2(xv.x, xv.y), hi = make_float2(xv.z, xv.w);
+                    part[i][j] = q == 0 ? __fmul2_rn(lo, make_float2(wv[j].x, wv[j].y)) : __ffma2_rn(lo, make_float2(wv[j].x, wv[j].y), part[i][j]);
+                    part[i][j] = __ffma2_rn(hi, make_float2(wv[j].z, wv[j].w), part[i][j]);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const float2 s = make_float2(part[i][2 * j].x + part[i][2 * j].y, part[i][2 * j + 1].x + part[i][2 * j + 1].y);
+                const float2 yv = __fadd2_rn(s, make_float2(-comp[i][j].x, -comp[i][j].y));
+                const float2 t = __fadd2_rn(acc[i][j], yv);
+                const float2 d = __fadd2_rn(t, make_float2(-acc[i][j].x, -acc[i][j].y));
+                comp[i][j] = __fadd2_rn(d, make_float2(-yv.x, -yv.y));
+                acc[i][j] = t;
+            }
+        if (MODE == L_DW && bias_sum && tid < LM) {
+            float s = 0.f;
+#pragma unroll
+            for (int k = 0; k < LK; ++k) s += A[tid * LP + k];
+            bsum += s;
+        }
+    }
+    if (MODE == L_DW && bias_sum) *bias_sum = bsum;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { out[i][0] = acc[i][0].x; out[i][1] = acc[i][0].y; out[i][2] = acc[i][1].x; out[i][3] = acc[i][1].y; }
+}
+
+__device__ __forceinline__ uint32_t ctarank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ void cluster_sync() { asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ float4 ld_cluster(uint32_t local, uint32_t rank) {
+    uint32_t r; float4 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(r) : "memory");
+    return v;
+}
+
+// Four consecutive outputs of one row: bias, ReLU, accumulation, store (T, or fp32 with EPI_OUT_F32).
+template <typename T>
+__device__ __forceinline__ void emit(const LinArgs& a, int r, int c, int rows, int cols, float (&v)[4], const float* bias) {
+    if (r >= rows) return;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (c + j >= cols) continue;
+        const size_t o = (size_t)r * cols + c + j;
+        float t = v[j];
+        if (bias) t += bias[c + j];
+        if (a.epi & EPI_RELU) t = fmaxf(t, 0.f);
+        if (a.epi & EPI_OUT_F32) ((float*)a.out)[o] = t;
+        else {
+            T* const d = (T*)a.out + o;
+            if (a.epi & EPI_ACCUM) t += to_f(*d);
+            put(d, t);
+        }
+    }
+}
+
+// A tile that the cluster's CTAs have each done a part of: CTA `rank` adds rows rank, rank + split, ... over the CTAs in rank order.
+template <typename T>
+__device__ __forceinline__ void join_tile(const LinArgs& a, int row0, int col0, int rows, int cols, float (&v)[4][4], const float* bias, float* sm) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane & 7, cg = lane >> 3;
+    if (a.split == 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) emit<T>(a, row0 + g + 8 * i, col0 + warp * 16 + 4 * cg, rows, cols, v[i], bias);
+        return;
+    }
+    __syncthreads();                     // the operand buffers are no longer read
+    constexpr int TP = LN + 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) *(float4*)(sm + (g + 8 * i) * TP + warp * 16 + 4 * cg) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+    cluster_sync();
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm);
+    const int rank = (int)ctarank();
+    for (int e = tid; e < LM * LN / 4 / a.split; e += LT) {
+        const int r = (e / (LN / 4)) * a.split + rank, c = 4 * (e % (LN / 4));
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int q = 0; q < a.split; ++q) { const float4 t = ld_cluster(base + (uint32_t)(r * TP + c) * 4u, q); s[0] += t.x; s[1] += t.y; s[2] += t.z; s[3] += t.w; }
+        emit<T>(a, row0 + r, col0 + c, rows, cols, s, bias);
+    }
+    cluster_sync();                      // no CTA leaves while another reads its tile
+}
+
+__device__ __forceinline__ void my_range(int K, int split, int rank, int& k0, int& k1) {
+    const int per = ((K + split - 1) / split + LK - 1) / LK * LK;
+    k0 = min(K, rank * per); k1 = min(K, k0 + per);
+}
+
+// grid = column tiles x row tiles x split (the cluster) along x
+template <typename T>
+__global__ void __launch_bounds__(LT) lin_fwd_kernel(const LinArgs a) {
+    __shared__ __align__(16) float sm[2 * (LM + LN) * LP];
+    const int tile = blockIdx.x / a.split, rank = blockIdx.x % a.split;
+    const int tiles_n = (a.N + LN - 1) / LN, row0 = tile / tiles_n * LM, col0 = tile % tiles_n * LN;
+    int k0, k1; my_range(a.K, a.split, rank, k0, k1);
+    float v[4][4];
+    tile_product<T, L_FWD>(a, row0, col0, k0, k1, sm, v, nullptr);
+    join_tile<T>(a, row0, col0, a.M, a.N, v, a.bias, sm);
+}
+
+// The first dx_clusters clusters: input gradient; the others: `split` weight-gradient tiles each.
+template <typename T>
+__global__ void __launch_bounds__(LT) lin_bwd_kernel(const LinArgs a) {
+    __shared__ __align__(16) float sm[2 * (LM + LN) * LP];
+    const int cl = blockIdx.x / a.split, rank = blockIdx.x % a.split;
+    float v[4][4];
+    if (cl < a.dx_clusters) {
+        const int row0 = cl / a.dx_tiles_n * LM, col0 = cl % a.dx_tiles_n * LN;
+        int k0, k1; my_range(a.N, a.split, rank, k0, k1);
+        tile_product<T, L_DX>(a, row0, col0, k0, k1, sm, v, nullptr);
+        join_tile<T>(a, row0, col0, a.M, a.K, v, nullptr, sm);
+        return;
+    }
+    const int tile = (cl - a.dx_clusters) * a.split + rank;
+    if (tile >= a.dw_tiles) return;
+    const int row0 = tile / a.dw_tiles_n * LM, col0 = tile % a.dw_tiles_n * LN;
+    float bs = 0.f;
+    tile_product<T, L_DW>(a, row0, col0, 0, a.M, sm, v, a.db && col0 == 0 ? &bs : nullptr);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane & 7, cg = lane >> 3;
+    const int c = col0 + warp * 16 + 4 * cg;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = row0 + g + 8 * i;
+        if (r >= a.N || c >= a.K) continue;
+        float* const d = a.dw + (size_t)r * a.K + c;
+        if (a.vec_k && (((uintptr_t)a.dw) & 15) == 0) {
+            float4 o = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+            if (a.accum_p) { const float4 old = *(const float4*)d; o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w; }
+            *(float4*)d = o;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) if (c + j < a.K) d[j] = a.accum_p ? d[j] + v[i][j] : v[i][j];
+        }
+    }
+    if (a.db && col0 == 0 && tid < LM && row0 + tid < a.N) a.db[row0 + tid] = a.accum_p ? a.db[row0 + tid] + bs : bs;
+}
+
+// CTAs per cluster: as many as fill the device once (148 SMs, four CTAs each take the latency), a power of two up to 8 (the portable
+// cluster size), with at least two chunks of the contraction each.
+int pick_split(int tiles, int contraction) {
+    int s = 1;
+    while (s < 8 && tiles * s * 2 <= 148 * 2 && contraction >= s * 2 * 2 * LK) s *= 2;
+    return s;
+}
+bool aligned4(const void* p, int dt) { return ((uintptr_t)p & (dt ? 7 : 15)) == 0; }
+
+}  // namespace
+
+bool linear_supported(const ConvGeom& g) { return g.H * g.W == 1 && g.R == 1; }
+
+void linear_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, cudaStream_t s) {
+    LinArgs a{};
+    a.x = x; a.w = w; a.bias = bias; a.out = y; a.M = g.N; a.N = g.Co; a.K = g.C; a.epi = epi;
+    a.vec_k = g.C % 4 == 0 && aligned4(x, dt) && aligned4(w, dt);
+    const int tiles = ((a.M + LM - 1) / LM) * ((a.N + LN - 1) / LN);
+    a.split = pick_split(tiles, a.K);
+    const double esz = dt ? 2.0 : 4.0;
+    Scope sc(KC_FMA_FWD, 2.0 * a.M * a.N * a.K, esz * ((double)a.M * a.K + (double)a.N * a.K + (double)a.M * a.N), s);
+    if (dt) klaunch_cluster(lin_fwd_kernel<bf16>, tiles * a.split, LT, 0, s, a.split, a);
+    else klaunch_cluster(lin_fwd_kernel<float>, tiles * a.split, LT, 0, s, a.split, a);
+}
+
+void linear_backward(int dt, const void* x, const void* w, const void* y_or_null, const void* dy, void* dx_or_null, bool accum_dx, float* dw, float* db_or_null,
+                     const ConvGeom& g, bool accum_p, cudaStream_t s) {
+    LinArgs a{};
+    a.x = x; a.w = w; a.y = y_or_null; a.dy = dy; a.out = dx_or_null; a.dw = dw; a.db = db_or_null; a.M = g.N; a.N = g.Co; a.K = g.C;
+    a.epi = accum_dx ? EPI_ACCUM : 0; a.accum_p = accum_p;
+    a.vec_k = g.C % 4 == 0 && aligned4(x, dt) && aligned4(w, dt);
+    a.vec_n = g.Co % 4 == 0 && aligned4(dy, dt) && (!y_or_null || aligned4(y_or_null, dt));
+    a.dx_tiles_n = (a.K + LN - 1) / LN;
+    const int dx_tiles = dx_or_null ? ((a.M + LM - 1) / LM) * a.dx_tiles_n : 0;
+    a.split = dx_tiles ? pick_split(dx_tiles, a.N) : 1;
+    a.dx_clusters = dx_tiles;
+    a.dw_tiles_n = (a.K + LN - 1) / LN;
+    a.dw_tiles = ((a.N + LM - 1) / LM) * a.dw_tiles_n;
+    const int clusters = dx_tiles + (a.dw_tiles + a.split - 1) / a.split;
+    const double esz = dt ? 2.0 : 4.0;
+    Scope sc(KC_FMA_WGRAD, (dx_or_null ? 4.0 : 2.0) * a.M * a.N * a.K, esz * ((double)a.M * a.K * (dx_or_null ? 2 : 1) + (double)a.N * a.K + (double)a.M * a.N * (y_or_null ? 2 : 1)) + 4.0 * a.N * a.K, s);
+    if (dt) klaunch_cluster(lin_bwd_kernel<bf16>, clusters * a.split, LT, 0, s, a.split, a);
+    else klaunch_cluster(lin_bwd_kernel<float>, clusters * a.split, LT, 0, s, a.split, a);
+}
+
+}  // namespace fdg

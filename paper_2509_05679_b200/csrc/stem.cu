@@ -3,6 +3,7 @@
 // FMA kernels with register tiles; the weight gradient keeps a 64 x 27 accumulator tile per CTA across
 // many pixel tiles and reduces the per-CTA partials in a fixed order.
 #include "kernels.h"
+#include "launch.h"
 
 #include <cuda_bf16.h>
 
@@ -174,7 +175,7 @@ void stem_forward(const void* x, const void* w, const float* bias, void* y, cons
     dim3 grid(g.H / TH, g.N, g.Co / 64);
     const double pix = (double)g.N * g.H * g.W;
     Scope sc(KC_FMA_FWD, 2.0 * pix * g.Co * K, 2.0 * pix * (g.C + g.Co), s);
-    stem_fwd_kernel<<<grid, ST_THREADS, smem, s>>>((const bf16*)x, (const bf16*)w, bias, (bf16*)y, g.H, g.W, g.C, g.Co, relu);
+    klaunch(stem_fwd_kernel, grid, ST_THREADS, smem, s, (const bf16*)x, (const bf16*)w, bias, (bf16*)y, g.H, g.W, g.C, g.Co, relu);
 }
 
 void stem_wgrad(const void* x, const void* dy, float* dw, float* workspace, const ConvGeom& g, bool accum, cudaStream_t s) {
@@ -186,9 +187,9 @@ void stem_wgrad(const void* x, const void* dy, float* dw, float* workspace, cons
     const int blocks = tiles < stem_wgrad_blocks() ? tiles : stem_wgrad_blocks();
     const double pix = (double)g.N * g.H * g.W;
     { Scope sc(KC_FMA_WGRAD, 2.0 * pix * g.Co * K, 2.0 * pix * (g.C + g.Co), s);
-      stem_wgrad_kernel<<<dim3(blocks, 1, g.Co / 64), ST_THREADS, smem, s>>>((const bf16*)x, (const bf16*)dy, workspace, g.N, g.H, g.W, g.C, g.Co); }
+      klaunch(stem_wgrad_kernel, dim3(blocks, 1, g.Co / 64), ST_THREADS, smem, s, (const bf16*)x, (const bf16*)dy, workspace, g.N, g.H, g.W, g.C, g.Co); }
     Scope sc(KC_SPLITK, 0.0, 4.0 * blocks * g.Co * K, s);
-    stem_wgrad_reduce<<<(g.Co * K + 127) / 128, 128, 0, s>>>(workspace, dw, blocks, K, g.Co, accum);
+    klaunch(stem_wgrad_reduce, (g.Co * K + 127) / 128, 128, 0, s, workspace, dw, blocks, K, g.Co, accum);
 }
 
 }  // namespace fdg

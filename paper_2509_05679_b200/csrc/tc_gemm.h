@@ -119,6 +119,6 @@ struct UpdTable {
     UpdRange ranges[14];
 };
 cudaError_t run_update_module(const UpdTable& tb, float* master, const float* grad, void* wcopy, void* wtcopy, float* small_copy, float lr,
-                              bool has_grad, cudaStream_t s);
+                              bool has_grad, long long* stamp, cudaStream_t s);
 }  // namespace tc
 }  // namespace fdg

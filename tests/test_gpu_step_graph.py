@@ -1,0 +1,97 @@
+"""Steady-state iterations run as CUDA graphs whose kernels' parameters are refreshed (one graph per module, or two for
+networks with more work per step).  They must do what the kernel-by-kernel enqueuing does: bit-identical weights whatever
+the source of the inputs, whenever that source changes, and with profiling (which switches graphs off) in between; an input buffer
+may be overwritten as soon as fdg_wait_ingest returns; a new fdg_set_params starts over."""
+import numpy as np
+import pytest
+
+from paper_2509_05679_b200 import synth as sy
+from harness import make_ctx
+
+pytestmark = pytest.mark.gpu
+
+
+def nets():
+    small = sy.Net("mlp", sy.mlp_layers([70, 33, 65, 17, 5]), [2, 4, 6], 1, 1, 70, 5, 3, 7, 0.05, "fp32")      # one graph per module
+    one = sy.Net("mlp-k1", sy.mlp_layers([40, 32, 10]), [], 1, 1, 40, 10, 2, 9, 0.05, "fp32")                  # a single module
+    layers, bs = sy.resnet_layers(widths=(16, 32, 64), blocks=1)
+    large = sy.Net("resnet", layers, [bs[1], bs[2]], 32, 32, 3, 10, 4, 48, 0.05, "bf16")                       # two graphs per module
+    return {"small": small, "one": one, "large": large}
+
+
+def _run(net, p0, steps, how, reset_at=None, **kw):
+    """how(t) -> 'device', 'host' or 'profile' (device inputs, kernel by kernel)."""
+    import torch
+    ctx = make_ctx(net, p0, **kw)
+    dt = torch.bfloat16 if net.dtype == "bf16" else torch.float32
+    xb = torch.empty((net.M, net.in_h, net.in_w, net.in_c), dtype=dt, device="cuda")        # ONE buffer, overwritten before every step
+    yb = torch.empty(net.M, dtype=torch.int32, device="cuda")
+    losses = []
+    for t in range(steps):
+        if t == reset_at:
+            ctx.set_params(p0)
+        x, y = torch.from_numpy(sy.batch_inputs(net, t)).to(dt), torch.from_numpy(sy.batch_labels(net, t))
+        if how(t) == "host":
+            losses.append(ctx.step_host(x.pin_memory(), y.pin_memory(), want_loss=True))
+            ctx.wait_ingest()
+            continue
+        xb.copy_(x); yb.copy_(y)
+        torch.cuda.current_stream().synchronize()
+        if how(t) == "profile":
+            ctx.profile(True)
+        losses.append(ctx.step(xb, yb, want_loss=t % 3 == 0))
+        ctx.wait_ingest()
+        if how(t) == "profile":
+            ctx.profile(False)
+    out = ctx.params(), ctx.grads(), [np.nan if l is None else l for l in losses]
+    ms = ctx.module_times()
+    ctx.close()
+    assert np.all(ms > 0)
+    return out
+
+
+@pytest.mark.parametrize("name", ["small", "one", "large"])
+def test_sources_and_interruptions_do_not_change_the_weights(name):
+    net = nets()[name]
+    p0 = sy.perturb_params(sy.init_params(net.layers, 0, bf16=net.dtype == "bf16"), net.layers, 7, 0.1)
+    steps = 4 * net.K + 9
+    ref = _run(net, p0, steps, lambda t: "profile")                                       # never a graph
+    dev = _run(net, p0, steps, lambda t: "device")
+    assert np.array_equal(ref[0], dev[0]) and np.array_equal(ref[1], dev[1])
+    assert all(a == b for a, b in zip(ref[2], dev[2]) if not (np.isnan(a) or np.isnan(b)))
+    mixed = _run(net, p0, steps, lambda t: ("device", "host", "host", "profile", "device")[(t // 2) % 5])
+    assert np.array_equal(ref[0], mixed[0]) and np.array_equal(ref[1], mixed[1])
+    host = _run(net, p0, steps, lambda t: "host")
+    assert np.array_equal(ref[0], host[0])
+
+
+def test_set_params_starts_over():
+    net = nets()["small"]
+    p0 = sy.init_params(net.layers, 0)
+    a = _run(net, p0, 25, lambda t: "device", reset_at=12)
+    import torch
+    from paper_2509_05679_b200 import binding
+    ctx = make_ctx(net, p0)
+    for t in range(12, 25):
+        ctx.step(binding.to_device("fp32", sy.batch_inputs(net, t)), torch.from_numpy(sy.batch_labels(net, t)).cuda())
+        ctx.wait_ingest()
+    assert np.array_equal(a[0], ctx.params())
+    ctx.close()
+
+
+def test_two_contexts_interleaved():
+    import torch
+    from paper_2509_05679_b200 import binding
+    net = nets()["small"]
+    p = [sy.init_params(net.layers, s) for s in (0, 1)]
+    alone = [_run(net, q, 15, lambda t: "device")[0] for q in p]
+    ctxs = [make_ctx(net, q) for q in p]
+    for t in range(15):
+        x, y = binding.to_device("fp32", sy.batch_inputs(net, t)), torch.from_numpy(sy.batch_labels(net, t)).cuda()
+        for c in ctxs:
+            c.step(x, y)
+        for c in ctxs:
+            c.wait_ingest()
+    for c, a in zip(ctxs, alone):
+        assert np.array_equal(c.params(), a)
+        c.close()
