@@ -29,28 +29,35 @@ struct BnfArgs {
     long rpw; int C, relu, mask_from_x;
 };
 
-// (mean, invstd) of worker w from its tiles' (mean, sum of squared deviations, count):
-//   mean = sum n_t m_t / N,  N var = sum (q_t + n_t (m_t - mean)^2), in double, for the channels c0 .. c0 + nc - 1 (nc <= 256, a power
-// of two or a multiple of 256 handled by the caller's loop).  tmp: BT doubles.
-__device__ __forceinline__ void merge_tiles(const float* __restrict__ part, int tiles, int w, int nw, int C, int c0, int nc, long rows, float4* dst, double* tmp) {
+// (mean, invstd) of worker w from its tiles' (mean m_t, sum of squared deviations q_t, count n_t), in double, in one pass: with the first
+// tile's mean as the pivot p and d_t = m_t - p,  mean = p + S1 / N,  N var = S2 - S1^2 / N,  S1 = sum n_t d_t,  S2 = sum (q_t + n_t d_t^2);
+// for the channels c0 .. c0 + nc - 1 (nc <= BT, a power of two).  Every CTA of a normalising launch does this by itself, so it is the
+// launch's latency that counts: four records in flight per thread.  tmp: BT double2.
+__device__ __forceinline__ void merge_tiles(const float* __restrict__ part, int tiles, int w, int nw, int C, int c0, int nc, long rows, float4* dst, double2* tmp) {
     const int tid = threadIdx.x, lanes = BT / nc, c = tid % nc, pt = tid / nc;
     const float2* p = (const float2*)part + (size_t)w * tiles * C + c0 + c;
     const float* cnt = part + (size_t)nw * tiles * C * 2 + (size_t)w * tiles;
-    double s = 0.0;
-    for (int t = pt; t < tiles; t += lanes) s += (double)cnt[t] * (double)p[(size_t)t * C].x;
-    tmp[tid] = s;
+    const double pivot = (double)p[0].x;
+    double s1 = 0.0, s2 = 0.0;
+    auto add = [&](float2 v, float n) { const double d = (double)v.x - pivot, nd = (double)n * d; s1 += nd; s2 += (double)v.y + nd * d; };
+    int t = pt;
+    for (; t + 3 * lanes < tiles; t += 4 * lanes) {
+        float2 v[4]; float n[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { v[u] = p[(size_t)(t + u * lanes) * C]; n[u] = cnt[t + u * lanes]; }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) add(v[u], n[u]);
+    }
+    for (; t < tiles; t += lanes) add(p[(size_t)t * C], cnt[t]);
+    tmp[tid] = make_double2(s1, s2);
     __syncthreads();
-    double mean = 0.0;
-    for (int q = 0; q < lanes; ++q) mean += tmp[q * nc + c];
-    mean /= (double)rows;
-    __syncthreads();
-    s = 0.0;
-    for (int t = pt; t < tiles; t += lanes) { const float2 v = p[(size_t)t * C]; const double d = (double)v.x - mean; s += (double)v.y + (double)cnt[t] * d * d; }
-    tmp[tid] = s;
-    __syncthreads();
+    for (int d = lanes / 2; d > 0; d >>= 1) {
+        if (pt < d) { const double2 o = tmp[tid + d * nc]; tmp[tid].x += o.x; tmp[tid].y += o.y; }
+        __syncthreads();
+    }
     if (pt == 0) {
-        double m2 = 0.0;
-        for (int q = 0; q < lanes; ++q) m2 += tmp[q * nc + c];
+        const double2 a = tmp[c];
+        const double mean = pivot + a.x / (double)rows, m2 = fmax(a.y - a.x * a.x / (double)rows, 0.0);
         const double istd = 1.0 / sqrt(m2 / (double)rows + 1e-5);
         const float mh = (float)mean, ih = (float)istd;
         dst[c] = make_float4(mh, ih, (float)(mean - (double)mh), (float)(istd - (double)ih));
@@ -60,7 +67,7 @@ __device__ __forceinline__ void merge_tiles(const float* __restrict__ part, int 
 
 // stats only (bf16 storage: the streamed apply kernel of kernels.cu follows).  grid = (channel blocks of min(C, 64), workers)
 __global__ void __launch_bounds__(BT) bn_merge_tiles_k(const float* __restrict__ part, float* __restrict__ stats, int tiles, int C, int nc, long rows) {
-    __shared__ double tmp[BT];
+    __shared__ double2 tmp[BT];
     __shared__ float4 res[BT];
     const int c0 = blockIdx.x * nc, w = blockIdx.y;
     merge_tiles(part, tiles, w, gridDim.y, C, c0, nc, rows, res, tmp);
@@ -95,7 +102,7 @@ __device__ __forceinline__ float2 warp_sum(float2 v) {
 // MODE 2: dx (+)= gamma * invstd * (dy - mean(dy) - xhat * mean(dy xhat)), dres (+)= dy, dgamma, dbeta.
 template <int MODE>
 __global__ void __launch_bounds__(BT) bnf_kernel(const BnfArgs a) {
-    __shared__ double tmp[BT];
+    __shared__ double2 tmp[BT];
     __shared__ float4 st4[1024];                 // MODE 0: statistics; MODE 2: (sum dy, sum dy xhat); MODE 1: reduction
     float2* const st = (float2*)st4;
     const int C = a.C, cgs = C / 4, rows_it = BT / cgs, tid = threadIdx.x, cg = tid % cgs, rl = tid / cgs;

@@ -31,7 +31,8 @@ constexpr int FC_CO = 16;
 constexpr int FC_KC = 16;                // channels per chunk
 constexpr int PITCH = 20;                // floats per pixel (or weight row) in shared memory: 16 + 4, so that the eight 16-byte reads
                                          // of neighbouring pixels fall into different banks
-constexpr int FW_THREADS = 288;          // 9 taps x 2 groups of 8 c_in x 4 groups of 4 c_out x 4 pixel slices
+constexpr int FW_THREADS = 160;          // 9 taps x 2 groups of 8 c_in x 4 groups of 4 c_out x 2 pixel slices = 144, in five warps: three CTAs put
+                                         // four warps on each scheduler and leave 128 registers a thread (nine warps, two CTAs: 96, and spills)
 constexpr int FW_CO = 16, FW_CI = 16;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -96,6 +97,14 @@ __device__ __forceinline__ void load_region(const bool VEC, const T* __restrict_
 template <typename T> __device__ __forceinline__ float stored(float v);
 template <> __device__ __forceinline__ float stored<float>(float v) { return v; }
 template <> __device__ __forceinline__ float stored<bf16>(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
+
+// sum += part, compensated: part, which started at what the sum lost last time, becomes what it loses this time
+__device__ __forceinline__ void kahan(float2& sum, float2& part) {
+    const float2 t = __fadd2_rn(sum, part);
+    const float2 d = __fadd2_rn(t, make_float2(-sum.x, -sum.y));
+    part = __fadd2_rn(part, make_float2(-d.x, -d.y));
+    sum = t;
+}
 
 struct Yes { static constexpr bool value = true; };
 struct No { static constexpr bool value = false; };
@@ -321,14 +330,19 @@ struct FwParams {
 };
 
 // grid = (splits, c_out blocks x c_in blocks, groups).  Thread = 4 c_out x 8 c_in of one tap, for one slice of every tile's
-// pixels.  dy is kept twice in shared memory ((d, d) pairs: the multiplier of a packed FMA), x as in fc_kernel.
+// pixels.  dy is kept twice in shared memory ((d, d) pairs: the multiplier of a packed FMA), x as in fc_kernel.  While a tile is used, the
+// next one's x is on its way into the other buffer (fp32: cp.async) and its dy into registers.
+// Compensated sum: a chain of FW_CHAIN products starts at what the running sum lost at its last addition, so that the compensation
+// costs neither registers nor an instruction of its own.  (Chains of 32 lose sqrt(2) more than chains of 16; the error of the whole is
+// that of the sum over the splits, of which no lane of fw_reduce_kernel adds more than 56 one after the other.)
 // part: [group][block][split][16 c_out][taps][8 * G c_in]
+constexpr int FW_CHAIN = 32;
+constexpr int FW_DYV = 4;                                    // float4s of dy per thread and tile: 128 pixels x 4 / 160 threads
 template <typename T, int XS, int G, int RUN>
-__global__ void __launch_bounds__(FW_THREADS, 2) fw_kernel(const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ part_out,
+__global__ void __launch_bounds__(FW_THREADS, 3) fw_kernel(const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ part_out,
                                                            const __grid_constant__ FwParams p) {
     extern __shared__ __align__(16) float fsm[];
-    float* const xs_ = fsm;
-    float* const ds_ = fsm + p.x_floats;                     // [pixel][16][2]
+    float* const ds_ = fsm + 2 * p.x_floats;                 // [pixel][16][2]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int grp = blockIdx.z, cob = blockIdx.y / p.ci_blocks, cib = blockIdx.y % p.ci_blocks;
     const int co0 = cob * FW_CO, ci0 = cib * FW_CI;
@@ -337,79 +351,83 @@ __global__ void __launch_bounds__(FW_THREADS, 2) fw_kernel(const T* __restrict__
     const int cog = rest & 3, ng = rest >> 2, tap = ng / G, half = ng - tap * G;
     const bool active = slice < p.nslices;
     const int npix = p.Wt * p.Ht * p.Nt;
-    float2 acc[4][4], comp[4][4];                            // [c_out][c_in pair]
+    float2 acc[4][4], part[4][4];                            // [c_out][c_in pair]
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) { acc[i][j] = make_float2(0.f, 0.f); comp[i][j] = make_float2(0.f, 0.f); }
-    const float* const xt = xs_ + (active ? p.toff[tap] : 0) + half * 8;
+        for (int j = 0; j < 4; ++j) { acc[i][j] = make_float2(0.f, 0.f); part[i][j] = make_float2(0.f, 0.f); }
+    const int xoff = (active ? p.toff[tap] : 0) + half * 8;
     const float* const dt = ds_ + cog * 8;
     const int per = (p.tiles + p.splits - 1) / p.splits;
-    const int tile_end = min(p.tiles, ((int)blockIdx.x + 1) * per);
-    for (int tile = blockIdx.x * per; tile < tile_end; ++tile) {
-        int tl = tile;
+    const int tile0 = blockIdx.x * per, tile_end = min(p.tiles, tile0 + per), n_end = (grp + 1) * p.ngroup;
+    float4 dv[FW_DYV];
+    auto fetch = [&](int tl, int buf) {
         const int tw = tl % p.tiles_w; tl /= p.tiles_w;
         const int th = tl % p.tiles_h, tn = tl / p.tiles_h;
-        const int n_end = (grp + 1) * p.ngroup, n0 = grp * p.ngroup + tn * p.Nt;
-        const int ho0 = th * p.Ht, wo0 = tw * p.Wt;
-        __syncthreads();                                     // the previous tile is consumed
-        load_region<T>((p.C & 3) == 0, x, xs_, n0, n_end, p.Nt, ho0 * p.hstep - p.pad, wo0 * p.hstep - p.pad, p.RH, p.RW, p.step, p.H, p.W, p.C, ci0,
-                            G == 2 ? 4 : 2, warp, FW_THREADS / 32, lane);
+        const int n0 = grp * p.ngroup + tn * p.Nt, ho0 = th * p.Ht, wo0 = tw * p.Wt;
+        load_region<T>((p.C & 3) == 0, x, fsm + buf * p.x_floats, n0, n_end, p.Nt, ho0 * p.hstep - p.pad, wo0 * p.hstep - p.pad, p.RH, p.RW, p.step, p.H, p.W, p.C,
+                       ci0, G == 2 ? 4 : 2, warp, FW_THREADS / 32, lane);
         cp_commit();
-        for (int i = tid; i < npix * 4; i += FW_THREADS) {
+#pragma unroll
+        for (int u = 0; u < FW_DYV; ++u) {
+            const int i = tid + u * FW_THREADS;
+            dv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (i >= npix * 4) continue;
             const int px = i >> 2, q = i & 3;
             const int w = wo0 + (px & (p.Wt - 1)), h = ho0 + ((px >> p.lw) & (p.Ht - 1)), n = n0 + (px >> (p.lw + p.lh));
-            const bool ok = n < n_end && h < p.Ho && w < p.Wo;
             const int c = co0 + 4 * q;
-            const T* s = dy + (((size_t)(ok ? n : 0) * p.Ho + (ok ? h : 0)) * p.Wo + (ok ? w : 0)) * p.Co;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if ((p.Co & 3) == 0) { if (ok && c < p.Co) v = ld4(s + c); }
-            else if (ok) {
-                v.x = c < p.Co ? to_f(s[c]) : 0.f; v.y = c + 1 < p.Co ? to_f(s[c + 1]) : 0.f;
-                v.z = c + 2 < p.Co ? to_f(s[c + 2]) : 0.f; v.w = c + 3 < p.Co ? to_f(s[c + 3]) : 0.f;
-            }
-            float* d = ds_ + px * 32 + q * 8;
-            *(float4*)d = make_float4(v.x, v.x, v.y, v.y);
-            *(float4*)(d + 4) = make_float4(v.z, v.z, v.w, v.w);
+            if (n >= n_end || h >= p.Ho || w >= p.Wo || c >= p.Co) continue;
+            const T* s = dy + (((size_t)n * p.Ho + h) * p.Wo + w) * p.Co + c;
+            if ((p.Co & 3) == 0) dv[u] = ld4(s);
+            else { dv[u].x = to_f(s[0]); dv[u].y = c + 1 < p.Co ? to_f(s[1]) : 0.f; dv[u].z = c + 2 < p.Co ? to_f(s[2]) : 0.f; dv[u].w = c + 3 < p.Co ? to_f(s[3]) : 0.f; }
+        }
+    };
+    if (tile0 < tile_end) fetch(tile0, 0);
+    for (int tile = tile0; tile < tile_end; ++tile) {
+        const int buf = (tile - tile0) & 1;
+#pragma unroll
+        for (int u = 0; u < FW_DYV; ++u) {
+            const int i = tid + u * FW_THREADS;
+            if (i >= npix * 4) continue;
+            float* d = ds_ + (i >> 2) * 32 + (i & 3) * 8;
+            *(float4*)d = make_float4(dv[u].x, dv[u].x, dv[u].y, dv[u].y);
+            *(float4*)(d + 4) = make_float4(dv[u].z, dv[u].z, dv[u].w, dv[u].w);
         }
         cp_wait<0>();
         __syncthreads();
-        if (!active) continue;
-        for (int r = 0; r < p.pps; r += 16) {                // 16 pixels = one compensated step
-            float2 part[4][4];
+        if (tile + 1 < tile_end) fetch(tile + 1, buf ^ 1);
+        if (active) {
+            const float* const xt = fsm + buf * p.x_floats + xoff;
+#pragma unroll 1
+            for (int r = 0; r < p.pps; r += FW_CHAIN) {
 #pragma unroll
-            for (int rr = 0; rr < 16; rr += RUN) {
-                const int px = slice * p.pps + r + rr;
-                if (rr > 0 && r + rr >= p.pps) break;
-                const int pw = px & (p.Wt - 1), ph = (px >> p.lw) & (p.Ht - 1), pn = px >> (p.lw + p.lh);
-                const float* xp = xt + ((pn * p.RH + ph * XS) * p.RW + pw * XS) * PITCH;
-                const float* dp = dt + px * 32;
+                for (int rr = 0; rr < FW_CHAIN; rr += RUN) {
+                    const int px = slice * p.pps + r + rr;
+                    if (rr > 0 && r + rr >= p.pps) break;
+                    const int pw = px & (p.Wt - 1), ph = (px >> p.lw) & (p.Ht - 1), pn = px >> (p.lw + p.lh);
+                    const float* xp = xt + ((pn * p.RH + ph * XS) * p.RW + pw * XS) * PITCH;
+                    const float* dp = dt + px * 32;
 #pragma unroll
-                for (int k = 0; k < RUN; ++k) {
-                    const float4 xa = *(const float4*)(xp + k * XS * PITCH), xc = *(const float4*)(xp + k * XS * PITCH + 4);
-                    const float4 d0 = *(const float4*)(dp + k * 32), d1 = *(const float4*)(dp + k * 32 + 4);
-                    const float2 xv[4] = {make_float2(xa.x, xa.y), make_float2(xa.z, xa.w), make_float2(xc.x, xc.y), make_float2(xc.z, xc.w)};
-                    const float2 dv[4] = {make_float2(d0.x, d0.y), make_float2(d0.z, d0.w), make_float2(d1.x, d1.y), make_float2(d1.z, d1.w)};
+                    for (int k = 0; k < RUN; ++k) {
+                        const float4 xa = *(const float4*)(xp + k * XS * PITCH), xc = *(const float4*)(xp + k * XS * PITCH + 4);
+                        const float4 d0 = *(const float4*)(dp + k * 32), d1 = *(const float4*)(dp + k * 32 + 4);
+                        const float2 xv[4] = {make_float2(xa.x, xa.y), make_float2(xa.z, xa.w), make_float2(xc.x, xc.y), make_float2(xc.z, xc.w)};
+                        const float2 d2[4] = {make_float2(d0.x, d0.y), make_float2(d0.z, d0.w), make_float2(d1.x, d1.y), make_float2(d1.z, d1.w)};
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
+                        for (int i = 0; i < 4; ++i)
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) part[i][j] = rr == 0 && k == 0 ? __fmul2_rn(dv[i], xv[j]) : __ffma2_rn(dv[i], xv[j], part[i][j]);
+                            for (int j = 0; j < 4; ++j) part[i][j] = __ffma2_rn(d2[i], xv[j], part[i][j]);
+                    }
                 }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) kahan(acc[i][j], part[i][j]);
             }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 yv = __fadd2_rn(part[i][j], make_float2(-comp[i][j].x, -comp[i][j].y));
-                    const float2 t = __fadd2_rn(acc[i][j], yv);
-                    const float2 d = __fadd2_rn(t, make_float2(-acc[i][j].x, -acc[i][j].y));
-                    comp[i][j] = __fadd2_rn(d, make_float2(-yv.x, -yv.y));
-                    acc[i][j] = t;
-                }
         }
+        __syncthreads();                                     // dy and this x buffer are consumed
     }
     // the slices' sums in slice order, then the CTA's partial matrix
-    __syncthreads();
     const int nout = FW_CO * p.ntaps * 8 * G;
     float* const red = fsm;                                  // [slice][16][taps][8 G]
     if (active) {
@@ -428,7 +446,7 @@ __global__ void __launch_bounds__(FW_THREADS, 2) fw_kernel(const T* __restrict__
     }
 }
 
-// dW[c_out][tap][c_in] = sum over the splits; 8 lanes per element take every 8th split, then a fixed tree.
+// dW[c_out][tap][c_in] = sum over the splits (at most 444): 8 lanes per element take every 8th split, eight loads in flight each, then a fixed tree.
 __global__ void __launch_bounds__(256) fw_reduce_kernel(const float* __restrict__ part, float* __restrict__ dw, int splits, int nout, int ntaps, int cw, int ci_blocks,
                                                         int C, int Co, size_t w_group, bool accum) {
     __shared__ float sh[8][33];
@@ -438,9 +456,12 @@ __global__ void __launch_bounds__(256) fw_reduce_kernel(const float* __restrict_
     float s = 0.f;
     if (e < nout) {
         int k = ty;
-        for (; k + 24 < splits; k += 32) {                   // four loads in flight
-            const float a = src[(size_t)k * nout], b = src[(size_t)(k + 8) * nout], c = src[(size_t)(k + 16) * nout], d = src[(size_t)(k + 24) * nout];
-            s += (a + b) + (c + d);
+        for (; k + 56 < splits; k += 64) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = src[(size_t)(k + 8 * u) * nout];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) s += v[u];
         }
         for (; k < splits; k += 8) s += src[(size_t)k * nout];
     }
@@ -476,7 +497,7 @@ Tile pick_tile(int H, int W, int pixels) {
     return t;
 }
 
-constexpr size_t FC_SMEM_MAX = 200 * 1024;
+constexpr size_t FC_SMEM_MAX = 224 * 1024;
 
 // Geometry of a forward (back == 0) or input-gradient launch over `groups` groups of g.N / groups images; false: not covered.
 bool plan_fc(const ConvGeom& g, int groups, bool back, FcParams& p) {
@@ -549,10 +570,10 @@ void dispatch_fc(const void* x, const void* w, const float* bias, void* y, float
     else { if (vec) launch_fc<T, 4, true>(x, w, bias, y, stat, p, groups, s); else launch_fc<T, 4, false>(x, w, bias, y, stat, p, groups, s); }
 }
 
-// Weight gradient: 256 pixels per tile (128 for 3x3 stride 2, whose input region is four times its output).
+// Weight gradient: 128 pixels per tile (64 for 3x3 stride 2, whose input region is four times its output).
 bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_t& smem) {
     if ((g.H * g.W == 1 && g.R == 1) || (g.R != 3 && g.R != 1) || (g.stride != 1 && g.stride != 2) || g.N % groups) return false;
-  for (int pixels = g.R == 3 && g.stride == 2 ? 128 : 256; pixels >= 32; pixels /= 2) {        // smaller tiles where the halo of tiny images outgrows shared memory
+  for (int pixels = g.R == 3 && g.stride == 2 ? 64 : 128; pixels >= 32; pixels /= 2) {        // smaller tiles where the halo of tiny images outgrows shared memory
     p = FwParams{};
     const Tile t = pick_tile(g.Ho, g.Wo, pixels);
     run = t.Wt >= 8 ? 8 : (t.Wt >= 4 ? 4 : 1);
@@ -573,15 +594,15 @@ bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_
     p.pps = npix / p.nslices;
     p.ci_blocks = (g.C + FW_CI - 1) / FW_CI;
     const int blocks = p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO) * groups;
-    // two CTAs per SM once around the device, each with at least one tile
-    int want = 2 * 148 / blocks;
+    // three CTAs per SM once around the device, each with at least one tile
+    int want = 3 * 148 / blocks;
     if (want > p.tiles) want = p.tiles;
     if (want < 1) want = 1;
     p.max_splits = want;
     const int per = (p.tiles + want - 1) / want;
     p.splits = (p.tiles + per - 1) / per;
     p.x_floats = t.Nt * p.RH * p.RW * PITCH;
-    smem = ((size_t)p.x_floats + (size_t)npix * 32) * sizeof(float);
+    smem = ((size_t)2 * p.x_floats + (size_t)npix * 32) * sizeof(float);
     const size_t red = (size_t)p.nslices * FW_CO * p.ntaps * 8 * G * sizeof(float);
     if (red > smem) smem = red;
     if (smem <= FC_SMEM_MAX) return true;

@@ -419,6 +419,7 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             if (o.stem) m.ws_elems = std::max(m.ws_elems, stem_wgrad_workspace_elems(o.g));
             if (o.stem_tc) m.ws_elems = std::max(m.ws_elems, tc::stem_wg_workspace_elems(o.g.Co, (long)o.g.N * o.g.H, ctx->grid_sms));
             m.ws_elems = std::max(m.ws_elems, wgrad_workspace_elems(o.g));
+            if (ctx->R > 1) m.ws_elems = std::max(m.ws_elems, fconv_wgrad_workspace_elems(o.g, ctx->R));
             m.scratch_elems = std::max(m.scratch_elems, (size_t)64 * o.g.Co);
             if (relu_bias_backward_supported(ctx->dt, o.g.Co)) m.scratch_elems = std::max(m.scratch_elems, relu_bias_backward_scratch_elems(o.g.Co));
         }
@@ -596,16 +597,17 @@ size_t row_off(const fdg_ctx* c, const TensorDesc& d, const Win& wn) {
     return (size_t)wn.n0 * d.elems() * (d.loc == LOC_LOGITS ? sizeof(float) : (size_t)c->esz);
 }
 
-void forward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int group) {
+// The ops [i0, i1) of a module's forward pass on one group's rows.
+void forward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int group, size_t i0, size_t i1) {
     Module& m = c->mod[kk];
     StepPtrs P{c, &m, kk, batch};
     const Win wn = group_window(c, m, group);
     const int rep = c->R > 1 ? group : 0;               // worker `group` runs on its own weights w_{s,k}
     cudaStream_t s = m.fstream;
     const int dt = c->dt;
-    m.fused_stats_tensor[0] = m.fused_stats_tensor[1] = -1;
     auto T = [&](int id) { return P.tensor(id) + row_off(c, m.t[id], wn); };
-    for (const Op& o : m.ops) {
+    for (size_t i = i0; i < i1; ++i) {
+        const Op& o = m.ops[i];
         const TensorDesc& ti = m.t[o.in];
         const TensorDesc& to = m.t[o.out];
         size_t n_out = to.elems() * wn.n;
@@ -675,6 +677,65 @@ void forward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int grou
     }
 }
 
+// One op on ALL workers' rows, every worker's with its own weight replica, in one launch.  false: this op has to be run worker by worker.
+bool forward_op_replicas(fdg_ctx* c, int kk, int64_t batch, int64_t version, size_t i) {
+    Module& m = c->mod[kk];
+    StepPtrs P{c, &m, kk, batch};
+    cudaStream_t s = m.fstream;
+    const int dt = c->dt;
+    const Op& o = m.ops[i];
+    const TensorDesc& ti = m.t[o.in];
+    const TensorDesc& to = m.t[o.out];
+    const size_t wg = m.wslot_bytes / c->esz, pg = m.wslot_bytes / sizeof(float);        // between replicas: matrices, vectors
+    switch (o.type) {
+        case OP_CONV: {
+            const int epi = (o.relu ? EPI_RELU : 0) | (to.loc == LOC_LOGITS ? EPI_OUT_F32 : 0);
+            const char* const w = wbig(c, m, version, o.w_off);
+            const float* const b = o.bias ? wsmall(c, m, version, o.b_off) : nullptr;
+            profile_detail(o.shape);
+            bool ok = true;
+            if (linear_supported(o.g)) linear_forward(dt, P.tensor(o.in), w, b, P.tensor(o.out), o.g, epi, c->R, wg, pg, s);
+            else ok = fconv_forward(dt, P.tensor(o.in), w, b, P.tensor(o.out), o.g, epi, c->R, wg, pg, o.fstat_tiles ? m.cstat[o.stat_buf] : nullptr, s);
+            if (ok && o.fstat_tiles) { m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.fstat_tiles; }
+            profile_detail(nullptr);
+            return ok; }
+        case OP_BN:
+            if (!o.bn_from_conv) return false;
+            if (dt != 0) {               // statistics of all workers, then the streamed apply kernel with each worker's parameters
+                const long rpw = (long)c->B * ti.h * ti.w;
+                bn_merge_tiles(m.cstat[o.stat_buf], P.stats(o), m.fused_stats_chunks[o.stat_buf], c->n_workers, rpw, ti.c, s);
+                for (int r = 0; r < c->R; ++r) {
+                    const Win wn = group_window(c, m, r);
+                    auto T = [&](int id) { return P.tensor(id) + row_off(c, m.t[id], wn); };
+                    bn_forward(dt, T(o.in), wsmall(c, m, version, o.gamma_off, r), wsmall(c, m, version, o.beta_off, r), o.has_res ? T(o.in2) : nullptr, T(o.out),
+                               P.stats(o) + (size_t)r * ti.c * 2, m.scratch_f, 1, rpw, ti.c, o.relu, nullptr, -1, c->grid_sms, c->tc_err, s);
+                }
+                return true;
+            }
+            bnf_forward((const float*)P.tensor(o.in), wsmall(c, m, version, o.gamma_off), wsmall(c, m, version, o.beta_off), pg,
+                        o.has_res ? (const float*)P.tensor(o.in2) : nullptr, (float*)P.tensor(o.out), P.stats(o), m.cstat[o.stat_buf], m.fused_stats_chunks[o.stat_buf],
+                        c->n_workers, (long)c->B * ti.h * ti.w, ti.c, o.relu, s);
+            return true;
+        case OP_RELU: relu_forward(dt, P.tensor(o.in), P.tensor(o.out), to.elems() * c->M, s); return true;
+        case OP_POOL: maxpool_forward(dt, P.tensor(o.in), P.tensor(o.out), c->M, ti.h, ti.w, ti.c, s); return true;
+        case OP_GAP: gap_forward(dt, P.tensor(o.in), P.tensor(o.out), c->M, ti.h * ti.w, ti.c, s); return true;
+        case OP_ADD: add_forward(dt, P.tensor(o.in), P.tensor(o.in2), P.tensor(o.out), to.elems() * c->M, s); return true;
+    }
+    return false;
+}
+
+void forward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version) {
+    Module& m = c->mod[kk];
+    m.fused_stats_tensor[0] = m.fused_stats_tensor[1] = -1;
+    if (c->R == 1) {
+        for (int g = 0; g < m.groups; ++g) { forward_ops(c, kk, batch, version, g, 0, m.ops.size()); m.fused_stats_tensor[0] = m.fused_stats_tensor[1] = -1; }
+        return;
+    }
+    for (size_t i = 0; i < m.ops.size(); ++i)
+        if (!forward_op_replicas(c, kk, batch, version, i))
+            for (int g = 0; g < m.groups; ++g) forward_ops(c, kk, batch, version, g, i, i + 1);
+}
+
 // gradient buffer of a tensor during iteration t
 char* grad_ptr(fdg_ctx* c, int kk, int id, int64_t t) {
     Module& m = c->mod[kk];
@@ -686,7 +747,8 @@ char* grad_ptr(fdg_ctx* c, int kk, int id, int64_t t) {
     return n.d2 + (size_t)((t - 1) & 1) * n.in_slot_bytes;
 }
 
-void backward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t, int group) {
+// The ops i1 - 1 down to i0 of a module's backward pass on one group's rows.
+void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t, int group, int i0, int i1) {
     Module& m = c->mod[kk];
     StepPtrs P{c, &m, kk, batch};
     const Win wn = group_window(c, m, group);
@@ -698,7 +760,7 @@ void backward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t
     auto T = [&](int id) { return P.tensor(id) + row_off(c, m.t[id], wn); };
     // gradients are stored in the storage dtype (also the one of the logits)
     auto G = [&](int id) -> char* { char* b = grad_ptr(c, kk, id, t); return b ? b + (size_t)wn.n0 * m.t[id].elems() * c->esz : nullptr; };
-    for (int i = (int)m.ops.size() - 1; i >= 0; --i) {
+    for (int i = i1 - 1; i >= i0; --i) {
         const Op& o = m.ops[i];
         const TensorDesc& ti = m.t[o.in];
         const TensorDesc& to = m.t[o.out];
@@ -718,7 +780,7 @@ void backward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t
                 if (!o.tc && linear_supported(g)) {
                     profile_detail(o.shape);
                     linear_backward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.relu ? T(o.out) : nullptr, gout, gin, o.acc_in, mgrad + o.w_off,
-                                    o.bias ? mgrad + m.n_big + o.b_off : nullptr, g, acc_p, s);
+                                    o.bias ? mgrad + m.n_big + o.b_off : nullptr, g, 1, 0, 0, acc_p, s);
                     profile_detail(nullptr);
                     break;
                 }
@@ -768,6 +830,66 @@ void backward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t
                 break; }
         }
     }
+}
+
+// See forward_op_replicas: every worker's own gradient g_{s,k} (replica s of m.grad).
+bool backward_op_replicas(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t, int i) {
+    Module& m = c->mod[kk];
+    StepPtrs P{c, &m, kk, batch};
+    cudaStream_t s = m.stream;
+    const int dt = c->dt;
+    const Op& o = m.ops[i];
+    const TensorDesc& ti = m.t[o.in];
+    const size_t wg = m.wslot_bytes / c->esz, pg = m.wslot_bytes / sizeof(float), gg = npar(m);
+    const size_t n_in = ti.elems() * c->M;
+    char* const gout = grad_ptr(c, kk, o.out, t);
+    char* const gin = grad_ptr(c, kk, o.in, t);
+    switch (o.type) {
+        case OP_CONV: {
+            char* const w = wbig(c, m, version, o.w_off);
+            if (linear_supported(o.g)) {
+                profile_detail(o.shape);
+                linear_backward(dt, P.tensor(o.in), w, o.relu ? P.tensor(o.out) : nullptr, gout, gin, o.acc_in, m.grad + o.w_off,
+                                o.bias ? m.grad + m.n_big + o.b_off : nullptr, o.g, c->R, wg, gg, false, s);
+                profile_detail(nullptr);
+                return true;
+            }
+            if (o.bias || o.relu) return false;
+            profile_detail(o.shape);
+            cudaStream_t ws = m.wstream;
+            if (ws != s) { step_record(m.wev, s); step_wait(ws, m.wev); }
+            fconv_wgrad(dt, P.tensor(o.in), gout, m.grad + o.w_off, m.ws, o.g, c->R, gg, false, ws);
+            if (gin) fconv_dgrad(dt, gout, w, gin, o.g, o.acc_in ? EPI_ACCUM : 0, c->R, wg, s);
+            profile_detail(nullptr);
+            return true; }
+        case OP_BN:
+            if (dt != 0 || !o.bn_from_conv) return false;
+            bnf_backward((const float*)P.tensor(o.in), (const float*)P.tensor(o.out), (const float*)gout, wsmall(c, m, version, o.gamma_off),
+                         wsmall(c, m, version, o.beta_off), pg, P.stats(o), (float*)gin, o.acc_in, o.has_res ? (float*)grad_ptr(c, kk, o.in2, t) : nullptr, o.acc_in2,
+                         m.grad + m.n_big + o.gamma_off, m.grad + m.n_big + o.beta_off, gg, m.scratch, c->n_workers, (long)c->B * ti.h * ti.w, ti.c, o.relu,
+                         o.relu && !o.has_res, false, s);
+            return true;
+        case OP_RELU: if (gin) relu_backward(dt, P.tensor(o.out), gout, gin, n_in, o.acc_in, s); return true;
+        case OP_POOL: if (gin) maxpool_backward(dt, P.tensor(o.in), gout, gin, c->M, ti.h, ti.w, ti.c, o.acc_in, s); return true;
+        case OP_GAP: if (gin) gap_backward(dt, gout, gin, c->M, ti.h * ti.w, ti.c, o.acc_in, s); return true;
+        case OP_ADD: {
+            if (gin) copy_or_accumulate(dt, gout, gin, n_in, o.acc_in, s);
+            if (char* g2 = grad_ptr(c, kk, o.in2, t)) copy_or_accumulate(dt, gout, g2, n_in, o.acc_in2, s);
+            return true; }
+    }
+    return false;
+}
+
+void backward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t) {
+    Module& m = c->mod[kk];
+    const int n = (int)m.ops.size();
+    if (c->R == 1) {
+        for (int g = 0; g < m.groups; ++g) backward_ops(c, kk, batch, version, t, g, 0, n);
+        return;
+    }
+    for (int i = n - 1; i >= 0; --i)
+        if (!backward_op_replicas(c, kk, batch, version, t, i))
+            for (int g = 0; g < m.groups; ++g) backward_ops(c, kk, batch, version, t, g, i, i + 1);
 }
 
 // Emit the transposed (and tap-flipped) copies of weight version `version` that the input-gradient kernel reads.
@@ -987,7 +1109,7 @@ fdg_status module_step(fdg_ctx* ctx, int kk, int64_t t, const Ingest* in, int pa
     }
 
     if (part & FORWARD) {
-    if (tau_f >= 0) for (int g = 0; g < m.groups; ++g) forward_module(ctx, kk, tau_f, t, g);
+    if (tau_f >= 0) forward_module(ctx, kk, tau_f, t);
     if (part == WHOLE) CK(step_record(m.fdone, m.fstream));
     }
     if (!(part & BACKWARD)) return FDG_OK;
@@ -1001,7 +1123,7 @@ fdg_status module_step(fdg_ctx* ctx, int kk, int64_t t, const Ingest* in, int pa
         else if (!fused_head) softmax_ce(ctx->dt, ctx->logits, ctx->labels + (size_t)(tau_f % ctx->label_depth) * ctx->M, ctx->dlogits, rec, ctx->tc_err, t + 1,
                                          ctx->M, ctx->classes, ctx->R > 1 ? 1.f / (float)ctx->B : 1.f / (float)ctx->M, m.stream);
     }
-    if (tau_b >= 0) for (int g = 0; g < m.groups; ++g) backward_module(ctx, kk, tau_b, v_b, t, g);
+    if (tau_b >= 0) backward_module(ctx, kk, tau_b, v_b, t);
     // Eq. dl_update with P = 11^T/N: w(t+1) = w(t) - lr * averaged gradient; also emits version t+1
     // (after the forward pass has read version t: with a one-slot ring the update overwrites it)
     if (part == WHOLE && !lastm && m.fstream != m.stream) CK(step_wait(m.stream, m.fdone));

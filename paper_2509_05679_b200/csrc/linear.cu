@@ -53,7 +53,23 @@ struct LinArgs {
     int vec_k, vec_n;                    // rows of length K / N can be read 4 elements at a time
     int split;                           // CTAs per cluster
     int dx_clusters, dx_tiles_n, dw_tiles_n, dw_tiles;
+    size_t w_group, b_group, g_group;    // grid.y groups of M samples each: elements between their weights, biases, parameter gradients
 };
+
+// the arguments of group blockIdx.y
+template <typename T>
+__device__ __forceinline__ LinArgs of_group(const LinArgs& in, bool fwd) {
+    LinArgs a = in;
+    const size_t g = blockIdx.y, mk = g * a.M * a.K, mn = g * a.M * a.N;
+    a.x = (const T*)a.x + mk; a.w = (const T*)a.w + g * a.w_group;
+    if (a.dy) a.dy = (const T*)a.dy + mn;
+    if (a.y) a.y = (const T*)a.y + mn;
+    if (a.bias) a.bias += g * a.b_group;
+    if (a.out) a.out = (a.epi & EPI_OUT_F32) ? (void*)((float*)a.out + mn) : (void*)((T*)a.out + (fwd ? mn : mk));
+    if (a.dw) a.dw += g * a.g_group;
+    if (a.db) a.db += g * a.g_group;
+    return a;
+}
 
 enum { L_FWD, L_DX, L_DW };
 
@@ -227,7 +243,8 @@ __device__ __forceinline__ void my_range(int K, int split, int rank, int& k0, in
 
 // grid = column tiles x row tiles x split (the cluster) along x
 template <typename T>
-__global__ void __launch_bounds__(LT) lin_fwd_kernel(const LinArgs a) {
+__global__ void __launch_bounds__(LT) lin_fwd_kernel(const LinArgs args) {
+    const LinArgs a = of_group<T>(args, true);
     __shared__ __align__(16) float sm[2 * (LM + LN) * LP];
     const int tile = blockIdx.x / a.split, rank = blockIdx.x % a.split;
     const int tiles_n = (a.N + LN - 1) / LN, row0 = tile / tiles_n * LM, col0 = tile % tiles_n * LN;
@@ -239,7 +256,8 @@ __global__ void __launch_bounds__(LT) lin_fwd_kernel(const LinArgs a) {
 
 // The first dx_clusters clusters: input gradient; the others: `split` weight-gradient tiles each.
 template <typename T>
-__global__ void __launch_bounds__(LT) lin_bwd_kernel(const LinArgs a) {
+__global__ void __launch_bounds__(LT) lin_bwd_kernel(const LinArgs args) {
+    const LinArgs a = of_group<T>(args, false);
     __shared__ __align__(16) float sm[2 * (LM + LN) * LP];
     const int cl = blockIdx.x / a.split, rank = blockIdx.x % a.split;
     float v[4][4];
@@ -262,7 +280,7 @@ __global__ void __launch_bounds__(LT) lin_bwd_kernel(const LinArgs a) {
         const int r = row0 + g + 8 * i;
         if (r >= a.N || c >= a.K) continue;
         float* const d = a.dw + (size_t)r * a.K + c;
-        if (a.vec_k && (((uintptr_t)a.dw) & 15) == 0) {
+        if ((a.K & 3) == 0 && (((uintptr_t)a.dw) & 15) == 0) {
             float4 o = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
             if (a.accum_p) { const float4 old = *(const float4*)d; o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w; }
             *(float4*)d = o;
@@ -287,36 +305,38 @@ bool aligned4(const void* p, int dt) { return ((uintptr_t)p & (dt ? 7 : 15)) == 
 
 bool linear_supported(const ConvGeom& g) { return g.H * g.W == 1 && g.R == 1; }
 
-void linear_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, cudaStream_t s) {
+void linear_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
+                    cudaStream_t s) {
     LinArgs a{};
-    a.x = x; a.w = w; a.bias = bias; a.out = y; a.M = g.N; a.N = g.Co; a.K = g.C; a.epi = epi;
-    a.vec_k = g.C % 4 == 0 && aligned4(x, dt) && aligned4(w, dt);
+    a.x = x; a.w = w; a.bias = bias; a.out = y; a.M = g.N / groups; a.N = g.Co; a.K = g.C; a.epi = epi; a.w_group = w_group; a.b_group = b_group;
+    a.vec_k = g.C % 4 == 0 && w_group % 4 == 0 && aligned4(x, dt) && aligned4(w, dt);
     const int tiles = ((a.M + LM - 1) / LM) * ((a.N + LN - 1) / LN);
-    a.split = pick_split(tiles, a.K);
+    a.split = pick_split(tiles * groups, a.K);
     const double esz = dt ? 2.0 : 4.0;
-    Scope sc(KC_FMA_FWD, 2.0 * a.M * a.N * a.K, esz * ((double)a.M * a.K + (double)a.N * a.K + (double)a.M * a.N), s);
-    if (dt) klaunch_cluster(lin_fwd_kernel<bf16>, tiles * a.split, LT, 0, s, a.split, a);
-    else klaunch_cluster(lin_fwd_kernel<float>, tiles * a.split, LT, 0, s, a.split, a);
+    Scope sc(KC_FMA_FWD, 2.0 * g.N * a.N * a.K, esz * ((double)a.M * a.K + (double)a.N * a.K + (double)a.M * a.N), s);
+    if (dt) klaunch_cluster(lin_fwd_kernel<bf16>, dim3(tiles * a.split, groups), LT, 0, s, a.split, a);
+    else klaunch_cluster(lin_fwd_kernel<float>, dim3(tiles * a.split, groups), LT, 0, s, a.split, a);
 }
 
 void linear_backward(int dt, const void* x, const void* w, const void* y_or_null, const void* dy, void* dx_or_null, bool accum_dx, float* dw, float* db_or_null,
-                     const ConvGeom& g, bool accum_p, cudaStream_t s) {
+                     const ConvGeom& g, int groups, size_t w_group, size_t g_group, bool accum_p, cudaStream_t s) {
     LinArgs a{};
-    a.x = x; a.w = w; a.y = y_or_null; a.dy = dy; a.out = dx_or_null; a.dw = dw; a.db = db_or_null; a.M = g.N; a.N = g.Co; a.K = g.C;
+    a.x = x; a.w = w; a.y = y_or_null; a.dy = dy; a.out = dx_or_null; a.dw = dw; a.db = db_or_null; a.M = g.N / groups; a.N = g.Co; a.K = g.C;
+    a.w_group = w_group; a.g_group = g_group;
     a.epi = accum_dx ? EPI_ACCUM : 0; a.accum_p = accum_p;
-    a.vec_k = g.C % 4 == 0 && aligned4(x, dt) && aligned4(w, dt);
+    a.vec_k = g.C % 4 == 0 && w_group % 4 == 0 && aligned4(x, dt) && aligned4(w, dt);
     a.vec_n = g.Co % 4 == 0 && aligned4(dy, dt) && (!y_or_null || aligned4(y_or_null, dt));
     a.dx_tiles_n = (a.K + LN - 1) / LN;
     const int dx_tiles = dx_or_null ? ((a.M + LM - 1) / LM) * a.dx_tiles_n : 0;
-    a.split = dx_tiles ? pick_split(dx_tiles, a.N) : 1;
+    a.split = dx_tiles ? pick_split(dx_tiles * groups, a.N) : 1;
     a.dx_clusters = dx_tiles;
     a.dw_tiles_n = (a.K + LN - 1) / LN;
     a.dw_tiles = ((a.N + LM - 1) / LM) * a.dw_tiles_n;
     const int clusters = dx_tiles + (a.dw_tiles + a.split - 1) / a.split;
     const double esz = dt ? 2.0 : 4.0;
-    Scope sc(KC_FMA_WGRAD, (dx_or_null ? 4.0 : 2.0) * a.M * a.N * a.K, esz * ((double)a.M * a.K * (dx_or_null ? 2 : 1) + (double)a.N * a.K + (double)a.M * a.N * (y_or_null ? 2 : 1)) + 4.0 * a.N * a.K, s);
-    if (dt) klaunch_cluster(lin_bwd_kernel<bf16>, clusters * a.split, LT, 0, s, a.split, a);
-    else klaunch_cluster(lin_bwd_kernel<float>, clusters * a.split, LT, 0, s, a.split, a);
+    Scope sc(KC_FMA_WGRAD, (dx_or_null ? 4.0 : 2.0) * g.N * a.N * a.K, esz * ((double)a.M * a.K * (dx_or_null ? 2 : 1) + (double)a.N * a.K + (double)a.M * a.N * (y_or_null ? 2 : 1)) + 4.0 * a.N * a.K, s);
+    if (dt) klaunch_cluster(lin_bwd_kernel<bf16>, dim3(clusters * a.split, groups), LT, 0, s, a.split, a);
+    else klaunch_cluster(lin_bwd_kernel<float>, dim3(clusters * a.split, groups), LT, 0, s, a.split, a);
 }
 
 }  // namespace fdg

@@ -40,3 +40,31 @@ def test_bf16_storage(orc, shape):
 @pytest.mark.parametrize("workers,batch", [(1, 1), (2, 130), (5, 3)])
 def test_batch_sizes(orc, workers, batch):
     run_parity(orc, _net(((8, 8), 16, sy.CONV3X3, 32, 2), "fp32", workers, batch, True), 2, param_tol=1e-5, loss_tol=1e-5)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_replicas_in_one_launch_equal_the_single_copy_path(dtype):
+    """With P = (1/N) 1 1^T given explicitly every worker has its own weights and gradients; convolutions, batch-norm and linear layers run
+    once for all of them.  Same weights as the single-copy path up to the rounding of another summation order, relative to what the
+    steps changed (fp32: 1e-4, ten steps' roundings of 1e-6 with a margin; bf16 storage: the 2e-2 of the bf16 gradients)."""
+    import numpy as np
+    import torch
+    from paper_2509_05679_b200 import binding
+    layers, bs = sy.resnet_layers(widths=(8, 16), blocks=1)
+    net = sy.without_relu(sy.Net("replicas", layers, [bs[0], bs[1]], 8, 8, 3, 10, 3, 5, 0.05, dtype))
+    p0 = sy.perturb_params(sy.init_params(net.layers, 0, bf16=dtype == "bf16"), net.layers, 7, 0.1)
+    kw = dict(dtype=dtype, in_shape=(8, 8, 3), num_classes=10)
+    a = binding.Context(net.layers, net.splits, 3, 5, net.lr, mixing=np.full((3, 3), 1.0 / 3), **kw)
+    b = binding.Context(net.layers, net.splits, 3, 5, net.lr, kernel_path=1, **kw)
+    for c in (a, b):
+        c.set_params(p0)
+    for t in range(2 * net.K + 3):
+        x, y = binding.to_device(dtype, sy.batch_inputs(net, t)), torch.from_numpy(sy.batch_labels(net, t)).cuda()
+        for c in (a, b):
+            c.step(x, y)
+            c.wait_ingest()
+    pb = b.params()
+    for s in range(3):
+        err = np.linalg.norm(a.params_worker(s) - pb) / np.linalg.norm(pb - p0)          # of what the steps changed
+        assert err <= (1e-4 if dtype == "fp32" else 2e-2), (s, err)
+    a.close(); b.close()
