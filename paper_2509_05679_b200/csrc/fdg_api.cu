@@ -67,6 +67,7 @@ struct Op {
     bool head;                                               // the network's last linear layer: fused with the loss (head_* kernels)
     char shape[40];                                          // "HxW Cin->Cout kR sS", the profiler's detail tag
     int n_tile_f, n_tile_d, n_tile_w, wg_splits;
+    bool small_f, small_d;                                   // few tiles: forward / input gradient by tc::run_small (n_tile_f / n_tile_d = 64)
     tc::KmParams kf;
     tc::KmParams kd;                                         // all output-parity classes of the input gradient in one launch
     bool dgrad_needs_zero;                                   // some parity classes receive no gradient (1x1 stride 2)
@@ -291,6 +292,13 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             o.n_tile_f = g.Co % 256 == 0 ? 256 : (g.Co % 128 == 0 ? 128 : 64);
             o.n_tile_d = g.C % 256 == 0 ? 256 : (g.C % 128 == 0 ? 128 : 64);
             o.n_tile_w = g.Co % 256 == 0 ? 256 : (g.Co % 128 == 0 ? 128 : 64);
+            {
+                const long pix = (long)(g.Wo / wt) * (g.Ho / ht) * ((g.N + nt - 1) / nt);
+                o.small_f = tc::small_problem(pix * (g.Co / 64));
+                o.small_d = tc::small_problem(pix * (g.C / 64) * g.stride * g.stride);
+                if (o.small_f) o.n_tile_f = 64;
+                if (o.small_d) o.n_tile_d = 64;
+            }
             tc::pixel_tile(g.Ho, g.Wo, 64, &wt, &ht, &nt);
             int row_blocks = g.R * g.R * g.C / 64;
             long ptiles = (long)(g.Wo / wt) * (g.Ho / ht) * ((g.N + nt - 1) / nt);
@@ -518,7 +526,7 @@ bool tc_forward(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* y_base, 
     const int io = find_buf(o.y_ptrs, y_base);
     const tc::KmMaps maps{&o.fa[ia], o.far.empty() ? nullptr : &o.far[ia], &o.fb[version % m.D], o.fbh.empty() ? nullptr : &o.fbh[version % m.D],
                           io >= 0 ? &o.fo[io] : nullptr};
-    const bool ok = tc::run_km(maps, p, o.n_tile_f, s) == cudaSuccess;
+    const bool ok = (o.small_f ? tc::run_small(*maps.a, *maps.b, p, s) : tc::run_km(maps, p, o.n_tile_f, s)) == cudaSuccess;
     if (ok && o.stat_chunks) { m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.stat_chunks; }
     return ok;
 }
@@ -540,7 +548,7 @@ bool tc_dgrad(fdg_ctx* c, Module& m, const Op& o, char* dy_base, char* dx_base, 
     const int io = find_buf(o.dx_ptrs, dx_base);
     const tc::KmMaps maps{&o.da[ia], o.dar.empty() ? nullptr : &o.dar[ia], &o.db[version % m.D], o.dbh.empty() ? nullptr : &o.dbh[version % m.D],
                           io >= 0 ? &o.dox[io] : nullptr};
-    return tc::run_km(maps, p, o.n_tile_d, s) == cudaSuccess;
+    return (o.small_d ? tc::run_small(*maps.a, *maps.b, p, s) : tc::run_km(maps, p, o.n_tile_d, s)) == cudaSuccess;
 }
 bool tc_wgrad(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* dy_base, float* dw, const Win& wn, cudaStream_t s) {
     int ix = find_buf(o.a_ptrs, x_base), id = find_buf(o.dy_ptrs, dy_base);
@@ -968,7 +976,7 @@ bool build_tc_plans(fdg_ctx* c) {
             o.fo.resize(o.y_ptrs.size());
             for (size_t i = 0; i < o.y_ptrs.size(); ++i) ok = ok && tc::make_map_out(&o.fo[i], o.y_ptrs[i], g.Co, g.Wo, g.Ho, g.N, wt, ht);
             const bool pairs = c->kernel_path == 0;          // CTA-pair kernels for the 256-column tile (kernel_path 2: none)
-            if (pairs && (o.n_tile_f >= 256 || (rows_ok && o.n_tile_f == 128))) {
+            if (pairs && !o.small_f && (o.n_tile_f >= 256 || (rows_ok && o.n_tile_f == 128))) {
                 o.fbh.resize(m.D);
                 for (int v = 0; v < m.D; ++v) ok = ok && tc::make_map_2d(&o.fbh[v], wbig(c, m, v, o.w_off), Ktot, g.Co, 64, o.n_tile_f / 2);
             }
@@ -1009,7 +1017,7 @@ bool build_tc_plans(fdg_ctx* c) {
             }
             o.db.resize(m.D);
             for (int v = 0; v < m.D; ++v) ok = ok && tc::make_map_2d(&o.db[v], wtslot(m, v, o.w_off), (long)taps * g.Co, g.C, 64, o.n_tile_d);
-            if (pairs && (o.n_tile_d >= 256 || (rows_ok && o.n_tile_d == 128))) {
+            if (pairs && !o.small_d && (o.n_tile_d >= 256 || (rows_ok && o.n_tile_d == 128))) {
                 o.dbh.resize(m.D);
                 for (int v = 0; v < m.D; ++v) ok = ok && tc::make_map_2d(&o.dbh[v], wtslot(m, v, o.w_off), (long)taps * g.Co, g.C, 64, o.n_tile_d / 2);
             }

@@ -272,8 +272,8 @@ constexpr int EPI_BUF_BYTES = 32 * EPI_SLICE * 2; // one staged slice: 32 rows x
 // One 64-column slice of a warp's 32 accumulator rows (v: this lane's row): bias / ReLU / accumulation into the stored
 // gradient, rounding to bf16, the staged copy in shared memory (stg: one EPI_BUF_BYTES buffer), the store (a TMA store of
 // the box at (cx, cw, chh, cn) of tmO, or row by row through rowptr), and the per-column sums for a following batch-norm.
-// bias, rowptr and stat_dst already point at the slice's first column (or are null).
-__device__ __forceinline__ void epi_slice(uint32_t (&v)[EPI_SLICE], const float* bias, int epi, unsigned long long rowptr, unsigned vmask, bool ok,
+// maskptr: this lane's row of the mask tensor.  bias, rowptr, maskptr and stat_dst already point at the slice's first column (or are null).
+__device__ __forceinline__ void epi_slice(uint32_t (&v)[EPI_SLICE], const float* bias, int epi, unsigned long long rowptr, unsigned long long maskptr, unsigned vmask, bool ok,
                                           bool tma_out, const CUtensorMap* tmO, int cx, int cw, int chh, int cn, uint32_t stg, int lane,
                                           float* stat_dst) {
     const uint32_t swz = (uint32_t)(lane & 7);
@@ -300,6 +300,19 @@ __device__ __forceinline__ void epi_slice(uint32_t (&v)[EPI_SLICE], const float*
             for (int j = 0; j < 4; ++j) {
                 v[8 * g + 2 * j] = __float_as_uint(__uint_as_float(v[8 * g + 2 * j]) + __uint_as_float(w4[j] << 16));
                 v[8 * g + 2 * j + 1] = __float_as_uint(__uint_as_float(v[8 * g + 2 * j + 1]) + __uint_as_float(w4[j] & 0xffff0000u));
+            }
+        }
+    }
+    if (maskptr) {
+        const uint4* o = (const uint4*)((const bf16*)maskptr);
+#pragma unroll
+        for (int g = 0; g < EPI_SLICE / 8; ++g) {
+            const uint4 mk = __ldg(o + g);
+            const uint32_t w4[4] = {mk.x, mk.y, mk.z, mk.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (!(__uint_as_float(w4[j] << 16) > 0.f)) v[8 * g + 2 * j] = 0u;
+                if (!(__uint_as_float(w4[j] & 0xffff0000u) > 0.f)) v[8 * g + 2 * j + 1] = 0u;
             }
         }
     }
@@ -598,6 +611,7 @@ km_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         int ti = 0;
         bool ok = true;
         const bool tma_out = p.tma_out != 0;
+        const unsigned long long mask_off = (unsigned long long)p.mask - (unsigned long long)p.out;
         const uint32_t tmem_empty0 = PAIR ? map_to_cta(smem_u32(&tmem_empty[0]), 0) : 0u;
         // this lane's row of the tile, and the first row of the warp, as (pixel column, pixel row, sample) inside the tile
         const int row = q * 32 + lane;
@@ -617,6 +631,7 @@ km_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
             const unsigned long long rowptr = valid ? (unsigned long long)((bf16*)p.out + (((size_t)n * p.Ho + (h * p.os + p.cls_oph[cls])) * p.Wo +
                                                                                                 (w * p.os + p.cls_opw[cls])) * p.Co + co0) : 0ull;
             const unsigned vmask = __ballot_sync(0xffffffffu, rowptr != 0ull);
+            const size_t rec = (size_t)(cls * (p.tiles_w * p.tiles_h * p.tiles_n) + tmi) * 4 + q;
             ok = mbar_wait_sleep(&tmem_full[buf], use & 1, p.err, 3);
             tc_fence_after();
 #pragma unroll 1
@@ -631,9 +646,10 @@ km_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                     __syncwarp();
                     if (lane == 0) { if (PAIR) mbar_arrive_cluster(tmem_empty0 + 8 * buf); else mbar_arrive(&tmem_empty[buf]); }
                 }
-                epi_slice(v, p.bias ? p.bias + co0 + c : nullptr, p.epi, rowptr ? rowptr + 2ull * c : 0ull, vmask, ok, tma_out, &tmO, co0 + c,
+                epi_slice(v, p.bias ? p.bias + co0 + c : nullptr, p.epi, rowptr ? rowptr + 2ull * c : 0ull, p.mask && rowptr ? rowptr + mask_off + 2ull * c : 0ull, vmask, ok, tma_out,
+                          &tmO, co0 + c,
                           tw * p.Wt + bw0, th * p.Ht + bh0, p.n_base + tn * p.Nt + bn0, stg0 + sbuf * EPI_BUF_BYTES, lane,
-                          p.stat_part ? p.stat_part + (((size_t)tmi * 4 + q) * p.Cn + co0 + c) * 2 : nullptr);
+                          p.stat_part ? p.stat_part + (rec * p.Cn + co0 + c) * 2 : nullptr);
                 sbuf ^= 1u;
             }
         }
@@ -645,6 +661,215 @@ km_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     __syncwarp();
     if (PAIR) cluster_sync_all(); else __syncthreads();       // neither CTA of a pair leaves while the other may still signal it
     if (warp == 1) { tc_fence_after(); if (PAIR) tmem_dealloc_pair(tmem_base, TMEM_COLS); else tmem_dealloc(tmem_base, TMEM_COLS); }
+}
+
+// ------------------------------------------------------------------------------------------ few tiles
+// The same computation when there are fewer tiles than SMs (a few hundred samples through a linear layer, 4x4 images of a small
+// batch): km_kernel then runs a handful of CTAs through the whole contraction, 16 to 72 steps one after the other (17-35 us).
+// Here a tile is 128 pixels x 64 columns, a cluster of S CTAs takes equal parts of its contraction, every CTA leaves its fp32
+// partial tile in shared memory, and CTA r adds the columns [64 r / S, 64 (r + 1) / S) over the cluster in rank order (a fixed order).
+// One tile per cluster, four stages of 24 KB (two CTAs per SM).
+constexpr int KS_STAGES = 4, KS_STAGE_BYTES = BLOCK_M * 128 + 64 * 128, KS_PITCH = 68;        // floats per row of the partial tile
+static_assert(KS_STAGES * KS_STAGE_BYTES >= BLOCK_M * KS_PITCH * 4, "the partial tile reuses the stages");
+template <int S>
+__global__ void __launch_bounds__(NUM_THREADS, 2)
+ks_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, KmParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = align1024(smem_raw);
+    uint64_t* full = (uint64_t*)(smem + KS_STAGES * KS_STAGE_BYTES);
+    uint64_t* empty = full + KS_STAGES;
+    uint64_t* accum_bar = empty + KS_STAGES;
+    uint32_t* tmem_slot = (uint32_t*)(accum_bar + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = S > 1 ? (int)cluster_rank() : 0, tile = (int)blockIdx.x / S;
+    const int tiles_m = p.tiles_w * p.tiles_h * p.tiles_n, tiles_c = p.Cn / 64, per_cls = tiles_m * tiles_c;
+    const int cls = tile / per_cls, tl = tile - cls * per_cls;
+    int tm = tl / tiles_c;
+    const int co0 = (tl - tm * tiles_c) * 64;
+    const int tmi = tm + (p.n_base / p.Nt) * (p.tiles_h * p.tiles_w);
+    const int tw = tm % p.tiles_w; tm /= p.tiles_w;
+    const int th = tm % p.tiles_h, tn = tm / p.tiles_h;
+    const int tap0 = p.cls_tap0[cls], kb_total = (p.cls_tap0[cls + 1] - tap0) * p.kchunks;
+    const int kb0 = kb_total * rank / S, num_kb = kb_total * (rank + 1) / S - kb0;
+
+    if (threadIdx.x == 0) {
+        tma_prefetch_desc(&tmA); tma_prefetch_desc(&tmB);
+        for (int s = 0; s < KS_STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+        mbar_init(accum_bar, 1);
+        fence_barrier_init();
+    }
+    if (warp == 1) tmem_alloc(tmem_slot, 64);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+
+    if (warp == 0) {
+        const int w0 = tw * p.Wt * p.xs, h0 = th * p.Ht * p.xs, n0 = p.n_base + tn * p.Nt;
+        int tap = tap0 + kb0 / p.kchunks, kc = kb0 % p.kchunks;
+        const uint32_t smem0 = smem_u32(smem), full0 = smem_u32(full), empty0 = smem_u32(empty);
+        uint32_t st = 0, ph = 1;
+        for (int kb = 0; kb < num_kb; ++kb) {
+            if (!mbar_wait_a(empty0 + 8 * st, ph, p.err, 31)) break;
+            if (elect_one()) {
+                const uint32_t dst = smem0 + st * KS_STAGE_BYTES, fb = full0 + 8 * st;
+                mbar_expect_tx_a(fb, KS_STAGE_BYTES);
+                tma_load_4d_a(dst, &tmA, fb, kc * BLOCK_K, w0 + p.dw[tap], h0 + p.dh[tap], n0);
+                tma_load_2d_a(dst + BLOCK_M * 128, &tmB, fb, p.koff[tap] + kc * BLOCK_K, co0);
+            }
+            __syncwarp();
+            if (++kc == p.kchunks) { kc = 0; ++tap; }
+            if (++st == KS_STAGES) { st = 0; ph ^= 1u; }
+        }
+    } else if (warp == 1) {
+        const uint32_t idesc = make_idesc(BLOCK_M, 64, 0, 0);
+        const uint64_t dconst = make_desc(0, 16, 1024);
+        const uint32_t d_hi = (uint32_t)(dconst >> 32), d_lo = (uint32_t)dconst, a16_0 = smem_u32(smem) >> 4;
+        const uint32_t full0 = smem_u32(full), empty0 = smem_u32(empty);
+        uint32_t st = 0, ph = 0;
+        for (int kb = 0; kb < num_kb; ++kb) {
+            if (!mbar_wait_a(full0 + 8 * st, ph, p.err, 32)) break;
+            tc_fence_after();
+            const uint32_t a_lo = d_lo + a16_0 + st * (KS_STAGE_BYTES >> 4), b_lo = a_lo + (BLOCK_M * 128 >> 4);
+            if (elect_one()) {
+#pragma unroll
+                for (int k = 0; k < BLOCK_K / UMMA_K; ++k) umma_bf16_w<false>(tmem_base, a_lo + 2 * k, b_lo + 2 * k, d_hi, idesc, kb > 0 || k > 0 ? 1u : 0u);
+                umma_commit_a<false>(empty0 + 8 * st);
+                if (kb == num_kb - 1) umma_commit(accum_bar);
+            }
+            __syncwarp();
+            if (++st == KS_STAGES) { st = 0; ph ^= 1u; }
+        }
+    }
+    constexpr int NC = 64 / S;                           // columns this CTA finishes
+    const int q = warp & 3, row = q * 32 + lane;
+    const uint32_t part = smem_u32(smem);
+    float v[NC];
+    bool ok = true;
+    if (warp >= 2) {
+        ok = num_kb > 0 ? mbar_wait(accum_bar, 0, p.err, 33) : true;
+        tc_fence_after();
+        const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
+        if (S == 1) {
+            uint32_t u[64];
+            tmem_ld32_nowait(taddr, u);
+            tmem_ld32_nowait(taddr + 32, u + 32);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < NC; ++j) v[j] = num_kb > 0 ? __uint_as_float(u[j]) : 0.f;
+        } else {
+#pragma unroll
+            for (int c = 0; c < 64; c += 32) {
+                uint32_t u[32];
+                tmem_ld32(taddr + c, u);
+#pragma unroll
+                for (int g = 0; g < 8; ++g) {
+                    if (num_kb == 0) u[4 * g] = u[4 * g + 1] = u[4 * g + 2] = u[4 * g + 3] = 0u;
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(part + (uint32_t)(row * KS_PITCH + c + 4 * g) * 4u), "r"(u[4 * g]), "r"(u[4 * g + 1]),
+                                 "r"(u[4 * g + 2]), "r"(u[4 * g + 3]) : "memory");
+                }
+            }
+        }
+    }
+    __syncwarp();
+    if (S > 1) cluster_sync_all();
+    if (warp >= 2) {
+        const int c0 = rank * NC;
+        if (S > 1) {
+#pragma unroll
+            for (int j = 0; j < NC; ++j) v[j] = 0.f;
+#pragma unroll
+            for (int r = 0; r < S; ++r) {
+                const uint32_t src = map_to_cta(part + (uint32_t)(row * KS_PITCH + c0) * 4u, (uint32_t)r);
+                float4 t[NC / 4];
+#pragma unroll
+                for (int g = 0; g < NC / 4; ++g)
+                    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t[g].x), "=f"(t[g].y), "=f"(t[g].z), "=f"(t[g].w) : "r"(src + 16u * g) : "memory");
+#pragma unroll
+                for (int g = 0; g < NC / 4; ++g) { v[4 * g] += t[g].x; v[4 * g + 1] += t[g].y; v[4 * g + 2] += t[g].z; v[4 * g + 3] += t[g].w; }
+            }
+        }
+        const int pw = row % p.Wt, ph = (row / p.Wt) % p.Ht, pn = row / (p.Wt * p.Ht);
+        const int n = p.n_base + tn * p.Nt + pn, h = th * p.Ht + ph, w = tw * p.Wt + pw;
+        const bool valid = ok && n < p.N && h < p.Hd && w < p.Wd;
+        const size_t off = (((size_t)(valid ? n : 0) * p.Ho + (h * p.os + p.cls_oph[cls])) * p.Wo + (w * p.os + p.cls_opw[cls])) * p.Co + co0 + c0;
+        bf16* const out = (bf16*)p.out + off;
+        const bf16* const mask = p.mask ? (const bf16*)p.mask + off : nullptr;
+        if (p.bias) {
+#pragma unroll
+            for (int j = 0; j < NC; j += 4) {
+                const float4 b = __ldg((const float4*)(p.bias + co0 + c0 + j));
+                v[j] += b.x; v[j + 1] += b.y; v[j + 2] += b.z; v[j + 3] += b.w;
+            }
+        }
+        uint32_t pk[NC / 2];
+#pragma unroll
+        for (int g = 0; g < NC / 8; ++g) {
+            float* const f = v + 8 * g;
+            if (p.epi & EPI_RELU) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) f[j] = fmaxf(f[j], 0.f);
+            }
+            if ((p.epi & EPI_ACCUM) && valid) {
+                const uint4 old = *(const uint4*)(out + 8 * g);
+                const uint32_t w4[4] = {old.x, old.y, old.z, old.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) { f[2 * j] += __uint_as_float(w4[j] << 16); f[2 * j + 1] += __uint_as_float(w4[j] & 0xffff0000u); }
+            }
+            if (mask && valid) {
+                const uint4 mk = __ldg((const uint4*)(mask + 8 * g));
+                const uint32_t w4[4] = {mk.x, mk.y, mk.z, mk.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (!(__uint_as_float(w4[j] << 16) > 0.f)) f[2 * j] = 0.f;
+                    if (!(__uint_as_float(w4[j] & 0xffff0000u) > 0.f)) f[2 * j + 1] = 0.f;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const __nv_bfloat162 t = __floats2bfloat162_rn(f[2 * j], f[2 * j + 1]);
+                pk[4 * g + j] = *(const uint32_t*)&t;
+            }
+            if (valid) *(uint4*)(out + 8 * g) = make_uint4(pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
+        }
+        if (p.stat_part) {
+            // column sums over the warp's 32 rows, of the values as stored: every exchange halves the columns a lane is left with
+            float s1[NC], s2[NC];
+#pragma unroll
+            for (int j = 0; j < NC / 2; ++j) {
+                const float a = valid ? __uint_as_float(pk[j] << 16) : 0.f, b = valid ? __uint_as_float(pk[j] & 0xffff0000u) : 0.f;
+                s1[2 * j] = a; s2[2 * j] = a * a; s1[2 * j + 1] = b; s2[2 * j + 1] = b * b;
+            }
+            int col = 0;
+#pragma unroll
+            for (int st = 0; st < 5; ++st) {
+                const int d = 16 >> st, left = NC >> (st + 1);           // columns left after this step (0: one column, plain sum)
+                if (left >= 1) {
+                    const bool up = (lane & d) != 0;
+#pragma unroll
+                    for (int j = 0; j < left; ++j) {
+                        const float a1 = up ? s1[j] : s1[left + j], a2 = up ? s2[j] : s2[left + j];
+                        const float b1 = __shfl_xor_sync(0xffffffffu, a1, d), b2 = __shfl_xor_sync(0xffffffffu, a2, d);
+                        s1[j] = (up ? s1[left + j] : s1[j]) + b1; s2[j] = (up ? s2[left + j] : s2[j]) + b2;
+                    }
+                    if (up) col += left;
+                } else {
+                    s1[0] += __shfl_xor_sync(0xffffffffu, s1[0], d); s2[0] += __shfl_xor_sync(0xffffffffu, s2[0], d);
+                }
+            }
+            const size_t rec = (size_t)(cls * tiles_m + tmi) * 4 + q;
+            float* const dst = p.stat_part + (rec * p.Cn + co0 + c0 + col) * 2;
+            constexpr int LEFT = NC > 32 ? NC / 32 : 1, DUP = NC < 32 ? 32 / NC : 1;        // columns per lane at the end / lanes that hold the same one
+            if (lane % DUP == 0) {
+#pragma unroll
+                for (int j = 0; j < LEFT; ++j) *(float2*)(dst + 2 * j) = make_float2(s1[j], s2[j]);
+            }
+        }
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (S > 1) cluster_sync_all(); else __syncthreads();       // no CTA leaves while another reads its partial tile
+    if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, 64); }
 }
 
 // ------------------------------------------------------------------------------------------ weight gradient
@@ -741,8 +966,9 @@ wg_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUten
         tc_fence_after();
         const int rb = rb0 + (row >> 6);
         const bool valid = ok && rb < p.row_blocks;
-        // partial[z][row-block][64][c_out]
-        float* out = p.partial + (((size_t)blockIdx.z * p.row_blocks + rb) * 64 + (row & 63)) * p.Co + co0;
+        // partial[z][c_out][row-block][64]: the lanes of a warp write 128 consecutive bytes per column
+        const size_t R = (size_t)p.row_blocks * 64;
+        float* out = p.partial + ((size_t)blockIdx.z * p.Co + co0) * R + rb * 64 + (row & 63);
 #pragma unroll 1
         for (int c = 0; c < N_TILE; c += 32) {
             uint32_t v[32];
@@ -752,9 +978,8 @@ wg_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUten
                 for (int j = 0; j < 32; ++j) v[j] = 0u;
             }
             if (!valid) continue;
-            uint4* o4 = (uint4*)(out + c);
 #pragma unroll
-            for (int g = 0; g < 8; ++g) o4[g] = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+            for (int j = 0; j < 32; ++j) out[(c + j) * R] = __uint_as_float(v[j]);
         }
     }
     tc_fence_before();
@@ -774,7 +999,7 @@ struct Wg2Params {
     int W, Ht, Nt, tiles_h, tiles_n;          // contraction step = W x Ht x Nt = 128 pixels
     int ptiles, ptiles_per_split, n_base;
     int kchunks, row_blocks, Co;
-    float* partial;                           // [splits][row_blocks * 64][Co]
+    float* partial;                           // [splits][Co][row_blocks * 64]
     int* err;
 };
 template <int N_TILE, int NX, int XSUB_KB, int STAGES>
@@ -890,7 +1115,8 @@ wg2_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUte
             const int sx = rb / 3, dhi = rb % 3;
             const int dwi = NX == 3 ? sx : dw_fixed, chunk = NX == 3 ? 0 : chunk0 + sx;
             const int grb = (dhi * 3 + dwi) * p.kchunks + chunk;     // row block of the whole matrix: (tap, chunk)
-            float* out = p.partial + (((size_t)blockIdx.z * p.row_blocks + grb) * 64 + (row & 63)) * p.Co + co0;
+            const size_t R = (size_t)p.row_blocks * 64;
+            float* out = p.partial + ((size_t)blockIdx.z * p.Co + co0) * R + grb * 64 + (row & 63);
 #pragma unroll 1
             for (int c = 0; c < N_TILE; c += 32) {
                 uint32_t v[32];
@@ -900,9 +1126,8 @@ wg2_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUte
                     for (int j = 0; j < 32; ++j) v[j] = 0u;
                 }
                 if (!valid) continue;
-                uint4* o4 = (uint4*)(out + c);
 #pragma unroll
-                for (int gq = 0; gq < 8; ++gq) o4[gq] = make_uint4(v[4 * gq], v[4 * gq + 1], v[4 * gq + 2], v[4 * gq + 3]);
+                for (int j = 0; j < 32; ++j) out[(c + j) * R] = __uint_as_float(v[j]);
             }
         }
     }
@@ -1235,7 +1460,7 @@ stem_fw_kernel(const __grid_constant__ CUtensorMap tmRaw, const __grid_constant_
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tmem_empty[buf]);
-            epi_slice(v, p.bias ? p.bias + co0 : nullptr, p.epi, 0ull, 0xffffffffu, ok, true, &tmO, co0, bw0, th * p.Ht + bh0, n,
+            epi_slice(v, p.bias ? p.bias + co0 : nullptr, p.epi, 0ull, 0ull, 0xffffffffu, ok, true, &tmO, co0, bw0, th * p.Ht + bh0, n,
                       stg0 + sbuf * EPI_BUF_BYTES, lane, p.stat_part ? p.stat_part + (((size_t)tile * 4 + q) * p.Co + co0) * 2 : nullptr);
             sbuf ^= 1u;
         }
@@ -1247,33 +1472,35 @@ stem_fw_kernel(const __grid_constant__ CUtensorMap tmRaw, const __grid_constant_
     if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, 128); }
 }
 
-// dW[co][tap][ci] = sum_z partial[z][(tap, cc)][ci % 64][co], z ascending.  A CTA of 256 threads (it fits beside a
-// resident tensor-core CTA of another stream) transposes a tile of 8 rows x 32 columns: many small CTAs, because a layer
-// has few output elements (36 864 for 64 -> 64) and many partial matrices (up to 147), so the kernel lives on the number of
-// loads in flight; a thread owns one element and keeps 16 independent loads in flight along z.
-__global__ void __launch_bounds__(256) wg_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, int splits, int row_blocks, int Co,
-                                                        bool accum) {
-    __shared__ float t[8][33];
-    const int R = row_blocks * 64;                       // = taps * Cin
-    const int r0 = blockIdx.x * 8, c0 = blockIdx.y * 32;
-    const int tx = threadIdx.x, ty = threadIdx.y;        // 32 x 8
-    const unsigned zs = (unsigned)R * Co;                // one partial matrix (< 2^32 elements)
-    const float* p = partial + (size_t)(r0 + ty) * Co + c0 + tx;
-    float s = 0.f;
-    int z = 0;
-    for (; z + 16 <= splits; z += 16, p += (size_t)16 * zs) {
-        float v[16];
+// dW = sum over z of the partial matrices, n4 float4 each: 32 float4 per CTA, eight threads of different z per float4, four loads in
+// flight each, then their sums in order (a layer has few output elements, 36 864 for 64 -> 64, and many partial matrices, up to 147, so
+// the kernel lives on the number of loads in flight).  256 threads: it fits beside a resident tensor-core CTA of another stream.
+__global__ void __launch_bounds__(256) wg_reduce_kernel(const float4* __restrict__ partial, float4* __restrict__ dw, int splits, int n4, bool accum) {
+    __shared__ float4 t[8][32];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, e = blockIdx.x * 32 + tx;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (e < n4) {
+        const float4* p = partial + e;
+        int z = ty;
+        for (; z + 24 < splits; z += 32) {
+            float4 v[4];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = __ldg(p + j * zs);
+            for (int j = 0; j < 4; ++j) v[j] = __ldg(p + (size_t)(z + 8 * j) * n4);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) s += v[j];
+            for (int j = 0; j < 4; ++j) { s.x += v[j].x; s.y += v[j].y; s.z += v[j].z; s.w += v[j].w; }
+        }
+        for (; z < splits; z += 8) { const float4 v = __ldg(p + (size_t)z * n4); s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }
     }
-    for (; z < splits; ++z, p += zs) s += __ldg(p);
     t[ty][tx] = s;
     __syncthreads();
-    const int tid = ty * 32 + tx, c = tid >> 3, r = tid & 7;      // 8 consecutive threads write 8 consecutive elements of a row of dW
-    float* d = dw + (size_t)(c0 + c) * R + r0 + r;
-    *d = accum ? *d + t[r][c] : t[r][c];
+    if (ty != 0 || e >= n4) return;
+#pragma unroll
+    for (int j = 1; j < 8; ++j) { const float4 v = t[j][tx]; s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }
+    if (accum) { const float4 v = dw[e]; s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }
+    dw[e] = s;
+}
+static cudaError_t reduce_partials(const float* partial, float* dw, int splits, size_t n, bool accum, cudaStream_t s) {
+    return klaunch(wg_reduce_kernel, (unsigned)((n / 4 + 31) / 32), 256, 0, s, (const float4*)partial, (float4*)dw, splits, (int)(n / 4), accum);
 }
 
 // One launch per module and step: the update of Eq. dl_update for ALL of the module's parameters.
@@ -1509,6 +1736,34 @@ cudaError_t run_km(const KmMaps& m, const KmParams& p_in, int n_tile, cudaStream
     return cudaErrorInvalidValue;
 }
 
+// One CTA per tile fills the device once or twice (two fit on an SM); beyond that the wider tiles of km_kernel read their operands less often.
+bool small_problem(long tiles) { return tiles <= 2 * 148; }
+template <int S>
+static cudaError_t launch_ks(const TensorMap& a, const TensorMap& b, const KmParams& p, int tiles, cudaStream_t s) {
+    constexpr int smem = KS_STAGES * KS_STAGE_BYTES + 1024 + 256;
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(ks_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        attr = true;
+    }
+    return klaunch_cluster(ks_kernel<S>, dim3(tiles * S), dim3(NUM_THREADS), smem, s, S > 1 ? S : 0, *(const CUtensorMap*)&a, *(const CUtensorMap*)&b, p);
+}
+cudaError_t run_small(const TensorMap& a, const TensorMap& b, const KmParams& p, cudaStream_t s) {
+    const int tiles = p.tiles_w * p.tiles_h * p.tiles_n * (p.Cn / 64) * p.ncls;
+    int kb = 1 << 30;                                    // the shortest contraction of a class, in steps of 64
+    for (int c = 0; c < p.ncls; ++c) { const int n = (p.cls_tap0[c + 1] - p.cls_tap0[c]) * p.kchunks; if (n < kb) kb = n; }
+    // as many CTAs per tile as fill the device once, with at least two steps each
+    int split = 1;
+    while (split < 8 && tiles * split * 2 <= 148 && kb >= split * 2 * 2) split *= 2;
+    switch (split) {
+        case 1: return launch_ks<1>(a, b, p, tiles, s);
+        case 2: return launch_ks<2>(a, b, p, tiles, s);
+        case 4: return launch_ks<4>(a, b, p, tiles, s);
+        default: return launch_ks<8>(a, b, p, tiles, s);
+    }
+}
+
 template <int N_TILE, int STAGES>
 static cudaError_t launch_wg(const TensorMap& x, const TensorMap& dy, const WgParams& p, dim3 grid, cudaStream_t s) {
     constexpr int smem = STAGES * (2 + N_TILE / 64) * 8192 + 1024 + 256;
@@ -1522,17 +1777,17 @@ static cudaError_t launch_wg(const TensorMap& x, const TensorMap& dy, const WgPa
     return cudaGetLastError();
 }
 
-cudaError_t run_wg(const TensorMap& x, const TensorMap& dy, const WgParams& p, int n_tile, int splits, float* dw, bool accum, cudaStream_t s) {
+cudaError_t run_wg(const TensorMap& x, const TensorMap& dy, const WgParams& p_in, int n_tile, int splits, float* dw, bool accum, cudaStream_t s) {
+    WgParams p = p_in;
+    if (splits == 1 && !accum) p.partial = dw;             // the one partial matrix is the gradient (same layout)
     dim3 grid((p.row_blocks + 1) / 2, p.Co / n_tile, splits);
     cudaError_t e;
     if (n_tile == 64) e = launch_wg<64, 4>(x, dy, p, grid, s);      // 96 KB of stages: two CTAs per SM
     else if (n_tile == 128) e = launch_wg<128, 5>(x, dy, p, grid, s);
     else if (n_tile == 256) e = launch_wg<256, 4>(x, dy, p, grid, s);
     else return cudaErrorInvalidValue;
-    if (e != cudaSuccess) return e;
-    dim3 rgrid(p.row_blocks * 8, p.Co / 32), rblk(32, 8);
-    klaunch(wg_reduce_kernel, rgrid, rblk, 0, s, p.partial, dw, splits, p.row_blocks, p.Co, accum);
-    return cudaGetLastError();
+    if (e != cudaSuccess || p.partial == dw) return e;
+    return reduce_partials(p.partial, dw, splits, (size_t)p.row_blocks * 64 * p.Co, accum, s);
 }
 
 template <int N_TILE, int NX, int XSUB_KB, int STAGES>
@@ -1571,14 +1826,14 @@ cudaError_t run_wg_rows(const TensorMap& x_rows, const TensorMap& dy128, const W
     p.ptiles = q.tiles_h * q.tiles_n; p.ptiles_per_split = (p.ptiles + splits - 1) / splits;
     p.kchunks = q.C / 64; p.row_blocks = 9 * p.kchunks; p.Co = q.Co; p.partial = q.partial; p.err = q.err;
     const int z = (p.ptiles + p.ptiles_per_split - 1) / p.ptiles_per_split;
+    if (z == 1 && !accum) p.partial = dw;
     cudaError_t e;
     if (variant == 1) e = launch_wg2<64, 3, 24, 2>(x_rows, dy128, p, dim3(1, q.Co / 64, z), s);
     else if (variant == 2) e = launch_wg2<128, 2, 20, 3>(x_rows, dy128, p, dim3(3 * (q.C / 128), q.Co / 128, z), s);
     else return cudaErrorInvalidValue;
     if (e != cudaSuccess) return e;
-    dim3 rgrid(p.row_blocks * 8, p.Co / 32), rblk(32, 8);
-    klaunch(wg_reduce_kernel, rgrid, rblk, 0, s, p.partial, dw, z, p.row_blocks, p.Co, accum);
-    return cudaGetLastError();
+    if (p.partial == dw) return cudaSuccess;
+    return reduce_partials(p.partial, dw, z, (size_t)p.row_blocks * 64 * p.Co, accum, s);
 }
 
 bool make_map_raw_rows(TensorMap* out, const void* base, int C, int W, int H, int N, int box_rows) {

@@ -31,7 +31,9 @@ struct KmParams {
     int sms;                                     // SMs the grid is sized for (0: all)
     const float* bias;                           // or nullptr
     void* out;
-    float* stat_part;                            // or nullptr: [tile_m * 4 + warp][Cn][2] = (sum, sum of squares) over the
+    const void* mask;                            // or nullptr: bf16 tensor of the output's shape; outputs whose mask value is not > 0 become 0
+                                                 // (the ReLU of the layer below, applied to its error gradient while that is produced)
+    float* stat_part;                            // or nullptr: [(class * tiles + tile_m) * 4 + warp][Cn][2] = (sum, sum of squares) over the
                                                  // warp's 32 output rows, of the values as stored (rounded to bf16)
     int* err;                                    // device word, set non-zero if a bounded wait gave up
 };
@@ -43,7 +45,7 @@ struct WgParams {
     int kchunks, row_blocks, xs;                 // 64-channel chunks of c_in; row blocks = taps * kchunks
     int dh[9], dw[9];
     int Co;
-    float* partial;                              // [splits][row_blocks * 64][Co]
+    float* partial;                              // [splits][Co][row_blocks * 64]
     int* err;
 };
 
@@ -71,6 +73,10 @@ bool make_map_out(TensorMap* out, const void* base, int C, int W, int H, int N, 
 //   out    : nullptr, or the output tensor's map from make_map_out: dense outputs are then written by TMA stores
 struct KmMaps { const TensorMap* a; const TensorMap* a_rows; const TensorMap* b; const TensorMap* b_half; const TensorMap* out; };
 cudaError_t run_km(const KmMaps& m, const KmParams& p, int n_tile, cudaStream_t s);
+// The same computation for problems of few tiles: 64-column tiles, each split over the contraction among the CTAs of a cluster.  b: box of 64 rows.
+// small_problem: whether run_small is the kernel for `tiles` = pixel tiles x 64-column tiles x classes (decided when the maps are made).
+bool small_problem(long tiles);
+cudaError_t run_small(const TensorMap& a, const TensorMap& b, const KmParams& p, cudaStream_t s);
 // accum: dw += the result (second and later groups of workers)
 cudaError_t run_wg(const TensorMap& x, const TensorMap& dy, const WgParams& p, int n_tile, int splits, float* dw, bool accum, cudaStream_t s);
 // Weight gradient of a 3x3, stride-1, pad-1 layer in rows mode (x is fetched once per horizontal shift and 64-channel
@@ -82,7 +88,7 @@ cudaError_t run_wg(const TensorMap& x, const TensorMap& dy, const WgParams& p, i
 struct WgRowsParams {
     int W, Ht, Nt, tiles_h, tiles_n, n_base;
     int C, Co;
-    float* partial;                              // [splits][9 * C][Co]
+    float* partial;                              // [splits][Co][9 * C]
     int* err;
 };
 int wg_rows_variant(int H, int W, int C, int Co);
