@@ -67,6 +67,10 @@ struct Op {
     bool head;                                               // the network's last linear layer: fused with the loss (head_* kernels)
     char shape[40];                                          // "HxW Cin->Cout kR sS", the profiler's detail tag
     int n_tile_f, n_tile_d, n_tile_w, wg_splits;
+    int masked_by;                                           // > 0: op masked_by - 1, the only consumer of this layer's (ReLU) output, applies the mask to the error
+                                                             // gradient it produces and leaves the bias gradient's records
+    int masks;                                               // > 0: the reverse: this op does that for op masks - 1
+    size_t col_off; int col_recs;                            // of the masked layer: its records in the module's bstat
     bool small_f, small_d;                                   // few tiles: forward / input gradient by tc::run_small (n_tile_f / n_tile_d = 64)
     tc::KmParams kf;
     tc::KmParams kd;                                         // all output-parity classes of the input gradient in one launch
@@ -103,7 +107,7 @@ struct Module {
     size_t stash_slot_bytes, wslot_bytes, grad_pool_bytes, in_slot_bytes;
     size_t ws_elems, scratch_elems, red_elems;
     char *in_ring, *stash, *gradpool, *d2, *wring, *wtring;
-    float *master, *grad, *ws, *scratch, *red, *cstat[2];
+    float *master, *grad, *ws, *scratch, *red, *cstat[2], *bstat;
     bool fused_update;             // one kernel per step updates all parameters and emits the next weight version (both layouts)
     tc::UpdTable upd;
     size_t cstat_elems[2];
@@ -530,7 +534,7 @@ bool tc_forward(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* y_base, 
     if (ok && o.stat_chunks) { m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.stat_chunks; }
     return ok;
 }
-bool tc_dgrad(fdg_ctx* c, Module& m, const Op& o, char* dy_base, char* dx_base, int64_t version, bool accum, const Win& wn, cudaStream_t s) {
+bool tc_dgrad(fdg_ctx* c, Module& m, const Op& o, char* dy_base, char* dx_base, int64_t version, bool accum, const char* mask, float* col, const Win& wn, cudaStream_t s) {
     int ia = find_buf(o.dy_ptrs, dy_base);
     if (ia < 0) return false;
     const ConvGeom& g = o.g;
@@ -540,7 +544,7 @@ bool tc_dgrad(fdg_ctx* c, Module& m, const Op& o, char* dy_base, char* dx_base, 
         zero_fill(dx_base + (size_t)wn.n0 * g.H * g.W * g.C * 2, (size_t)rows * g.C * 2, s);
     }
     tc::KmParams p = o.kd;
-    p.bias = nullptr; p.out = dx_base; p.epi = accum ? EPI_ACCUM : 0; p.err = c->tc_err; p.stat_part = nullptr; p.sms = c->grid_sms;
+    p.bias = nullptr; p.out = dx_base; p.epi = accum ? EPI_ACCUM : 0; p.err = c->tc_err; p.mask = mask; p.stat_part = col; p.sms = c->grid_sms;
     p.n_base = wn.n0; p.N = wn.n0 + wn.n; p.tiles_n = (wn.n + p.Nt - 1) / p.Nt;
     const double crows = (double)wn.n * p.Hd * p.Wd;         // pixels of one class; every tap belongs to exactly one class
     Scope sc(KC_TC_DGRAD, 2.0 * crows * g.C * p.ntaps * g.Co,
@@ -775,13 +779,18 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
         size_t n_out = to.elems() * wn.n, n_in = ti.elems() * wn.n;
         char* gout = G(o.out);
         char* gin = G(o.in);
+        // the layer below ends in a ReLU whose mask this op applies
+        const Op* const below = o.masks > 0 ? &m.ops[o.masks - 1] : nullptr;
+        float* const col = below && below->bias ? m.bstat + below->col_off : nullptr;
         switch (o.type) {
             case OP_CONV: {
                 ConvGeom g = o.g; g.N = wn.n;
                 if (o.head && m.groups == 1) {
                     profile_detail(o.shape);
-                    head_backward(dt, T(o.in), wbig(c, m, version, o.w_off), gout, gin, o.acc_in, mgrad + o.w_off, o.bias ? mgrad + m.n_big + o.b_off : nullptr,
-                                  m.head_scratch, c->M, g.C, g.Co, s);
+                    head_backward(dt, T(o.in), wbig(c, m, version, o.w_off), gout, gin, o.acc_in, o.masks > 0, col, m.head_scratch, c->M, g.C, g.Co, s);
+                    cudaStream_t ws = m.wstream;                     // the sum of the partials is needed by the update only
+                    if (ws != s) { step_record(m.wev, s); step_wait(ws, m.wev); }
+                    head_reduce(mgrad + o.w_off, o.bias ? mgrad + m.n_big + o.b_off : nullptr, m.head_scratch, c->M, g.C, g.Co, ws);
                     profile_detail(nullptr);
                     break;
                 }
@@ -795,18 +804,21 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
                 // dZ = dA * (A > 0) in place and the bias gradient, in one pass over dA where the width allows
                 const long orows = (long)g.N * g.Ho * g.Wo;
                 const bool fused_rb = (o.relu || o.bias) && relu_bias_backward_supported(dt, g.Co);
-                if (fused_rb) relu_bias_backward(dt, o.relu ? T(o.out) : nullptr, gout, o.bias ? mgrad + m.n_big + o.b_off : nullptr, m.scratch, orows, g.Co, acc_p, s);
+                if (o.masked_by) {}                                  // done by the op above; the records are added below
+                else if (fused_rb) relu_bias_backward(dt, o.relu ? T(o.out) : nullptr, gout, o.bias ? mgrad + m.n_big + o.b_off : nullptr, m.scratch, orows, g.Co, acc_p, s);
                 else if (o.relu) relu_backward(dt, T(o.out), gout, gout, n_out, false, s);
                 profile_detail(o.shape);
                 // the weight gradient needs dy as it stands now and is needed only by the update: it goes to its own stream
                 cudaStream_t ws = m.wstream;
                 if (ws != s) { step_record(m.wev, s); step_wait(ws, m.wev); }
+                if (o.masked_by && o.bias) colsum_records(m.bstat + o.col_off, mgrad + m.n_big + o.b_off, o.col_recs, g.Co, false, ws);
                 if (o.stem && tc_stem_wgrad(c, m, o, P.tensor(o.in), grad_ptr(c, kk, o.out, t), mgrad + o.w_off, wn, ws)) {}
                 else if (o.stem) stem_wgrad(T(o.in), gout, mgrad + o.w_off, m.ws, g, acc_p, ws);
                 else if (!(o.tc && tc_wgrad(c, m, o, P.tensor(o.in), grad_ptr(c, kk, o.out, t), mgrad + o.w_off, wn, ws)))
                     fconv_wgrad(dt, T(o.in), gout, mgrad + o.w_off, m.ws, g, 1, 0, acc_p, ws);
-                if (o.bias && !fused_rb) bias_grad(dt, gout, mgrad + m.n_big + o.b_off, m.scratch, orows, g.Co, acc_p, s);
-                if (gin && !(o.tc && tc_dgrad(c, m, o, grad_ptr(c, kk, o.out, t), grad_ptr(c, kk, o.in, t), version, o.acc_in, wn, s)))
+                if (o.bias && !fused_rb && !o.masked_by) bias_grad(dt, gout, mgrad + m.n_big + o.b_off, m.scratch, orows, g.Co, acc_p, s);
+                if (gin && !(o.tc && tc_dgrad(c, m, o, grad_ptr(c, kk, o.out, t), grad_ptr(c, kk, o.in, t), version, o.acc_in,
+                                                     below ? P.tensor(o.in) : nullptr, col, wn, s)))
                     fconv_dgrad(dt, gout, wbig(c, m, version, o.w_off, rep), gin, g, o.acc_in ? EPI_ACCUM : 0, 1, 0, s);
                 profile_detail(nullptr);
                 break; }
@@ -829,8 +841,8 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
                 profile_detail(nullptr);
                 break; }
             case OP_RELU: if (gin) relu_backward(dt, T(o.out), gout, gin, n_out, o.acc_in, s); break;
-            case OP_POOL: if (gin) maxpool_backward(dt, T(o.in), gout, gin, wn.n, ti.h, ti.w, ti.c, o.acc_in, s); break;
-            case OP_GAP: if (gin) gap_backward(dt, gout, gin, wn.n, ti.h * ti.w, ti.c, o.acc_in, s); break;
+            case OP_POOL: if (gin) maxpool_backward(dt, T(o.in), gout, gin, wn.n, ti.h, ti.w, ti.c, o.acc_in, col, s); break;
+            case OP_GAP: if (gin) gap_backward(dt, gout, gin, wn.n, ti.h * ti.w, ti.c, o.acc_in, below ? T(o.in) : nullptr, col, s); break;
             case OP_ADD: {
                 if (gin) copy_or_accumulate(dt, gout, gin, n_in, o.acc_in, s);
                 char* g2 = G(o.in2);
@@ -878,8 +890,8 @@ bool backward_op_replicas(fdg_ctx* c, int kk, int64_t batch, int64_t version, in
                          o.relu && !o.has_res, false, s);
             return true;
         case OP_RELU: if (gin) relu_backward(dt, P.tensor(o.out), gout, gin, n_in, o.acc_in, s); return true;
-        case OP_POOL: if (gin) maxpool_backward(dt, P.tensor(o.in), gout, gin, c->M, ti.h, ti.w, ti.c, o.acc_in, s); return true;
-        case OP_GAP: if (gin) gap_backward(dt, gout, gin, c->M, ti.h * ti.w, ti.c, o.acc_in, s); return true;
+        case OP_POOL: if (gin) maxpool_backward(dt, P.tensor(o.in), gout, gin, c->M, ti.h, ti.w, ti.c, o.acc_in, nullptr, s); return true;
+        case OP_GAP: if (gin) gap_backward(dt, gout, gin, c->M, ti.h * ti.w, ti.c, o.acc_in, nullptr, nullptr, s); return true;
         case OP_ADD: {
             if (gin) copy_or_accumulate(dt, gout, gin, n_in, o.acc_in, s);
             if (char* g2 = grad_ptr(c, kk, o.in2, t)) copy_or_accumulate(dt, gout, g2, n_in, o.acc_in2, s);
@@ -1482,6 +1494,33 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
         const int n = ctx->M / m.groups;
         for (const Op& o : m.ops)
             if (o.tc && (n % o.kf.Nt || (o.kd.Nt && n % o.kd.Nt) || n % o.kw.Nt)) m.groups = 1;
+    }
+    // ReLU masks and bias gradients that the layer above a conv / linear layer can take along while it produces the error gradient: one pass over
+    // it less (read, masked, written again) and one or two launches less in the module's chain.  bf16, all workers at once, the layer's output
+    // has one consumer in the module, which writes (does not add to) its gradient.
+    for (Module& m : ctx->mod) {
+        m.bstat = nullptr;
+        if (ctx->dt != 1 || ctx->R != 1 || m.groups != 1) continue;
+        size_t elems = 0;
+        for (size_t i = 0; i < m.ops.size(); ++i) {
+            Op& o = m.ops[i];
+            const TensorDesc& to = m.t[o.out];
+            if (o.type != OP_CONV || !(o.tc || o.stem) || !o.relu || to.loc != LOC_STASH || !relu_bias_backward_supported(ctx->dt, o.g.Co)) continue;
+            int users = 0; size_t j = 0;
+            for (size_t k = i + 1; k < m.ops.size(); ++k) if (m.ops[k].in == o.out || m.ops[k].in2 == o.out) { ++users; j = k; }
+            if (users != 1 || m.ops[j].in != o.out || m.ops[j].acc_in) continue;
+            Op& u = m.ops[j];
+            int recs = 0;
+            if (u.type == OP_CONV && u.head) recs = head_col_records(ctx->M);
+            else if (u.type == OP_CONV && u.tc && !u.dgrad_needs_zero) recs = u.kd.tiles_w * u.kd.tiles_h * u.kd.tiles_n * u.kd.ncls * 4;
+            else if (u.type == OP_POOL && o.bias) recs = pool_col_records(ctx->dt, ctx->M, to.h, to.w, to.c);
+            else if (u.type == OP_GAP) recs = gap_col_records(ctx->dt, ctx->M, to.h * to.w, to.c);
+            if (!recs) continue;
+            o.masked_by = (int)j + 1; u.masks = (int)i + 1;
+            o.col_off = elems; o.col_recs = recs;
+            if (o.bias) elems += align_up((size_t)recs * o.g.Co * 2, 64);
+        }
+        if (elems && !(m.bstat = (float*)get(elems * sizeof(float)))) return bail(FDG_ERR_OOM, "the allocator returned NULL");
     }
     // modules whose update runs as one kernel (instead of two update launches and one transposing launch per tensor-core
     // layer): bf16, one weight copy, all workers at once, at least one tensor-core layer

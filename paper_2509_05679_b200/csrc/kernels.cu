@@ -103,6 +103,10 @@ __device__ __forceinline__ float ld(const bf16* p) { return __bfloat162float(*p)
 __device__ __forceinline__ void st(float* p, float v) { *p = v; }
 __device__ __forceinline__ void st(bf16* p, float v) { *p = __float2bfloat16_rn(v); }
 
+template <typename T> __device__ __forceinline__ float rounded(float v);        // v as T stores it
+template <> __device__ __forceinline__ float rounded<float>(float v) { return v; }
+template <> __device__ __forceinline__ float rounded<bf16>(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
+
 static inline unsigned cdiv(size_t a, size_t b) { return (unsigned)((a + b - 1) / b); }
 
 // Convolutions and linear layers on the CUDA cores: fconv.cu and linear.cu.
@@ -286,6 +290,44 @@ __global__ void colsum_final_warp(const float* __restrict__ part, float* __restr
     for (int d = 16; d > 0; d >>= 1) a += __shfl_xor_sync(0xffffffffu, a, d);
     if (lane == 0) out[c] = accum ? out[c] + a : a;
 }
+// out[c] = sum over the records of part[rec][c][0] (records that a kernel's epilogue left, see KmParams::stat_part): one block per 4
+// channels, a thread owns one channel and every 64th record, eight loads in flight, then a fixed tree.
+__global__ void __launch_bounds__(256) colsum_records_k(const float* __restrict__ part, float* __restrict__ out, int recs, int C, bool accum) {
+    __shared__ float sh[64][5];
+    const int cl = threadIdx.x & 3, kl = threadIdx.x >> 2, c = blockIdx.x * 4 + cl;
+    const float* p = part + (size_t)c * 2;
+    float a = 0.f;
+    int k = kl;
+    for (; k + 448 < recs; k += 512) {
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = p[(size_t)(k + 64 * j) * C * 2];
+        a += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+    }
+    for (; k < recs; k += 64) a += p[(size_t)k * C * 2];
+    sh[kl][cl] = a;
+    __syncthreads();
+    for (int d = 32; d > 0; d >>= 1) { if (kl < d) sh[kl][cl] += sh[kl + d][cl]; __syncthreads(); }
+    if (kl == 0) out[c] = accum ? out[c] + sh[0][cl] : sh[0][cl];
+}
+void colsum_records(const float* part, float* out, int recs, int C, bool accum, cudaStream_t s) {
+    Scope sc(KC_BIAS_GRAD, 0.0, 8.0 * recs * C, s);
+    klaunch(colsum_records_k, C / 4, 256, 0, s, part, out, recs, C, accum);
+}
+// The sums a block's threads hold for their channel group (thread t: group t % cgs, V values) -> rec[c][0], in a fixed order.
+template <int V>
+__device__ __forceinline__ void block_colsum(const float (&s)[8], float* rec, int cgs) {
+    __shared__ float sh[256][9];
+#pragma unroll
+    for (int j = 0; j < V; ++j) sh[threadIdx.x][j] = s[j];
+    __syncthreads();
+    for (int t = threadIdx.x; t < cgs * V; t += 256) {
+        const int q = t / V, k = t % V;
+        float a = 0.f;
+        for (int r = q; r < 256; r += cgs) a += sh[r][k];
+        rec[(size_t)t * 2] = a;
+    }
+}
 bool relu_bias_backward_supported(int dt, int C) {
     const int V = dt ? 8 : 4;
     if (C % V) return false;
@@ -356,10 +398,13 @@ __global__ void __launch_bounds__(256) maxpool_fwd_vk(const T* __restrict__ x, T
     }
 }
 template <typename T>
-__global__ void __launch_bounds__(256) maxpool_bwd_vk(const T* __restrict__ x, const T* __restrict__ dy, T* dx, int N, int H, int W, int C, bool accum) {
+__global__ void __launch_bounds__(256) maxpool_bwd_vk(const T* __restrict__ x, const T* __restrict__ dy, T* dx, int N, int H, int W, int C, bool accum, float* col) {
     constexpr int V = Vec<T>::V;
     const int Ho = H / 2, Wo = W / 2, cgs = C / V;
     const size_t total = (size_t)N * Ho * Wo * cgs;
+    float sum[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sum[j] = 0.f;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const int cg = (int)(i % cgs); size_t p = i / cgs; const int ox = (int)(p % Wo); p /= Wo; const int oy = (int)(p % Ho); const size_t n = p / Ho;
         const size_t base = ((n * H + 2 * oy) * W + 2 * ox) * C + (size_t)cg * V;
@@ -375,6 +420,7 @@ __global__ void __launch_bounds__(256) maxpool_bwd_vk(const T* __restrict__ x, c
 #pragma unroll
             for (int q = 1; q < 4; ++q) if (a[q][j] > m) { m = a[q][j]; b = q; }            // first maximum wins
             best[j] = b;
+            if (col) { if (!(m > 0.f)) g[j] = 0.f; sum[j] += g[j]; }        // x is a ReLU's output: its gradient, masked, and that layer's bias gradient
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -385,6 +431,7 @@ __global__ void __launch_bounds__(256) maxpool_bwd_vk(const T* __restrict__ x, c
             Vec<T>::store(dx + o[q], v);
         }
     }
+    if (col) block_colsum<V>(sum, col + (size_t)blockIdx.x * C * 2, cgs);
 }
 void maxpool_forward(int dt, const void* x, void* y, int N, int H, int W, int C, cudaStream_t s) {
     const double esz_ = dt ? 2.0 : 4.0;
@@ -398,13 +445,14 @@ void maxpool_forward(int dt, const void* x, void* y, int N, int H, int W, int C,
     if (dt) klaunch(maxpool_fwd_k<bf16>, cdiv(n, 256), 256, 0, s, (const bf16*)x, (bf16*)y, N, H, W, C);
     else klaunch(maxpool_fwd_k<float>, cdiv(n, 256), 256, 0, s, (const float*)x, (float*)y, N, H, W, C);
 }
-void maxpool_backward(int dt, const void* x, const void* dy, void* dx, int N, int H, int W, int C, bool accum, cudaStream_t s) {
+int pool_col_records(int dt, int N, int H, int W, int C) { return (int)ew_grid((size_t)N * (H / 2) * (W / 2) * C / (dt ? 8 : 4)); }
+void maxpool_backward(int dt, const void* x, const void* dy, void* dx, int N, int H, int W, int C, bool accum, float* col_or_null, cudaStream_t s) {
     const double esz_ = dt ? 2.0 : 4.0;
     Scope sc(KC_POOL_BWD, 0.0, 2.25 * esz_ * (double)N * H * W * C, s);
     size_t n = (size_t)N * (H / 2) * (W / 2) * C;
     if (C % (dt ? 8 : 4) == 0) {
-        if (dt) klaunch(maxpool_bwd_vk<bf16>, ew_grid(n / 8), 256, 0, s, (const bf16*)x, (const bf16*)dy, (bf16*)dx, N, H, W, C, accum);
-        else klaunch(maxpool_bwd_vk<float>, ew_grid(n / 4), 256, 0, s, (const float*)x, (const float*)dy, (float*)dx, N, H, W, C, accum);
+        if (dt) klaunch(maxpool_bwd_vk<bf16>, ew_grid(n / 8), 256, 0, s, (const bf16*)x, (const bf16*)dy, (bf16*)dx, N, H, W, C, accum, col_or_null);
+        else klaunch(maxpool_bwd_vk<float>, ew_grid(n / 4), 256, 0, s, (const float*)x, (const float*)dy, (float*)dx, N, H, W, C, accum, col_or_null);
         return;
     }
     if (dt) klaunch(maxpool_bwd_k<bf16>, cdiv(n, 256), 256, 0, s, (const bf16*)x, (const bf16*)dy, (bf16*)dx, N, H, W, C, accum);
@@ -431,8 +479,11 @@ __global__ void gap_bwd_k(const T* dy, T* dx, int N, int HW, int C, bool accum) 
 }
 // the same with one 16-byte vector (4 fp32 / 8 bf16 channels) per thread; C a multiple of the vector length
 template <typename T>
-__global__ void __launch_bounds__(256) gap_bwd_vk(const T* __restrict__ dy, T* __restrict__ dx, size_t nvec, int HW, int Cv, bool accum) {
+__global__ void __launch_bounds__(256) gap_bwd_vk(const T* __restrict__ dy, T* __restrict__ dx, size_t nvec, int HW, int Cv, bool accum, const T* __restrict__ x, float* col) {
     constexpr int V = Vec<T>::V;
+    float sum[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sum[j] = 0.f;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
         const int cv = (int)(i % Cv); const size_t n = i / ((size_t)HW * Cv);
         float g[8], o[8];
@@ -440,8 +491,15 @@ __global__ void __launch_bounds__(256) gap_bwd_vk(const T* __restrict__ dy, T* _
         if (accum) Vec<T>::load(dx + i * V, o);
 #pragma unroll
         for (int j = 0; j < V; ++j) g[j] = accum ? g[j] / (float)HW + o[j] : g[j] / (float)HW;
+        if (x) {                             // x is a ReLU's output: its gradient, masked, and (col) that layer's bias gradient
+            float xv[8];
+            Vec<T>::load(x + i * V, xv);
+#pragma unroll
+            for (int j = 0; j < V; ++j) { if (!(xv[j] > 0.f)) g[j] = 0.f; sum[j] += rounded<T>(g[j]); }
+        }
         Vec<T>::store(dx + i * V, g);
     }
+    if (col) block_colsum<V>(sum, col + (size_t)blockIdx.x * Cv * V * 2, Cv);
 }
 void gap_forward(int dt, const void* x, void* y, int N, int HW, int C, cudaStream_t s) {
     const double esz_ = dt ? 2.0 : 4.0; (void)esz_;
@@ -451,15 +509,16 @@ void gap_forward(int dt, const void* x, void* y, int N, int HW, int C, cudaStrea
     else klaunch(gap_fwd_k<float>, cdiv(n, 128), 128, 0, s, (const float*)x, (float*)y, N, HW, C);
     
 }
-void gap_backward(int dt, const void* dy, void* dx, int N, int HW, int C, bool accum, cudaStream_t s) {
+int gap_col_records(int dt, int N, int HW, int C) { return (int)ew_grid((size_t)N * HW * C / (dt ? 8 : 4)); }
+void gap_backward(int dt, const void* dy, void* dx, int N, int HW, int C, bool accum, const void* mask_x_or_null, float* col_or_null, cudaStream_t s) {
     const double esz_ = dt ? 2.0 : 4.0; (void)esz_;
     Scope sc(KC_GAP_BWD, 0.0, esz_ * (double)N * (HW + 1) * C, s);
     size_t n = (size_t)N * HW * C;
     const int V = dt ? 8 : 4;
     if (C % V == 0 && ((uintptr_t)dy | (uintptr_t)dx) % 16 == 0) {
         const size_t nvec = n / V;
-        if (dt) klaunch(gap_bwd_vk<bf16>, ew_grid(nvec), 256, 0, s, (const bf16*)dy, (bf16*)dx, nvec, HW, C / V, accum);
-        else klaunch(gap_bwd_vk<float>, ew_grid(nvec), 256, 0, s, (const float*)dy, (float*)dx, nvec, HW, C / V, accum);
+        if (dt) klaunch(gap_bwd_vk<bf16>, ew_grid(nvec), 256, 0, s, (const bf16*)dy, (bf16*)dx, nvec, HW, C / V, accum, (const bf16*)mask_x_or_null, col_or_null);
+        else klaunch(gap_bwd_vk<float>, ew_grid(nvec), 256, 0, s, (const float*)dy, (float*)dx, nvec, HW, C / V, accum, (const float*)mask_x_or_null, col_or_null);
         return;
     }
     if (dt) klaunch(gap_bwd_k<bf16>, cdiv(n, 256), 256, 0, s, (const bf16*)dy, (bf16*)dx, N, HW, C, accum);
@@ -1106,6 +1165,7 @@ __global__ void __launch_bounds__(256) head_fwd_loss_k(const T* __restrict__ x, 
         float z = 0.f;                       // lane c keeps logit c
 #pragma unroll
         for (int c = 0; c < HEAD_MAX_C; ++c) {
+            if (c >= C) break;
             float v = acc[c];
 #pragma unroll
             for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
@@ -1137,56 +1197,83 @@ __global__ void __launch_bounds__(256) head_fwd_loss_k(const T* __restrict__ x, 
         last = atomicAdd(counter, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (last && threadIdx.x == 0) {
+    if (last) {                              // the last CTA adds the partials: 256 lanes, then a fixed tree
         __threadfence();
+        __shared__ float ls[256];
         float s = 0.f;
-        for (unsigned i = 0; i < gridDim.x; ++i) s += ((volatile float*)loss_part)[i];
-        *counter = 0u;
-        publish_loss(rec, s / (float)M, err, seq);
+        for (unsigned i = threadIdx.x; i < gridDim.x; i += 256) s += __ldcg(loss_part + i);
+        ls[threadIdx.x] = s;
+        __syncthreads();
+        for (int d = 128; d > 0; d >>= 1) { if ((int)threadIdx.x < d) ls[threadIdx.x] += ls[threadIdx.x + d]; __syncthreads(); }
+        if (threadIdx.x == 0) { *counter = 0u; publish_loss(rec, ls[0] / (float)M, err, seq); }
     }
 }
-// grid = ceil(M / HEAD_ROWS_PER_CTA).  part: [CTA][C][K + 1]
+// grid = (ceil(M / HEAD_ROWS_PER_CTA), slices of `kvs` vectors of the K columns): the sums over a CTA's 32 samples are serial chains, so the
+// columns are what is spread over the device.  part: [CTA row][C][K + 1].
+// mask: the head's input is the output of a ReLU layer: dx *= (x > 0), and col receives the column sums of the masked dx (that layer's bias
+// gradient), [CTA row][K][2].
 template <typename T>
 __global__ void __launch_bounds__(256) head_bwd_k(const T* __restrict__ x, const T* __restrict__ W, const T* __restrict__ dz, T* dx, float* __restrict__ part,
-                                                  int M, int K, int C, bool accum_dx) {
+                                                  float* __restrict__ col, int M, int K, int C, int kvs, bool accum_dx, bool mask) {
     constexpr int V = Vec<T>::V;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r0 = blockIdx.x * HEAD_ROWS_PER_CTA, r1 = min(M, r0 + HEAD_ROWS_PER_CTA);
+    const int nkv = K / V, kv0 = blockIdx.y * kvs, nk = min(nkv - kv0, kvs);
     __shared__ float dzs[HEAD_ROWS_PER_CTA][HEAD_MAX_C];
+    __shared__ float cs[256][V + 1];
     for (int i = threadIdx.x; i < (r1 - r0) * C; i += 256) dzs[i / C][i % C] = ld(dz + (size_t)r0 * C + i);
     __syncthreads();
     if (dx) {
-        for (int r = r0 + warp; r < r1; r += 8) {
-            for (int kv = lane; kv < K / V; kv += 32) {
+        // thread = one vector of columns for every (256 / kvs)-th sample
+        const int kv = threadIdx.x % kvs, rl = threadIdx.x / kvs, rstep = 256 / kvs;
+        float sum[8];
+#pragma unroll
+        for (int j = 0; j < V; ++j) sum[j] = 0.f;
+        if (kv < nk && rl < rstep)
+            for (int r = r0 + rl; r < r1; r += rstep) {
                 float a[8];
 #pragma unroll
                 for (int j = 0; j < V; ++j) a[j] = 0.f;
                 for (int c = 0; c < C; ++c) {
                     float wv[8];
-                    Vec<T>::load(W + (size_t)c * K + (size_t)kv * V, wv);
+                    Vec<T>::load(W + (size_t)c * K + (size_t)(kv0 + kv) * V, wv);
                     const float g = dzs[r - r0][c];
 #pragma unroll
                     for (int j = 0; j < V; ++j) a[j] = fmaf(g, wv[j], a[j]);
                 }
-                T* d = dx + (size_t)r * K + (size_t)kv * V;
+                T* d = dx + (size_t)r * K + (size_t)(kv0 + kv) * V;
                 if (accum_dx) {
                     float old[8];
                     Vec<T>::load(d, old);
 #pragma unroll
                     for (int j = 0; j < V; ++j) a[j] += old[j];
                 }
+                if (mask) {
+                    float xv[8];
+                    Vec<T>::load(x + (size_t)r * K + (size_t)(kv0 + kv) * V, xv);
+#pragma unroll
+                    for (int j = 0; j < V; ++j) { if (!(xv[j] > 0.f)) a[j] = 0.f; sum[j] += rounded<T>(a[j]); }
+                }
                 Vec<T>::store(d, a);
+            }
+        if (mask && col) {
+#pragma unroll
+            for (int j = 0; j < V; ++j) cs[threadIdx.x][j] = sum[j];
+            __syncthreads();
+            for (int t = threadIdx.x; t < nk * V; t += 256) {
+                float a = 0.f;
+                for (int q = 0; q < rstep; ++q) a += cs[q * kvs + t / V][t % V];
+                col[((size_t)blockIdx.x * K + kv0 * V + t) * 2] = a;
             }
         }
     }
     // partial sums: (class, vector of V columns) pairs round-robin over the threads, rows in ascending order
     float* out = part + (size_t)blockIdx.x * C * (K + 1);
-    const int nkv = K / V;
-    for (int p = threadIdx.x; p < C * nkv; p += 256) {
-        const int c = p / nkv, kv = p - c * nkv;
+    for (int p = threadIdx.x; p < C * nk; p += 256) {
+        const int c = p / nk, kv = kv0 + p - c * nk;
         float a[8];
 #pragma unroll
         for (int j = 0; j < V; ++j) a[j] = 0.f;
+#pragma unroll 8
         for (int r = r0; r < r1; ++r) {
             float xv[8];
             Vec<T>::load(x + (size_t)r * K + (size_t)kv * V, xv);
@@ -1197,7 +1284,7 @@ __global__ void __launch_bounds__(256) head_bwd_k(const T* __restrict__ x, const
 #pragma unroll
         for (int j = 0; j < V; ++j) out[(size_t)c * (K + 1) + kv * V + j] = a[j];
     }
-    if (threadIdx.x < C) {
+    if (blockIdx.y == 0 && threadIdx.x < C) {
         float a = 0.f;
         for (int r = r0; r < r1; ++r) a += dzs[r - r0][threadIdx.x];
         out[(size_t)threadIdx.x * (K + 1) + K] = a;
@@ -1207,6 +1294,7 @@ __global__ void head_reduce_k(const float* __restrict__ part, float* __restrict_
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= C * (K + 1)) return;
     float s = 0.f;
+#pragma unroll 8
     for (int b = 0; b < ctas; ++b) s += part[(size_t)b * C * (K + 1) + i];
     const int c = i / (K + 1), k = i - c * (K + 1);
     if (k < K) dW[(size_t)c * K + k] = s;
@@ -1224,14 +1312,23 @@ void head_forward_loss(int dt, const void* x, const void* W, const float* bias, 
     if (dt) klaunch(head_fwd_loss_k<bf16>, grid, 256, 0, s, (const bf16*)x, (const bf16*)W, bias, labels, logits, (bf16*)dlogits, scratch, counter, rec, err, seq, M, K, C, scale);
     else klaunch(head_fwd_loss_k<float>, grid, 256, 0, s, (const float*)x, (const float*)W, bias, labels, logits, (float*)dlogits, scratch, counter, rec, err, seq, M, K, C, scale);
 }
-void head_backward(int dt, const void* x, const void* W, const void* dlogits, void* dx_or_null, bool accum_dx, float* dW, float* db_or_null, float* scratch,
-                   int M, int K, int C, cudaStream_t s) {
+int head_col_records(int M) { return (M + HEAD_ROWS_PER_CTA - 1) / HEAD_ROWS_PER_CTA; }
+void head_backward(int dt, const void* x, const void* W, const void* dlogits, void* dx_or_null, bool accum_dx, bool mask_dx, float* col_or_null, float* scratch, int M,
+                   int K, int C, cudaStream_t s) {
     const unsigned ctas = (M + HEAD_ROWS_PER_CTA - 1) / HEAD_ROWS_PER_CTA;
-    { Scope sc(KC_FMA_WGRAD, (dx_or_null ? 4.0 : 2.0) * M * K * C, (dt ? 2.0 : 4.0) * ((double)M * K * (dx_or_null ? 2 : 1) + (double)C * K + (double)M * C), s);
-      if (dt) klaunch(head_bwd_k<bf16>, ctas, 256, 0, s, (const bf16*)x, (const bf16*)W, (const bf16*)dlogits, (bf16*)dx_or_null, scratch, M, K, C, accum_dx);
-      else klaunch(head_bwd_k<float>, ctas, 256, 0, s, (const float*)x, (const float*)W, (const float*)dlogits, (float*)dx_or_null, scratch, M, K, C, accum_dx); }
+    const int nkv = K / (dt ? 8 : 4);
+    // vectors of columns per CTA: a power of two that puts about one CTA on every SM, at least eight (a warp then reads whole sectors)
+    int kvs = 256;
+    while (kvs > 8 && ctas * ((nkv + kvs - 1) / kvs) < 148) kvs /= 2;
+    const dim3 grid(ctas, (nkv + kvs - 1) / kvs);
+    Scope sc(KC_FMA_WGRAD, (dx_or_null ? 4.0 : 2.0) * M * K * C, (dt ? 2.0 : 4.0) * ((double)M * K * (dx_or_null ? 2 : 1) + (double)C * K + (double)M * C), s);
+    if (dt) klaunch(head_bwd_k<bf16>, grid, 256, 0, s, (const bf16*)x, (const bf16*)W, (const bf16*)dlogits, (bf16*)dx_or_null, scratch, col_or_null, M, K, C, kvs, accum_dx, mask_dx);
+    else klaunch(head_bwd_k<float>, grid, 256, 0, s, (const float*)x, (const float*)W, (const float*)dlogits, (float*)dx_or_null, scratch, col_or_null, M, K, C, kvs, accum_dx, mask_dx);
+}
+void head_reduce(float* dW, float* db_or_null, const float* scratch, int M, int K, int C, cudaStream_t s) {
+    const unsigned ctas = (M + HEAD_ROWS_PER_CTA - 1) / HEAD_ROWS_PER_CTA;
     Scope sc(KC_SPLITK, 0.0, 4.0 * (ctas + 1) * C * (K + 1), s);
-    klaunch(head_reduce_k, cdiv((size_t)C * (K + 1), 256), 256, 0, s, scratch, dW, db_or_null, (int)ctas, K, C);
+    klaunch(head_reduce_k, cdiv((size_t)C * (K + 1), 64), 64, 0, s, scratch, dW, db_or_null, (int)ctas, K, C);
 }
 
 // ------------------------------------------------------------------------------------------

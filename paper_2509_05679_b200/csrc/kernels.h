@@ -61,9 +61,15 @@ void relu_backward(int dt, const void* y, const void* dy, void* dx, size_t n, bo
 void add_forward(int dt, const void* a, const void* b, void* y, size_t n, cudaStream_t st);
 void copy_or_accumulate(int dt, const void* src, void* dst, size_t n, bool accum, cudaStream_t st);
 void maxpool_forward(int dt, const void* x, void* y, int N, int H, int W, int C, cudaStream_t st);
-void maxpool_backward(int dt, const void* x, const void* dy, void* dx, int N, int H, int W, int C, bool accum, cudaStream_t st);
+// Where the input of a backward pass's layer is a ReLU layer's output, the pass can apply that ReLU's mask to the gradient it produces and leave
+// the masked gradient's column sums (the layer's bias gradient) as records [rec][C][2], the sums in element 0: col_or_null (C / V a power
+// of two <= 256, V = 8 bf16 / 4 fp32 values), *_col_records records, added by colsum_records.
+void colsum_records(const float* part, float* out, int recs, int C, bool accum, cudaStream_t st);
+int  pool_col_records(int dt, int N, int H, int W, int C);
+int  gap_col_records(int dt, int N, int HW, int C);
+void maxpool_backward(int dt, const void* x, const void* dy, void* dx, int N, int H, int W, int C, bool accum, float* col_or_null, cudaStream_t st);
 void gap_forward(int dt, const void* x, void* y, int N, int HW, int C, cudaStream_t st);
-void gap_backward(int dt, const void* dy, void* dx, int N, int HW, int C, bool accum, cudaStream_t st);
+void gap_backward(int dt, const void* dy, void* dx, int N, int HW, int C, bool accum, const void* mask_x_or_null, float* col_or_null, cudaStream_t st);
 
 // Batch-norm with per-worker statistics.  x: [n_workers * rows_per_worker, C].
 // err: device word that a kernel sets non-zero if a bounded wait on an asynchronous copy gave up (nullptr: the
@@ -108,14 +114,17 @@ void softmax_ce(int dt, const float* logits, const int32_t* labels, void* dlogit
 
 // Classifier head (the last linear layer, c_in = K -> C classes, C <= 16) fused with the loss.  head_forward_loss: logits
 // (fp32), dlogits = (softmax - onehot) * scale (storage dtype) and the mean loss in one launch; `counter` is a device word
-// that is zero between launches.  head_backward: dx (+)= dlogits W (dx_or_null == nullptr: not needed), dW, db.
+// that is zero between launches.  head_backward: dx (+)= dlogits W (dx_or_null == nullptr: not needed) and the
+// partial sums of dW, db, which head_reduce adds; mask_dx, col: see below.
 // scratch: head_scratch_elems floats, used by both (the loss partials follow the weight-gradient partials).
 bool   head_supported(int dt, int K, int C);
 size_t head_scratch_elems(int M, int K, int C);
 void   head_forward_loss(int dt, const void* x, const void* W, const float* bias, const int32_t* labels, float* logits, void* dlogits, float* scratch,
                          unsigned* counter, LossRecord* rec, const int* err, long long seq, int M, int K, int C, float scale, cudaStream_t st);
-void   head_backward(int dt, const void* x, const void* W, const void* dlogits, void* dx_or_null, bool accum_dx, float* dW, float* db_or_null, float* scratch,
-                     int M, int K, int C, cudaStream_t st);
+int    head_col_records(int M);
+void   head_backward(int dt, const void* x, const void* W, const void* dlogits, void* dx_or_null, bool accum_dx, bool mask_dx, float* col_or_null, float* scratch, int M,
+                     int K, int C, cudaStream_t st);
+void   head_reduce(float* dW, float* db_or_null, const float* scratch, int M, int K, int C, cudaStream_t st);        // what head_backward left in scratch
 
 // master -= lr * grad (skipped when grad == nullptr: w(t+1) = w(t)); copy_next = storage-dtype copy of
 // the new master (the next weight version).  n must be a multiple of 4; pointers 16-byte aligned.
