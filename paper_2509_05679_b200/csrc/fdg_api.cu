@@ -79,6 +79,7 @@ struct Op {
                                                              //      (this many per worker) for the batch-norm that follows
     int fstat_tiles;                                         // > 0: the same from the FMA kernel (fconv.cu): records of this many tiles per worker
     int stat_buf;                                            // which of the module's two buffers holds them (both ops)
+    bool bn_small; size_t red_off;                           // OP_BN: bnc_* kernels; offset of its worker sums in the module's red
     bool bn_from_conv;                                       // OP_BN: the convolution in front leaves such records (fp32: bnf_forward)
     tc::WgParams kw;
     std::vector<char*> a_ptrs, dy_ptrs;                      // the buffers the A / dY maps below were built for
@@ -306,13 +307,17 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             tc::pixel_tile(g.Ho, g.Wo, 64, &wt, &ht, &nt);
             int row_blocks = g.R * g.R * g.C / 64;
             long ptiles = (long)(g.Wo / wt) * (g.Ho / ht) * ((g.N + nt - 1) / nt);
+            // a short contraction and many tiles: one CTA per tile goes through all of it and writes the gradient itself (no partial matrices, no
+            // reduction); the widest tile that still gives two thirds of the SMs something to do
+            const bool direct = ptiles <= 24 && (row_blocks + 1) / 2 * (g.Co / 64) >= 64;
+            if (direct) while (o.n_tile_w > 64 && (row_blocks + 1) / 2 * (g.Co / o.n_tile_w) < 100) o.n_tile_w /= 2;
             int tiles = ((row_blocks + 1) / 2) * (g.Co / o.n_tile_w);
             long want = ((o.n_tile_w == 64 ? 4 : 2) * ctx->grid_sms) / tiles;   // CTAs = tiles * splits fill whole waves of the context's SMs (two CTAs per SM fit for the 64-column tile)
-            long splits = want < 1 ? 1 : want;
+            long splits = want < 1 || direct ? 1 : want;
             if (splits > ptiles) splits = ptiles;
             long pps = (ptiles + splits - 1) / splits;
             o.wg_splits = (int)((ptiles + pps - 1) / pps);
-            o.wgr_variant = (g.R == 3 && g.stride == 1) ? tc::wg_rows_variant(g.H, g.W, g.C, g.Co) : 0;
+            o.wgr_variant = (g.R == 3 && g.stride == 1 && !direct) ? tc::wg_rows_variant(g.H, g.W, g.C, g.Co) : 0;
             if (o.wgr_variant) {
                 tc::pixel_tile(g.Ho, g.Wo, 128, &wt, &ht, &nt);
                 o.wgr_splits = tc::wg_rows_splits(o.wgr_variant, g.C, g.Co, (long)(g.Ho / ht) * ((g.N + nt - 1) / nt), ctx->grid_sms);
@@ -419,12 +424,15 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
         if (d.loc == LOC_STASH) { d.off = soff; soff += align_up(d.elems() * ctx->M * ctx->esz, 256); }
         if (d.own_grad) { d.goff = goff; goff += align_up(d.elems() * ctx->M * ctx->esz, 256); }
     }
+    size_t red_pos = 0;
     m.ws_elems = 0; m.scratch_elems = 64; m.red_elems = 4;
     for (Op& o : m.ops) {
         if (o.type == OP_BN) {
             o.stats_off = soff; soff += align_up((size_t)ctx->n_workers * o.g.C * (ctx->dt == 0 ? 4 : 2) * sizeof(float), 256);
             m.scratch_elems = std::max(m.scratch_elems, (size_t)128 * ctx->n_workers * o.g.C * 2);
-            m.red_elems = std::max(m.red_elems, (size_t)ctx->n_workers * o.g.C * 2);
+            o.red_off = red_pos; red_pos += (size_t)ctx->n_workers * o.g.C * 2;
+            m.red_elems = std::max(m.red_elems, red_pos);
+            o.bn_small = ctx->R == 1 && bnc_supported(ctx->dt, ctx->n_workers, (long)ctx->B * m.t[o.in].h * m.t[o.in].w, o.g.C);
         }
         if (o.type == OP_CONV) {
             if (o.tc) m.ws_elems = std::max(m.ws_elems, (size_t)std::max(o.wg_splits, o.wgr_variant ? o.wgr_splits : 0) * o.g.R * o.g.R * o.g.C * o.g.Co);
@@ -447,6 +455,7 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
         while (j < m.ops.size() && !(m.ops[j].type == OP_BN && m.ops[j].in == o.out)) ++j;
         if (j == m.ops.size()) continue;
         Op& bn = m.ops[j];
+        if (bn.bn_small) continue;                           // takes its statistics itself
         o.stat_buf = bn.stat_buf = j == i + 1 ? 0 : 1;
         size_t& elems = m.cstat_elems[o.stat_buf];
         if (o.tc || o.stem_tc) {
@@ -656,6 +665,12 @@ void forward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int group, 
                 char tag[40];
                 std::snprintf(tag, sizeof tag, "%dx%dx%d%s%s", ti.h, ti.w, ti.c, o.has_res ? " +res" : "", o.relu ? " relu" : "");
                 profile_detail(tag);
+                if (o.bn_small && m.groups == 1) {
+                    bnc_forward(T(o.in), wsmall(c, m, version, o.gamma_off, rep), wsmall(c, m, version, o.beta_off, rep), o.has_res ? T(o.in2) : nullptr, T(o.out), P.stats(o),
+                                c->n_workers, (long)c->B * ti.h * ti.w, ti.c, o.relu, s);
+                    profile_detail(nullptr);
+                    break;
+                }
                 const bool fused = m.fused_stats_tensor[o.stat_buf] == o.in;
                 float* const cstat = m.cstat[o.stat_buf];
                 const int fused_chunks = m.fused_stats_chunks[o.stat_buf];
@@ -827,6 +842,15 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
                 std::snprintf(tag, sizeof tag, "%dx%dx%d%s%s", ti.h, ti.w, ti.c, o.has_res ? " +res" : "", o.relu ? " relu" : "");
                 profile_detail(tag);
                 char* gres = o.has_res ? G(o.in2) : nullptr;
+                if (o.bn_small && m.groups == 1) {
+                    bnc_backward(T(o.in), T(o.out), gout, wsmall(c, m, version, o.gamma_off, rep), wsmall(c, m, version, o.beta_off, rep), P.stats(o), gin, o.acc_in, gres,
+                                 o.acc_in2, m.red + o.red_off, c->n_workers, (long)c->B * ti.h * ti.w, ti.c, o.relu, o.has_res, s);
+                    cudaStream_t ws = m.wstream;                     // the parameter gradients are needed by the update only
+                    if (ws != s) { step_record(m.wev, s); step_wait(ws, m.wev); }
+                    bnc_params(m.red + o.red_off, mgrad + m.n_big + o.gamma_off, mgrad + m.n_big + o.beta_off, c->n_workers, ti.c, ws);
+                    profile_detail(nullptr);
+                    break;
+                }
                 if (o.bn_from_conv && dt == 0) {
                     bnf_backward((const float*)T(o.in), (const float*)T(o.out), (const float*)gout, wsmall(c, m, version, o.gamma_off, rep),
                                  wsmall(c, m, version, o.beta_off, rep), 0, P.stats(o) + (size_t)wn.w0 * ti.c * 4, (float*)gin, o.acc_in, (float*)gres, o.acc_in2,

@@ -1153,13 +1153,15 @@ __global__ void __launch_bounds__(256) head_fwd_loss_k(const T* __restrict__ x, 
             float xv[8];
             Vec<T>::load(xr + (size_t)kv * V, xv);
 #pragma unroll
-            for (int c = 0; c < HEAD_MAX_C; ++c) {
-                if (c < C) {
-                    float wv[8];
-                    Vec<T>::load(W + (size_t)c * K + (size_t)kv * V, wv);
+            for (int c = 0; c < HEAD_MAX_C; c += 8) {            // eight classes' loads in flight; a class that does not exist repeats the last one
+                if (c >= C) break;
+                float wv[8][8];
 #pragma unroll
-                    for (int j = 0; j < V; ++j) acc[c] = fmaf(xv[j], wv[j], acc[c]);
-                }
+                for (int q = 0; q < 8; ++q) Vec<T>::load(W + (size_t)min(c + q, C - 1) * K + (size_t)kv * V, wv[q]);
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+#pragma unroll
+                    for (int j = 0; j < V; ++j) acc[c + q] = fmaf(xv[j], wv[q][j], acc[c + q]);
             }
         }
         float z = 0.f;                       // lane c keeps logit c
