@@ -438,10 +438,11 @@ int bnf_chunks(int nw, long rpw, int C) {
 }  // namespace
 
 template <bool BWD>
-static void bnc_launch(const BncArgs& a, int nw, cudaStream_t s) {
-    // channels per cluster: 64 (whole 128-byte lines), fewer where that leaves most SMs without a CTA
+static void bnc_launch(const BncArgs& a, int nw, int nw_all, cudaStream_t s) {
+    // channels per cluster: 64 (whole 128-byte lines), fewer where that leaves most SMs without a CTA (by the number of ALL workers: a launch for
+    // a group of them adds in the same order)
     int sl = 64;
-    while (sl > 16 && (a.C / sl) * nw * BNC_RANKS < 100) sl /= 2;
+    while (sl > 16 && (a.C / sl) * nw_all * BNC_RANKS < 100) sl /= 2;
     const dim3 grid((a.C / sl) * BNC_RANKS, nw);
     if (sl == 64) klaunch_cluster(bnc_kernel<64, BWD>, grid, BT, 0, s, BNC_RANKS, a);
     else if (sl == 32) klaunch_cluster(bnc_kernel<32, BWD>, grid, BT, 0, s, BNC_RANKS, a);
@@ -450,19 +451,19 @@ static void bnc_launch(const BncArgs& a, int nw, cudaStream_t s) {
 // Tensors up to 8 MB: read twice out of L2 (beyond that the streamed kernels' DRAM rate counts, not the launches), and few enough rows per
 // thread for plain fp32 sums (at most 16 384 / 8 / 32 = 64).
 bool bnc_supported(int dt, int nw, long rpw, int C) { return dt == 1 && C % 64 == 0 && rpw <= 16384 && (double)nw * rpw * C * 2.0 <= 8e6; }
-void bnc_forward(const void* x, const float* gamma, const float* beta, const void* res, void* y, float* stats, int nw, long rpw, int C, bool relu, cudaStream_t s) {
+void bnc_forward(const void* x, const float* gamma, const float* beta, const void* res, void* y, float* stats, int nw, int nw_all, long rpw, int C, bool relu, cudaStream_t s) {
     BncArgs a{};
     a.x = (const bf16*)x; a.gamma = gamma; a.beta = beta; a.res = (const bf16*)res; a.y = (bf16*)y; a.stats = stats; a.rpw = (int)rpw; a.C = C; a.relu = relu;
     Scope sc(KC_BN_FWD_APPLY, 0.0, 2.0 * nw * rpw * C * (res ? 3 : 2), s);
-    bnc_launch<false>(a, nw, s);
+    bnc_launch<false>(a, nw, nw_all, s);
 }
 void bnc_backward(const void* x, const void* out, const void* dout, const float* gamma, const float* beta, const float* stats, void* dx, bool accum_dx, void* dres,
-                  bool accum_dres, float* red, int nw, long rpw, int C, bool relu, bool has_res, cudaStream_t s) {
+                  bool accum_dres, float* red, int nw, int nw_all, long rpw, int C, bool relu, bool has_res, cudaStream_t s) {
     BncArgs a{};
     a.x = (const bf16*)x; a.out = (const bf16*)out; a.dout = (const bf16*)dout; a.gamma = gamma; a.beta = beta; a.stats = (float*)stats; a.y = (bf16*)dx;
     a.accum_dx = accum_dx; a.dres = (bf16*)dres; a.accum_dres = accum_dres; a.red = red; a.rpw = (int)rpw; a.C = C; a.relu = relu; a.mask_from_x = relu && !has_res;
     Scope sc(KC_BN_BWD_APPLY, 0.0, 2.0 * nw * rpw * C * (3 + (relu && has_res ? 1 : 0) + (accum_dx ? 1 : 0) + (dres ? (accum_dres ? 2 : 1) : 0)), s);
-    bnc_launch<true>(a, nw, s);
+    bnc_launch<true>(a, nw, nw_all, s);
 }
 void bnc_params(const float* red, float* dgamma, float* dbeta, int nw, int C, cudaStream_t s) {
     Scope sc(KC_BN_BWD_REDUCE, 0.0, 8.0 * nw * C, s);
