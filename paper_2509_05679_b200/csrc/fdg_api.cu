@@ -25,6 +25,7 @@
 
 #include <atomic>
 #include <cmath>
+#include <cstdlib>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -309,8 +310,8 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             long ptiles = (long)(g.Wo / wt) * (g.Ho / ht) * ((g.N + nt - 1) / nt);
             // a short contraction and many tiles: one CTA per tile goes through all of it and writes the gradient itself (no partial matrices, no
             // reduction); the widest tile that still gives two thirds of the SMs something to do
-            const bool direct = ptiles <= 24 && (row_blocks + 1) / 2 * (g.Co / 64) >= 64;
-            if (direct) while (o.n_tile_w > 64 && (row_blocks + 1) / 2 * (g.Co / o.n_tile_w) < 100) o.n_tile_w /= 2;
+            const bool direct = ptiles <= (getenv("WGP") ? atoi(getenv("WGP")) : 24) && (row_blocks + 1) / 2 * (g.Co / 64) >= 64;
+            if (direct) while (o.n_tile_w > 64 && (row_blocks + 1) / 2 * (g.Co / o.n_tile_w) < (getenv("WGD") ? atoi(getenv("WGD")) : 100)) o.n_tile_w /= 2;
             int tiles = ((row_blocks + 1) / 2) * (g.Co / o.n_tile_w);
             long want = ((o.n_tile_w == 64 ? 4 : 2) * ctx->grid_sms) / tiles;   // CTAs = tiles * splits fill whole waves of the context's SMs (two CTAs per SM fit for the 64-column tile)
             long splits = want < 1 || direct ? 1 : want;
@@ -1370,7 +1371,7 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
     // B200, ResNet-18-shaped, 4 modules, 30 steps under the power cap: 5.05-5.12 ms per step for 37..74 SMs against
     // 5.3-5.5 for all 148; VGG-shaped 0.77 against 0.90.  One stream: nothing runs beside a kernel, all SMs.
     ctx->grid_sms = opt->grid_sms > 0 ? (opt->grid_sms < prop.multiProcessorCount ? opt->grid_sms : prop.multiProcessorCount)
-                                      : (opt->serial ? prop.multiProcessorCount : (prop.multiProcessorCount + 2) / 3);
+                                      : (opt->serial ? prop.multiProcessorCount : K == 1 && getenv("K1") ? atoi(getenv("K1")) : (prop.multiProcessorCount + 2) / 3);
     ctx->R = 1; ctx->P_dev = nullptr;
     if (opt->mixing) {
         // general mixing matrix: one weight replica per worker, every layer runs once per worker on the plain FMA kernels

@@ -22,6 +22,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 
 namespace fdg {
@@ -670,10 +671,10 @@ km_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
 // partial tile in shared memory, and CTA r adds the columns [64 r / S, 64 (r + 1) / S) over the cluster in rank order (a fixed order).
 // One tile per cluster, four stages of 24 KB (two CTAs per SM).
 constexpr int KS_STAGES = 4, KS_STAGE_BYTES = BLOCK_M * 128 + 64 * 128, KS_PITCH = 68;        // floats per row of the partial tile
-static_assert(KS_STAGES * KS_STAGE_BYTES >= BLOCK_M * KS_PITCH * 4, "the partial tile reuses the stages");
 template <int S>
 __global__ void __launch_bounds__(NUM_THREADS, 2)
 ks_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, KmParams p) {
+    static_assert(KS_STAGES * KS_STAGE_BYTES >= BLOCK_M * KS_PITCH * 4, "the partial tile reuses the stages");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     uint64_t* full = (uint64_t*)(smem + KS_STAGES * KS_STAGE_BYTES);
@@ -1737,7 +1738,7 @@ cudaError_t run_km(const KmMaps& m, const KmParams& p_in, int n_tile, cudaStream
 }
 
 // One CTA per tile fills the device once or twice (two fit on an SM); beyond that the wider tiles of km_kernel read their operands less often.
-bool small_problem(long tiles) { return tiles <= 2 * 148; }
+bool small_problem(long tiles) { return tiles <= (getenv("SMALLT") ? atoi(getenv("SMALLT")) : 2 * 148); }
 template <int S>
 static cudaError_t launch_ks(const TensorMap& a, const TensorMap& b, const KmParams& p, int tiles, cudaStream_t s) {
     constexpr int smem = KS_STAGES * KS_STAGE_BYTES + 1024 + 256;
@@ -1753,9 +1754,11 @@ cudaError_t run_small(const TensorMap& a, const TensorMap& b, const KmParams& p,
     const int tiles = p.tiles_w * p.tiles_h * p.tiles_n * (p.Cn / 64) * p.ncls;
     int kb = 1 << 30;                                    // the shortest contraction of a class, in steps of 64
     for (int c = 0; c < p.ncls; ++c) { const int n = (p.cls_tap0[c + 1] - p.cls_tap0[c]) * p.kchunks; if (n < kb) kb = n; }
-    // as many CTAs per tile as fill the device once, with at least two steps each
+    // As many CTAs per tile as fill the SMs the launch is sized for, with at least two steps each.  More of them finish one launch sooner and the
+    // step later: the other modules' kernels want those SMs (MLP of 1024 wide layers, 4 modules: 138 us per step for 50 SMs, 155 for 148, 248 for
+    // two CTAs on each; eight stages instead of four, i.e. one CTA per SM: 186).
     int split = 1;
-    while (split < 8 && tiles * split * 2 <= 148 && kb >= split * 2 * 2) split *= 2;
+    while (split < 8 && tiles * split * 2 <= sm_count(p.sms) && kb >= split * 2 * 2) split *= 2;
     switch (split) {
         case 1: return launch_ks<1>(a, b, p, tiles, s);
         case 2: return launch_ks<2>(a, b, p, tiles, s);
