@@ -120,7 +120,7 @@ typedef struct {
     int32_t grid_sms;          /* SMs the persistent kernels (tensor-core convolutions / GEMMs, streamed batch-norm) size
                                   their grids for.  0: a third of the device's SMs when the modules run on streams of their
                                   own (the concurrency of Sec. 3.2: a tensor-core kernel of one module then runs beside a
-                                  memory-bound kernel of another instead of after it), all of them with serial = 1.
+                                  memory-bound kernel of another instead of after it), two thirds with one module, all of them with serial = 1.
                                   n > 0: n SMs (clamped to the device).  Results depend on it only through fp32 summation
                                   order (contraction splits, batch-norm row chunks): two contexts with the same value are
                                   bit-identical whatever their streams                                              */

@@ -25,7 +25,6 @@
 
 #include <atomic>
 #include <cmath>
-#include <cstdlib>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -72,6 +71,7 @@ struct Op {
                                                              // gradient it produces and leaves the bias gradient's records
     int masks;                                               // > 0: the reverse: this op does that for op masks - 1
     size_t col_off; int col_recs;                            // of the masked layer: its records in the module's bstat
+    int split_f, split_d;                                    // CTAs per tile of those launches
     bool small_f, small_d;                                   // few tiles: forward / input gradient by tc::run_small (n_tile_f / n_tile_d = 64)
     tc::KmParams kf;
     tc::KmParams kd;                                         // all output-parity classes of the input gradient in one launch
@@ -300,8 +300,8 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             o.n_tile_w = g.Co % 256 == 0 ? 256 : (g.Co % 128 == 0 ? 128 : 64);
             {
                 const long pix = (long)(g.Wo / wt) * (g.Ho / ht) * ((g.N + nt - 1) / nt);
-                o.small_f = tc::small_problem(pix * (g.Co / 64));
-                o.small_d = tc::small_problem(pix * (g.C / 64) * g.stride * g.stride);
+                o.small_f = tc::small_problem(pix * (g.Co / 64), ctx->grid_sms);
+                o.small_d = tc::small_problem(pix * (g.C / 64) * g.stride * g.stride, ctx->grid_sms);
                 if (o.small_f) o.n_tile_f = 64;
                 if (o.small_d) o.n_tile_d = 64;
             }
@@ -309,9 +309,9 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             int row_blocks = g.R * g.R * g.C / 64;
             long ptiles = (long)(g.Wo / wt) * (g.Ho / ht) * ((g.N + nt - 1) / nt);
             // a short contraction and many tiles: one CTA per tile goes through all of it and writes the gradient itself (no partial matrices, no
-            // reduction); the widest tile that still gives two thirds of the SMs something to do
-            const bool direct = ptiles <= (getenv("WGP") ? atoi(getenv("WGP")) : 24) && (row_blocks + 1) / 2 * (g.Co / 64) >= 64;
-            if (direct) while (o.n_tile_w > 64 && (row_blocks + 1) / 2 * (g.Co / o.n_tile_w) < (getenv("WGD") ? atoi(getenv("WGD")) : 100)) o.n_tile_w /= 2;
+            // reduction); the widest tile that still gives half of the launch's SMs something to do
+            const bool direct = ptiles <= 24 && (row_blocks + 1) / 2 * (g.Co / 64) >= 64;
+            if (direct) while (o.n_tile_w > 64 && (row_blocks + 1) / 2 * (g.Co / o.n_tile_w) < ctx->grid_sms / 2) o.n_tile_w /= 2;
             int tiles = ((row_blocks + 1) / 2) * (g.Co / o.n_tile_w);
             long want = ((o.n_tile_w == 64 ? 4 : 2) * ctx->grid_sms) / tiles;   // CTAs = tiles * splits fill whole waves of the context's SMs (two CTAs per SM fit for the 64-column tile)
             long splits = want < 1 || direct ? 1 : want;
@@ -540,7 +540,7 @@ bool tc_forward(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* y_base, 
     const int io = find_buf(o.y_ptrs, y_base);
     const tc::KmMaps maps{&o.fa[ia], o.far.empty() ? nullptr : &o.far[ia], &o.fb[version % m.D], o.fbh.empty() ? nullptr : &o.fbh[version % m.D],
                           io >= 0 ? &o.fo[io] : nullptr};
-    const bool ok = (o.small_f ? tc::run_small(*maps.a, *maps.b, p, s) : tc::run_km(maps, p, o.n_tile_f, s)) == cudaSuccess;
+    const bool ok = (o.small_f ? tc::run_small(*maps.a, *maps.b, p, o.split_f, s) : tc::run_km(maps, p, o.n_tile_f, s)) == cudaSuccess;
     if (ok && o.stat_chunks) { m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.stat_chunks; }
     return ok;
 }
@@ -562,7 +562,7 @@ bool tc_dgrad(fdg_ctx* c, Module& m, const Op& o, char* dy_base, char* dx_base, 
     const int io = find_buf(o.dx_ptrs, dx_base);
     const tc::KmMaps maps{&o.da[ia], o.dar.empty() ? nullptr : &o.dar[ia], &o.db[version % m.D], o.dbh.empty() ? nullptr : &o.dbh[version % m.D],
                           io >= 0 ? &o.dox[io] : nullptr};
-    return (o.small_d ? tc::run_small(*maps.a, *maps.b, p, s) : tc::run_km(maps, p, o.n_tile_d, s)) == cudaSuccess;
+    return (o.small_d ? tc::run_small(*maps.a, *maps.b, p, o.split_d, s) : tc::run_km(maps, p, o.n_tile_d, s)) == cudaSuccess;
 }
 bool tc_wgrad(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* dy_base, float* dw, const Win& wn, cudaStream_t s) {
     int ix = find_buf(o.a_ptrs, x_base), id = find_buf(o.dy_ptrs, dy_base);
@@ -1079,6 +1079,8 @@ bool build_tc_plans(fdg_ctx* c) {
                 o.wxr.resize(o.a_ptrs.size());
                 for (size_t i = 0; i < o.a_ptrs.size(); ++i) ok = ok && tc::make_map_4d(&o.wxr[i], o.a_ptrs[i], g.C, g.W, g.H, g.N, 64, g.W, ht + 2, nt, 1);
             }
+            o.kf.sms = o.kd.sms = c->grid_sms;
+            o.split_f = tc::small_split(o.kf); o.split_d = tc::small_split(o.kd);
             if (!ok) return false;
             c->any_tc = true;
         }
@@ -1369,9 +1371,10 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
     // of different modules run side by side instead of one after the other (a streamed batch-norm kernel keeps 92 % of
     // its bandwidth on half of the SMs, a tensor-core kernel takes 1.6 times as long there, not twice).  Measured on a
     // B200, ResNet-18-shaped, 4 modules, 30 steps under the power cap: 5.05-5.12 ms per step for 37..74 SMs against
-    // 5.3-5.5 for all 148; VGG-shaped 0.77 against 0.90.  One stream: nothing runs beside a kernel, all SMs.
+    // 5.3-5.5 for all 148; VGG-shaped 0.77 against 0.90.  One module: two thirds (only its weight gradients run beside its other kernels; ResNet-18-
+    // shaped, 4 workers x 30: 1.57 ms per step for 74..148 SMs against 1.67 for 50).  One stream: nothing runs beside a kernel, all SMs.
     ctx->grid_sms = opt->grid_sms > 0 ? (opt->grid_sms < prop.multiProcessorCount ? opt->grid_sms : prop.multiProcessorCount)
-                                      : (opt->serial ? prop.multiProcessorCount : K == 1 && getenv("K1") ? atoi(getenv("K1")) : (prop.multiProcessorCount + 2) / 3);
+                                      : (opt->serial ? prop.multiProcessorCount : K == 1 ? (2 * prop.multiProcessorCount + 2) / 3 : (prop.multiProcessorCount + 2) / 3);
     ctx->R = 1; ctx->P_dev = nullptr;
     if (opt->mixing) {
         // general mixing matrix: one weight replica per worker, every layer runs once per worker on the plain FMA kernels

@@ -22,7 +22,6 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cstdio>
-#include <cstdlib>
 #include <cstring>
 
 namespace fdg {
@@ -1737,8 +1736,22 @@ cudaError_t run_km(const KmMaps& m, const KmParams& p_in, int n_tile, cudaStream
     return cudaErrorInvalidValue;
 }
 
-// One CTA per tile fills the device once or twice (two fit on an SM); beyond that the wider tiles of km_kernel read their operands less often.
-bool small_problem(long tiles) { return tiles <= (getenv("SMALLT") ? atoi(getenv("SMALLT")) : 2 * 148); }
+static int sm_count(int sms);
+// Tiles for up to two CTAs on each of the SMs a launch is sized for; beyond that the wider tiles of km_kernel, which read their operands less often,
+// are faster (ResNet-18-shaped, 4 modules on 50 SMs each, 4 workers x 16: 678 us per step with the line at 100 tiles, 693 at 148, 729 at 296, 781 at 600).
+bool small_problem(long tiles, int sms) { return tiles <= 2 * sm_count(sms); }
+// As many CTAs per tile as fill the SMs the launch is sized for, with at least two steps of 64 each (by the whole batch: a launch for a group of the
+// workers splits, and adds, in the same way).  More of them finish one launch sooner and the step later: the other modules' kernels want
+// those SMs (MLP of 1024 wide layers, 4 modules: 138 us per step for 50 SMs, 155 for 148, 248 for two CTAs on each; eight stages instead of
+// four, i.e. one CTA per SM: 186).
+int small_split(const KmParams& p) {
+    const int tiles = p.tiles_w * p.tiles_h * p.tiles_n * (p.Cn / 64) * p.ncls;
+    int kb = 1 << 30;                                    // the shortest contraction of a class
+    for (int c = 0; c < p.ncls; ++c) { const int n = (p.cls_tap0[c + 1] - p.cls_tap0[c]) * p.kchunks; if (n < kb) kb = n; }
+    int split = 1;
+    while (split < 8 && tiles * split * 2 <= sm_count(p.sms) && kb >= split * 2 * 2) split *= 2;
+    return split;
+}
 template <int S>
 static cudaError_t launch_ks(const TensorMap& a, const TensorMap& b, const KmParams& p, int tiles, cudaStream_t s) {
     constexpr int smem = KS_STAGES * KS_STAGE_BYTES + 1024 + 256;
@@ -1750,15 +1763,8 @@ static cudaError_t launch_ks(const TensorMap& a, const TensorMap& b, const KmPar
     }
     return klaunch_cluster(ks_kernel<S>, dim3(tiles * S), dim3(NUM_THREADS), smem, s, S > 1 ? S : 0, *(const CUtensorMap*)&a, *(const CUtensorMap*)&b, p);
 }
-cudaError_t run_small(const TensorMap& a, const TensorMap& b, const KmParams& p, cudaStream_t s) {
+cudaError_t run_small(const TensorMap& a, const TensorMap& b, const KmParams& p, int split, cudaStream_t s) {
     const int tiles = p.tiles_w * p.tiles_h * p.tiles_n * (p.Cn / 64) * p.ncls;
-    int kb = 1 << 30;                                    // the shortest contraction of a class, in steps of 64
-    for (int c = 0; c < p.ncls; ++c) { const int n = (p.cls_tap0[c + 1] - p.cls_tap0[c]) * p.kchunks; if (n < kb) kb = n; }
-    // As many CTAs per tile as fill the SMs the launch is sized for, with at least two steps each.  More of them finish one launch sooner and the
-    // step later: the other modules' kernels want those SMs (MLP of 1024 wide layers, 4 modules: 138 us per step for 50 SMs, 155 for 148, 248 for
-    // two CTAs on each; eight stages instead of four, i.e. one CTA per SM: 186).
-    int split = 1;
-    while (split < 8 && tiles * split * 2 <= sm_count(p.sms) && kb >= split * 2 * 2) split *= 2;
     switch (split) {
         case 1: return launch_ks<1>(a, b, p, tiles, s);
         case 2: return launch_ks<2>(a, b, p, tiles, s);

@@ -75,8 +75,10 @@ struct KmMaps { const TensorMap* a; const TensorMap* a_rows; const TensorMap* b;
 cudaError_t run_km(const KmMaps& m, const KmParams& p, int n_tile, cudaStream_t s);
 // The same computation for problems of few tiles: 64-column tiles, each split over the contraction among the CTAs of a cluster.  b: box of 64 rows.
 // small_problem: whether run_small is the kernel for `tiles` = pixel tiles x 64-column tiles x classes (decided when the maps are made).
-bool small_problem(long tiles);
-cudaError_t run_small(const TensorMap& a, const TensorMap& b, const KmParams& p, cudaStream_t s);
+// small_split: CTAs per tile (p of the whole batch).
+bool small_problem(long tiles, int sms);
+int small_split(const KmParams& p);
+cudaError_t run_small(const TensorMap& a, const TensorMap& b, const KmParams& p, int split, cudaStream_t s);
 // accum: dw += the result (second and later groups of workers)
 cudaError_t run_wg(const TensorMap& x, const TensorMap& dy, const WgParams& p, int n_tile, int splits, float* dw, bool accum, cudaStream_t s);
 // Weight gradient of a 3x3, stride-1, pad-1 layer in rows mode (x is fetched once per horizontal shift and 64-channel
