@@ -443,7 +443,7 @@ static void bnc_launch(const BncArgs& a, int nw, int nw_all, cudaStream_t s) {
     // wanted by the other modules (18 samples, 4 modules: 386 us per step with this line, 432 with 100 CTAs; by the number of ALL workers: a launch for
     // a group of them adds in the same order)
     int sl = 64;
-    while (sl > 16 && (a.C / sl) * nw_all * BNC_RANKS < 25) sl /= 2;
+    while (sl > 16 && (a.C % sl || (a.C / sl) * nw_all * BNC_RANKS < 25)) sl /= 2;
     const dim3 grid((a.C / sl) * BNC_RANKS, nw);
     if (sl == 64) klaunch_cluster(bnc_kernel<64, BWD>, grid, BT, 0, s, BNC_RANKS, a);
     else if (sl == 32) klaunch_cluster(bnc_kernel<32, BWD>, grid, BT, 0, s, BNC_RANKS, a);
@@ -451,7 +451,7 @@ static void bnc_launch(const BncArgs& a, int nw, int nw_all, cudaStream_t s) {
 }
 // Tensors up to 4 MB: read twice out of L2 (beyond that the streamed kernels' rate counts, not the launches: 4 workers x 16, 693 us per step with the
 // line at 4 MB, 729 at 8 MB, 820 at 17 MB), and few enough rows per thread for plain fp32 sums (at most 16 384 / 8 / 32 = 64).
-bool bnc_supported(int dt, int nw, long rpw, int C) { return dt == 1 && C % 64 == 0 && rpw <= 16384 && (double)nw * rpw * C * 2.0 <= 4e6; }
+bool bnc_supported(int dt, int nw, long rpw, int C) { return dt == 1 && C % 16 == 0 && rpw <= 16384 && (double)nw * rpw * C * 2.0 <= 4e6; }
 void bnc_forward(const void* x, const float* gamma, const float* beta, const void* res, void* y, float* stats, int nw, int nw_all, long rpw, int C, bool relu, cudaStream_t s) {
     BncArgs a{};
     a.x = (const bf16*)x; a.gamma = gamma; a.beta = beta; a.res = (const bf16*)res; a.y = (bf16*)y; a.stats = stats; a.rpw = (int)rpw; a.C = C; a.relu = relu;
