@@ -159,6 +159,7 @@ struct fdg_ctx {
     LossRecord* loss_ring;         // pinned host memory, 64 records
     int64_t* tags;
     int* tc_err;                   // device word: set by a tensor-core kernel whose bounded wait gave up
+    bool mask_lost = false;        // a launch that had to apply a ReLU mask was refused: the kernels that could replace it do not apply it
     bool any_tc;
     bool graphs;                   // steady-state iterations run as graphs (off once recording one has failed)
     cudaEvent_t ingested;
@@ -208,22 +209,26 @@ struct HostReader {
 };
 HostReader g_reader;
 
-// Device floats [src, src + n) -> pieces of a host array.  piece(off, count, from) copies count floats that start at element off.
+// Device floats -> pieces of a host array: n floats from src, handed to piece(tag, off, count, from) in chunks that start at element off.
+struct HostRead { const float* src; size_t n; int tag; };
 // What this costs is the host side: a plain copy into pageable memory runs through the driver's single staging thread, and the
 // caller's fresh array takes a page fault per 4 KB (11 M parameters: 14-16 ms).  Several threads each take the next chunk, copy it to a
-// pinned lane of their own on a stream of their own (DMA at the link's rate) and move it out while the other lanes' copies run.
+// pinned lane of their own on a stream of their own (DMA at the link's rate) and move it out while the other lanes' copies run.  One set of
+// threads for all the reads of a call (4.2 M parameters in four modules: 2.1-2.6 ms, 4.4 with a set per module).
 template <typename F>
-cudaError_t read_floats(const float* src, size_t n, int device, F piece) {
+cudaError_t read_floats(const std::vector<HostRead>& reads, int device, F piece) {
     constexpr size_t chunk = HostReader::LANE_BYTES / sizeof(float);
+    struct Job { const float* src; size_t off, cnt; int tag; };
+    std::vector<Job> jobs;
+    for (const HostRead& r : reads)
+        for (size_t off = 0; off < r.n; off += chunk) jobs.push_back({r.src + off, off, std::min(chunk, r.n - off), r.tag});
     std::lock_guard<std::mutex> lk(g_reader.mu);
-    const size_t jobs = (n + chunk - 1) / chunk;
     if (!g_reader.pinned || g_reader.device != device) {
         std::vector<float> h(chunk);
-        for (size_t j = 0; j < jobs; ++j) {
-            const size_t off = j * chunk, cnt = n - off < chunk ? n - off : chunk;
-            cudaError_t e = cudaMemcpy(h.data(), src + off, cnt * sizeof(float), cudaMemcpyDeviceToHost);
+        for (const Job& b : jobs) {
+            cudaError_t e = cudaMemcpy(h.data(), b.src, b.cnt * sizeof(float), cudaMemcpyDeviceToHost);
             if (e != cudaSuccess) return e;
-            piece(off, cnt, h.data());
+            piece(b.tag, b.off, b.cnt, h.data());
         }
         return cudaSuccess;
     }
@@ -232,16 +237,16 @@ cudaError_t read_floats(const float* src, size_t n, int device, F piece) {
     auto work = [&](int lane) {
         float* const buf = (float*)(g_reader.pinned + lane * HostReader::LANE_BYTES);
         if (lane > 0) cudaSetDevice(device);
-        for (size_t j; (j = next.fetch_add(1)) < jobs && err.load() == (int)cudaSuccess;) {
-            const size_t off = j * chunk, cnt = n - off < chunk ? n - off : chunk;
-            cudaError_t e = cudaMemcpyAsync(buf, src + off, cnt * sizeof(float), cudaMemcpyDeviceToHost, g_reader.stream[lane]);
+        for (size_t j; (j = next.fetch_add(1)) < jobs.size() && err.load() == (int)cudaSuccess;) {
+            const Job& b = jobs[j];
+            cudaError_t e = cudaMemcpyAsync(buf, b.src, b.cnt * sizeof(float), cudaMemcpyDeviceToHost, g_reader.stream[lane]);
             if (e == cudaSuccess) e = cudaStreamSynchronize(g_reader.stream[lane]);
             if (e != cudaSuccess) { err.store((int)e); break; }
-            piece(off, cnt, buf);
+            piece(b.tag, b.off, b.cnt, buf);
         }
     };
     // a thread is worth starting from two chunks of its own
-    const int extra = (int)std::min<size_t>(HostReader::LANES - 1, jobs / 2 > 0 ? jobs / 2 - 1 : 0);
+    const int extra = (int)std::min<size_t>(HostReader::LANES - 1, jobs.size() / 2 > 0 ? jobs.size() / 2 - 1 : 0);
     std::vector<std::thread> threads;
     try { for (int i = 1; i <= extra; ++i) threads.emplace_back(work, i); } catch (...) {}      // fewer threads then
     work(0);
@@ -834,8 +839,10 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
                     fconv_wgrad(dt, T(o.in), gout, mgrad + o.w_off, m.ws, g, 1, 0, acc_p, ws);
                 if (o.bias && !fused_rb && !o.masked_by) bias_grad(dt, gout, mgrad + m.n_big + o.b_off, m.scratch, orows, g.Co, acc_p, s);
                 if (gin && !(o.tc && tc_dgrad(c, m, o, grad_ptr(c, kk, o.out, t), grad_ptr(c, kk, o.in, t), version, o.acc_in,
-                                                     below ? P.tensor(o.in) : nullptr, col, wn, s)))
+                                                     below ? P.tensor(o.in) : nullptr, col, wn, s))) {
+                    c->mask_lost = c->mask_lost || below;
                     fconv_dgrad(dt, gout, wbig(c, m, version, o.w_off, rep), gin, g, o.acc_in ? EPI_ACCUM : 0, 1, 0, s);
+                }
                 profile_detail(nullptr);
                 break; }
             case OP_BN: {
@@ -1309,6 +1316,7 @@ fdg_status run_step(fdg_ctx* ctx, const void* inputs, const int32_t* labels, boo
         CK(cudaEventRecord(m.done[now], m.stream));
     }
     CK(cudaGetLastError());
+    if (ctx->mask_lost) return fail(ctx, FDG_ERR_CUDA, "an input-gradient kernel could not be launched");
     ctx->t = t + 1;
     if (host_loss) {
         float l = 0.f;                                  // the loss only: the last module's backward pass and update go on
@@ -1715,15 +1723,18 @@ static fdg_status gather(fdg_ctx* ctx, bool grads, int worker, float* host_out, 
     if (worker >= ctx->n_workers) return fail(ctx, FDG_ERR_INVALID_ARG, "worker %d out of range", worker);
     CK(cudaDeviceSynchronize());
     { fdg_status es = check_device_error(ctx); if (es != FDG_OK) return es; }
-    for (Module& m : ctx->mod) {
+    // internal elements [off, off + cnt) of module kk -> their places in the canonical vector
+    auto scatter = [&](int kk, size_t off, size_t cnt, const float* from) {
+        const Module& m = ctx->mod[kk];
+        for (const Segment& s : m.segs) {
+            const size_t at = (s.big ? 0 : m.n_big) + s.internal, lo = std::max(at, off), hi = std::min(at + s.count, off + cnt);
+            if (lo < hi) std::memcpy(host_out + s.canon + (lo - at), from + (lo - off), (hi - lo) * sizeof(float));
+        }
+    };
+    std::vector<HostRead> reads;
+    for (int kk = 0; kk < ctx->K; ++kk) {
+        Module& m = ctx->mod[kk];
         const size_t n = npar(m);
-        // internal elements [off, off + cnt) -> their places in the canonical vector (m.segs is in internal order within each segment class)
-        auto scatter = [&](size_t off, size_t cnt, const float* from) {
-            for (const Segment& s : m.segs) {
-                const size_t at = (s.big ? 0 : m.n_big) + s.internal, lo = std::max(at, off), hi = std::min(at + s.count, off + cnt);
-                if (lo < hi) std::memcpy(host_out + s.canon + (lo - at), from + (lo - off), (hi - lo) * sizeof(float));
-            }
-        };
         if (grads && !m.had_bwd) {
             for (const Segment& s : m.segs) std::memset(host_out + s.canon, 0, s.count * sizeof(float));
         } else if (grads && worker < 0 && ctx->R > 1) {
@@ -1735,12 +1746,13 @@ static fdg_status gather(fdg_ctx* ctx, bool grads, int worker, float* host_out, 
                 for (size_t i = 0; i < n; ++i) acc[i] += one[i];
             }
             for (size_t i = 0; i < n; ++i) one[i] = (float)(acc[i] / ctx->R);
-            scatter(0, n, one.data());
+            scatter(kk, 0, n, one.data());
         } else {
             const int r = (ctx->R > 1 && worker > 0) ? worker : 0;       // one copy: every worker has the same
-            CK(read_floats((grads ? m.grad : m.master) + (size_t)r * n, n, ctx->device, scatter));
+            reads.push_back({(grads ? m.grad : m.master) + (size_t)r * n, n, kk});
         }
     }
+    CK(read_floats(reads, ctx->device, scatter));
     if (count) *count = ctx->n_params;
     return FDG_OK;
 }

@@ -1700,7 +1700,7 @@ static cudaError_t launch_km_pair(const TensorMap& a, const TensorMap& b, const 
         if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n <= 0) { cudaGetLastError(); n = device_sms() / 2; }
         resident_pairs = n;
     }
-    const int max_pairs = resident_pairs < sm_count(p.sms) / 2 ? resident_pairs : sm_count(p.sms) / 2;
+    const int budget = sm_count(p.sms) > 1 ? sm_count(p.sms) / 2 : 1, max_pairs = resident_pairs < budget ? resident_pairs : budget;
     const int total = (p.tiles_w * p.tiles_h * p.tiles_n / 2) * (p.Cn / N_TILE) * p.ncls;
     return klaunch_cluster(kernel, dim3(2 * (total < max_pairs ? total : max_pairs)), dim3(64 + 32 * EPI_WARPS), smem, s, 2, *(const CUtensorMap*)&a, *(const CUtensorMap*)&b,
                            *(const CUtensorMap*)&o, p);
