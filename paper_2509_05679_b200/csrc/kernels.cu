@@ -1,7 +1,5 @@
-// Plain-FMA (CUDA-core) kernels: every layer kind in fp32 or bf16 storage with fp32 arithmetic.
-// They are the whole fp32 path (true fp32 FMAs: TF32 would break the 1e-5 parameter tolerance)
-// and, on the bf16 path, serve the shapes the tensor-core kernels do not take (3-channel stem,
-// strided convs, 10-class head) plus all memory-bound elementwise / reduction work.
+// Memory-bound and small kernels in fp32 or bf16 storage with fp32 arithmetic: elementwise layers, pooling, streamed batch-norm,
+// the classifier head with the loss, column sums, mixing and SGD, input copies; and the profiler all launchers report to.
 #include "kernels.h"
 #include "launch.h"
 

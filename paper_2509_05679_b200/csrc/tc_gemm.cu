@@ -5,15 +5,18 @@
 //   warp 1 : tensor-memory allocation, MMA issue (same scheme), deallocation
 //   warps 2-5 (or 2-9) : epilogue (tcgen05.ld -> registers -> bf16 tile in shared memory -> TMA store)
 //
-// Two kernels:
+// The kernels:
 //   km_kernel  (forward and input-gradient): D[pixel][c_out] = sum_{tap, c} A[pixel + tap][c] * B[c_out][tap, c]
 //              A is an NHWC activation read through a 4-D tensor map (one box per filter tap, shifted by
 //              the tap; out-of-bounds elements are zero-filled, which is the padding), B a K-major weight
 //              matrix.  Both operands are K-major in shared memory.
+//   ks_kernel  the same with few tiles: the contraction split over a cluster, added through distributed shared memory.
 //   wg_kernel  (weight gradient): D[(tap, c_in)][c_out] = sum_{pixel} X[pixel + tap][c_in] * dY[pixel][c_out]
 //              The contraction runs over pixels = worker x batch x H x W, so the average over workers is
 //              part of the contraction.  Both operands are MN-major in shared memory (channel contiguous).
 //              Split over pixels across CTAs; partial sums are reduced in a fixed order by a second kernel.
+//   wg2_kernel the same for 3x3, stride 1: three vertical taps from one fetched tile.
+//   stem_*     the 3-channel first layer: im2col lines built in shared memory.
 // Every wait on an mbarrier is bounded; a wait that gives up sets an error word and the CTA leaves
 // through the common exit (tensor memory is always released).
 #include "tc_gemm.h"
