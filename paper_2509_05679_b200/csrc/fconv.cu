@@ -11,7 +11,7 @@
 // contraction (channels 2i and 2i + 1) in fc_kernel and along c_in in fw_kernel, so that operands come out of NHWC data as
 // 16-byte vectors without shuffling.  Chains of at most 16 products are added to a compensated (Kahan) running sum, so the rounding error of a long contraction stays at a few ulps.
 //
-// What bounds them: the FMA pipe (fc_kernel issues 32 packed FMAs for eight 16-byte shared loads, fw_kernel 16 for four).
+// What bounds them: the FMA pipe (fc_kernel issues 32 packed FMAs for eight 16-byte shared loads, or 16 for six, fw_kernel 16 for four).
 // The implicit-GEMM kernel they replace fetched every operand element by itself with two integer divisions and reached
 // 2.5-9 TFLOP/s on the ResNet-20 layers.
 #include "kernels.h"
@@ -25,8 +25,7 @@ typedef __nv_bfloat16 bf16;
 
 namespace {
 
-constexpr int FC_THREADS = 128;          // 4 warps: 32 pixels x 16 output channels each, 4 pixels x 4 channels per thread
-constexpr int FC_PIX = 128;
+constexpr int FC_PIX = 128;              // 4 rows of 32 pixels x 16 output channels; a thread has PP = 4 or 2 pixels x 4 channels: 4 or 8 warps
 constexpr int FC_CO = 16;
 constexpr int FC_KC = 16;                // channels per chunk
 constexpr int PITCH = 20;                // floats per pixel (or weight row) in shared memory: 16 + 4, so that the eight 16-byte reads
@@ -128,8 +127,8 @@ struct FcParams {
 // 16 output channels x up to 16 input channels of every tap of the class into dst[tap][row][PITCH]; channel n sits in row
 // (n % 4) * 4 + n / 4, so that the four channel groups of a warp read neighbouring rows.
 template <typename T, bool VEC>
-__device__ __forceinline__ void load_weights(const T* __restrict__ w, float* dst, const FcParams& p, int t0, int t1, int co0, int c0, int nq, int tid) {
-    for (int i = tid; i < (t1 - t0) * 64; i += FC_THREADS) {
+__device__ __forceinline__ void load_weights(const T* __restrict__ w, float* dst, const FcParams& p, int t0, int t1, int co0, int c0, int nq, int tid, int nthreads) {
+    for (int i = tid; i < (t1 - t0) * 64; i += nthreads) {
         const int t = i >> 6, e = i & 63;
         const int tap = p.wtap[t0 + t];
         if (!p.back) {
@@ -161,9 +160,13 @@ __device__ __forceinline__ void load_weights(const T* __restrict__ w, float* dst
     }
 }
 
+// CTAs per SM that the register allocation allows: fp32 at four pixels a thread without spills (168 registers: ResNet-20 with one module
+// 2.77 -> 2.70 ms per step; bf16, whose operands are unpacked to the same registers, is 3 % faster with four CTAs and ten words spilled).
+template <typename T> constexpr int fc_ctas(int pp) { return pp == 2 ? 2 : sizeof(T) == 4 ? 3 : 4; }
+
 // grid = (pixel tiles, blocks of 16 output channels, groups x classes).  NQ: 4-channel quads per chunk (1: at most 4 channels).
-template <typename T, int NQ, bool VEC>
-__global__ void __launch_bounds__(FC_THREADS, 4) fc_kernel(const T* __restrict__ x, const T* __restrict__ w, const float* __restrict__ bias, T* __restrict__ y,
+template <typename T, int NQ, bool VEC, int PP>
+__global__ void __launch_bounds__(512 / PP, fc_ctas<T>(PP)) fc_kernel(const T* __restrict__ x, const T* __restrict__ w, const float* __restrict__ bias, T* __restrict__ y,
                                                            float* __restrict__ stat, const __grid_constant__ FcParams p) {
     extern __shared__ __align__(16) float fsm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -177,26 +180,27 @@ __global__ void __launch_bounds__(FC_THREADS, 4) fc_kernel(const T* __restrict__
     const int RH = p.cls_rh[cls], RW = p.cls_rw[cls], h0 = hd0 * p.xs + p.cls_h0[cls], w0 = wd0 * p.xs + p.cls_w0[cls];
     w += (size_t)grp * p.w_group;
 
-    // this thread: pixels warp * 32 + g + 8 i (i = 0..3), channels co0 + 4 cg + j
-    const int g = lane & 7, cg = lane >> 3;
-    uint32_t xb[4];
+    // this thread: pixels px0 + 8 i (i = 0..PP - 1), channels co0 + 4 cg + j; warps of the same `row` share 32 pixels
+    constexpr int NT = 512 / PP, PARTS = 4 / PP;
+    const int g = lane & 7, cg = lane >> 3, row = warp / PARTS, part_of = warp % PARTS, px0 = row * 32 + g + 8 * PP * part_of;
+    uint32_t xb[PP];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int px = warp * 32 + g + 8 * i;
+    for (int i = 0; i < PP; ++i) {
+        const int px = px0 + 8 * i;
         const int pw = px & (p.Wt - 1), ph = (px >> p.lw) & (p.Ht - 1), pn = px >> (p.lw + p.lh);
         xb[i] = (uint32_t)(((pn * RH + ph * p.xs) * RW + pw * p.xs) * PITCH);
     }
-    float2 acc[4][2], comp[4][2], part[4][4];
+    float2 acc[PP][2], comp[PP][2], part[PP][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < PP; ++i)
 #pragma unroll
         for (int j = 0; j < 2; ++j) { acc[i][j] = make_float2(0.f, 0.f); comp[i][j] = make_float2(0.f, 0.f); }
 
     const int chunks = t1 > t0 ? (p.C + FC_KC - 1) / FC_KC : 0;
     auto fetch = [&](int c, int buf) {
         float* xs_ = fsm + (size_t)buf * (p.x_floats + p.w_floats);
-        load_region<T>(VEC, x, xs_, n0, n_end, p.Nt, h0, w0, RH, RW, 1, p.H, p.W, p.C, c * FC_KC, NQ, warp, FC_THREADS / 32, lane);
-        load_weights<T, VEC>(w, xs_ + p.x_floats, p, t0, t1, co0, c * FC_KC, NQ, tid);
+        load_region<T>(VEC, x, xs_, n0, n_end, p.Nt, h0, w0, RH, RW, 1, p.H, p.W, p.C, c * FC_KC, NQ, warp, NT / 32, lane);
+        load_weights<T, VEC>(w, xs_ + p.x_floats, p, t0, t1, co0, c * FC_KC, NQ, tid, NT);
         cp_commit();
     };
     if (chunks) fetch(0, 0);
@@ -215,7 +219,7 @@ __global__ void __launch_bounds__(FC_THREADS, 4) fc_kernel(const T* __restrict__
 #pragma unroll
                 for (int j = 0; j < 4; ++j) wv[j] = *(const float4*)(wt + j * (4 * PITCH) + 4 * q);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < PP; ++i) {
                     const float4 xv = *(const float4*)(xt + xb[i] + 4 * q);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
@@ -229,7 +233,7 @@ __global__ void __launch_bounds__(FC_THREADS, 4) fc_kernel(const T* __restrict__
         };
         auto flush = [&]() {             // Kahan: acc += even + odd part, two channels per instruction
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < PP; ++i)
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
                     const float2 s = make_float2(part[i][2 * j].x + part[i][2 * j].y, part[i][2 * j + 1].x + part[i][2 * j + 1].y);
@@ -248,12 +252,12 @@ __global__ void __launch_bounds__(FC_THREADS, 4) fc_kernel(const T* __restrict__
         if (p.buffers == 1 && c + 1 < chunks) fetch(c + 1, 0);
     }
 
-    float val[4][4];
-    bool valid[4];
+    float val[PP][4];
+    bool valid[PP];
     const int co = co0 + 4 * cg;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int px = warp * 32 + g + 8 * i;
+    for (int i = 0; i < PP; ++i) {
+        const int px = px0 + 8 * i;
         const int wd = wd0 + (px & (p.Wt - 1)), hd = hd0 + ((px >> p.lw) & (p.Ht - 1)), n = n0 + (px >> (p.lw + p.lh));
         valid[i] = n < n_end && hd < p.Hd && wd < p.Wd;
         float (&v)[4] = val[i];
@@ -282,33 +286,49 @@ __global__ void __launch_bounds__(FC_THREADS, 4) fc_kernel(const T* __restrict__
     // deviations from that mean (no cancellation, whatever the mean)
     const int cnt = min(p.Wt, p.Wd - wd0) * min(p.Ht, p.Hd - hd0) * min(p.Nt, n_end - n0);
     float s[4], m[4];
-    float* const red = fsm + warp * 16 + 4 * cg;
-    auto over_pixels = [&](float* out) {             // sums over the tile's pixels: 4 per thread, 8 lanes, 4 warps, in a fixed order
+    float* const red = fsm + row * 16 + 4 * cg;
+    float4* const carry = (float4*)(fsm + 64) + row * 32 + lane;
+    // sums over the tile's pixels in a fixed order, the same for every PP: 4 pixels of a lane one after the other (over the warps that share
+    // them), 8 lanes, 4 rows of 32 pixels.  add(s) adds this thread's pixels.
+    auto over_pixels = [&](auto add) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < 4; ++j) s[j] = 0.f;
 #pragma unroll
-            for (int d = 1; d < 8; d <<= 1) out[j] += __shfl_xor_sync(0xffffffffu, out[j], d);
-            if (g == 0) red[j] = out[j];
+        for (int k = 0; k < PARTS; ++k) {
+            if (part_of == k) {
+                if (k > 0) { const float4 c4 = *carry; s[0] = c4.x; s[1] = c4.y; s[2] = c4.z; s[3] = c4.w; }
+                add();
+                if (k + 1 < PARTS) *carry = make_float4(s[0], s[1], s[2], s[3]);
+            }
+            if (k + 1 < PARTS) __syncthreads();
+        }
+        if (part_of == PARTS - 1) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+#pragma unroll
+                for (int d = 1; d < 8; d <<= 1) s[j] += __shfl_xor_sync(0xffffffffu, s[j], d);
+                if (g == 0) red[j] = s[j];
+            }
         }
         __syncthreads();
 #pragma unroll
-        for (int j = 0; j < 4; ++j) out[j] = (fsm[4 * cg + j] + fsm[16 + 4 * cg + j]) + (fsm[32 + 4 * cg + j] + fsm[48 + 4 * cg + j]);
+        for (int j = 0; j < 4; ++j) s[j] = (fsm[4 * cg + j] + fsm[16 + 4 * cg + j]) + (fsm[32 + 4 * cg + j] + fsm[48 + 4 * cg + j]);
         __syncthreads();
     };
+    over_pixels([&] {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        s[j] = 0.f;
+        for (int j = 0; j < 4; ++j)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { val[i][j] = stored<T>(val[i][j]); if (valid[i]) s[j] += val[i][j]; }
-    }
-    over_pixels(s);
+            for (int i = 0; i < PP; ++i) { val[i][j] = stored<T>(val[i][j]); if (valid[i]) s[j] += val[i][j]; }
+    });
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        m[j] = s[j] / (float)cnt; s[j] = 0.f;
+    for (int j = 0; j < 4; ++j) m[j] = s[j] / (float)cnt;
+    over_pixels([&] {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) if (valid[i]) { const float d = val[i][j] - m[j]; s[j] = fmaf(d, d, s[j]); }
-    }
-    over_pixels(s);
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int i = 0; i < PP; ++i) if (valid[i]) { const float d = val[i][j] - m[j]; s[j] = fmaf(d, d, s[j]); }
+    });
     if (warp == 0 && g == 0) {
         const int tiles = gridDim.x, groups = gridDim.z;
         const size_t rec = (size_t)grp * tiles + blockIdx.x;
@@ -553,13 +573,23 @@ bool plan_fc(const ConvGeom& g, int groups, bool back, FcParams& p) {
     return one <= FC_SMEM_MAX;
 }
 
-template <typename T, int NQ, bool VEC>
-void launch_fc(const void* x, const void* w, const float* bias, void* y, float* stat, const FcParams& p, int groups, cudaStream_t s) {
+template <typename T, int NQ, bool VEC, int PP>
+void launch_fc_pp(const void* x, const void* w, const float* bias, void* y, float* stat, const FcParams& p, int groups, cudaStream_t s) {
     const size_t smem = (size_t)p.buffers * (p.x_floats + p.w_floats) * sizeof(float);
     static bool attr = false;
-    if (!attr) { cudaFuncSetAttribute(fc_kernel<T, NQ, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FC_SMEM_MAX); attr = true; }
+    if (!attr) { cudaFuncSetAttribute(fc_kernel<T, NQ, VEC, PP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FC_SMEM_MAX); attr = true; }
     const int tiles = p.tiles_w * p.tiles_h * ((p.ngroup + p.Nt - 1) / p.Nt);
-    klaunch(fc_kernel<T, NQ, VEC>, dim3(tiles, (p.Co + FC_CO - 1) / FC_CO, groups * p.ncls), FC_THREADS, smem, s, (const T*)x, (const T*)w, bias, (T*)y, stat, p);
+    klaunch(fc_kernel<T, NQ, VEC, PP>, dim3(tiles, (p.Co + FC_CO - 1) / FC_CO, groups * p.ncls), 512 / PP, smem, s, (const T*)x, (const T*)w, bias, (T*)y, stat, p);
+}
+// Two pixels a thread while all CTAs fit at two per SM: such launches leave each scheduler one to three warps of four pixels a thread, which wait for
+// shared memory (short scoreboard, ncu: 41 % of the issue slots used at 2.6 warps), and twice the warps pay for half as many FMAs per shared load.
+// ResNet-20 fp32, 2 x 7 samples, K = 2: 701 -> 584 us per step, 4 x 9, K = 1: 1364 -> 1080; with every launch that way, 4 x 48 goes from 2.70
+// to 2.88 ms.  One pixel a thread below 60 to 148 CTAs gave nothing (584 -> 626, 1075 -> 1125).  Both give the same bits.
+template <typename T, int NQ, bool VEC>
+void launch_fc(const void* x, const void* w, const float* bias, void* y, float* stat, const FcParams& p, int groups, cudaStream_t s) {
+    const long ctas = (long)p.tiles_w * p.tiles_h * ((p.ngroup + p.Nt - 1) / p.Nt) * ((p.Co + FC_CO - 1) / FC_CO) * groups * p.ncls;
+    if (ctas <= 2 * 148) launch_fc_pp<T, NQ, VEC, 2>(x, w, bias, y, stat, p, groups, s);
+    else launch_fc_pp<T, NQ, VEC, 4>(x, w, bias, y, stat, p, groups, s);
 }
 template <typename T>
 void dispatch_fc(const void* x, const void* w, const float* bias, void* y, float* stat, const FcParams& p, int groups, cudaStream_t s) {

@@ -43,6 +43,17 @@ def test_batch_sizes(orc, workers, batch):
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("batch", [74, 75])
+def test_pixels_per_thread(orc, dtype, batch):
+    """2 x 74 and 2 x 75 images of 8x8, 16 -> 64 channels: 296 CTAs of two pixels a thread, 300 of four."""
+    net = _net(((8, 8), 16, sy.CONV3X3, 64, 1), dtype, 2, batch, dtype == "fp32")
+    if dtype == "fp32":
+        run_parity(orc, net, 1, param_tol=1e-5, loss_tol=1e-5)
+    else:
+        run_parity(orc, net, 1, grad_tol=2e-2, loss_tol=1e-4)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
 def test_replicas_in_one_launch_equal_the_single_copy_path(dtype):
     """With P = (1/N) 1 1^T given explicitly every worker has its own weights and gradients; convolutions, batch-norm and linear layers run
     once for all of them.  Same weights as the single-copy path up to the rounding of another summation order, relative to what the
