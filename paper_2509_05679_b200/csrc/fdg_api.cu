@@ -180,31 +180,45 @@ fdg_status fail(fdg_ctx* c, fdg_status s, const char* fmt, ...) {
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Pinned staging memory and copy streams for reading parameters back, shared by the contexts of the process: allocated with the first
-// context, given back with the last.  One reader at a time (the lock); LANES x LANE_BYTES = 8 MB whatever the networks are.
+// Pinned staging memory and copy streams for reading parameters back, shared by the contexts of the process and given back with the last:
+// as many lanes as the largest network's parameters keep busy, at most LANES x LANE_BYTES = 8 MB, pinned in one piece.  Pinning is paid once, by
+// fdg_create (about 0.5 ms per lane); 256 KB lanes would halve that and slow every read (42 MB: 1.8 ms, 2.4 with 512 KB, 2.7 with 256 KB).
+// One reader at a time (the lock).
 struct HostReader {
     static constexpr int LANES = 8;
     static constexpr size_t LANE_BYTES = 1 << 20;
     std::mutex mu;
-    int users = 0, device = -1;
-    char* pinned = nullptr;
+    int users = 0, device = -1, lanes = 0;
+    char* pinned[LANES] = {};
     cudaStream_t stream[LANES] = {};
+    std::vector<char*> blocks;
     void acquire() {
         std::lock_guard<std::mutex> lk(mu);
-        if (users++ > 0) return;
-        cudaGetDevice(&device);
-        bool ok = cudaMallocHost((void**)&pinned, LANES * LANE_BYTES) == cudaSuccess;
-        for (int i = 0; ok && i < LANES; ++i) ok = cudaStreamCreateWithFlags(&stream[i], cudaStreamNonBlocking) == cudaSuccess;
-        if (!ok) { cudaGetLastError(); drop(); }            // plain copies then (see read_floats)
+        ++users;
+    }
+    // threads that this many bytes keep busy: one is worth starting from 2 MB of its own
+    static int wanted(size_t bytes) { return (int)std::min<size_t>(LANES, std::max<size_t>(1, bytes >> 21)); }
+    void reserve(size_t bytes) {
+        std::lock_guard<std::mutex> lk(mu);
+        int dev = -1;
+        cudaGetDevice(&dev);
+        if (lanes == 0) device = dev;
+        const int n = wanted(bytes);
+        if (dev != device || lanes >= n) return;                // another device: plain copies (see read_floats), as without any lane
+        char* block = nullptr;
+        if (cudaMallocHost((void**)&block, (n - lanes) * LANE_BYTES) != cudaSuccess) { cudaGetLastError(); return; }
+        blocks.push_back(block);
+        for (; lanes < n; ++lanes, block += LANE_BYTES) {
+            if (cudaStreamCreateWithFlags(&stream[lanes], cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); return; }
+            pinned[lanes] = block;
+        }
     }
     void release() {
         std::lock_guard<std::mutex> lk(mu);
-        if (--users == 0) drop();
-    }
-    void drop() {
-        for (cudaStream_t& s : stream) { if (s) cudaStreamDestroy(s); s = nullptr; }
-        if (pinned) cudaFreeHost(pinned);
-        pinned = nullptr;
+        if (--users > 0) return;
+        for (; lanes > 0; --lanes) cudaStreamDestroy(stream[lanes - 1]);
+        for (char* b : blocks) cudaFreeHost(b);
+        blocks.clear();
     }
 };
 HostReader g_reader;
@@ -223,7 +237,7 @@ cudaError_t read_floats(const std::vector<HostRead>& reads, int device, F piece)
     for (const HostRead& r : reads)
         for (size_t off = 0; off < r.n; off += chunk) jobs.push_back({r.src + off, off, std::min(chunk, r.n - off), r.tag});
     std::lock_guard<std::mutex> lk(g_reader.mu);
-    if (!g_reader.pinned || g_reader.device != device) {
+    if (!g_reader.lanes || g_reader.device != device) {
         std::vector<float> h(chunk);
         for (const Job& b : jobs) {
             cudaError_t e = cudaMemcpy(h.data(), b.src, b.cnt * sizeof(float), cudaMemcpyDeviceToHost);
@@ -235,7 +249,7 @@ cudaError_t read_floats(const std::vector<HostRead>& reads, int device, F piece)
     std::atomic<size_t> next{0};
     std::atomic<int> err{(int)cudaSuccess};
     auto work = [&](int lane) {
-        float* const buf = (float*)(g_reader.pinned + lane * HostReader::LANE_BYTES);
+        float* const buf = (float*)g_reader.pinned[lane];
         if (lane > 0) cudaSetDevice(device);
         for (size_t j; (j = next.fetch_add(1)) < jobs.size() && err.load() == (int)cudaSuccess;) {
             const Job& b = jobs[j];
@@ -245,8 +259,9 @@ cudaError_t read_floats(const std::vector<HostRead>& reads, int device, F piece)
             piece(b.tag, b.off, b.cnt, buf);
         }
     };
-    // a thread is worth starting from two chunks of its own
-    const int extra = (int)std::min<size_t>(HostReader::LANES - 1, jobs.size() / 2 > 0 ? jobs.size() / 2 - 1 : 0);
+    size_t total = 0;
+    for (const HostRead& r : reads) total += r.n * sizeof(float);
+    const int extra = std::min(g_reader.lanes, HostReader::wanted(total)) - 1;
     std::vector<std::thread> threads;
     try { for (int i = 1; i <= extra; ++i) threads.emplace_back(work, i); } catch (...) {}      // fewer threads then
     work(0);
@@ -1443,6 +1458,7 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
     for (int kk = 0; kk < K; ++kk) ctx->mod[kk].split = kk + 1 < K && !ctx->serial && work_us > 500.0;
     if (h * w * c != opt->num_classes) return bail(FDG_ERR_INVALID_ARG, "the last layer's width differs from num_classes");
     ctx->n_params = canon;
+    g_reader.reserve(canon * sizeof(float));
     ctx->label_depth = 2 * K;
 
     // ---- device memory
