@@ -885,7 +885,7 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
                 }
                 bn_backward(dt, T(o.in), T(o.out), gout, wsmall(c, m, version, o.gamma_off, rep), wsmall(c, m, version, o.beta_off, rep),
                             P.stats(o) + (size_t)wn.w0 * ti.c * 2, gin, o.acc_in, gres, o.acc_in2, mgrad + m.n_big + o.gamma_off,
-                            mgrad + m.n_big + o.beta_off, m.red, m.scratch, wn.nw, (long)c->B * ti.h * ti.w, ti.c, o.relu, o.has_res, acc_p, c->grid_sms, c->tc_err, s);
+                            mgrad + m.n_big + o.beta_off, m.red + o.red_off, m.scratch, wn.nw, (long)c->B * ti.h * ti.w, ti.c, o.relu, o.has_res, acc_p, c->grid_sms, c->tc_err, s);
                 profile_detail(nullptr);
                 break; }
             case OP_RELU: if (gin) relu_backward(dt, T(o.out), gout, gin, n_out, o.acc_in, s); break;

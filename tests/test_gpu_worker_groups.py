@@ -68,3 +68,12 @@ def test_bf16_grouped_run_equals_ungrouped_run_up_to_summation_order(groups):
     scale = np.sqrt(np.mean(g1.astype(np.float64) ** 2))
     assert np.max(np.abs(gg - g1)) <= 1e-3 * scale, "first full gradient differs by more than fp32 summation order"
     assert np.max(np.abs(pg - p1)) <= 1e-3 * np.max(np.abs(p1))
+
+
+def test_bf16_batch_norms_of_different_kernels_grouped(orc):
+    """A batch-norm of 48 channels that the one-launch kernels take (its workers' sums are added after the last group) in front of one of
+    192 channels over 4 MB that the general kernels take (no power of two; their sums are per group): each has sums of its own."""
+    layers = [(sy.CONV3X3, 3, 48, 1, 0), (sy.BATCHNORM, 48, 48, 1, 0), (sy.CONV3X3, 48, 192, 1, 0), (sy.BATCHNORM, 192, 192, 1, 0),
+              (sy.GLOBAL_AVGPOOL, 192, 192, 1, 0), (sy.LINEAR, 192, 10, 1, 1)]
+    net = sy.Net("bn-48-192", layers, [], 16, 16, 3, 10, 4, 11, 0.05, "bf16")
+    run_parity(orc, net, 1, grad_tol=2e-2, elem_tol=3e-2, pair_bn=True, loss_tol=1e-3, worker_groups=2)
