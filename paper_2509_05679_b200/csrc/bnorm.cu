@@ -238,7 +238,7 @@ struct BncArgs {
     const float* gamma; const float* beta;
     float* stats;                                // [worker][C][2] (mean, invstd)
     float* red;                                  // backward: [worker][C][2] (sum dy, sum dy xhat)
-    bf16* y; bf16* dres; int accum_dx, accum_dres;
+    bf16* y; bf16* dres; int accum_dx, accum_dres;   // backward: y = dx, or nullptr (not needed)
     int rpw, C, relu, mask_from_x;
 };
 constexpr int BNC_RANKS = 8;
@@ -395,15 +395,17 @@ __global__ void __launch_bounds__(BT) bnc_kernel(const BncArgs a) {
                 *(uint4*)(a.y + o) = pack(f);
             } else {
                 masked(xv[u], dv[u], ov[u], f, g);
+                if (a.y) {                           // none for the network's input
 #pragma unroll
-                for (int j = 0; j < 8; ++j) f[j] = fmaf(sc[j], g[j], fmaf(f[j], ka[j], kb[j]));
-                if (a.accum_dx) {
-                    float old[8];
-                    unpack(*(const uint4*)(a.y + o), old);
+                    for (int j = 0; j < 8; ++j) f[j] = fmaf(sc[j], g[j], fmaf(f[j], ka[j], kb[j]));
+                    if (a.accum_dx) {
+                        float old[8];
+                        unpack(*(const uint4*)(a.y + o), old);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) f[j] += old[j];
+                        for (int j = 0; j < 8; ++j) f[j] += old[j];
+                    }
+                    *(uint4*)(a.y + o) = pack(f);
                 }
-                *(uint4*)(a.y + o) = pack(f);
                 if (a.dres) {
                     if (a.accum_dres) {
                         float old[8];

@@ -619,9 +619,11 @@ __global__ void bn_bwd_apply_k(const T* __restrict__ x, const T* __restrict__ ou
     if (relu && !(ld(out + i) > 0.f)) dy = 0.f;
     float xh = (ld(x + i) - mean) * istd;
     float inv_n = 1.f / (float)rpw;
-    float v = gamma[c] * istd * (dy - red[so] * inv_n - xh * red[so + 1] * inv_n);
-    if (accum_dx) v += ld(dx + i);
-    st(dx + i, v);
+    if (dx) {
+        float v = gamma[c] * istd * (dy - red[so] * inv_n - xh * red[so + 1] * inv_n);
+        if (accum_dx) v += ld(dx + i);
+        st(dx + i, v);
+    }
     if (dres) { float r = dy; if (accum_dres) r += ld(dres + i); st(dres + i, r); }
 }
 
@@ -707,7 +709,7 @@ struct BnsArgs {
     const float* gamma; const float* beta; const float* stats; const bf16* res;
     float* part;                // modes 0, 1: partial sums [chunk][worker][C][2], written; mode 3: the same, read (gridDim.x chunks)
     float* dgamma; float* dbeta; int accum_params;   // mode 3: parameter gradients, written by one CTA
-    bf16* y;                    // mode 2: output; mode 3: dx
+    bf16* y;                    // mode 2: output; mode 3: dx, or nullptr (the network's input: not needed)
     bf16* dres;                 // mode 3: gradient of the residual input, or nullptr
     long rpw; int C; int relu; int mask_from_x; int accum_dx; int accum_dres;
     int reverse;                // walk the CTA's tiles from the last to the first: a kernel that re-reads what the kernel before it
@@ -864,15 +866,17 @@ __global__ void __launch_bounds__(BNV_THREADS, BNS_CTAS) bns_kernel(const BnsArg
 #pragma unroll
                     for (int j = 0; j < BP; ++j) { s1[j] = __fadd2_rn(s1[j], dv[j]); s2[j] = __ffma2_rn(dv[j], xv[j], s2[j]); }
                 } else {
-                    float2 t[BP];
+                    if (a.y) {
+                        float2 t[BP];
 #pragma unroll
-                    for (int j = 0; j < BP; ++j) t[j] = __ffma2_rn(sc[j], dv[j], __ffma2_rn(xv[j], ka[j], kb[j]));
-                    if (a.accum_dx) {
-                        float2 old[BP]; unpack8(*(const uint4*)(a.y + o), old);
+                        for (int j = 0; j < BP; ++j) t[j] = __ffma2_rn(sc[j], dv[j], __ffma2_rn(xv[j], ka[j], kb[j]));
+                        if (a.accum_dx) {
+                            float2 old[BP]; unpack8(*(const uint4*)(a.y + o), old);
 #pragma unroll
-                        for (int j = 0; j < BP; ++j) t[j] = __fadd2_rn(t[j], old[j]);
+                            for (int j = 0; j < BP; ++j) t[j] = __fadd2_rn(t[j], old[j]);
+                        }
+                        *(uint4*)(a.y + o) = pack8<false>(t);
                     }
-                    *(uint4*)(a.y + o) = pack8<false>(t);
                     if (a.dres) {
                         if (a.accum_dres) {
                             float2 old[BP]; unpack8(*(const uint4*)(a.dres + o), old);

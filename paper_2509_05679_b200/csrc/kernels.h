@@ -103,7 +103,7 @@ void bnf_forward(const float* x, const float* gamma, const float* beta, size_t p
 void bnf_backward(const float* x, const float* out, const float* dout, const float* gamma, const float* beta, size_t p_group, const float* stats, float* dx,
                   bool accum_dx, float* dres, bool accum_dres, float* dgamma, float* dbeta, size_t g_group, float* scratch, int nw, long rpw, int C, bool relu,
                   bool mask_from_x, bool accum_params, cudaStream_t st);
-// dy_eff = dout * (out > 0 if relu).  dx (+)= BN backward of dy_eff; dres (+)= dy_eff;
+// dy_eff = dout * (out > 0 if relu).  dx (+)= BN backward of dy_eff (dx == nullptr: not needed, in every backward of this file); dres (+)= dy_eff;
 // dgamma, dbeta (fp32) = sums over all workers.  red: fp32 [n_workers][C][2] scratch for (sum dy, sum dy xhat).
 void bn_backward(int dt, const void* x, const void* out, const void* dout, const float* gamma, const float* beta,
                  const float* stats, void* dx, bool accum_dx, void* dres_or_null, bool accum_dres, float* dgamma, float* dbeta,

@@ -61,3 +61,19 @@ def test_masks_taken_along_by_the_large_kernels(orc):
     run_parity(orc, net, 2, grad_tol=2e-2, noise_factor=3.0, loss_tol=1e-3, grid_sms=1)
     shape, layers = CONV["pool-gap"]
     run_parity(orc, sy.Net("pool-gap", layers, [], *shape, 10, 2, 9, 0.05, "bf16"), 1, grad_tol=2e-2, noise_factor=3.0, loss_tol=1e-3, grid_sms=1)
+
+
+# batch-norm as the network's first layer has no input gradient to write: general kernels (fp32; bf16 with 48 channels over 4 MB), one-launch
+# kernels, streamed kernels (64 channels, 4.2 MB), with a ReLU and with a residual, whose gradients are not needed either
+@pytest.mark.parametrize("dtype,c,workers,batch,size", [("fp32", 8, 2, 3, 8), ("bf16", 16, 2, 3, 8), ("bf16", 64, 2, 64, 16), ("bf16", 48, 2, 82, 16)])
+@pytest.mark.parametrize("residual", [False, True])
+def test_batch_norm_on_the_network_input(orc, dtype, c, workers, batch, size, residual):
+    first = [(sy.BATCHNORM, c, c, 1, 0)]
+    if residual:
+        first = [(sy.RES_BEGIN, c, c, 1, 0)] + first + [(sy.RES_ADD, c, c, 1, 0)]
+    layers = first + [(sy.CONV3X3, c, 8, 1, 1)] + _head(8)
+    net = sy.Net("bn-first", layers, [], size, size, c, 10, workers, batch, 0.05, dtype)
+    if dtype == "fp32":
+        run_parity(orc, net, 2, param_tol=1e-5, loss_tol=1e-5)
+    else:
+        run_parity(orc, net, 1, grad_tol=2e-2, elem_tol=3e-2, pair_bn=True, loss_tol=1e-3)
