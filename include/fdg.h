@@ -181,7 +181,8 @@ FDG_API fdg_status fdg_set_params_worker(fdg_ctx* ctx, int32_t worker, const flo
  *                (the library's streams do not synchronise with the caller's), and the buffer
  *                must stay valid and unchanged until the library has copied it into its own FIFO:
  *                that copy is enqueued on module 1's stream; fdg_wait_ingest() blocks until it
- *                is done.  The library does not keep the pointer.
+ *                is done.  The library does not keep the pointer.  Pinned host memory and another device's
+ *                memory work too; an address the device cannot read fails with FDG_ERR_INVALID_ARG.
  *   dev_labels : device, int32 [M].
  *   host_loss_or_null : if non-NULL the call waits until the last module has computed the loss
  *                of the batch it forwards in this iteration (tau = t-K+1; NaN while tau < 0) and

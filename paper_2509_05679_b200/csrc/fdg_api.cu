@@ -121,7 +121,7 @@ struct Module {
     cudaEvent_t wev, wdone;        // dy ready for the weight-gradient stream / its work of this iteration finished
     cudaEvent_t done[2], fdone;    // this module's iteration t has finished: done[t & 1]; its forward pass: fdone (not when the iteration ran as one graph)
     cudaEvent_t fork;              // opens the side streams inside a capture
-    StepGraph graph[3];            // the steady-state iteration of this module (module 1: [1] with inputs from host memory, no ingest kernel), or, `split`,
+    StepGraph graph[3];            // the steady-state iteration of this module (module 1: [1] with inputs that are copied in, no ingest kernel), or, `split`,
                                    // its forward pass; [2]: its backward pass and update
     bool split;
     bool fdone_valid, ran_direct;  // the last iteration recorded fdone / a full iteration was enqueued kernel by kernel before
@@ -1141,6 +1141,21 @@ fdg_status check_device_error(fdg_ctx* ctx) {
 // Where the batch of iteration t comes from when it already is in device memory (module 1 copies it into its FIFO slot).
 struct Ingest { const void* x; const int32_t* y; };
 
+// How a buffer that the caller passes as device memory can be read: by the ingest kernel (memory of this device, on the boundary of its words),
+// by a copy (other addresses the device knows: pinned host memory, another device, an odd start), or not at all (an address a kernel
+// would fault on).  Looked at on every step, first and last byte.
+enum Readable { BY_KERNEL, BY_COPY, NOT_READABLE };
+Readable readable(const fdg_ctx* ctx, const void* p, size_t bytes, size_t word) {
+    Readable how = (uintptr_t)p % word ? BY_COPY : BY_KERNEL;
+    for (const char* q : {(const char*)p, (const char*)p + bytes - 1}) {
+        cudaPointerAttributes a{};
+        if (cudaPointerGetAttributes(&a, q) != cudaSuccess) { cudaGetLastError(); return NOT_READABLE; }
+        if (a.type == cudaMemoryTypeUnregistered) return NOT_READABLE;
+        if (a.type == cudaMemoryTypeHost || (a.type == cudaMemoryTypeDevice && a.device != ctx->device)) how = BY_COPY;
+    }
+    return how;
+}
+
 // One iteration of module kk on its streams.  FORWARD: ingest (module 1), forward on tau_f.  BACKWARD: tags, loss, backward on tau_b, update.
 enum { FORWARD = 1, BACKWARD = 2, WHOLE = 3 };
 fdg_status module_step(fdg_ctx* ctx, int kk, int64_t t, const Ingest* in, int part) {
@@ -1269,6 +1284,14 @@ fdg_status run_step(fdg_ctx* ctx, const void* inputs, const int32_t* labels, boo
     if (!inputs || !labels) return fail(ctx, FDG_ERR_INVALID_ARG, "inputs and labels must not be NULL");
     if (!ctx->have_params) return fail(ctx, FDG_ERR_STATE, "fdg_set_params must be called before fdg_step");
     if (ctx->broken) return fail(ctx, FDG_ERR_STATE, "an earlier step failed after part of its work was enqueued; call fdg_set_params to start over");
+    const size_t x_bytes = (size_t)ctx->M * ctx->mod[0].in_elems * ctx->esz, y_bytes = (size_t)ctx->M * sizeof(int32_t);
+    bool by_copy = host_src;
+    if (!host_src) {
+        const Readable x = readable(ctx, inputs, x_bytes, 2), y = readable(ctx, labels, y_bytes, 4);
+        if (x == NOT_READABLE || y == NOT_READABLE)
+            return fail(ctx, FDG_ERR_INVALID_ARG, "%s must be device memory of %zu bytes", x == NOT_READABLE ? "inputs" : "labels", x == NOT_READABLE ? x_bytes : y_bytes);
+        by_copy = x == BY_COPY || y == BY_COPY;
+    }
     const int K = ctx->K;
     const int64_t t = ctx->t;
     const int now = (int)(t & 1), prev = now ^ 1;
@@ -1292,14 +1315,15 @@ fdg_status run_step(fdg_ctx* ctx, const void* inputs, const int32_t* labels, boo
             if (kk + 1 < K) CK(cudaStreamWaitEvent(m.stream, ctx->mod[kk + 1].done[prev], 0));
         }
     // 2. module 1 "samples" the batch of iteration t into its FIFO slot, the labels go into the label FIFO: from device memory by a
-    //    kernel of its own iteration, from host memory by copies on their own stream.  Those may run beside iteration t-1: the slots
+    //    kernel of its own iteration, from elsewhere by copies on their own stream.  Those may run beside iteration t-1: the slots
     //    they fill were last read in iteration t-3 (inputs; t-2 with K = 1) or before iteration t-2 of module 1 ended (labels).
     Ingest in{inputs, labels};
-    if (host_src) {
+    if (by_copy) {
         Module& m0 = ctx->mod[0];
+        const cudaMemcpyKind kind = host_src ? cudaMemcpyHostToDevice : cudaMemcpyDefault;
         if (t > 1) CK(cudaStreamWaitEvent(ctx->copy, m0.done[now], 0));                      // iteration t-2 (this iteration's record comes later)
-        CK(cudaMemcpyAsync(m0.in_ring + (size_t)(t % m0.in_depth) * m0.in_slot_bytes, inputs, (size_t)ctx->M * m0.in_elems * ctx->esz, cudaMemcpyHostToDevice, ctx->copy));
-        CK(cudaMemcpyAsync(ctx->labels + (size_t)(t % ctx->label_depth) * ctx->M, labels, (size_t)ctx->M * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->copy));
+        CK(cudaMemcpyAsync(m0.in_ring + (size_t)(t % m0.in_depth) * m0.in_slot_bytes, inputs, x_bytes, kind, ctx->copy));
+        CK(cudaMemcpyAsync(ctx->labels + (size_t)(t % ctx->label_depth) * ctx->M, labels, y_bytes, kind, ctx->copy));
         CK(cudaEventRecord(ctx->ingested, ctx->copy));
         CK(cudaStreamWaitEvent(as_graph(m0, 0) && !m0.split ? m0.stream : m0.fstream, ctx->ingested, 0));
         // the last module reads the labels: K - 1 iterations from now, ordered by the hand-offs; with one module in this iteration's forward pass
@@ -1307,7 +1331,7 @@ fdg_status run_step(fdg_ctx* ctx, const void* inputs, const int32_t* labels, boo
     // 3. every module: forward on tau_f, backward on tau_b, update
     for (int kk = 0; kk < K; ++kk) {
         Module& m = ctx->mod[kk];
-        const Ingest* const src = kk == 0 && !host_src ? &in : nullptr;
+        const Ingest* const src = kk == 0 && !by_copy ? &in : nullptr;
         bool ran = false, half = false;
         if (as_graph(m, kk)) {
             if (!m.split) ran = module_step_graph(ctx, kk, t, src, WHOLE);
@@ -1320,7 +1344,7 @@ fdg_status run_step(fdg_ctx* ctx, const void* inputs, const int32_t* labels, boo
             if (as_graph(m, kk) && !m.split) {
                 // the waits of a kernel-by-kernel iteration, which were not made above
                 if (!ctx->serial && t > 0) { const fdg_status st = wait_forward(kk); if (st != FDG_OK) return st; }
-                if (host_src && kk == 0) CK(cudaStreamWaitEvent(m.fstream, ctx->ingested, 0));
+                if (by_copy && kk == 0) CK(cudaStreamWaitEvent(m.fstream, ctx->ingested, 0));
             }
             const fdg_status st = module_step(ctx, kk, t, src, half ? BACKWARD : WHOLE);
             if (st != FDG_OK) return st;

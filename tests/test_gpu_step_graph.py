@@ -95,3 +95,38 @@ def test_two_contexts_interleaved():
     for c, a in zip(ctxs, alone):
         assert np.array_equal(c.params(), a)
         c.close()
+
+
+def test_inputs_that_the_ingest_kernel_cannot_read():
+    """fdg_step takes any address a copy can read: device buffers that start off the kernel's words and pinned host memory give the
+    same weights as aligned device buffers, in kernel-by-kernel iterations and in graphs.  Ordinary host memory is refused before anything is
+    enqueued, and the run goes on as if the call had not been made."""
+    import torch
+    from paper_2509_05679_b200 import binding
+    net = nets()["small"]
+    p0 = sy.init_params(net.layers, 0)
+    steps = 4 * net.K + 9
+    ref = _run(net, p0, steps, lambda t: "device")
+    ctx = make_ctx(net, p0)
+    xraw = torch.empty(net.M * 70 * 4 + 16, dtype=torch.uint8, device="cuda")
+    yraw = torch.empty(net.M * 4 + 16, dtype=torch.uint8, device="cuda")
+    for t in range(steps):
+        x, y = torch.from_numpy(sy.batch_inputs(net, t)), torch.from_numpy(sy.batch_labels(net, t))
+        if t % 4 == 0:
+            xd, yd = x.cuda(), y.cuda()
+        elif t % 4 == 3:
+            xd, yd = x.pin_memory(), y.pin_memory()
+        else:
+            off = (1, 2)[t % 2]
+            xd, yd = xraw[off:off + net.M * 70 * 4], yraw[off:off + net.M * 4]
+            xd.copy_(x.reshape(-1).view(torch.uint8)); yd.copy_(y.view(torch.uint8))
+        torch.cuda.synchronize()
+        if t in (0, 2, 20):
+            for bad in ((x.numpy(), yd), (xd, y.numpy()), (xd, 1)):
+                with pytest.raises(binding.FdgError) as e:
+                    ctx.step(*bad)
+                assert e.value.status == 1
+        ctx.step(xd, yd)
+        ctx.wait_ingest()
+    assert np.array_equal(ref[0], ctx.params())
+    ctx.close()
