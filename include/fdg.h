@@ -192,7 +192,9 @@ FDG_API fdg_status fdg_step(fdg_ctx* ctx, const void* dev_inputs, const int32_t*
                     float* host_loss_or_null);
 
 /* Same as fdg_step with HOST input buffers (pinned memory makes the copies asynchronous); the
- * host-to-device copies go straight into the FIFO slot, ordered on module 1's stream. */
+ * host-to-device copies go straight into the FIFO slot.  With fdg_options.streams (or serial = 1) they are
+ * ordered on module 1's stream, so work queued there before the call may still fill the buffers; with the
+ * context's own streams they may start at once, beside the previous iteration. */
 FDG_API fdg_status fdg_step_host(fdg_ctx* ctx, const void* host_inputs, const int32_t* host_labels,
                          float* host_loss_or_null);
 

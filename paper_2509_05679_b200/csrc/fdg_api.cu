@@ -164,7 +164,7 @@ struct fdg_ctx {
     bool graphs;                   // steady-state iterations run as graphs (off once recording one has failed)
     cudaEvent_t ingested;
     cudaStream_t cap;              // captures are recorded on it
-    cudaStream_t copy;             // host-to-device copies of the inputs
+    cudaStream_t copy;             // copies of the inputs that run ahead of module 1's stream
     std::string err;
 };
 
@@ -1315,16 +1315,19 @@ fdg_status run_step(fdg_ctx* ctx, const void* inputs, const int32_t* labels, boo
             if (kk + 1 < K) CK(cudaStreamWaitEvent(m.stream, ctx->mod[kk + 1].done[prev], 0));
         }
     // 2. module 1 "samples" the batch of iteration t into its FIFO slot, the labels go into the label FIFO: from device memory by a
-    //    kernel of its own iteration, from elsewhere by copies on their own stream.  Those may run beside iteration t-1: the slots
-    //    they fill were last read in iteration t-3 (inputs; t-2 with K = 1) or before iteration t-2 of module 1 ended (labels).
+    //    kernel of its own iteration, from elsewhere by copies.  With streams of the context's own the copies have one more, and may run beside
+    //    iteration t-1: the slots they fill were last read in iteration t-3 (inputs; t-2 with K = 1) or before iteration t-2 of module 1 ended
+    //    (labels).  The caller's streams, and serial mode: on module 1's stream, behind what the caller has queued there (it may fill the buffers).
     Ingest in{inputs, labels};
     if (by_copy) {
         Module& m0 = ctx->mod[0];
         const cudaMemcpyKind kind = host_src ? cudaMemcpyHostToDevice : cudaMemcpyDefault;
-        if (t > 1) CK(cudaStreamWaitEvent(ctx->copy, m0.done[now], 0));                      // iteration t-2 (this iteration's record comes later)
-        CK(cudaMemcpyAsync(m0.in_ring + (size_t)(t % m0.in_depth) * m0.in_slot_bytes, inputs, x_bytes, kind, ctx->copy));
-        CK(cudaMemcpyAsync(ctx->labels + (size_t)(t % ctx->label_depth) * ctx->M, labels, y_bytes, kind, ctx->copy));
-        CK(cudaEventRecord(ctx->ingested, ctx->copy));
+        const bool ahead = ctx->own_streams && !ctx->serial;
+        const cudaStream_t copy = ahead ? ctx->copy : m0.stream;
+        if (ahead && t > 1) CK(cudaStreamWaitEvent(copy, m0.done[now], 0));                  // iteration t-2 (this iteration's record comes later)
+        CK(cudaMemcpyAsync(m0.in_ring + (size_t)(t % m0.in_depth) * m0.in_slot_bytes, inputs, x_bytes, kind, copy));
+        CK(cudaMemcpyAsync(ctx->labels + (size_t)(t % ctx->label_depth) * ctx->M, labels, y_bytes, kind, copy));
+        CK(cudaEventRecord(ctx->ingested, copy));
         CK(cudaStreamWaitEvent(as_graph(m0, 0) && !m0.split ? m0.stream : m0.fstream, ctx->ingested, 0));
         // the last module reads the labels: K - 1 iterations from now, ordered by the hand-offs; with one module in this iteration's forward pass
     }

@@ -130,3 +130,31 @@ def test_inputs_that_the_ingest_kernel_cannot_read():
         ctx.wait_ingest()
     assert np.array_equal(ref[0], ctx.params())
     ctx.close()
+
+
+@pytest.mark.parametrize("serial", [True, False])
+@pytest.mark.parametrize("name", ["small", "large"])
+def test_host_buffers_filled_by_work_queued_on_the_callers_stream(name, serial):
+    """With the caller's streams the host copies are ordered on module 1's stream: a pinned buffer that work queued there is still
+    going to fill when fdg_step_host is called gives the weights of buffers that were complete."""
+    import torch
+    net = nets()[name]
+    p0 = sy.init_params(net.layers, 0, bf16=net.dtype == "bf16")
+    steps = 2 * net.K + 4
+    ref = _run(net, p0, steps, lambda t: "host", serial=serial)
+    dt = torch.bfloat16 if net.dtype == "bf16" else torch.float32
+    streams = [torch.cuda.Stream() for _ in range(net.K)]
+    ctx = make_ctx(net, p0, serial=serial, streams=[s.cuda_stream for s in streams])
+    xp = torch.zeros((net.M, net.in_h, net.in_w, net.in_c), dtype=dt).pin_memory()
+    yp = torch.zeros(net.M, dtype=torch.int32).pin_memory()
+    for t in range(steps):
+        xd, yd = torch.from_numpy(sy.batch_inputs(net, t)).to(dt).cuda(), torch.from_numpy(sy.batch_labels(net, t)).cuda()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(streams[0]):
+            torch.cuda._sleep(4_000_000)                    # about 2 ms
+            xp.copy_(xd, non_blocking=True)
+            yp.copy_(yd, non_blocking=True)
+        ctx.step_host(xp, yp)
+        ctx.wait_ingest()
+    assert np.array_equal(ref[0], ctx.params())
+    ctx.close()
