@@ -850,13 +850,15 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
                 if (o.masked_by && o.bias) colsum_records(m.bstat + o.col_off, mgrad + m.n_big + o.b_off, o.col_recs, g.Co, false, ws);
                 if (o.stem && tc_stem_wgrad(c, m, o, P.tensor(o.in), grad_ptr(c, kk, o.out, t), mgrad + o.w_off, wn, ws)) {}
                 else if (o.stem) stem_wgrad(T(o.in), gout, mgrad + o.w_off, m.ws, g, acc_p, ws);
-                else if (!(o.tc && tc_wgrad(c, m, o, P.tensor(o.in), grad_ptr(c, kk, o.out, t), mgrad + o.w_off, wn, ws)))
-                    fconv_wgrad(dt, T(o.in), gout, mgrad + o.w_off, m.ws, g, 1, 0, acc_p, ws);
+                else if (o.tc && tc_wgrad(c, m, o, P.tensor(o.in), grad_ptr(c, kk, o.out, t), mgrad + o.w_off, wn, ws)) {}
+                else if (linear_supported(g)) linear_backward(dt, T(o.in), nullptr, nullptr, gout, nullptr, false, mgrad + o.w_off, nullptr, g, 1, 0, 0, acc_p, ws);
+                else fconv_wgrad(dt, T(o.in), gout, mgrad + o.w_off, m.ws, g, 1, 0, acc_p, ws);
                 if (o.bias && !fused_rb && !o.masked_by) bias_grad(dt, gout, mgrad + m.n_big + o.b_off, m.scratch, orows, g.Co, acc_p, s);
                 if (gin && !(o.tc && tc_dgrad(c, m, o, grad_ptr(c, kk, o.out, t), grad_ptr(c, kk, o.in, t), version, o.acc_in,
                                                      below ? P.tensor(o.in) : nullptr, col, wn, s))) {
                     c->mask_lost = c->mask_lost || below;
-                    fconv_dgrad(dt, gout, wbig(c, m, version, o.w_off, rep), gin, g, o.acc_in ? EPI_ACCUM : 0, 1, 0, s);
+                    if (linear_supported(g)) linear_backward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), nullptr, gout, gin, o.acc_in, nullptr, nullptr, g, 1, 0, 0, false, s);
+                    else fconv_dgrad(dt, gout, wbig(c, m, version, o.w_off, rep), gin, g, o.acc_in ? EPI_ACCUM : 0, 1, 0, s);
                 }
                 profile_detail(nullptr);
                 break; }

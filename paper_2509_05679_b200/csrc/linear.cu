@@ -318,10 +318,10 @@ void linear_forward(int dt, const void* x, const void* w, const float* bias, voi
     else klaunch_cluster(lin_fwd_kernel<float>, dim3(tiles * a.split, groups), LT, 0, s, a.split, a);
 }
 
-void linear_backward(int dt, const void* x, const void* w, const void* y_or_null, const void* dy, void* dx_or_null, bool accum_dx, float* dw, float* db_or_null,
+void linear_backward(int dt, const void* x, const void* w, const void* y_or_null, const void* dy, void* dx_or_null, bool accum_dx, float* dw_or_null, float* db_or_null,
                      const ConvGeom& g, int groups, size_t w_group, size_t g_group, bool accum_p, cudaStream_t s) {
     LinArgs a{};
-    a.x = x; a.w = w; a.y = y_or_null; a.dy = dy; a.out = dx_or_null; a.dw = dw; a.db = db_or_null; a.M = g.N / groups; a.N = g.Co; a.K = g.C;
+    a.x = x; a.w = w; a.y = y_or_null; a.dy = dy; a.out = dx_or_null; a.dw = dw_or_null; a.db = db_or_null; a.M = g.N / groups; a.N = g.Co; a.K = g.C;
     a.w_group = w_group; a.g_group = g_group;
     a.epi = accum_dx ? EPI_ACCUM : 0; a.accum_p = accum_p;
     a.vec_k = g.C % 4 == 0 && w_group % 4 == 0 && aligned4(x, dt) && aligned4(w, dt);
@@ -331,7 +331,7 @@ void linear_backward(int dt, const void* x, const void* w, const void* y_or_null
     a.split = dx_tiles ? pick_split(dx_tiles * groups, a.N) : 1;
     a.dx_clusters = dx_tiles;
     a.dw_tiles_n = (a.K + LN - 1) / LN;
-    a.dw_tiles = ((a.N + LM - 1) / LM) * a.dw_tiles_n;
+    a.dw_tiles = dw_or_null ? ((a.N + LM - 1) / LM) * a.dw_tiles_n : 0;
     const int clusters = dx_tiles + (a.dw_tiles + a.split - 1) / a.split;
     const double esz = dt ? 2.0 : 4.0;
     Scope sc(KC_FMA_WGRAD, (dx_or_null ? 4.0 : 2.0) * g.N * a.N * a.K, esz * ((double)a.M * a.K * (dx_or_null ? 2 : 1) + (double)a.N * a.K + (double)a.M * a.N * (y_or_null ? 2 : 1)) + 4.0 * a.N * a.K, s);

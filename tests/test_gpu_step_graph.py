@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 from paper_2509_05679_b200 import synth as sy
-from harness import make_ctx
+from harness import grad_rel_l2, make_ctx
 
 pytestmark = pytest.mark.gpu
 
@@ -158,3 +158,33 @@ def test_host_buffers_filled_by_work_queued_on_the_callers_stream(name, serial):
         ctx.wait_ingest()
     assert np.array_equal(ref[0], ctx.params())
     ctx.close()
+
+
+def _failing_create():
+    """A context whose first large buffer (6 TB) no allocator has: fdg_create fails with FDG_ERR_OOM, through the library's own cudaMalloc."""
+    from paper_2509_05679_b200 import binding
+    with pytest.raises(binding.FdgError) as e:
+        binding.Context(sy.mlp_layers([1 << 18, 10]), [], 1, 1 << 22, 0.05, dtype="bf16", in_shape=(1, 1, 1 << 18), num_classes=10, use_torch_allocator=False)
+    assert e.value.status == 5
+
+
+@pytest.mark.parametrize("fail_at", [2, 5, 8])
+def test_a_failed_create_does_not_change_what_other_contexts_compute(fail_at):
+    """The CUDA runtime keeps the failed allocation's error for the thread.  The next step of another context on tensor-core linear layers, enqueued
+    kernel by kernel (the first with a backward pass) or as a graph, computes the gradients it would have computed without it."""
+    import torch
+    from paper_2509_05679_b200 import binding
+    net = sy.Net("mlp-tc", sy.mlp_layers([256, 256, 256, 10]), [2], 1, 1, 256, 10, 2, 96, 0.05, "bf16")
+    p0 = sy.init_params(net.layers, 0, bf16=True)
+    steps = fail_at + 1
+    ref = _run(net, p0, steps, lambda t: "device")
+    ctx = make_ctx(net, p0)
+    for t in range(steps):
+        if t == fail_at:
+            _failing_create()
+        x, y = binding.to_device("bf16", sy.batch_inputs(net, t)), torch.from_numpy(sy.batch_labels(net, t)).cuda()
+        ctx.step(x, y)
+        ctx.wait_ingest()
+    err, where, _ = grad_rel_l2(ctx.grads(), ref[1], net.layers)
+    ctx.close()
+    assert err <= 2e-2, (err, where)
