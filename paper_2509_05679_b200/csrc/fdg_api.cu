@@ -176,7 +176,9 @@ fdg_status fail(fdg_ctx* c, fdg_status s, const char* fmt, ...) {
     if (c) c->err = buf; else g_create_error = buf;
     return s;
 }
-#define CK(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) return fail(ctx, FDG_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e_)); } while (0)
+// The runtime also keeps an error for the thread until someone asks for it: asked for here, and wherever else a failure is dealt with, so
+// that it is not found after a later call and taken for that one's.
+#define CK(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) { cudaGetLastError(); return fail(ctx, FDG_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e_)); } } while (0)
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -269,7 +271,12 @@ cudaError_t read_floats(const std::vector<HostRead>& reads, int device, F piece)
     return (cudaError_t)err.load();
 }
 
-void* default_alloc(size_t bytes, void*) { void* p = nullptr; return cudaMalloc(&p, bytes) == cudaSuccess ? p : nullptr; }
+void* default_alloc(size_t bytes, void*) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+    cudaGetLastError();
+    return nullptr;
+}
 void default_free(void* p, void*) { cudaFree(p); }
 
 // ---- compile layers [p,q) into ops; returns "" or an error text
@@ -546,6 +553,9 @@ Win group_window(const fdg_ctx* c, const Module& m, int g) {
     return Win{g * nw * c->B, nw * c->B, g * nw, nw, g == 0};
 }
 
+// A launch that was refused is made up for by other kernels: its error is not kept.
+bool launched(cudaError_t e) { if (e != cudaSuccess) cudaGetLastError(); return e == cudaSuccess; }
+
 bool tc_forward(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* y_base, int64_t version, const Win& wn, cudaStream_t s) {
     int ia = find_buf(o.a_ptrs, x_base);
     if (ia < 0) return false;
@@ -560,7 +570,7 @@ bool tc_forward(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* y_base, 
     const int io = find_buf(o.y_ptrs, y_base);
     const tc::KmMaps maps{&o.fa[ia], o.far.empty() ? nullptr : &o.far[ia], &o.fb[version % m.D], o.fbh.empty() ? nullptr : &o.fbh[version % m.D],
                           io >= 0 ? &o.fo[io] : nullptr};
-    const bool ok = (o.small_f ? tc::run_small(*maps.a, *maps.b, p, o.split_f, s) : tc::run_km(maps, p, o.n_tile_f, s)) == cudaSuccess;
+    const bool ok = launched(o.small_f ? tc::run_small(*maps.a, *maps.b, p, o.split_f, s) : tc::run_km(maps, p, o.n_tile_f, s));
     if (ok && o.stat_chunks) { m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.stat_chunks; }
     return ok;
 }
@@ -582,7 +592,7 @@ bool tc_dgrad(fdg_ctx* c, Module& m, const Op& o, char* dy_base, char* dx_base, 
     const int io = find_buf(o.dx_ptrs, dx_base);
     const tc::KmMaps maps{&o.da[ia], o.dar.empty() ? nullptr : &o.dar[ia], &o.db[version % m.D], o.dbh.empty() ? nullptr : &o.dbh[version % m.D],
                           io >= 0 ? &o.dox[io] : nullptr};
-    return (o.small_d ? tc::run_small(*maps.a, *maps.b, p, o.split_d, s) : tc::run_km(maps, p, o.n_tile_d, s)) == cudaSuccess;
+    return launched(o.small_d ? tc::run_small(*maps.a, *maps.b, p, o.split_d, s) : tc::run_km(maps, p, o.n_tile_d, s));
 }
 bool tc_wgrad(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* dy_base, float* dw, const Win& wn, cudaStream_t s) {
     int ix = find_buf(o.a_ptrs, x_base), id = find_buf(o.dy_ptrs, dy_base);
@@ -595,7 +605,7 @@ bool tc_wgrad(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* dy_base, f
         const int splits = o.wgr_splits < steps ? o.wgr_splits : (int)steps;
         double rows = (double)wn.n * g.Ho * g.Wo, R = (double)g.R * g.R * g.C;
         Scope sc(KC_TC_WGRAD, 2.0 * rows * g.Co * R, 2.0 * ((double)wn.n * g.H * g.W * g.C + rows * g.Co) + 4.0 * R * g.Co, s);
-        return tc::run_wg_rows(o.wxr[ix], o.da[id], q, o.wgr_variant, splits, dw, !wn.first, s) == cudaSuccess;
+        return launched(tc::run_wg_rows(o.wxr[ix], o.da[id], q, o.wgr_variant, splits, dw, !wn.first, s));
     }
     tc::WgParams p = o.kw;
     p.partial = m.ws; p.err = c->tc_err;
@@ -606,7 +616,7 @@ bool tc_wgrad(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* dy_base, f
     splits = (p.ptiles + p.ptiles_per_split - 1) / p.ptiles_per_split;
     double rows = (double)wn.n * g.Ho * g.Wo, R = (double)g.R * g.R * g.C;
     Scope sc(KC_TC_WGRAD, 2.0 * rows * g.Co * R, 2.0 * ((double)wn.n * g.H * g.W * g.C + rows * g.Co) + 4.0 * R * g.Co, s);
-    return tc::run_wg(o.wx[ix], o.wdy[id], p, o.n_tile_w, splits, dw, !wn.first, s) == cudaSuccess;
+    return launched(tc::run_wg(o.wx[ix], o.wdy[id], p, o.n_tile_w, splits, dw, !wn.first, s));
 }
 
 // first-layer forward on the tensor cores (whole batch only)
@@ -617,8 +627,8 @@ bool tc_stem_forward(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* y_b
     const ConvGeom& g = o.g;
     const double pix = (double)g.N * g.H * g.W;
     Scope sc(KC_FMA_FWD, 2.0 * pix * g.Co * 9 * g.C, 2.0 * pix * (g.C + g.Co), s);
-    const bool ok = tc::run_stem_fw(o.sxr[ix], o.fo[io], g.H, g.W, g.N, g.Co, wbig(c, m, version, o.w_off), o.bias ? wsmall(c, m, version, o.b_off) : nullptr,
-                                    o.relu, o.stat_chunks ? m.cstat[o.stat_buf] : nullptr, c->tc_err, c->grid_sms, s) == cudaSuccess;
+    const bool ok = launched(tc::run_stem_fw(o.sxr[ix], o.fo[io], g.H, g.W, g.N, g.Co, wbig(c, m, version, o.w_off), o.bias ? wsmall(c, m, version, o.b_off) : nullptr,
+                                    o.relu, o.stat_chunks ? m.cstat[o.stat_buf] : nullptr, c->tc_err, c->grid_sms, s));
     if (ok && o.stat_chunks) { m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.stat_chunks; }
     return ok;
 }
@@ -631,7 +641,7 @@ bool tc_stem_wgrad(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* dy_ba
     const ConvGeom& g = o.g;
     const double pix = (double)g.N * g.H * g.W;
     Scope sc(KC_FMA_WGRAD, 2.0 * pix * g.Co * 9 * g.C, 2.0 * pix * (g.C + g.Co), s);
-    return tc::run_stem_wg(o.sxr[ix], o.sdy[id], g.H, g.W, g.N, g.Co, m.ws, dw, false, c->tc_err, c->grid_sms, s) == cudaSuccess;
+    return launched(tc::run_stem_wg(o.sxr[ix], o.sdy[id], g.H, g.W, g.N, g.Co, m.ws, dw, false, c->tc_err, c->grid_sms, s));
 }
 
 // byte offset of the group's first sample inside a tensor of the module
@@ -1259,7 +1269,7 @@ bool module_step_graph(fdg_ctx* ctx, int kk, int64_t t, const Ingest* in, int pa
         const bool ok = module_step(ctx, kk, t, in, part) == FDG_OK;
         if (!graph.end_update() || !ok) return false;
     }
-    return graph.launch(part == FORWARD ? m.fstream : m.stream) == cudaSuccess;
+    return launched(graph.launch(part == FORWARD ? m.fstream : m.stream));
 }
 
 // Waits until the step numbered `seq` has published its loss.
@@ -1412,7 +1422,7 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0) { cudaGetLastError(); return fail(nullptr, FDG_ERR_ARCH, "no CUDA device"); }
     int dev = 0; cudaDeviceProp prop;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return fail(nullptr, FDG_ERR_CUDA, "cannot query the device");
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess) { cudaGetLastError(); return fail(nullptr, FDG_ERR_CUDA, "cannot query the device"); }
     if (prop.major != 10) return fail(nullptr, FDG_ERR_ARCH, "device is sm_%d%d; this library is built for sm_100a only", prop.major, prop.minor);
 
     ctx = new fdg_ctx();
@@ -1449,7 +1459,7 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
     ctx->device = dev;
     ctx->mod.resize(K);
     g_reader.acquire();                    // released by fdg_destroy, which every error path below goes through
-    auto bail = [&](fdg_status s, const std::string& msg) { g_create_error = msg; fdg_destroy(ctx); return s; };
+    auto bail = [&](fdg_status s, const std::string& msg) { g_create_error = msg; fdg_destroy(ctx); cudaGetLastError(); return s; };
 
     int h = opt->in_h, w = opt->in_w, c = opt->in_c;
     size_t canon = 0;

@@ -1579,8 +1579,7 @@ cudaError_t run_update_module(const UpdTable& tb, float* master, const float* gr
     for (int j = 0; j < tb.nranges; ++j) plain4 += tb.ranges[j].count / 4;
     const unsigned blocks = (unsigned)(tb.total_tiles + (plain4 + 255) / 256);
     if (!blocks) return cudaSuccess;
-    klaunch(update_module_kernel, blocks, dim3(32, 8), 0, s, tb, master, grad, (bf16*)wcopy, (bf16*)wtcopy, small_copy, lr, has_grad ? 1 : 0, stamp);
-    return cudaGetLastError();
+    return klaunch(update_module_kernel, blocks, dim3(32, 8), 0, s, tb, master, grad, (bf16*)wcopy, (bf16*)wtcopy, small_copy, lr, has_grad ? 1 : 0, stamp);
 }
 
 // Wt[ci][R*R-1-tap][co] = W[co][tap][ci]: the weights of the transposed convolution, K-major for km_kernel.
@@ -1678,8 +1677,7 @@ static cudaError_t launch_km(const TensorMap& a, const TensorMap& b, const Tenso
     const int total = p.tiles_w * p.tiles_h * p.tiles_n * (p.Cn / N_TILE) * p.ncls;
     const int slots = sm_count(p.sms) * per_sm;
     const int grid = total < slots ? total : slots;
-    klaunch(kernel, grid, 64 + 32 * EPI_WARPS, smem, s, *(const CUtensorMap*)&a, *(const CUtensorMap*)&b, *(const CUtensorMap*)&o, p);
-    return cudaGetLastError();
+    return klaunch(kernel, grid, 64 + 32 * EPI_WARPS, smem, s, *(const CUtensorMap*)&a, *(const CUtensorMap*)&b, *(const CUtensorMap*)&o, p);
 }
 
 // CTA pairs: `b` is a tensor map whose box holds N_TILE / 2 weight rows.
@@ -1785,8 +1783,7 @@ static cudaError_t launch_wg(const TensorMap& x, const TensorMap& dy, const WgPa
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    klaunch(wg_kernel<N_TILE, STAGES>, grid, NUM_THREADS, smem, s, *(const CUtensorMap*)&x, *(const CUtensorMap*)&dy, p);
-    return cudaGetLastError();
+    return klaunch(wg_kernel<N_TILE, STAGES>, grid, NUM_THREADS, smem, s, *(const CUtensorMap*)&x, *(const CUtensorMap*)&dy, p);
 }
 
 cudaError_t run_wg(const TensorMap& x, const TensorMap& dy, const WgParams& p_in, int n_tile, int splits, float* dw, bool accum, cudaStream_t s) {
@@ -1812,8 +1809,7 @@ static cudaError_t launch_wg2(const TensorMap& x, const TensorMap& dy, const Wg2
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    klaunch(wg2_kernel<N_TILE, NX, XSUB_KB, STAGES>, grid, NUM_THREADS, smem, s, *(const CUtensorMap*)&x, *(const CUtensorMap*)&dy, p);
-    return cudaGetLastError();
+    return klaunch(wg2_kernel<N_TILE, NX, XSUB_KB, STAGES>, grid, NUM_THREADS, smem, s, *(const CUtensorMap*)&x, *(const CUtensorMap*)&dy, p);
 }
 
 int wg_rows_variant(int H, int W, int C, int Co) {
@@ -1881,11 +1877,9 @@ cudaError_t run_stem_wg(const TensorMap& x_raw, const TensorMap& dy128, int H, i
     const int ctas = stem_wg_ctas(p.steps, sms);
     p.steps_per_cta = (p.steps + ctas - 1) / ctas;
     p.partial = partial; p.err = err;
-    klaunch(stem_wg_kernel<STAGES>, dim3(ctas, Co / 64), NUM_THREADS, smem, s, *(const CUtensorMap*)&x_raw, *(const CUtensorMap*)&dy128, p);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = klaunch(stem_wg_kernel<STAGES>, dim3(ctas, Co / 64), NUM_THREADS, smem, s, *(const CUtensorMap*)&x_raw, *(const CUtensorMap*)&dy128, p);
     if (e != cudaSuccess) return e;
-    klaunch(stem_wg_reduce_kernel, (Co * 27 + 127) / 128, 128, 0, s, partial, dw, ctas, Co, accum);
-    return cudaGetLastError();
+    return klaunch(stem_wg_reduce_kernel, (Co * 27 + 127) / 128, 128, 0, s, partial, dw, ctas, Co, accum);
 }
 
 cudaError_t run_stem_fw(const TensorMap& x_raw, const TensorMap& out_map, int H, int W, int N, int Co, const void* w, const float* bias, bool relu,
@@ -1902,14 +1896,12 @@ cudaError_t run_stem_fw(const TensorMap& x_raw, const TensorMap& out_map, int H,
     p.W = W; p.Ht = 128 / W; p.tiles_h = H / p.Ht; p.tiles = N * p.tiles_h; p.Co = Co; p.epi = relu ? EPI_RELU : 0;
     p.w = (const bf16*)w; p.bias = bias; p.stat_part = stat_part; p.err = err;
     const int slots = 2 * sm_count(sms);
-    klaunch(stem_fw_kernel<STAGES>, dim3(p.tiles < slots ? p.tiles : slots, Co / 64), 320, smem, s, *(const CUtensorMap*)&x_raw, *(const CUtensorMap*)&out_map, p);
-    return cudaGetLastError();
+    return klaunch(stem_fw_kernel<STAGES>, dim3(p.tiles < slots ? p.tiles : slots, Co / 64), 320, smem, s, *(const CUtensorMap*)&x_raw, *(const CUtensorMap*)&out_map, p);
 }
 
 cudaError_t run_flip_transpose(const void* w, void* wt, int Co, int taps, int Ci, cudaStream_t s) {
     dim3 grid(Ci / 32, Co / 32, taps), blk(32, 8);
-    klaunch(flip_transpose_kernel, grid, blk, 0, s, (const bf16*)w, (bf16*)wt, Co, taps, Ci);
-    return cudaGetLastError();
+    return klaunch(flip_transpose_kernel, grid, blk, 0, s, (const bf16*)w, (bf16*)wt, Co, taps, Ci);
 }
 
 }  // namespace tc

@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 from paper_2509_05679_b200 import synth as sy
-from harness import grad_rel_l2, make_ctx
+from harness import make_ctx
 
 pytestmark = pytest.mark.gpu
 
@@ -185,6 +185,5 @@ def test_a_failed_create_does_not_change_what_other_contexts_compute(fail_at):
         x, y = binding.to_device("bf16", sy.batch_inputs(net, t)), torch.from_numpy(sy.batch_labels(net, t)).cuda()
         ctx.step(x, y)
         ctx.wait_ingest()
-    err, where, _ = grad_rel_l2(ctx.grads(), ref[1], net.layers)
+    assert np.array_equal(ctx.grads(), ref[1]) and np.array_equal(ctx.params(), ref[0])
     ctx.close()
-    assert err <= 2e-2, (err, where)
