@@ -159,7 +159,7 @@ struct fdg_ctx {
     LossRecord* loss_ring;         // pinned host memory, 64 records
     int64_t* tags;
     int* tc_err;                   // device word: set by a tensor-core kernel whose bounded wait gave up
-    bool mask_lost = false;        // a launch that had to apply a ReLU mask was refused: the kernels that could replace it do not apply it
+    bool mask_lost;                // during a module's backward pass: a launch that had to apply a ReLU mask was refused (the kernels that could replace it do not apply it)
     bool any_tc;
     bool graphs;                   // steady-state iterations run as graphs (off once recording one has failed)
     cudaEvent_t ingested;
@@ -1220,7 +1220,11 @@ fdg_status module_step(fdg_ctx* ctx, int kk, int64_t t, const Ingest* in, int pa
         else if (!fused_head) softmax_ce(ctx->dt, ctx->logits, ctx->labels + (size_t)(tau_f % ctx->label_depth) * ctx->M, ctx->dlogits, rec, ctx->tc_err, t + 1,
                                          ctx->M, ctx->classes, ctx->R > 1 ? 1.f / (float)ctx->B : 1.f / (float)ctx->M, m.stream);
     }
-    if (tau_b >= 0) backward_module(ctx, kk, tau_b, v_b, t);
+    if (tau_b >= 0) {
+        ctx->mask_lost = false;
+        backward_module(ctx, kk, tau_b, v_b, t);
+        if (ctx->mask_lost) return fail(ctx, FDG_ERR_CUDA, "an input-gradient kernel could not be launched");
+    }
     // Eq. dl_update with P = 11^T/N: w(t+1) = w(t) - lr * averaged gradient; also emits version t+1
     // (after the forward pass has read version t: with a one-slot ring the update overwrites it)
     if (part == WHOLE && !lastm && m.fstream != m.stream) CK(step_wait(m.stream, m.fdone));
@@ -1370,7 +1374,6 @@ fdg_status run_step(fdg_ctx* ctx, const void* inputs, const int32_t* labels, boo
         CK(cudaEventRecord(m.done[now], m.stream));
     }
     CK(cudaGetLastError());
-    if (ctx->mask_lost) return fail(ctx, FDG_ERR_CUDA, "an input-gradient kernel could not be launched");
     ctx->t = t + 1;
     if (host_loss) {
         float l = 0.f;                                  // the loss only: the last module's backward pass and update go on
