@@ -251,8 +251,8 @@ FDG_API fdg_status fdg_set_lr(fdg_ctx* ctx, float lr);
 /* Bytes of device memory the context holds, and how many kernels it has launched so far. */
 FDG_API fdg_status fdg_stats(const fdg_ctx* ctx, size_t* device_bytes, uint64_t* kernel_launches);
 
-/* Device time of the last completed step of every module (ms, between time stamps that its first and its
- * last kernel take on the device; array of K floats) -- waits for the modules. */
+/* Device time of the last completed step of every module (ms, from where its first kernel may start, all that it
+ * waits for being done, to the end of its last; array of K floats) -- waits for the modules. */
 FDG_API fdg_status fdg_module_times(fdg_ctx* ctx, float* ms, int32_t K);
 
 /* Per-kernel-class device timing for measurements.  fdg_profile(ctx, 1) clears the statistics and

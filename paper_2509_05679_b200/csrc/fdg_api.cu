@@ -125,7 +125,8 @@ struct Module {
                                    // its forward pass; [2]: its backward pass and update
     bool split;
     bool fdone_valid, ran_direct;  // the last iteration recorded fdone / a full iteration was enqueued kernel by kernel before
-    long long* stamps;             // device: start and end of the last iteration, ns
+    long long* stamps;             // device: start and end of the last iteration, ns (not of a `split` module)
+    cudaEvent_t ev_f, ev_b, ev_end;// `split`: the iteration's beginning on either stream, its end
     float* scratch_f;              // reduction scratch of the forward stream
     float* head_scratch;           // classifier head: weight-gradient partials, then loss partials
     size_t head_elems, head_part_elems;
@@ -1230,7 +1231,8 @@ fdg_status module_step(fdg_ctx* ctx, int kk, int64_t t, const Ingest* in, int pa
     if (part == WHOLE && !lastm && m.fstream != m.stream) CK(step_wait(m.stream, m.fdone));
     if (tau_b >= 0 && m.wstream != m.stream) { CK(step_record(m.wdone, m.wstream)); CK(step_wait(m.stream, m.wdone)); }
     long long* const end = m.stamps + 1;
-    if (ctx->R > 1) {
+    if (!npar(m)) stamp_time(end, m.stream);                // nothing to update (a module of poolings and ReLUs)
+    else if (ctx->R > 1) {
         // Eq. dl_update (a), (b) with a general P: u_r = w_r - lr g_r, w_s(t+1) = sum_r P_sr u_r, all replicas in one pass
         mix_update(ctx->dt, m.master, tau_b >= 0 ? m.grad : nullptr, wslot(ctx, m, t + 1, 0), m.n_big, m.n_small, m.wslot_bytes, ctx->R, ctx->P_dev,
                    ctx->lr, end, m.stream);
@@ -1238,11 +1240,13 @@ fdg_status module_step(fdg_ctx* ctx, int kk, int64_t t, const Ingest* in, int pa
         Scope sc(KC_SGD, 0.0, (double)npar(m) * (tau_b >= 0 ? 12.0 : 4.0) + 2.0 * m.n_big + 4.0 * m.n_small + 2.0 * m.n_big, m.stream);
         CK(tc::run_update_module(m.upd, m.master, m.grad, wslot(ctx, m, t + 1), wtslot(m, t + 1, 0), wsmall(ctx, m, t + 1, 0), ctx->lr, tau_b >= 0, end, m.stream));
     } else {
-        sgd_update(ctx->dt, m.master, tau_b >= 0 ? m.grad : nullptr, wslot(ctx, m, t + 1), m.n_big, ctx->lr, end, m.stream);
+        // the last launch takes the time
+        sgd_update(ctx->dt, m.master, tau_b >= 0 ? m.grad : nullptr, wslot(ctx, m, t + 1), m.n_big, ctx->lr, nullptr, m.stream);
+        emit_transposed_weights(ctx, m, t + 1);
         if (m.n_small)
             sgd_update(0, m.master + m.n_big, tau_b >= 0 ? m.grad + m.n_big : nullptr,
                        wsmall(ctx, m, t + 1, 0), m.n_small, ctx->lr, end, m.stream);
-        emit_transposed_weights(ctx, m, t + 1);
+        else stamp_time(end, m.stream);
     }
     m.had_bwd = tau_b >= 0;
     return FDG_OK;
@@ -1352,6 +1356,7 @@ fdg_status run_step(fdg_ctx* ctx, const void* inputs, const int32_t* labels, boo
         Module& m = ctx->mod[kk];
         const Ingest* const src = kk == 0 && !by_copy ? &in : nullptr;
         bool ran = false, half = false;
+        if (m.split) { CK(cudaEventRecord(m.ev_f, m.fstream)); CK(cudaEventRecord(m.ev_b, m.stream)); }
         if (as_graph(m, kk)) {
             if (!m.split) ran = module_step_graph(ctx, kk, t, src, WHOLE);
             else if ((half = module_step_graph(ctx, kk, t, src, FORWARD))) {
@@ -1370,6 +1375,7 @@ fdg_status run_step(fdg_ctx* ctx, const void* inputs, const int32_t* labels, boo
             if (t - kk >= 0 && m.had_bwd) m.ran_direct = true;
         }
         if (half) CK(cudaStreamWaitEvent(m.stream, m.fdone, 0));        // `done` covers the forward pass too
+        if (m.split) CK(cudaEventRecord(m.ev_end, m.stream));
         m.fdone_valid = !ran || half;
         CK(cudaEventRecord(m.done[now], m.stream));
     }
@@ -1397,6 +1403,7 @@ void fdg_destroy(fdg_ctx* ctx) {
     for (Module& m : ctx->mod) {
         for (cudaEvent_t e : m.done) if (e) cudaEventDestroy(e);
         if (m.fork) cudaEventDestroy(m.fork);
+        for (cudaEvent_t e : {m.ev_f, m.ev_b, m.ev_end}) if (e) cudaEventDestroy(e);
         for (StepGraph& g : m.graph) g.clear();
         if (m.fdone) cudaEventDestroy(m.fdone);
         if (m.wev) cudaEventDestroy(m.wev);
@@ -1566,6 +1573,7 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
         for (cudaEvent_t& d : m.done) if (e == cudaSuccess) e = cudaEventCreateWithFlags(&d, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.fork, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.fdone, cudaEventDisableTiming);
+        for (cudaEvent_t* v : {&m.ev_f, &m.ev_b, &m.ev_end}) if (m.split && e == cudaSuccess) e = cudaEventCreate(v);
         if (e == cudaSuccess) e = cudaMemset(m.grad, 0, (size_t)ctx->R * (m.n_big + m.n_small) * sizeof(float));
         if (e == cudaSuccess) e = cudaMemset(m.master, 0, (size_t)ctx->R * (m.n_big + m.n_small) * sizeof(float));
         if (e != cudaSuccess) return bail(FDG_ERR_CUDA, cudaGetErrorString(e));
@@ -1919,8 +1927,16 @@ fdg_status fdg_module_times(fdg_ctx* ctx, float* ms, int32_t K) {
     if (ctx->t == 0) return fail(ctx, FDG_ERR_STATE, "no step has run yet");
     CK(cudaDeviceSynchronize());
     for (int kk = 0; kk < K; ++kk) {
+        const Module& m = ctx->mod[kk];
+        if (m.split) {
+            float f = 0.f, b = 0.f;
+            CK(cudaEventElapsedTime(&f, m.ev_f, m.ev_end));
+            CK(cudaEventElapsedTime(&b, m.ev_b, m.ev_end));
+            ms[kk] = std::max(f, b);
+            continue;
+        }
         long long st[2];
-        CK(cudaMemcpy(st, ctx->mod[kk].stamps, sizeof st, cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy(st, m.stamps, sizeof st, cudaMemcpyDeviceToHost));
         ms[kk] = (float)((double)(st[1] - st[0]) * 1e-6);
     }
     return FDG_OK;

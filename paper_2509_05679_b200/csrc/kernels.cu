@@ -1085,6 +1085,11 @@ __device__ __forceinline__ void publish_loss(LossRecord* rec, float loss, const 
     __threadfence_system();
     r->seq = seq;
 }
+__global__ void stamp_k(long long* stamp) { *stamp = device_time_ns(); }
+void stamp_time(long long* stamp, cudaStream_t s) {
+    Scope sc(KC_FILL, 0.0, 8.0, s);
+    klaunch(stamp_k, 1, 1, 0, s, stamp);
+}
 __global__ void publish_k(LossRecord* rec, float loss, const int* err, long long seq) { publish_loss(rec, loss, err, seq); }
 void publish_loss_value(LossRecord* rec, float loss, const int* err, long long seq, cudaStream_t s) {
     Scope sc(KC_FILL, 0.0, sizeof(LossRecord), s);

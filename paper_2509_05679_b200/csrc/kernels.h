@@ -156,6 +156,7 @@ struct TagOps {
 };
 void tags_step(const TagOps& ops, cudaStream_t st);
 
+void stamp_time(long long* stamp, cudaStream_t st);              // the device's time in ns
 void zero_fill(void* p, size_t bytes, cudaStream_t st);          // p and bytes multiples of 16
 // x_bytes of a batch and its m labels into their FIFO slots
 void ingest(const void* x, void* x_slot, size_t x_bytes, const int32_t* y, int32_t* y_slot, int m, cudaStream_t st);

@@ -187,3 +187,28 @@ def test_a_failed_create_does_not_change_what_other_contexts_compute(fail_at):
         ctx.wait_ingest()
     assert np.array_equal(ctx.grads(), ref[1]) and np.array_equal(ctx.params(), ref[0])
     ctx.close()
+
+
+def test_module_times_cover_the_iteration():
+    """Every module has a time of its own: one that only pools has no update to end with, and one whose forward pass is a graph of its own counts it.
+    A module's time is positive and no longer than its step by the host's clock; in serial mode, where nothing overlaps, all of them together are not."""
+    import time
+    import torch
+    from paper_2509_05679_b200 import binding
+    C = 16
+    pool = sy.Net("pool-only", [(sy.CONV3X3, 3, C, 1, 1), (sy.RELU, C, C, 1, 0), (sy.MAXPOOL2, C, C, 2, 0), (sy.GLOBAL_AVGPOOL, C, C, 1, 0), (sy.LINEAR, C, 10, 1, 1)],
+                  [2, 3], 16, 16, 3, 10, 2, 4, 0.05, "fp32")
+    for net, serial in ((pool, False), (pool, True), (nets()["large"], False)):
+        ctx = make_ctx(net, sy.init_params(net.layers, 0, bf16=net.dtype == "bf16"), serial=serial)
+        x, y = binding.to_device(net.dtype, sy.batch_inputs(net, 0)), torch.from_numpy(sy.batch_labels(net, 0)).cuda()
+        for t in range(2 * net.K + 4):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            ctx.step(x, y)
+            torch.cuda.synchronize()
+            wall = (time.perf_counter() - t0) * 1e3
+            ms = ctx.module_times()
+            assert np.all(ms > 0) and np.all(ms < wall), (t, ms, wall)
+            if serial:
+                assert ms.sum() < wall, (t, ms, wall)
+        ctx.close()
