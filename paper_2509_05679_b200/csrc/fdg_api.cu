@@ -64,6 +64,7 @@ struct Op {
     // tensor-core plan (bf16 storage, channel counts that are multiples of 64, power-of-two images)
     bool tc;
     bool stem;                                               // thin first-layer conv: dedicated FMA kernels
+    size_t lin_off;                                          // linear layer on the CUDA cores: its weight-gradient workspace in the module's lin_ws (elements)
     bool head;                                               // the network's last linear layer: fused with the loss (head_* kernels)
     char shape[40];                                          // "HxW Cin->Cout kR sS", the profiler's detail tag
     int n_tile_f, n_tile_d, n_tile_w, wg_splits;
@@ -109,7 +110,8 @@ struct Module {
     size_t stash_slot_bytes, wslot_bytes, grad_pool_bytes, in_slot_bytes;
     size_t ws_elems, scratch_elems, red_elems;
     char *in_ring, *stash, *gradpool, *d2, *wring, *wtring;
-    float *master, *grad, *ws, *scratch, *red, *cstat[2], *bstat;
+    float *master, *grad, *ws, *lin_ws, *scratch, *red, *cstat[2], *bstat;
+    size_t lin_elems;
     bool fused_update;             // one kernel per step updates all parameters and emits the next weight version (both layouts)
     tc::UpdTable upd;
     size_t cstat_elems[2];
@@ -454,7 +456,7 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
         if (d.own_grad) { d.goff = goff; goff += align_up(d.elems() * ctx->M * ctx->esz, 256); }
     }
     size_t red_pos = 0;
-    m.ws_elems = 0; m.scratch_elems = 64; m.red_elems = 4;
+    m.ws_elems = 0; m.scratch_elems = 64; m.red_elems = 4; m.lin_elems = 0;
     for (Op& o : m.ops) {
         if (o.type == OP_BN) {
             o.stats_off = soff; soff += align_up((size_t)ctx->n_workers * o.g.C * (ctx->dt == 0 ? 4 : 2) * sizeof(float), 256);
@@ -468,6 +470,10 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             if (o.stem) m.ws_elems = std::max(m.ws_elems, stem_wgrad_workspace_elems(o.g));
             if (o.stem_tc) m.ws_elems = std::max(m.ws_elems, tc::stem_wg_workspace_elems(o.g.Co, (long)o.g.N * o.g.H, ctx->grid_sms));
             m.ws_elems = std::max(m.ws_elems, wgrad_workspace_elems(o.g));
+            if (!o.tc && linear_supported(o.g)) {            // (a layer whose tensor-core launch is refused goes without)
+                o.lin_off = m.lin_elems;
+                m.lin_elems += align_up(std::max(linear_workspace_elems(o.g, 1), ctx->R > 1 ? linear_workspace_elems(o.g, ctx->R) : 0), 64);
+            }
             if (ctx->R > 1) m.ws_elems = std::max(m.ws_elems, fconv_wgrad_workspace_elems(o.g, ctx->R));
             m.scratch_elems = std::max(m.scratch_elems, (size_t)64 * o.g.Co);
             if (relu_bias_backward_supported(ctx->dt, o.g.Co)) m.scratch_elems = std::max(m.scratch_elems, relu_bias_backward_scratch_elems(o.g.Co));
@@ -795,6 +801,8 @@ void forward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version) {
             for (int g = 0; g < m.groups; ++g) forward_ops(c, kk, batch, version, g, i, i + 1);
 }
 
+float* lin_ws(const Module& m, const Op& o) { return m.lin_ws ? m.lin_ws + o.lin_off : nullptr; }
+
 // gradient buffer of a tensor during iteration t
 char* grad_ptr(fdg_ctx* c, int kk, int id, int64_t t) {
     Module& m = c->mod[kk];
@@ -843,8 +851,9 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
                 }
                 if (!o.tc && linear_supported(g)) {
                     profile_detail(o.shape);
+                    // the workspace is this layer's own: with several groups the next one's launch waits for the sums on its stream
                     linear_backward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.relu ? T(o.out) : nullptr, gout, gin, o.acc_in, mgrad + o.w_off,
-                                    o.bias ? mgrad + m.n_big + o.b_off : nullptr, g, 1, 0, 0, acc_p, s);
+                                    o.bias ? mgrad + m.n_big + o.b_off : nullptr, g, 1, 0, 0, acc_p, lin_ws(m, o), s, m.groups > 1 ? s : m.wstream, m.wev);
                     profile_detail(nullptr);
                     break;
                 }
@@ -862,13 +871,13 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
                 if (o.stem && tc_stem_wgrad(c, m, o, P.tensor(o.in), grad_ptr(c, kk, o.out, t), mgrad + o.w_off, wn, ws)) {}
                 else if (o.stem) stem_wgrad(T(o.in), gout, mgrad + o.w_off, m.ws, g, acc_p, ws);
                 else if (o.tc && tc_wgrad(c, m, o, P.tensor(o.in), grad_ptr(c, kk, o.out, t), mgrad + o.w_off, wn, ws)) {}
-                else if (linear_supported(g)) linear_backward(dt, T(o.in), nullptr, nullptr, gout, nullptr, false, mgrad + o.w_off, nullptr, g, 1, 0, 0, acc_p, ws);
+                else if (linear_supported(g)) linear_backward(dt, T(o.in), nullptr, nullptr, gout, nullptr, false, mgrad + o.w_off, nullptr, g, 1, 0, 0, acc_p, nullptr, ws, ws, m.wev);
                 else fconv_wgrad(dt, T(o.in), gout, mgrad + o.w_off, m.ws, g, 1, 0, acc_p, ws);
                 if (o.bias && !fused_rb && !o.masked_by) bias_grad(dt, gout, mgrad + m.n_big + o.b_off, m.scratch, orows, g.Co, acc_p, s);
                 if (gin && !(o.tc && tc_dgrad(c, m, o, grad_ptr(c, kk, o.out, t), grad_ptr(c, kk, o.in, t), version, o.acc_in,
                                                      below ? P.tensor(o.in) : nullptr, col, wn, s))) {
                     c->mask_lost = c->mask_lost || below;
-                    if (linear_supported(g)) linear_backward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), nullptr, gout, gin, o.acc_in, nullptr, nullptr, g, 1, 0, 0, false, s);
+                    if (linear_supported(g)) linear_backward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), nullptr, gout, gin, o.acc_in, nullptr, nullptr, g, 1, 0, 0, false, nullptr, s, s, m.wev);
                     else fconv_dgrad(dt, gout, wbig(c, m, version, o.w_off, rep), gin, g, o.acc_in ? EPI_ACCUM : 0, 1, 0, s);
                 }
                 profile_detail(nullptr);
@@ -931,7 +940,7 @@ bool backward_op_replicas(fdg_ctx* c, int kk, int64_t batch, int64_t version, in
             if (linear_supported(o.g)) {
                 profile_detail(o.shape);
                 linear_backward(dt, P.tensor(o.in), w, o.relu ? P.tensor(o.out) : nullptr, gout, gin, o.acc_in, m.grad + o.w_off,
-                                o.bias ? m.grad + m.n_big + o.b_off : nullptr, o.g, c->R, wg, gg, false, s);
+                                o.bias ? m.grad + m.n_big + o.b_off : nullptr, o.g, c->R, wg, gg, false, lin_ws(m, o), s, m.wstream, m.wev);
                 profile_detail(nullptr);
                 return true;
             }
@@ -1542,6 +1551,7 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
         m.master = (float*)get((size_t)ctx->R * (m.n_big + m.n_small) * sizeof(float));
         m.grad = (float*)get((size_t)ctx->R * (m.n_big + m.n_small) * sizeof(float));
         m.ws = (float*)get(m.ws_elems * sizeof(float));
+        m.lin_ws = m.lin_elems ? (float*)get(m.lin_elems * sizeof(float)) : nullptr;
         m.scratch = (float*)get(m.scratch_elems * sizeof(float));
         m.red = (float*)get(m.red_elems * sizeof(float));
         m.scratch_f = (float*)get(m.scratch_elems * sizeof(float));

@@ -20,13 +20,16 @@ void   conv_forward(int dt, const void* x, const void* w, const float* bias, voi
 // Linear layers (linear.cu).  linear_backward: dx (+)= dy' W (dx_or_null == nullptr: not needed), dW (+)= dy'^T x, db (+)= column sums of
 // dy' in one launch; dy' = dy * [y > 0] if y_or_null is given (the layer ends in a ReLU), else dy.  The sums run over the worker x
 // batch axis, which is the worker average of Eq. dl_update (b) for P = 11^T/N.  accum_p: dW and db are added to (a second group of workers).  dw_or_null ==
-// nullptr: dx alone; dx_or_null == nullptr: w is not read.
+// nullptr: dx alone; dx_or_null == nullptr: w is not read.  Many samples: dW and db go through partial matrices in workspace
+// (linear_workspace_elems floats, the layer's own; nullptr: one part) that a second launch on st_reduce, behind `ready`, adds up.
 bool   linear_supported(const ConvGeom& g);
+size_t linear_workspace_elems(const ConvGeom& g, int groups);
 // groups, w_group, b_group, g_group: as for the convolutions below (g.N counts the samples of all groups).
 void   linear_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
                       cudaStream_t st);
 void   linear_backward(int dt, const void* x, const void* w, const void* y_or_null, const void* dy, void* dx_or_null, bool accum_dx, float* dw_or_null, float* db_or_null,
-                       const ConvGeom& g, int groups, size_t w_group, size_t g_group, bool accum_p, cudaStream_t st);
+                       const ConvGeom& g, int groups, size_t w_group, size_t g_group, bool accum_p, float* workspace, cudaStream_t st, cudaStream_t st_reduce,
+                       cudaEvent_t ready);
 // Convolutions (3x3 and 1x1, stride 1 and 2) in the packed-FMA kernels of fconv.cu: forward, dx (+)= conv_transpose(dy, W), dW (+)= the sum
 // over all N*Ho*Wo rows of dy^T (x) patches(x) (fp32).  `groups`: consecutive equal groups of images, each with its own weights
 // (w_group elements apart; biases b_group apart; weight gradients w_group apart).  false: shape not covered, nothing launched.

@@ -8,7 +8,8 @@
 // two launches each with serial chains of up to 3072 / 16 slices or a few CTAs (62 us for the input gradient of 512 -> 256 on 64
 // samples).  So: 32 x 64 tiles of 128 threads, and a forward or input-gradient tile is split over the contraction among the CTAs of a
 // cluster, which add their partial tiles through distributed shared memory in rank order: no workspace, no second launch.  A
-// weight-gradient tile contracts over the samples, has no split, and the CTAs of a cluster take tiles of their own.
+// weight-gradient tile contracts over the samples; the CTAs of a cluster take tiles of their own.  From 1024 samples on that chain
+// is split over CTAs that leave partial matrices in a workspace, and a second launch (off the chain of the backward pass) adds them.
 // Arithmetic as in fconv.cu: packed FMAs with the pairs along the contraction, chains of at most 16 products into a compensated sum.
 #include "kernels.h"
 #include "launch.h"
@@ -53,6 +54,7 @@ struct LinArgs {
     int vec_k, vec_n;                    // rows of length K / N can be read 4 elements at a time
     int split;                           // CTAs per cluster
     int dx_clusters, dx_tiles_n, dw_tiles_n, dw_tiles;
+    int dw_splits; float* part;          // > 1: every dW tile in this many parts of the samples, to part: [group][split][N * K, then N sums of db]
     size_t w_group, b_group, g_group;    // grid.y groups of M samples each: elements between their weights, biases, parameter gradients
 };
 
@@ -68,6 +70,7 @@ __device__ __forceinline__ LinArgs of_group(const LinArgs& in, bool fwd) {
     if (a.out) a.out = (a.epi & EPI_OUT_F32) ? (void*)((float*)a.out + mn) : (void*)((T*)a.out + (fwd ? mn : mk));
     if (a.dw) a.dw += g * a.g_group;
     if (a.db) a.db += g * a.g_group;
+    if (a.part) a.part += g * a.dw_splits * ((size_t)a.N * a.K + a.N);
     return a;
 }
 
@@ -254,7 +257,7 @@ __global__ void __launch_bounds__(LT) lin_fwd_kernel(const LinArgs args) {
     join_tile<T>(a, row0, col0, a.M, a.N, v, a.bias, sm);
 }
 
-// The first dx_clusters clusters: input gradient; the others: `split` weight-gradient tiles each.
+// The first dx_clusters clusters: input gradient; the others: `split` weight-gradient tiles (or parts of tiles) each.
 template <typename T>
 __global__ void __launch_bounds__(LT) lin_bwd_kernel(const LinArgs args) {
     const LinArgs a = of_group<T>(args, false);
@@ -268,28 +271,65 @@ __global__ void __launch_bounds__(LT) lin_bwd_kernel(const LinArgs args) {
         join_tile<T>(a, row0, col0, a.M, a.K, v, nullptr, sm);
         return;
     }
-    const int tile = (cl - a.dx_clusters) * a.split + rank;
-    if (tile >= a.dw_tiles) return;
+    const int item = (cl - a.dx_clusters) * a.split + rank;
+    if (item >= a.dw_tiles * a.dw_splits) return;
+    const int tile = item % a.dw_tiles, sp = item / a.dw_tiles;
     const int row0 = tile / a.dw_tiles_n * LM, col0 = tile % a.dw_tiles_n * LN;
+    float* dw = a.dw; float* db = a.db;
+    int s0 = 0, s1 = a.M, accum = a.accum_p;
+    if (a.dw_splits > 1) {
+        my_range(a.M, a.dw_splits, sp, s0, s1);
+        dw = a.part + sp * ((size_t)a.N * a.K + a.N); accum = 0;
+        if (db) db = dw + (size_t)a.N * a.K;
+    }
     float bs = 0.f;
-    tile_product<T, L_DW>(a, row0, col0, 0, a.M, sm, v, a.db && col0 == 0 ? &bs : nullptr);
+    tile_product<T, L_DW>(a, row0, col0, s0, s1, sm, v, db && col0 == 0 ? &bs : nullptr);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane & 7, cg = lane >> 3;
     const int c = col0 + warp * 16 + 4 * cg;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int r = row0 + g + 8 * i;
         if (r >= a.N || c >= a.K) continue;
-        float* const d = a.dw + (size_t)r * a.K + c;
-        if ((a.K & 3) == 0 && (((uintptr_t)a.dw) & 15) == 0) {
+        float* const d = dw + (size_t)r * a.K + c;
+        if ((a.K & 3) == 0 && (((uintptr_t)dw) & 15) == 0) {
             float4 o = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
-            if (a.accum_p) { const float4 old = *(const float4*)d; o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w; }
+            if (accum) { const float4 old = *(const float4*)d; o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w; }
             *(float4*)d = o;
         } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) if (c + j < a.K) d[j] = a.accum_p ? d[j] + v[i][j] : v[i][j];
+            for (int j = 0; j < 4; ++j) if (c + j < a.K) d[j] = accum ? d[j] + v[i][j] : v[i][j];
         }
     }
-    if (a.db && col0 == 0 && tid < LM && row0 + tid < a.N) a.db[row0 + tid] = a.accum_p ? a.db[row0 + tid] + bs : bs;
+    if (db && col0 == 0 && tid < LM && row0 + tid < a.N) db[row0 + tid] = accum ? db[row0 + tid] + bs : bs;
+}
+
+// dW and db from the partial matrices: 32 elements per CTA, eight threads of different splits per element, four loads in flight each, then their
+// sums in order.
+__global__ void __launch_bounds__(256) lin_reduce_kernel(const float* __restrict__ part, float* __restrict__ dw, float* __restrict__ db, int splits, size_t nk, int N,
+                                                         size_t g_group, bool accum) {
+    __shared__ float sh[8][32];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const size_t e = (size_t)blockIdx.x * 32 + tx, n = nk + N;
+    const float* const src = part + blockIdx.y * (splits * n) + e;
+    float s = 0.f;
+    if (e < n) {
+        int k = ty;
+        for (; k + 24 < splits; k += 32) {
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = src[(size_t)(k + 8 * u) * n];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s += v[u];
+        }
+        for (; k < splits; k += 8) s += src[(size_t)k * n];
+    }
+    sh[ty][tx] = s;
+    __syncthreads();
+    if (ty != 0 || e >= n || (e >= nk && !db)) return;
+#pragma unroll
+    for (int k = 1; k < 8; ++k) s += sh[k][tx];
+    float* const d = (e < nk ? dw + e : db + (e - nk)) + blockIdx.y * g_group;
+    *d = accum ? *d + s : s;
 }
 
 // CTAs per cluster: as many as fill the device once (148 SMs, four CTAs each take the latency), a power of two up to 8 (the portable
@@ -299,11 +339,28 @@ int pick_split(int tiles, int contraction) {
     while (s < 8 && tiles * s * 2 <= 148 * 2 && contraction >= s * 2 * 2 * LK) s *= 2;
     return s;
 }
+// Parts of a weight-gradient tile's samples: at least DW_CHUNKS chunks each, and no more CTAs than four per SM.  Without them 16 x 1024 samples of
+// a 70-33-65-17-5 network took 2565 us per step (the implicit GEMM that these kernels replaced 385), 784-64-32-10 1100 (380), bf16 4352 (397) and 1670
+// (394); 8 x 256 samples 344 (210) and 144 (128).  With them 296, 262, 366, 290, 125 and 80.
+constexpr int DW_CHUNKS = 16;
+int max_dw_splits(int tiles, int samples) {
+    const int by_samples = (samples + LK - 1) / LK / DW_CHUNKS, by_ctas = 4 * 148 / tiles, s = by_samples < by_ctas ? by_samples : by_ctas;
+    return s < 2 ? 1 : s;
+}
+int pick_dw_splits(int tiles, int samples) {                          // parts that are not empty
+    const int s = max_dw_splits(tiles, samples), per = ((samples + s - 1) / s + LK - 1) / LK * LK;       // as my_range
+    return (samples + per - 1) / per;
+}
+int dw_tile_count(const ConvGeom& g) { return ((g.Co + LM - 1) / LM) * ((g.C + LN - 1) / LN); }
 bool aligned4(const void* p, int dt) { return ((uintptr_t)p & (dt ? 7 : 15)) == 0; }
 
 }  // namespace
 
 bool linear_supported(const ConvGeom& g) { return g.H * g.W == 1 && g.R == 1; }
+size_t linear_workspace_elems(const ConvGeom& g, int groups) {
+    const int s = max_dw_splits(dw_tile_count(g) * groups, g.N / groups);     // a window of the batch has no more
+    return s > 1 ? (size_t)groups * s * ((size_t)g.Co * g.C + g.Co) : 0;
+}
 
 void linear_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
                     cudaStream_t s) {
@@ -319,7 +376,8 @@ void linear_forward(int dt, const void* x, const void* w, const float* bias, voi
 }
 
 void linear_backward(int dt, const void* x, const void* w, const void* y_or_null, const void* dy, void* dx_or_null, bool accum_dx, float* dw_or_null, float* db_or_null,
-                     const ConvGeom& g, int groups, size_t w_group, size_t g_group, bool accum_p, cudaStream_t s) {
+                     const ConvGeom& g, int groups, size_t w_group, size_t g_group, bool accum_p, float* workspace, cudaStream_t s, cudaStream_t s_reduce,
+                     cudaEvent_t ready) {
     LinArgs a{};
     a.x = x; a.w = w; a.y = y_or_null; a.dy = dy; a.out = dx_or_null; a.dw = dw_or_null; a.db = db_or_null; a.M = g.N / groups; a.N = g.Co; a.K = g.C;
     a.w_group = w_group; a.g_group = g_group;
@@ -331,12 +389,21 @@ void linear_backward(int dt, const void* x, const void* w, const void* y_or_null
     a.split = dx_tiles ? pick_split(dx_tiles * groups, a.N) : 1;
     a.dx_clusters = dx_tiles;
     a.dw_tiles_n = (a.K + LN - 1) / LN;
-    a.dw_tiles = dw_or_null ? ((a.N + LM - 1) / LM) * a.dw_tiles_n : 0;
-    const int clusters = dx_tiles + (a.dw_tiles + a.split - 1) / a.split;
+    a.dw_tiles = dw_or_null ? dw_tile_count(g) : 0;
+    a.dw_splits = dw_or_null && workspace ? pick_dw_splits(a.dw_tiles * groups, a.M) : 1;
+    if (a.dw_splits > 1) a.part = workspace;
+    const int clusters = dx_tiles + (a.dw_tiles * a.dw_splits + a.split - 1) / a.split;
     const double esz = dt ? 2.0 : 4.0;
-    Scope sc(KC_FMA_WGRAD, (dx_or_null ? 4.0 : 2.0) * g.N * a.N * a.K, esz * ((double)a.M * a.K * (dx_or_null ? 2 : 1) + (double)a.N * a.K + (double)a.M * a.N * (y_or_null ? 2 : 1)) + 4.0 * a.N * a.K, s);
-    if (dt) klaunch_cluster(lin_bwd_kernel<bf16>, dim3(clusters * a.split, groups), LT, 0, s, a.split, a);
-    else klaunch_cluster(lin_bwd_kernel<float>, dim3(clusters * a.split, groups), LT, 0, s, a.split, a);
+    {
+        Scope sc(KC_FMA_WGRAD, (dx_or_null ? 4.0 : 2.0) * g.N * a.N * a.K, esz * ((double)a.M * a.K * (dx_or_null ? 2 : 1) + (double)a.N * a.K + (double)a.M * a.N * (y_or_null ? 2 : 1)) + 4.0 * a.N * a.K, s);
+        if (dt) klaunch_cluster(lin_bwd_kernel<bf16>, dim3(clusters * a.split, groups), LT, 0, s, a.split, a);
+        else klaunch_cluster(lin_bwd_kernel<float>, dim3(clusters * a.split, groups), LT, 0, s, a.split, a);
+    }
+    if (a.dw_splits == 1) return;
+    const size_t nk = (size_t)a.N * a.K;
+    if (s_reduce != s) { step_record(ready, s); step_wait(s_reduce, ready); }
+    Scope sc(KC_SPLITK, 0.0, 4.0 * groups * (a.dw_splits + 1) * (nk + a.N), s_reduce);
+    klaunch(lin_reduce_kernel, dim3((unsigned)((nk + a.N + 31) / 32), groups), 256, 0, s_reduce, workspace, dw_or_null, db_or_null, a.dw_splits, nk, a.N, g_group, accum_p);
 }
 
 }  // namespace fdg

@@ -48,6 +48,18 @@ def test_single_module_single_worker_is_plain_sgd(orc):
     run_parity(orc, net, 3, param_tol=TOL, loss_tol=1e-5)
 
 
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("workers,batch,groups", [(1, 1023, 0), (1, 1024, 0), (3, 345, 0), (2, 1537, 2), (4, 2048, 0), (2, 1100, "replicas")])
+def test_linear_layers_of_many_samples(orc, dtype, workers, batch, groups):
+    """The weight gradient's sum over the samples in one part (below 1024), in two, in parts that are not equally long, per group of
+    workers or per worker's replica, and in 16 parts (8192 samples).  Without ReLU layers."""
+    net = sy.without_relu(sy.Net("mlp", sy.mlp_layers([20, 33, 70, 5]), [2], 1, 1, 20, 5, workers, batch, 0.05, dtype))
+    # bf16: the tolerances of test_gpu_small_problems.py (1 / 1035 is no power of two, so stored error gradients round differently here and there)
+    tol = dict(param_tol=TOL, loss_tol=1e-5) if dtype == "fp32" else dict(grad_tol=2e-2, loss_tol=1e-3)
+    kw = dict(mixing=np.full((workers, workers), 1.0 / workers)) if groups == "replicas" else dict(worker_groups=groups)
+    run_parity(orc, net, 2 * net.K, **kw, **tol)
+
+
 def test_serial_and_concurrent_modes_are_bit_identical():
     import torch
     from paper_2509_05679_b200 import binding
