@@ -1299,12 +1299,22 @@ __global__ void __launch_bounds__(256) head_bwd_k(const T* __restrict__ x, const
         out[(size_t)threadIdx.x * (K + 1) + K] = a;
     }
 }
+// blockDim = (elements, lanes): lane y adds the CTAs y, y + lanes, ...
 __global__ void head_reduce_k(const float* __restrict__ part, float* __restrict__ dW, float* __restrict__ db, int ctas, int K, int C) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= C * (K + 1)) return;
+    __shared__ float sh[8][32];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, lanes = blockDim.y, n = C * (K + 1);
     float s = 0.f;
+    if (i < n) {
 #pragma unroll 8
-    for (int b = 0; b < ctas; ++b) s += part[(size_t)b * C * (K + 1) + i];
+        for (int b = threadIdx.y; b < ctas; b += lanes) s += part[(size_t)b * n + i];
+    }
+    if (lanes > 1) {
+        sh[threadIdx.y][threadIdx.x] = s;
+        __syncthreads();
+        if (threadIdx.y > 0) return;
+        for (int y = 1; y < lanes; ++y) s += sh[y][threadIdx.x];
+    }
+    if (i >= n) return;
     const int c = i / (K + 1), k = i - c * (K + 1);
     if (k < K) dW[(size_t)c * K + k] = s;
     else if (db) db[c] = s;
@@ -1326,8 +1336,10 @@ void head_backward(int dt, const void* x, const void* W, const void* dlogits, vo
                    int K, int C, cudaStream_t s) {
     const unsigned ctas = (M + HEAD_ROWS_PER_CTA - 1) / HEAD_ROWS_PER_CTA;
     const int nkv = K / (dt ? 8 : 4);
-    // vectors of columns per CTA: a power of two that puts about one CTA on every SM, at least eight (a warp then reads whole sectors)
-    int kvs = 256;
+    // vectors of columns per CTA: a power of two that puts about one CTA on every SM, at least eight (a warp then reads whole sectors), and no
+    // more than there are: the other threads take other samples (16384 samples, 256 columns in bf16: 50 us with 256 whatever there are, 31 so)
+    int kvs = 8;
+    while (kvs < 256 && kvs < nkv) kvs *= 2;
     while (kvs > 8 && ctas * ((nkv + kvs - 1) / kvs) < 148) kvs /= 2;
     const dim3 grid(ctas, (nkv + kvs - 1) / kvs);
     Scope sc(KC_FMA_WGRAD, (dx_or_null ? 4.0 : 2.0) * M * K * C, (dt ? 2.0 : 4.0) * ((double)M * K * (dx_or_null ? 2 : 1) + (double)C * K + (double)M * C), s);
@@ -1337,7 +1349,9 @@ void head_backward(int dt, const void* x, const void* W, const void* dlogits, vo
 void head_reduce(float* dW, float* db_or_null, const float* scratch, int M, int K, int C, cudaStream_t s) {
     const unsigned ctas = (M + HEAD_ROWS_PER_CTA - 1) / HEAD_ROWS_PER_CTA;
     Scope sc(KC_SPLITK, 0.0, 4.0 * (ctas + 1) * C * (K + 1), s);
-    klaunch(head_reduce_k, cdiv((size_t)C * (K + 1), 64), 64, 0, s, scratch, dW, db_or_null, (int)ctas, K, C);
+    // from 65 partial matrices on eight threads per element (512 of them, 2570 elements: 62 us with one, 10 so; 68: 15 and 7)
+    if (ctas > 64) klaunch(head_reduce_k, cdiv((size_t)C * (K + 1), 32), dim3(32, 8), 0, s, scratch, dW, db_or_null, (int)ctas, K, C);
+    else klaunch(head_reduce_k, cdiv((size_t)C * (K + 1), 64), 64, 0, s, scratch, dW, db_or_null, (int)ctas, K, C);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -77,3 +77,12 @@ def test_batch_norm_on_the_network_input(orc, dtype, c, workers, batch, size, re
         run_parity(orc, net, 2, param_tol=1e-5, loss_tol=1e-5)
     else:
         run_parity(orc, net, 1, grad_tol=2e-2, elem_tol=3e-2, pair_bn=True, loss_tol=1e-3)
+
+
+@pytest.mark.parametrize("batch", [2048, 2049, 4737])
+@pytest.mark.parametrize("hidden", [64, 320])
+def test_classifier_head_of_many_samples(orc, batch, hidden):
+    """64 and 65 blocks of 32 samples (the line between the two ways of adding their partial gradients), and 149 (all columns in one block), with 8 and 40
+    vectors of columns; the masked error and the bias gradient that the head takes along for the layer below."""
+    net = sy.Net("mlp", sy.mlp_layers([64, hidden, 10]), [], 1, 1, 64, 10, 1, batch, 0.05, "bf16")
+    run_parity(orc, net, 1, grad_tol=2e-2, noise_factor=3.0, loss_tol=1e-3)
