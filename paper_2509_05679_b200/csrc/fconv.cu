@@ -33,6 +33,7 @@ constexpr int PITCH = 20;                // floats per pixel (or weight row) in 
 constexpr int FW_THREADS = 160;          // 9 taps x 2 groups of 8 c_in x 4 groups of 4 c_out x 2 pixel slices = 144, in five warps: three CTAs put
                                          // four warps on each scheduler and leave 128 registers a thread (nine warps, two CTAs: 96, and spills)
 constexpr int FW_CO = 16, FW_CI = 16;
+constexpr int FW_CTAS = 3 * 148;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
@@ -344,7 +345,7 @@ struct FwParams {
     int pad, hstep;                      // region origin = tile origin * hstep - pad
     int RH, RW, ntaps, toff[9];          // region of a tile; per tap: offset inside it (floats)
     int Wt, Ht, Nt, lw, lh, tiles_w, tiles_h, tiles;     // tile = Wt x Ht x Nt output pixels (powers of two)
-    int ngroup, splits, max_splits, ci_blocks;
+    int ngroup, splits, ci_blocks;
     int nslices, pps;                    // pixel slices of a tile, pixels per slice
     int x_floats;
 };
@@ -509,10 +510,25 @@ int best_tile(int n, int cap) {
 }
 
 struct Tile { int Wt, Ht, Nt; };
-Tile pick_tile(int H, int W, int pixels) {
+// Tile of `pixels` pixels for n images of H x W per group; a tile needs R x R windows, `step` apart, of what it reads.
+// First choice: the exact cover of an image, as best_tile has it.  Images that no power of two covers (7x7, 5x7) leave it tiles of single pixels from
+// 128 images: half empty for the images of one worker, nine pixels read for one.  Where another tile costs less than three quarters
+// (pixels computed, used or not, plus a quarter per pixel read), that one (step times of 24-channel networks on 4 workers x 48: 7x7 fp32 590 us
+// with the exact cover, 290 so; 489 with the implicit GEMM that these kernels replaced; 5x7 511, 291, 483).
+Tile pick_tile(int H, int W, int n, int pixels, int R, int step) {
+    auto cost = [&](int wt, int ht) {
+        const int nt = pixels / (wt * ht);
+        const double tiles = (double)((W + wt - 1) / wt) * ((H + ht - 1) / ht) * ((n + nt - 1) / nt);
+        return tiles * (pixels + 0.25 * nt * ((wt - 1) * step + R) * ((ht - 1) * step + R));
+    };
     Tile t;
     t.Wt = best_tile(W, pixels < 32 ? pixels : 32);
     t.Ht = best_tile(H, pixels / t.Wt);
+    const auto pow2 = [](int v) { return (v & (v - 1)) == 0; };
+    double best = pow2(H) && pow2(W) ? 0.0 : 0.75 * cost(t.Wt, t.Ht);
+    for (int wt = pixels < 32 ? pixels : 32; wt >= 1; wt /= 2)
+        for (int ht = pixels / wt; ht >= 1; ht /= 2)
+            if (cost(wt, ht) < best) { best = cost(wt, ht); t.Wt = wt; t.Ht = ht; }
     t.Nt = pixels / (t.Wt * t.Ht);
     return t;
 }
@@ -546,7 +562,7 @@ bool plan_fc(const ConvGeom& g, int groups, bool back, FcParams& p) {
             p.cls_tap0[++p.ncls] = n;
         }
     }
-    const Tile t = pick_tile(p.Hd, p.Wd, FC_PIX);
+    const Tile t = pick_tile(p.Hd, p.Wd, p.ngroup, FC_PIX, g.R, p.xs);
     p.Wt = t.Wt; p.Ht = t.Ht; p.Nt = t.Nt; p.lw = ilog2(t.Wt); p.lh = ilog2(t.Ht);
     p.tiles_w = (p.Wd + t.Wt - 1) / t.Wt; p.tiles_h = (p.Hd + t.Ht - 1) / t.Ht;
     int maxt = 0;
@@ -605,7 +621,7 @@ bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_
     if ((g.H * g.W == 1 && g.R == 1) || (g.R != 3 && g.R != 1) || (g.stride != 1 && g.stride != 2) || g.N % groups) return false;
   for (int pixels = g.R == 3 && g.stride == 2 ? 64 : 128; pixels >= 32; pixels /= 2) {        // smaller tiles where the halo of tiny images outgrows shared memory
     p = FwParams{};
-    const Tile t = pick_tile(g.Ho, g.Wo, pixels);
+    const Tile t = pick_tile(g.Ho, g.Wo, g.N / groups, pixels, g.R, g.R == 1 ? 1 : g.stride);
     run = t.Wt >= 8 ? 8 : (t.Wt >= 4 ? 4 : 1);
     p.H = g.H; p.W = g.W; p.C = g.C; p.Ho = g.Ho; p.Wo = g.Wo; p.Co = g.Co;
     p.Wt = t.Wt; p.Ht = t.Ht; p.Nt = t.Nt; p.lw = ilog2(t.Wt); p.lh = ilog2(t.Ht);
@@ -625,10 +641,9 @@ bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_
     p.ci_blocks = (g.C + FW_CI - 1) / FW_CI;
     const int blocks = p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO) * groups;
     // three CTAs per SM once around the device, each with at least one tile
-    int want = 3 * 148 / blocks;
+    int want = FW_CTAS / blocks;
     if (want > p.tiles) want = p.tiles;
     if (want < 1) want = 1;
-    p.max_splits = want;
     const int per = (p.tiles + want - 1) / want;
     p.splits = (p.tiles + per - 1) / per;
     p.x_floats = t.Nt * p.RH * p.RW * PITCH;
@@ -689,8 +704,9 @@ int fconv_stat_tiles(const ConvGeom& g, int groups) {
 size_t fconv_wgrad_workspace_elems(const ConvGeom& g, int groups) {
     FwParams p; int G, run; size_t smem;
     if (!plan_fw(g, groups, p, G, run, smem)) return 0;
-    // a window of the batch (fewer tiles) may use more splits than the whole batch, but never more than max_splits of the whole
-    return (size_t)groups * p.max_splits * p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO) * FW_CO * p.ntaps * 8 * G;
+    // a window of the batch may be cut into other tiles, but never uses more splits than fill the device
+    const int blocks = p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO) * groups;
+    return (size_t)blocks * (FW_CTAS > blocks ? FW_CTAS / blocks : 1) * FW_CO * p.ntaps * 8 * G;
 }
 bool fconv_wgrad(int dt, const void* x, const void* dy, float* dw, float* ws, const ConvGeom& g, int groups, size_t w_group, bool accum, cudaStream_t s) {
     FwParams p; int G, run; size_t smem;

@@ -37,6 +37,13 @@ def test_bf16_storage(orc, shape):
     run_parity(orc, _net(shape, "bf16", 2, 4, False), 1, grad_tol=2e-3 if terms <= 144 else 2e-2, loss_tol=1e-4)
 
 
+@pytest.mark.parametrize("workers,batch,groups", [(4, 3, 0), (4, 20, 2), (2, 70, 0)])
+@pytest.mark.parametrize("size,stride", [((7, 7), 1), ((14, 14), 2), ((9, 9), 1), ((3, 3), 1), ((6, 10), 2), ((33, 9), 1)], ids=str)
+def test_images_that_no_power_of_two_covers(orc, size, stride, workers, batch, groups):
+    """Tiles that reach over the image's edge, for few and for many images of one worker; windows of the batch are cut into other tiles than the whole."""
+    run_parity(orc, _net((size, 16, sy.CONV3X3, 24, stride), "fp32", workers, batch, True), 1, param_tol=1e-5, loss_tol=1e-5, worker_groups=groups)
+
+
 @pytest.mark.parametrize("workers,batch", [(1, 1), (2, 130), (5, 3)])
 def test_batch_sizes(orc, workers, batch):
     run_parity(orc, _net(((8, 8), 16, sy.CONV3X3, 32, 2), "fp32", workers, batch, True), 2, param_tol=1e-5, loss_tol=1e-5)
