@@ -215,7 +215,7 @@ Tensor maxpool_fwd(const Tensor& x) {
             double v[4] = {x.at(i, 2 * oy, 2 * ox)[c], x.at(i, 2 * oy, 2 * ox + 1)[c], x.at(i, 2 * oy + 1, 2 * ox)[c], x.at(i, 2 * oy + 1, 2 * ox + 1)[c]};
             double m = std::max(std::max(v[0], v[1]), std::max(v[2], v[3]));
             std::sort(v, v + 4);
-            margin = std::min(margin, v[3] - v[2]);
+            if (v[3] != 0.0 || v[2] != 0.0) margin = std::min(margin, v[3] - v[2]);      // two zeros of a ReLU tie in every precision
             y.at(i, oy, ox)[c] = m;
         }
     note_kink(margin);

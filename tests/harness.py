@@ -139,7 +139,7 @@ def closed_form_trace(K, t):
 
 def run_parity(orc, net: sy.Net, steps: int, *, param_tol=None, grad_tol=None, grad_best_tol=None, loss_tol=None,
                perturb=True, kink_guard=None, grad_steps=None, grad_tol_later=None, elem_tol=None, pair_bn=False,
-               noise_factor=None, elem_noise_factor=None, **ctx_kw):
+               noise_factor=None, elem_noise_factor=None, data_stream=None, **ctx_kw):
     """Step both implementations `steps` times; check the schedule bit-exactly after every step and
     parameters / gradients / loss within the given tolerances.  Returns the per-step records.
 
@@ -155,7 +155,10 @@ def run_parity(orc, net: sy.Net, steps: int, *, param_tol=None, grad_tol=None, g
     tens of percent, see tests/test_oracle_pins.py): a second oracle runs beside the first on inputs of which
     0.1 % were moved by one bf16 ulp; a tensor may deviate from the oracle by `grad_tol` or by `noise_factor`
     times what that twin deviates, whichever is larger (`elem_noise_factor`: the same for the element-wise
-    bound `elem_tol`)."""
+    bound `elem_tol`).
+    `kink_guard`: the run is on the first data stream on which the oracle keeps that distance from every kink
+    (pick_data_stream), or on `data_stream`, for which the oracle's run beside the library's has to show it.  A library that is
+    right within that distance takes the oracle's branches whatever the order of its sums."""
     from paper_2509_05679_b200 import binding
     import torch
     bf16 = net.dtype == "bf16"
@@ -164,13 +167,14 @@ def run_parity(orc, net: sy.Net, steps: int, *, param_tol=None, grad_tol=None, g
         p0 = sy.perturb_params(p0, net.layers, 7, 0.1)
     if bf16:
         p0 = sy.round_to_bf16(p0)
-    stream = pick_data_stream(orc, net, p0, steps, kink_guard) if kink_guard else 0
+    stream = data_stream if data_stream is not None else pick_data_stream(orc, net, p0, steps, kink_guard) if kink_guard else 0
     if kink_guard:
         print(f"{net.name}: data stream {stream} keeps every pre-activation {kink_guard:g} away from the kinks")
     o = make_oracle(orc, net, p0)
     twin = make_oracle(orc, net, p0) if noise_factor else None
     ctx = make_ctx(net, p0, **ctx_kw)
     rec, best = [], {}
+    orc.kink_margin(True)
     try:
         for t in range(steps):
             x, y = sy.batch_inputs(net, t, stream), sy.batch_labels(net, t, stream)
@@ -216,6 +220,8 @@ def run_parity(orc, net: sy.Net, steps: int, *, param_tol=None, grad_tol=None, g
             rec.append(r)
     finally:
         ctx.close()
+    if kink_guard:
+        assert orc.kink_margin(True) >= kink_guard, "the oracle's run comes nearer to a kink than this test allows"
     if grad_best_tol is not None:
         assert best and len(best) == len(gradient_groups(net.layers, pair_bn)), "some tensor never received a gradient"
         bad = {k_: e_ for k_, e_ in best.items() if e_ > grad_best_tol}

@@ -21,31 +21,39 @@ def test_config1_mlp_20_iterations(orc):
     assert len(rec) == 20 and not np.isnan(rec[-1]["loss_g"])
 
 
-def test_mlp_four_modules_ragged_sizes(orc):
+# Networks with ReLU layers run on data on which the oracle keeps every ReLU input and every max-pool gap further from its kink than
+# fp32 rounding moves them (some 1e-7 after a dozen layers and iterations; the distance is checked in each run), so that every equally
+# accurate order of summation passes or fails alike.  The streams were picked by the oracle alone.
+@pytest.mark.parametrize("stream", [4416, 21693])
+def test_mlp_four_modules_ragged_sizes(orc, stream):
     net = sy.Net("mlp-k4", sy.mlp_layers([70, 33, 65, 17, 5]), [2, 4, 6], 1, 1, 70, 5, 3, 7, 0.05, "fp32")
-    run_parity(orc, net, 4 * net.K + 2, param_tol=TOL, loss_tol=1e-5)
+    run_parity(orc, net, 4 * net.K + 2, param_tol=TOL, loss_tol=1e-5, data_stream=stream, kink_guard=3e-4)
 
 
-def test_vgg_shaped_four_modules(orc):
+@pytest.mark.parametrize("stream", [40069, 8274])
+def test_vgg_shaped_four_modules(orc, stream):
     layers, starts = sy.vgg_layers(widths=(6, 10, 12, 20), in_c=3, classes=10)
     net = sy.Net("vgg-small", layers, starts[1:], 16, 16, 3, 10, 2, 3, 0.05, "fp32")
-    run_parity(orc, net, 4 * net.K, param_tol=TOL, loss_tol=1e-5, grad_tol=0.2, grad_best_tol=1e-5)
+    run_parity(orc, net, 4 * net.K, param_tol=TOL, loss_tol=1e-5, grad_tol=0.2, grad_best_tol=1e-5, data_stream=stream, kink_guard=3e-5)
 
 
-def test_resnet_shaped_four_modules_per_worker_batchnorm(orc):
+@pytest.mark.parametrize("stream", [26244, 23998])
+def test_resnet_shaped_four_modules_per_worker_batchnorm(orc, stream):
     net = as_fp32(sy.config(3, n_workers=2, batch=3, width_div=8))
-    rec = run_parity(orc, net, 4 * net.K, param_tol=TOL, loss_tol=1e-5, grad_tol=0.2, grad_best_tol=1e-5)
+    rec = run_parity(orc, net, 4 * net.K, param_tol=TOL, loss_tol=1e-5, grad_tol=0.2, grad_best_tol=1e-5, data_stream=stream, kink_guard=2e-6)
     assert rec[-1]["grad_err"] > 0
 
 
-def test_resnet_shaped_eight_modules_max_delay(orc):
+@pytest.mark.parametrize("stream", [190, 17])
+def test_resnet_shaped_eight_modules_max_delay(orc, stream):
     net = as_fp32(sy.config(4, n_workers=2, batch=2, width_div=16))
-    run_parity(orc, net, 2 * net.K + 3, param_tol=TOL, loss_tol=1e-5)
+    run_parity(orc, net, 2 * net.K + 3, param_tol=TOL, loss_tol=1e-5, data_stream=stream, kink_guard=2.6e-6)
 
 
-def test_single_module_single_worker_is_plain_sgd(orc):
+@pytest.mark.parametrize("stream", [135, 44])
+def test_single_module_single_worker_is_plain_sgd(orc, stream):
     net = as_fp32(sy.config(3, n_workers=1, batch=4, width_div=8, K=1))
-    run_parity(orc, net, 3, param_tol=TOL, loss_tol=1e-5)
+    run_parity(orc, net, 3, param_tol=TOL, loss_tol=1e-5, data_stream=stream, kink_guard=1e-5)
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
