@@ -592,8 +592,8 @@ bool plan_fc(const ConvGeom& g, int groups, bool back, FcParams& p) {
 template <typename T, int NQ, bool VEC, int PP>
 void launch_fc_pp(const void* x, const void* w, const float* bias, void* y, float* stat, const FcParams& p, int groups, cudaStream_t s) {
     const size_t smem = (size_t)p.buffers * (p.x_floats + p.w_floats) * sizeof(float);
-    static bool attr = false;
-    if (!attr) { cudaFuncSetAttribute(fc_kernel<T, NQ, VEC, PP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FC_SMEM_MAX); attr = true; }
+    static OncePerDevice once;
+    allow_smem(once, (const void*)fc_kernel<T, NQ, VEC, PP>, (int)FC_SMEM_MAX);
     const int tiles = p.tiles_w * p.tiles_h * ((p.ngroup + p.Nt - 1) / p.Nt);
     klaunch(fc_kernel<T, NQ, VEC, PP>, dim3(tiles, (p.Co + FC_CO - 1) / FC_CO, groups * p.ncls), 512 / PP, smem, s, (const T*)x, (const T*)w, bias, (T*)y, stat, p);
 }
@@ -656,8 +656,8 @@ bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_
 }
 template <typename T, int XS, int G, int RUN>
 void launch_fw(const void* x, const void* dy, float* ws, const FwParams& p, int groups, size_t smem, cudaStream_t s) {
-    static bool attr = false;
-    if (!attr) { cudaFuncSetAttribute(fw_kernel<T, XS, G, RUN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FC_SMEM_MAX); attr = true; }
+    static OncePerDevice once;
+    allow_smem(once, (const void*)fw_kernel<T, XS, G, RUN>, (int)FC_SMEM_MAX);
     klaunch(fw_kernel<T, XS, G, RUN>, dim3(p.splits, p.ci_blocks * ((p.Co + FW_CO - 1) / FW_CO), groups), FW_THREADS, smem, s, (const T*)x, (const T*)dy, ws, p);
 }
 template <typename T, int XS, int G>

@@ -989,9 +989,9 @@ static int bns_chunks(int nw, long rpw, int C, int sms_wanted) {
 }
 template <int MODE>
 static void bns_launch(const BnsArgs& a, int chunks, int nw, cudaStream_t s) {
-    static bool attr = false;
     constexpr int smem = BNS_SMEM + (MODE == 3 ? BNS_RED_BYTES : 0);
-    if (!attr) { cudaFuncSetAttribute(bns_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); attr = true; }
+    static OncePerDevice once;
+    allow_smem(once, (const void*)bns_kernel<MODE>, smem);
     klaunch(bns_kernel<MODE>, dim3(chunks, nw), BNV_THREADS, smem, s, a);
 }
 

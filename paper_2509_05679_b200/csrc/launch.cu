@@ -6,6 +6,15 @@ namespace fdg {
 static thread_local StepGraph* t_graph = nullptr;
 StepGraph* StepGraph::current() { return t_graph; }
 
+cudaError_t allow_smem(OncePerDevice& once, const void* kernel, int bytes) {
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess || once.done(dev)) return e;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) once.set(dev);
+    return e;
+}
+
 static cudaError_t launch_now(const void* func, dim3 grid, dim3 block, size_t smem, cudaStream_t s, void** args, int cluster) {
     if (!cluster) return cudaLaunchKernel(func, grid, block, args, smem, s);
     cudaLaunchConfig_t cfg = {};

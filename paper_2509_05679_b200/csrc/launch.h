@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <cstring>
 #include <tuple>
 #include <utility>
@@ -41,6 +42,17 @@ private:
     size_t next_ = 0;
     bool bad_ = false;
 };
+
+// Something done once per device and process (devices 0 to 63; done again every time on others).  Two threads may both do it.
+class OncePerDevice {
+public:
+    bool done(int device) const { return device >= 0 && device < 64 && (mask_.load(std::memory_order_acquire) >> device & 1); }
+    void set(int device) { if (device >= 0 && device < 64) mask_.fetch_or(1ull << device, std::memory_order_release); }
+private:
+    std::atomic<uint64_t> mask_{0};
+};
+// Lets `kernel` have `bytes` of dynamic shared memory on the current device (a kernel's attributes are those of one device); `once` is the kernel's.
+cudaError_t allow_smem(OncePerDevice& once, const void* kernel, int bytes);
 
 // cluster: CTAs per cluster along x (0: none)
 cudaError_t launch_raw(const void* func, dim3 grid, dim3 block, size_t smem, cudaStream_t s, void** args, const size_t* sizes, int nargs, int cluster);

@@ -181,8 +181,8 @@ void stem_forward(const void* x, const void* w, const float* bias, void* y, cons
 void stem_wgrad(const void* x, const void* dy, float* dw, float* workspace, const ConvGeom& g, bool accum, cudaStream_t s) {
     const int TH = ST_THREADS / g.W, K = 9 * g.C;
     const size_t smem = ((size_t)(TH + 2) * (g.W + 2) * g.C + 8) * sizeof(float) + 16 + (size_t)ST_THREADS * 64 * 2 + 64 * 28 * sizeof(float);
-    static bool attr = false;
-    if (!attr) { cudaFuncSetAttribute(stem_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024); attr = true; }
+    static OncePerDevice once;
+    allow_smem(once, (const void*)stem_wgrad_kernel, 96 * 1024);
     const int tiles = g.N * (g.H / TH);
     const int blocks = tiles < stem_wgrad_blocks() ? tiles : stem_wgrad_blocks();
     const double pix = (double)g.N * g.H * g.W;

@@ -1668,12 +1668,8 @@ static cudaError_t launch_km(const TensorMap& a, const TensorMap& b, const Tenso
     constexpr int per_sm = by_smem < by_tmem ? by_smem : by_tmem;
     static_assert(per_sm >= 1 && per_sm <= 2, "CTAs per SM");
     auto kernel = km_kernel<N_TILE, STAGES, EPI_WARPS, false, KSUB, per_sm, ROWS, RES_KB>;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static OncePerDevice once;
+    if (const cudaError_t e = allow_smem(once, (const void*)kernel, smem); e != cudaSuccess) return e;
     const int total = p.tiles_w * p.tiles_h * p.tiles_n * (p.Cn / N_TILE) * p.ncls;
     const int slots = sm_count(p.sms) * per_sm;
     const int grid = total < slots ? total : slots;
@@ -1692,16 +1688,16 @@ static cudaError_t launch_km_pair(const TensorMap& a, const TensorMap& b, const 
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.blockDim = dim3(64 + 32 * EPI_WARPS); cfg.dynamicSmemBytes = smem; cfg.stream = s; cfg.attrs = at; cfg.numAttrs = 1;
-    static int resident_pairs = 0;              // pairs that can be resident at once on the whole device
+    static OncePerDevice once;
+    if (const cudaError_t e = allow_smem(once, (const void*)kernel, smem); e != cudaSuccess) return e;
+    static std::atomic<int> resident_pairs{0};  // pairs that can be resident at once on the whole device (the devices of one machine are alike)
     if (!resident_pairs) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
         cfg.gridDim = dim3(device_sms());
         int n = 0;
         if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n <= 0) { cudaGetLastError(); n = device_sms() / 2; }
         resident_pairs = n;
     }
-    const int budget = sm_count(p.sms) > 1 ? sm_count(p.sms) / 2 : 1, max_pairs = resident_pairs < budget ? resident_pairs : budget;
+    const int budget = sm_count(p.sms) > 1 ? sm_count(p.sms) / 2 : 1, resident = resident_pairs, max_pairs = resident < budget ? resident : budget;
     const int total = (p.tiles_w * p.tiles_h * p.tiles_n / 2) * (p.Cn / N_TILE) * p.ncls;
     return klaunch_cluster(kernel, dim3(2 * (total < max_pairs ? total : max_pairs)), dim3(64 + 32 * EPI_WARPS), smem, s, 2, *(const CUtensorMap*)&a, *(const CUtensorMap*)&b,
                            *(const CUtensorMap*)&o, p);
@@ -1756,12 +1752,8 @@ int small_split(const KmParams& p) {
 template <int S>
 static cudaError_t launch_ks(const TensorMap& a, const TensorMap& b, const KmParams& p, int tiles, cudaStream_t s) {
     constexpr int smem = KS_STAGES * KS_STAGE_BYTES + 1024 + 256;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(ks_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static OncePerDevice once;
+    if (const cudaError_t e = allow_smem(once, (const void*)ks_kernel<S>, smem); e != cudaSuccess) return e;
     return klaunch_cluster(ks_kernel<S>, dim3(tiles * S), dim3(NUM_THREADS), smem, s, S > 1 ? S : 0, *(const CUtensorMap*)&a, *(const CUtensorMap*)&b, p);
 }
 cudaError_t run_small(const TensorMap& a, const TensorMap& b, const KmParams& p, int split, cudaStream_t s) {
@@ -1777,12 +1769,8 @@ cudaError_t run_small(const TensorMap& a, const TensorMap& b, const KmParams& p,
 template <int N_TILE, int STAGES>
 static cudaError_t launch_wg(const TensorMap& x, const TensorMap& dy, const WgParams& p, dim3 grid, cudaStream_t s) {
     constexpr int smem = STAGES * (2 + N_TILE / 64) * 8192 + 1024 + 256;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(wg_kernel<N_TILE, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static OncePerDevice once;
+    if (const cudaError_t e = allow_smem(once, (const void*)wg_kernel<N_TILE, STAGES>, smem); e != cudaSuccess) return e;
     return klaunch(wg_kernel<N_TILE, STAGES>, grid, NUM_THREADS, smem, s, *(const CUtensorMap*)&x, *(const CUtensorMap*)&dy, p);
 }
 
@@ -1803,12 +1791,8 @@ template <int N_TILE, int NX, int XSUB_KB, int STAGES>
 static cudaError_t launch_wg2(const TensorMap& x, const TensorMap& dy, const Wg2Params& p, dim3 grid, cudaStream_t s) {
     constexpr int smem = STAGES * (NX * XSUB_KB * 1024 + (N_TILE / 64) * 128 * 128) + 1024 + 256;
     static_assert(smem <= 232448, "shared memory");
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(wg2_kernel<N_TILE, NX, XSUB_KB, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static OncePerDevice once;
+    if (const cudaError_t e = allow_smem(once, (const void*)wg2_kernel<N_TILE, NX, XSUB_KB, STAGES>, smem); e != cudaSuccess) return e;
     return klaunch(wg2_kernel<N_TILE, NX, XSUB_KB, STAGES>, grid, NUM_THREADS, smem, s, *(const CUtensorMap*)&x, *(const CUtensorMap*)&dy, p);
 }
 
@@ -1866,12 +1850,8 @@ cudaError_t run_stem_wg(const TensorMap& x_raw, const TensorMap& dy128, int H, i
                         int sms, cudaStream_t s) {
     constexpr int STAGES = 4;
     constexpr int smem = STAGES * (2 * 128 * 128 + STEM_RAW_BYTES) + 1024 + 256;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(stem_wg_kernel<STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static OncePerDevice once;
+    if (const cudaError_t e = allow_smem(once, (const void*)stem_wg_kernel<STAGES>, smem); e != cudaSuccess) return e;
     StemWgParams p{};
     p.W = W; p.Ht = 128 / W; p.tiles_h = H / p.Ht; p.steps = N * p.tiles_h;
     const int ctas = stem_wg_ctas(p.steps, sms);
@@ -1886,12 +1866,8 @@ cudaError_t run_stem_fw(const TensorMap& x_raw, const TensorMap& out_map, int H,
                         float* stat_part, int* err, int sms, cudaStream_t s) {
     constexpr int STAGES = 3;
     constexpr int smem = STAGES * (128 * 128 + STEM_RAW_BYTES) + 64 * 128 + 4 * 2 * EPI_BUF_BYTES + 1024 + 256;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(stem_fw_kernel<STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static OncePerDevice once;
+    if (const cudaError_t e = allow_smem(once, (const void*)stem_fw_kernel<STAGES>, smem); e != cudaSuccess) return e;
     StemFwParams p{};
     p.W = W; p.Ht = 128 / W; p.tiles_h = H / p.Ht; p.tiles = N * p.tiles_h; p.Co = Co; p.epi = relu ? EPI_RELU : 0;
     p.w = (const bf16*)w; p.bias = bias; p.stat_part = stat_part; p.err = err;
