@@ -321,7 +321,7 @@ def main():
                     "kernel_ms_per_step_all_classes": total_ms / kernel_steps, "traffic": traffic_per_launch(name),
                     "timing": f"CUDA events around every launch, separate pass of {kernel_steps} steps with all modules on one stream "
                               "(each event pair brackets one kernel running alone); not part of the timed region of `value`"}
-            if name.startswith("tc_gemm") or name.startswith("igemm_fma"):
+            if name.startswith("tc_gemm") or name.startswith("fma_"):
                 tensor = name.startswith("tc_gemm")
                 ach = st["flops"] / (st["ms"] * 1e-3) / 1e12
                 peak = pk["tensor_burst"] if tensor else FMA_PEAK_TFLOPS

@@ -19,9 +19,10 @@ uint64_t launches() { return g_launches.load(); }
 // ---- per-kernel-class device timing (off by default): every launcher opens a Scope, which counts the
 // launch and, while profiling is on, brackets it with two events on the launching stream.
 static const char* kClassNames[KC_COUNT] = {
-    "igemm_fma_fwd", "igemm_fma_dgrad", "igemm_fma_wgrad", "splitk_reduce", "bias_grad", "relu_fwd", "relu_bwd", "add_fwd",
+    "fma_fwd", "fma_dgrad", "fma_wgrad", "splitk_reduce", "bias_grad", "relu_fwd", "relu_bwd", "add_fwd",
     "copy_accumulate", "maxpool_fwd", "maxpool_bwd", "gap_fwd", "gap_bwd", "bn_fwd_stats", "bn_fwd_apply", "bn_bwd_reduce",
-    "bn_bwd_apply", "softmax_ce", "sgd_update", "tags", "fill", "tc_gemm_fwd", "tc_gemm_dgrad", "tc_gemm_wgrad", "tc_aux"};
+    "bn_bwd_apply", "softmax_ce", "sgd_update", "tags", "fill", "tc_gemm_fwd", "tc_gemm_dgrad", "tc_gemm_wgrad", "tc_aux", "ingest",
+};
 namespace prof {
 struct Rec { int cls; cudaEvent_t a, b; };
 static bool g_on = false;
@@ -1479,7 +1480,7 @@ __global__ void __launch_bounds__(256) zero_k(uint4* p, size_t n16) {
 }
 void zero_fill(void* p, size_t bytes, cudaStream_t s) { klaunch(zero_k, ew_grid(bytes / 16), 256, 0, s, (uint4*)p, bytes / 16); }
 
-// The step's batch and labels into their FIFO slots, one launch.  vec: all four addresses are 16-byte aligned.
+// The step's batch and labels into their FIFO slots, one launch.  vec: both input addresses are 16-byte aligned (labels go word by word).
 __global__ void __launch_bounds__(256) ingest_k(const char* __restrict__ x, char* __restrict__ xd, size_t x_bytes, const int32_t* __restrict__ y, int32_t* __restrict__ yd, int m, bool vec) {
     const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
     const size_t n16 = vec ? x_bytes / 16 : 0;
@@ -1497,6 +1498,7 @@ __global__ void __launch_bounds__(256) ingest_k(const char* __restrict__ x, char
 }
 void ingest(const void* x, void* xd, size_t x_bytes, const int32_t* y, int32_t* yd, int m, cudaStream_t s) {
     const bool vec = (((uintptr_t)x | (uintptr_t)xd) & 15) == 0;
+    Scope sc(KC_INGEST, 0.0, 2.0 * (double)x_bytes + 8.0 * m, s);
     klaunch(ingest_k, ew_grid(vec ? x_bytes / 64 : x_bytes / 2), 256, 0, s, (const char*)x, (char*)xd, x_bytes, y, yd, m, vec);
 }
 

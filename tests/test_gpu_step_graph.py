@@ -212,3 +212,24 @@ def test_module_times_cover_the_iteration():
             if serial:
                 assert ms.sum() < wall, (t, ms, wall)
         ctx.close()
+
+
+def test_every_kernel_of_a_step_is_counted():
+    """Inputs in device memory cost one kernel more than inputs that are copied in from the host: the one that takes them into the FIFO."""
+    import torch
+    from paper_2509_05679_b200 import binding
+    net = nets()["small"]
+    ctx = make_ctx(net, sy.init_params(net.layers, 0))
+    x, y = sy.batch_inputs(net, 0), sy.batch_labels(net, 0)
+    xd, yd = binding.to_device(net.dtype, x), torch.from_numpy(y).cuda()
+    per_step = []
+    for step in (lambda: ctx.step(xd, yd), lambda: ctx.step_host(x, y)):
+        for _ in range(2 * net.K + 2):
+            step()
+            ctx.wait_ingest()
+        before = ctx.stats()[1]
+        step()
+        ctx.wait_ingest()
+        per_step.append(ctx.stats()[1] - before)
+    ctx.close()
+    assert per_step[0] == per_step[1] + 1
