@@ -9,7 +9,8 @@
 //
 // Arithmetic: packed fp32 (fma.rn.f32x2: 65.6 TFLOP/s on a B200 where scalar fma gives 46.7).  The pairs lie along the
 // contraction (channels 2i and 2i + 1) in fc_kernel and along c_in in fw_kernel, so that operands come out of NHWC data as
-// 16-byte vectors without shuffling.  Chains of at most 16 products are added to a compensated (Kahan) running sum, so the rounding error of a long contraction stays at a few ulps.
+// 16-byte vectors without shuffling.  Chains of at most 16 products (fw_kernel: 32 in long sums) are added to a compensated (Kahan) running sum, so the
+// rounding error of a long contraction stays at a few ulps.
 //
 // What bounds them: the FMA pipe (fc_kernel issues 32 packed FMAs for eight 16-byte shared loads, or 16 for six, fw_kernel 16 for four).
 // The implicit-GEMM kernel they replace fetched every operand element by itself with two integer divisions and reached
@@ -106,6 +107,13 @@ __device__ __forceinline__ void kahan(float2& sum, float2& part) {
     sum = t;
 }
 
+// the two lanes of a sum, with what either has lost
+__device__ __forceinline__ float lanes_sum(float2 sum, float2 lost) {
+    const float s = __fadd_rn(sum.x, sum.y), b = __fsub_rn(s, sum.x);
+    const float e = __fadd_rn(__fsub_rn(sum.x, __fsub_rn(s, b)), __fsub_rn(sum.y, b));          // two-sum: sum.x + sum.y = s + e
+    return __fadd_rn(s, __fadd_rn(e, __fadd_rn(lost.x, lost.y)));
+}
+
 struct Yes { static constexpr bool value = true; };
 struct No { static constexpr bool value = false; };
 
@@ -191,11 +199,15 @@ __global__ void __launch_bounds__(512 / PP, fc_ctas<T>(PP)) fc_kernel(const T* _
         const int pw = px & (p.Wt - 1), ph = (px >> p.lw) & (p.Ht - 1), pn = px >> (p.lw + p.lh);
         xb[i] = (uint32_t)(((pn * RH + ph * p.xs) * RW + pw * p.xs) * PITCH);
     }
-    float2 acc[PP][2], comp[PP][2], part[PP][4];
+    // fp32 storage: per channel the sums of its even and of its odd products.  bf16 storage: per pair of channels their sums (0, 1) and what the last
+    // additions lost (2, 3); rounding the two lanes' sum at every flush adds 2.6 % to an error that the rounded result hides, and the other form
+    // spills there (+5 % per step).
+    constexpr bool LANES = sizeof(T) == 4;
+    float2 acc[PP][4], part[PP][4];
 #pragma unroll
     for (int i = 0; i < PP; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) { acc[i][j] = make_float2(0.f, 0.f); comp[i][j] = make_float2(0.f, 0.f); }
+        for (int j = 0; j < 4; ++j) { acc[i][j] = make_float2(0.f, 0.f); part[i][j] = make_float2(0.f, 0.f); }
 
     const int chunks = t1 > t0 ? (p.C + FC_KC - 1) / FC_KC : 0;
     auto fetch = [&](int c, int buf) {
@@ -225,25 +237,31 @@ __global__ void __launch_bounds__(512 / PP, fc_ctas<T>(PP)) fc_kernel(const T* _
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const float2 lo = make_float2(xv.x, xv.y), hi = make_float2(xv.z, xv.w);
-                        if (decltype(first)::value && q == 0) part[i][j] = __fmul2_rn(lo, make_float2(wv[j].x, wv[j].y));
+                        if (!LANES && decltype(first)::value && q == 0) part[i][j] = __fmul2_rn(lo, make_float2(wv[j].x, wv[j].y));
                         else part[i][j] = __ffma2_rn(lo, make_float2(wv[j].x, wv[j].y), part[i][j]);
                         part[i][j] = __ffma2_rn(hi, make_float2(wv[j].z, wv[j].w), part[i][j]);
                     }
                 }
             }
         };
-        auto flush = [&]() {             // Kahan: acc += even + odd part, two channels per instruction
+        auto flush = [&]() {             // Kahan
 #pragma unroll
-            for (int i = 0; i < PP; ++i)
+            for (int i = 0; i < PP; ++i) {
+                if (LANES) {
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    const float2 s = make_float2(part[i][2 * j].x + part[i][2 * j].y, part[i][2 * j + 1].x + part[i][2 * j + 1].y);
-                    const float2 yv = __fadd2_rn(s, make_float2(-comp[i][j].x, -comp[i][j].y));
-                    const float2 t = __fadd2_rn(acc[i][j], yv);
-                    const float2 d = __fadd2_rn(t, make_float2(-acc[i][j].x, -acc[i][j].y));
-                    comp[i][j] = __fadd2_rn(d, make_float2(-yv.x, -yv.y));
-                    acc[i][j] = t;
+                    for (int j = 0; j < 4; ++j) kahan(acc[i][j], part[i][j]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const float2 s = make_float2(part[i][2 * j].x + part[i][2 * j].y, part[i][2 * j + 1].x + part[i][2 * j + 1].y);
+                        const float2 yv = __fadd2_rn(s, make_float2(-acc[i][2 + j].x, -acc[i][2 + j].y));
+                        const float2 t = __fadd2_rn(acc[i][j], yv);
+                        const float2 d = __fadd2_rn(t, make_float2(-acc[i][j].x, -acc[i][j].y));
+                        acc[i][2 + j] = __fadd2_rn(d, make_float2(-yv.x, -yv.y));
+                        acc[i][j] = t;
+                    }
                 }
+            }
         };
         int t = 0;
 #pragma unroll 1
@@ -262,7 +280,8 @@ __global__ void __launch_bounds__(512 / PP, fc_ctas<T>(PP)) fc_kernel(const T* _
         const int wd = wd0 + (px & (p.Wt - 1)), hd = hd0 + ((px >> p.lw) & (p.Ht - 1)), n = n0 + (px >> (p.lw + p.lh));
         valid[i] = n < n_end && hd < p.Hd && wd < p.Wd;
         float (&v)[4] = val[i];
-        v[0] = acc[i][0].x; v[1] = acc[i][0].y; v[2] = acc[i][1].x; v[3] = acc[i][1].y;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = LANES ? lanes_sum(acc[i][j], part[i][j]) : (j & 1 ? acc[i][j >> 1].y : acc[i][j >> 1].x);
         if (!valid[i] || co >= p.Co) continue;
         const size_t o = (((size_t)n * p.Ho + (hd * p.os + p.cls_oph[cls])) * p.Wo + (wd * p.os + p.cls_opw[cls])) * p.Co + co;
 #pragma unroll
@@ -353,13 +372,18 @@ struct FwParams {
 // grid = (splits, c_out blocks x c_in blocks, groups).  Thread = 4 c_out x 8 c_in of one tap, for one slice of every tile's
 // pixels.  dy is kept twice in shared memory ((d, d) pairs: the multiplier of a packed FMA), x as in fc_kernel.  While a tile is used, the
 // next one's x is on its way into the other buffer (fp32: cp.async) and its dy into registers.
-// Compensated sum: a chain of FW_CHAIN products starts at what the running sum lost at its last addition, so that the compensation
-// costs neither registers nor an instruction of its own.  (Chains of 32 lose sqrt(2) more than chains of 16; the error of the whole is
-// that of the sum over the splits, of which no lane of fw_reduce_kernel adds more than 56 one after the other.)
+// Compensated sum: a chain of CHAIN products starts at what the running sum lost at its last addition, so that the compensation
+// costs neither registers nor an instruction of its own.  Chains of 32 (16 take 3 to 4 % of a ResNet-20 step) where a group has FW_LONG or more pixels: the
+// sums over slices and splits in double leave the error below that of the implicit GEMM this replaced, which added its splits in fp32 (rms
+// error against double sums, normal data, of the result's rms: 12288 pixels of 8x8, 64 -> 64 channels 1.06e-7 against 1.50e-7, of 32x32, 16 -> 16
+// 1.08e-7 against 1.47e-7).  Shorter sums were better there (4096 pixels: 1.12e-7 against 1.13e-7 with chains of 32; 768: 8.5e-8, 1.06e-7) and get chains of 16
+// (768: 8.5e-8).  bf16 storage: chains of 32, sums over slices and splits in fp32 (its inputs are rounded to 4e-3).
 // part: [group][block][split][16 c_out][taps][8 * G c_in]
-constexpr int FW_CHAIN = 32;
+template <typename T> struct FwSum { typedef float type; };
+template <> struct FwSum<float> { typedef double type; };
+constexpr long FW_LONG = 6144;
 constexpr int FW_DYV = 4;                                    // float4s of dy per thread and tile: 128 pixels x 4 / 160 threads
-template <typename T, int XS, int G, int RUN>
+template <typename T, int XS, int G, int RUN, int CHAIN>
 __global__ void __launch_bounds__(FW_THREADS, 3) fw_kernel(const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ part_out,
                                                            const __grid_constant__ FwParams p) {
     extern __shared__ __align__(16) float fsm[];
@@ -420,9 +444,9 @@ __global__ void __launch_bounds__(FW_THREADS, 3) fw_kernel(const T* __restrict__
         if (active) {
             const float* const xt = fsm + buf * p.x_floats + xoff;
 #pragma unroll 1
-            for (int r = 0; r < p.pps; r += FW_CHAIN) {
+            for (int r = 0; r < p.pps; r += CHAIN) {
 #pragma unroll
-                for (int rr = 0; rr < FW_CHAIN; rr += RUN) {
+                for (int rr = 0; rr < CHAIN; rr += RUN) {
                     const int px = slice * p.pps + r + rr;
                     if (rr > 0 && r + rr >= p.pps) break;
                     const int pw = px & (p.Wt - 1), ph = (px >> p.lw) & (p.Ht - 1), pn = px >> (p.lw + p.lh);
@@ -461,20 +485,22 @@ __global__ void __launch_bounds__(FW_THREADS, 3) fw_kernel(const T* __restrict__
     __syncthreads();
     float* out = part_out + (((size_t)grp * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * nout;
     for (int i = tid; i < nout; i += FW_THREADS) {
-        float s = 0.f;
+        typename FwSum<T>::type s = 0;
         for (int k = 0; k < p.nslices; ++k) s += red[(size_t)k * nout + i];
-        out[i] = s;
+        out[i] = (float)s;
     }
 }
 
-// dW[c_out][tap][c_in] = sum over the splits (at most 444): 8 lanes per element take every 8th split, eight loads in flight each, then a fixed tree.
+// dW[c_out][tap][c_in] = sum over the splits (at most 444): 8 lanes per element take every 8th split, eight loads in flight each, then a
+// fixed tree.  S: what they are added in.
+template <typename S>
 __global__ void __launch_bounds__(256) fw_reduce_kernel(const float* __restrict__ part, float* __restrict__ dw, int splits, int nout, int ntaps, int cw, int ci_blocks,
                                                         int C, int Co, size_t w_group, bool accum) {
-    __shared__ float sh[8][33];
+    __shared__ S sh[8][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int e = blockIdx.x * 32 + tx, blk = blockIdx.y, grp = blockIdx.z;
     const float* src = part + ((size_t)grp * gridDim.y + blk) * splits * nout + e;
-    float s = 0.f;
+    S s = 0;
     if (e < nout) {
         int k = ty;
         for (; k + 56 < splits; k += 64) {
@@ -493,7 +519,7 @@ __global__ void __launch_bounds__(256) fw_reduce_kernel(const float* __restrict_
     const int co = (blk / ci_blocks) * FW_CO + e / (ntaps * cw), tap = e / cw % ntaps, ci = (blk % ci_blocks) * FW_CI + e % cw;
     if (co >= Co || ci >= C) return;
     float* d = dw + (size_t)grp * w_group + ((size_t)co * ntaps + tap) * C + ci;
-    *d = accum ? *d + s : s;
+    *d = accum ? *d + (float)s : (float)s;
 }
 
 int ilog2(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
@@ -654,11 +680,16 @@ bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_
   }
     return false;
 }
+template <typename T, int XS, int G, int RUN, int CHAIN>
+void launch_fw_chain(const void* x, const void* dy, float* ws, const FwParams& p, int groups, size_t smem, cudaStream_t s) {
+    static OncePerDevice once;
+    allow_smem(once, (const void*)fw_kernel<T, XS, G, RUN, CHAIN>, (int)FC_SMEM_MAX);
+    klaunch(fw_kernel<T, XS, G, RUN, CHAIN>, dim3(p.splits, p.ci_blocks * ((p.Co + FW_CO - 1) / FW_CO), groups), FW_THREADS, smem, s, (const T*)x, (const T*)dy, ws, p);
+}
 template <typename T, int XS, int G, int RUN>
 void launch_fw(const void* x, const void* dy, float* ws, const FwParams& p, int groups, size_t smem, cudaStream_t s) {
-    static OncePerDevice once;
-    allow_smem(once, (const void*)fw_kernel<T, XS, G, RUN>, (int)FC_SMEM_MAX);
-    klaunch(fw_kernel<T, XS, G, RUN>, dim3(p.splits, p.ci_blocks * ((p.Co + FW_CO - 1) / FW_CO), groups), FW_THREADS, smem, s, (const T*)x, (const T*)dy, ws, p);
+    if (sizeof(T) == 4 && (long)p.ngroup * p.Ho * p.Wo < FW_LONG) launch_fw_chain<T, XS, G, RUN, 16>(x, dy, ws, p, groups, smem, s);
+    else launch_fw_chain<T, XS, G, RUN, 32>(x, dy, ws, p, groups, smem, s);
 }
 template <typename T, int XS, int G>
 void dispatch_fw_run(const void* x, const void* dy, float* ws, const FwParams& p, int run, int groups, size_t smem, cudaStream_t s) {
@@ -718,7 +749,9 @@ bool fconv_wgrad(int dt, const void* x, const void* dy, float* dw, float* ws, co
         if (dt) dispatch_fw<bf16>(x, dy, ws, p, xs, G, run, groups, smem, s); else dispatch_fw<float>(x, dy, ws, p, xs, G, run, groups, smem, s);
     }
     Scope sc(KC_SPLITK, 0.0, 4.0 * groups * (p.splits + 1) * blocks * nout, s);
-    klaunch(fw_reduce_kernel, dim3((nout + 31) / 32, blocks, groups), 256, 0, s, ws, dw, p.splits, nout, p.ntaps, 8 * G, p.ci_blocks, g.C, g.Co, w_group, accum);
+    const dim3 rgrid((nout + 31) / 32, blocks, groups);
+    if (dt) klaunch(fw_reduce_kernel<FwSum<bf16>::type>, rgrid, 256, 0, s, ws, dw, p.splits, nout, p.ntaps, 8 * G, p.ci_blocks, g.C, g.Co, w_group, accum);
+    else klaunch(fw_reduce_kernel<FwSum<float>::type>, rgrid, 256, 0, s, ws, dw, p.splits, nout, p.ntaps, 8 * G, p.ci_blocks, g.C, g.Co, w_group, accum);
     return true;
 }
 

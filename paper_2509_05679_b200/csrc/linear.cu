@@ -76,16 +76,23 @@ __device__ __forceinline__ LinArgs of_group(const LinArgs& in, bool fwd) {
 
 enum { L_FWD, L_DX, L_DW };
 
+// What a CTA hands on of its part of a contraction.  fp32 storage: both lanes' compensated sums together, in double, so that neither the lanes nor the
+// split cost precision (with parts rounded to fp32 the error of 512 samples through 500 -> 300 was 9 % above that of an unsplit sum).  bf16 storage: fp32, the
+// lanes added at every flush; the rounded result hides the difference, and the sums in double take 3 % of a small network's step.
+template <typename T> struct Part { typedef float type; };
+template <> struct Part<float> { typedef double type; };
+
 // One 32 x 64 tile over the contraction range [k0, k1).  Operands in shared memory as [row][contraction], double buffered; the next
 // chunk travels in registers while this one is used.
 template <typename T, int MODE>
-__device__ __forceinline__ void tile_product(const LinArgs& a, int row0, int col0, int k0, int k1, float* sm, float (&out)[4][4], float* bias_sum) {
+__device__ __forceinline__ void tile_product(const LinArgs& a, int row0, int col0, int k0, int k1, float* sm, typename Part<T>::type (&out)[4][4], float* bias_sum) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane & 7, cg = lane >> 3;
-    float2 acc[4][2], comp[4][2], part[4][4];
+    constexpr bool LANES = sizeof(T) == 4;
+    float2 acc[4][4], part[4][4];            // LANES: per output even and odd products; else per pair of outputs their sums (0, 1), what these have lost (2, 3)
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) acc[i][j] = comp[i][j] = make_float2(0.f, 0.f);
+        for (int j = 0; j < 4; ++j) acc[i][j] = part[i][j] = make_float2(0.f, 0.f);
     float4 ra[2], rb[4];
     const T* const X = (const T*)a.x; const T* const W = (const T*)a.w; const T* const DY = (const T*)a.dy; const T* const Y = (const T*)a.y;
     // column n of the tile sits in row (n / 16) * 16 + (n % 4) * 4 + (n % 16) / 4 of the B tile: a warp's four channel groups read neighbours
@@ -157,22 +164,34 @@ __device__ __forceinline__ void tile_product(const LinArgs& a, int row0, int col
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const float2 lo = make_float2(xv.x, xv.y), hi = make_float2(xv.z, xv.w);
-                    part[i][j] = q == 0 ? __fmul2_rn(lo, make_float2(wv[j].x, wv[j].y)) : __ffma2_rn(lo, make_float2(wv[j].x, wv[j].y), part[i][j]);
+                    if (!LANES && q == 0) part[i][j] = __fmul2_rn(lo, make_float2(wv[j].x, wv[j].y));
+                    else part[i][j] = __ffma2_rn(lo, make_float2(wv[j].x, wv[j].y), part[i][j]);
                     part[i][j] = __ffma2_rn(hi, make_float2(wv[j].z, wv[j].w), part[i][j]);
                 }
             }
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i) {                // Kahan
+            if (LANES) {
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const float2 s = make_float2(part[i][2 * j].x + part[i][2 * j].y, part[i][2 * j + 1].x + part[i][2 * j + 1].y);
-                const float2 yv = __fadd2_rn(s, make_float2(-comp[i][j].x, -comp[i][j].y));
-                const float2 t = __fadd2_rn(acc[i][j], yv);
-                const float2 d = __fadd2_rn(t, make_float2(-acc[i][j].x, -acc[i][j].y));
-                comp[i][j] = __fadd2_rn(d, make_float2(-yv.x, -yv.y));
-                acc[i][j] = t;
+                for (int j = 0; j < 4; ++j) {        // the next chain starts at what the sum lost
+                    const float2 t = __fadd2_rn(acc[i][j], part[i][j]);
+                    const float2 d = __fadd2_rn(t, make_float2(-acc[i][j].x, -acc[i][j].y));
+                    part[i][j] = __fadd2_rn(part[i][j], make_float2(-d.x, -d.y));
+                    acc[i][j] = t;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const float2 s = make_float2(part[i][2 * j].x + part[i][2 * j].y, part[i][2 * j + 1].x + part[i][2 * j + 1].y);
+                    const float2 yv = __fadd2_rn(s, make_float2(-acc[i][2 + j].x, -acc[i][2 + j].y));
+                    const float2 t = __fadd2_rn(acc[i][j], yv);
+                    const float2 d = __fadd2_rn(t, make_float2(-acc[i][j].x, -acc[i][j].y));
+                    acc[i][2 + j] = __fadd2_rn(d, make_float2(-yv.x, -yv.y));
+                    acc[i][j] = t;
+                }
             }
+        }
         if (MODE == L_DW && bias_sum && tid < LM) {
             float s = 0.f;
 #pragma unroll
@@ -182,16 +201,29 @@ __device__ __forceinline__ void tile_product(const LinArgs& a, int row0, int col
     }
     if (MODE == L_DW && bias_sum) *bias_sum = bsum;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) { out[i][0] = acc[i][0].x; out[i][1] = acc[i][0].y; out[i][2] = acc[i][1].x; out[i][3] = acc[i][1].y; }
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (LANES) out[i][j] = (typename Part<T>::type)(((double)acc[i][j].x + (double)acc[i][j].y) + ((double)part[i][j].x + (double)part[i][j].y));    // part: what the lanes have lost
+            else out[i][j] = j & 1 ? acc[i][j >> 1].y : acc[i][j >> 1].x;
+        }
 }
 
 __device__ __forceinline__ uint32_t ctarank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
 __device__ __forceinline__ void cluster_sync() { asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ float4 ld_cluster(uint32_t local, uint32_t rank) {
-    uint32_t r; float4 v;
+__device__ __forceinline__ void st_part(float* d, const float (&v)[4]) { *(float4*)d = make_float4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ void st_part(double* d, const double (&v)[4]) { *(double2*)d = make_double2(v[0], v[1]); *(double2*)(d + 2) = make_double2(v[2], v[3]); }
+// four consecutive parts of another CTA of the cluster
+__device__ __forceinline__ void ld_cluster(uint32_t local, uint32_t rank, float (&v)[4]) {
+    uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(r) : "memory");
-    return v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(r) : "memory");
+}
+__device__ __forceinline__ void ld_cluster(uint32_t local, uint32_t rank, double (&v)[4]) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(r) : "memory");
+    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v[2]), "=d"(v[3]) : "r"(r + 16) : "memory");
 }
 
 // Four consecutive outputs of one row: bias, ReLU, accumulation, store (T, or fp32 with EPI_OUT_F32).
@@ -216,25 +248,41 @@ __device__ __forceinline__ void emit(const LinArgs& a, int r, int c, int rows, i
 
 // A tile that the cluster's CTAs have each done a part of: CTA `rank` adds rows rank, rank + split, ... over the CTAs in rank order.
 template <typename T>
-__device__ __forceinline__ void join_tile(const LinArgs& a, int row0, int col0, int rows, int cols, float (&v)[4][4], const float* bias, float* sm) {
+__device__ __forceinline__ void join_tile(const LinArgs& a, int row0, int col0, int rows, int cols, typename Part<T>::type (&v)[4][4], const float* bias, float* sm) {
+    typedef typename Part<T>::type P;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane & 7, cg = lane >> 3;
     if (a.split == 1) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) emit<T>(a, row0 + g + 8 * i, col0 + warp * 16 + 4 * cg, rows, cols, v[i], bias);
+        for (int i = 0; i < 4; ++i) {
+            float f[4] = {(float)v[i][0], (float)v[i][1], (float)v[i][2], (float)v[i][3]};
+            emit<T>(a, row0 + g + 8 * i, col0 + warp * 16 + 4 * cg, rows, cols, f, bias);
+        }
         return;
     }
     __syncthreads();                     // the operand buffers are no longer read
-    constexpr int TP = LN + 4;
+    constexpr int TP = LN + 16 / (int)sizeof(P);
+    static_assert(LM * TP * sizeof(P) <= 2 * (LM + LN) * LP * sizeof(float), "the parts reuse the operand buffers");
+    P* const part = (P*)sm;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) *(float4*)(sm + (g + 8 * i) * TP + warp * 16 + 4 * cg) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+    for (int i = 0; i < 4; ++i) st_part(part + (g + 8 * i) * TP + warp * 16 + 4 * cg, v[i]);
     cluster_sync();
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm);
     const int rank = (int)ctarank();
     for (int e = tid; e < LM * LN / 4 / a.split; e += LT) {
         const int r = (e / (LN / 4)) * a.split + rank, c = 4 * (e % (LN / 4));
-        float s[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int q = 0; q < a.split; ++q) { const float4 t = ld_cluster(base + (uint32_t)(r * TP + c) * 4u, q); s[0] += t.x; s[1] += t.y; s[2] += t.z; s[3] += t.w; }
-        emit<T>(a, row0 + r, col0 + c, rows, cols, s, bias);
+        const uint32_t at = base + (uint32_t)((r * TP + c) * sizeof(P));
+        P s[4] = {0, 0, 0, 0};
+        for (int q = 0; q < a.split; q += 2) {       // split is a power of two; two CTAs' parts in flight
+            P t[2][4];
+            ld_cluster(at, q, t[0]);
+            ld_cluster(at, q + 1, t[1]);
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) s[j] += t[u][j];
+        }
+        float f[4] = {(float)s[0], (float)s[1], (float)s[2], (float)s[3]};
+        emit<T>(a, row0 + r, col0 + c, rows, cols, f, bias);
     }
     cluster_sync();                      // no CTA leaves while another reads its tile
 }
@@ -252,7 +300,7 @@ __global__ void __launch_bounds__(LT) lin_fwd_kernel(const LinArgs args) {
     const int tile = blockIdx.x / a.split, rank = blockIdx.x % a.split;
     const int tiles_n = (a.N + LN - 1) / LN, row0 = tile / tiles_n * LM, col0 = tile % tiles_n * LN;
     int k0, k1; my_range(a.K, a.split, rank, k0, k1);
-    float v[4][4];
+    typename Part<T>::type v[4][4];
     tile_product<T, L_FWD>(a, row0, col0, k0, k1, sm, v, nullptr);
     join_tile<T>(a, row0, col0, a.M, a.N, v, a.bias, sm);
 }
@@ -263,7 +311,7 @@ __global__ void __launch_bounds__(LT) lin_bwd_kernel(const LinArgs args) {
     const LinArgs a = of_group<T>(args, false);
     __shared__ __align__(16) float sm[2 * (LM + LN) * LP];
     const int cl = blockIdx.x / a.split, rank = blockIdx.x % a.split;
-    float v[4][4];
+    typename Part<T>::type v[4][4];
     if (cl < a.dx_clusters) {
         const int row0 = cl / a.dx_tiles_n * LM, col0 = cl % a.dx_tiles_n * LN;
         int k0, k1; my_range(a.N, a.split, rank, k0, k1);
@@ -292,26 +340,26 @@ __global__ void __launch_bounds__(LT) lin_bwd_kernel(const LinArgs args) {
         if (r >= a.N || c >= a.K) continue;
         float* const d = dw + (size_t)r * a.K + c;
         if ((a.K & 3) == 0 && (((uintptr_t)dw) & 15) == 0) {
-            float4 o = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+            float4 o = make_float4((float)v[i][0], (float)v[i][1], (float)v[i][2], (float)v[i][3]);
             if (accum) { const float4 old = *(const float4*)d; o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w; }
             *(float4*)d = o;
         } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) if (c + j < a.K) d[j] = accum ? d[j] + v[i][j] : v[i][j];
+            for (int j = 0; j < 4; ++j) if (c + j < a.K) d[j] = accum ? d[j] + (float)v[i][j] : (float)v[i][j];
         }
     }
     if (db && col0 == 0 && tid < LM && row0 + tid < a.N) db[row0 + tid] = accum ? db[row0 + tid] + bs : bs;
 }
 
 // dW and db from the partial matrices: 32 elements per CTA, eight threads of different splits per element, four loads in flight each, then their
-// sums in order.
+// sums in order, in double.
 __global__ void __launch_bounds__(256) lin_reduce_kernel(const float* __restrict__ part, float* __restrict__ dw, float* __restrict__ db, int splits, size_t nk, int N,
                                                          size_t g_group, bool accum) {
-    __shared__ float sh[8][32];
+    __shared__ double sh[8][32];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const size_t e = (size_t)blockIdx.x * 32 + tx, n = nk + N;
     const float* const src = part + blockIdx.y * (splits * n) + e;
-    float s = 0.f;
+    double s = 0.0;
     if (e < n) {
         int k = ty;
         for (; k + 24 < splits; k += 32) {
@@ -319,9 +367,9 @@ __global__ void __launch_bounds__(256) lin_reduce_kernel(const float* __restrict
 #pragma unroll
             for (int u = 0; u < 4; ++u) v[u] = src[(size_t)(k + 8 * u) * n];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) s += v[u];
+            for (int u = 0; u < 4; ++u) s += (double)v[u];
         }
-        for (; k < splits; k += 8) s += src[(size_t)k * n];
+        for (; k < splits; k += 8) s += (double)src[(size_t)k * n];
     }
     sh[ty][tx] = s;
     __syncthreads();
@@ -329,7 +377,7 @@ __global__ void __launch_bounds__(256) lin_reduce_kernel(const float* __restrict
 #pragma unroll
     for (int k = 1; k < 8; ++k) s += sh[k][tx];
     float* const d = (e < nk ? dw + e : db + (e - nk)) + blockIdx.y * g_group;
-    *d = accum ? *d + s : s;
+    *d = accum ? *d + (float)s : (float)s;
 }
 
 // CTAs per cluster: as many as fill the device once (148 SMs, four CTAs each take the latency), a power of two up to 8 (the portable
