@@ -340,6 +340,8 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             long ptiles = (long)(g.Wo / wt) * (g.Ho / ht) * ((g.N + nt - 1) / nt);
             // a short contraction and many tiles: one CTA per tile goes through all of it and writes the gradient itself (no partial matrices, no
             // reduction); the widest tile that still gives half of the launch's SMs something to do
+            // (four modules of 1024-wide layers, us per step with splits and so: 161, 118 at 4 steps of 64 samples; 187, 132 at 8; 244, 182 at 24; still 271, 207
+            // at 32 and 373, 313 at 64.  ResNet-18-shaped, 2 x 9 samples: 394, 378; 4 x 16: 648, 630; 4 x 64, which has few such layers: 1493, 1486)
             const bool direct = ptiles <= 24 && (row_blocks + 1) / 2 * (g.Co / 64) >= 64;
             if (direct) while (o.n_tile_w > 64 && (row_blocks + 1) / 2 * (g.Co / o.n_tile_w) < ctx->grid_sms / 2) o.n_tile_w /= 2;
             int tiles = ((row_blocks + 1) / 2) * (g.Co / o.n_tile_w);
