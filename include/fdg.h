@@ -92,7 +92,7 @@ typedef struct {
     int32_t serial;            /* 1: run every module on one stream (results are bit-identical
                                   to the concurrent mode when both contexts have the same
                                   grid_sms; used to test the event wiring)                      */
-    int32_t kernel_path;       /* 0: tensor-core kernels where shapes allow (bf16 only), the 256-column
+    int32_t kernel_path;       /* 0: tensor-core kernels where shapes allow, the 256-column
                                      tile (and the 128-column tile of 3x3 stride-1 layers on 16x16 images) as
                                      pairs of CTAs on two SMs (tcgen05 cta_group::2);
                                   1: plain FMA kernels only;
@@ -113,7 +113,7 @@ typedef struct {
                                   "weight_matrix": P_ij = alpha on the edges of the model-group graph, 1 - kappa_i alpha on
                                   the diagonal); every row must sum to 1.  The library then keeps one weight replica
                                   w^_{s,k} per worker s and module k, runs every layer once per worker on that
-                                  worker's replica (plain FMA kernels: kernel_path is taken as 1), computes each
+                                  worker's replica (without the tcgen05 kernels), computes each
                                   worker's own gradient with scale 1/per_worker_batch, and updates
                                   u_{s,k} = w^_{s,k} - lr g_{s,k},  w^_{s,k}(t+1) = sum_r P_sr u_{r,k}  (Eq. "dl_update").
                                   At most 32 workers.  The matrix is copied.                                     */

@@ -1,6 +1,6 @@
-// FMA convolutions (CUDA cores, fp32 arithmetic, fp32 or bf16 storage) for the layers the tensor-core kernels do not take:
-// the whole fp32 path (TF32 would break its 1e-5 tolerance) and, with bf16 storage, channel counts that are no multiple of
-// 64 (the paper's ResNet-20 has 16 and 32).  3x3 and 1x1, stride 1 and 2, any channel counts, any image size.
+// FMA convolutions (CUDA cores, fp32 arithmetic, fp32 or bf16 storage) for the layers the tensor-core kernels do not take: channel counts that
+// are no multiple of 16 (the first layer's 3 among them), all of them with kernel_path 1.  3x3 and 1x1, stride 1 and 2, any channel counts, any image
+// size.  The tiles, the partial matrices of a weight gradient and their reduction are shared with mconv.cu.
 //
 //   fc_kernel : forward and input gradient.  A CTA computes 128 pixels x 16 output channels: the input region of its
 //               pixels (halo included) is fetched ONCE per 16-channel chunk and every filter tap reads it from shared memory.
@@ -15,6 +15,7 @@
 // What bounds them: the FMA pipe (fc_kernel issues 32 packed FMAs for eight 16-byte shared loads, or 16 for six, fw_kernel 16 for four).
 // The implicit-GEMM kernel they replace fetched every operand element by itself with two integer divisions and reached
 // 2.5-9 TFLOP/s on the ResNet-20 layers.
+#include "fconv.h"
 #include "kernels.h"
 #include "launch.h"
 
@@ -26,23 +27,9 @@ typedef __nv_bfloat16 bf16;
 
 namespace {
 
-constexpr int FC_PIX = 128;              // 4 rows of 32 pixels x 16 output channels; a thread has PP = 4 or 2 pixels x 4 channels: 4 or 8 warps
-constexpr int FC_CO = 16;
-constexpr int FC_KC = 16;                // channels per chunk
-constexpr int PITCH = 20;                // floats per pixel (or weight row) in shared memory: 16 + 4, so that the eight 16-byte reads
-                                         // of neighbouring pixels fall into different banks
+// fc_kernel: 4 rows of 32 pixels x 16 output channels; a thread has PP = 4 or 2 pixels x 4 channels: 4 or 8 warps
 constexpr int FW_THREADS = 160;          // 9 taps x 2 groups of 8 c_in x 4 groups of 4 c_out x 2 pixel slices = 144, in five warps: three CTAs put
                                          // four warps on each scheduler and leave 128 registers a thread (nine warps, two CTAs: 96, and spills)
-constexpr int FW_CO = 16, FW_CI = 16;
-constexpr int FW_CTAS = 3 * 148;
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
-    const int n = valid ? 16 : 0;        // 0: the 16 bytes are zero-filled
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 __device__ __forceinline__ float to_f(float v) { return v; }
 __device__ __forceinline__ float to_f(bf16 v) { return __bfloat162float(v); }
@@ -95,18 +82,6 @@ __device__ __forceinline__ void load_region(const bool VEC, const T* __restrict_
     }
 }
 
-template <typename T> __device__ __forceinline__ float stored(float v);
-template <> __device__ __forceinline__ float stored<float>(float v) { return v; }
-template <> __device__ __forceinline__ float stored<bf16>(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
-
-// sum += part, compensated: part, which started at what the sum lost last time, becomes what it loses this time
-__device__ __forceinline__ void kahan(float2& sum, float2& part) {
-    const float2 t = __fadd2_rn(sum, part);
-    const float2 d = __fadd2_rn(t, make_float2(-sum.x, -sum.y));
-    part = __fadd2_rn(part, make_float2(-d.x, -d.y));
-    sum = t;
-}
-
 // the two lanes of a sum, with what either has lost
 __device__ __forceinline__ float lanes_sum(float2 sum, float2 lost) {
     const float s = __fadd_rn(sum.x, sum.y), b = __fsub_rn(s, sum.x);
@@ -116,22 +91,6 @@ __device__ __forceinline__ float lanes_sum(float2 sum, float2 lost) {
 
 struct Yes { static constexpr bool value = true; };
 struct No { static constexpr bool value = false; };
-
-struct FcParams {
-    int H, W, C;                         // input tensor (the error gradient in the backward direction)
-    int Ho, Wo, Co;                      // output tensor
-    int Hd, Wd, os, xs;                  // destination grid of a class, its stride in the output, stride of the input per destination pixel
-    int ngroup;                          // images per group (a group has its own weights)
-    int ncls, cls_tap0[5], cls_oph[4], cls_opw[4];       // output parity classes (one, unless this is a stride-2 input gradient)
-    int cls_h0[4], cls_w0[4], cls_rh[4], cls_rw[4];      // per class: offset and size of the input region of a tile
-    int toff[9], wtap[9];                // per tap: offset inside the region (floats), index of its weights
-    int Wt, Ht, Nt, lw, lh, tiles_w, tiles_h;            // tile = Wt x Ht x Nt = 128 destination pixels (powers of two)
-    int taps;                            // taps of the weight tensor
-    int back;                            // 0: B[n][k] = W[n][tap][k]; 1: B[n][k] = W[k][tap][n]
-    size_t w_group, b_group;             // elements between the groups' weights / biases
-    int epi;
-    int x_floats, w_floats, buffers;     // shared memory of one buffer
-};
 
 // 16 output channels x up to 16 input channels of every tap of the class into dst[tap][row][PITCH]; channel n sits in row
 // (n % 4) * 4 + n / 4, so that the four channel groups of a warp read neighbouring rows.
@@ -358,17 +317,6 @@ __global__ void __launch_bounds__(512 / PP, fc_ctas<T>(PP)) fc_kernel(const T* _
     }
 }
 
-struct FwParams {
-    int H, W, C, Ho, Wo, Co;
-    int step;                            // pixels of x between neighbours of the region (the stride for 1x1 layers, else 1)
-    int pad, hstep;                      // region origin = tile origin * hstep - pad
-    int RH, RW, ntaps, toff[9];          // region of a tile; per tap: offset inside it (floats)
-    int Wt, Ht, Nt, lw, lh, tiles_w, tiles_h, tiles;     // tile = Wt x Ht x Nt output pixels (powers of two)
-    int ngroup, splits, ci_blocks;
-    int nslices, pps;                    // pixel slices of a tile, pixels per slice
-    int x_floats;
-};
-
 // grid = (splits, c_out blocks x c_in blocks, groups).  Thread = 4 c_out x 8 c_in of one tap, for one slice of every tile's
 // pixels.  dy is kept twice in shared memory ((d, d) pairs: the multiplier of a packed FMA), x as in fc_kernel.  While a tile is used, the
 // next one's x is on its way into the other buffer (fp32: cp.async) and its dy into registers.
@@ -522,10 +470,12 @@ __global__ void __launch_bounds__(256) fw_reduce_kernel(const float* __restrict_
     *d = accum ? *d + (float)s : (float)s;
 }
 
-int ilog2(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
+}  // namespace
+
+static int ilog2(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
 
 // The largest power of two <= cap that wastes least when it tiles `n`.
-int best_tile(int n, int cap) {
+static int best_tile(int n, int cap) {
     int best = 1; long best_cover = n;
     for (int t = 2; t <= cap; t *= 2) {
         const long cover = (long)((n + t - 1) / t) * t;
@@ -535,13 +485,13 @@ int best_tile(int n, int cap) {
     return best;
 }
 
-struct Tile { int Wt, Ht, Nt; };
+namespace { struct Tile { int Wt, Ht, Nt; }; }
 // Tile of `pixels` pixels for n images of H x W per group; a tile needs R x R windows, `step` apart, of what it reads.
 // First choice: the exact cover of an image, as best_tile has it.  Images that no power of two covers (7x7, 5x7) leave it tiles of single pixels from
 // 128 images: half empty for the images of one worker, nine pixels read for one.  Where another tile costs less than three quarters
 // (pixels computed, used or not, plus a quarter per pixel read), that one (step times of 24-channel networks on 4 workers x 48: 7x7 fp32 590 us
 // with the exact cover, 290 so; 489 with the implicit GEMM that these kernels replaced; 5x7 511, 291, 483).
-Tile pick_tile(int H, int W, int n, int pixels, int R, int step) {
+static Tile pick_tile(int H, int W, int n, int pixels, int R, int step) {
     auto cost = [&](int wt, int ht) {
         const int nt = pixels / (wt * ht);
         const double tiles = (double)((W + wt - 1) / wt) * ((H + ht - 1) / ht) * ((n + nt - 1) / nt);
@@ -558,8 +508,6 @@ Tile pick_tile(int H, int W, int n, int pixels, int R, int step) {
     t.Nt = pixels / (t.Wt * t.Ht);
     return t;
 }
-
-constexpr size_t FC_SMEM_MAX = 224 * 1024;
 
 // Geometry of a forward (back == 0) or input-gradient launch over `groups` groups of g.N / groups images; false: not covered.
 bool plan_fc(const ConvGeom& g, int groups, bool back, FcParams& p) {
@@ -615,6 +563,8 @@ bool plan_fc(const ConvGeom& g, int groups, bool back, FcParams& p) {
     return one <= FC_SMEM_MAX;
 }
 
+namespace {
+
 template <typename T, int NQ, bool VEC, int PP>
 void launch_fc_pp(const void* x, const void* w, const float* bias, void* y, float* stat, const FcParams& p, int groups, cudaStream_t s) {
     const size_t smem = (size_t)p.buffers * (p.x_floats + p.w_floats) * sizeof(float);
@@ -641,6 +591,8 @@ void dispatch_fc(const void* x, const void* w, const float* bias, void* y, float
     if (p.C <= 4) { if (vec) launch_fc<T, 1, true>(x, w, bias, y, stat, p, groups, s); else launch_fc<T, 1, false>(x, w, bias, y, stat, p, groups, s); }
     else { if (vec) launch_fc<T, 4, true>(x, w, bias, y, stat, p, groups, s); else launch_fc<T, 4, false>(x, w, bias, y, stat, p, groups, s); }
 }
+
+}  // namespace
 
 // Weight gradient: 128 pixels per tile (64 for 3x3 stride 2, whose input region is four times its output).
 bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_t& smem) {
@@ -680,6 +632,8 @@ bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_
   }
     return false;
 }
+namespace {
+
 template <typename T, int XS, int G, int RUN, int CHAIN>
 void launch_fw_chain(const void* x, const void* dy, float* ws, const FwParams& p, int groups, size_t smem, cudaStream_t s) {
     static OncePerDevice once;
@@ -710,21 +664,23 @@ bool fconv_supported(const ConvGeom& g) {
     return plan_fc(g, 1, false, p) && plan_fc(g, 1, true, p) && plan_fw(g, 1, q, G, run, smem);
 }
 bool fconv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
-                   float* stat, cudaStream_t s) {
+                   float* stat, const Packed& pk, cudaStream_t s) {
     FcParams p;
     if (!plan_fc(g, groups, false, p)) return false;
     p.epi = epi; p.w_group = w_group; p.b_group = b_group;
     const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
     Scope sc(KC_FMA_FWD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + g.Co * K + rows * g.Co), s);
+    if (pk.data && mconv_forward(dt, x, pk.data, bias, y, stat, g, epi, groups, b_group, pk.group, s)) return true;
     if (dt) dispatch_fc<bf16>(x, w, bias, y, stat, p, groups, s); else dispatch_fc<float>(x, w, bias, y, stat, p, groups, s);
     return true;
 }
-bool fconv_dgrad(int dt, const void* dy, const void* w, void* dx, const ConvGeom& g, int epi, int groups, size_t w_group, cudaStream_t s) {
+bool fconv_dgrad(int dt, const void* dy, const void* w, void* dx, const ConvGeom& g, int epi, int groups, size_t w_group, const Packed& pk, cudaStream_t s) {
     FcParams p;
     if (!plan_fc(g, groups, true, p)) return false;
     p.epi = epi; p.w_group = w_group;
     const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
     Scope sc(KC_FMA_DGRAD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + g.Co * K + rows * g.Co), s);
+    if (pk.data && mconv_dgrad(dt, dy, pk.data, dx, g, epi, groups, pk.group, s)) return true;
     if (dt) dispatch_fc<bf16>(dy, w, nullptr, dx, nullptr, p, groups, s); else dispatch_fc<float>(dy, w, nullptr, dx, nullptr, p, groups, s);
     return true;
 }
@@ -739,14 +695,16 @@ size_t fconv_wgrad_workspace_elems(const ConvGeom& g, int groups) {
     const int blocks = p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO) * groups;
     return (size_t)blocks * (FW_CTAS > blocks ? FW_CTAS / blocks : 1) * FW_CO * p.ntaps * 8 * G;
 }
-bool fconv_wgrad(int dt, const void* x, const void* dy, float* dw, float* ws, const ConvGeom& g, int groups, size_t w_group, bool accum, cudaStream_t s) {
+bool fconv_wgrad(int dt, const void* x, const void* dy, float* dw, float* ws, const ConvGeom& g, int groups, size_t w_group, bool accum, bool tensor, cudaStream_t s) {
     FwParams p; int G, run; size_t smem;
     if (!plan_fw(g, groups, p, G, run, smem)) return false;
     const int xs = g.R == 1 ? 1 : g.stride, blocks = p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO), nout = FW_CO * p.ntaps * 8 * G;
     const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
     {
         Scope sc(KC_FMA_WGRAD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + rows * g.Co) + 4.0 * K * g.Co, s);
-        if (dt) dispatch_fw<bf16>(x, dy, ws, p, xs, G, run, groups, smem, s); else dispatch_fw<float>(x, dy, ws, p, xs, G, run, groups, smem, s);
+        const int splits = tensor ? mconv_wgrad(dt, x, dy, ws, g, groups, s) : 0;
+        if (splits) p.splits = splits;
+        else if (dt) dispatch_fw<bf16>(x, dy, ws, p, xs, G, run, groups, smem, s); else dispatch_fw<float>(x, dy, ws, p, xs, G, run, groups, smem, s);
     }
     Scope sc(KC_SPLITK, 0.0, 4.0 * groups * (p.splits + 1) * blocks * nout, s);
     const dim3 rgrid((nout + 31) / 32, blocks, groups);

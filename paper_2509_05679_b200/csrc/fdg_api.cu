@@ -64,6 +64,7 @@ struct Op {
     // tensor-core plan (bf16 storage, channel counts that are multiples of 64, power-of-two images)
     bool tc;
     bool stem;                                               // thin first-layer conv: dedicated FMA kernels
+    bool packed; size_t pack_off;                            // convolution in mconv.cu: where its weights are in the module's pack_f / pack_b (bytes)
     size_t lin_off;                                          // linear layer on the CUDA cores: its weight-gradient workspace in the module's lin_ws (elements)
     bool head;                                               // the network's last linear layer: fused with the loss (head_* kernels)
     char shape[40];                                          // "HxW Cin->Cout kR sS", the profiler's detail tag
@@ -112,6 +113,10 @@ struct Module {
     char *in_ring, *stash, *gradpool, *d2, *wring, *wtring;
     float *master, *grad, *ws, *lin_ws, *scratch, *red, *cstat[2], *bstat;
     size_t lin_elems;
+    size_t pack_bytes;             // the weights of the convolutions of mconv.cu, per replica, as their kernels read them: of the version that the forward /
+    char *pack_f, *pack_b;         // the backward pass is at, laid out at its beginning
+    struct Pack { PackArgs args; int blocks; };
+    std::vector<Pack> packs;
     bool fused_update;             // one kernel per step updates all parameters and emits the next weight version (both layouts)
     tc::UpdTable upd;
     size_t cstat_elems[2];
@@ -139,6 +144,7 @@ struct Module {
 
 struct fdg_ctx {
     int K, n_workers, B, M, dt, esz, classes, serial, kernel_path;
+    bool fma_only;                 // the caller's kernel_path is 1 (one replica per worker sets the one above, to keep off the TMA kernels)
     int grid_sms;                  // SMs the persistent kernels of this context size their grids for (see fdg_options.grid_sms)
     int R;                         // weight replicas per module: 1 (exact averaging, P = 11^T/N), or n_workers (general mixing matrix)
     std::vector<double> P;         // R x R mixing matrix (row-major) when R > 1
@@ -458,7 +464,7 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
         if (d.own_grad) { d.goff = goff; goff += align_up(d.elems() * ctx->M * ctx->esz, 256); }
     }
     size_t red_pos = 0;
-    m.ws_elems = 0; m.scratch_elems = 64; m.red_elems = 4; m.lin_elems = 0;
+    m.ws_elems = 0; m.scratch_elems = 64; m.red_elems = 4; m.lin_elems = 0; m.pack_bytes = 0;
     for (Op& o : m.ops) {
         if (o.type == OP_BN) {
             o.stats_off = soff; soff += align_up((size_t)ctx->n_workers * o.g.C * (ctx->dt == 0 ? 4 : 2) * sizeof(float), 256);
@@ -478,6 +484,14 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             }
             if (ctx->R > 1) m.ws_elems = std::max(m.ws_elems, fconv_wgrad_workspace_elems(o.g, ctx->R));
             m.scratch_elems = std::max(m.scratch_elems, (size_t)64 * o.g.Co);
+            const size_t pack = ctx->fma_only || o.tc || o.stem || o.head || linear_supported(o.g) ? 0 : mconv_pack_bytes(ctx->dt, o.g, 1);
+            if (pack) {
+                o.packed = true; o.pack_off = m.pack_bytes; m.pack_bytes += pack;
+                if (m.packs.empty() || m.packs.back().args.n == PackArgs::MAX) m.packs.push_back({});
+                Module::Pack& k = m.packs.back();
+                k.args.layer[k.args.n++] = PackLayer{o.w_off, o.pack_off / 16, o.g.C, o.g.Co, o.g.R * o.g.R, k.blocks};
+                k.blocks += (o.g.C / 16) * (o.g.Co / 16);
+            }
             if (relu_bias_backward_supported(ctx->dt, o.g.Co)) m.scratch_elems = std::max(m.scratch_elems, relu_bias_backward_scratch_elems(o.g.Co));
         }
     }
@@ -658,6 +672,18 @@ size_t row_off(const fdg_ctx* c, const TensorDesc& d, const Win& wn) {
     return (size_t)wn.n0 * d.elems() * (d.loc == LOC_LOGITS ? sizeof(float) : (size_t)c->esz);
 }
 
+// The weights of version `version` for one pass of the convolutions in mconv.cu: one launch for all of a module's (up to PackArgs::MAX).
+void pack_weights(fdg_ctx* c, Module& m, int64_t version, bool back, cudaStream_t s) {
+    for (const Module::Pack& k : m.packs) {
+        PackArgs a = k.args; a.back = back;
+        mconv_pack(c->dt, wbig(c, m, version, 0), m.wslot_bytes / c->esz, back ? m.pack_b : m.pack_f, m.pack_bytes, a, k.blocks, c->R, s);
+    }
+}
+Packed packed_f(const Module& m, const Op& o, int rep) { return o.packed ? Packed{m.pack_f + rep * m.pack_bytes + o.pack_off, m.pack_bytes} : Packed{}; }
+Packed packed_b(const Module& m, const Op& o, int rep) { return o.packed ? Packed{m.pack_b + rep * m.pack_bytes + o.pack_off, m.pack_bytes} : Packed{}; }
+// all groups of a launch read the same weights
+Packed shared(Packed p) { p.group = 0; return p; }
+
 // The ops [i0, i1) of a module's forward pass on one group's rows.
 void forward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int group, size_t i0, size_t i1) {
     Module& m = c->mod[kk];
@@ -693,12 +719,12 @@ void forward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int group, 
                     break;
                 }
                 if (o.fstat_tiles && fconv_forward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.bias ? wsmall(c, m, version, o.b_off, rep) : nullptr, T(o.out), g, epi,
-                                                   wn.nw, 0, 0, m.cstat[o.stat_buf], s)) {
+                                                   wn.nw, 0, 0, m.cstat[o.stat_buf], shared(packed_f(m, o, rep)), s)) {
                     m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.fstat_tiles;
                     profile_detail(nullptr);
                     break;
                 }
-                conv_forward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.bias ? wsmall(c, m, version, o.b_off, rep) : nullptr, T(o.out), g, epi, s);
+                conv_forward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.bias ? wsmall(c, m, version, o.b_off, rep) : nullptr, T(o.out), g, epi, packed_f(m, o, rep), s);
                 profile_detail(nullptr);
                 break; }
             case OP_BN: {
@@ -762,7 +788,7 @@ bool forward_op_replicas(fdg_ctx* c, int kk, int64_t batch, int64_t version, siz
             profile_detail(o.shape);
             bool ok = true;
             if (linear_supported(o.g)) linear_forward(dt, P.tensor(o.in), w, b, P.tensor(o.out), o.g, epi, c->R, wg, pg, s);
-            else ok = fconv_forward(dt, P.tensor(o.in), w, b, P.tensor(o.out), o.g, epi, c->R, wg, pg, o.fstat_tiles ? m.cstat[o.stat_buf] : nullptr, s);
+            else ok = fconv_forward(dt, P.tensor(o.in), w, b, P.tensor(o.out), o.g, epi, c->R, wg, pg, o.fstat_tiles ? m.cstat[o.stat_buf] : nullptr, packed_f(m, o, 0), s);
             if (ok && o.fstat_tiles) { m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.fstat_tiles; }
             profile_detail(nullptr);
             return ok; }
@@ -794,6 +820,7 @@ bool forward_op_replicas(fdg_ctx* c, int kk, int64_t batch, int64_t version, siz
 void forward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version) {
     Module& m = c->mod[kk];
     m.fused_stats_tensor[0] = m.fused_stats_tensor[1] = -1;
+    pack_weights(c, m, version, false, m.fstream);
     if (c->R == 1) {
         for (int g = 0; g < m.groups; ++g) { forward_ops(c, kk, batch, version, g, 0, m.ops.size()); m.fused_stats_tensor[0] = m.fused_stats_tensor[1] = -1; }
         return;
@@ -874,13 +901,13 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
                 else if (o.stem) stem_wgrad(T(o.in), gout, mgrad + o.w_off, m.ws, g, acc_p, ws);
                 else if (o.tc && tc_wgrad(c, m, o, P.tensor(o.in), grad_ptr(c, kk, o.out, t), mgrad + o.w_off, wn, ws)) {}
                 else if (linear_supported(g)) linear_backward(dt, T(o.in), nullptr, nullptr, gout, nullptr, false, mgrad + o.w_off, nullptr, g, 1, 0, 0, acc_p, nullptr, ws, ws, m.wev);
-                else fconv_wgrad(dt, T(o.in), gout, mgrad + o.w_off, m.ws, g, 1, 0, acc_p, ws);
+                else fconv_wgrad(dt, T(o.in), gout, mgrad + o.w_off, m.ws, g, 1, 0, acc_p, o.packed, ws);
                 if (o.bias && !fused_rb && !o.masked_by) bias_grad(dt, gout, mgrad + m.n_big + o.b_off, m.scratch, orows, g.Co, acc_p, s);
                 if (gin && !(o.tc && tc_dgrad(c, m, o, grad_ptr(c, kk, o.out, t), grad_ptr(c, kk, o.in, t), version, o.acc_in,
                                                      below ? P.tensor(o.in) : nullptr, col, wn, s))) {
                     c->mask_lost = c->mask_lost || below;
                     if (linear_supported(g)) linear_backward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), nullptr, gout, gin, o.acc_in, nullptr, nullptr, g, 1, 0, 0, false, nullptr, s, s, m.wev);
-                    else fconv_dgrad(dt, gout, wbig(c, m, version, o.w_off, rep), gin, g, o.acc_in ? EPI_ACCUM : 0, 1, 0, s);
+                    else fconv_dgrad(dt, gout, wbig(c, m, version, o.w_off, rep), gin, g, o.acc_in ? EPI_ACCUM : 0, 1, 0, packed_b(m, o, rep), s);
                 }
                 profile_detail(nullptr);
                 break; }
@@ -950,8 +977,8 @@ bool backward_op_replicas(fdg_ctx* c, int kk, int64_t batch, int64_t version, in
             profile_detail(o.shape);
             cudaStream_t ws = m.wstream;
             if (ws != s) { step_record(m.wev, s); step_wait(ws, m.wev); }
-            fconv_wgrad(dt, P.tensor(o.in), gout, m.grad + o.w_off, m.ws, o.g, c->R, gg, false, ws);
-            if (gin) fconv_dgrad(dt, gout, w, gin, o.g, o.acc_in ? EPI_ACCUM : 0, c->R, wg, s);
+            fconv_wgrad(dt, P.tensor(o.in), gout, m.grad + o.w_off, m.ws, o.g, c->R, gg, false, o.packed, ws);
+            if (gin) fconv_dgrad(dt, gout, w, gin, o.g, o.acc_in ? EPI_ACCUM : 0, c->R, wg, packed_b(m, o, 0), s);
             profile_detail(nullptr);
             return true; }
         case OP_BN:
@@ -975,6 +1002,7 @@ bool backward_op_replicas(fdg_ctx* c, int kk, int64_t batch, int64_t version, in
 void backward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t) {
     Module& m = c->mod[kk];
     const int n = (int)m.ops.size();
+    pack_weights(c, m, version, true, m.stream);
     if (c->R == 1) {
         for (int g = 0; g < m.groups; ++g) backward_ops(c, kk, batch, version, t, g, 0, n);
         return;
@@ -1449,7 +1477,7 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
     ctx = new fdg_ctx();
     ctx->K = K; ctx->n_workers = n_workers; ctx->B = per_worker_batch; ctx->M = n_workers * per_worker_batch;
     ctx->dt = opt->dtype; ctx->esz = opt->dtype ? 2 : 4; ctx->classes = opt->num_classes; ctx->serial = opt->serial;
-    ctx->kernel_path = opt->kernel_path;
+    ctx->kernel_path = opt->kernel_path; ctx->fma_only = opt->kernel_path == 1;
     // modules on streams of their own: grids for a third of the SMs, so that tensor-core kernels and memory-bound kernels
     // of different modules run side by side instead of one after the other (a streamed batch-norm kernel keeps 92 % of
     // its bandwidth on half of the SMs, a tensor-core kernel takes 1.6 times as long there, not twice).  Measured on a
@@ -1554,6 +1582,8 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
         m.grad = (float*)get((size_t)ctx->R * (m.n_big + m.n_small) * sizeof(float));
         m.ws = (float*)get(m.ws_elems * sizeof(float));
         m.lin_ws = m.lin_elems ? (float*)get(m.lin_elems * sizeof(float)) : nullptr;
+        m.pack_f = m.pack_bytes ? get(m.pack_bytes * ctx->R) : nullptr;
+        m.pack_b = m.pack_bytes ? get(m.pack_bytes * ctx->R) : nullptr;
         m.scratch = (float*)get(m.scratch_elems * sizeof(float));
         m.red = (float*)get(m.red_elems * sizeof(float));
         m.scratch_f = (float*)get(m.scratch_elems * sizeof(float));

@@ -111,9 +111,9 @@ static inline unsigned cdiv(size_t a, size_t b) { return (unsigned)((a + b - 1) 
 // Convolutions and linear layers on the CUDA cores: fconv.cu and linear.cu.
 size_t wgrad_workspace_elems(const ConvGeom& g) { return linear_supported(g) ? 0 : fconv_wgrad_workspace_elems(g, 1); }
 bool conv_supported(const ConvGeom& g) { return linear_supported(g) || fconv_supported(g); }
-void conv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, cudaStream_t s) {
+void conv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, const Packed& pk, cudaStream_t s) {
     if (linear_supported(g)) linear_forward(dt, x, w, bias, y, g, epi, 1, 0, 0, s);
-    else fconv_forward(dt, x, w, bias, y, g, epi, 1, 0, 0, nullptr, s);
+    else fconv_forward(dt, x, w, bias, y, g, epi, 1, 0, 0, nullptr, pk, s);
 }
 
 // ------------------------------------------------------------------------------------------

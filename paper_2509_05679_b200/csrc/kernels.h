@@ -16,7 +16,8 @@ enum { EPI_RELU = 1, EPI_ACCUM = 2, EPI_OUT_F32 = 4 };
 
 bool   conv_supported(const ConvGeom& g);
 size_t wgrad_workspace_elems(const ConvGeom& g);      // fp32 elements fconv_wgrad needs
-void   conv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, cudaStream_t st);
+struct Packed;
+void   conv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, const Packed& pk, cudaStream_t st);
 // Linear layers (linear.cu).  linear_backward: dx (+)= dy' W (dx_or_null == nullptr: not needed), dW (+)= dy'^T x, db (+)= column sums of
 // dy' in one launch; dy' = dy * [y > 0] if y_or_null is given (the layer ends in a ReLU), else dy.  The sums run over the worker x
 // batch axis, which is the worker average of Eq. dl_update (b) for P = 11^T/N.  accum_p: dW and db are added to (a second group of workers).  dw_or_null ==
@@ -34,14 +35,23 @@ void   linear_backward(int dt, const void* x, const void* w, const void* y_or_nu
 // over all N*Ho*Wo rows of dy^T (x) patches(x) (fp32).  `groups`: consecutive equal groups of images, each with its own weights
 // (w_group elements apart; biases b_group apart; weight gradients w_group apart).  false: shape not covered, nothing launched.
 bool   fconv_supported(const ConvGeom& g);
+// Layers of channel counts that are multiples of 16 run on warp-level tensor-core instructions (mconv.cu) if their weights are there in the order
+// that these read: mconv_pack lays out a module's layers (PackArgs, `blocks` 16 x 16 blocks in all) for one direction, per group `group` bytes apart.
+// mconv_pack_bytes: of one layer and direction, a multiple of 16; 0: shape not covered.
+struct Packed { const void* data; size_t group; };       // data == nullptr: the packed-FMA kernels
+struct PackLayer { size_t w_off, out_off; int C, Co, taps, block0; };        // elements into the matrices, 16-byte words into the result; first block
+struct PackArgs { enum { MAX = 48 }; PackLayer layer[MAX]; int n, back; };
+size_t mconv_pack_bytes(int dt, const ConvGeom& g, int groups);
+void   mconv_pack(int dt, const void* wbig, size_t w_group, void* out, size_t out_group, const PackArgs& a, int blocks, int groups, cudaStream_t st);
 bool   fconv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
-                     float* stat_or_null, cudaStream_t st);
+                     float* stat_or_null, const Packed& pk, cudaStream_t st);
 // Batch-norm statistics taken along by fconv_forward (groups = workers): per worker and pixel tile the channels' (mean, sum of
 // squared deviations), then the tiles' pixel counts: [groups][tiles][Co][2], [groups][tiles] floats.  0: shape not covered.
 int    fconv_stat_tiles(const ConvGeom& g, int groups);
-bool   fconv_dgrad(int dt, const void* dy, const void* w, void* dx, const ConvGeom& g, int epi, int groups, size_t w_group, cudaStream_t st);
+bool   fconv_dgrad(int dt, const void* dy, const void* w, void* dx, const ConvGeom& g, int epi, int groups, size_t w_group, const Packed& pk, cudaStream_t st);
 size_t fconv_wgrad_workspace_elems(const ConvGeom& g, int groups);
-bool   fconv_wgrad(int dt, const void* x, const void* dy, float* dw, float* workspace, const ConvGeom& g, int groups, size_t w_group, bool accum, cudaStream_t st);
+// tensor: by mconv.cu where it covers the shape.
+bool   fconv_wgrad(int dt, const void* x, const void* dy, float* dw, float* workspace, const ConvGeom& g, int groups, size_t w_group, bool accum, bool tensor, cudaStream_t st);
 // db[c] = sum over rows of dy[row][c]; scratch: fp32 [64 * C]
 void bias_grad(int dt, const void* dy, float* db, float* scratch, long rows, int C, bool accum, cudaStream_t st);
 

@@ -1,0 +1,592 @@
+// Convolutions (3x3 and 1x1, stride 1 and 2) of channel counts that are multiples of 16 on the warp-level tensor-core instruction: the fp32
+// path, and with bf16 storage the layers whose channels are no multiple of 64 (the paper's ResNet-20 has 16, 32 and 64).
+//
+//   mc_kernel : forward and input gradient.  A CTA computes 128 pixels x 16 or 32 output channels; the input region of its pixels (halo
+//               included) is fetched once per 16-channel chunk and every filter tap reads it from shared memory, shifted.
+//   mw_kernel : weight gradient.  A CTA keeps a 16 c_out x (taps x 16 c_in) tile of dW in registers over the pixels of its split.
+//   mc_pack_kernel : a layer's weights in the order in which the lanes of a warp hold them (one launch per pass for all layers of a module).
+//
+// Arithmetic with fp32 storage: a value is the sum of three bf16 values, x = hi + mid + lo (8 bits each, rounded to nearest, so that nothing is left), and
+// a product the sum of the six that matter: lo hi + mid mid + hi lo + mid hi + hi mid + hi hi (the rest is 6e-9 of it; 6e-8, and one-sided, with parts by
+// truncation).  Every product is exact; an mma adds 16 of them to its running sum and truncates to 24 bits of the largest term: 2.5e-8 of the
+// result's rms for 16 fresh products of 16 bits, 1.3e-7 for nine such steps in a chain, 5.3e-7 for 36, 1e-7 as soon as a 24-bit running sum of
+// like size is among the terms.  So hi hi starts from zero in every step and goes into an fp32 sum on the CUDA cores, one per 16-channel chunk (9 steps) or
+// four steps of a weight gradient, and that one into a compensated (Kahan) sum; the other five, 2^-8 of it, run on in one accumulator per chunk.
+// Error against double sums, of the result's rms (normal data; packed-FMA kernels of fconv.cu beside it): forward and input gradient 3x3 5.4e-8 to
+// 7.0e-8 (7.6e-8), 1x1 3.6e-8 to 4.7e-8 (6.1e-8), weight gradients 4.8e-8 to 6.2e-8 (5.6e-8 to 1.1e-7).  Two fp16 parts and three products were off by 9.4e-8:
+// 22-bit products lose more where the terms are aligned.  bf16 storage: one exact product a step.
+//
+// Time, 192 images, launch included (packed FMA beside it): fp32 32x32 16 -> 16 forward 23 us (38), weight gradient with its reduction 37 (54); 16x16 32 -> 32 23
+// (40), 35 (53); 8x8 64 -> 64 27 (41), 41 (57).  What bounds them: a third to 40 % of the mma.sync rate (980 multiply-adds per clock and SM, six per
+// product), the rest is latency of one warp's chain (fixed-latency waits, ncu) and the splitting, which every block of 16 or 32 output channels repeats.
+#include "fconv.h"
+#include "launch.h"
+
+namespace fdg {
+
+namespace {
+
+constexpr int MC_THREADS = 128;
+
+template <typename T> constexpr bool SPLIT = sizeof(T) == 4;
+template <typename T> constexpr int PARTS = SPLIT<T> ? 3 : 1;             // bf16 values per value
+template <typename T> constexpr int PACK16 = 32 * PARTS<T>;               // 16-byte words of the packed weights per (16 x 16 block, tap)
+
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ldsm2t(uint32_t (&r)[2], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(a) : "memory");
+}
+// d = a b (+ d): 16 x 16 times 16 x 8
+__device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1, bool add) {
+    const float c0 = add ? d[0] : 0.f, c1 = add ? d[1] : 0.f, c2 = add ? d[2] : 0.f, c3 = add ? d[3] : 0.f;
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
+}
+// product `k` of a step, smallest first: parts of a and of b (0 hi, 1 mid, 2 lo)
+template <typename T> constexpr int PRODUCTS = SPLIT<T> ? 6 : 1;
+template <typename T> __host__ __device__ constexpr int part_a(int k) { return !SPLIT<T> ? 0 : k == 0 ? 2 : k == 1 || k == 3 ? 1 : 0; }
+template <typename T> __host__ __device__ constexpr int part_b(int k) { return !SPLIT<T> ? 0 : k == 2 ? 2 : k == 1 || k == 4 ? 1 : 0; }
+
+// two values' parts
+__device__ __forceinline__ uint32_t pair_rn(float a, float b) { const __nv_bfloat162 v = __floats2bfloat162_rn(a, b); return *(const uint32_t*)&v; }
+__device__ __forceinline__ float2 pair_value(uint32_t v) { return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u)); }
+__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+    const float2 minus = make_float2(-1.f, -1.f);
+    hi = pair_rn(a, b);
+    const float2 r = __ffma2_rn(pair_value(hi), minus, make_float2(a, b));
+    mid = pair_rn(r.x, r.y);
+    const float2 l = __ffma2_rn(pair_value(mid), minus, r);
+    lo = pair_rn(l.x, l.y);
+}
+
+// fp32 values of a pixel's 16 channels as they arrive: quad q sits at position q ^ (pixel / 2 % 4), so that eight pixels' quads q lie in different banks
+__device__ __forceinline__ int raw_at(int pix, int q) { return pix * 16 + ((q ^ ((pix >> 1) & 3)) << 2); }
+
+// A region (see load_region in fconv.cu) of 16 channels from c0 on.  fp32: into raw.  bf16: into planes[half][pixel][8], halves `xp` pixels apart.
+template <typename T>
+__device__ __forceinline__ void fetch_region(const T* __restrict__ x, char* dst, int xp, int n0, int n_end, int nimg, int h0, int w0, int RH, int RW, int step,
+                                             int H, int W, int C, int c0, int warp, int nwarps, int lane) {
+    constexpr int Q = SPLIT<T> ? 4 : 2;              // 16-byte pieces of a pixel
+    int ni = 0, rh = warp;
+    while (rh >= RH) { rh -= RH; ++ni; }
+    while (ni < nimg) {
+        const int n = n0 + ni, h = h0 + rh * step;
+        const bool row_ok = n < n_end && h >= 0 && h < H;
+        // a lane keeps its piece q and steps over pixels, 8 (fp32) or 16 at a time: the position in dst moves by a constant (raw_at: pixel / 2 % 4 stays)
+        constexpr int STEP = 32 / Q;
+        const int q = lane % Q, pix = (ni * RH + rh) * RW + lane / Q;
+        int w = w0 + lane / Q * step;
+        const T* s = x + (((ptrdiff_t)n * H + h) * W + w) * C + c0 + q * (16 / Q);
+        uint32_t d = smem_addr(dst) + (uint32_t)(SPLIT<T> ? raw_at(pix, q) * 4 : (q * xp + pix) * 16);
+        for (int rw = lane / Q; rw < RW; rw += STEP) {
+            const bool in = row_ok && w >= 0 && w < W;
+            cp_async16(d, in ? s : x, in);
+            w += STEP * step; s += (size_t)STEP * step * C; d += STEP * (SPLIT<T> ? 64 : 16);
+        }
+        rh += nwarps;
+        while (rh >= RH) { rh -= RH; ++ni; }
+    }
+}
+// raw -> planes [hi, mid, lo][half][pixel][8], parts `part_bytes` apart
+__device__ __forceinline__ void split_pixels(const float* raw, char* dst, int xp, int part_bytes, int npix, int tid, int nthreads) {
+    for (int pix = tid; pix < npix; pix += nthreads)
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const float4 a = *(const float4*)(raw + raw_at(pix, 2 * half)), b = *(const float4*)(raw + raw_at(pix, 2 * half + 1));
+            uint4 h, m, l;
+            split2(a.x, a.y, h.x, m.x, l.x); split2(a.z, a.w, h.y, m.y, l.y); split2(b.x, b.y, h.z, m.z, l.z); split2(b.z, b.w, h.w, m.w, l.w);
+            char* const d = dst + (half * xp + pix) * 16;
+            *(uint4*)d = h; *(uint4*)(d + part_bytes) = m; *(uint4*)(d + 2 * part_bytes) = l;
+        }
+}
+
+// sum += y + lost, compensated; lost: what the sum has lost so far
+__device__ __forceinline__ void add_kahan(float2& sum, float2& lost, float2 y) {
+    const float2 minus = make_float2(-1.f, -1.f);
+    y = __fadd2_rn(y, lost);
+    const float2 t = __fadd2_rn(sum, y);
+    lost = __ffma2_rn(__ffma2_rn(sum, minus, t), minus, y);          // y - (t - sum)
+    sum = t;
+}
+
+struct McParams {
+    FcParams p;                          // geometry; toff in pixels
+    int xp;                              // pixels of the largest class's region
+    int wtaps;                           // taps of the largest class
+    size_t pack_group;                   // 16-byte words between the groups' packed weights
+};
+template <typename T> constexpr int mc_x_bytes(int xp) { return xp * (SPLIT<T> ? 64 + 96 : 2 * 32); }            // fp32: raw + parts; bf16: two buffers
+template <typename T, int NB> constexpr int mc_w_bytes(int taps, int chunks) { return (chunks > 1 ? 2 : 1) * taps * (NB / 2) * PACK16<T> * 16; }
+
+// grid = (pixel tiles, blocks of 8 NB output channels, groups x classes); a warp computes 32 pixels x 8 NB channels.
+template <typename T, int NB>
+__global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc_kernel(const T* __restrict__ x, const uint4* __restrict__ pk, const float* __restrict__ bias,
+                                                                        T* __restrict__ y, float* __restrict__ stat, const __grid_constant__ McParams q) {
+    constexpr bool S = SPLIT<T>;
+    constexpr int NW = MC_THREADS / 32, BLKS = NB / 2, U = PACK16<T>;
+    extern __shared__ __align__(16) char msm[];
+    const FcParams& p = q.p;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tq = lane & 3;
+    const int cls = blockIdx.z % p.ncls, grp = blockIdx.z / p.ncls;
+    int tile = blockIdx.x;
+    const int tw = tile % p.tiles_w; tile /= p.tiles_w;
+    const int th = tile % p.tiles_h, tn = tile / p.tiles_h;
+    const int n_end = (grp + 1) * p.ngroup, n0 = grp * p.ngroup + tn * p.Nt;
+    const int hd0 = th * p.Ht, wd0 = tw * p.Wt, co0 = blockIdx.y * (8 * NB);
+    const int t0 = p.cls_tap0[cls], nt = p.cls_tap0[cls + 1] - t0;
+    const int RH = p.cls_rh[cls], RW = p.cls_rw[cls], h0 = hd0 * p.xs + p.cls_h0[cls], w0 = wd0 * p.xs + p.cls_w0[cls];
+    const int kc = p.C >> 4, chunks = nt > 0 ? kc : 0, npix = p.Nt * RH * RW;
+    pk += (size_t)grp * q.pack_group;
+
+    float* const raw = (float*)msm;                                              // fp32 only
+    char* const planes = msm + (S ? q.xp * 64 : 0);                              // fp32: [part][half][pixel] 16 bytes; bf16: [buffer][half][pixel]
+    const int plane_bytes = q.xp * 32;
+    char* const wst = planes + (S ? 3 : 2) * plane_bytes;
+    const int wbuf = q.wtaps * BLKS * U * 16;
+
+    // the pixel whose 16 bytes this lane hands to ldmatrix (row lane % 16 of the 16-pixel group i; channels 8 (lane / 16) ...)
+    uint32_t abase[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int px = warp * 32 + i * 16 + (lane & 15);
+        const int pw = px & (p.Wt - 1), ph = (px >> p.lw) & (p.Ht - 1), pn = px >> (p.lw + p.lh);
+        abase[i] = smem_addr(planes) + (uint32_t)(((lane >> 4) * q.xp + (pn * RH + ph * p.xs) * RW + pw * p.xs) * 16);
+    }
+    float2 sum[2][NB][2], lost[2][NB][2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < NB; ++j)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) sum[i][j][r] = lost[i][j][r] = make_float2(0.f, 0.f);
+
+    auto fetch_w = [&](int c, int buf) {
+        for (int tb = warp; tb < nt * BLKS; tb += NW) {
+            const int b = tb % BLKS, t = tb / BLKS;
+            const uint4* const s = pk + ((size_t)((blockIdx.y * BLKS + b) * kc + c) * p.taps + p.wtap[t0 + t]) * U + lane;
+            const uint32_t d = smem_addr(wst + buf * wbuf + (tb * U + lane) * 16);
+#pragma unroll
+            for (int i = 0; i < U / 32; ++i) cp_async16(d + i * 512, s + i * 32, true);
+        }
+    };
+    auto fetch_x = [&](int c, int buf) {
+        fetch_region<T>(x, S ? (char*)raw : planes + buf * plane_bytes, q.xp, n0, n_end, p.Nt, h0, w0, RH, RW, 1, p.H, p.W, p.C, c * FC_KC, warp, NW, lane);
+    };
+    if (chunks) { fetch_x(0, 0); fetch_w(0, 0); cp_commit(); }
+    for (int c = 0; c < chunks; ++c) {
+        const int buf = c & 1;
+        if (S) {
+            cp_wait<0>();
+            __syncthreads();
+            split_pixels(raw, planes, q.xp, plane_bytes, npix, tid, MC_THREADS);
+            __syncthreads();
+            if (c + 1 < chunks) { fetch_x(c + 1, 0); fetch_w(c + 1, buf ^ 1); cp_commit(); }
+        } else {
+            if (c + 1 < chunks) { fetch_x(c + 1, buf ^ 1); fetch_w(c + 1, buf ^ 1); cp_commit(); cp_wait<1>(); } else cp_wait<0>();
+            __syncthreads();
+        }
+        float2 acc[2][NB][2];                        // this chunk's sum of hi hi
+        float rest[2][NB][4];                        // fp32 storage: of the other products
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                acc[i][j][0] = acc[i][j][1] = make_float2(0.f, 0.f);
+                rest[i][j][0] = rest[i][j][1] = rest[i][j][2] = rest[i][j][3] = 0.f;
+            }
+        const char* const ws_ = wst + buf * wbuf + lane * (S ? 16 : 8);
+        const uint32_t xo = S ? 0u : (uint32_t)(buf * plane_bytes);
+#pragma unroll 1
+        for (int t = 0; t < nt; ++t) {
+            const uint32_t off = xo + (uint32_t)p.toff[t0 + t] * 16u;
+            uint32_t a[2][PARTS<T>][4], w[NB][PARTS<T>][2];
+            float part[2][NB][4];
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int k = 0; k < PARTS<T>; ++k) ldsm4(a[i][k], abase[i] + off + k * plane_bytes);
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                const char* const s = ws_ + (t * BLKS + (j >> 1)) * (U * 16);
+                if (S) {
+                    const uint4 v = *(const uint4*)(s + (j & 1) * 512);
+                    const uint2 l = *(const uint2*)(s - lane * 8 + 1024 + (j & 1) * 256);
+                    w[j][0][0] = v.x; w[j][0][1] = v.y; w[j][PARTS<T> / 2][0] = v.z; w[j][PARTS<T> / 2][1] = v.w; w[j][PARTS<T> - 1][0] = l.x; w[j][PARTS<T> - 1][1] = l.y;
+                } else { const uint2 v = *(const uint2*)(s + (j & 1) * 256); w[j][0][0] = v.x; w[j][0][1] = v.y; }
+            }
+#pragma unroll
+            for (int k = 0; k < PRODUCTS<T>; ++k)
+#pragma unroll
+                for (int j = 0; j < NB; ++j)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        if (k + 1 < PRODUCTS<T>) mma(rest[i][j], a[i][part_a<T>(k)], w[j][part_b<T>(k)][0], w[j][part_b<T>(k)][1], true);
+                        else mma(part[i][j], a[i][0], w[j][0][0], w[j][0][1], false);
+                    }
+#pragma unroll
+            for (int j = 0; j < NB; ++j)
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) acc[i][j][r] = __fadd2_rn(acc[i][j][r], make_float2(part[i][j][2 * r], part[i][j][2 * r + 1]));
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < NB; ++j)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    if (S) lost[i][j][r] = __fadd2_rn(lost[i][j][r], make_float2(rest[i][j][2 * r], rest[i][j][2 * r + 1]));
+                    add_kahan(sum[i][j][r], lost[i][j][r], acc[i][j][r]);
+                }
+        if (!S) __syncthreads();                     // this buffer is consumed
+    }
+
+    float val[2][NB][2][2];
+    bool valid[2][2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int px = warp * 32 + i * 16 + r * 8 + g;
+            const int wd = wd0 + (px & (p.Wt - 1)), hd = hd0 + ((px >> p.lw) & (p.Ht - 1)), n = n0 + (px >> (p.lw + p.lh));
+            valid[i][r] = n < n_end && hd < p.Hd && wd < p.Wd;
+            const size_t o = (((size_t)n * p.Ho + (hd * p.os + p.cls_oph[cls])) * p.Wo + (wd * p.os + p.cls_opw[cls])) * p.Co + co0 + 2 * tq;
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                float a = __fadd_rn(sum[i][j][r].x, lost[i][j][r].x), b = __fadd_rn(sum[i][j][r].y, lost[i][j][r].y);
+                if (valid[i][r]) {
+                    const int co = co0 + 8 * j + 2 * tq;
+                    if (bias) { a += bias[(size_t)grp * p.b_group + co]; b += bias[(size_t)grp * p.b_group + co + 1]; }
+                    if (p.epi & EPI_RELU) { a = fmaxf(a, 0.f); b = fmaxf(b, 0.f); }
+                    if (S || (p.epi & EPI_OUT_F32)) {
+                        float2* const d = (float2*)((float*)y + o + 8 * j);
+                        if (p.epi & EPI_ACCUM) { const float2 old = *d; a += old.x; b += old.y; }
+                        *d = make_float2(a, b);
+                    } else {
+                        __nv_bfloat162* const d = (__nv_bfloat162*)((bf16*)y + o + 8 * j);
+                        if (p.epi & EPI_ACCUM) { const __nv_bfloat162 old = *d; a += __low2float(old); b += __high2float(old); }
+                        *d = __floats2bfloat162_rn(a, b);
+                    }
+                }
+                val[i][j][r][0] = stored<T>(a); val[i][j][r][1] = stored<T>(b);
+            }
+        }
+    if (!stat) return;
+    // batch-norm statistics of the tile, from the values as stored: per channel the mean over its pixels and the sum of squared
+    // deviations from that mean (no cancellation, whatever the mean); in a fixed order
+    const int cnt = min(p.Wt, p.Wd - wd0) * min(p.Ht, p.Hd - hd0) * min(p.Nt, n_end - n0);
+    float* const red = (float*)msm;                  // [warp][8 NB]
+    float s[NB][2], mean[NB][2];
+    auto over_pixels = [&](auto term) {
+#pragma unroll
+        for (int j = 0; j < NB; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                s[j][e] = 0.f;
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) if (valid[i][r]) s[j][e] += term(val[i][j][r][e], mean[j][e]);
+#pragma unroll
+                for (int d = 4; d < 32; d <<= 1) s[j][e] += __shfl_xor_sync(0xffffffffu, s[j][e], d);
+            }
+        __syncthreads();
+        if (g == 0)
+#pragma unroll
+            for (int j = 0; j < NB; ++j) *(float2*)(red + warp * (8 * NB) + 8 * j + 2 * tq) = make_float2(s[j][0], s[j][1]);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < NB; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float* const c = red + 8 * j + 2 * tq + e;
+                s[j][e] = (c[0] + c[8 * NB]) + (c[16 * NB] + c[24 * NB]);
+            }
+    };
+    over_pixels([](float v, float) { return v; });
+#pragma unroll
+    for (int j = 0; j < NB; ++j)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) mean[j][e] = s[j][e] / (float)cnt;
+    over_pixels([](float v, float m) { const float d = v - m; return d * d; });
+    if (warp == 0 && g == 0) {
+        const int tiles = gridDim.x, groups = gridDim.z;
+        const size_t rec = (size_t)grp * tiles + blockIdx.x;
+#pragma unroll
+        for (int j = 0; j < NB; ++j)
+            *(float4*)(stat + (rec * p.Co + co0 + 8 * j + 2 * tq) * 2) = make_float4(mean[j][0], s[j][0], mean[j][1], s[j][1]);
+        if (blockIdx.y == 0 && tq == 0) stat[(size_t)groups * tiles * p.Co * 2 + rec] = (float)cnt;
+    }
+}
+
+constexpr int MW_WARPS = 6;              // two halves of c_in x (3x3: three rows of taps; 1x1: three pixel slices)
+struct MwParams {
+    FwParams p;                          // geometry; toff in pixels
+    int npix, xp;                        // pixels of a tile, of its region
+};
+__host__ __device__ constexpr int mw_slices(int taps_a_warp) { return taps_a_warp == 3 ? 1 : 3; }
+template <typename T> constexpr int mw_smem(int npix, int xp) { return (npix + xp) * (SPLIT<T> ? 64 + 96 : 2 * 32); }      // fp32: raw + parts; bf16: two buffers
+
+// grid = (splits, c_out blocks x c_in blocks, groups).  part_out: [group][block][split][16 c_out][taps][16 c_in], as fw_kernel's.
+template <typename T, int XS, int TW>
+__global__ void __launch_bounds__(MW_WARPS * 32, 3) mw_kernel(const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ part_out,
+                                                              const __grid_constant__ MwParams q) {
+    constexpr bool S = SPLIT<T>;
+    constexpr int SL = mw_slices(TW);
+    extern __shared__ __align__(16) char msm[];
+    const FwParams& p = q.p;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tq = lane & 3;
+    const int grp = blockIdx.z, cob = blockIdx.y / p.ci_blocks, cib = blockIdx.y % p.ci_blocks;
+    const int co0 = cob * FW_CO, ci0 = cib * FW_CI;
+    const int half = warp & 1, slice = SL > 1 ? warp >> 1 : 0, tap0 = SL > 1 ? 0 : (warp >> 1) * TW;
+    const int xp = q.xp, npix = q.npix;
+    float* const raw_x = (float*)msm;                                            // fp32 only
+    float* const raw_d = raw_x + xp * 16;
+    char* const px_ = msm + (S ? (xp + npix) * 64 : 0);                          // planes of x: fp32 [part][half][pixel] 16 bytes; bf16 [buffer][half][pixel]
+    char* const pd_ = px_ + xp * 32 * (S ? 3 : 2);                               // planes of dy
+    float2 sum[TW][2], lost[TW][2];
+#pragma unroll
+    for (int s = 0; s < TW; ++s)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) sum[s][r] = lost[s][r] = make_float2(0.f, 0.f);
+    const int per = (p.tiles + p.splits - 1) / p.splits;
+    const int tile0 = blockIdx.x * per, tile_end = min(p.tiles, tile0 + per), n_end = (grp + 1) * p.ngroup;
+    auto fetch = [&](int tl, int buf) {
+        const int tw = tl % p.tiles_w; tl /= p.tiles_w;
+        const int th = tl % p.tiles_h, tn = tl / p.tiles_h;
+        const int n0 = grp * p.ngroup + tn * p.Nt, ho0 = th * p.Ht, wo0 = tw * p.Wt;
+        fetch_region<T>(x, S ? (char*)raw_x : px_ + buf * xp * 32, xp, n0, n_end, p.Nt, ho0 * p.hstep - p.pad, wo0 * p.hstep - p.pad, p.RH, p.RW, p.step, p.H, p.W, p.C,
+                        ci0, warp, MW_WARPS, lane);
+        constexpr int Q = S ? 4 : 2;
+        const int c = tid % Q;
+        const T* const d0 = dy + co0 + c * (16 / Q);
+        for (int px = tid / Q; px < npix; px += MW_WARPS * 32 / Q) {
+            const int w = wo0 + (px & (p.Wt - 1)), h = ho0 + ((px >> p.lw) & (p.Ht - 1)), n = n0 + (px >> (p.lw + p.lh));
+            const bool in = n < n_end && h < p.Ho && w < p.Wo;
+            cp_async16(smem_addr(S ? (char*)(raw_d + raw_at(px, c)) : pd_ + buf * npix * 32 + (c * npix + px) * 16), in ? d0 + (((size_t)n * p.Ho + h) * p.Wo + w) * p.Co : dy, in);
+        }
+        cp_commit();
+    };
+    // what a few steps have added up goes into the compensated sum
+    auto flush = [](float2 (&acc)[TW][2], float2 (&sum)[TW][2], float2 (&lost)[TW][2]) {
+#pragma unroll
+        for (int s = 0; s < TW; ++s)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) { add_kahan(sum[s][r], lost[s][r], acc[s][r]); acc[s][r] = make_float2(0.f, 0.f); }
+    };
+    auto region_pixel = [&](int px) { return ((px >> (p.lw + p.lh)) * p.RH + ((px >> p.lw) & (p.Ht - 1)) * XS) * p.RW + (px & (p.Wt - 1)) * XS; };
+    if (tile0 < tile_end) fetch(tile0, 0);
+    for (int tile = tile0; tile < tile_end; ++tile) {
+        const int buf = (tile - tile0) & 1;
+        if (S) {
+            cp_wait<0>();
+            __syncthreads();
+            split_pixels(raw_x, px_, xp, xp * 32, xp, tid, MW_WARPS * 32);
+            split_pixels(raw_d, pd_, npix, npix * 32, npix, tid, MW_WARPS * 32);
+            __syncthreads();
+            if (tile + 1 < tile_end) fetch(tile + 1, 0);
+        } else {
+            if (tile + 1 < tile_end) { fetch(tile + 1, buf ^ 1); cp_wait<1>(); } else cp_wait<0>();
+            __syncthreads();
+        }
+        const uint32_t dbase = smem_addr(pd_) + (S ? 0 : buf * npix * 32) + (((lane >> 3) & 1) * npix + (lane & 7) + 8 * (lane >> 4)) * 16;
+        // rows of x that this lane hands to ldmatrix: pixel lane % 16; lanes 16..31 those of the second part (fp32), nobody's (bf16)
+        const uint32_t xbase = smem_addr(px_) + (S ? 0 : buf * xp * 32) + (half * xp + p.toff[tap0]) * 16;
+        float2 acc[TW][2];                           // this tile's sum of hi hi
+        float rest[TW][4];                           // fp32 storage: of the other products
+#pragma unroll
+        for (int s = 0; s < TW; ++s) {
+            acc[s][0] = acc[s][1] = make_float2(0.f, 0.f);
+            rest[s][0] = rest[s][1] = rest[s][2] = rest[s][3] = 0.f;
+        }
+#pragma unroll 1
+        for (int ks = slice; ks * 16 < npix; ks += SL) {
+            uint32_t a[PARTS<T>][4], b[TW][PARTS<T>][2];
+            float part[TW][4];
+            const uint32_t xa = xbase + region_pixel(ks * 16 + (lane & 15)) * 16;
+#pragma unroll
+            for (int k = 0; k < PARTS<T>; ++k) ldsm4t(a[k], dbase + ks * 256 + k * npix * 32);
+#pragma unroll
+            for (int s = 0; s < TW; ++s) {
+                if (S) {
+                    uint32_t v[4];
+                    ldsm4t(v, xa + s * 16 + (lane >> 4) * xp * 32);
+                    b[s][0][0] = v[0]; b[s][0][1] = v[1]; b[s][PARTS<T> / 2][0] = v[2]; b[s][PARTS<T> / 2][1] = v[3];
+                }
+                ldsm2t(b[s][PARTS<T> - 1], xa + s * 16 + (PARTS<T> - 1) * xp * 32);
+            }
+#pragma unroll
+            for (int k = 0; k < PRODUCTS<T>; ++k)
+#pragma unroll
+                for (int s = 0; s < TW; ++s) {
+                    if (k + 1 < PRODUCTS<T>) mma(rest[s], a[part_a<T>(k)], b[s][part_b<T>(k)][0], b[s][part_b<T>(k)][1], true);
+                    else mma(part[s], a[0], b[s][0][0], b[s][0][1], false);
+                }
+#pragma unroll
+            for (int s = 0; s < TW; ++s)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) acc[s][r] = __fadd2_rn(acc[s][r], make_float2(part[s][2 * r], part[s][2 * r + 1]));
+            if (S && (ks & 3) == 3) flush(acc, sum, lost);
+        }
+        flush(acc, sum, lost);
+        if (S)
+#pragma unroll
+            for (int s = 0; s < TW; ++s)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) lost[s][r] = __fadd2_rn(lost[s][r], make_float2(rest[s][2 * r], rest[s][2 * r + 1]));
+        if (!S) __syncthreads();                     // this buffer is consumed
+    }
+    // the slices' sums in slice order, then the CTA's partial matrix
+    const int nout = FW_CO * p.ntaps * FW_CI;
+    float* const red = (float*)msm;                  // [slice][16][taps][16]
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < TW; ++s)
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+            *(float2*)(red + (size_t)slice * nout + ((g + 8 * r) * p.ntaps + tap0 + s) * 16 + 8 * half + 2 * tq) =
+                make_float2(__fadd_rn(sum[s][r].x, lost[s][r].x), __fadd_rn(sum[s][r].y, lost[s][r].y));
+    __syncthreads();
+    float* const out = part_out + (((size_t)grp * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * nout;
+    for (int i = tid; i < nout; i += MW_WARPS * 32) {
+        double s = 0;
+        for (int k = 0; k < SL; ++k) s += (double)red[(size_t)k * nout + i];
+        out[i] = (float)s;
+    }
+}
+
+// One CTA per 16 x 16 block of a layer's matrices (all taps): [n block][k chunk][tap][n8][lane], per lane the B operand of one mma: the values (k = 2 t, 2 t + 1
+// and 2 t + 8, 2 t + 9; n = lane / 4), t = lane % 4; fp32: 16 bytes of hi and mid each, then 8 of lo each.  Forward: n = output, k = input channel; back: the reverse.
+template <typename T>
+__global__ void __launch_bounds__(256) mc_pack_kernel(const T* __restrict__ wbig, size_t w_group, uint4* __restrict__ out, size_t out_group, const __grid_constant__ PackArgs a) {
+    __shared__ float ws[9 * 256 + 16];
+    int l = 0;
+    while (l + 1 < a.n && (int)blockIdx.x >= a.layer[l + 1].block0) ++l;
+    const PackLayer& L = a.layer[l];
+    const int blk = blockIdx.x - L.block0, cib = blk % (L.C / 16), cob = blk / (L.C / 16), tid = threadIdx.x;
+    wbig += (size_t)blockIdx.y * w_group + L.w_off;
+    out += (size_t)blockIdx.y * out_group + L.out_off;
+    for (int i = tid; i < L.taps * 256; i += 256) {
+        const int ci = i & 15, tap = (i >> 4) % L.taps, co = (i >> 4) / L.taps;
+        ws[(co * L.taps + tap) * 16 + ci] = (float)wbig[((size_t)(cob * 16 + co) * L.taps + tap) * L.C + cib * 16 + ci];
+    }
+    __syncthreads();
+    const int nb = a.back ? cib : cob, kb = a.back ? cob : cib, kc = (a.back ? L.Co : L.C) / 16;
+    for (int i = tid; i < L.taps * 64; i += 256) {
+        const int lane = i & 31, n8 = (i >> 5) & 1, tap = i >> 6, n = n8 * 8 + (lane >> 2), k0 = 2 * (lane & 3);
+        uint32_t h[2], mid[2], lo[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            float v[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int k = k0 + 8 * u + j;
+                v[j] = ws[((a.back ? k : n) * L.taps + tap) * 16 + (a.back ? n : k)];
+            }
+            if (SPLIT<T>) {
+                split2(v[0], v[1], h[u], mid[u], lo[u]);
+            } else {
+                const __nv_bfloat162 b = __floats2bfloat162_rn(v[0], v[1]);
+                h[u] = *(const uint32_t*)&b;
+            }
+        }
+        uint4* const d = out + ((size_t)(nb * kc + kb) * L.taps + tap) * PACK16<T>;
+        if (SPLIT<T>) { d[n8 * 32 + lane] = make_uint4(h[0], h[1], mid[0], mid[1]); ((uint2*)(d + 64))[n8 * 32 + lane] = make_uint2(lo[0], lo[1]); }
+        else ((uint2*)d)[n8 * 32 + lane] = make_uint2(h[0], h[1]);
+    }
+}
+
+bool channels_ok(const ConvGeom& g) { return g.C % 16 == 0 && g.Co % 16 == 0; }
+template <typename T, int NB> size_t mc_smem(const McParams& q) { return (size_t)mc_x_bytes<T>(q.xp) + mc_w_bytes<T, NB>(q.wtaps, q.p.C / 16); }
+
+template <typename T>
+bool plan_mc(const ConvGeom& g, int groups, bool back, McParams& q) {
+    if (!channels_ok(g) || !plan_fc(g, groups, back, q.p)) return false;
+    q.xp = q.p.x_floats / PITCH;
+    q.wtaps = q.p.w_floats / (16 * PITCH);
+    for (int& t : q.p.toff) t /= PITCH;
+    return mc_smem<T, 4>(q) <= FC_SMEM_MAX;
+}
+template <typename T>
+bool plan_mw(const ConvGeom& g, int groups, MwParams& q, size_t& smem) {
+    int G, run; size_t fw;
+    if (!channels_ok(g) || !plan_fw(g, groups, q.p, G, run, fw)) return false;
+    q.npix = q.p.Wt * q.p.Ht * q.p.Nt;
+    q.xp = q.p.x_floats / PITCH;
+    for (int i = 0; i < q.p.ntaps; ++i) q.p.toff[i] /= PITCH;
+    const size_t red = (size_t)mw_slices(g.R) * FW_CO * q.p.ntaps * FW_CI * sizeof(float);
+    smem = mw_smem<T>(q.npix, q.xp);
+    if (red > smem) smem = red;
+    return q.npix % 16 == 0 && smem <= FC_SMEM_MAX;
+}
+
+template <typename T, int NB>
+cudaError_t launch_mc(const void* x, const void* pk, const float* bias, void* y, float* stat, const McParams& q, int groups, cudaStream_t s) {
+    static OncePerDevice once;
+    if (cudaError_t e = allow_smem(once, (const void*)mc_kernel<T, NB>, (int)FC_SMEM_MAX)) return e;
+    const int tiles = q.p.tiles_w * q.p.tiles_h * ((q.p.ngroup + q.p.Nt - 1) / q.p.Nt);
+    return klaunch(mc_kernel<T, NB>, dim3(tiles, q.p.Co / (8 * NB), groups * q.p.ncls), MC_THREADS, mc_smem<T, NB>(q), s, (const T*)x, (const uint4*)pk, bias, (T*)y, stat, q);
+}
+template <typename T>
+bool run_mc(const void* x, const void* pk, const float* bias, void* y, float* stat, const ConvGeom& g, int epi, int groups, size_t b_group, size_t pack_group, bool back, cudaStream_t s) {
+    McParams q;
+    if (!plan_mc<T>(g, groups, back, q)) return false;
+    q.p.epi = epi; q.p.b_group = b_group;
+    q.pack_group = pack_group / 16;
+    const long tiles = (long)q.p.tiles_w * q.p.tiles_h * ((q.p.ngroup + q.p.Nt - 1) / q.p.Nt) * groups * q.p.ncls;
+    // 32 output channels a CTA (a third less shared-memory traffic per product, the region split for twice the work), unless 16 fill the device more evenly;
+    // large regions (stride 2) leave an SM two CTAs at the most either way
+    const auto waves = [](long ctas) { return (ctas + 147) / 148; };
+    const bool wide = q.p.Co % 32 == 0 && (mc_smem<T, 2>(q) > 75 * 1024 || 2 * waves(tiles * (q.p.Co / 32)) <= 1.15 * waves(tiles * (q.p.Co / 16)));
+    return (wide ? launch_mc<T, 4>(x, pk, bias, y, stat, q, groups, s) : launch_mc<T, 2>(x, pk, bias, y, stat, q, groups, s)) == cudaSuccess;
+}
+template <typename T, int XS, int TW>
+cudaError_t launch_mw(const void* x, const void* dy, float* ws, const MwParams& q, int groups, int blocks, size_t smem, cudaStream_t s) {
+    static OncePerDevice once;
+    if (cudaError_t e = allow_smem(once, (const void*)mw_kernel<T, XS, TW>, (int)FC_SMEM_MAX)) return e;
+    return klaunch(mw_kernel<T, XS, TW>, dim3(q.p.splits, blocks, groups), MW_WARPS * 32, smem, s, (const T*)x, (const T*)dy, ws, q);
+}
+template <typename T>
+int run_mw(const void* x, const void* dy, float* ws, const ConvGeom& g, int groups, cudaStream_t s) {
+    MwParams q; size_t smem;
+    if (!plan_mw<T>(g, groups, q, smem)) return 0;
+    const int blocks = q.p.ci_blocks * (g.Co / FW_CO);
+    cudaError_t e;
+    if (g.R == 1) e = launch_mw<T, 1, 1>(x, dy, ws, q, groups, blocks, smem, s);
+    else if (g.stride == 1) e = launch_mw<T, 1, 3>(x, dy, ws, q, groups, blocks, smem, s);
+    else e = launch_mw<T, 2, 3>(x, dy, ws, q, groups, blocks, smem, s);
+    return e == cudaSuccess ? q.p.splits : 0;
+}
+
+}  // namespace
+
+size_t mconv_pack_bytes(int dt, const ConvGeom& g, int groups) {
+    McParams q;
+    const bool ok = dt ? plan_mc<bf16>(g, groups, false, q) && plan_mc<bf16>(g, groups, true, q) : plan_mc<float>(g, groups, false, q) && plan_mc<float>(g, groups, true, q);
+    if (!ok) return 0;
+    const size_t blocks = (size_t)(g.C / 16) * (g.Co / 16);
+    return blocks * g.R * g.R * (dt ? PACK16<bf16> : PACK16<float>) * 16;
+}
+void mconv_pack(int dt, const void* wbig, size_t w_group, void* out, size_t out_group, const PackArgs& a, int blocks, int groups, cudaStream_t s) {
+    Scope sc(KC_TC_AUX, 0.0, (double)blocks * groups * 9 * 256 * (dt ? 4.0 : 8.0), s);
+    if (dt) klaunch(mc_pack_kernel<bf16>, dim3(blocks, groups), 256, 0, s, (const bf16*)wbig, w_group, (uint4*)out, out_group / 16, a);
+    else klaunch(mc_pack_kernel<float>, dim3(blocks, groups), 256, 0, s, (const float*)wbig, w_group, (uint4*)out, out_group / 16, a);
+}
+bool mconv_forward(int dt, const void* x, const void* pack, const float* bias, void* y, float* stat, const ConvGeom& g, int epi, int groups, size_t b_group, size_t pack_group,
+                   cudaStream_t s) {
+    return dt ? run_mc<bf16>(x, pack, bias, y, stat, g, epi, groups, b_group, pack_group, false, s) : run_mc<float>(x, pack, bias, y, stat, g, epi, groups, b_group, pack_group, false, s);
+}
+bool mconv_dgrad(int dt, const void* dy, const void* pack, void* dx, const ConvGeom& g, int epi, int groups, size_t pack_group, cudaStream_t s) {
+    return dt ? run_mc<bf16>(dy, pack, nullptr, dx, nullptr, g, epi, groups, 0, pack_group, true, s) : run_mc<float>(dy, pack, nullptr, dx, nullptr, g, epi, groups, 0, pack_group, true, s);
+}
+int mconv_wgrad(int dt, const void* x, const void* dy, float* ws, const ConvGeom& g, int groups, cudaStream_t s) {
+    return dt ? run_mw<bf16>(x, dy, ws, g, groups, s) : run_mw<float>(x, dy, ws, g, groups, s);
+}
+
+}  // namespace fdg

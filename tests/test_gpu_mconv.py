@@ -1,0 +1,71 @@
+"""The tensor-core convolutions off the TMA path (mconv.cu: channel counts that are multiples of 16) at the edges of their tiles: images of odd sides, of one
+row, smaller than a tile; strides 1 and 2, 3x3 and 1x1; one, two and three blocks of 16 channels; batches that leave a tile ragged; magnitudes far from 1,
+where the parts of a split value get small.  One step of ReLU-free networks against the oracle, with the tolerances of tests/test_gpu_fconv.py."""
+import numpy as np
+import pytest
+
+from paper_2509_05679_b200 import synth as sy
+from harness import make_ctx, make_oracle, max_rel_err, run_parity
+
+pytestmark = pytest.mark.gpu
+
+# (H, W), first layer's width, kind, second layer's width, stride
+SHAPES = [((5, 7), 16, sy.CONV3X3, 48, 1), ((33, 9), 16, sy.CONV3X3, 16, 1), ((16, 1), 16, sy.CONV3X3, 32, 1), ((2, 2), 32, sy.CONV3X3, 16, 1), ((6, 10), 32, sy.CONV3X3, 64, 2),
+          ((14, 14), 16, sy.CONV3X3, 32, 2), ((7, 11), 16, sy.CONV1X1, 32, 1), ((6, 10), 48, sy.CONV1X1, 16, 2), ((4, 4), 80, sy.CONV3X3, 96, 1)]
+
+
+def _net(shape, dtype, workers, batch, bn):
+    (h, w), c, kind, co, stride = shape
+    norm = lambda n: [(sy.BATCHNORM, n, n, 1, 0)] if bn else []
+    bias = 0 if bn else sy.FLAG_BIAS
+    layers = [(sy.CONV3X3, 3, c, 1, bias)] + norm(c) + [(kind, c, co, stride, bias)] + norm(co) + [(sy.GLOBAL_AVGPOOL, co, co, 1, 0), (sy.LINEAR, co, 10, 1, 1)]
+    return sy.Net("mconv", layers, [], h, w, 3, 10, workers, batch, 0.05, dtype)
+
+
+def _id(s):
+    return f"{s[0][0]}x{s[0][1]}-{s[1]}-{s[3]}-k{3 if s[2] == sy.CONV3X3 else 1}-s{s[4]}"
+
+
+@pytest.mark.parametrize("workers,batch", [(1, 1), (3, 9), (2, 70)])
+@pytest.mark.parametrize("shape", SHAPES, ids=_id)
+def test_fp32(orc, shape, workers, batch):
+    run_parity(orc, _net(shape, "fp32", workers, batch, False), 1, param_tol=1e-5, loss_tol=1e-5, grad_tol=1e-5)
+    run_parity(orc, _net(shape, "fp32", workers, batch + 1, True), 1, param_tol=1e-5, loss_tol=1e-5)
+
+
+@pytest.mark.parametrize("workers,batch", [(1, 1), (2, 9)])
+@pytest.mark.parametrize("shape", SHAPES, ids=_id)
+def test_bf16_storage(orc, shape, workers, batch):
+    terms = shape[1] * (9 if shape[2] == sy.CONV3X3 else 1)
+    run_parity(orc, _net(shape, "bf16", workers, batch, False), 1, grad_tol=2e-3 if terms <= 144 and workers * batch in (1, 2, 4, 8) else 2e-2, loss_tol=1e-4)
+
+
+@pytest.mark.parametrize("exponent", [-60, 40])
+def test_values_far_from_one(orc, exponent):
+    """First layer's weights times 2^exponent, second layer's divided by it: the second layer's inputs are that far from 1, its outputs as before; all
+    scalings are exact, so gradients are compared as scaled (the parts of a split value reach down to 2^-24 of it, 2^-84 here)."""
+    import torch
+    from paper_2509_05679_b200 import binding
+    net = _net(((9, 8), 16, sy.CONV3X3, 32, 1), "fp32", 2, 5, False)
+    p0 = sy.init_params(net.layers, 0)
+    n1 = 16 * 27
+    p0[n1:n1 + 16] = 0.0
+    scaled = p0.copy()
+    scaled[:n1] = np.ldexp(p0[:n1], exponent)
+    n2 = n1 + 16 + 32 * 9 * 16
+    scaled[n1 + 16:n2] = np.ldexp(p0[n1 + 16:n2], -exponent)
+    x, y = sy.batch_inputs(net, 0), sy.batch_labels(net, 0)
+    o = make_oracle(orc, net, p0)
+    o.step(x, y, 0.0)
+    g = np.mean([o.grads(s) for s in range(net.n_workers)], axis=0)
+    ctx = make_ctx(net, scaled)
+    try:
+        ctx.set_lr(0.0)
+        ctx.step(binding.to_device("fp32", x), torch.from_numpy(y).cuda())
+        got = np.asarray(ctx.grads(), np.float64)
+    finally:
+        ctx.close()
+    got[:n1 + 16] = np.ldexp(got[:n1 + 16], exponent)          # d/d(w 2^e) = 2^-e d/dw
+    got[n1 + 16:n2] = np.ldexp(got[n1 + 16:n2], -exponent)
+    err, where = max_rel_err(got, g, net.layers)
+    assert err <= 1e-5, (err, where)
