@@ -445,7 +445,9 @@ static void bnc_launch(const BncArgs& a, int nw, int nw_all, cudaStream_t s) {
     // wanted by the other modules (18 samples, 4 modules: 386 us per step with this line, 432 with 100 CTAs; by the number of ALL workers: a launch for
     // a group of them adds in the same order)
     int sl = 64;
-    while (sl > 16 && (a.C % sl || (a.C / sl) * nw_all * BNC_RANKS < 25)) sl /= 2;
+    const auto ctas = [&] { return (a.C / sl) * nw_all * BNC_RANKS; };
+    const auto rows_a_thread = [&] { return (a.rpw + BNC_RANKS - 1) / BNC_RANKS * (sl / 8) / BT; };
+    while (sl > 16 && (a.C % sl || ctas() < 25 || (rows_a_thread() > 20 && ctas() < 148))) sl /= 2;
     const dim3 grid((a.C / sl) * BNC_RANKS, nw);
     if (sl == 64) klaunch_cluster(bnc_kernel<64, BWD>, grid, BT, 0, s, BNC_RANKS, a);
     else if (sl == 32) klaunch_cluster(bnc_kernel<32, BWD>, grid, BT, 0, s, BNC_RANKS, a);
