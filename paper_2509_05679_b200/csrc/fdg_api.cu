@@ -704,10 +704,10 @@ void forward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int group, 
                 ConvGeom g = o.g; g.N = wn.n;
                 profile_detail(o.shape);
                 if (o.head && m.groups == 1) {
-                    // logits, loss and dphi/dlogits / M of batch `batch` in one launch (version == the iteration t)
+                    // logits, parts of the loss and dphi/dlogits / M of batch `batch` in one launch; the backward pass of the same iteration adds the parts
                     head_forward_loss(dt, T(o.in), wbig(c, m, version, o.w_off), o.bias ? wsmall(c, m, version, o.b_off) : nullptr,
                                       c->labels + (size_t)(batch % c->label_depth) * c->M, c->logits, c->dlogits, m.head_scratch + m.head_part_elems,
-                                      (unsigned*)(c->tc_err + 16), c->loss_ring + (version % 64), c->tc_err, version + 1, c->M, g.C, g.Co, 1.f / (float)c->M, s);
+                                      c->M, g.C, g.Co, 1.f / (float)c->M, s);
                     profile_detail(nullptr);
                     break;
                 }
@@ -874,7 +874,8 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
                     head_backward(dt, T(o.in), wbig(c, m, version, o.w_off), gout, gin, o.acc_in, o.masks > 0, col, m.head_scratch, c->M, g.C, g.Co, s);
                     cudaStream_t ws = m.wstream;                     // the sum of the partials is needed by the update only
                     if (ws != s) { step_record(m.wev, s); step_wait(ws, m.wev); }
-                    head_reduce(mgrad + o.w_off, o.bias ? mgrad + m.n_big + o.b_off : nullptr, m.head_scratch, c->M, g.C, g.Co, ws);
+                    head_reduce(mgrad + o.w_off, o.bias ? mgrad + m.n_big + o.b_off : nullptr, m.head_scratch, m.head_scratch + m.head_part_elems, c->loss_ring + (t % 64), c->tc_err,
+                                t + 1, c->M, g.C, g.Co, ws);
                     profile_detail(nullptr);
                     break;
                 }

@@ -1131,26 +1131,35 @@ void softmax_ce(int dt, const float* logits, const int32_t* labels, void* dlogit
 // ------------------------------------------------------------------------------------------
 // Classifier head: the network's last linear layer (c_in -> a few classes) fused with the loss.
 //   head_fwd_loss_k : one warp per sample: logits = x W^T + b (fp32, kept for the caller), softmax cross-entropy,
-//                     dlogits = (softmax - onehot) * scale in the storage dtype, per-CTA loss partials; the CTA that
-//                     finishes last adds the partials in index order (a fixed order) and writes the mean loss.
+//                     dlogits = (softmax - onehot) * scale in the storage dtype, per-CTA loss partials.
 //   head_bwd_k      : a CTA owns a range of samples: dx = dlogits W (one warp per sample) and the partial sums of
 //                     dW[c][k] = sum_rows dlogits[row][c] x[row][k] and db[c] = sum_rows dlogits[row][c] (column k = K).
-//   head_reduce_k   : dW / db = partials added in CTA order.
+//   head_reduce_k   : dW / db = partials added in CTA order; one CTA more adds the loss partials and hands the mean loss to the host.
+// The first two stand in the last module's chain, so latency is all that counts: operands come in one round trip to L2 (weights and tiles through shared
+// memory, HEAD_W_SMEM, HEAD_STAGE_VECS; a loop over the classes waited for four to eight), and what waits for other CTAs or for the host's memory is in
+// the third, off the chain.  512 samples, 1024 columns, 10 classes in bf16, cold: forward 20.3 -> 9.9 us, backward 10.5 -> 8.0; steps of the 512-wide fp32 MLP 62 -> 58 us.
 // Replaces an implicit-GEMM launch on 64 x 64 tiles (8-16 CTAs), a one-CTA loss kernel, two bias-gradient launches, a
 // split weight gradient with its reduction and an input-gradient launch.  classes <= 16, c_in a multiple of the vector width.
 // ------------------------------------------------------------------------------------------
 constexpr int HEAD_MAX_C = 16;
 constexpr int HEAD_ROWS_PER_CTA = 32;       // samples per CTA of head_bwd_k
+constexpr size_t HEAD_W_SMEM = 40 * 1024;   // a larger W is read from L2 by every warp (static and dynamic shared memory stay below the 48 KB of any launch)
+constexpr int HEAD_STAGE_VECS = 32;         // wider slices are there for many samples, where other CTAs cover the latency
 template <typename T>
 __global__ void __launch_bounds__(256) head_fwd_loss_k(const T* __restrict__ x, const T* __restrict__ W, const float* __restrict__ bias,
                                                        const int32_t* __restrict__ labels, float* __restrict__ logits, T* __restrict__ dz,
-                                                       float* __restrict__ loss_part, unsigned* __restrict__ counter, LossRecord* rec, const int* err, long long seq,
-                                                       int M, int K, int C, float scale) {
+                                                       float* __restrict__ loss_part, int M, int K, int C, float scale, bool w_smem) {
     constexpr int V = Vec<T>::V;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = blockIdx.x * 8 + warp;
     __shared__ float wl[8];
-    __shared__ bool last;
+    extern __shared__ __align__(16) char hsm[];
+    const T* Wp = W;
+    if (w_smem) {                            // (uniform) all of W, 16 bytes a thread at a time
+        for (int i = threadIdx.x; i < C * K / V; i += 256) ((uint4*)hsm)[i] = ((const uint4*)W)[i];
+        Wp = (const T*)hsm;
+        __syncthreads();
+    }
     float rloss = 0.f;
     if (row < M) {
         float acc[HEAD_MAX_C];
@@ -1165,7 +1174,7 @@ __global__ void __launch_bounds__(256) head_fwd_loss_k(const T* __restrict__ x, 
                 if (c >= C) break;
                 float wv[8][8];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) Vec<T>::load(W + (size_t)min(c + q, C - 1) * K + (size_t)kv * V, wv[q]);
+                for (int q = 0; q < 8; ++q) Vec<T>::load(Wp + (size_t)min(c + q, C - 1) * K + (size_t)kv * V, wv[q]);
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
 #pragma unroll
@@ -1195,7 +1204,7 @@ __global__ void __launch_bounds__(256) head_fwd_loss_k(const T* __restrict__ x, 
         const int y = labels[row];
         const float zy = __shfl_sync(0xffffffffu, z, y);
         rloss = (float)(lse - (double)zy);
-        if (mine) st(dz + (size_t)row * C + lane, (float)((exp((double)z - lse) - (lane == y ? 1.0 : 0.0)) * (double)scale));
+        if (mine) st(dz + (size_t)row * C + lane, (float)((e / se - (lane == y ? 1.0 : 0.0)) * (double)scale));
     }
     if (lane == 0) wl[warp] = rloss;
     __syncthreads();
@@ -1203,19 +1212,6 @@ __global__ void __launch_bounds__(256) head_fwd_loss_k(const T* __restrict__ x, 
         float s = 0.f;
         for (int i = 0; i < 8; ++i) s += wl[i];
         loss_part[blockIdx.x] = s;
-        __threadfence();
-        last = atomicAdd(counter, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last) {                              // the last CTA adds the partials: 256 lanes, then a fixed tree
-        __threadfence();
-        __shared__ float ls[256];
-        float s = 0.f;
-        for (unsigned i = threadIdx.x; i < gridDim.x; i += 256) s += __ldcg(loss_part + i);
-        ls[threadIdx.x] = s;
-        __syncthreads();
-        for (int d = 128; d > 0; d >>= 1) { if ((int)threadIdx.x < d) ls[threadIdx.x] += ls[threadIdx.x + d]; __syncthreads(); }
-        if (threadIdx.x == 0) { *counter = 0u; publish_loss(rec, ls[0] / (float)M, err, seq); }
     }
 }
 // grid = (ceil(M / HEAD_ROWS_PER_CTA), slices of `kvs` vectors of the K columns): the sums over a CTA's 32 samples are serial chains, so the
@@ -1224,12 +1220,25 @@ __global__ void __launch_bounds__(256) head_fwd_loss_k(const T* __restrict__ x, 
 // gradient), [CTA row][K][2].
 template <typename T>
 __global__ void __launch_bounds__(256) head_bwd_k(const T* __restrict__ x, const T* __restrict__ W, const T* __restrict__ dz, T* dx, float* __restrict__ part,
-                                                  float* __restrict__ col, int M, int K, int C, int kvs, bool accum_dx, bool mask) {
+                                                  float* __restrict__ col, int M, int K, int C, int kvs, bool accum_dx, bool mask, bool staged) {
     constexpr int V = Vec<T>::V;
     const int r0 = blockIdx.x * HEAD_ROWS_PER_CTA, r1 = min(M, r0 + HEAD_ROWS_PER_CTA);
     const int nkv = K / V, kv0 = blockIdx.y * kvs, nk = min(nkv - kv0, kvs);
     __shared__ float dzs[HEAD_ROWS_PER_CTA][HEAD_MAX_C];
     __shared__ float cs[256][V + 1];
+    extern __shared__ __align__(16) char hsm[];
+    // this CTA's part of x and of W; staged (kvs <= HEAD_STAGE_VECS): copies [rows][kvs], [C][kvs] in shared memory
+    const T* xp = x + (size_t)r0 * K + (size_t)kv0 * V;
+    const T* wp = W + (size_t)kv0 * V;
+    size_t pitch = K;
+    if (staged) {
+        uint4* const xs = (uint4*)hsm;
+        for (int i = threadIdx.x; i < (r1 - r0 + C) * kvs; i += 256) {
+            const int r = i / kvs, kv = i - r * kvs;
+            if (kv < nk) xs[i] = *(const uint4*)(r < r1 - r0 ? xp + (size_t)r * K + kv * V : wp + (size_t)(r - (r1 - r0)) * K + kv * V);
+        }
+        xp = (const T*)xs; wp = (const T*)(xs + (size_t)(r1 - r0) * kvs); pitch = (size_t)kvs * V;
+    }
     for (int i = threadIdx.x; i < (r1 - r0) * C; i += 256) dzs[i / C][i % C] = ld(dz + (size_t)r0 * C + i);
     __syncthreads();
     if (dx) {
@@ -1245,7 +1254,7 @@ __global__ void __launch_bounds__(256) head_bwd_k(const T* __restrict__ x, const
                 for (int j = 0; j < V; ++j) a[j] = 0.f;
                 for (int c = 0; c < C; ++c) {
                     float wv[8];
-                    Vec<T>::load(W + (size_t)c * K + (size_t)(kv0 + kv) * V, wv);
+                    Vec<T>::load(wp + c * pitch + kv * V, wv);
                     const float g = dzs[r - r0][c];
 #pragma unroll
                     for (int j = 0; j < V; ++j) a[j] = fmaf(g, wv[j], a[j]);
@@ -1259,7 +1268,7 @@ __global__ void __launch_bounds__(256) head_bwd_k(const T* __restrict__ x, const
                 }
                 if (mask) {
                     float xv[8];
-                    Vec<T>::load(x + (size_t)r * K + (size_t)(kv0 + kv) * V, xv);
+                    Vec<T>::load(xp + (r - r0) * pitch + kv * V, xv);
 #pragma unroll
                     for (int j = 0; j < V; ++j) { if (!(xv[j] > 0.f)) a[j] = 0.f; sum[j] += rounded<T>(a[j]); }
                 }
@@ -1279,20 +1288,20 @@ __global__ void __launch_bounds__(256) head_bwd_k(const T* __restrict__ x, const
     // partial sums: (class, vector of V columns) pairs round-robin over the threads, rows in ascending order
     float* out = part + (size_t)blockIdx.x * C * (K + 1);
     for (int p = threadIdx.x; p < C * nk; p += 256) {
-        const int c = p / nk, kv = kv0 + p - c * nk;
+        const int c = p / nk, kv = p - c * nk;
         float a[8];
 #pragma unroll
         for (int j = 0; j < V; ++j) a[j] = 0.f;
 #pragma unroll 8
         for (int r = r0; r < r1; ++r) {
             float xv[8];
-            Vec<T>::load(x + (size_t)r * K + (size_t)kv * V, xv);
+            Vec<T>::load(xp + (r - r0) * pitch + kv * V, xv);
             const float g = dzs[r - r0][c];
 #pragma unroll
             for (int j = 0; j < V; ++j) a[j] = fmaf(g, xv[j], a[j]);
         }
 #pragma unroll
-        for (int j = 0; j < V; ++j) out[(size_t)c * (K + 1) + kv * V + j] = a[j];
+        for (int j = 0; j < V; ++j) out[(size_t)c * (K + 1) + (kv0 + kv) * V + j] = a[j];
     }
     if (blockIdx.y == 0 && threadIdx.x < C) {
         float a = 0.f;
@@ -1300,8 +1309,20 @@ __global__ void __launch_bounds__(256) head_bwd_k(const T* __restrict__ x, const
         out[(size_t)threadIdx.x * (K + 1) + K] = a;
     }
 }
-// blockDim = (elements, lanes): lane y adds the CTAs y, y + lanes, ...
-__global__ void head_reduce_k(const float* __restrict__ part, float* __restrict__ dW, float* __restrict__ db, int ctas, int K, int C) {
+// blockDim = (elements, lanes): lane y adds the CTAs y, y + lanes, ...  The last CTA: the mean of the M losses from `blocks` partials, for the host.
+__global__ void head_reduce_k(const float* __restrict__ part, float* __restrict__ dW, float* __restrict__ db, int ctas, int K, int C, const float* __restrict__ loss_part,
+                              int blocks, int M, LossRecord* rec, const int* err, long long seq) {
+    if (blockIdx.x == gridDim.x - 1) {
+        __shared__ double ls[256];
+        const int tid = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * blockDim.y;      // nt: a power of two
+        double s = 0.0;
+        for (int i = tid; i < blocks; i += nt) s += (double)loss_part[i];
+        ls[tid] = s;
+        __syncthreads();
+        for (int d = nt / 2; d > 0; d >>= 1) { if (tid < d) ls[tid] += ls[tid + d]; __syncthreads(); }
+        if (tid == 0) publish_loss(rec, (float)(ls[0] / (double)M), err, seq);
+        return;
+    }
     __shared__ float sh[8][32];
     const int i = blockIdx.x * blockDim.x + threadIdx.x, lanes = blockDim.y, n = C * (K + 1);
     float s = 0.f;
@@ -1325,12 +1346,13 @@ size_t head_scratch_elems(int M, int K, int C) {
     const size_t ctas = (M + HEAD_ROWS_PER_CTA - 1) / HEAD_ROWS_PER_CTA;
     return ctas * C * (K + 1) + (M + 7) / 8;
 }
-void head_forward_loss(int dt, const void* x, const void* W, const float* bias, const int32_t* labels, float* logits, void* dlogits, float* scratch,
-                       unsigned* counter, LossRecord* rec, const int* err, long long seq, int M, int K, int C, float scale, cudaStream_t s) {
+void head_forward_loss(int dt, const void* x, const void* W, const float* bias, const int32_t* labels, float* logits, void* dlogits, float* loss_part, int M, int K, int C,
+                       float scale, cudaStream_t s) {
     Scope sc(KC_SOFTMAX_CE, 2.0 * M * K * C, (dt ? 2.0 : 4.0) * ((double)M * K + (double)C * K + (double)M * C) + 4.0 * M * C, s);
     const unsigned grid = (M + 7) / 8;
-    if (dt) klaunch(head_fwd_loss_k<bf16>, grid, 256, 0, s, (const bf16*)x, (const bf16*)W, bias, labels, logits, (bf16*)dlogits, scratch, counter, rec, err, seq, M, K, C, scale);
-    else klaunch(head_fwd_loss_k<float>, grid, 256, 0, s, (const float*)x, (const float*)W, bias, labels, logits, (float*)dlogits, scratch, counter, rec, err, seq, M, K, C, scale);
+    const size_t w_bytes = (size_t)C * K * (dt ? 2 : 4), smem = w_bytes <= HEAD_W_SMEM ? w_bytes : 0;
+    if (dt) klaunch(head_fwd_loss_k<bf16>, grid, 256, smem, s, (const bf16*)x, (const bf16*)W, bias, labels, logits, (bf16*)dlogits, loss_part, M, K, C, scale, smem > 0);
+    else klaunch(head_fwd_loss_k<float>, grid, 256, smem, s, (const float*)x, (const float*)W, bias, labels, logits, (float*)dlogits, loss_part, M, K, C, scale, smem > 0);
 }
 int head_col_records(int M) { return (M + HEAD_ROWS_PER_CTA - 1) / HEAD_ROWS_PER_CTA; }
 void head_backward(int dt, const void* x, const void* W, const void* dlogits, void* dx_or_null, bool accum_dx, bool mask_dx, float* col_or_null, float* scratch, int M,
@@ -1343,16 +1365,19 @@ void head_backward(int dt, const void* x, const void* W, const void* dlogits, vo
     while (kvs < 256 && kvs < nkv) kvs *= 2;
     while (kvs > 8 && ctas * ((nkv + kvs - 1) / kvs) < 148) kvs /= 2;
     const dim3 grid(ctas, (nkv + kvs - 1) / kvs);
+    const bool staged = kvs <= HEAD_STAGE_VECS;
+    const size_t smem = staged ? (size_t)(HEAD_ROWS_PER_CTA + C) * kvs * 16 : 0;
     Scope sc(KC_FMA_WGRAD, (dx_or_null ? 4.0 : 2.0) * M * K * C, (dt ? 2.0 : 4.0) * ((double)M * K * (dx_or_null ? 2 : 1) + (double)C * K + (double)M * C), s);
-    if (dt) klaunch(head_bwd_k<bf16>, grid, 256, 0, s, (const bf16*)x, (const bf16*)W, (const bf16*)dlogits, (bf16*)dx_or_null, scratch, col_or_null, M, K, C, kvs, accum_dx, mask_dx);
-    else klaunch(head_bwd_k<float>, grid, 256, 0, s, (const float*)x, (const float*)W, (const float*)dlogits, (float*)dx_or_null, scratch, col_or_null, M, K, C, kvs, accum_dx, mask_dx);
+    if (dt) klaunch(head_bwd_k<bf16>, grid, 256, smem, s, (const bf16*)x, (const bf16*)W, (const bf16*)dlogits, (bf16*)dx_or_null, scratch, col_or_null, M, K, C, kvs, accum_dx, mask_dx, staged);
+    else klaunch(head_bwd_k<float>, grid, 256, smem, s, (const float*)x, (const float*)W, (const float*)dlogits, (float*)dx_or_null, scratch, col_or_null, M, K, C, kvs, accum_dx, mask_dx, staged);
 }
-void head_reduce(float* dW, float* db_or_null, const float* scratch, int M, int K, int C, cudaStream_t s) {
+void head_reduce(float* dW, float* db_or_null, const float* scratch, const float* loss_part, LossRecord* rec, const int* err, long long seq, int M, int K, int C, cudaStream_t s) {
     const unsigned ctas = (M + HEAD_ROWS_PER_CTA - 1) / HEAD_ROWS_PER_CTA;
     Scope sc(KC_SPLITK, 0.0, 4.0 * (ctas + 1) * C * (K + 1), s);
     // from 65 partial matrices on eight threads per element (512 of them, 2570 elements: 62 us with one, 10 so; 68: 15 and 7)
-    if (ctas > 64) klaunch(head_reduce_k, cdiv((size_t)C * (K + 1), 32), dim3(32, 8), 0, s, scratch, dW, db_or_null, (int)ctas, K, C);
-    else klaunch(head_reduce_k, cdiv((size_t)C * (K + 1), 64), 64, 0, s, scratch, dW, db_or_null, (int)ctas, K, C);
+    const bool many = ctas > 64;
+    klaunch(head_reduce_k, cdiv((size_t)C * (K + 1), many ? 32 : 64) + 1, many ? dim3(32, 8) : dim3(64), 0, s, scratch, dW, db_or_null, (int)ctas, K, C, loss_part, (M + 7) / 8, M, rec,
+            err, seq);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -134,18 +134,19 @@ void softmax_ce(int dt, const float* logits, const int32_t* labels, void* dlogit
                 float scale, cudaStream_t st);
 
 // Classifier head (the last linear layer, c_in = K -> C classes, C <= 16) fused with the loss.  head_forward_loss: logits
-// (fp32), dlogits = (softmax - onehot) * scale (storage dtype) and the mean loss in one launch; `counter` is a device word
-// that is zero between launches.  head_backward: dx (+)= dlogits W (dx_or_null == nullptr: not needed) and the
-// partial sums of dW, db, which head_reduce adds; mask_dx, col: see below.
-// scratch: head_scratch_elems floats, used by both (the loss partials follow the weight-gradient partials).
+// (fp32), dlogits = (softmax - onehot) * scale (storage dtype) and partial sums of the loss in one launch.  head_backward: dx (+)= dlogits W
+// (dx_or_null == nullptr: not needed) and the partial sums of dW, db, which head_reduce adds, with those of the loss; mask_dx, col: see above.
+// scratch: head_scratch_elems floats: the weight-gradient partials, then the loss partials.
 bool   head_supported(int dt, int K, int C);
 size_t head_scratch_elems(int M, int K, int C);
-void   head_forward_loss(int dt, const void* x, const void* W, const float* bias, const int32_t* labels, float* logits, void* dlogits, float* scratch,
-                         unsigned* counter, LossRecord* rec, const int* err, long long seq, int M, int K, int C, float scale, cudaStream_t st);
+void   head_forward_loss(int dt, const void* x, const void* W, const float* bias, const int32_t* labels, float* logits, void* dlogits, float* loss_part, int M, int K, int C,
+                         float scale, cudaStream_t st);
 int    head_col_records(int M);
 void   head_backward(int dt, const void* x, const void* W, const void* dlogits, void* dx_or_null, bool accum_dx, bool mask_dx, float* col_or_null, float* scratch, int M,
                      int K, int C, cudaStream_t st);
-void   head_reduce(float* dW, float* db_or_null, const float* scratch, int M, int K, int C, cudaStream_t st);        // what head_backward left in scratch
+// what head_backward left in scratch, and the mean loss
+void   head_reduce(float* dW, float* db_or_null, const float* scratch, const float* loss_part, LossRecord* rec, const int* err, long long seq, int M, int K, int C,
+                   cudaStream_t st);
 
 // master -= lr * grad (skipped when grad == nullptr: w(t+1) = w(t)); copy_next = storage-dtype copy of
 // the new master (the next weight version).  n must be a multiple of 4; pointers 16-byte aligned.
