@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(FW_THREADS, 3) fw_kernel(const T* __restrict__
     }
 }
 
-// dW[c_out][tap][c_in] = sum over the splits (at most 444): 8 lanes per element take every 8th split, eight loads in flight each, then a
+// dW[c_out][tap][c_in] = sum over the splits (at most 592): 8 lanes per element take every 8th split, eight loads in flight each, then a
 // fixed tree.  S: what they are added in.
 template <typename S>
 __global__ void __launch_bounds__(256) fw_reduce_kernel(const float* __restrict__ part, float* __restrict__ dw, int splits, int nout, int ntaps, int cw, int ci_blocks,
@@ -595,7 +595,7 @@ void dispatch_fc(const void* x, const void* w, const float* bias, void* y, float
 }  // namespace
 
 // Weight gradient: 128 pixels per tile (64 for 3x3 stride 2, whose input region is four times its output).
-bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_t& smem) {
+bool plan_fw(const ConvGeom& g, int groups, int ctas, FwParams& p, int& G, int& run, size_t& smem) {
     if ((g.H * g.W == 1 && g.R == 1) || (g.R != 3 && g.R != 1) || (g.stride != 1 && g.stride != 2) || g.N % groups) return false;
   for (int pixels = g.R == 3 && g.stride == 2 ? 64 : 128; pixels >= 32; pixels /= 2) {        // smaller tiles where the halo of tiny images outgrows shared memory
     p = FwParams{};
@@ -618,8 +618,8 @@ bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_
     p.pps = npix / p.nslices;
     p.ci_blocks = (g.C + FW_CI - 1) / FW_CI;
     const int blocks = p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO) * groups;
-    // three CTAs per SM once around the device, each with at least one tile
-    int want = FW_CTAS / blocks;
+    // once around the device, each CTA with at least one tile
+    int want = ctas / blocks;
     if (want > p.tiles) want = p.tiles;
     if (want < 1) want = 1;
     const int per = (p.tiles + want - 1) / want;
@@ -661,7 +661,7 @@ void dispatch_fw(const void* x, const void* dy, float* ws, const FwParams& p, in
 
 bool fconv_supported(const ConvGeom& g) {
     FcParams p; FwParams q; int G, run; size_t smem;
-    return plan_fc(g, 1, false, p) && plan_fc(g, 1, true, p) && plan_fw(g, 1, q, G, run, smem);
+    return plan_fc(g, 1, false, p) && plan_fc(g, 1, true, p) && plan_fw(g, 1, FW_CTAS, q, G, run, smem);
 }
 bool fconv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
                    float* stat, const Packed& pk, cudaStream_t s) {
@@ -690,14 +690,14 @@ int fconv_stat_tiles(const ConvGeom& g, int groups) {
 }
 size_t fconv_wgrad_workspace_elems(const ConvGeom& g, int groups) {
     FwParams p; int G, run; size_t smem;
-    if (!plan_fw(g, groups, p, G, run, smem)) return 0;
+    if (!plan_fw(g, groups, FW_CTAS, p, G, run, smem)) return 0;
     // a window of the batch may be cut into other tiles, but never uses more splits than fill the device
     const int blocks = p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO) * groups;
-    return (size_t)blocks * (FW_CTAS > blocks ? FW_CTAS / blocks : 1) * FW_CO * p.ntaps * 8 * G;
+    return (size_t)blocks * (MW_CTAS > blocks ? MW_CTAS / blocks : 1) * FW_CO * p.ntaps * 8 * G;
 }
 bool fconv_wgrad(int dt, const void* x, const void* dy, float* dw, float* ws, const ConvGeom& g, int groups, size_t w_group, bool accum, bool tensor, cudaStream_t s) {
     FwParams p; int G, run; size_t smem;
-    if (!plan_fw(g, groups, p, G, run, smem)) return false;
+    if (!plan_fw(g, groups, FW_CTAS, p, G, run, smem)) return false;
     const int xs = g.R == 1 ? 1 : g.stride, blocks = p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO), nout = FW_CO * p.ntaps * 8 * G;
     const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
     {

@@ -17,7 +17,7 @@ constexpr int FC_KC = 16;                // channels per chunk
 constexpr int PITCH = 20;                // floats per pixel (or weight row) in shared memory: 16 + 4, so that the eight 16-byte reads
                                          // of neighbouring pixels fall into different banks
 constexpr int FW_CO = 16, FW_CI = 16;
-constexpr int FW_CTAS = 3 * 148;
+constexpr int FW_CTAS = 3 * 148, MW_CTAS = 4 * 148;      // of a weight gradient, fconv.cu's and mconv.cu's: as many as the device holds at a time
 constexpr size_t FC_SMEM_MAX = 224 * 1024;
 
 struct FcParams {
@@ -49,8 +49,8 @@ struct FwParams {
 
 // Geometry of a forward (back == false) or input-gradient launch over `groups` groups of g.N / groups images; false: not covered.
 bool plan_fc(const ConvGeom& g, int groups, bool back, FcParams& p);
-// Of a weight gradient; smem: of fw_kernel.
-bool plan_fw(const ConvGeom& g, int groups, FwParams& p, int& G, int& run, size_t& smem);
+// Of a weight gradient by `ctas` CTAs; smem: of fw_kernel.
+bool plan_fw(const ConvGeom& g, int groups, int ctas, FwParams& p, int& G, int& run, size_t& smem);
 
 // The tensor-core forms (mconv.cu), tried first by the fconv_* functions; false / 0: not covered or refused, nothing launched.
 // mconv_wgrad leaves partial matrices as fw_kernel does and returns their number per block.

@@ -10,8 +10,9 @@
 // a product the sum of the six that matter: lo hi + mid mid + hi lo + mid hi + hi mid + hi hi (the rest is 6e-9 of it; 6e-8, and one-sided, with parts by
 // truncation).  Every product is exact; an mma adds 16 of them to its running sum and truncates to 24 bits of the largest term: 2.5e-8 of the
 // result's rms for 16 fresh products of 16 bits, 1.3e-7 for nine such steps in a chain, 5.3e-7 for 36, 1e-7 as soon as a 24-bit running sum of
-// like size is among the terms.  So hi hi starts from zero in every step and goes into an fp32 sum on the CUDA cores, one per 16-channel chunk (9 steps) or
-// four steps of a weight gradient, and that one into a compensated (Kahan) sum; the other five, 2^-8 of it, run on in one accumulator per chunk.
+// like size is among the terms.  So hi hi starts from zero in every step and goes into an fp32 sum on the CUDA cores, one per 16-channel chunk (9
+// steps), and that one into a compensated (Kahan) sum, in a weight gradient of fp32
+// storage straight into the latter (four CTAs per SM have no registers for both); the other five, 2^-8 of it, run on in one accumulator per chunk.
 // Error against double sums, of the result's rms (normal data; packed-FMA kernels of fconv.cu beside it): forward and input gradient 3x3 5.4e-8 to
 // 7.0e-8 (7.6e-8), 1x1 3.6e-8 to 4.7e-8 (6.1e-8), weight gradients 4.8e-8 to 6.2e-8 (5.6e-8 to 1.1e-7).  Two fp16 parts and three products were off by 9.4e-8:
 // 22-bit products lose more where the terms are aligned.  bf16 storage: one exact product a step.
@@ -335,7 +336,7 @@ template <typename T> constexpr int mw_smem(int npix, int xp) { return (npix + x
 
 // grid = (splits, c_out blocks x c_in blocks, groups).  part_out: [group][block][split][16 c_out][taps][16 c_in], as fw_kernel's.
 template <typename T, int XS, int TW>
-__global__ void __launch_bounds__(MW_WARPS * 32, 3) mw_kernel(const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ part_out,
+__global__ void __launch_bounds__(MW_WARPS * 32, SPLIT<T> ? 4 : 3) mw_kernel(const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ part_out,
                                                               const __grid_constant__ MwParams q) {
     constexpr bool S = SPLIT<T>;
     constexpr int SL = mw_slices(TW);
@@ -373,13 +374,6 @@ __global__ void __launch_bounds__(MW_WARPS * 32, 3) mw_kernel(const T* __restric
         }
         cp_commit();
     };
-    // what a few steps have added up goes into the compensated sum
-    auto flush = [](float2 (&acc)[TW][2], float2 (&sum)[TW][2], float2 (&lost)[TW][2]) {
-#pragma unroll
-        for (int s = 0; s < TW; ++s)
-#pragma unroll
-            for (int r = 0; r < 2; ++r) { add_kahan(sum[s][r], lost[s][r], acc[s][r]); acc[s][r] = make_float2(0.f, 0.f); }
-    };
     auto region_pixel = [&](int px) { return ((px >> (p.lw + p.lh)) * p.RH + ((px >> p.lw) & (p.Ht - 1)) * XS) * p.RW + (px & (p.Wt - 1)) * XS; };
     if (tile0 < tile_end) fetch(tile0, 0);
     for (int tile = tile0; tile < tile_end; ++tile) {
@@ -398,12 +392,12 @@ __global__ void __launch_bounds__(MW_WARPS * 32, 3) mw_kernel(const T* __restric
         const uint32_t dbase = smem_addr(pd_) + (S ? 0 : buf * npix * 32) + (((lane >> 3) & 1) * npix + (lane & 7) + 8 * (lane >> 4)) * 16;
         // rows of x that this lane hands to ldmatrix: pixel lane % 16; lanes 16..31 those of the second part (fp32), nobody's (bf16)
         const uint32_t xbase = smem_addr(px_) + (S ? 0 : buf * xp * 32) + (half * xp + p.toff[tap0]) * 16;
-        float2 acc[TW][2];                           // this tile's sum of hi hi
-        float rest[TW][4];                           // fp32 storage: of the other products
+        float rest[TW][4];                           // fp32 storage: this tile's sum of all products but hi hi
+        float2 acc[TW][2];                           // bf16 storage: this tile's sum
 #pragma unroll
         for (int s = 0; s < TW; ++s) {
-            acc[s][0] = acc[s][1] = make_float2(0.f, 0.f);
             rest[s][0] = rest[s][1] = rest[s][2] = rest[s][3] = 0.f;
+            acc[s][0] = acc[s][1] = make_float2(0.f, 0.f);
         }
 #pragma unroll 1
         for (int ks = slice; ks * 16 < npix; ks += SL) {
@@ -431,10 +425,16 @@ __global__ void __launch_bounds__(MW_WARPS * 32, 3) mw_kernel(const T* __restric
 #pragma unroll
             for (int s = 0; s < TW; ++s)
 #pragma unroll
-                for (int r = 0; r < 2; ++r) acc[s][r] = __fadd2_rn(acc[s][r], make_float2(part[s][2 * r], part[s][2 * r + 1]));
-            if (S && (ks & 3) == 3) flush(acc, sum, lost);
+                for (int r = 0; r < 2; ++r) {
+                    const float2 v = make_float2(part[s][2 * r], part[s][2 * r + 1]);
+                    if (S) add_kahan(sum[s][r], lost[s][r], v); else acc[s][r] = __fadd2_rn(acc[s][r], v);
+                }
         }
-        flush(acc, sum, lost);
+        if (!S)
+#pragma unroll
+            for (int s = 0; s < TW; ++s)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) add_kahan(sum[s][r], lost[s][r], acc[s][r]);
         if (S)
 #pragma unroll
             for (int s = 0; s < TW; ++s)
@@ -516,7 +516,7 @@ bool plan_mc(const ConvGeom& g, int groups, bool back, McParams& q) {
 template <typename T>
 bool plan_mw(const ConvGeom& g, int groups, MwParams& q, size_t& smem) {
     int G, run; size_t fw;
-    if (!channels_ok(g) || !plan_fw(g, groups, q.p, G, run, fw)) return false;
+    if (!channels_ok(g) || !plan_fw(g, groups, SPLIT<T> ? MW_CTAS : FW_CTAS, q.p, G, run, fw)) return false;
     q.npix = q.p.Wt * q.p.Ht * q.p.Nt;
     q.xp = q.p.x_floats / PITCH;
     for (int i = 0; i < q.p.ntaps; ++i) q.p.toff[i] /= PITCH;
