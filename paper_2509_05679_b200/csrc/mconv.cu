@@ -23,6 +23,8 @@
 #include "fconv.h"
 #include "launch.h"
 
+#include <algorithm>
+
 namespace fdg {
 
 namespace {
@@ -537,6 +539,12 @@ template <typename T>
 bool run_mc(const void* x, const void* pk, const float* bias, void* y, float* stat, const ConvGeom& g, int epi, int groups, size_t b_group, size_t pack_group, bool back, cudaStream_t s) {
     McParams q;
     if (!plan_mc<T>(g, groups, back, q)) return false;
+    // Left to the packed-FMA kernel: tiles of many short rows (images of 3x3 and smaller; a warp fetches row by row: 2x2, 64 channels, fp32 41 us against 35, 3x3,
+    // 16 channels 43 against 23, 1x1 in bf16 22.7 against 20.6, but 2x2 in bf16 31 against 47), and fp32 1x1 stride 2, which would split four pixels
+    // for each that it uses, from two chunks on (8x8 256 -> 512 64 us against 51, 16x16 32 -> 64 8.9 against 8.3; one chunk 10.5 against 14.5).
+    int rows = 0;
+    for (int c = 0; c < q.p.ncls; ++c) rows = std::max(rows, q.p.Nt * q.p.cls_rh[c]);
+    if (rows > (SPLIT<T> ? 64 : 128) || (SPLIT<T> && q.p.taps == 1 && q.p.xs == 2 && q.p.C > FC_KC)) return false;
     q.p.epi = epi; q.p.b_group = b_group;
     q.pack_group = pack_group / 16;
     const long tiles = (long)q.p.tiles_w * q.p.tiles_h * ((q.p.ngroup + q.p.Nt - 1) / q.p.Nt) * groups * q.p.ncls;
