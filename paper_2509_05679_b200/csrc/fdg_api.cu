@@ -1003,7 +1003,6 @@ bool backward_op_replicas(fdg_ctx* c, int kk, int64_t batch, int64_t version, in
 void backward_module(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t) {
     Module& m = c->mod[kk];
     const int n = (int)m.ops.size();
-    pack_weights(c, m, version, true, m.stream);
     if (c->R == 1) {
         for (int g = 0; g < m.groups; ++g) backward_ops(c, kk, batch, version, t, g, 0, n);
         return;
@@ -1244,6 +1243,7 @@ fdg_status module_step(fdg_ctx* ctx, int kk, int64_t t, const Ingest* in, int pa
     tg.fwd_batch = tau_f >= 0 ? tau_f : -1; tg.bwd_batch = tau_b >= 0 ? tau_b : -1; tg.version_now = t;
     tg.trace = m.trace; tg.time_start = m.stamps;
     tags_step(tg, m.stream);
+    if (tau_b >= 0) pack_weights(ctx, m, v_b, true, m.stream);      // in front of the last module's wait for its forward pass
     }
 
     if (part & FORWARD) {
@@ -1279,6 +1279,8 @@ fdg_status module_step(fdg_ctx* ctx, int kk, int64_t t, const Ingest* in, int pa
     } else if (m.fused_update) {
         Scope sc(KC_SGD, 0.0, (double)npar(m) * (tau_b >= 0 ? 12.0 : 4.0) + 2.0 * m.n_big + 4.0 * m.n_small + 2.0 * m.n_big, m.stream);
         CK(tc::run_update_module(m.upd, m.master, m.grad, wslot(ctx, m, t + 1), wtslot(m, t + 1, 0), wsmall(ctx, m, t + 1, 0), ctx->lr, tau_b >= 0, end, m.stream));
+    } else if (ctx->dt == 0) {                              // matrices and vectors follow each other in the master, the gradient and the ring slot: one launch
+        sgd_update(0, m.master, tau_b >= 0 ? m.grad : nullptr, wslot(ctx, m, t + 1), npar(m), ctx->lr, end, m.stream);
     } else {
         // the last launch takes the time
         sgd_update(ctx->dt, m.master, tau_b >= 0 ? m.grad : nullptr, wslot(ctx, m, t + 1), m.n_big, ctx->lr, nullptr, m.stream);
