@@ -14,11 +14,11 @@
 // steps), and that one into a compensated (Kahan) sum, in a weight gradient of fp32
 // storage straight into the latter (four CTAs per SM have no registers for both); the other five, 2^-8 of it, run on in one accumulator per chunk.
 // Error against double sums, of the result's rms (normal data; packed-FMA kernels of fconv.cu beside it): forward and input gradient 3x3 5.4e-8 to
-// 7.0e-8 (7.6e-8), 1x1 3.6e-8 to 4.7e-8 (6.1e-8), weight gradients 4.8e-8 to 6.2e-8 (5.6e-8 to 1.1e-7).  Two fp16 parts and three products were off by 9.4e-8:
+// 7.0e-8 (7.6e-8), 1x1 3.6e-8 to 4.7e-8 (6.1e-8), weight gradients 4.7e-8 to 5.5e-8 (5.6e-8 to 1.1e-7).  Two fp16 parts and three products were off by 9.4e-8:
 // 22-bit products lose more where the terms are aligned.  bf16 storage: one exact product a step.
 //
 // Time, 192 images, launch included (packed FMA beside it): fp32 32x32 16 -> 16 forward 23 us (38), weight gradient with its reduction 37 (54); 16x16 32 -> 32 23
-// (40), 35 (53); 8x8 64 -> 64 27 (41), 41 (57).  What bounds them: a third to 40 % of the mma.sync rate (980 multiply-adds per clock and SM, six per
+// (40), 35 (53); 8x8 64 -> 64 27 (41), 39 (57).  What bounds them: a third to 40 % of the mma.sync rate (980 multiply-adds per clock and SM, six per
 // product), the rest is latency of one warp's chain (fixed-latency waits, ncu) and the splitting, which every block of 16 or 32 output channels repeats.
 #include "fconv.h"
 #include "launch.h"
