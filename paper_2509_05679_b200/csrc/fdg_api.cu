@@ -114,7 +114,8 @@ struct Module {
     float *master, *grad, *ws, *lin_ws, *scratch, *red, *cstat[2], *bstat;
     size_t lin_elems;
     size_t pack_bytes;             // the weights of the convolutions of mconv.cu, per replica, as their kernels read them: of the version that the forward /
-    char *pack_f, *pack_b;         // the backward pass is at, laid out at its beginning
+    char *pack_f, *pack_b;         // the backward pass is at, laid out at its beginning,
+    bool pack_f_ok, pack_b_ok;     // if that launch was not refused (the packed-FMA kernels read the weights themselves)
     struct Pack { PackArgs args; int blocks; };
     std::vector<Pack> packs;
     bool fused_update;             // one kernel per step updates all parameters and emits the next weight version (both layouts)
@@ -577,7 +578,6 @@ Win group_window(const fdg_ctx* c, const Module& m, int g) {
 }
 
 // A launch that was refused is made up for by other kernels: its error is not kept.
-bool launched(cudaError_t e) { if (e != cudaSuccess) cudaGetLastError(); return e == cudaSuccess; }
 
 bool tc_forward(fdg_ctx* c, Module& m, const Op& o, char* x_base, char* y_base, int64_t version, const Win& wn, cudaStream_t s) {
     int ia = find_buf(o.a_ptrs, x_base);
@@ -674,13 +674,15 @@ size_t row_off(const fdg_ctx* c, const TensorDesc& d, const Win& wn) {
 
 // The weights of version `version` for one pass of the convolutions in mconv.cu: one launch for all of a module's (up to PackArgs::MAX).
 void pack_weights(fdg_ctx* c, Module& m, int64_t version, bool back, cudaStream_t s) {
+    bool& ok = back ? m.pack_b_ok : m.pack_f_ok;
+    ok = true;
     for (const Module::Pack& k : m.packs) {
         PackArgs a = k.args; a.back = back;
-        mconv_pack(c->dt, wbig(c, m, version, 0), m.wslot_bytes / c->esz, back ? m.pack_b : m.pack_f, m.pack_bytes, a, k.blocks, c->R, s);
+        ok = mconv_pack(c->dt, wbig(c, m, version, 0), m.wslot_bytes / c->esz, back ? m.pack_b : m.pack_f, m.pack_bytes, a, k.blocks, c->R, s) && ok;
     }
 }
-Packed packed_f(const Module& m, const Op& o, int rep) { return o.packed ? Packed{m.pack_f + rep * m.pack_bytes + o.pack_off, m.pack_bytes} : Packed{}; }
-Packed packed_b(const Module& m, const Op& o, int rep) { return o.packed ? Packed{m.pack_b + rep * m.pack_bytes + o.pack_off, m.pack_bytes} : Packed{}; }
+Packed packed_f(const Module& m, const Op& o, int rep) { return o.packed && m.pack_f_ok ? Packed{m.pack_f + rep * m.pack_bytes + o.pack_off, m.pack_bytes} : Packed{}; }
+Packed packed_b(const Module& m, const Op& o, int rep) { return o.packed && m.pack_b_ok ? Packed{m.pack_b + rep * m.pack_bytes + o.pack_off, m.pack_bytes} : Packed{}; }
 // all groups of a launch read the same weights
 Packed shared(Packed p) { p.group = 0; return p; }
 

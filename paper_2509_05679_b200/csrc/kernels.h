@@ -42,7 +42,7 @@ struct Packed { const void* data; size_t group; };       // data == nullptr: the
 struct PackLayer { size_t w_off, out_off; int C, Co, taps, block0; };        // elements into the matrices, 16-byte words into the result; first block
 struct PackArgs { enum { MAX = 48 }; PackLayer layer[MAX]; int n, back; };
 size_t mconv_pack_bytes(int dt, const ConvGeom& g, int groups);
-void   mconv_pack(int dt, const void* wbig, size_t w_group, void* out, size_t out_group, const PackArgs& a, int blocks, int groups, cudaStream_t st);
+bool   mconv_pack(int dt, const void* wbig, size_t w_group, void* out, size_t out_group, const PackArgs& a, int blocks, int groups, cudaStream_t st);      // false: refused
 bool   fconv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
                      float* stat_or_null, const Packed& pk, cudaStream_t st);
 // Batch-norm statistics taken along by fconv_forward (groups = workers): per worker and pixel tile the channels' (mean, sum of

@@ -56,6 +56,8 @@ cudaError_t allow_smem(OncePerDevice& once, const void* kernel, int bytes);
 
 // cluster: CTAs per cluster along x (0: none)
 cudaError_t launch_raw(const void* func, dim3 grid, dim3 block, size_t smem, cudaStream_t s, void** args, const size_t* sizes, int nargs, int cluster);
+// Whether a launch went through.  A refused one leaves no error behind: its caller has another way, and the next launch is not to be blamed for it.
+inline bool launched(cudaError_t e) { if (e != cudaSuccess) cudaGetLastError(); return e == cudaSuccess; }
 // the order between streams inside one module's step: nothing to do while a graph is only refreshed
 cudaError_t step_record(cudaEvent_t e, cudaStream_t s);
 cudaError_t step_wait(cudaStream_t s, cudaEvent_t e);

@@ -552,7 +552,7 @@ bool run_mc(const void* x, const void* pk, const float* bias, void* y, float* st
     // large regions (stride 2) leave an SM two CTAs at the most either way
     const auto waves = [](long ctas) { return (ctas + 147) / 148; };
     const bool wide = q.p.Co % 32 == 0 && (mc_smem<T, 2>(q) > 75 * 1024 || 2 * waves(tiles * (q.p.Co / 32)) <= 1.15 * waves(tiles * (q.p.Co / 16)));
-    return (wide ? launch_mc<T, 4>(x, pk, bias, y, stat, q, groups, s) : launch_mc<T, 2>(x, pk, bias, y, stat, q, groups, s)) == cudaSuccess;
+    return launched(wide ? launch_mc<T, 4>(x, pk, bias, y, stat, q, groups, s) : launch_mc<T, 2>(x, pk, bias, y, stat, q, groups, s));
 }
 template <typename T, int XS, int TW>
 cudaError_t launch_mw(const void* x, const void* dy, float* ws, const MwParams& q, int groups, int blocks, size_t smem, cudaStream_t s) {
@@ -569,7 +569,7 @@ int run_mw(const void* x, const void* dy, float* ws, const ConvGeom& g, int grou
     if (g.R == 1) e = launch_mw<T, 1, 1>(x, dy, ws, q, groups, blocks, smem, s);
     else if (g.stride == 1) e = launch_mw<T, 1, 3>(x, dy, ws, q, groups, blocks, smem, s);
     else e = launch_mw<T, 2, 3>(x, dy, ws, q, groups, blocks, smem, s);
-    return e == cudaSuccess ? q.p.splits : 0;
+    return launched(e) ? q.p.splits : 0;
 }
 
 }  // namespace
@@ -581,10 +581,10 @@ size_t mconv_pack_bytes(int dt, const ConvGeom& g, int groups) {
     const size_t blocks = (size_t)(g.C / 16) * (g.Co / 16);
     return blocks * g.R * g.R * (dt ? PACK16<bf16> : PACK16<float>) * 16;
 }
-void mconv_pack(int dt, const void* wbig, size_t w_group, void* out, size_t out_group, const PackArgs& a, int blocks, int groups, cudaStream_t s) {
+bool mconv_pack(int dt, const void* wbig, size_t w_group, void* out, size_t out_group, const PackArgs& a, int blocks, int groups, cudaStream_t s) {
     Scope sc(KC_TC_AUX, 0.0, (double)blocks * groups * 9 * 256 * (dt ? 4.0 : 8.0), s);
-    if (dt) klaunch(mc_pack_kernel<bf16>, dim3(blocks, groups), 256, 0, s, (const bf16*)wbig, w_group, (uint4*)out, out_group / 16, a);
-    else klaunch(mc_pack_kernel<float>, dim3(blocks, groups), 256, 0, s, (const float*)wbig, w_group, (uint4*)out, out_group / 16, a);
+    return launched(dt ? klaunch(mc_pack_kernel<bf16>, dim3(blocks, groups), 256, 0, s, (const bf16*)wbig, w_group, (uint4*)out, out_group / 16, a)
+                       : klaunch(mc_pack_kernel<float>, dim3(blocks, groups), 256, 0, s, (const float*)wbig, w_group, (uint4*)out, out_group / 16, a));
 }
 bool mconv_forward(int dt, const void* x, const void* pack, const float* bias, void* y, float* stat, const ConvGeom& g, int epi, int groups, size_t b_group, size_t pack_group,
                    cudaStream_t s) {

@@ -1,0 +1,91 @@
+"""Host side of csrc/mconv.cu and csrc/fconv.cu without a GPU: their objects linked against a runtime that records launches and refuses the
+ones it is told to."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2509_05679_b200 import build
+
+FAKE = r"""
+#include "kernels.h"
+#include "launch.h"
+#include <cstdio>
+#include <cstdlib>
+using namespace fdg;
+
+static cudaError_t last = cudaSuccess;      // CUDA's last error
+static int refuse = 0;                      // this many launches are refused
+static std::vector<const void*> ran;        // kernels of the others
+extern "C" {
+cudaError_t cudaGetLastError() { const cudaError_t e = last; last = cudaSuccess; return e; }
+cudaError_t cudaLaunchKernel(const void*, dim3, dim3, void**, size_t, cudaStream_t) { abort(); }
+void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
+void __cudaRegisterFatBinaryEnd(void**) {}
+void __cudaUnregisterFatBinary(void**) {}
+void __cudaRegisterFunction(void**, const char*, char*, const char*, int, void*, void*, void*, void*, int*) {}
+unsigned __cudaPopCallConfiguration(dim3*, dim3*, size_t*, void*) { return 0; }
+}
+namespace fdg {
+cudaError_t allow_smem(OncePerDevice&, const void*, int) { return cudaSuccess; }
+cudaError_t launch_raw(const void* f, dim3, dim3, size_t, cudaStream_t, void**, const size_t*, int, int) {
+    if (refuse > 0) { --refuse; return last = cudaErrorInvalidConfiguration; }
+    ran.push_back(f);
+    return cudaSuccess;
+}
+Scope::Scope(int, double, double, cudaStream_t) {}
+Scope::~Scope() {}
+}
+static ConvGeom conv(int n, int h, int w, int c, int co, int r, int stride) {
+    ConvGeom g{}; g.N = n; g.H = h; g.W = w; g.C = c; g.Co = co; g.R = r; g.stride = stride; g.pad = r == 3;
+    g.Ho = (h + 2 * g.pad - r) / stride + 1; g.Wo = (w + 2 * g.pad - r) / stride + 1;
+    return g;
+}
+#define CHECK(x) do { if (!(x)) { printf("line %d: %s\n", __LINE__, #x); return 1; } } while (0)
+"""
+
+REFUSED = r"""
+int main() {
+    alignas(16) static char b[16];
+    const ConvGeom g = conv(8, 16, 16, 32, 32, 3, 1);
+    const Packed pk{b, 0};
+    PackArgs a{}; a.n = 1; a.layer[0] = PackLayer{0, 0, 32, 32, 9, 0};
+    for (int dt = 0; dt < 2; ++dt) {
+        // taken: one launch, the tensor-core kernel's
+        CHECK(fconv_forward(dt, b, b, nullptr, b, g, 0, 1, 0, 0, nullptr, pk, 0) && ran.size() == 1);
+        const void* const tensor = ran[0]; ran.clear();
+        // refused: the packed-FMA kernel computes the same layer, and nobody finds an error afterwards
+        refuse = 1;
+        CHECK(fconv_forward(dt, b, b, nullptr, b, g, 0, 1, 0, 0, nullptr, pk, 0));
+        CHECK(ran.size() == 1 && ran[0] != tensor && last == cudaSuccess); ran.clear();
+        refuse = 1;
+        CHECK(fconv_dgrad(dt, b, b, b, g, 0, 1, 0, pk, 0) && ran.size() == 1 && ran[0] != tensor && last == cudaSuccess); ran.clear();
+        refuse = 1;
+        CHECK(fconv_wgrad(dt, b, b, (float*)b, (float*)b, g, 1, 0, false, true, 0) && ran.size() == 2 && last == cudaSuccess); ran.clear();    // and its reduction
+        // the layout of the weights says whether it is there
+        CHECK(mconv_pack(dt, b, 0, b, 0, a, 4, 1, 0) && ran.size() == 1); ran.clear();
+        refuse = 1;
+        CHECK(!mconv_pack(dt, b, 0, b, 0, a, 4, 1, 0) && ran.empty() && last == cudaSuccess);
+    }
+    return 0;
+}
+"""
+
+
+def run(tmp_path, program):
+    inc = "/usr/local/cuda/include"
+    if not os.path.exists(os.path.join(inc, "cuda_runtime.h")):
+        pytest.skip("no CUDA headers")
+    build.build_lib()
+    objs = [os.path.join(build.CSRC, f) for f in ("mconv.o", "fconv.o")]
+    if not all(os.path.exists(o) for o in objs):
+        pytest.skip("the library was built elsewhere: no objects")
+    src, exe = tmp_path / "t.cpp", tmp_path / "t"
+    src.write_text(FAKE + program)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", inc, "-I", build.CSRC, str(src), *objs, "-o", str(exe)])
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
+
+
+def test_a_refused_launch_is_made_up_for(tmp_path):
+    run(tmp_path, REFUSED)
