@@ -700,15 +700,17 @@ bool fconv_wgrad(int dt, const void* x, const void* dy, float* dw, float* ws, co
     if (!plan_fw(g, groups, FW_CTAS, p, G, run, smem)) return false;
     const int xs = g.R == 1 ? 1 : g.stride, blocks = p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO), nout = FW_CO * p.ntaps * 8 * G;
     const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
+    int splits;
     {
         Scope sc(KC_FMA_WGRAD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + rows * g.Co) + 4.0 * K * g.Co, s);
-        const int splits = tensor ? mconv_wgrad(dt, x, dy, ws, g, groups, s) : 0;
+        splits = tensor ? mconv_wgrad(dt, x, dy, ws, g, groups, s) : 0;
         if (splits) p.splits = splits;
         else if (dt) dispatch_fw<bf16>(x, dy, ws, p, xs, G, run, groups, smem, s); else dispatch_fw<float>(x, dy, ws, p, xs, G, run, groups, smem, s);
     }
     Scope sc(KC_SPLITK, 0.0, 4.0 * groups * (p.splits + 1) * blocks * nout, s);
     const dim3 rgrid((nout + 31) / 32, blocks, groups);
-    if (dt) klaunch(fw_reduce_kernel<FwSum<bf16>::type>, rgrid, 256, 0, s, ws, dw, p.splits, nout, p.ntaps, 8 * G, p.ci_blocks, g.C, g.Co, w_group, accum);
+    // bf16: the packed-FMA kernel's partial matrices in fp32, mconv.cu's in double (in fp32 the error was up to 1.1 times that of the former); one is only copied
+    if (dt && splits <= 1) klaunch(fw_reduce_kernel<FwSum<bf16>::type>, rgrid, 256, 0, s, ws, dw, p.splits, nout, p.ntaps, 8 * G, p.ci_blocks, g.C, g.Co, w_group, accum);
     else klaunch(fw_reduce_kernel<FwSum<float>::type>, rgrid, 256, 0, s, ws, dw, p.splits, nout, p.ntaps, 8 * G, p.ci_blocks, g.C, g.Co, w_group, accum);
     return true;
 }

@@ -10,15 +10,22 @@
 // a product the sum of the six that matter: lo hi + mid mid + hi lo + mid hi + hi mid + hi hi (the rest is 6e-9 of it; 6e-8, and one-sided, with parts by
 // truncation).  Every product is exact; an mma adds 16 of them to its running sum and truncates to 24 bits of the largest term: 2.5e-8 of the
 // result's rms for 16 fresh products of 16 bits, 1.3e-7 for nine such steps in a chain, 5.3e-7 for 36, 1e-7 as soon as a 24-bit running sum of
-// like size is among the terms.  So hi hi starts from zero in every step and goes into an fp32 sum on the CUDA cores, one per 16-channel chunk (9
-// steps), and that one into a compensated (Kahan) sum, in a weight gradient of fp32
-// storage straight into the latter (four CTAs per SM have no registers for both); the other five, 2^-8 of it, run on in one accumulator per chunk.
-// Error against double sums, of the result's rms (normal data; packed-FMA kernels of fconv.cu beside it): forward and input gradient 3x3 5.4e-8 to
-// 7.0e-8 (7.6e-8), 1x1 3.6e-8 to 4.7e-8 (6.1e-8), weight gradients 4.7e-8 to 5.5e-8 (5.6e-8 to 1.1e-7).  Two fp16 parts and three products were off by 9.4e-8:
-// 22-bit products lose more where the terms are aligned.  bf16 storage: one exact product a step.
+// like size is among the terms.  So hi hi starts from zero in every step and goes into an fp32 sum on the CUDA cores, two taps of it (MC_RUN) into a
+// compensated (Kahan) sum, in a weight gradient of fp32 storage every step (four CTAs per SM have no registers for both); the other five, 2^-6 of
+// it at the most, run on in one accumulator per chunk.  What truncation takes away has the sign of the sum: 1.7e-8 of a sum of products of one sign with 16-bit
+// products.  One operand's hi (the weights', where the pack does it once; dy's in a weight gradient) therefore has 6 bits, as few as three parts allow: 14-bit
+// products, 6e-9.
+// Error against double sums, of the result's rms (packed-FMA kernels of fconv.cu beside it), 3x3: normal data, forward and input gradient 4.1e-8 to 4.8e-8
+// (7.6e-8), weight gradient 4.5e-8 (8e-8 to 1.1e-7); ReLU'd x, weights and dy with a mean of half their deviation 2.4e-8 to 3.7e-8 (2.5e-8 to
+// 4.7e-8), weight gradient 2.6e-8 to 3.0e-8 (2.8e-8 to 3.8e-8); every product of one sign 2.5e-8 to 3.5e-8 (2.5e-8 to 3.9e-8; 2 % more than there from 256
+// channels on), weight gradient 2.0e-8 (1.9e-8; 1x1 6 % more).  With 8 bits and nine taps a run the last two of forward and input gradient were up to
+// 1.6 and 1.75 times those of the packed-FMA kernels (22.7 us for what takes 24.7 now).  Two fp16 parts and three products were off by 9.4e-8:
+// 22-bit products lose more where the terms are aligned.  bf16 storage: one exact product a step, weight gradients flushed every MW_RUN steps and the splits
+// added in double: 1.00 times the packed-FMA kernels' errors at the most, 0.8 on average (1.19 with a flush per tile).  Forward and input gradient keep to
+// one flush per chunk there: 6.5e-8 before the result is rounded to bf16, by 1.7e-3 (4.4e-8; a flush every MC_RUN taps gives 4.6e-8 for 4.5 % of a step).
 //
-// Time, 192 images, launch included (packed FMA beside it): fp32 32x32 16 -> 16 forward 23 us (38), weight gradient with its reduction 37 (54); 16x16 32 -> 32 23
-// (40), 35 (53); 8x8 64 -> 64 27 (41), 39 (57).  What bounds them: a third to 40 % of the mma.sync rate (980 multiply-adds per clock and SM, six per
+// Time, 192 images, launch included (packed FMA beside it): fp32 32x32 16 -> 16 forward 25 us (38), weight gradient with its reduction 37 (54); 16x16 32 -> 32 25
+// (40), 35 (53); 8x8 64 -> 64 29 (41), 39 (57).  What bounds them: a third to 40 % of the mma.sync rate (980 multiply-adds per clock and SM, six per
 // product), the rest is latency of one warp's chain (fixed-latency waits, ncu) and the splitting, which every block of 16 or 32 output channels repeats.
 #include "fconv.h"
 #include "launch.h"
@@ -30,6 +37,9 @@ namespace fdg {
 namespace {
 
 constexpr int MC_THREADS = 128;
+constexpr int W_HI = 6, DY_HI = 6;       // bits of hi in the weights and, in a weight gradient, in dy
+constexpr int MC_RUN = 2;                // taps whose sums of hi hi are added before they go into the compensated sum (fp32 storage)
+constexpr int MW_RUN = 4;                // the same in a weight gradient: 16-pixel steps (bf16 storage)
 
 template <typename T> constexpr bool SPLIT = sizeof(T) == 4;
 template <typename T> constexpr int PARTS = SPLIT<T> ? 3 : 1;             // bf16 values per value
@@ -55,12 +65,16 @@ template <typename T> constexpr int PRODUCTS = SPLIT<T> ? 6 : 1;
 template <typename T> __host__ __device__ constexpr int part_a(int k) { return !SPLIT<T> ? 0 : k == 0 ? 2 : k == 1 || k == 3 ? 1 : 0; }
 template <typename T> __host__ __device__ constexpr int part_b(int k) { return !SPLIT<T> ? 0 : k == 2 ? 2 : k == 1 || k == 4 ? 1 : 0; }
 
-// two values' parts
+// two values' parts.  HI: significant bits of hi, 8 or fewer (at least 6: mid and lo hold 8 each and a sign)
 __device__ __forceinline__ uint32_t pair_rn(float a, float b) { const __nv_bfloat162 v = __floats2bfloat162_rn(a, b); return *(const uint32_t*)&v; }
 __device__ __forceinline__ float2 pair_value(uint32_t v) { return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u)); }
-__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+template <int HI> __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
     const float2 minus = make_float2(-1.f, -1.f);
-    hi = pair_rn(a, b);
+    if (HI == 8) hi = pair_rn(a, b);
+    else {
+        constexpr uint32_t half = 1u << (23 - HI), keep = (0xffffu << (8 - HI)) & 0xffffu;
+        hi = __byte_perm(__float_as_uint(a) + half, __float_as_uint(b) + half, 0x7632) & (keep << 16 | keep);
+    }
     const float2 r = __ffma2_rn(pair_value(hi), minus, make_float2(a, b));
     mid = pair_rn(r.x, r.y);
     const float2 l = __ffma2_rn(pair_value(mid), minus, r);
@@ -96,13 +110,13 @@ __device__ __forceinline__ void fetch_region(const T* __restrict__ x, char* dst,
     }
 }
 // raw -> planes [hi, mid, lo][half][pixel][8], parts `part_bytes` apart
-__device__ __forceinline__ void split_pixels(const float* raw, char* dst, int xp, int part_bytes, int npix, int tid, int nthreads) {
+template <int HI> __device__ __forceinline__ void split_pixels(const float* raw, char* dst, int xp, int part_bytes, int npix, int tid, int nthreads) {
     for (int pix = tid; pix < npix; pix += nthreads)
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
             const float4 a = *(const float4*)(raw + raw_at(pix, 2 * half)), b = *(const float4*)(raw + raw_at(pix, 2 * half + 1));
             uint4 h, m, l;
-            split2(a.x, a.y, h.x, m.x, l.x); split2(a.z, a.w, h.y, m.y, l.y); split2(b.x, b.y, h.z, m.z, l.z); split2(b.z, b.w, h.w, m.w, l.w);
+            split2<HI>(a.x, a.y, h.x, m.x, l.x); split2<HI>(a.z, a.w, h.y, m.y, l.y); split2<HI>(b.x, b.y, h.z, m.z, l.z); split2<HI>(b.z, b.w, h.w, m.w, l.w);
             char* const d = dst + (half * xp + pix) * 16;
             *(uint4*)d = h; *(uint4*)(d + part_bytes) = m; *(uint4*)(d + 2 * part_bytes) = l;
         }
@@ -186,26 +200,29 @@ __global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc
         if (S) {
             cp_wait<0>();
             __syncthreads();
-            split_pixels(raw, planes, q.xp, plane_bytes, npix, tid, MC_THREADS);
+            split_pixels<8>(raw, planes, q.xp, plane_bytes, npix, tid, MC_THREADS);
             __syncthreads();
             if (c + 1 < chunks) { fetch_x(c + 1, 0); fetch_w(c + 1, buf ^ 1); cp_commit(); }
         } else {
             if (c + 1 < chunks) { fetch_x(c + 1, buf ^ 1); fetch_w(c + 1, buf ^ 1); cp_commit(); cp_wait<1>(); } else cp_wait<0>();
             __syncthreads();
         }
-        float2 acc[2][NB][2];                        // this chunk's sum of hi hi
-        float rest[2][NB][4];                        // fp32 storage: of the other products
+        float2 acc[2][NB][2];                        // of hi hi, over MC_RUN taps (bf16 storage: over all)
+        float rest[2][NB][4];                        // fp32 storage: of the other products, over the chunk
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
-            for (int j = 0; j < NB; ++j) {
-                acc[i][j][0] = acc[i][j][1] = make_float2(0.f, 0.f);
-                rest[i][j][0] = rest[i][j][1] = rest[i][j][2] = rest[i][j][3] = 0.f;
-            }
+            for (int j = 0; j < NB; ++j) rest[i][j][0] = rest[i][j][1] = rest[i][j][2] = rest[i][j][3] = 0.f;
         const char* const ws_ = wst + buf * wbuf + lane * (S ? 16 : 8);
         const uint32_t xo = S ? 0u : (uint32_t)(buf * plane_bytes);
 #pragma unroll 1
         for (int t = 0; t < nt; ++t) {
+            if (t == 0 || (S && t % MC_RUN == 0)) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < NB; ++j) acc[i][j][0] = acc[i][j][1] = make_float2(0.f, 0.f);
+            }
             const uint32_t off = xo + (uint32_t)p.toff[t0 + t] * 16u;
             uint32_t a[2][PARTS<T>][4], w[NB][PARTS<T>][2];
             float part[2][NB][4];
@@ -237,16 +254,22 @@ __global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc
                 for (int i = 0; i < 2; ++i)
 #pragma unroll
                     for (int r = 0; r < 2; ++r) acc[i][j][r] = __fadd2_rn(acc[i][j][r], make_float2(part[i][j][2 * r], part[i][j][2 * r + 1]));
+            if (t + 1 == nt || (S && t % MC_RUN == MC_RUN - 1)) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < NB; ++j)
+#pragma unroll
+                        for (int r = 0; r < 2; ++r) add_kahan(sum[i][j][r], lost[i][j][r], acc[i][j][r]);
+            }
         }
+        if (S)
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < 2; ++i)
 #pragma unroll
-            for (int j = 0; j < NB; ++j)
+                for (int j = 0; j < NB; ++j)
 #pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    if (S) lost[i][j][r] = __fadd2_rn(lost[i][j][r], make_float2(rest[i][j][2 * r], rest[i][j][2 * r + 1]));
-                    add_kahan(sum[i][j][r], lost[i][j][r], acc[i][j][r]);
-                }
+                    for (int r = 0; r < 2; ++r) lost[i][j][r] = __fadd2_rn(lost[i][j][r], make_float2(rest[i][j][2 * r], rest[i][j][2 * r + 1]));
         if (!S) __syncthreads();                     // this buffer is consumed
     }
 
@@ -383,8 +406,8 @@ __global__ void __launch_bounds__(MW_WARPS * 32, SPLIT<T> ? 4 : 3) mw_kernel(con
         if (S) {
             cp_wait<0>();
             __syncthreads();
-            split_pixels(raw_x, px_, xp, xp * 32, xp, tid, MW_WARPS * 32);
-            split_pixels(raw_d, pd_, npix, npix * 32, npix, tid, MW_WARPS * 32);
+            split_pixels<8>(raw_x, px_, xp, xp * 32, xp, tid, MW_WARPS * 32);
+            split_pixels<DY_HI>(raw_d, pd_, npix, npix * 32, npix, tid, MW_WARPS * 32);
             __syncthreads();
             if (tile + 1 < tile_end) fetch(tile + 1, 0);
         } else {
@@ -395,12 +418,13 @@ __global__ void __launch_bounds__(MW_WARPS * 32, SPLIT<T> ? 4 : 3) mw_kernel(con
         // rows of x that this lane hands to ldmatrix: pixel lane % 16; lanes 16..31 those of the second part (fp32), nobody's (bf16)
         const uint32_t xbase = smem_addr(px_) + (S ? 0 : buf * xp * 32) + (half * xp + p.toff[tap0]) * 16;
         float rest[TW][4];                           // fp32 storage: this tile's sum of all products but hi hi
-        float2 acc[TW][2];                           // bf16 storage: this tile's sum
+        float2 acc[TW][2];                           // bf16 storage: of MW_RUN steps
 #pragma unroll
         for (int s = 0; s < TW; ++s) {
             rest[s][0] = rest[s][1] = rest[s][2] = rest[s][3] = 0.f;
             acc[s][0] = acc[s][1] = make_float2(0.f, 0.f);
         }
+        int run = 0;
 #pragma unroll 1
         for (int ks = slice; ks * 16 < npix; ks += SL) {
             uint32_t a[PARTS<T>][4], b[TW][PARTS<T>][2];
@@ -431,12 +455,14 @@ __global__ void __launch_bounds__(MW_WARPS * 32, SPLIT<T> ? 4 : 3) mw_kernel(con
                     const float2 v = make_float2(part[s][2 * r], part[s][2 * r + 1]);
                     if (S) add_kahan(sum[s][r], lost[s][r], v); else acc[s][r] = __fadd2_rn(acc[s][r], v);
                 }
+            if (!S && (++run == MW_RUN || (ks + SL) * 16 >= npix)) {
+                run = 0;
+#pragma unroll
+                for (int s = 0; s < TW; ++s)
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) { add_kahan(sum[s][r], lost[s][r], acc[s][r]); acc[s][r] = make_float2(0.f, 0.f); }
+            }
         }
-        if (!S)
-#pragma unroll
-            for (int s = 0; s < TW; ++s)
-#pragma unroll
-                for (int r = 0; r < 2; ++r) add_kahan(sum[s][r], lost[s][r], acc[s][r]);
         if (S)
 #pragma unroll
             for (int s = 0; s < TW; ++s)
@@ -492,7 +518,7 @@ __global__ void __launch_bounds__(256) mc_pack_kernel(const T* __restrict__ wbig
                 v[j] = ws[((a.back ? k : n) * L.taps + tap) * 16 + (a.back ? n : k)];
             }
             if (SPLIT<T>) {
-                split2(v[0], v[1], h[u], mid[u], lo[u]);
+                split2<W_HI>(v[0], v[1], h[u], mid[u], lo[u]);
             } else {
                 const __nv_bfloat162 b = __floats2bfloat162_rn(v[0], v[1]);
                 h[u] = *(const uint32_t*)&b;

@@ -1,0 +1,96 @@
+"""Rounding errors of the tensor-core convolutions (mconv.cu) beside those of the packed-FMA kernels (kernel_path 1), against double: no larger, also where
+products have one sign and truncation inside the tensor core adds up.  A convolution as the first layer, its outputs straight into a linear layer
+of two classes whose first row is zero.  Samples are all the same, so dz (the second class's) is one number, the linear layer's bias gradient
+over the number of samples (a power of two).  That layer's weight gradient is dz times the convolution's output (one sample), and dy is dz times its second
+row, rounded once (bf16: powers of two, nothing to round).
+Bound: the errors' ratio is known to 1 % (10^4 and more outputs each, the same inputs); 1.06 is the largest measured, 1.19 to 1.75 what the tests are there to find."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2509_05679_b200 import binding, synth as sy
+
+pytestmark = pytest.mark.gpu
+
+
+def _gradients(dtype, x, w, head, stride, path):
+    n, h, wd, c = x.shape
+    co, r = w.shape[0], w.shape[1]
+    layers = [(sy.CONV3X3 if r == 3 else sy.CONV1X1, c, co, stride, 0), (sy.LINEAR, head.shape[1], 2, 1, sy.FLAG_BIAS)]
+    ctx = binding.Context(layers, [], 1, n, 0.0, dtype=dtype, in_shape=(h, wd, c), num_classes=2, kernel_path=path)
+    try:
+        ctx.set_params(np.concatenate([w.ravel(), head.ravel(), np.zeros(2)]).astype(np.float32))
+        ctx.step(binding.to_device(dtype, x), torch.zeros(n, dtype=torch.int32, device="cuda"))
+        g = np.asarray(ctx.grads(), np.float64)
+    finally:
+        ctx.close()
+    dz = np.float32(g[-1] / n)
+    return g[:w.size].reshape(w.shape), g[w.size:-2].reshape(2, -1)[1], dz
+
+
+def _error(got, ref):
+    return np.linalg.norm(got - ref) / np.linalg.norm(ref)
+
+
+def _conv(x, w, stride):
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(np.moveaxis(a.astype(np.float64), 3, 1))).cuda()
+    y = torch.nn.functional.conv2d(t(x), t(w), stride=stride, padding=w.shape[1] // 2)
+    return np.moveaxis(y.cpu().numpy(), 1, 3)
+
+
+def _wgrad(x, dy, w, stride):
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(np.moveaxis(a.astype(np.float64), 3, 1))).cuda()
+    wt = torch.zeros_like(t(w)).requires_grad_()
+    torch.nn.functional.conv2d(t(x), wt, stride=stride, padding=w.shape[1] // 2).backward(t(dy))
+    return np.moveaxis(wt.grad.cpu().numpy(), 1, 3)
+
+
+# (batch, side, c, c_out, taps a side, stride)
+SIZES = [(1, 32, 16, 16, 3, 1), (1, 16, 32, 32, 3, 1), (1, 32, 64, 64, 3, 1), (1, 32, 16, 32, 3, 2), (1, 32, 48, 32, 1, 1)]
+
+
+@pytest.mark.parametrize("kind", ["normal", "relu", "positive"])
+@pytest.mark.parametrize("size", SIZES, ids=str)
+def test_fp32_forward(size, kind):
+    n, side, c, co, r, stride = size
+    g = np.random.default_rng(5)
+    x, w = g.standard_normal((n, side, side, c)), g.standard_normal((co, r, r, c)) * 0.1
+    if kind == "relu":
+        x, w = np.maximum(x, 0), w + 0.05
+    if kind == "positive":
+        x, w = np.abs(x), np.abs(w)
+    x, w = x.astype(np.float32), w.astype(np.float32)
+    ref = _conv(x, w, stride).ravel()
+    head = np.zeros((2, ref.size), np.float32)
+    head[1] = 1e-6
+    fma, tensor = [_error(g[1], float(g[2]) * ref) for g in (_gradients("fp32", x, w, head, stride, p) for p in (1, 0))]
+    assert tensor <= 1.1 * fma, (tensor, fma)
+
+
+@pytest.mark.parametrize("kind", ["normal", "positive"])
+@pytest.mark.parametrize("size", [(4, 32, 16, 16, 3, 1), (2, 32, 16, 32, 3, 2), (8, 16, 32, 32, 3, 1), (4, 32, 32, 32, 1, 1)], ids=str)
+def test_fp32_weight_gradient(size, kind):
+    n, side, c, co, r, stride = size
+    g = np.random.default_rng(6)
+    x, w = g.standard_normal((n, side, side, c)), (g.standard_normal((co, r, r, c)) * 0.1).astype(np.float32)
+    so = (side - 1) // stride + 1
+    dy = g.standard_normal((so, so, co)) * 1e-6
+    if kind == "positive":
+        x, dy = np.abs(x), np.abs(dy)
+    x, dy = x.astype(np.float32), dy.astype(np.float32)
+    x = np.repeat(x[:1], n, 0)                   # the same sample, so that dz is the same number for all
+    head = np.stack([np.zeros(dy.size, np.float32), dy.ravel()])
+    fma, tensor = [_error(g[0], n * _wgrad(x[:1], (g[2] * head[1]).reshape(dy.shape)[None], w, stride)) for g in (_gradients("fp32", x, w, head, stride, p) for p in (1, 0))]
+    assert tensor <= 1.1 * fma, (tensor, fma)
+
+
+@pytest.mark.parametrize("size", [(8, 8, 240, 240, 3, 1), (1, 32, 16, 16, 3, 1), (4, 16, 32, 32, 3, 1)], ids=str)
+def test_bf16_weight_gradient(size):
+    n, side, c, co, r, stride = size
+    g = np.random.default_rng(7)
+    x = sy.round_to_bf16(np.repeat(g.standard_normal((1, side, side, c)).astype(np.float32), n, 0))
+    w = sy.round_to_bf16((g.standard_normal((co, r, r, c)) * 0.1).astype(np.float32))
+    v = g.standard_normal((side, side, co)).astype(np.float32)
+    head = np.stack([np.zeros(v.size, np.float32), np.exp2(np.floor(np.log2(np.abs(v.ravel()))) - 20) * np.sign(v.ravel())]).astype(np.float32)
+    fma, tensor = [_error(g[0], n * _wgrad(x[:1], (g[2] * head[1]).reshape(v.shape)[None], w, stride)) for g in (_gradients("bf16", x, w, head, stride, p) for p in (1, 0))]
+    assert tensor <= 1.1 * fma, (tensor, fma)
