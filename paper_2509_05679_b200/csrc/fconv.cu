@@ -670,7 +670,7 @@ bool fconv_forward(int dt, const void* x, const void* w, const float* bias, void
     p.epi = epi; p.w_group = w_group; p.b_group = b_group;
     const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
     Scope sc(KC_FMA_FWD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + g.Co * K + rows * g.Co), s);
-    if (pk.data && mconv_forward(dt, x, pk.data, bias, y, stat, g, epi, groups, b_group, pk.group, s)) return true;
+    if (pk.data && mconv_forward(dt, x, w, pk, bias, y, stat, g, epi, groups, w_group, b_group, s)) return true;
     if (dt) dispatch_fc<bf16>(x, w, bias, y, stat, p, groups, s); else dispatch_fc<float>(x, w, bias, y, stat, p, groups, s);
     return true;
 }
@@ -680,7 +680,7 @@ bool fconv_dgrad(int dt, const void* dy, const void* w, void* dx, const ConvGeom
     p.epi = epi; p.w_group = w_group;
     const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
     Scope sc(KC_FMA_DGRAD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + g.Co * K + rows * g.Co), s);
-    if (pk.data && mconv_dgrad(dt, dy, pk.data, dx, g, epi, groups, pk.group, s)) return true;
+    if (pk.data && mconv_dgrad(dt, dy, w, pk, dx, g, epi, groups, w_group, s)) return true;
     if (dt) dispatch_fc<bf16>(dy, w, nullptr, dx, nullptr, p, groups, s); else dispatch_fc<float>(dy, w, nullptr, dx, nullptr, p, groups, s);
     return true;
 }

@@ -54,9 +54,9 @@ bool plan_fw(const ConvGeom& g, int groups, int ctas, FwParams& p, int& G, int& 
 
 // The tensor-core forms (mconv.cu), tried first by the fconv_* functions; false / 0: not covered or refused, nothing launched.
 // mconv_wgrad leaves partial matrices as fw_kernel does and returns their number per block.
-bool mconv_forward(int dt, const void* x, const void* pack, const float* bias, void* y, float* stat, const ConvGeom& g, int epi, int groups, size_t b_group, size_t pack_group,
+bool mconv_forward(int dt, const void* x, const void* w, const Packed& pk, const float* bias, void* y, float* stat, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
                    cudaStream_t s);
-bool mconv_dgrad(int dt, const void* dy, const void* pack, void* dx, const ConvGeom& g, int epi, int groups, size_t pack_group, cudaStream_t s);
+bool mconv_dgrad(int dt, const void* dy, const void* w, const Packed& pk, void* dx, const ConvGeom& g, int epi, int groups, size_t w_group, cudaStream_t s);
 int  mconv_wgrad(int dt, const void* x, const void* dy, float* ws, const ConvGeom& g, int groups, cudaStream_t s);
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }

@@ -19,13 +19,13 @@
 // (7.6e-8), weight gradient 4.5e-8 (8e-8 to 1.1e-7); ReLU'd x, weights and dy with a mean of half their deviation 2.4e-8 to 3.7e-8 (2.5e-8 to
 // 4.7e-8), weight gradient 2.6e-8 to 3.0e-8 (2.8e-8 to 3.8e-8); every product of one sign 2.5e-8 to 3.5e-8 (2.5e-8 to 3.9e-8; 2 % more than there from 256
 // channels on), weight gradient 2.0e-8 (1.9e-8; 1x1 6 % more).  With 8 bits and nine taps a run the last two of forward and input gradient were up to
-// 1.6 and 1.75 times those of the packed-FMA kernels (22.7 us for what takes 24.7 now).  Two fp16 parts and three products were off by 9.4e-8:
+// 1.6 and 1.75 times those of the packed-FMA kernels (22.7 us for what takes 25 now).  Two fp16 parts and three products were off by 9.4e-8:
 // 22-bit products lose more where the terms are aligned.  bf16 storage: one exact product a step, weight gradients flushed every MW_RUN steps and the splits
 // added in double: 1.00 times the packed-FMA kernels' errors at the most, 0.8 on average (1.19 with a flush per tile).  Forward and input gradient keep to
 // one flush per chunk there: 6.5e-8 before the result is rounded to bf16, by 1.7e-3 (4.4e-8; a flush every MC_RUN taps gives 4.6e-8 for 4.5 % of a step).
 //
-// Time, 192 images, launch included (packed FMA beside it): fp32 32x32 16 -> 16 forward 25 us (38), weight gradient with its reduction 37 (54); 16x16 32 -> 32 25
-// (40), 35 (53); 8x8 64 -> 64 29 (41), 39 (57).  What bounds them: a third to 40 % of the mma.sync rate (980 multiply-adds per clock and SM, six per
+// Time, 192 images, launch included (packed FMA beside it): fp32 32x32 16 -> 16 forward 25 us (38), weight gradient with its reduction 38 (54); 16x16 32 -> 32 27
+// (40), 36 (53); 8x8 64 -> 64 29 (41), 39 (57).  What bounds them: a third to 40 % of the mma.sync rate (980 multiply-adds per clock and SM, six per
 // product), the rest is latency of one warp's chain (fixed-latency waits, ncu) and the splitting, which every block of 16 or 32 output channels repeats.
 #include "fconv.h"
 #include "launch.h"
@@ -65,6 +65,11 @@ template <typename T> constexpr int PRODUCTS = SPLIT<T> ? 6 : 1;
 template <typename T> __host__ __device__ constexpr int part_a(int k) { return !SPLIT<T> ? 0 : k == 0 ? 2 : k == 1 || k == 3 ? 1 : 0; }
 template <typename T> __host__ __device__ constexpr int part_b(int k) { return !SPLIT<T> ? 0 : k == 2 ? 2 : k == 1 || k == 4 ? 1 : 0; }
 
+// Range: before the split a value is multiplied by RANGE = 2^16, so that lo of the smallest normal number, 2^-126, still is a multiple of bf16's smallest, 2^-133
+// (the exponents reach as far down as fp32's, the digits 16 places less far); sums carry RANGE^2 until they are stored.  The price is at the other
+// end: from 2^111 on (sums: 2^95) parts are infinite, and since a part that overflows leaves NaN in the next one, so is no sum that they enter.  Such outputs are computed
+// once more, product by product (direct_*).
+constexpr float RANGE = 65536.f, UNRANGE2 = 1.f / (65536.f * 65536.f);
 // two values' parts.  HI: significant bits of hi, 8 or fewer (at least 6: mid and lo hold 8 each and a sign)
 __device__ __forceinline__ uint32_t pair_rn(float a, float b) { const __nv_bfloat162 v = __floats2bfloat162_rn(a, b); return *(const uint32_t*)&v; }
 __device__ __forceinline__ float2 pair_value(uint32_t v) { return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u)); }
@@ -115,8 +120,11 @@ template <int HI> __device__ __forceinline__ void split_pixels(const float* raw,
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
             const float4 a = *(const float4*)(raw + raw_at(pix, 2 * half)), b = *(const float4*)(raw + raw_at(pix, 2 * half + 1));
+            const float2 range = make_float2(RANGE, RANGE);
+            const float2 v[4] = {__fmul2_rn(make_float2(a.x, a.y), range), __fmul2_rn(make_float2(a.z, a.w), range), __fmul2_rn(make_float2(b.x, b.y), range),
+                                 __fmul2_rn(make_float2(b.z, b.w), range)};
             uint4 h, m, l;
-            split2<HI>(a.x, a.y, h.x, m.x, l.x); split2<HI>(a.z, a.w, h.y, m.y, l.y); split2<HI>(b.x, b.y, h.z, m.z, l.z); split2<HI>(b.z, b.w, h.w, m.w, l.w);
+            split2<HI>(v[0].x, v[0].y, h.x, m.x, l.x); split2<HI>(v[1].x, v[1].y, h.y, m.y, l.y); split2<HI>(v[2].x, v[2].y, h.z, m.z, l.z); split2<HI>(v[3].x, v[3].y, h.w, m.w, l.w);
             char* const d = dst + (half * xp + pix) * 16;
             *(uint4*)d = h; *(uint4*)(d + part_bytes) = m; *(uint4*)(d + 2 * part_bytes) = l;
         }
@@ -137,13 +145,48 @@ struct McParams {
     int wtaps;                           // taps of the largest class
     size_t pack_group;                   // 16-byte words between the groups' packed weights
 };
+// a compensated sum that overflowed has lost NaN
+__device__ __forceinline__ float total(float sum, float lost) { return isinf(sum) ? sum : __fadd_rn(sum, lost); }
+// the compensated sums of the packed-FMA kernels end as NaN where they overflow
+__device__ __forceinline__ float finite_or_nan(double s) { const float v = (float)s; return isfinite(v) ? v : __int_as_float(0x7fffffff); }
+
+// One output of mc_kernel, product by product; w: this group's weights.
+__device__ __noinline__ float direct_output(const float* __restrict__ x, const float* __restrict__ w, const FcParams& p, int cls, int n, int hd, int wd, int co) {
+    double s = 0.0;
+    for (int t = p.cls_tap0[cls]; t < p.cls_tap0[cls + 1] && isfinite(s); ++t) {
+        const int h = hd * p.xs + p.cls_h0[cls] + p.toff[t] / p.cls_rw[cls], wi = wd * p.xs + p.cls_w0[cls] + p.toff[t] % p.cls_rw[cls];
+        const bool in = h >= 0 && h < p.H && wi >= 0 && wi < p.W;
+        const float* const xs = x + (((size_t)n * p.H + (in ? h : 0)) * p.W + (in ? wi : 0)) * p.C;
+        const float* const ws = p.back ? w + (size_t)p.wtap[t] * p.Co + co : w + ((size_t)co * p.taps + p.wtap[t]) * p.C;
+        const size_t step = p.back ? (size_t)p.taps * p.Co : 1;
+        for (int c = 0; c < p.C; ++c) s += (in ? (double)xs[c] : 0.0) * (double)ws[c * step];
+    }
+    return finite_or_nan(s);
+}
+// One element of mw_kernel's partial matrix.
+__device__ __noinline__ float direct_wgrad(const float* __restrict__ x, const float* __restrict__ dy, const FwParams& p, int grp, int tile0, int tile_end, int co, int tap, int ci) {
+    const int R = p.ntaps == 9 ? 3 : 1, n_end = (grp + 1) * p.ngroup;
+    double s = 0.0;
+    for (int t = tile0; t < tile_end && isfinite(s); ++t) {
+        const int tw = t % p.tiles_w, th = t / p.tiles_w % p.tiles_h, tn = t / p.tiles_w / p.tiles_h;
+        for (int px = 0; px < p.Wt * p.Ht * p.Nt; ++px) {
+            const int wo = tw * p.Wt + (px & (p.Wt - 1)), ho = th * p.Ht + ((px >> p.lw) & (p.Ht - 1)), n = grp * p.ngroup + tn * p.Nt + (px >> (p.lw + p.lh));
+            const int h = ho * p.hstep - p.pad + tap / R, w = wo * p.hstep - p.pad + tap % R;
+            if (n >= n_end || ho >= p.Ho || wo >= p.Wo) continue;
+            const bool in = h >= 0 && h < p.H && w >= 0 && w < p.W;
+            s += (in ? (double)x[(((size_t)n * p.H + h) * p.W + w) * p.C + ci] : 0.0) * (double)dy[(((size_t)n * p.Ho + ho) * p.Wo + wo) * p.Co + co];
+        }
+    }
+    return finite_or_nan(s);
+}
+
 template <typename T> constexpr int mc_x_bytes(int xp) { return xp * (SPLIT<T> ? 64 + 96 : 2 * 32); }            // fp32: raw + parts; bf16: two buffers
 template <typename T, int NB> constexpr int mc_w_bytes(int taps, int chunks) { return (chunks > 1 ? 2 : 1) * taps * (NB / 2) * PACK16<T> * 16; }
 
 // grid = (pixel tiles, blocks of 8 NB output channels, groups x classes); a warp computes 32 pixels x 8 NB channels.
 template <typename T, int NB>
-__global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc_kernel(const T* __restrict__ x, const uint4* __restrict__ pk, const float* __restrict__ bias,
-                                                                        T* __restrict__ y, float* __restrict__ stat, const __grid_constant__ McParams q) {
+__global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc_kernel(const T* __restrict__ x, const T* __restrict__ w, const uint4* __restrict__ pk,
+                                                                        const float* __restrict__ bias, T* __restrict__ y, float* __restrict__ stat, const __grid_constant__ McParams q) {
     constexpr bool S = SPLIT<T>;
     constexpr int NW = MC_THREADS / 32, BLKS = NB / 2, U = PACK16<T>;
     extern __shared__ __align__(16) char msm[];
@@ -159,6 +202,7 @@ __global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc
     const int RH = p.cls_rh[cls], RW = p.cls_rw[cls], h0 = hd0 * p.xs + p.cls_h0[cls], w0 = wd0 * p.xs + p.cls_w0[cls];
     const int kc = p.C >> 4, chunks = nt > 0 ? kc : 0, npix = p.Nt * RH * RW;
     pk += (size_t)grp * q.pack_group;
+    w += (size_t)grp * p.w_group;                    // read by direct_output only
 
     float* const raw = (float*)msm;                                              // fp32 only
     char* const planes = msm + (S ? q.xp * 64 : 0);                              // fp32: [part][half][pixel] 16 bytes; bf16: [buffer][half][pixel]
@@ -224,7 +268,7 @@ __global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc
                     for (int j = 0; j < NB; ++j) acc[i][j][0] = acc[i][j][1] = make_float2(0.f, 0.f);
             }
             const uint32_t off = xo + (uint32_t)p.toff[t0 + t] * 16u;
-            uint32_t a[2][PARTS<T>][4], w[NB][PARTS<T>][2];
+            uint32_t a[2][PARTS<T>][4], b[NB][PARTS<T>][2];
             float part[2][NB][4];
 #pragma unroll
             for (int i = 0; i < 2; ++i)
@@ -236,8 +280,8 @@ __global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc
                 if (S) {
                     const uint4 v = *(const uint4*)(s + (j & 1) * 512);
                     const uint2 l = *(const uint2*)(s - lane * 8 + 1024 + (j & 1) * 256);
-                    w[j][0][0] = v.x; w[j][0][1] = v.y; w[j][PARTS<T> / 2][0] = v.z; w[j][PARTS<T> / 2][1] = v.w; w[j][PARTS<T> - 1][0] = l.x; w[j][PARTS<T> - 1][1] = l.y;
-                } else { const uint2 v = *(const uint2*)(s + (j & 1) * 256); w[j][0][0] = v.x; w[j][0][1] = v.y; }
+                    b[j][0][0] = v.x; b[j][0][1] = v.y; b[j][PARTS<T> / 2][0] = v.z; b[j][PARTS<T> / 2][1] = v.w; b[j][PARTS<T> - 1][0] = l.x; b[j][PARTS<T> - 1][1] = l.y;
+                } else { const uint2 v = *(const uint2*)(s + (j & 1) * 256); b[j][0][0] = v.x; b[j][0][1] = v.y; }
             }
 #pragma unroll
             for (int k = 0; k < PRODUCTS<T>; ++k)
@@ -245,8 +289,8 @@ __global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc
                 for (int j = 0; j < NB; ++j)
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
-                        if (k + 1 < PRODUCTS<T>) mma(rest[i][j], a[i][part_a<T>(k)], w[j][part_b<T>(k)][0], w[j][part_b<T>(k)][1], true);
-                        else mma(part[i][j], a[i][0], w[j][0][0], w[j][0][1], false);
+                        if (k + 1 < PRODUCTS<T>) mma(rest[i][j], a[i][part_a<T>(k)], b[j][part_b<T>(k)][0], b[j][part_b<T>(k)][1], true);
+                        else mma(part[i][j], a[i][0], b[j][0][0], b[j][0][1], false);
                     }
 #pragma unroll
             for (int j = 0; j < NB; ++j)
@@ -275,6 +319,32 @@ __global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc
 
     float val[2][NB][2][2];
     bool valid[2][2];
+    if constexpr (S) {
+        uint32_t direct = 0;                         // outputs that are not finite, in the order of the loops
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < NB; ++j)
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const float v = e ? total(sum[i][j][r].y, lost[i][j][r].y) : total(sum[i][j][r].x, lost[i][j][r].x);
+                        val[i][j][r][e] = v * UNRANGE2;
+                        direct |= (uint32_t)!isfinite(v) << (((i * NB + j) * 2 + r) * 2 + e);
+                    }
+        if (direct) {                                // apart from the loop above, whose code it would triple (2 us a launch)
+            float redo[2 * NB * 4];
+#pragma unroll 1
+            for (int k = 0; k < 2 * NB * 4; ++k) {
+                const int px = warp * 32 + k / (NB * 4) * 16 + (k >> 1 & 1) * 8 + g;
+                const int wd = wd0 + (px & (p.Wt - 1)), hd = hd0 + ((px >> p.lw) & (p.Ht - 1)), n = n0 + (px >> (p.lw + p.lh));
+                if (direct >> k & 1 && n < n_end && hd < p.Hd && wd < p.Wd) redo[k] = direct_output(x, w, p, cls, n, hd, wd, co0 + 8 * (k / 4 % NB) + 2 * tq + (k & 1));
+            }
+#pragma unroll
+            for (int k = 0; k < 2 * NB * 4; ++k) if (direct >> k & 1) val[k / (NB * 4)][k / 4 % NB][k >> 1 & 1][k & 1] = redo[k];
+        }
+    }
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -285,7 +355,7 @@ __global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc
             const size_t o = (((size_t)n * p.Ho + (hd * p.os + p.cls_oph[cls])) * p.Wo + (wd * p.os + p.cls_opw[cls])) * p.Co + co0 + 2 * tq;
 #pragma unroll
             for (int j = 0; j < NB; ++j) {
-                float a = __fadd_rn(sum[i][j][r].x, lost[i][j][r].x), b = __fadd_rn(sum[i][j][r].y, lost[i][j][r].y);
+                float a = S ? val[i][j][r][0] : total(sum[i][j][r].x, lost[i][j][r].x), b = S ? val[i][j][r][1] : total(sum[i][j][r].y, lost[i][j][r].y);
                 if (valid[i][r]) {
                     const int co = co0 + 8 * j + 2 * tq;
                     if (bias) { a += bias[(size_t)grp * p.b_group + co]; b += bias[(size_t)grp * p.b_group + co + 1]; }
@@ -479,14 +549,21 @@ __global__ void __launch_bounds__(MW_WARPS * 32, SPLIT<T> ? 4 : 3) mw_kernel(con
 #pragma unroll
         for (int r = 0; r < 2; ++r)
             *(float2*)(red + (size_t)slice * nout + ((g + 8 * r) * p.ntaps + tap0 + s) * 16 + 8 * half + 2 * tq) =
-                make_float2(__fadd_rn(sum[s][r].x, lost[s][r].x), __fadd_rn(sum[s][r].y, lost[s][r].y));
+                make_float2(total(sum[s][r].x, lost[s][r].x), total(sum[s][r].y, lost[s][r].y));
     __syncthreads();
     float* const out = part_out + (((size_t)grp * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * nout;
+    bool direct = false;
     for (int i = tid; i < nout; i += MW_WARPS * 32) {
         double s = 0;
         for (int k = 0; k < SL; ++k) s += (double)red[(size_t)k * nout + i];
+        if (S) { direct |= !isfinite(s); s *= UNRANGE2; }
         out[i] = (float)s;
     }
+    if constexpr (S)
+        if (direct)
+#pragma unroll 1
+            for (int i = tid; i < nout; i += MW_WARPS * 32)
+                if (!isfinite(out[i])) out[i] = direct_wgrad(x, dy, p, grp, tile0, tile_end, co0 + i / (p.ntaps * 16), i / 16 % p.ntaps, ci0 + i % 16);
 }
 
 // One CTA per 16 x 16 block of a layer's matrices (all taps): [n block][k chunk][tap][n8][lane], per lane the B operand of one mma: the values (k = 2 t, 2 t + 1
@@ -518,7 +595,7 @@ __global__ void __launch_bounds__(256) mc_pack_kernel(const T* __restrict__ wbig
                 v[j] = ws[((a.back ? k : n) * L.taps + tap) * 16 + (a.back ? n : k)];
             }
             if (SPLIT<T>) {
-                split2<W_HI>(v[0], v[1], h[u], mid[u], lo[u]);
+                split2<W_HI>(v[0] * RANGE, v[1] * RANGE, h[u], mid[u], lo[u]);
             } else {
                 const __nv_bfloat162 b = __floats2bfloat162_rn(v[0], v[1]);
                 h[u] = *(const uint32_t*)&b;
@@ -555,14 +632,15 @@ bool plan_mw(const ConvGeom& g, int groups, MwParams& q, size_t& smem) {
 }
 
 template <typename T, int NB>
-cudaError_t launch_mc(const void* x, const void* pk, const float* bias, void* y, float* stat, const McParams& q, int groups, cudaStream_t s) {
+cudaError_t launch_mc(const void* x, const void* w, const void* pk, const float* bias, void* y, float* stat, const McParams& q, int groups, cudaStream_t s) {
     static OncePerDevice once;
     if (cudaError_t e = allow_smem(once, (const void*)mc_kernel<T, NB>, (int)FC_SMEM_MAX)) return e;
     const int tiles = q.p.tiles_w * q.p.tiles_h * ((q.p.ngroup + q.p.Nt - 1) / q.p.Nt);
-    return klaunch(mc_kernel<T, NB>, dim3(tiles, q.p.Co / (8 * NB), groups * q.p.ncls), MC_THREADS, mc_smem<T, NB>(q), s, (const T*)x, (const uint4*)pk, bias, (T*)y, stat, q);
+    return klaunch(mc_kernel<T, NB>, dim3(tiles, q.p.Co / (8 * NB), groups * q.p.ncls), MC_THREADS, mc_smem<T, NB>(q), s, (const T*)x, (const T*)w, (const uint4*)pk, bias, (T*)y, stat, q);
 }
 template <typename T>
-bool run_mc(const void* x, const void* pk, const float* bias, void* y, float* stat, const ConvGeom& g, int epi, int groups, size_t b_group, size_t pack_group, bool back, cudaStream_t s) {
+bool run_mc(const void* x, const void* w, const void* pk, const float* bias, void* y, float* stat, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group, size_t pack_group, bool back,
+            cudaStream_t s) {
     McParams q;
     if (!plan_mc<T>(g, groups, back, q)) return false;
     // Left to the packed-FMA kernel: tiles of many short rows (images of 3x3 and smaller; a warp fetches row by row: 2x2, 64 channels, fp32 41 us against 35, 3x3,
@@ -571,14 +649,14 @@ bool run_mc(const void* x, const void* pk, const float* bias, void* y, float* st
     int rows = 0;
     for (int c = 0; c < q.p.ncls; ++c) rows = std::max(rows, q.p.Nt * q.p.cls_rh[c]);
     if (rows > (SPLIT<T> ? 64 : 128) || (SPLIT<T> && q.p.taps == 1 && q.p.xs == 2 && q.p.C > FC_KC)) return false;
-    q.p.epi = epi; q.p.b_group = b_group;
+    q.p.epi = epi; q.p.w_group = w_group; q.p.b_group = b_group;
     q.pack_group = pack_group / 16;
     const long tiles = (long)q.p.tiles_w * q.p.tiles_h * ((q.p.ngroup + q.p.Nt - 1) / q.p.Nt) * groups * q.p.ncls;
     // 32 output channels a CTA (a third less shared-memory traffic per product, the region split for twice the work), unless 16 fill the device more evenly;
     // large regions (stride 2) leave an SM two CTAs at the most either way
     const auto waves = [](long ctas) { return (ctas + 147) / 148; };
     const bool wide = q.p.Co % 32 == 0 && (mc_smem<T, 2>(q) > 75 * 1024 || 2 * waves(tiles * (q.p.Co / 32)) <= 1.15 * waves(tiles * (q.p.Co / 16)));
-    return launched(wide ? launch_mc<T, 4>(x, pk, bias, y, stat, q, groups, s) : launch_mc<T, 2>(x, pk, bias, y, stat, q, groups, s));
+    return launched(wide ? launch_mc<T, 4>(x, w, pk, bias, y, stat, q, groups, s) : launch_mc<T, 2>(x, w, pk, bias, y, stat, q, groups, s));
 }
 template <typename T, int XS, int TW>
 cudaError_t launch_mw(const void* x, const void* dy, float* ws, const MwParams& q, int groups, int blocks, size_t smem, cudaStream_t s) {
@@ -612,12 +690,12 @@ bool mconv_pack(int dt, const void* wbig, size_t w_group, void* out, size_t out_
     return launched(dt ? klaunch(mc_pack_kernel<bf16>, dim3(blocks, groups), 256, 0, s, (const bf16*)wbig, w_group, (uint4*)out, out_group / 16, a)
                        : klaunch(mc_pack_kernel<float>, dim3(blocks, groups), 256, 0, s, (const float*)wbig, w_group, (uint4*)out, out_group / 16, a));
 }
-bool mconv_forward(int dt, const void* x, const void* pack, const float* bias, void* y, float* stat, const ConvGeom& g, int epi, int groups, size_t b_group, size_t pack_group,
+bool mconv_forward(int dt, const void* x, const void* w, const Packed& pk, const float* bias, void* y, float* stat, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
                    cudaStream_t s) {
-    return dt ? run_mc<bf16>(x, pack, bias, y, stat, g, epi, groups, b_group, pack_group, false, s) : run_mc<float>(x, pack, bias, y, stat, g, epi, groups, b_group, pack_group, false, s);
+    return (dt ? run_mc<bf16> : run_mc<float>)(x, w, pk.data, bias, y, stat, g, epi, groups, w_group, b_group, pk.group, false, s);
 }
-bool mconv_dgrad(int dt, const void* dy, const void* pack, void* dx, const ConvGeom& g, int epi, int groups, size_t pack_group, cudaStream_t s) {
-    return dt ? run_mc<bf16>(dy, pack, nullptr, dx, nullptr, g, epi, groups, 0, pack_group, true, s) : run_mc<float>(dy, pack, nullptr, dx, nullptr, g, epi, groups, 0, pack_group, true, s);
+bool mconv_dgrad(int dt, const void* dy, const void* w, const Packed& pk, void* dx, const ConvGeom& g, int epi, int groups, size_t w_group, cudaStream_t s) {
+    return (dt ? run_mc<bf16> : run_mc<float>)(dy, w, pk.data, nullptr, dx, nullptr, g, epi, groups, w_group, 0, pk.group, true, s);
 }
 int mconv_wgrad(int dt, const void* x, const void* dy, float* ws, const ConvGeom& g, int groups, cudaStream_t s) {
     return dt ? run_mw<bf16>(x, dy, ws, g, groups, s) : run_mw<float>(x, dy, ws, g, groups, s);

@@ -94,3 +94,16 @@ def test_bf16_weight_gradient(size):
     head = np.stack([np.zeros(v.size, np.float32), np.exp2(np.floor(np.log2(np.abs(v.ravel()))) - 20) * np.sign(v.ravel())]).astype(np.float32)
     fma, tensor = [_error(g[0], n * _wgrad(x[:1], (g[2] * head[1]).reshape(v.shape)[None], w, stride)) for g in (_gradients("bf16", x, w, head, stride, p) for p in (1, 0))]
     assert tensor <= 1.1 * fma, (tensor, fma)
+
+
+@pytest.mark.parametrize("x_exp,w_exp", [(-126, 100), (-110, 80), (60, -60), (96, -100), (100, -126), (127, -128)])
+def test_fp32_range(x_exp, w_exp):
+    """Inputs and weights near both ends of fp32's range (2^127 times up to 1.998: beyond bf16's largest), outputs that are not.  The errors' ratio is that of ordinary values."""
+    g = np.random.default_rng(8)
+    x, w = g.uniform(1, 1.998, (1, 32, 32, 16)) * g.choice([-1, 1], (1, 32, 32, 16)), g.uniform(0.5, 1.998, (16, 3, 3, 16)) * g.choice([-1, 1], (16, 3, 3, 16))
+    x, w = np.ldexp(x, x_exp).astype(np.float32), np.ldexp(w, w_exp).astype(np.float32)
+    ref = _conv(x, w, 1).ravel()
+    head = np.zeros((2, ref.size), np.float32)
+    head[1] = np.float32(1e-6 * 2.0 ** -max(0, x_exp + w_exp))
+    fma, tensor = [_error(g[1], float(g[2]) * ref) for g in (_gradients("fp32", x, w, head, 1, p) for p in (1, 0))]
+    assert tensor <= 1.1 * fma, (tensor, fma)
