@@ -17,7 +17,7 @@ constexpr int FC_KC = 16;                // channels per chunk
 constexpr int PITCH = 20;                // floats per pixel (or weight row) in shared memory: 16 + 4, so that the eight 16-byte reads
                                          // of neighbouring pixels fall into different banks
 constexpr int FW_CO = 16, FW_CI = 16;
-constexpr int FW_CTAS = 3 * 148, MW_CTAS = 4 * 148;      // of a weight gradient, fconv.cu's and mconv.cu's: as many as the device holds at a time
+constexpr int FW_CTAS = 3 * 148, MW_CTAS = 4 * 148;      // of a weight gradient, fconv.cu's and mconv.cu's: as many as registers allow at a time
 constexpr size_t FC_SMEM_MAX = 224 * 1024;
 
 struct FcParams {

@@ -607,6 +607,8 @@ __global__ void __launch_bounds__(256) mc_pack_kernel(const T* __restrict__ wbig
     }
 }
 
+constexpr int SM_SMEM = 228 * 1024, CTA_SMEM = 1024;      // of an SM; what every CTA takes beside its own
+
 bool channels_ok(const ConvGeom& g) { return g.C % 16 == 0 && g.Co % 16 == 0; }
 template <typename T, int NB> size_t mc_smem(const McParams& q) { return (size_t)mc_x_bytes<T>(q.xp) + mc_w_bytes<T, NB>(q.wtaps, q.p.C / 16); }
 
@@ -621,9 +623,13 @@ bool plan_mc(const ConvGeom& g, int groups, bool back, McParams& q) {
 template <typename T>
 bool plan_mw(const ConvGeom& g, int groups, MwParams& q, size_t& smem) {
     int G, run; size_t fw;
-    if (!channels_ok(g) || !plan_fw(g, groups, SPLIT<T> ? MW_CTAS : FW_CTAS, q.p, G, run, fw)) return false;
+    if (!channels_ok(g) || !plan_fw(g, groups, FW_CTAS, q.p, G, run, fw)) return false;
     q.npix = q.p.Wt * q.p.Ht * q.p.Nt;
     q.xp = q.p.x_floats / PITCH;
+    // splits for one wave: registers allow four CTAs per SM (bf16 storage three), shared memory as few as one where regions are large (stride 2, small
+    // images); with four for all of them a second wave ran: 32 -> 64 stride 2, 64 images of 28x28 52 us (packed FMA 49), now 45; 768 of 20x20 263 (233), now 203
+    const int fit = (int)(SM_SMEM / (mw_smem<T>(q.npix, q.xp) + CTA_SMEM)), most = (SPLIT<T> ? MW_CTAS : FW_CTAS) / 148;
+    if (!plan_fw(g, groups, 148 * std::max(1, std::min(fit, most)), q.p, G, run, fw)) return false;
     for (int i = 0; i < q.p.ntaps; ++i) q.p.toff[i] /= PITCH;
     const size_t red = (size_t)mw_slices(g.R) * FW_CO * q.p.ntaps * FW_CI * sizeof(float);
     smem = mw_smem<T>(q.npix, q.xp);

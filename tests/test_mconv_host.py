@@ -10,6 +10,7 @@ from paper_2509_05679_b200 import build
 FAKE = r"""
 #include "kernels.h"
 #include "launch.h"
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 using namespace fdg;
@@ -17,6 +18,7 @@ using namespace fdg;
 static cudaError_t last = cudaSuccess;      // CUDA's last error
 static int refuse = 0;                      // this many launches are refused
 static std::vector<const void*> ran;        // kernels of the others
+static std::vector<std::pair<dim3, size_t>> grids;      // and their grids and shared memory
 extern "C" {
 cudaError_t cudaGetLastError() { const cudaError_t e = last; last = cudaSuccess; return e; }
 cudaError_t cudaLaunchKernel(const void*, dim3, dim3, void**, size_t, cudaStream_t) { abort(); }
@@ -28,9 +30,10 @@ unsigned __cudaPopCallConfiguration(dim3*, dim3*, size_t*, void*) { return 0; }
 }
 namespace fdg {
 cudaError_t allow_smem(OncePerDevice&, const void*, int) { return cudaSuccess; }
-cudaError_t launch_raw(const void* f, dim3, dim3, size_t, cudaStream_t, void**, const size_t*, int, int) {
+cudaError_t launch_raw(const void* f, dim3 grid, dim3, size_t smem, cudaStream_t, void**, const size_t*, int, int) {
     if (refuse > 0) { --refuse; return last = cudaErrorInvalidConfiguration; }
     ran.push_back(f);
+    grids.push_back({grid, smem});
     return cudaSuccess;
 }
 Scope::Scope(int, double, double, cudaStream_t) {}
@@ -89,3 +92,24 @@ def run(tmp_path, program):
 
 def test_a_refused_launch_is_made_up_for(tmp_path):
     run(tmp_path, REFUSED)
+
+
+ONE_WAVE = r"""
+int main() {
+    alignas(16) static char b[16];
+    for (int dt = 0; dt < 2; ++dt)
+        for (const ConvGeom& g : {conv(64, 28, 28, 32, 64, 3, 2), conv(192, 32, 32, 16, 32, 3, 2), conv(768, 4, 4, 64, 64, 3, 1), conv(192, 16, 16, 32, 32, 3, 1), conv(500, 2, 2, 16, 16, 3, 1),
+                                  conv(96, 32, 32, 16, 16, 1, 1), conv(64, 12, 20, 48, 32, 3, 2)}) {
+            grids.clear();
+            CHECK(fconv_wgrad(dt, b, b, (float*)b, (float*)b, g, 1, 0, false, true, 0));
+            const dim3 n = grids[0].first;
+            CHECK((long)n.x * n.y * n.z <= std::min(dt ? 3 : 4, (int)(228 * 1024 / (grids[0].second + 1024))) * 148L);
+        }
+    return 0;
+}
+"""
+
+
+def test_a_weight_gradient_is_one_wave(tmp_path):
+    """As many CTAs as 148 SMs hold at a time: registers for four (bf16 storage three), 228 KB of shared memory with 1 KB more for each than it asks for."""
+    run(tmp_path, ONE_WAVE)
