@@ -1,6 +1,6 @@
 // FMA convolutions (CUDA cores, fp32 arithmetic, fp32 or bf16 storage) for the layers the tensor-core kernels do not take: channel counts that
-// are no multiple of 16 (the first layer's 3 among them), all of them with kernel_path 1.  3x3 and 1x1, stride 1 and 2, any channel counts, any image
-// size.  The tiles, the partial matrices of a weight gradient and their reduction are shared with mconv.cu.
+// are no multiple of 16 (the first layer's 3 among them), launches of such channels in which mconv.cu would be slower (worth_it there: small images, few 1x1
+// tiles), all of them with kernel_path 1.  3x3 and 1x1, stride 1 and 2, any channel counts, any image size.  The tiles, the partial matrices of a weight gradient and their reduction are shared with mconv.cu.
 //
 //   fc_kernel : forward and input gradient.  A CTA computes 128 pixels x 16 output channels: the input region of its
 //               pixels (halo included) is fetched ONCE per 16-channel chunk and every filter tap reads it from shared memory.

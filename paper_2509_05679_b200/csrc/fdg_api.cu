@@ -64,7 +64,8 @@ struct Op {
     // tensor-core plan (bf16 storage, channel counts that are multiples of 64, power-of-two images)
     bool tc;
     bool stem;                                               // thin first-layer conv: dedicated FMA kernels
-    bool packed; size_t pack_off;                            // convolution in mconv.cu: where its weights are in the module's pack_f / pack_b (bytes)
+    bool mma;                                                // convolution that mconv.cu is asked for
+    bool packed[2]; size_t pack_off[2];                      // forward, backward: whether its weights are in the module's pack[], and where (bytes)
     size_t lin_off;                                          // linear layer on the CUDA cores: its weight-gradient workspace in the module's lin_ws (elements)
     bool head;                                               // the network's last linear layer: fused with the loss (head_* kernels)
     char shape[40];                                          // "HxW Cin->Cout kR sS", the profiler's detail tag
@@ -113,11 +114,11 @@ struct Module {
     char *in_ring, *stash, *gradpool, *d2, *wring, *wtring;
     float *master, *grad, *ws, *lin_ws, *scratch, *red, *cstat[2], *bstat;
     size_t lin_elems;
-    size_t pack_bytes;             // the weights of the convolutions of mconv.cu, per replica, as their kernels read them: of the version that the forward /
-    char *pack_f, *pack_b;         // the backward pass is at, laid out at its beginning,
-    bool pack_f_ok, pack_b_ok;     // if that launch was not refused (the packed-FMA kernels read the weights themselves)
+    size_t pack_bytes[2];          // [0] forward, [1] backward: the weights of the convolutions that mconv.cu takes, per replica, as their kernels read them,
+    char* pack[2];                 // of the version that the pass is at, laid out at its beginning
+    bool pack_ok[2];               // if that launch was not refused (the packed-FMA kernels read the weights themselves)
     struct Pack { PackArgs args; int blocks; };
-    std::vector<Pack> packs;
+    std::vector<Pack> packs[2];
     bool fused_update;             // one kernel per step updates all parameters and emits the next weight version (both layouts)
     tc::UpdTable upd;
     size_t cstat_elems[2];
@@ -288,6 +289,26 @@ void* default_alloc(size_t bytes, void*) {
     return nullptr;
 }
 void default_free(void* p, void*) { cudaFree(p); }
+
+// Which passes of which layers read their weights as mconv.cu wants them: those with a launch that goes there, of the whole batch, a group of workers or one
+// worker, as the passes make them.
+void plan_packs(const fdg_ctx* ctx, Module& m, bool first) {
+    m.pack_bytes[0] = m.pack_bytes[1] = 0;
+    for (Op& o : m.ops)
+        for (int back = 0; back < 2; ++back) {
+            if (o.type != OP_CONV || !o.mma || (back && first && o.in == 0)) continue;              // nobody wants the network's input gradient
+            const auto takes = [&](int n, int groups) { ConvGeom g = o.g; g.N = n; return mconv_takes(ctx->dt, g, groups, back); };
+            const auto window = [&](int groups) { const int nw = ctx->n_workers / groups; return takes(nw * ctx->B, !back && o.fstat_tiles ? nw : 1); };
+            // (a module whose tensor-core tiles do not fit its groups falls back to one)
+            o.packed[back] = ctx->R > 1 ? takes(ctx->M, ctx->R) || takes(ctx->B, 1) : window(m.groups) || window(1);
+            if (!o.packed[back]) continue;
+            o.pack_off[back] = m.pack_bytes[back]; m.pack_bytes[back] += mconv_pack_bytes(ctx->dt, o.g);
+            if (m.packs[back].empty() || m.packs[back].back().args.n == PackArgs::MAX) m.packs[back].push_back({});
+            Module::Pack& k = m.packs[back].back();
+            k.args.layer[k.args.n++] = PackLayer{o.w_off, o.pack_off[back] / 16, o.g.C, o.g.Co, o.g.R * o.g.R, k.blocks};
+            k.blocks += (o.g.C / 16) * (o.g.Co / 16);
+        }
+}
 
 // ---- compile layers [p,q) into ops; returns "" or an error text
 std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool last, size_t& canon_off) {
@@ -465,7 +486,7 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
         if (d.own_grad) { d.goff = goff; goff += align_up(d.elems() * ctx->M * ctx->esz, 256); }
     }
     size_t red_pos = 0;
-    m.ws_elems = 0; m.scratch_elems = 64; m.red_elems = 4; m.lin_elems = 0; m.pack_bytes = 0;
+    m.ws_elems = 0; m.scratch_elems = 64; m.red_elems = 4; m.lin_elems = 0;
     for (Op& o : m.ops) {
         if (o.type == OP_BN) {
             o.stats_off = soff; soff += align_up((size_t)ctx->n_workers * o.g.C * (ctx->dt == 0 ? 4 : 2) * sizeof(float), 256);
@@ -485,14 +506,7 @@ std::string compile_module(fdg_ctx* ctx, Module& m, int& h, int& w, int& c, bool
             }
             if (ctx->R > 1) m.ws_elems = std::max(m.ws_elems, fconv_wgrad_workspace_elems(o.g, ctx->R));
             m.scratch_elems = std::max(m.scratch_elems, (size_t)64 * o.g.Co);
-            const size_t pack = ctx->fma_only || o.tc || o.stem || o.head || linear_supported(o.g) ? 0 : mconv_pack_bytes(ctx->dt, o.g, 1);
-            if (pack) {
-                o.packed = true; o.pack_off = m.pack_bytes; m.pack_bytes += pack;
-                if (m.packs.empty() || m.packs.back().args.n == PackArgs::MAX) m.packs.push_back({});
-                Module::Pack& k = m.packs.back();
-                k.args.layer[k.args.n++] = PackLayer{o.w_off, o.pack_off / 16, o.g.C, o.g.Co, o.g.R * o.g.R, k.blocks};
-                k.blocks += (o.g.C / 16) * (o.g.Co / 16);
-            }
+            o.mma = !ctx->fma_only && !o.tc && !o.stem && !o.head && !linear_supported(o.g);
             if (relu_bias_backward_supported(ctx->dt, o.g.Co)) m.scratch_elems = std::max(m.scratch_elems, relu_bias_backward_scratch_elems(o.g.Co));
         }
     }
@@ -674,15 +688,15 @@ size_t row_off(const fdg_ctx* c, const TensorDesc& d, const Win& wn) {
 
 // The weights of version `version` for one pass of the convolutions in mconv.cu: one launch for all of a module's (up to PackArgs::MAX).
 void pack_weights(fdg_ctx* c, Module& m, int64_t version, bool back, cudaStream_t s) {
-    bool& ok = back ? m.pack_b_ok : m.pack_f_ok;
-    ok = true;
-    for (const Module::Pack& k : m.packs) {
+    m.pack_ok[back] = true;
+    for (const Module::Pack& k : m.packs[back]) {
         PackArgs a = k.args; a.back = back;
-        ok = mconv_pack(c->dt, wbig(c, m, version, 0), m.wslot_bytes / c->esz, back ? m.pack_b : m.pack_f, m.pack_bytes, a, k.blocks, c->R, s) && ok;
+        m.pack_ok[back] = mconv_pack(c->dt, wbig(c, m, version, 0), m.wslot_bytes / c->esz, m.pack[back], m.pack_bytes[back], a, k.blocks, c->R, s) && m.pack_ok[back];
     }
 }
-Packed packed_f(const Module& m, const Op& o, int rep) { return o.packed && m.pack_f_ok ? Packed{m.pack_f + rep * m.pack_bytes + o.pack_off, m.pack_bytes} : Packed{}; }
-Packed packed_b(const Module& m, const Op& o, int rep) { return o.packed && m.pack_b_ok ? Packed{m.pack_b + rep * m.pack_bytes + o.pack_off, m.pack_bytes} : Packed{}; }
+Packed packed(const Module& m, const Op& o, bool back, int rep) {
+    return o.packed[back] && m.pack_ok[back] ? Packed{m.pack[back] + rep * m.pack_bytes[back] + o.pack_off[back], m.pack_bytes[back]} : Packed{};
+}
 // all groups of a launch read the same weights
 Packed shared(Packed p) { p.group = 0; return p; }
 
@@ -721,12 +735,12 @@ void forward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int group, 
                     break;
                 }
                 if (o.fstat_tiles && fconv_forward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.bias ? wsmall(c, m, version, o.b_off, rep) : nullptr, T(o.out), g, epi,
-                                                   wn.nw, 0, 0, m.cstat[o.stat_buf], shared(packed_f(m, o, rep)), s)) {
+                                                   wn.nw, 0, 0, m.cstat[o.stat_buf], shared(packed(m, o, false, rep)), s)) {
                     m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.fstat_tiles;
                     profile_detail(nullptr);
                     break;
                 }
-                conv_forward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.bias ? wsmall(c, m, version, o.b_off, rep) : nullptr, T(o.out), g, epi, packed_f(m, o, rep), s);
+                conv_forward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), o.bias ? wsmall(c, m, version, o.b_off, rep) : nullptr, T(o.out), g, epi, packed(m, o, false, rep), s);
                 profile_detail(nullptr);
                 break; }
             case OP_BN: {
@@ -790,7 +804,7 @@ bool forward_op_replicas(fdg_ctx* c, int kk, int64_t batch, int64_t version, siz
             profile_detail(o.shape);
             bool ok = true;
             if (linear_supported(o.g)) linear_forward(dt, P.tensor(o.in), w, b, P.tensor(o.out), o.g, epi, c->R, wg, pg, s);
-            else ok = fconv_forward(dt, P.tensor(o.in), w, b, P.tensor(o.out), o.g, epi, c->R, wg, pg, o.fstat_tiles ? m.cstat[o.stat_buf] : nullptr, packed_f(m, o, 0), s);
+            else ok = fconv_forward(dt, P.tensor(o.in), w, b, P.tensor(o.out), o.g, epi, c->R, wg, pg, o.fstat_tiles ? m.cstat[o.stat_buf] : nullptr, packed(m, o, false, 0), s);
             if (ok && o.fstat_tiles) { m.fused_stats_tensor[o.stat_buf] = o.out; m.fused_stats_chunks[o.stat_buf] = o.fstat_tiles; }
             profile_detail(nullptr);
             return ok; }
@@ -904,13 +918,13 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
                 else if (o.stem) stem_wgrad(T(o.in), gout, mgrad + o.w_off, m.ws, g, acc_p, ws);
                 else if (o.tc && tc_wgrad(c, m, o, P.tensor(o.in), grad_ptr(c, kk, o.out, t), mgrad + o.w_off, wn, ws)) {}
                 else if (linear_supported(g)) linear_backward(dt, T(o.in), nullptr, nullptr, gout, nullptr, false, mgrad + o.w_off, nullptr, g, 1, 0, 0, acc_p, nullptr, ws, ws, m.wev);
-                else fconv_wgrad(dt, T(o.in), gout, mgrad + o.w_off, m.ws, g, 1, 0, acc_p, o.packed, ws);
+                else fconv_wgrad(dt, T(o.in), gout, mgrad + o.w_off, m.ws, g, 1, 0, acc_p, o.mma, ws);
                 if (o.bias && !fused_rb && !o.masked_by) bias_grad(dt, gout, mgrad + m.n_big + o.b_off, m.scratch, orows, g.Co, acc_p, s);
                 if (gin && !(o.tc && tc_dgrad(c, m, o, grad_ptr(c, kk, o.out, t), grad_ptr(c, kk, o.in, t), version, o.acc_in,
                                                      below ? P.tensor(o.in) : nullptr, col, wn, s))) {
                     c->mask_lost = c->mask_lost || below;
                     if (linear_supported(g)) linear_backward(dt, T(o.in), wbig(c, m, version, o.w_off, rep), nullptr, gout, gin, o.acc_in, nullptr, nullptr, g, 1, 0, 0, false, nullptr, s, s, m.wev);
-                    else fconv_dgrad(dt, gout, wbig(c, m, version, o.w_off, rep), gin, g, o.acc_in ? EPI_ACCUM : 0, 1, 0, packed_b(m, o, rep), s);
+                    else fconv_dgrad(dt, gout, wbig(c, m, version, o.w_off, rep), gin, g, o.acc_in ? EPI_ACCUM : 0, 1, 0, packed(m, o, true, rep), s);
                 }
                 profile_detail(nullptr);
                 break; }
@@ -980,8 +994,8 @@ bool backward_op_replicas(fdg_ctx* c, int kk, int64_t batch, int64_t version, in
             profile_detail(o.shape);
             cudaStream_t ws = m.wstream;
             if (ws != s) { step_record(m.wev, s); step_wait(ws, m.wev); }
-            fconv_wgrad(dt, P.tensor(o.in), gout, m.grad + o.w_off, m.ws, o.g, c->R, gg, false, o.packed, ws);
-            if (gin) fconv_dgrad(dt, gout, w, gin, o.g, o.acc_in ? EPI_ACCUM : 0, c->R, wg, packed_b(m, o, 0), s);
+            fconv_wgrad(dt, P.tensor(o.in), gout, m.grad + o.w_off, m.ws, o.g, c->R, gg, false, o.mma, ws);
+            if (gin) fconv_dgrad(dt, gout, w, gin, o.g, o.acc_in ? EPI_ACCUM : 0, c->R, wg, packed(m, o, true, 0), s);
             profile_detail(nullptr);
             return true; }
         case OP_BN:
@@ -1537,6 +1551,7 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
             while (g * 2 <= opt->worker_groups && n_workers % (g * 2) == 0) g *= 2;
             m.groups = g;
         }
+        plan_packs(ctx, m, kk == 0);
         m.in_slot_bytes = align_up((size_t)ctx->M * m.in_elems * ctx->esz, 256);
         m.wslot_bytes = align_up(m.n_big * ctx->esz + m.n_small * sizeof(float), 256);
     }
@@ -1587,8 +1602,7 @@ fdg_status fdg_create(const fdg_layer* layers, int32_t n_layers, const int32_t* 
         m.grad = (float*)get((size_t)ctx->R * (m.n_big + m.n_small) * sizeof(float));
         m.ws = (float*)get(m.ws_elems * sizeof(float));
         m.lin_ws = m.lin_elems ? (float*)get(m.lin_elems * sizeof(float)) : nullptr;
-        m.pack_f = m.pack_bytes ? get(m.pack_bytes * ctx->R) : nullptr;
-        m.pack_b = m.pack_bytes ? get(m.pack_bytes * ctx->R) : nullptr;
+        for (int back = 0; back < 2; ++back) m.pack[back] = m.pack_bytes[back] ? get(m.pack_bytes[back] * ctx->R) : nullptr;
         m.scratch = (float*)get(m.scratch_elems * sizeof(float));
         m.red = (float*)get(m.red_elems * sizeof(float));
         m.scratch_f = (float*)get(m.scratch_elems * sizeof(float));

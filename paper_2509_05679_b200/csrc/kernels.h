@@ -37,11 +37,13 @@ void   linear_backward(int dt, const void* x, const void* w, const void* y_or_nu
 bool   fconv_supported(const ConvGeom& g);
 // Layers of channel counts that are multiples of 16 run on warp-level tensor-core instructions (mconv.cu) if their weights are there in the order
 // that these read: mconv_pack lays out a module's layers (PackArgs, `blocks` 16 x 16 blocks in all) for one direction, per group `group` bytes apart.
-// mconv_pack_bytes: of one layer and direction, a multiple of 16; 0: shape not covered.
+// mconv_takes: whether a forward (back == false) or input-gradient launch of this many images and groups goes that way, given them.
+// mconv_pack_bytes: of one such layer and direction, a multiple of 16.
 struct Packed { const void* data; size_t group; };       // data == nullptr: the packed-FMA kernels
 struct PackLayer { size_t w_off, out_off; int C, Co, taps, block0; };        // elements into the matrices, 16-byte words into the result; first block
 struct PackArgs { enum { MAX = 48 }; PackLayer layer[MAX]; int n, back; };
-size_t mconv_pack_bytes(int dt, const ConvGeom& g, int groups);
+bool   mconv_takes(int dt, const ConvGeom& g, int groups, bool back);
+size_t mconv_pack_bytes(int dt, const ConvGeom& g);
 bool   mconv_pack(int dt, const void* wbig, size_t w_group, void* out, size_t out_group, const PackArgs& a, int blocks, int groups, cudaStream_t st);      // false: refused
 bool   fconv_forward(int dt, const void* x, const void* w, const float* bias, void* y, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,
                      float* stat_or_null, const Packed& pk, cudaStream_t st);

@@ -612,13 +612,39 @@ constexpr int SM_SMEM = 228 * 1024, CTA_SMEM = 1024;      // of an SM; what ever
 bool channels_ok(const ConvGeom& g) { return g.C % 16 == 0 && g.Co % 16 == 0; }
 template <typename T, int NB> size_t mc_smem(const McParams& q) { return (size_t)mc_x_bytes<T>(q.xp) + mc_w_bytes<T, NB>(q.wtaps, q.p.C / 16); }
 
+// CTAs of 16 output channels; the four parity classes of a 1x1 stride-2 input gradient, three of which have no tap and only write, count as two
+long mc_ctas(const McParams& q, int groups) {
+    const int classes = q.p.ncls > 1 && q.p.taps == 1 ? 2 : q.p.ncls;
+    return (long)classes * q.p.tiles_w * q.p.tiles_h * ((q.p.ngroup + q.p.Nt - 1) / q.p.Nt) * groups * (q.p.Co / 16);
+}
+// Whether mc_kernel takes a launch; the packed-FMA kernel has the others.  Both cut images into the same tiles.  A tile's region is fetched row by row, a warp a
+// row, and with fp32 storage split pixel by pixel before it is used; the packed-FMA kernel reads it as it is.  So the line lies where a
+// tile has many rows or, per tap, many pixels for its 128 outputs: small images, sides that exact covers of 2x2x32 or 1x1x128 pixels leave
+// (5, 6, 9, 10, 13, 14 ...), 1x1 layers; and further out where the CTAs of one wave have nobody to cover for them.  From 3 to 25 sides of 1 to
+// 56, 16 to 256 channels, 4 to 768 images (tensor core : packed FMA of the launches just inside / just outside):
+//   fp32 3x3            region of 300 pixels in up to one wave, 512 beyond      0.92 / 1.2 (5x5 and 6x6 images, 16 of them), 1.05 / 2.0 (1x1)
+//   fp32 3x3 stride 2   forward: 36 rows; backward: 180 pixels, 288 beyond      1.08 / 1.6 (20x20, 28x28 in 16 channels); 1.07 / 1.27 (4x4)
+//   fp32 1x1            4 rows in up to one wave, 16 in up to two, any beyond   1.0 / 1.25, 1.05 / 1.18, 1.05 / -
+//   bf16                128 rows in up to one wave, any beyond; 1x1 with fewer images than a tile holds: 32     0.96 / 1.26, 1.0 / 1.17
+// Some launches outside would gain: 0.7 at the best (bf16, 1x1 images, one wave).
+template <typename T> bool worth_it(const McParams& q, int groups) {
+    int rows = 0;
+    for (int c = 0; c < q.p.ncls; ++c) rows = std::max(rows, q.p.Nt * q.p.cls_rh[c]);
+    const long ctas = mc_ctas(q, groups);
+    const bool few = ctas <= 148;
+    if (!SPLIT<T>) return (rows <= 128 || !few) && !(q.p.taps == 1 && rows > 32 && q.p.ngroup < q.p.Nt);
+    if (q.p.taps == 1) return ctas > 2 * 148 || rows <= (few ? 4 : 16);
+    if (q.p.xs == 2) return rows <= 36;
+    if (q.p.ncls > 1) return q.xp <= (few ? 180 : 288);
+    return q.xp <= (few ? 300 : 512);
+}
 template <typename T>
 bool plan_mc(const ConvGeom& g, int groups, bool back, McParams& q) {
     if (!channels_ok(g) || !plan_fc(g, groups, back, q.p)) return false;
     q.xp = q.p.x_floats / PITCH;
     q.wtaps = q.p.w_floats / (16 * PITCH);
     for (int& t : q.p.toff) t /= PITCH;
-    return mc_smem<T, 4>(q) <= FC_SMEM_MAX;
+    return mc_smem<T, 4>(q) <= FC_SMEM_MAX && worth_it<T>(q, groups);
 }
 template <typename T>
 bool plan_mw(const ConvGeom& g, int groups, MwParams& q, size_t& smem) {
@@ -649,12 +675,6 @@ bool run_mc(const void* x, const void* w, const void* pk, const float* bias, voi
             cudaStream_t s) {
     McParams q;
     if (!plan_mc<T>(g, groups, back, q)) return false;
-    // Left to the packed-FMA kernel: tiles of many short rows (images of 3x3 and smaller; a warp fetches row by row: 2x2, 64 channels, fp32 41 us against 35, 3x3,
-    // 16 channels 43 against 23, 1x1 in bf16 22.7 against 20.6, but 2x2 in bf16 31 against 47), and fp32 1x1 stride 2, which would split four pixels
-    // for each that it uses, from two chunks on (8x8 256 -> 512 64 us against 51, 16x16 32 -> 64 8.9 against 8.3; one chunk 10.5 against 14.5).
-    int rows = 0;
-    for (int c = 0; c < q.p.ncls; ++c) rows = std::max(rows, q.p.Nt * q.p.cls_rh[c]);
-    if (rows > (SPLIT<T> ? 64 : 128) || (SPLIT<T> && q.p.taps == 1 && q.p.xs == 2 && q.p.C > FC_KC)) return false;
     q.p.epi = epi; q.p.w_group = w_group; q.p.b_group = b_group;
     q.pack_group = pack_group / 16;
     const long tiles = (long)q.p.tiles_w * q.p.tiles_h * ((q.p.ngroup + q.p.Nt - 1) / q.p.Nt) * groups * q.p.ncls;
@@ -684,13 +704,11 @@ int run_mw(const void* x, const void* dy, float* ws, const ConvGeom& g, int grou
 
 }  // namespace
 
-size_t mconv_pack_bytes(int dt, const ConvGeom& g, int groups) {
+bool mconv_takes(int dt, const ConvGeom& g, int groups, bool back) {
     McParams q;
-    const bool ok = dt ? plan_mc<bf16>(g, groups, false, q) && plan_mc<bf16>(g, groups, true, q) : plan_mc<float>(g, groups, false, q) && plan_mc<float>(g, groups, true, q);
-    if (!ok) return 0;
-    const size_t blocks = (size_t)(g.C / 16) * (g.Co / 16);
-    return blocks * g.R * g.R * (dt ? PACK16<bf16> : PACK16<float>) * 16;
+    return dt ? plan_mc<bf16>(g, groups, back, q) : plan_mc<float>(g, groups, back, q);
 }
+size_t mconv_pack_bytes(int dt, const ConvGeom& g) { return (size_t)(g.C / 16) * (g.Co / 16) * g.R * g.R * (dt ? PACK16<bf16> : PACK16<float>) * 16; }
 bool mconv_pack(int dt, const void* wbig, size_t w_group, void* out, size_t out_group, const PackArgs& a, int blocks, int groups, cudaStream_t s) {
     Scope sc(KC_TC_AUX, 0.0, (double)blocks * groups * 9 * 256 * (dt ? 4.0 : 8.0), s);
     return launched(dt ? klaunch(mc_pack_kernel<bf16>, dim3(blocks, groups), 256, 0, s, (const bf16*)wbig, w_group, (uint4*)out, out_group / 16, a)

@@ -74,3 +74,28 @@ def test_values_far_from_one(orc, exponent):
         got[:n1 + 16] = g[:n1 + 16]
     err, where = max_rel_err(got, g, net.layers)
     assert err <= 1e-5, (err, where)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_nothing_is_laid_out_for_other_kernels(dtype):
+    """Images of one pixel are left to the packed-FMA kernels: as much device memory and as many launches as with kernel_path 1.  Of images of 16x16 in the first layer only the
+    forward pass reads laid-out weights (nobody wants the network's input gradient): one launch more per iteration than there."""
+    import torch
+    from paper_2509_05679_b200 import binding
+    used = {}
+    for side in (1, 16):
+        layers = [(sy.CONV3X3, 16, 32, 1, 0), (sy.GLOBAL_AVGPOOL, 32, 32, 1, 0), (sy.LINEAR, 32, 10, 1, 1)]
+        net = sy.Net("mconv", layers, [], side, side, 16, 10, 2, 24, 0.05, dtype)
+        x, y = binding.to_device(dtype, sy.batch_inputs(net, 0)), torch.from_numpy(sy.batch_labels(net, 0)).cuda()
+        for path in (0, 1):
+            ctx = make_ctx(net, sy.init_params(layers, 0), kernel_path=path)
+            try:
+                ctx.step(x, y)
+                before = ctx.stats()[1]
+                for _ in range(3):
+                    ctx.step(x, y)
+                used[side, path] = (ctx.stats()[0], ctx.stats()[1] - before)
+            finally:
+                ctx.close()
+    assert used[1, 0] == used[1, 1], used
+    assert used[16, 0][1] == used[16, 1][1] + 3, used

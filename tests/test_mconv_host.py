@@ -113,3 +113,49 @@ int main() {
 def test_a_weight_gradient_is_one_wave(tmp_path):
     """As many CTAs as 148 SMs hold at a time: registers for four (bf16 storage three), 228 KB of shared memory with 1 KB more for each than it asks for."""
     run(tmp_path, ONE_WAVE)
+
+
+TAKEN = r"""
+// the kernel that a launch ran is the one that mconv_takes says
+static bool agrees(int dt, const ConvGeom& g, int groups, bool back, bool& taken) {
+    alignas(16) static char b[16];
+    const void* ran_[2];
+    for (int p = 0; p < 2; ++p) {
+        const Packed pk{p ? b : nullptr, 0};
+        ran.clear();
+        if (!(back ? fconv_dgrad(dt, b, b, b, g, 0, groups, 0, pk, 0) : fconv_forward(dt, b, b, nullptr, b, g, 0, groups, 0, 0, nullptr, pk, 0)) || ran.size() != 1) { taken = false; return !mconv_takes(dt, g, groups, back); }
+        ran_[p] = ran[0];
+    }
+    taken = ran_[0] != ran_[1];
+    return taken == mconv_takes(dt, g, groups, back);
+}
+int main() {
+    int n[2] = {};
+    for (int dt = 0; dt < 2; ++dt) for (int r : {1, 3}) for (int st : {1, 2}) for (int h : {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 13, 14, 16, 17, 20, 28, 32}) for (int w : {1, 2, 5, h})
+        for (int c : {16, 48, 64}) for (int images : {1, 4, 12, 192}) for (int groups : {1, 4}) for (int back = 0; back < 2; ++back) {
+            if (images % groups) continue;
+            bool taken;
+            CHECK(agrees(dt, conv(images, h, w, c, 32, r, st), groups, back, taken));
+            ++n[taken];
+        }
+    CHECK(n[0] > 1000 && n[1] > 1000);
+    // ordinary sizes, and the ends of each line of the rule
+    struct { int dt, images, side, c, co, r, st; bool back, taken; } list[] = {
+        {0, 192, 32, 16, 16, 3, 1, false, true}, {0, 192, 8, 64, 64, 3, 1, true, true}, {0, 192, 32, 16, 32, 3, 2, false, true}, {0, 192, 32, 16, 32, 3, 2, true, true}, {0, 192, 32, 16, 32, 1, 2, false, true},
+        {0, 192, 14, 64, 64, 3, 1, false, true}, {0, 16, 14, 16, 16, 3, 1, false, true}, {0, 192, 5, 32, 32, 3, 1, false, false}, {0, 768, 9, 64, 64, 3, 1, false, true}, {0, 768, 5, 64, 64, 3, 1, false, false}, {0, 768, 1, 16, 16, 3, 1, false, false},
+        {0, 192, 28, 16, 16, 3, 2, false, false}, {0, 768, 4, 32, 64, 3, 2, true, true}, {0, 16, 4, 32, 64, 3, 2, true, false},
+        {0, 4, 32, 16, 16, 1, 1, false, true}, {0, 16, 16, 16, 16, 1, 1, false, false}, {0, 64, 16, 48, 48, 1, 1, false, true}, {0, 768, 3, 64, 64, 1, 1, false, false}, {0, 768, 5, 64, 64, 1, 1, false, true},
+        {1, 192, 1, 16, 16, 3, 1, false, false}, {1, 4096, 1, 256, 256, 3, 1, false, true}, {1, 192, 2, 16, 16, 3, 1, false, true}, {1, 16, 2, 64, 64, 1, 1, false, false}, {1, 192, 2, 64, 64, 1, 1, false, true}};
+    for (const auto& l : list) {
+        bool taken;
+        if (!agrees(l.dt, conv(l.images, l.side, l.side, l.c, l.co, l.r, l.st), 1, l.back, taken) || taken != l.taken)
+            { printf("dt%d %d images of %d, %d -> %d k%d s%d %s: %d\n", l.dt, l.images, l.side, l.c, l.co, l.r, l.st, l.back ? "back" : "forward", taken); return 1; }
+    }
+    return 0;
+}
+"""
+
+
+def test_one_rule_says_who_takes_a_launch(tmp_path):
+    """What decides whether weights are laid out is what decides who reads them."""
+    run(tmp_path, TAKEN)
