@@ -10,7 +10,7 @@
 // a product the sum of the six that matter: lo hi + mid mid + hi lo + mid hi + hi mid + hi hi (the rest is 6e-9 of it; 6e-8, and one-sided, with parts by
 // truncation).  Every product is exact; an mma adds 16 of them to its running sum and truncates to 24 bits of the largest term: 2.5e-8 of the
 // result's rms for 16 fresh products of 16 bits, 1.3e-7 for nine such steps in a chain, 5.3e-7 for 36, 1e-7 as soon as a 24-bit running sum of
-// like size is among the terms.  So hi hi starts from zero in every step and goes into an fp32 sum on the CUDA cores, two taps of it (MC_RUN) into a
+// like size is among the terms.  So hi hi starts from zero in every step and goes into an fp32 sum on the CUDA cores, two taps of it into a
 // compensated (Kahan) sum, in a weight gradient of fp32 storage every step (four CTAs per SM have no registers for both); the other five, 2^-6 of
 // it at the most, run on in one accumulator per chunk.  What truncation takes away has the sign of the sum: 1.7e-8 of a sum of products of one sign with 16-bit
 // products.  One operand's hi (the weights', where the pack does it once; dy's in a weight gradient) therefore has 6 bits, as few as three parts allow: 14-bit
@@ -22,7 +22,7 @@
 // 1.6 and 1.75 times those of the packed-FMA kernels (22.7 us for what takes 25 now).  Two fp16 parts and three products were off by 9.4e-8:
 // 22-bit products lose more where the terms are aligned.  bf16 storage: one exact product a step, weight gradients flushed every MW_RUN steps and the splits
 // added in double: 1.00 times the packed-FMA kernels' errors at the most, 0.8 on average (1.19 with a flush per tile).  Forward and input gradient keep to
-// one flush per chunk there: 6.5e-8 before the result is rounded to bf16, by 1.7e-3 (4.4e-8; a flush every MC_RUN taps gives 4.6e-8 for 4.5 % of a step).
+// one flush per chunk there: 6.5e-8 before the result is rounded to bf16, by 1.7e-3 (4.4e-8; one every two taps gives 4.6e-8 for 4.5 % of a step).
 //
 // Time, 192 images, launch included (packed FMA beside it): fp32 32x32 16 -> 16 forward 25 us (38), weight gradient with its reduction 38 (54); 16x16 32 -> 32 27
 // (40), 36 (53); 8x8 64 -> 64 29 (41), 39 (57).  What bounds them: a third to 40 % of the mma.sync rate (980 multiply-adds per clock and SM, six per
@@ -38,8 +38,7 @@ namespace {
 
 constexpr int MC_THREADS = 128;
 constexpr int W_HI = 6, DY_HI = 6;       // bits of hi in the weights and, in a weight gradient, in dy
-constexpr int MC_RUN = 2;                // taps whose sums of hi hi are added before they go into the compensated sum (fp32 storage)
-constexpr int MW_RUN = 4;                // the same in a weight gradient: 16-pixel steps (bf16 storage)
+constexpr int MW_RUN = 4;                // steps of a weight gradient that are added before they go into the compensated sum (bf16 storage)
 
 template <typename T> constexpr bool SPLIT = sizeof(T) == 4;
 template <typename T> constexpr int PARTS = SPLIT<T> ? 3 : 1;             // bf16 values per value
@@ -251,25 +250,16 @@ __global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc
             if (c + 1 < chunks) { fetch_x(c + 1, buf ^ 1); fetch_w(c + 1, buf ^ 1); cp_commit(); cp_wait<1>(); } else cp_wait<0>();
             __syncthreads();
         }
-        float2 acc[2][NB][2];                        // of hi hi, over MC_RUN taps (bf16 storage: over all)
-        float rest[2][NB][4];                        // fp32 storage: of the other products, over the chunk
+        float rest[2][NB][4];                        // fp32 storage: of all products but hi hi, over the chunk
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
             for (int j = 0; j < NB; ++j) rest[i][j][0] = rest[i][j][1] = rest[i][j][2] = rest[i][j][3] = 0.f;
         const char* const ws_ = wst + buf * wbuf + lane * (S ? 16 : 8);
         const uint32_t xo = S ? 0u : (uint32_t)(buf * plane_bytes);
-#pragma unroll 1
-        for (int t = 0; t < nt; ++t) {
-            if (t == 0 || (S && t % MC_RUN == 0)) {
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-#pragma unroll
-                    for (int j = 0; j < NB; ++j) acc[i][j][0] = acc[i][j][1] = make_float2(0.f, 0.f);
-            }
+        auto tap = [&](int t, float (&part)[2][NB][4]) {
             const uint32_t off = xo + (uint32_t)p.toff[t0 + t] * 16u;
             uint32_t a[2][PARTS<T>][4], b[NB][PARTS<T>][2];
-            float part[2][NB][4];
 #pragma unroll
             for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -292,28 +282,34 @@ __global__ void __launch_bounds__(MC_THREADS, NB == 4 ? SPLIT<T> ? 2 : 3 : 4) mc
                         if (k + 1 < PRODUCTS<T>) mma(rest[i][j], a[i][part_a<T>(k)], b[j][part_b<T>(k)][0], b[j][part_b<T>(k)][1], true);
                         else mma(part[i][j], a[i][0], b[j][0][0], b[j][0][1], false);
                     }
-#pragma unroll
-            for (int j = 0; j < NB; ++j)
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-#pragma unroll
-                    for (int r = 0; r < 2; ++r) acc[i][j][r] = __fadd2_rn(acc[i][j][r], make_float2(part[i][j][2 * r], part[i][j][2 * r + 1]));
-            if (t + 1 == nt || (S && t % MC_RUN == MC_RUN - 1)) {
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-#pragma unroll
-                    for (int j = 0; j < NB; ++j)
-#pragma unroll
-                        for (int r = 0; r < 2; ++r) add_kahan(sum[i][j][r], lost[i][j][r], acc[i][j][r]);
-            }
-        }
-        if (S)
+        };
+        auto each = [&](auto f) {                    // over the lane's pairs of outputs
 #pragma unroll
             for (int i = 0; i < 2; ++i)
 #pragma unroll
                 for (int j = 0; j < NB; ++j)
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) lost[i][j][r] = __fadd2_rn(lost[i][j][r], make_float2(rest[i][j][2 * r], rest[i][j][2 * r + 1]));
+                    for (int r = 0; r < 2; ++r) f(i, j, r);
+        };
+        auto pair = [](const float (&v)[4], int r) { return make_float2(v[2 * r], v[2 * r + 1]); };
+        float one[2][NB][4];
+        if constexpr (S) {                           // two taps into the compensated sum at a time
+            int t = 0;
+#pragma unroll 1
+            for (; t + 1 < nt; t += 2) {
+                float two[2][NB][4];
+                tap(t, one); tap(t + 1, two);
+                each([&](int i, int j, int r) { add_kahan(sum[i][j][r], lost[i][j][r], __fadd2_rn(pair(one[i][j], r), pair(two[i][j], r))); });
+            }
+            if (t < nt) { tap(t, one); each([&](int i, int j, int r) { add_kahan(sum[i][j][r], lost[i][j][r], pair(one[i][j], r)); }); }
+            each([&](int i, int j, int r) { lost[i][j][r] = __fadd2_rn(lost[i][j][r], pair(rest[i][j], r)); });
+        } else {                                     // the whole chunk
+            float2 acc[2][NB][2];
+            each([&](int i, int j, int r) { acc[i][j][r] = make_float2(0.f, 0.f); });
+#pragma unroll 1
+            for (int t = 0; t < nt; ++t) { tap(t, one); each([&](int i, int j, int r) { acc[i][j][r] = __fadd2_rn(acc[i][j][r], pair(one[i][j], r)); }); }
+            each([&](int i, int j, int r) { add_kahan(sum[i][j][r], lost[i][j][r], acc[i][j][r]); });
+        }
         if (!S) __syncthreads();                     // this buffer is consumed
     }
 
