@@ -440,14 +440,20 @@ int bnf_chunks(int nw, long rpw, int C) {
 }  // namespace
 
 template <bool BWD>
-static void bnc_launch(const BncArgs& a, int nw, int nw_all, cudaStream_t s) {
+static void bnc_launch(const BncArgs& a, int nw, int nw_all, int modules, cudaStream_t s) {
     // channels per cluster: 64 (whole 128-byte lines), fewer where that makes less than 25 CTAs: many small CTAs end one launch sooner, but the SMs are
     // wanted by the other modules (18 samples, 4 modules: 386 us per step with this line, 432 with 100 CTAs; by the number of ALL workers: a launch for
-    // a group of them adds in the same order)
+    // a group of them adds in the same order).
+    // Long columns, more than 20 rows a thread: fewer until no SM is without a CTA, if the SMs are free for it.  With one module they are (us per step, left without):
+    // ResNet-18 2 x 12 931 (958), 4 x 6 904 (965), ResNet-20 4 x 48 1164 (1234).  With two, the other one's convolutions leave room on their SMs
+    // if they are those of mconv.cu, which is where channels are no multiple of 64 (ResNet-20 4 x 48 828 (849), 4 x 42 779 (792)), not if a
+    // CTA of theirs fills an SM (ResNet-18 2 x 12 553 (540)); with more modules somebody wants them (ResNet-20 4 x 48 K=3 765 (756), K=4 774 (755), ResNet-18 K=4 2 x 12
+    // 425 (406), 1 x 48 528 (514), 4 x 6 464 (444)).  Up to 20 rows a launch is short enough as it is (2 x 9, 18 rows: 378 (377)).
     int sl = 64;
+    const bool room = modules == 1 || (modules == 2 && a.C % 64 != 0);
     const auto ctas = [&] { return (a.C / sl) * nw_all * BNC_RANKS; };
-    const auto rows_a_thread = [&] { return (a.rpw + BNC_RANKS - 1) / BNC_RANKS * (sl / 8) / BT; };
-    while (sl > 16 && (a.C % sl || ctas() < 25 || (rows_a_thread() > 20 && ctas() < 148))) sl /= 2;
+    const auto long_columns = [&] { return (long)(a.rpw + BNC_RANKS - 1) / BNC_RANKS * (sl / 8) > 20L * BT; };
+    while (sl > 16 && (a.C % sl || ctas() < 25 || (room && long_columns() && ctas() < 148))) sl /= 2;
     const dim3 grid((a.C / sl) * BNC_RANKS, nw);
     if (sl == 64) klaunch_cluster(bnc_kernel<64, BWD>, grid, BT, 0, s, BNC_RANKS, a);
     else if (sl == 32) klaunch_cluster(bnc_kernel<32, BWD>, grid, BT, 0, s, BNC_RANKS, a);
@@ -456,19 +462,20 @@ static void bnc_launch(const BncArgs& a, int nw, int nw_all, cudaStream_t s) {
 // Tensors up to 4 MB: read twice out of L2 (beyond that the streamed kernels' rate counts, not the launches: 4 workers x 16, 693 us per step with the
 // line at 4 MB, 729 at 8 MB, 820 at 17 MB), and few enough rows per thread for plain fp32 sums (at most 16 384 / 8 / 32 = 64).
 bool bnc_supported(int dt, int nw, long rpw, int C) { return dt == 1 && C % 16 == 0 && rpw <= 16384 && (double)nw * rpw * C * 2.0 <= 4e6; }
-void bnc_forward(const void* x, const float* gamma, const float* beta, const void* res, void* y, float* stats, int nw, int nw_all, long rpw, int C, bool relu, cudaStream_t s) {
+void bnc_forward(const void* x, const float* gamma, const float* beta, const void* res, void* y, float* stats, int nw, int nw_all, int modules, long rpw, int C, bool relu,
+                 cudaStream_t s) {
     BncArgs a{};
     a.x = (const bf16*)x; a.gamma = gamma; a.beta = beta; a.res = (const bf16*)res; a.y = (bf16*)y; a.stats = stats; a.rpw = (int)rpw; a.C = C; a.relu = relu;
     Scope sc(KC_BN_FWD_APPLY, 0.0, 2.0 * nw * rpw * C * (res ? 3 : 2), s);
-    bnc_launch<false>(a, nw, nw_all, s);
+    bnc_launch<false>(a, nw, nw_all, modules, s);
 }
 void bnc_backward(const void* x, const void* out, const void* dout, const float* gamma, const float* beta, const float* stats, void* dx, bool accum_dx, void* dres,
-                  bool accum_dres, float* red, int nw, int nw_all, long rpw, int C, bool relu, bool has_res, cudaStream_t s) {
+                  bool accum_dres, float* red, int nw, int nw_all, int modules, long rpw, int C, bool relu, bool has_res, cudaStream_t s) {
     BncArgs a{};
     a.x = (const bf16*)x; a.out = (const bf16*)out; a.dout = (const bf16*)dout; a.gamma = gamma; a.beta = beta; a.stats = (float*)stats; a.y = (bf16*)dx;
     a.accum_dx = accum_dx; a.dres = (bf16*)dres; a.accum_dres = accum_dres; a.red = red; a.rpw = (int)rpw; a.C = C; a.relu = relu; a.mask_from_x = relu && !has_res;
     Scope sc(KC_BN_BWD_APPLY, 0.0, 2.0 * nw * rpw * C * (3 + (relu && has_res ? 1 : 0) + (accum_dx ? 1 : 0) + (dres ? (accum_dres ? 2 : 1) : 0)), s);
-    bnc_launch<true>(a, nw, nw_all, s);
+    bnc_launch<true>(a, nw, nw_all, modules, s);
 }
 void bnc_params(const float* red, float* dgamma, float* dbeta, int nw, int C, cudaStream_t s) {
     Scope sc(KC_BN_BWD_REDUCE, 0.0, 8.0 * nw * C, s);

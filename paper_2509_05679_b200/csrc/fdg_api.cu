@@ -749,7 +749,7 @@ void forward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int group, 
                 profile_detail(tag);
                 if (o.bn_small) {
                     bnc_forward(T(o.in), wsmall(c, m, version, o.gamma_off, rep), wsmall(c, m, version, o.beta_off, rep), o.has_res ? T(o.in2) : nullptr, T(o.out),
-                                P.stats(o) + (size_t)wn.w0 * ti.c * 2, wn.nw, c->n_workers, (long)c->B * ti.h * ti.w, ti.c, o.relu, s);
+                                P.stats(o) + (size_t)wn.w0 * ti.c * 2, wn.nw, c->n_workers, c->K, (long)c->B * ti.h * ti.w, ti.c, o.relu, s);
                     profile_detail(nullptr);
                     break;
                 }
@@ -935,7 +935,7 @@ void backward_ops(fdg_ctx* c, int kk, int64_t batch, int64_t version, int64_t t,
                 char* gres = o.has_res ? G(o.in2) : nullptr;
                 if (o.bn_small) {
                     bnc_backward(T(o.in), T(o.out), gout, wsmall(c, m, version, o.gamma_off, rep), wsmall(c, m, version, o.beta_off, rep), P.stats(o) + (size_t)wn.w0 * ti.c * 2,
-                                 gin, o.acc_in, gres, o.acc_in2, m.red + o.red_off + (size_t)wn.w0 * ti.c * 2, wn.nw, c->n_workers, (long)c->B * ti.h * ti.w, ti.c, o.relu, o.has_res, s);
+                                 gin, o.acc_in, gres, o.acc_in2, m.red + o.red_off + (size_t)wn.w0 * ti.c * 2, wn.nw, c->n_workers, c->K, (long)c->B * ti.h * ti.w, ti.c, o.relu, o.has_res, s);
                     if (wn.w0 + wn.nw < c->n_workers) { profile_detail(nullptr); break; }        // the last group adds up all workers' sums
                     cudaStream_t ws = m.wstream;                     // the parameter gradients are needed by the update only
                     if (ws != s) { step_record(m.wev, s); step_wait(ws, m.wev); }

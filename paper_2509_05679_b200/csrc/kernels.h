@@ -106,11 +106,13 @@ bool bn_accepts_conv_partials(int dt, int C);
 // summed over them).  mask_from_x: the forward output was bnf_forward's without a residual, so its sign can be recomputed from x.
 // scratch: as in bn_backward.  bn_merge_tiles: (mean, invstd) per worker and channel from such records, any storage type.
 // bf16 storage, tensors of a few MB (bnorm.cu): one launch per direction, statistics included.  red: [n_workers][C][2] floats, from which
-// bnc_params adds up dgamma, dbeta.  nw: the workers of this launch (pointers to the first one's), nw_all: all of them.
+// bnc_params adds up dgamma, dbeta.  nw: the workers of this launch (pointers to the first one's), nw_all: all of them; modules: of the network,
+// which share the device.
 bool bnc_supported(int dt, int nw, long rpw, int C);
-void bnc_forward(const void* x, const float* gamma, const float* beta, const void* res, void* y, float* stats, int nw, int nw_all, long rpw, int C, bool relu, cudaStream_t st);
+void bnc_forward(const void* x, const float* gamma, const float* beta, const void* res, void* y, float* stats, int nw, int nw_all, int modules, long rpw, int C, bool relu,
+                 cudaStream_t st);
 void bnc_backward(const void* x, const void* out, const void* dout, const float* gamma, const float* beta, const float* stats, void* dx, bool accum_dx, void* dres,
-                  bool accum_dres, float* red, int nw, int nw_all, long rpw, int C, bool relu, bool has_res, cudaStream_t st);
+                  bool accum_dres, float* red, int nw, int nw_all, int modules, long rpw, int C, bool relu, bool has_res, cudaStream_t st);
 void bnc_params(const float* red, float* dgamma, float* dbeta, int nw, int C, cudaStream_t st);
 bool bnf_supported(int dt, int C);
 void bn_merge_tiles(const float* tile_part, float* stats, int tiles, int nw, long rpw, int C, cudaStream_t st);

@@ -1,4 +1,4 @@
-"""Host side of csrc/mconv.cu and csrc/fconv.cu without a GPU: their objects linked against a runtime that records launches and refuses the
+"""Host side of csrc/mconv.cu, csrc/fconv.cu and csrc/bnorm.cu without a GPU: their objects linked against a runtime that records launches and refuses the
 ones it is told to."""
 import os
 import subprocess
@@ -80,7 +80,7 @@ def run(tmp_path, program):
     if not os.path.exists(os.path.join(inc, "cuda_runtime.h")):
         pytest.skip("no CUDA headers")
     build.build_lib()
-    objs = [os.path.join(build.CSRC, f) for f in ("mconv.o", "fconv.o")]
+    objs = [os.path.join(build.CSRC, f) for f in ("mconv.o", "fconv.o", "bnorm.o")]
     if not all(os.path.exists(o) for o in objs):
         pytest.skip("the library was built elsewhere: no objects")
     src, exe = tmp_path / "t.cpp", tmp_path / "t"
@@ -159,3 +159,26 @@ int main() {
 def test_one_rule_says_who_takes_a_launch(tmp_path):
     """What decides whether weights are laid out is what decides who reads them."""
     run(tmp_path, TAKEN)
+
+
+SLICES = r"""
+static int slice(int channels, int workers, long rows, int modules) {
+    alignas(16) static char b[16];
+    const float* const f = (const float*)b;
+    grids.clear();
+    bnc_forward(b, f, f, nullptr, b, (float*)b, workers, workers, modules, rows, channels, true, 0);
+    return channels * 8 / (int)grids[0].first.x;         // eight CTAs a cluster
+}
+int main() {
+    // 12288 rows: 24 a thread of 32 channels
+    CHECK(slice(64, 2, 12288, 1) == 16 && slice(64, 2, 12288, 2) == 32 && slice(64, 2, 12288, 4) == 32);
+    CHECK(slice(32, 4, 12288, 1) == 16 && slice(32, 4, 12288, 2) == 16 && slice(32, 4, 12288, 3) == 32);
+    // 18 rows, 20 rows a thread and one row more
+    CHECK(slice(64, 2, 9216, 1) == 32 && slice(32, 4, 10240, 1) == 32 && slice(32, 4, 10241, 1) == 16);
+    return 0;
+}
+"""
+
+
+def test_batch_norm_slices_leave_the_other_modules_room(tmp_path):
+    run(tmp_path, SLICES)
