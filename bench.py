@@ -60,6 +60,18 @@ def traffic_per_launch(kernel_class):
     return rec["bytes_per_launch"]
 
 
+def compute_peak(kernel_class, dtype, pk):
+    """(bound, TFLOP/s, source) of what a class of contraction kernels runs on; None for the others.  mma_*: fp32 storage takes six bf16 products for one."""
+    source = pk["source"] + ", burst bf16 GEMM (a kernel timed alone)"
+    if kernel_class.startswith("tc_gemm") or (kernel_class.startswith("mma_") and dtype == "bf16"):
+        return "tensor", pk["tensor_burst"], source
+    if kernel_class.startswith("mma_"):
+        return "tensor", pk["tensor_burst"] / 6, "a sixth of " + source
+    if kernel_class.startswith("fma_"):
+        return "alu", FMA_PEAK_TFLOPS, "derived: 148 SMs x 128 FMA x 2 x 1.965 GHz"
+    return None
+
+
 def peaks():
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(path):
@@ -321,16 +333,15 @@ def main():
                     "kernel_ms_per_step_all_classes": total_ms / kernel_steps, "traffic": traffic_per_launch(name),
                     "timing": f"CUDA events around every launch, separate pass of {kernel_steps} steps with all modules on one stream "
                               "(each event pair brackets one kernel running alone); not part of the timed region of `value`"}
-            if name.startswith("tc_gemm") or name.startswith("fma_"):
-                tensor = name.startswith("tc_gemm")
+            unit = compute_peak(name, net.dtype, pk)
+            if unit:
+                bound, peak, source = unit
                 ach = st["flops"] / (st["ms"] * 1e-3) / 1e12
-                peak = pk["tensor_burst"] if tensor else FMA_PEAK_TFLOPS
-                base.update({"bound": "tensor" if tensor else "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
+                base.update({"bound": bound, "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                              # the launch is sized for grid_sms of the device's SMs (others run kernels of other modules
                              # meanwhile): its fraction of what those SMs can do
                              "frac_of_sm_share": ach / (peak * kernel_grid_sms / device_sms),
-                             "peak_source": (pk["source"] + ", burst bf16 GEMM (a kernel timed alone)") if tensor
-                             else "derived: 148 SMs x 128 FMA x 2 x 1.965 GHz"})
+                             "peak_source": source})
             else:
                 ach = st["bytes"] / (st["ms"] * 1e-3) / 1e9
                 base.update({"bound": "hbm", "achieved": ach, "peak": pk["hbm"], "unit": "GB/s", "frac": ach / pk["hbm"], "peak_source": pk["source"]})

@@ -668,9 +668,8 @@ bool fconv_forward(int dt, const void* x, const void* w, const float* bias, void
     FcParams p;
     if (!plan_fc(g, groups, false, p)) return false;
     p.epi = epi; p.w_group = w_group; p.b_group = b_group;
-    const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
-    Scope sc(KC_FMA_FWD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + g.Co * K + rows * g.Co), s);
     if (pk.data && mconv_forward(dt, x, w, pk, bias, y, stat, g, epi, groups, w_group, b_group, s)) return true;
+    Scope sc(KC_FMA_FWD, conv_flops(g), conv_bytes(dt, g, false), s);
     if (dt) dispatch_fc<bf16>(x, w, bias, y, stat, p, groups, s); else dispatch_fc<float>(x, w, bias, y, stat, p, groups, s);
     return true;
 }
@@ -678,9 +677,8 @@ bool fconv_dgrad(int dt, const void* dy, const void* w, void* dx, const ConvGeom
     FcParams p;
     if (!plan_fc(g, groups, true, p)) return false;
     p.epi = epi; p.w_group = w_group;
-    const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
-    Scope sc(KC_FMA_DGRAD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + g.Co * K + rows * g.Co), s);
     if (pk.data && mconv_dgrad(dt, dy, w, pk, dx, g, epi, groups, w_group, s)) return true;
+    Scope sc(KC_FMA_DGRAD, conv_flops(g), conv_bytes(dt, g, false), s);
     if (dt) dispatch_fc<bf16>(dy, w, nullptr, dx, nullptr, p, groups, s); else dispatch_fc<float>(dy, w, nullptr, dx, nullptr, p, groups, s);
     return true;
 }
@@ -699,13 +697,11 @@ bool fconv_wgrad(int dt, const void* x, const void* dy, float* dw, float* ws, co
     FwParams p; int G, run; size_t smem;
     if (!plan_fw(g, groups, FW_CTAS, p, G, run, smem)) return false;
     const int xs = g.R == 1 ? 1 : g.stride, blocks = p.ci_blocks * ((g.Co + FW_CO - 1) / FW_CO), nout = FW_CO * p.ntaps * 8 * G;
-    const double rows = (double)g.N * g.Ho * g.Wo, K = (double)g.R * g.R * g.C;
-    int splits;
-    {
-        Scope sc(KC_FMA_WGRAD, 2.0 * rows * g.Co * K, (dt ? 2.0 : 4.0) * ((double)g.N * g.H * g.W * g.C + rows * g.Co) + 4.0 * K * g.Co, s);
-        splits = tensor ? mconv_wgrad(dt, x, dy, ws, g, groups, s) : 0;
-        if (splits) p.splits = splits;
-        else if (dt) dispatch_fw<bf16>(x, dy, ws, p, xs, G, run, groups, smem, s); else dispatch_fw<float>(x, dy, ws, p, xs, G, run, groups, smem, s);
+    const int splits = tensor ? mconv_wgrad(dt, x, dy, ws, g, groups, s) : 0;
+    if (splits) p.splits = splits;
+    else {
+        Scope sc(KC_FMA_WGRAD, conv_flops(g), conv_bytes(dt, g, true), s);
+        if (dt) dispatch_fw<bf16>(x, dy, ws, p, xs, G, run, groups, smem, s); else dispatch_fw<float>(x, dy, ws, p, xs, G, run, groups, smem, s);
     }
     Scope sc(KC_SPLITK, 0.0, 4.0 * groups * (p.splits + 1) * blocks * nout, s);
     const dim3 rgrid((nout + 31) / 32, blocks, groups);

@@ -52,6 +52,13 @@ bool plan_fc(const ConvGeom& g, int groups, bool back, FcParams& p);
 // Of a weight gradient by `ctas` CTAs; smem: of fw_kernel.
 bool plan_fw(const ConvGeom& g, int groups, int ctas, FwParams& p, int& G, int& run, size_t& smem);
 
+// Work of one pass of a layer for the profiler: multiply-adds, and its two activations and its weights (fp32 gradients) once each.
+inline double conv_flops(const ConvGeom& g) { return 2.0 * g.N * g.Ho * g.Wo * g.Co * g.R * g.R * g.C; }
+inline double conv_bytes(int dt, const ConvGeom& g, bool wgrad) {
+    const double w = (double)g.R * g.R * g.C * g.Co, e = dt ? 2.0 : 4.0;
+    return e * ((double)g.N * g.H * g.W * g.C + (double)g.N * g.Ho * g.Wo * g.Co) + (wgrad ? 4.0 : e) * w;
+}
+
 // The tensor-core forms (mconv.cu), tried first by the fconv_* functions; false / 0: not covered or refused, nothing launched.
 // mconv_wgrad leaves partial matrices as fw_kernel does and returns their number per block.
 bool mconv_forward(int dt, const void* x, const void* w, const Packed& pk, const float* bias, void* y, float* stat, const ConvGeom& g, int epi, int groups, size_t w_group, size_t b_group,

@@ -22,6 +22,7 @@ static const char* kClassNames[KC_COUNT] = {
     "fma_fwd", "fma_dgrad", "fma_wgrad", "splitk_reduce", "bias_grad", "relu_fwd", "relu_bwd", "add_fwd",
     "copy_accumulate", "maxpool_fwd", "maxpool_bwd", "gap_fwd", "gap_bwd", "bn_fwd_stats", "bn_fwd_apply", "bn_bwd_reduce",
     "bn_bwd_apply", "softmax_ce", "sgd_update", "tags", "fill", "tc_gemm_fwd", "tc_gemm_dgrad", "tc_gemm_wgrad", "tc_aux", "ingest",
+    "mma_fwd", "mma_dgrad", "mma_wgrad",
 };
 namespace prof {
 struct Rec { int cls; cudaEvent_t a, b; };

@@ -184,7 +184,9 @@ uint64_t launches();     // kernels launched so far through this interface
 enum KernelClass {
     KC_FMA_FWD, KC_FMA_DGRAD, KC_FMA_WGRAD, KC_SPLITK, KC_BIAS_GRAD, KC_RELU_FWD, KC_RELU_BWD, KC_ADD_FWD, KC_COPY_ACC,
     KC_POOL_FWD, KC_POOL_BWD, KC_GAP_FWD, KC_GAP_BWD, KC_BN_FWD_STATS, KC_BN_FWD_APPLY, KC_BN_BWD_REDUCE, KC_BN_BWD_APPLY,
-    KC_SOFTMAX_CE, KC_SGD, KC_TAGS, KC_FILL, KC_TC_FWD, KC_TC_DGRAD, KC_TC_WGRAD, KC_TC_AUX, KC_INGEST, KC_COUNT
+    KC_SOFTMAX_CE, KC_SGD, KC_TAGS, KC_FILL, KC_TC_FWD, KC_TC_DGRAD, KC_TC_WGRAD, KC_TC_AUX, KC_INGEST,
+    KC_MMA_FWD, KC_MMA_DGRAD, KC_MMA_WGRAD,        // mconv.cu
+    KC_COUNT
 };
 struct KernelStat { uint64_t launches; double ms, flops, bytes; };
 // Opened around every launch: counts it and, while profiling is enabled, records an event before and

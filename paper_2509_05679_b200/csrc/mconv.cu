@@ -671,6 +671,7 @@ bool run_mc(const void* x, const void* w, const void* pk, const float* bias, voi
             cudaStream_t s) {
     McParams q;
     if (!plan_mc<T>(g, groups, back, q)) return false;
+    Scope sc(back ? KC_MMA_DGRAD : KC_MMA_FWD, conv_flops(g), conv_bytes(SPLIT<T> ? 0 : 1, g, false), s);
     q.p.epi = epi; q.p.w_group = w_group; q.p.b_group = b_group;
     q.pack_group = pack_group / 16;
     const long tiles = (long)q.p.tiles_w * q.p.tiles_h * ((q.p.ngroup + q.p.Nt - 1) / q.p.Nt) * groups * q.p.ncls;
@@ -690,6 +691,7 @@ template <typename T>
 int run_mw(const void* x, const void* dy, float* ws, const ConvGeom& g, int groups, cudaStream_t s) {
     MwParams q; size_t smem;
     if (!plan_mw<T>(g, groups, q, smem)) return 0;
+    Scope sc(KC_MMA_WGRAD, conv_flops(g), conv_bytes(SPLIT<T> ? 0 : 1, g, true), s);
     const int blocks = q.p.ci_blocks * (g.Co / FW_CO);
     cudaError_t e;
     if (g.R == 1) e = launch_mw<T, 1, 1>(x, dy, ws, q, groups, blocks, smem, s);

@@ -23,6 +23,17 @@ def test_reference_arm_prints_the_contract_line():
     assert "workload" in d["config"] and "model" not in d["config"]
 
 
+def test_peaks_are_those_of_the_unit_that_a_kernel_runs_on():
+    sys.path.insert(0, ROOT)
+    import bench
+    pk = {"tensor_burst": 1640.0, "source": "measured"}
+    assert bench.compute_peak("tc_gemm_fwd", "bf16", pk)[:2] == ("tensor", 1640.0)
+    assert bench.compute_peak("mma_wgrad", "bf16", pk)[:2] == ("tensor", 1640.0)
+    assert bench.compute_peak("mma_dgrad", "fp32", pk)[:2] == ("tensor", 1640.0 / 6)
+    assert bench.compute_peak("fma_fwd", "fp32", pk)[:2] == ("alu", bench.FMA_PEAK_TFLOPS)
+    assert bench.compute_peak("bn_fwd_apply", "fp32", pk) is None
+
+
 import pytest
 
 

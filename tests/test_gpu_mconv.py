@@ -99,3 +99,23 @@ def test_nothing_is_laid_out_for_other_kernels(dtype):
                 ctx.close()
     assert used[1, 0] == used[1, 1], used
     assert used[16, 0][1] == used[16, 1][1] + 3, used
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("path", [0, 1])
+def test_kernel_classes(dtype, path):
+    """A layer of 16-multiple channels is counted under the tensor-core classes, one of 24 channels, and everything with kernel_path 1, under those of packed FMA."""
+    import torch
+    from paper_2509_05679_b200 import binding
+    layers = [(sy.CONV3X3, 32, 32, 1, 0), (sy.CONV3X3, 32, 32, 1, 0), (sy.CONV3X3, 32, 24, 1, 0), (sy.GLOBAL_AVGPOOL, 24, 24, 1, 0), (sy.LINEAR, 24, 10, 1, 1)]
+    net = sy.Net("mconv", layers, [], 16, 16, 32, 10, 2, 24, 0.05, dtype)
+    ctx = make_ctx(net, sy.init_params(layers, 0), kernel_path=path)
+    try:
+        ctx.profile(True)
+        ctx.step(binding.to_device(dtype, sy.batch_inputs(net, 0)), torch.from_numpy(sy.batch_labels(net, 0)).cuda())
+        n = {k: v["launches"] for k, v in ctx.profile_read().items() if "[" not in k}
+    finally:
+        ctx.close()
+    tensor, fma = ({"mma_fwd": 2, "mma_dgrad": 1, "mma_wgrad": 2}, {"fma_fwd": 1, "fma_dgrad": 1, "fma_wgrad": 1}) if path == 0 else ({}, {"fma_fwd": 3, "fma_dgrad": 2, "fma_wgrad": 3})
+    fma["fma_wgrad"] += 1                        # the classifier's backward pass
+    assert {k: v for k, v in n.items() if k.startswith(("mma_", "fma_"))} == {**tensor, **fma}, n
