@@ -1,7 +1,7 @@
 """The packed-FMA convolutions (fconv.cu) and the fp32 batch-norm (bnorm.cu) at sizes where their tilings can go wrong: images that
 are no power of two, smaller than a tile or one pixel wider, channel counts that are no multiple of 16 or of 4, strides 1 and 2, 3x3 and
 1x1, batches that leave a pixel tile ragged.  ReLU-free networks (no kinks), one step against the oracle: loss, every gradient and
-the updated parameters.  Tolerances: the fp32 path's 1e-5 (tests/harness.py: max_rel_err) on parameters and, in the 2-norm, on
+the updated parameters; with kernel_path 1, which keeps channels that are multiples of 16 on these kernels, and as they run without.  Tolerances: the fp32 path's 1e-5 (tests/harness.py: max_rel_err) on parameters and, in the 2-norm, on
 gradients; the bf16 storage model's 2e-3 of tests/test_gpu_bf16.py for contractions of at most 144 terms and its 2e-2 beyond."""
 import pytest
 
@@ -24,17 +24,19 @@ def _net(shape, dtype, workers, batch, bn):
     return sy.Net("fconv", layers, [], h, w, 3, 10, workers, batch, 0.05, dtype)
 
 
+@pytest.mark.parametrize("path", [0, 1])
 @pytest.mark.parametrize("bn", [False, True])
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: f"{s[0][0]}x{s[0][1]}-{s[1]}-{s[3]}-k{3 if s[2] == sy.CONV3X3 else 1}-s{s[4]}")
-def test_fp32(orc, shape, bn):
+def test_fp32(orc, shape, bn, path):
     # per-channel sums of normalised values cancel: with batch-norm in front of the average pool only the parameters have a scale of their own
-    run_parity(orc, _net(shape, "fp32", 3, 5, bn), 2, param_tol=1e-5, loss_tol=1e-5, grad_tol=None if bn else 1e-5)
+    run_parity(orc, _net(shape, "fp32", 3, 5, bn), 2, param_tol=1e-5, loss_tol=1e-5, grad_tol=None if bn else 1e-5, kernel_path=path)
 
 
+@pytest.mark.parametrize("path", [0, 1])
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: f"{s[0][0]}x{s[0][1]}-{s[1]}-{s[3]}-k{3 if s[2] == sy.CONV3X3 else 1}-s{s[4]}")
-def test_bf16_storage(orc, shape):
+def test_bf16_storage(orc, shape, path):
     terms = shape[1] * (9 if shape[2] == sy.CONV3X3 else 1)
-    run_parity(orc, _net(shape, "bf16", 2, 4, False), 1, grad_tol=2e-3 if terms <= 144 else 2e-2, loss_tol=1e-4)
+    run_parity(orc, _net(shape, "bf16", 2, 4, False), 1, grad_tol=2e-3 if terms <= 144 else 2e-2, loss_tol=1e-4, kernel_path=path)
 
 
 @pytest.mark.parametrize("workers,batch,groups", [(4, 3, 0), (4, 20, 2), (2, 70, 0)])
@@ -44,20 +46,21 @@ def test_images_that_no_power_of_two_covers(orc, size, stride, workers, batch, g
     run_parity(orc, _net((size, 16, sy.CONV3X3, 24, stride), "fp32", workers, batch, True), 1, param_tol=1e-5, loss_tol=1e-5, worker_groups=groups)
 
 
+@pytest.mark.parametrize("path", [0, 1])
 @pytest.mark.parametrize("workers,batch", [(1, 1), (2, 130), (5, 3)])
-def test_batch_sizes(orc, workers, batch):
-    run_parity(orc, _net(((8, 8), 16, sy.CONV3X3, 32, 2), "fp32", workers, batch, True), 2, param_tol=1e-5, loss_tol=1e-5)
+def test_batch_sizes(orc, workers, batch, path):
+    run_parity(orc, _net(((8, 8), 16, sy.CONV3X3, 32, 2), "fp32", workers, batch, True), 2, param_tol=1e-5, loss_tol=1e-5, kernel_path=path)
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
 @pytest.mark.parametrize("batch", [74, 75])
 def test_pixels_per_thread(orc, dtype, batch):
-    """2 x 74 and 2 x 75 images of 8x8, 16 -> 64 channels: 296 CTAs of two pixels a thread, 300 of four."""
+    """2 x 74 and 2 x 75 images of 8x8, 16 -> 64 channels: 296 CTAs of two pixels a thread, 300 of four (kernel_path 1: without, mconv.cu takes them)."""
     net = _net(((8, 8), 16, sy.CONV3X3, 64, 1), dtype, 2, batch, dtype == "fp32")
     if dtype == "fp32":
-        run_parity(orc, net, 1, param_tol=1e-5, loss_tol=1e-5)
+        run_parity(orc, net, 1, param_tol=1e-5, loss_tol=1e-5, kernel_path=1)
     else:
-        run_parity(orc, net, 1, grad_tol=2e-2, loss_tol=1e-4)
+        run_parity(orc, net, 1, grad_tol=2e-2, loss_tol=1e-4, kernel_path=1)
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])

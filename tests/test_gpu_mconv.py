@@ -1,6 +1,7 @@
-"""The tensor-core convolutions off the TMA path (mconv.cu: channel counts that are multiples of 16) at the edges of their tiles: images of odd sides, of one
-row, smaller than a tile; strides 1 and 2, 3x3 and 1x1; one, two and three blocks of 16 channels; batches that leave a tile ragged; magnitudes far from 1,
-where the parts of a split value get small.  One step of ReLU-free networks against the oracle, with the tolerances of tests/test_gpu_fconv.py."""
+"""The convolutions of 16-multiple channel counts off the TMA path, on both sides of the line between the tensor-core kernels (mconv.cu) and the packed-FMA kernels,
+at the edges of their tiles: images of odd sides, of one row or column, smaller than a tile; strides 1 and 2, 3x3 and 1x1; one, two and three blocks of 16
+channels; batches that leave a tile ragged; magnitudes far from 1, where the parts of a split value get small.  One step of ReLU-free networks against the
+oracle, with the tolerances of tests/test_gpu_fconv.py.  TAKEN: shapes whose three passes all run on mconv.cu, which the profiler has to say."""
 import numpy as np
 import pytest
 
@@ -13,6 +14,12 @@ pytestmark = pytest.mark.gpu
 SHAPES = [((5, 7), 16, sy.CONV3X3, 48, 1), ((33, 9), 16, sy.CONV3X3, 16, 1), ((16, 1), 16, sy.CONV3X3, 32, 1), ((2, 2), 32, sy.CONV3X3, 16, 1), ((6, 10), 32, sy.CONV3X3, 64, 2),
           ((14, 14), 16, sy.CONV3X3, 32, 2), ((7, 11), 16, sy.CONV1X1, 32, 1), ((6, 10), 48, sy.CONV1X1, 16, 2), ((4, 4), 80, sy.CONV3X3, 96, 1)]
 
+ALL, EVEN, ONE = [(1, 1), (3, 9), (2, 70)], [(1, 1), (2, 70)], [(1, 1)]
+# and the workers x batches that are taken with fp32 storage (bf16: all three); 16x16, 15x13 and 4x64: 2 x 70 with 32 output channels a CTA
+TAKEN = [(((12, 20), 16, sy.CONV3X3, 16, 1), ALL), (((33, 9), 16, sy.CONV3X3, 16, 1), EVEN), (((1, 40), 48, sy.CONV3X3, 16, 1), ONE), (((7, 7), 48, sy.CONV3X3, 32, 1), ALL),
+         (((15, 13), 32, sy.CONV3X3, 32, 1), ALL), (((16, 16), 32, sy.CONV3X3, 32, 1), ALL), (((4, 4), 80, sy.CONV3X3, 96, 1), ALL), (((14, 14), 16, sy.CONV3X3, 32, 2), ALL),
+         (((16, 30), 32, sy.CONV3X3, 48, 2), ALL), (((6, 10), 32, sy.CONV3X3, 64, 2), ONE), (((4, 64), 32, sy.CONV1X1, 32, 1), ALL), (((2, 64), 16, sy.CONV1X1, 32, 2), ALL)]
+
 
 def _net(shape, dtype, workers, batch, bn):
     (h, w), c, kind, co, stride = shape
@@ -24,6 +31,39 @@ def _net(shape, dtype, workers, batch, bn):
 
 def _id(s):
     return f"{s[0][0]}x{s[0][1]}-{s[1]}-{s[3]}-k{3 if s[2] == sy.CONV3X3 else 1}-s{s[4]}"
+
+
+def _assert_taken(net, shape):
+    """Forward, input gradient and weight gradient of the second layer ran on mconv.cu."""
+    import torch
+    from paper_2509_05679_b200 import binding
+    ctx = make_ctx(net, sy.init_params(net.layers, 0))
+    try:
+        ctx.profile(True)
+        ctx.step(binding.to_device(net.dtype, sy.batch_inputs(net, 0)), torch.from_numpy(sy.batch_labels(net, 0)).cuda())
+        ran = {k for k in ctx.profile_read() if k.startswith(("mma_", "fma_"))}
+    finally:
+        ctx.close()
+    (h, w), c, kind, co, stride = shape
+    tag = f"[{h}x{w} {c}->{co} k{3 if kind == sy.CONV3X3 else 1} s{stride}]"
+    assert {k for k in ran if k.endswith(tag)} == {f"mma_{p}{tag}" for p in ("fwd", "dgrad", "wgrad")}, ran
+
+
+@pytest.mark.parametrize("shape,workers,batch", [(s, w, b) for s, sizes in TAKEN for w, b in sizes], ids=lambda v: _id(v) if isinstance(v, tuple) else str(v))
+def test_fp32_on_tensor_cores(orc, shape, workers, batch):
+    net = _net(shape, "fp32", workers, batch, False)
+    _assert_taken(net, shape)
+    run_parity(orc, net, 1, param_tol=1e-5, loss_tol=1e-5, grad_tol=1e-5)
+    run_parity(orc, _net(shape, "fp32", workers, batch, True), 1, param_tol=1e-5, loss_tol=1e-5)
+
+
+@pytest.mark.parametrize("workers,batch", EVEN)
+@pytest.mark.parametrize("shape", [s for s, _ in TAKEN if s[0] != (6, 10)], ids=_id)
+def test_bf16_on_tensor_cores(orc, shape, workers, batch):
+    terms = shape[1] * (9 if shape[2] == sy.CONV3X3 else 1)
+    net = _net(shape, "bf16", workers, batch, False)
+    _assert_taken(net, shape)
+    run_parity(orc, net, 1, grad_tol=2e-3 if terms <= 144 and workers * batch in (1, 2, 4, 8) else 2e-2, loss_tol=1e-4)
 
 
 @pytest.mark.parametrize("workers,batch", [(1, 1), (3, 9), (2, 70)])
@@ -119,3 +159,28 @@ def test_kernel_classes(dtype, path):
     tensor, fma = ({"mma_fwd": 2, "mma_dgrad": 1, "mma_wgrad": 2}, {"fma_fwd": 1, "fma_dgrad": 1, "fma_wgrad": 1}) if path == 0 else ({}, {"fma_fwd": 3, "fma_dgrad": 2, "fma_wgrad": 3})
     fma["fma_wgrad"] += 1                        # the classifier's backward pass
     assert {k: v for k, v in n.items() if k.startswith(("mma_", "fma_"))} == {**tensor, **fma}, n
+
+
+def test_more_layers_than_one_launch_lays_out():
+    """50 layers: the weights of 48 in one launch, of the others in a second.  Gradients beside those of the packed-FMA kernels (1e-4 in the 2-norm: roundings of
+    1e-7 through 50 layers, times 20 for the last ones' cancellations)."""
+    import torch
+    from paper_2509_05679_b200 import binding
+    layers = [(sy.CONV3X3, 16, 16, 1, 0)] * 50 + [(sy.GLOBAL_AVGPOOL, 16, 16, 1, 0), (sy.LINEAR, 16, 10, 1, 1)]
+    net = sy.Net("mconv", layers, [], 8, 8, 16, 10, 2, 3, 0.0, "fp32")
+    p0 = sy.init_params(layers, 0) * np.float32(0.7)           # gain of about 1 a layer
+    x, y = binding.to_device("fp32", sy.batch_inputs(net, 0)), torch.from_numpy(sy.batch_labels(net, 0)).cuda()
+    g = []
+    for path in (0, 1):
+        ctx = make_ctx(net, p0, kernel_path=path)
+        try:
+            if path == 0:
+                ctx.profile(True)
+            ctx.step(x, y)
+            if path == 0:
+                assert ctx.profile_read()["mma_fwd"]["launches"] == 50
+            g.append(np.asarray(ctx.grads(), np.float64))
+        finally:
+            ctx.close()
+    for a, b in zip(np.split(g[0][:50 * 2304], 50), np.split(g[1][:50 * 2304], 50)):
+        assert 0 < np.linalg.norm(b) < np.inf and np.linalg.norm(a - b) <= 1e-4 * np.linalg.norm(b)
