@@ -1146,19 +1146,19 @@ constexpr int HEAD_MAX_C = 16;
 constexpr int HEAD_ROWS_PER_CTA = 32;       // samples per CTA of head_bwd_k
 constexpr size_t HEAD_W_SMEM = 40 * 1024;   // a larger W is read from L2 by every warp (static and dynamic shared memory stay below the 48 KB of any launch)
 constexpr int HEAD_STAGE_VECS = 32;         // wider slices are there for many samples, where other CTAs cover the latency
-template <typename T>
+// W_SMEM: W fits into HEAD_W_SMEM (a kernel of its own: through a pointer to either, loads from L2 are no longer known to be of constant global memory:
+// one bf16 layer of 4096 columns and 16 classes, one sample, 68 us a step instead of 47)
+template <typename T, bool W_SMEM>
 __global__ void __launch_bounds__(256) head_fwd_loss_k(const T* __restrict__ x, const T* __restrict__ W, const float* __restrict__ bias,
                                                        const int32_t* __restrict__ labels, float* __restrict__ logits, T* __restrict__ dz,
-                                                       float* __restrict__ loss_part, int M, int K, int C, float scale, bool w_smem) {
+                                                       float* __restrict__ loss_part, int M, int K, int C, float scale) {
     constexpr int V = Vec<T>::V;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = blockIdx.x * 8 + warp;
     __shared__ float wl[8];
     extern __shared__ __align__(16) char hsm[];
-    const T* Wp = W;
-    if (w_smem) {                            // (uniform) all of W, 16 bytes a thread at a time
+    if constexpr (W_SMEM) {                  // all of W, 16 bytes a thread at a time
         for (int i = threadIdx.x; i < C * K / V; i += 256) ((uint4*)hsm)[i] = ((const uint4*)W)[i];
-        Wp = (const T*)hsm;
         __syncthreads();
     }
     float rloss = 0.f;
@@ -1175,7 +1175,7 @@ __global__ void __launch_bounds__(256) head_fwd_loss_k(const T* __restrict__ x, 
                 if (c >= C) break;
                 float wv[8][8];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) Vec<T>::load(Wp + (size_t)min(c + q, C - 1) * K + (size_t)kv * V, wv[q]);
+                for (int q = 0; q < 8; ++q) Vec<T>::load((W_SMEM ? (const T*)hsm : W) + (size_t)min(c + q, C - 1) * K + (size_t)kv * V, wv[q]);
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
 #pragma unroll
@@ -1352,8 +1352,10 @@ void head_forward_loss(int dt, const void* x, const void* W, const float* bias, 
     Scope sc(KC_SOFTMAX_CE, 2.0 * M * K * C, (dt ? 2.0 : 4.0) * ((double)M * K + (double)C * K + (double)M * C) + 4.0 * M * C, s);
     const unsigned grid = (M + 7) / 8;
     const size_t w_bytes = (size_t)C * K * (dt ? 2 : 4), smem = w_bytes <= HEAD_W_SMEM ? w_bytes : 0;
-    if (dt) klaunch(head_fwd_loss_k<bf16>, grid, 256, smem, s, (const bf16*)x, (const bf16*)W, bias, labels, logits, (bf16*)dlogits, loss_part, M, K, C, scale, smem > 0);
-    else klaunch(head_fwd_loss_k<float>, grid, 256, smem, s, (const float*)x, (const float*)W, bias, labels, logits, (float*)dlogits, loss_part, M, K, C, scale, smem > 0);
+    if (dt) klaunch(smem ? head_fwd_loss_k<bf16, true> : head_fwd_loss_k<bf16, false>, grid, 256, smem, s, (const bf16*)x, (const bf16*)W, bias, labels, logits, (bf16*)dlogits, loss_part, M, K, C,
+                    scale);
+    else klaunch(smem ? head_fwd_loss_k<float, true> : head_fwd_loss_k<float, false>, grid, 256, smem, s, (const float*)x, (const float*)W, bias, labels, logits, (float*)dlogits, loss_part, M, K, C,
+                 scale);
 }
 int head_col_records(int M) { return (M + HEAD_ROWS_PER_CTA - 1) / HEAD_ROWS_PER_CTA; }
 void head_backward(int dt, const void* x, const void* W, const void* dlogits, void* dx_or_null, bool accum_dx, bool mask_dx, float* col_or_null, float* scratch, int M,
