@@ -676,9 +676,12 @@ bool run_mc(const void* x, const void* w, const void* pk, const float* bias, voi
     q.pack_group = pack_group / 16;
     const long tiles = (long)q.p.tiles_w * q.p.tiles_h * ((q.p.ngroup + q.p.Nt - 1) / q.p.Nt) * groups * q.p.ncls;
     // 32 output channels a CTA (a third less shared-memory traffic per product, the region split for twice the work), unless 16 fill the device more evenly;
-    // large regions (stride 2) leave an SM two CTAs at the most either way
+    // large regions (stride 2) leave an SM two CTAs at the most either way.  fp32 3x3 stride 1: 16 also where they make one wave of four per SM and up to three
+    // quarters of another, 0.82 to 0.98 of the time of 32 (192 images of 16x16, 32 -> 32: 25 us against 30; from 1.95 waves on 1.16 and more)
     const auto waves = [](long ctas) { return (ctas + 147) / 148; };
-    const bool wide = q.p.Co % 32 == 0 && (mc_smem<T, 2>(q) > 75 * 1024 || 2 * waves(tiles * (q.p.Co / 32)) <= 1.15 * waves(tiles * (q.p.Co / 16)));
+    const long narrow = tiles * (q.p.Co / 16);
+    const bool tail = SPLIT<T> && q.p.taps == 9 && q.p.ncls == 1 && q.p.xs == 1 && narrow > 4 * 148 && narrow <= 7 * 148;
+    const bool wide = q.p.Co % 32 == 0 && (mc_smem<T, 2>(q) > 75 * 1024 || (!tail && 2 * waves(tiles * (q.p.Co / 32)) <= 1.15 * waves(narrow)));
     return launched(wide ? launch_mc<T, 4>(x, w, pk, bias, y, stat, q, groups, s) : launch_mc<T, 2>(x, w, pk, bias, y, stat, q, groups, s));
 }
 template <typename T, int XS, int TW>
