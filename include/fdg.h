@@ -92,7 +92,9 @@ typedef struct {
     int32_t serial;            /* 1: run every module on one stream (results are bit-identical
                                   to the concurrent mode when both contexts have the same
                                   grid_sms; used to test the event wiring)                      */
-    int32_t kernel_path;       /* 0: tensor-core kernels where shapes allow, the 256-column
+    int32_t kernel_path;       /* 0: tensor-core kernels where shapes allow (fp32 storage: convolutions of channel counts
+                                     that are multiples of 16, every value as three bf16 parts, whose rounding errors are
+                                     no larger than those of 1), the 256-column
                                      tile (and the 128-column tile of 3x3 stride-1 layers on 16x16 images) as
                                      pairs of CTAs on two SMs (tcgen05 cta_group::2);
                                   1: plain FMA kernels only;

@@ -6,8 +6,8 @@
 //   mw_kernel : weight gradient.  A CTA keeps a 16 c_out x (taps x 16 c_in) tile of dW in registers over the pixels of its split.
 //   mc_pack_kernel : a layer's weights in the order in which the lanes of a warp hold them (one launch per pass for all layers of a module).
 //
-// Arithmetic with fp32 storage: a value is the sum of three bf16 values, x = hi + mid + lo (8 bits each, rounded to nearest, so that nothing is left), and
-// a product the sum of the six that matter: lo hi + mid mid + hi lo + mid hi + hi mid + hi hi (the rest is 6e-9 of it; 6e-8, and one-sided, with parts by
+// Arithmetic with fp32 storage: a value is the sum of three bf16 values, x = hi + mid + lo (8 bits each or, see below, 6 in hi; rounded to nearest, so that nothing is left), and
+// a product the sum of the six that matter: lo hi + mid mid + hi lo + mid hi + hi mid + hi hi (the rest is 2e-8 of it, of either sign; 6e-8, and one-sided, with parts by
 // truncation).  Every product is exact; an mma adds 16 of them to its running sum and truncates to 24 bits of the largest term: 2.5e-8 of the
 // result's rms for 16 fresh products of 16 bits, 1.3e-7 for nine such steps in a chain, 5.3e-7 for 36, 1e-7 as soon as a 24-bit running sum of
 // like size is among the terms.  So hi hi starts from zero in every step and goes into an fp32 sum on the CUDA cores, two taps of it into a
@@ -24,7 +24,7 @@
 // added in double: 1.00 times the packed-FMA kernels' errors at the most, 0.8 on average (1.19 with a flush per tile).  Forward and input gradient keep to
 // one flush per chunk there: 6.5e-8 before the result is rounded to bf16, by 1.7e-3 (4.4e-8; one every two taps gives 4.6e-8 for 4.5 % of a step).
 //
-// Time, 192 images, launch included (packed FMA beside it): fp32 32x32 16 -> 16 forward 25 us (38), weight gradient with its reduction 38 (54); 16x16 32 -> 32 27
+// Time, 192 images, launch included (packed FMA beside it): fp32 32x32 16 -> 16 forward 25 us (38), weight gradient with its reduction 38 (54); 16x16 32 -> 32 25
 // (40), 36 (53); 8x8 64 -> 64 29 (41), 39 (57).  What bounds them: a third to 40 % of the mma.sync rate (980 multiply-adds per clock and SM, six per
 // product), the rest is latency of one warp's chain (fixed-latency waits, ncu) and the splitting, which every block of 16 or 32 output channels repeats.
 #include "fconv.h"
