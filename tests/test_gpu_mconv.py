@@ -2,6 +2,8 @@
 at the edges of their tiles: images of odd sides, of one row or column, smaller than a tile; strides 1 and 2, 3x3 and 1x1; one, two and three blocks of 16
 channels; batches that leave a tile ragged; magnitudes far from 1, where the parts of a split value get small.  One step of ReLU-free networks against the
 oracle, with the tolerances of tests/test_gpu_fconv.py.  TAKEN: shapes whose three passes all run on mconv.cu, which the profiler has to say."""
+import time
+
 import numpy as np
 import pytest
 
@@ -114,6 +116,63 @@ def test_values_far_from_one(orc, exponent):
         got[:n1 + 16] = g[:n1 + 16]
     err, where = max_rel_err(got, g, net.layers)
     assert err <= 1e-5, (err, where)
+
+
+@pytest.mark.parametrize("stride", [1, 2])
+@pytest.mark.parametrize("at", ["weight looked at", "weight", "pixel", "infinite weight"])
+def test_nan_where_packed_fma_has_it(at, stride):
+    """One NaN (or infinity) among the second layer's weights or in the input: the gradients that are NaN, and the values of the others, are those of kernel_path 1.
+    ReLU turns NaN to 0, so that the loss is finite.  1e-5 of a tensor's largest: the tolerance of test_fp32."""
+    import torch
+    from paper_2509_05679_b200 import binding
+    layers = [(sy.CONV3X3, 16, 16, 1, 0), (sy.RELU, 16, 16, 1, 0), (sy.CONV3X3, 16, 32, stride, 0), (sy.RELU, 32, 32, 1, 0), (sy.GLOBAL_AVGPOOL, 32, 32, 1, 0), (sy.LINEAR, 32, 10, 1, 1)]
+    net = sy.Net("mconv", layers, [], 16, 16, 16, 10, 2, 9, 0.0, "fp32")
+    p0, x = sy.init_params(layers, 0), sy.batch_inputs(net, 0)
+    w2 = p0[2304:2304 + 4608].reshape(32, 9, 16)
+    if at == "weight looked at":
+        w2[3, 4, 0] = np.nan
+    elif at == "weight":
+        w2[30, 8, 13] = np.nan
+    elif at == "infinite weight":
+        w2[17, 2, 5] = np.inf
+    else:
+        x.reshape(18, 16, 16, 16)[7, 5, 9, 11] = np.nan
+    g = []
+    for path in (0, 1):
+        ctx = make_ctx(net, p0, kernel_path=path)
+        try:
+            ctx.step(binding.to_device("fp32", x), torch.from_numpy(sy.batch_labels(net, 0)).cuda())
+            g.append(np.asarray(ctx.grads(), np.float64))
+        finally:
+            ctx.close()
+    assert np.array_equal(np.isnan(g[0]), np.isnan(g[1])) and not np.isnan(g[0]).all()
+    for a, b in zip(*(np.split(v, [2304, 2304 + 4608, 2304 + 4608 + 320]) for v in g)):
+        ok = np.isfinite(b)
+        assert np.abs(a - b)[ok].max(initial=0) <= 1e-5 * np.abs(b)[ok].max(initial=0)
+
+
+def test_nan_everywhere_costs_little():
+    """A diverged run goes on at its pace: less than three times as long with NaN for all parameters (12 times without the look at an output's operands, 1.4 with it)."""
+    import torch
+    from paper_2509_05679_b200 import binding
+    layers = [(sy.CONV3X3, 3, 16, 1, 0)] + [(sy.CONV3X3, 16, 16, 1, 0)] * 8 + [(sy.CONV3X3, 16, 32, 2, 0), (sy.CONV3X3, 32, 32, 1, 0), (sy.GLOBAL_AVGPOOL, 32, 32, 1, 0), (sy.LINEAR, 32, 10, 1, 1)]
+    net = sy.Net("mconv", layers, [], 32, 32, 3, 10, 4, 48, 0.0, "fp32")
+    x, y = binding.to_device("fp32", sy.batch_inputs(net, 0)), torch.from_numpy(sy.batch_labels(net, 0)).cuda()
+    p0, ms = sy.init_params(layers, 0), []
+    for p in (p0, np.full_like(p0, np.nan)):
+        ctx = make_ctx(net, p)
+        try:
+            for _ in range(5):
+                ctx.step(x, y)
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            for _ in range(20):
+                ctx.step(x, y)
+            torch.cuda.synchronize()
+            ms.append((time.perf_counter() - t0) * 50)
+        finally:
+            ctx.close()
+    assert ms[1] < 3 * ms[0], ms
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
